@@ -34,6 +34,8 @@ struct CommitParams {
   uint32_t H;
   uint32_t class_mask;         // bit c set: commit class c from pending_amax[c] (or from amax_override)
   float pow2_neg_margin;       // 2^-margin
+  uint32_t early_mask;         // GEMM launches: classes whose amax is complete when the launch starts (committed then, with
+                               // the token); class_mask holds the ones its own epilogue completes
   uint32_t bump_token;         // 1 for F and dI, 0 otherwise
   const float* amax_override;  // if non-null: value to push for the single class in class_mask
 };

@@ -458,7 +458,8 @@ void add_forward(qe_layer* L, uint32_t p, const void* x, void* y, std::vector<qe
   }
   gp.amax_bits = &L->st->pending_amax[QE_CLASS_Y];
   gp.status = &L->st->status;
-  gp.commit = commit_params(L, (1u << QE_CLASS_X) | (1u << QE_CLASS_Y), 1, nullptr);  // done by the GEMM's last CTA
+  gp.commit = commit_params(L, 1u << QE_CLASS_Y, 1, nullptr);  // done by the GEMM's last CTA ...
+  gp.commit.early_mask = 1u << QE_CLASS_X;                     // ... and by its first, once the cast before it is complete
   if (gemm_out) *gemm_out = gp;
   else ls.push_back(qe::make_gemm(gp, L->ctx->dev->num_sms));
 }
@@ -498,7 +499,8 @@ void add_dI(qe_layer* L, uint32_t p, const void* dy, void* dx, std::vector<qe::L
   }
   gp.amax_bits = nullptr;
   gp.status = &L->st->status;
-  gp.commit = commit_params(L, 1u << QE_CLASS_G, 1, nullptr);  // backward amax/scale updated exactly once, here
+  gp.commit = commit_params(L, 0, 1, nullptr);  // backward amax/scale updated exactly once, here: the cast (or the
+  gp.commit.early_mask = 1u << QE_CLASS_G;      // hand-off) that made Gq has completed the amax before this GEMM starts
   if (gemm_out) *gemm_out = gp;
   else ls.push_back(qe::make_gemm(gp, L->ctx->dev->num_sms));
 }
