@@ -1,21 +1,23 @@
 // FP8 GEMM for sm_100a: D[M,N] = (A[M,Kc] . B[N,Kc]^T) * alpha, A and B bytes (E4M3 or E5M2, mixed freely), each
-// stored contraction-major ([rows, Kc]) or, in the paired variant, MN-major ([Kc, rows]: the transposed view of a
-// row-major tensor, read by the tensor cores directly), FP32 accumulation in tensor memory.
+// stored contraction-major ([rows, Kc]) or MN-major ([Kc, rows]: the transposed view of a row-major tensor, read by the
+// tensor cores directly), FP32 accumulation in tensor memory.
 //
-// Structure (one persistent CTA per SM, 320 threads):
-//   warp 0      TMA producer: cp.async.bulk.tensor 2D tiles (128-byte swizzle) into a shared-memory ring (6 stages
-//               of 32 KB in the paired variant, 4 of 48 KB in the single-CTA one)
-//   warp 1      allocates tensor memory, then one lane issues tcgen05.mma (128 x 256 x 32 per instruction) and
-//               tcgen05.commit to release ring stages / publish a finished accumulator
-//   warps 2-9   epilogue: tcgen05.ld the 128 x 256 FP32 accumulator (two warps per 32-lane quadrant, 128 columns
-//               each) in 32 x 32 blocks, scale, write each block into a swizzled per-warp shared-memory tile and
-//               hand it to the bulk-store unit: a bulk tensor store for bf16 (+ max|D| reduced by warp shuffles,
-//               one atomicMax per warp and tile) and for FP32 overwrite; a bulk tensor reduction (.add) for FP32
-//               accumulation straight into the destination (direct gradient placement): the addition is done in
+// Structure: persistent clusters of two CTAs on neighbouring SMs, 320 threads each, that compute one tile of 256 rows
+// and 256, 128 or 64 columns together with tcgen05.mma.cta_group::2:
+//   warp 0      TMA producer: cp.async.bulk.tensor 2D tiles into a six-stage shared-memory ring; per 128-byte K block
+//               each CTA loads its own 128 rows of A and its own half of the tile's B rows
+//   warp 1      allocates tensor memory, then one lane of the even CTA issues tcgen05.mma (256 x tile_n x 32 per
+//               instruction) and tcgen05.commit, which multicasts stage-free / accumulator-ready arrivals to both CTAs
+//   warps 2-9   epilogue: tcgen05.ld the CTA's 128 x tile_n FP32 accumulator (two warps per 32-lane quadrant, half of
+//               the columns each) in 32 x 32 blocks, scale, write each block into a swizzled per-warp shared-memory
+//               tile and hand it to the bulk-store unit: a bulk tensor store for bf16 (+ max|D| reduced by warp
+//               shuffles, one atomicMax per warp and tile) and for FP32 overwrite; a bulk tensor reduction (.add) for
+//               FP32 accumulation straight into the destination (direct gradient placement): the addition is done in
 //               L2, one per element and launch, and the destination tile is prefetched into L2 while the tile's
 //               main loop runs.  The reduction is a plain round-to-nearest FP32 addition (subnormal values kept).
 //   The launch may also carry up to eight independent problems (grouped launch): tiles are numbered problem after
 //   problem and each role looks its tile's problem up, so that one set of persistent CTAs packs them all.
+// Rows beyond M (M is a multiple of 128; a tile has 256) are read as zeros by TMA and never stored.
 // Scale commits (fold a pending amax into its history, update the scale) ride along, so that no extra launch is needed:
 // classes whose amax an earlier kernel completed (X of a forward, G of an input gradient) are committed by an idle
 // epilogue warp while the first tile is being computed; only the class the epilogue itself reduces (Y) waits for the
@@ -23,15 +25,10 @@
 // ended with a ticket and a chain of dependent loads: 3270 us per step, 2979 us with the early commits.
 // Two accumulators (2 x 256 tensor-memory columns) let the epilogue of tile i overlap the main loop of tile i+1.
 //
-// Two variants share the code below.  The single-CTA one computes 128 x 256 tiles.  The paired one (used whenever M
-// is a multiple of 256) runs as clusters of two CTAs on neighbouring SMs that compute one 256 x 256 tile together
-// with tcgen05.mma.cta_group::2: each CTA loads its own 128 rows of A and its own 128 rows of B (32 KB per stage
-// instead of 48 KB), the even CTA issues the MMAs for the pair, tcgen05.commit multicasts stage-free and
-// accumulator-ready arrivals to both CTAs, and each CTA drains its own 128 accumulator rows.  That halves the
-// B-operand shared-memory traffic per SM, which is what bounds the single-CTA variant.  No TMA multicast is used.
+// No TMA multicast is used.
 // Each output element is produced by exactly one thread with a fixed contraction order and reaches its destination
 // by exactly one store or one addition per launch, so results do not depend on the grid size or on how tiles are
-// scheduled (no split-K; launches that add to the same destination are ordered by their stream).
+// scheduled, nor on how wide they are (no split-K; launches that add to the same destination are ordered by their stream).
 //
 // Every wait on an mbarrier is bounded by a clock budget; on expiry the thread ORs an error bit into the status
 // word, raises a CTA-wide abort flag that all other waits observe, and the CTA falls through to its common exit
@@ -45,27 +42,20 @@
 namespace qe {
 namespace {
 
-constexpr int BM = 128, BN = 256, BK = 128;  // per-CTA rows, tile columns, bytes (= FP8 elements) per stage along K
+constexpr uint32_t BM = 128, BK = 128;  // rows per CTA; bytes (= FP8 elements) per stage along the contraction
+constexpr uint32_t TILE_M = 2 * BM;     // rows of D per tile (per CTA pair)
+constexpr uint32_t ACC_COLS = 256;      // tensor-memory columns between the two accumulators (the widest tile)
 constexpr int UMMA_K = 32;
 constexpr uint32_t A_BYTES = BM * BK;
+constexpr uint32_t STAGE_BYTES = 2 * A_BYTES;  // A and at most as many rows of B (nine stages of 20 KB measured no
+constexpr int STAGES = 6;                      // faster at 64 columns: the ring's latency is covered)
 constexpr uint32_t TMEM_COLS = 512;
-constexpr int MAX_STAGES = 6;
 constexpr uint32_t EPI_BUF_BYTES = 4096;                     // per epilogue warp: one FP32 or two bf16 32 x 32 output tiles
                                                              // (1 KB-aligned, swizzled) that the bulk-store unit reads
-template <bool TWO>
-struct Cfg {
-  static constexpr int STAGES = TWO ? 6 : 4;
-  static constexpr uint32_t B_ROWS = TWO ? 128 : 256;  // rows of B this CTA loads per stage
-  static constexpr uint32_t B_BYTES = B_ROWS * BK;
-  static constexpr uint32_t STAGE_BYTES = A_BYTES + B_BYTES;
-  static constexpr uint32_t TILE_M = TWO ? 256 : 128;  // rows of D per tile (per cluster)
-  static constexpr uint32_t CTAS = TWO ? 2 : 1;
-};
 constexpr int THREADS = 320;
 constexpr int EPI_WARPS = 8, EPI_THREADS = EPI_WARPS * 32;
 static_assert(EPI_WARPS == 8, "shared-memory budget below assumes 8 epilogue warps");
-constexpr uint32_t SMEM_BYTES = 6 * (A_BYTES + 128 * BK) + 1024 /*alignment slack*/ + 256 /*barriers, flags*/ +
-                                8 * EPI_BUF_BYTES;  // 192 KB of stages in either variant
+constexpr uint32_t SMEM_BYTES = STAGES * STAGE_BYTES + 1024 /*alignment slack*/ + 256 /*barriers, flags*/ + 8 * EPI_BUF_BYTES;
 constexpr long long WAIT_BUDGET_CYCLES = 4000000000ll;  // ~2 s at the maximum SM clock
 
 constexpr uint32_t ERR_PRODUCER = 1u, ERR_MMA = 2u, ERR_EPILOGUE = 4u;
@@ -78,9 +68,6 @@ __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
 }
 __device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
   uint32_t ok;
@@ -151,13 +138,6 @@ __device__ __forceinline__ void tc_mma_f8_pair(uint32_t d_tmem, uint64_t adesc, 
       : "memory");
 }
 
-__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, uint32_t bar, int c0, int c1) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
-      ::"r"(dst), "l"(map), "r"(bar), "r"(c0), "r"(c1)
-      : "memory");
-}
-
 __device__ __forceinline__ void tma_prefetch_2d(const CUtensorMap* map, int c0, int c1) {
   asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global.tile [%0, {%1, %2}];" ::"l"(map), "r"(c0), "r"(c1) : "memory");
 }
@@ -185,27 +165,11 @@ __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.a
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
-__device__ __forceinline__ void tc_commit(uint32_t bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
-}
-
-__device__ __forceinline__ void tc_mma_f8(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
-                                          uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %1, %2, %3, p;\n\t}"
-      ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
-
-// Shared-memory matrix descriptor for a contraction-major tile whose rows are 128 bytes, 128-byte swizzle:
-// start address (>>4) in bits 0-13; leading byte offset (unused for this layout) 1 in bits 16-29; stride byte
-// offset = 1024 (eight 128-byte rows) >>4 in bits 32-45; descriptor version 1 in bits 46-47; swizzle mode 2
-// (128 B) in bits 61-63.
-__device__ __forceinline__ uint64_t make_desc(uint32_t saddr) {
-  return (uint64_t)((saddr & 0x3ffffu) >> 4) | (1ull << 16) | ((uint64_t)(1024 >> 4) << 32) | (1ull << 46) |
-         (2ull << 61);
+// Shared-memory matrix descriptor: start address (>>4) in bits 0-13; leading byte offset (unused: one swizzle atom in
+// that direction) 1 in bits 16-29; the high word (stride byte offset >>4 in bits 32-45, descriptor version 1 in bits
+// 46-47, swizzle mode in bits 61-63) comes from the host: desc_hi() below.
+__device__ __forceinline__ uint64_t make_desc(uint32_t saddr, uint32_t hi) {
+  return (uint64_t)((saddr & 0x3ffffu) >> 4) | (1ull << 16) | ((uint64_t)hi << 32);
 }
 
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
@@ -231,17 +195,24 @@ __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
 // operand fastest means that operand is swept again and again (from L2, where it fits) while the larger one is
 // streamed from HBM once.
 __device__ __forceinline__ void tile_coords(uint32_t tile, uint32_t tiles_m, uint32_t tiles_n, bool m_fastest,
-                                            uint32_t tile_m, uint32_t& m0, uint32_t& n0) {
+                                            uint32_t tile_n, uint32_t& m0, uint32_t& n0) {
   if (m_fastest) {
-    m0 = (tile % tiles_m) * tile_m;
-    n0 = (tile / tiles_m) * BN;
+    m0 = (tile % tiles_m) * TILE_M;
+    n0 = (tile / tiles_m) * tile_n;
   } else {
-    n0 = (tile % tiles_n) * BN;
-    m0 = (tile / tiles_n) * tile_m;
+    n0 = (tile % tiles_n) * tile_n;
+    m0 = (tile / tiles_n) * TILE_M;
   }
 }
 
 __device__ __forceinline__ void epi_bar_sync() { asm volatile("bar.sync 1, %0;" ::"n"(EPI_THREADS) : "memory"); }
+
+// High word of the descriptor of a tile whose rows are `row` bytes (128, 64 or 32), swizzled over the row: eight rows
+// make up the stride; swizzle mode 2 / 4 / 6 for 128 / 64 / 32 bytes.
+__host__ __device__ constexpr uint32_t desc_hi(uint32_t row) {
+  return (8u * row >> 4) | (1u << 14) | ((row == 128u ? 2u : row == 64u ? 4u : 6u) << 29);
+}
+constexpr uint32_t A_DESC_HI = desc_hi(128u);  // an A tile always has 128-byte rows
 
 // Which tile cluster `first` of `step` clusters takes in wave w: the clusters walk the tile list back and forth, so
 // that with tiles sorted by decreasing duration the cluster that got the longest tile of one wave gets the shortest
@@ -255,7 +226,7 @@ __device__ __forceinline__ uint32_t snake_tile(uint32_t w, uint32_t first, uint3
 // other, so that one set of persistent CTAs packs them into common waves and the launch overhead is paid once.
 struct OneProblem {
   const GemmParams& p;
-  __device__ __forceinline__ uint32_t total_tiles(uint32_t tile_m) const { return (p.M / tile_m) * ((p.N + BN - 1) / BN); }
+  __device__ __forceinline__ uint32_t total_tiles() const { return ((p.M + TILE_M - 1) / TILE_M) * ((p.N + p.tile_n - 1) / p.tile_n); }
   __device__ __forceinline__ const GemmParams& at(uint32_t tile, uint32_t& local) const {
     local = tile;
     return p;
@@ -267,7 +238,7 @@ struct OneProblem {
 };
 struct ProblemGroup {
   const GemmGroupParams& g;
-  __device__ __forceinline__ uint32_t total_tiles(uint32_t) const { return g.tile_end[g.n - 1]; }
+  __device__ __forceinline__ uint32_t total_tiles() const { return g.tile_end[g.n - 1]; }
   __device__ __forceinline__ const GemmParams& at(uint32_t tile, uint32_t& local) const {
     uint32_t i = 0, base = 0;
     while (i + 1 < g.n && tile >= g.tile_end[i]) base = g.tile_end[i++];
@@ -281,35 +252,33 @@ struct ProblemGroup {
 };
 
 // ------------------------------------------------------------------------------------------------ kernel
-template <bool TWO, class PS>
+template <class PS>
 __device__ __forceinline__ void gemm_body(const PS& ps) {
-  using C = Cfg<TWO>;
-  constexpr int STAGES = C::STAGES;
-  constexpr uint32_t STAGE_BYTES = C::STAGE_BYTES;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   const uint32_t epi_base = smem_base + STAGES * STAGE_BYTES;  // 1 KB-aligned
   const uint32_t bar_base = epi_base + 8 * EPI_BUF_BYTES;
   // barrier block: full[STAGES], empty[STAGES], tmem_full[2], tmem_empty[2], then tmem address + abort flag
   auto full_bar = [&](int s) { return bar_base + 8u * s; };
-  auto empty_bar = [&](int s) { return bar_base + 8u * (MAX_STAGES + s); };
-  auto tfull_bar = [&](int a) { return bar_base + 8u * (2 * MAX_STAGES + a); };
-  auto tempty_bar = [&](int a) { return bar_base + 8u * (2 * MAX_STAGES + 2 + a); };
+  auto empty_bar = [&](int s) { return bar_base + 8u * (STAGES + s); };
+  auto tfull_bar = [&](int a) { return bar_base + 8u * (2 * STAGES + a); };
+  auto tempty_bar = [&](int a) { return bar_base + 8u * (2 * STAGES + 2 + a); };
   uint8_t* gen_base = smem_raw + (smem_base - smem_u32(smem_raw));
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(gen_base + STAGES * STAGE_BYTES + 8 * EPI_BUF_BYTES + 8 * (2 * MAX_STAGES + 4));
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(gen_base + STAGES * STAGE_BYTES + 8 * EPI_BUF_BYTES + 8 * (2 * STAGES + 4));
   volatile uint32_t* abort_flag = tmem_slot + 1;
   uint32_t* last_flag = tmem_slot + 2;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const uint32_t rank = TWO ? cluster_ctarank() : 0u;  // position in the CTA pair; rank 0 issues the MMAs
-  const uint32_t num_tiles = ps.total_tiles(C::TILE_M);
-  const uint32_t first_tile = blockIdx.x / C::CTAS, tile_step = gridDim.x / C::CTAS;
+  const uint32_t rank = cluster_ctarank();  // position in the CTA pair; rank 0 issues the MMAs
+  const uint32_t num_tiles = ps.total_tiles();
+  const uint32_t first_tile = blockIdx.x / 2u, tile_step = gridDim.x / 2u;
   uint32_t* const status = ps.first().status;
 // per tile: which problem it belongs to (`p`), its index inside that problem and the problem's tiling
-#define QE_TILE_PROBLEM()                                                                      \
-  uint32_t local_tile;                                                                         \
-  const GemmParams& p = ps.at(tile, local_tile);                                               \
-  const uint32_t tiles_m = p.M / C::TILE_M, tiles_n = (p.N + BN - 1) / BN, num_kb = p.Kc / BK; \
+#define QE_TILE_PROBLEM()                                                                                     \
+  uint32_t local_tile;                                                                                        \
+  const GemmParams& p = ps.at(tile, local_tile);                                                              \
+  const uint32_t tile_n = p.tile_n, tiles_m = (p.M + TILE_M - 1) / TILE_M, tiles_n = (p.N + tile_n - 1) / tile_n; \
+  const uint32_t num_kb = p.Kc / BK;                                                                          \
   const bool m_fastest = p.M <= p.N
 
   if (threadIdx.x == 32) {  // descriptor fetch overlaps the rest of the prologue (and the predecessor's tail)
@@ -325,28 +294,22 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
     }
     for (int a = 0; a < 2; ++a) {
       mbar_init(tfull_bar(a), 1);
-      mbar_init(tempty_bar(a), EPI_WARPS * C::CTAS);  // the epilogue warps of every CTA of the pair
+      mbar_init(tempty_bar(a), EPI_WARPS * 2);  // the epilogue warps of both CTAs of the pair
     }
     *abort_flag = 0u;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
   if (warp == 1) {
-    if (TWO) {  // same warp in both CTAs of the pair
-      asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
-                   "r"(TMEM_COLS)
-                   : "memory");
-      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
-    } else {
-      asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
-                   "r"(TMEM_COLS)
-                   : "memory");
-      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-    }
+    // same warp in both CTAs of the pair
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
+                 "r"(TMEM_COLS)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
   }
   tc_fence_before();
   __syncthreads();
-  if (TWO) cluster_sync_all();  // the peer's barriers are initialised before anything signals them
+  cluster_sync_all();  // the peer's barriers are initialised before anything signals them
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
   if (warp == 0 && lane == 0 && first_tile < num_tiles) {
@@ -355,8 +318,8 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
     const uint32_t tile = first_tile;
     QE_TILE_PROBLEM();
     uint32_t m0, n0;
-    tile_coords(local_tile, tiles_m, tiles_n, m_fastest, C::TILE_M, m0, n0);
-    const int rb = (int)(n0 + (TWO ? rank * C::B_ROWS : 0u));
+    tile_coords(local_tile, tiles_m, tiles_n, m_fastest, tile_n, m0, n0);
+    const int rb = (int)(n0 + rank * (tile_n / 2));
     for (uint32_t kb = 0; kb < num_kb && kb < (uint32_t)STAGES; ++kb) {
       const int ka = (int)(kb * BK);
       if (p.b_mn) tma_prefetch_2d(&p.tmB, rb, ka);
@@ -391,26 +354,21 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
       for (uint32_t wave = 0, tile = first_tile; ok && tile < num_tiles; ++wave, tile = snake_tile(wave, first_tile, tile_step)) {
         QE_TILE_PROBLEM();
         uint32_t m0, n0;
-        tile_coords(local_tile, tiles_m, tiles_n, m_fastest, C::TILE_M, m0, n0);
+        tile_coords(local_tile, tiles_m, tiles_n, m_fastest, tile_n, m0, n0);
+        const int ra = (int)(m0 + rank * BM), rb = (int)(n0 + rank * (tile_n / 2));
         for (uint32_t kb = 0; kb < num_kb; ++kb) {
           if (!(ok = mbar_wait(empty_bar(s), ph ^ 1u, abort_flag, status, ERR_PRODUCER))) break;
           const uint32_t a_dst = smem_base + s * STAGE_BYTES, b_dst = a_dst + A_BYTES;
-          if (TWO) {
-            // both CTAs credit the even CTA's barrier, which expects the bytes of the whole pair
-            if (rank == 0) mbar_expect_tx(full_bar(s), 2 * STAGE_BYTES);
-            const uint32_t bar = map_to_cta(full_bar(s), 0);
-            // contraction-major operand: box = 128 K-bytes x 128 rows at (k, row); MN-major operand (stored as
-            // [Kc, rows]): box = 128 row-bytes x 128 K-rows at (row, k).  Either way 16 KB land in shared memory.
-            const int ka = (int)(kb * BK), ra = (int)(m0 + rank * BM), rb = (int)(n0 + rank * C::B_ROWS);
-            if (p.a_mn) tma_load_2d_pair(a_dst, &p.tmA, bar, ra, ka);
-            else tma_load_2d_pair(a_dst, &p.tmA, bar, ka, ra);
-            if (p.b_mn) tma_load_2d_pair(b_dst, &p.tmB, bar, rb, ka);
-            else tma_load_2d_pair(b_dst, &p.tmB, bar, ka, rb);
-          } else {
-            mbar_expect_tx(full_bar(s), STAGE_BYTES);
-            tma_load_2d(a_dst, &p.tmA, full_bar(s), (int)(kb * BK), (int)m0);
-            tma_load_2d(b_dst, &p.tmB, full_bar(s), (int)(kb * BK), (int)n0);
-          }
+          // both CTAs credit the even CTA's barrier, which expects the bytes of the whole pair
+          if (rank == 0) mbar_expect_tx(full_bar(s), 2 * A_BYTES + tile_n * BK);
+          const uint32_t bar = map_to_cta(full_bar(s), 0);
+          // contraction-major operand: box = 128 K-bytes x rows at (k, row); MN-major operand (stored as [Kc, rows]):
+          // box = row-bytes x 128 K-rows at (row, k).  Either way 128 bytes per row land in shared memory.
+          const int ka = (int)(kb * BK);
+          if (p.a_mn) tma_load_2d_pair(a_dst, &p.tmA, bar, ra, ka);
+          else tma_load_2d_pair(a_dst, &p.tmA, bar, ka, ra);
+          if (p.b_mn) tma_load_2d_pair(b_dst, &p.tmB, bar, rb, ka);
+          else tma_load_2d_pair(b_dst, &p.tmB, bar, ka, rb);
           if (++s == STAGES) { s = 0; ph ^= 1u; }
         }
       }
@@ -431,63 +389,60 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
         (void)tiles_m; (void)tiles_n; (void)m_fastest;
         if (!(ok = mbar_wait(tempty_bar(acc), acc_ph ^ 1u, abort_flag, status, ERR_MMA))) break;
         tc_fence_after();
-        const uint32_t d_tmem = tmem_base + acc * (uint32_t)BN;
+        const uint32_t d_tmem = tmem_base + acc * ACC_COLS;
+        const uint32_t idesc = p.idesc, b_hi = p.b_desc_hi, a_step = p.a_mn ? 256u : 2u, b_step = p.b_step;
         for (uint32_t kb = 0; kb < num_kb; ++kb) {
           if (!(ok = mbar_wait(full_bar(s), ph, abort_flag, status, ERR_MMA))) break;
           tc_fence_after();
           const uint32_t a_src = smem_base + s * STAGE_BYTES, b_src = a_src + A_BYTES;
-          const uint64_t adesc = make_desc(a_src), bdesc = make_desc(b_src);
+          const uint64_t adesc = make_desc(a_src, A_DESC_HI), bdesc = make_desc(b_src, b_hi);
 #pragma unroll
-          for (int k = 0; k < BK / UMMA_K; ++k) {
+          for (int k = 0; k < (int)BK / UMMA_K; ++k)
             // advancing 32 along the contraction: 32 bytes inside the 128-byte swizzle row for a contraction-major
-            // tile (+2 in the address field), 32 rows of 128 bytes for an MN-major one (+256)
-            if (TWO) tc_mma_f8_pair(d_tmem, adesc + (p.a_mn ? 256u : 2u) * k, bdesc + (p.b_mn ? 256u : 2u) * k, p.idesc, (kb | (uint32_t)k) != 0u);
-            else tc_mma_f8(d_tmem, adesc + 2u * k, bdesc + 2u * k, p.idesc, (kb | (uint32_t)k) != 0u);
-          }
-          if (TWO) tc_commit_pair(empty_bar(s));  // stage reusable (in both CTAs) once these MMAs have read it
-          else tc_commit(empty_bar(s));
+            // tile (+2 in the address field), 32 rows for an MN-major one (+256 with rows of 128 bytes)
+            tc_mma_f8_pair(d_tmem, adesc + a_step * k, bdesc + b_step * k, idesc, (kb | (uint32_t)k) != 0u);
+          tc_commit_pair(empty_bar(s));  // stage reusable (in both CTAs) once these MMAs have read it
           if (++s == STAGES) { s = 0; ph ^= 1u; }
         }
         if (!ok) break;
-        if (TWO) tc_commit_pair(tfull_bar(acc));  // accumulator complete (each CTA holds its 128 rows)
-        else tc_commit(tfull_bar(acc));
+        tc_commit_pair(tfull_bar(acc));  // accumulator complete (each CTA holds its 128 rows)
         if (++acc == 2) { acc = 0; acc_ph ^= 1u; }
       }
     }
   } else {
     // ---------------------------------------------------------------- epilogue (warps 2..9)
     const uint32_t quad = (uint32_t)warp & 3u;          // tensor-memory lane quadrant this warp may read
-    const uint32_t half = ((uint32_t)warp - 2u) >> 2;   // which 128 of the tile's 256 columns
+    const uint32_t half = ((uint32_t)warp - 2u) >> 2;   // which half of the tile's columns
     const int etid = (int)threadIdx.x - 64;
     const uint32_t epi_smem = epi_base + (uint32_t)(warp - 2) * EPI_BUF_BYTES;  // this warp's two output tiles
     uint32_t n_groups = 0;  // bulk-store groups this warp has committed (buffer parity)
     uint32_t acc = 0, acc_ph = 0;
     bool ok = true;
-    const uint32_t tempty_leader0 = TWO ? map_to_cta(tempty_bar(0), 0) : tempty_bar(0);
-    const uint32_t tempty_leader1 = TWO ? map_to_cta(tempty_bar(1), 0) : tempty_bar(1);
+    const uint32_t tempty_leader0 = map_to_cta(tempty_bar(0), 0), tempty_leader1 = map_to_cta(tempty_bar(1), 0);
     for (uint32_t wave = 0, tile = first_tile; ok && tile < num_tiles; ++wave, tile = snake_tile(wave, first_tile, tile_step)) {
       QE_TILE_PROBLEM();
       (void)num_kb;
       const float alpha = __fmul_rn(*p.alpha_a, *p.alpha_b);
       uint32_t m0, n0;
-      tile_coords(local_tile, tiles_m, tiles_n, m_fastest, C::TILE_M, m0, n0);
-      const uint32_t row = m0 + rank * BM + quad * 32u + (uint32_t)lane;
-      const uint32_t col0 = n0 + half * 128u;
-      if (p.epi == 2 && col0 < p.N) {
-        // accumulate: pull this thread's 512 destination bytes into L2, where the reduction will add to them, while
-        // the MMAs of the tile run
-        const char* d = reinterpret_cast<const char*>(reinterpret_cast<const float*>(p.out) + (size_t)row * p.ldo + col0);
-#pragma unroll
-        for (int j = 0; j < 4; ++j) asm volatile("prefetch.global.L2 [%0];" ::"l"(d + 128 * j));
-      }
+      tile_coords(local_tile, tiles_m, tiles_n, m_fastest, tile_n, m0, n0);
       const uint32_t blk_row0 = m0 + rank * BM + quad * 32u;
-      const uint32_t nch = col0 >= p.N ? 0u : min(4u, (p.N - col0) / 32u);  // ragged last column tile; warp-uniform
+      const uint32_t col0 = n0 + half * (tile_n / 2);
+      // 32 x 32 blocks of this warp: none in rows beyond M, fewer in a ragged last column tile; warp-uniform
+      const uint32_t nch = blk_row0 >= p.M || col0 >= p.N ? 0u : min(tile_n / 64u, (p.N - col0) / 32u);
+      if (p.epi == 2) {
+        // accumulate: pull this thread's destination row segment into L2, where the reduction will add to it, while
+        // the MMAs of the tile run
+        const char* d = reinterpret_cast<const char*>(reinterpret_cast<const float*>(p.out) + (size_t)(blk_row0 + lane) * p.ldo + col0);
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if ((uint32_t)j < nch) asm volatile("prefetch.global.L2 [%0];" ::"l"(d + 128 * j));
+      }
       uint32_t r[2][32];
       if (!(ok = mbar_wait(tfull_bar(acc), acc_ph, abort_flag, status, ERR_EPILOGUE))) break;
       tc_fence_after();
-      const uint32_t t_row = tmem_base + ((quad * 32u) << 16) + acc * (uint32_t)BN + half * 128u;
+      const uint32_t t_row = tmem_base + ((quad * 32u) << 16) + acc * ACC_COLS + half * (tile_n / 2);
       uint32_t amax_bits = 0;
-      // Software pipeline over the warp's four 32 x 32 blocks: the tensor-memory load of block ch+1 is in flight
+      // Software pipeline over the warp's (up to four) 32 x 32 blocks: the tensor-memory load of block ch+1 is in flight
       // while block ch is scaled, written to shared memory and handed to the bulk-store unit.
       if (nch) tmem_ld32(t_row, r[0]);
 #pragma unroll
@@ -581,10 +536,7 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
       // accumulator drained: hand it back to the MMA warp
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) {
-        if (TWO) mbar_arrive_cluster(acc ? tempty_leader1 : tempty_leader0);  // the MMA issuer waits in the even CTA
-        else mbar_arrive(tempty_bar(acc));
-      }
+      if (lane == 0) mbar_arrive_cluster(acc ? tempty_leader1 : tempty_leader0);  // the MMA issuer waits in the even CTA
       if ((p.epi == 0 || p.epi == 3) && (p.amax_bits || p.amax_bits2)) {
         // two packed bf16 magnitudes -> FP32 bit pattern of the larger
         const uint32_t w = __reduce_max_sync(0xffffffffu, max(amax_bits & 0xffffu, amax_bits >> 16) << 16);
@@ -623,72 +575,88 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
     for (uint32_t i = 1; i < ps.count(); ++i)
       if (ps.status_of(i) && ps.status_of(i) != status) atomicOr(ps.status_of(i), bits);
   }
-  if (TWO) cluster_sync_all();  // no arrival may still be on its way to a CTA that has left
+  cluster_sync_all();  // no arrival may still be on its way to a CTA that has left
   if (warp == 1) {
     tc_fence_after();
-    if (TWO)
-      asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TMEM_COLS) : "memory");
-    else
-      asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TMEM_COLS) : "memory");
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TMEM_COLS) : "memory");
   }
 }
 
 #undef QE_TILE_PROBLEM
 
-__global__ void __launch_bounds__(THREADS, 1) gemm_fp8_kernel(const __grid_constant__ GemmParams p) {
-  gemm_body<false>(OneProblem{p});
-}
-
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
     gemm_fp8_pair_kernel(const __grid_constant__ GemmParams p) {
-  gemm_body<true>(OneProblem{p});
+  gemm_body(OneProblem{p});
 }
 
-// Up to eight independent GEMMs (each eligible for the paired variant) in one launch.
+// Up to eight independent GEMMs in one launch.
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
     gemm_fp8_pair_group_kernel(const __grid_constant__ GemmGroupParams g) {
-  gemm_body<true>(ProblemGroup{g});
+  gemm_body(ProblemGroup{g});
+}
+
+uint32_t tiles_of(const GemmDesc& d, uint32_t tile_n) { return ((d.M + TILE_M - 1) / TILE_M) * ((d.N + tile_n - 1) / tile_n); }
+
+// Columns per tile of a launch's problems (index into kTileWidths).  A tile's main loop takes 0.27 us per 128-byte K
+// block at ANY width (four dependent MMAs of ~128 clocks each), so width is free only as long as every CTA pair has a
+// tile; a launch that leaves pairs idle takes narrower tiles for their shorter epilogue: 256 columns against 64, back to
+// back, 5.0 -> 4.1 us (256 x 256 x 256), 7.4 -> 6.4 us (512 x 1024 x 1024, dI), 8.5 -> 6.6 us (1024 x 1024 x 512, FP32
+// accumulate); 256 against 128: 15.8 -> 14.7 us (256 x 8192 x 4096).  The narrowest only up to half the pairs: beyond,
+// the next launch's CTAs find no free SM to start on before this one ends (1024 x 1024 x 1024: 6.9 us at 128, 7.2 at 64).
+// More tiles than pairs lose at once (256 x 8192 x 4096 at 64 columns: 23.4 us).
+uint32_t choose_width(const GemmDesc* d, uint32_t n, uint32_t pairs) {
+  uint32_t w = 0;
+  while (w + 1 < kNumTileWidths) {
+    uint32_t tiles = 0;
+    for (uint32_t i = 0; i < n; ++i) tiles += tiles_of(d[i], kTileWidths[w + 1]);
+    if (tiles > (w == 0 ? pairs : pairs / 2)) break;
+    ++w;
+  }
+  return w;
+}
+
+// The device's parameter block of one problem at a tile width.
+void fill_problem(const GemmDesc& d, uint32_t w, GemmParams* p) {
+  *p = d;
+  const uint32_t tile_n = kTileWidths[w], per_cta = tile_n / 2;
+  p->tmA = *d.mapA;
+  p->tmB = d.mapB[w];
+  p->tile_n = tile_n;
+  // bits 4-5: accumulator format (1 = FP32); 7-9 / 10-12: A / B format (0 = E4M3, 1 = E5M2); 15 / 16: A / B major
+  // (0 = contraction-major); 17-22: N >> 3; 24-28: M >> 4 (256 for a CTA pair).
+  p->idesc = (1u << 4) | (d.a_fmt << 7) | (d.b_fmt << 10) | (d.a_mn << 15) | (d.b_mn << 16) | ((tile_n >> 3) << 17) | ((TILE_M >> 4) << 24);
+  // An MN-major B tile has rows of per_cta bytes, swizzled over exactly that width; a contraction-major one rows of 128.
+  const uint32_t row = d.b_mn ? per_cta : 128u;
+  p->b_desc_hi = desc_hi(row);
+  p->b_step = d.b_mn ? 32u * row / 16u : 2u;
 }
 
 }  // namespace
 
 bool gemm_uses_pair(uint32_t M) { return M % 256 == 0; }
 
-uint32_t gemm_b_box_rows(uint32_t M) { return gemm_uses_pair(M) ? 128u : 256u; }
-
-uint32_t gemm_idesc(int a_fmt, int b_fmt, uint32_t M, bool a_mn, bool b_mn) {
-  // bits 4-5: accumulator format (1 = FP32); 7-9 / 10-12: A / B format (0 = E4M3, 1 = E5M2); 15 / 16: A / B major
-  // (0 = contraction-major); 17-22: N >> 3; 24-28: M >> 4 (128 per CTA, 256 for a CTA pair).
-  const uint32_t mma_m = gemm_uses_pair(M) ? 256u : 128u;
-  return (1u << 4) | ((uint32_t)a_fmt << 7) | ((uint32_t)b_fmt << 10) | ((a_mn ? 1u : 0u) << 15) |
-         ((b_mn ? 1u : 0u) << 16) | ((uint32_t)(BN >> 3) << 17) | ((mma_m >> 4) << 24);
-}
-
 cudaError_t gemm_prepare() {
-  cudaError_t e = cudaFuncSetAttribute((const void*)gemm_fp8_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)SMEM_BYTES);
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute((const void*)gemm_fp8_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES);
+  cudaError_t e = cudaFuncSetAttribute((const void*)gemm_fp8_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES);
   if (e != cudaSuccess) return e;
   return cudaFuncSetAttribute((const void*)gemm_fp8_pair_group_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               (int)SMEM_BYTES);
 }
 
-bool make_gemm_group(const GemmParams* probs, uint32_t n, int num_sms, Launch* out) {
+bool make_gemm_group(const GemmDesc* probs, uint32_t n, int num_sms, Launch* out) {
   if (n < 2 || n > 8) return false;
   GemmGroupParams g{};
+  const uint32_t pairs = (uint32_t)num_sms / 2u, w = choose_width(probs, n, pairs);
   uint32_t tiles = 0;
   for (uint32_t i = 0; i < n; ++i) {
-    if (!gemm_uses_pair(probs[i].M)) return false;  // paired variant only
-    tiles += (probs[i].M / 256u) * ((probs[i].N + BN - 1) / BN);
+    if (!gemm_uses_pair(probs[i].M)) return false;
+    tiles += tiles_of(probs[i], kTileWidths[w]);
     g.tile_end[i] = tiles;
-    g.prob[i] = probs[i];
+    fill_problem(probs[i], w, &g.prob[i]);
   }
   g.n = n;
   Launch l;
   l.func = (const void*)gemm_fp8_pair_group_kernel;
-  const uint32_t ctas = 2u * tiles, cap = (uint32_t)num_sms & ~1u;
-  l.grid = dim3(ctas < cap ? ctas : cap, 1, 1);
+  l.grid = dim3(2u * (tiles < pairs ? tiles : pairs), 1, 1);
   l.block = dim3(THREADS, 1, 1);
   l.smem = SMEM_BYTES;
   l.set(g);
@@ -696,21 +664,13 @@ bool make_gemm_group(const GemmParams* probs, uint32_t n, int num_sms, Launch* o
   return true;
 }
 
-Launch make_gemm(const GemmParams& p, int num_sms) {
+Launch make_gemm(const GemmDesc& d, int num_sms) {
+  const uint32_t pairs = (uint32_t)num_sms / 2u, w = choose_width(&d, 1, pairs), tiles = tiles_of(d, kTileWidths[w]);
+  GemmParams p;
+  fill_problem(d, w, &p);
   Launch l;
-  if (gemm_uses_pair(p.M)) {
-    l.func = (const void*)gemm_fp8_pair_kernel;
-    const uint32_t ctas = 2u * (p.M / 256u) * ((p.N + BN - 1) / BN);
-    const uint32_t cap = (uint32_t)num_sms & ~1u;
-    l.grid = dim3(ctas < cap ? ctas : cap, 1, 1);
-    l.block = dim3(THREADS, 1, 1);
-    l.smem = SMEM_BYTES;
-    l.set(p);
-    return l;
-  }
-  l.func = (const void*)gemm_fp8_kernel;
-  const uint32_t tiles = (p.M / BM) * ((p.N + BN - 1) / BN);
-  l.grid = dim3(tiles < (uint32_t)num_sms ? tiles : (uint32_t)num_sms, 1, 1);
+  l.func = (const void*)gemm_fp8_pair_kernel;
+  l.grid = dim3(2u * (tiles < pairs ? tiles : pairs), 1, 1);
   l.block = dim3(THREADS, 1, 1);
   l.smem = SMEM_BYTES;
   l.set(p);

@@ -87,13 +87,19 @@ struct ArenaReduceParams {
   uint32_t pad;
 };
 
+// Tile widths the GEMM can be run with: the B operand's TMA box has half as many rows (each CTA of a pair loads half).
+constexpr uint32_t kNumTileWidths = 3;
+constexpr uint32_t kTileWidths[kNumTileWidths] = {256, 128, 64};
+
 struct GemmParams {
-  CUtensorMap tmA;             // A [M, Kc] bytes, box 128 x 128, 128-byte swizzle
-  CUtensorMap tmB;             // B [N, Kc] bytes, box 128 x gemm_b_box_rows(M)
+  CUtensorMap tmA;             // A: 128 rows x 128 contraction bytes, 128-byte swizzle
+  CUtensorMap tmB;             // B: tile_n / 2 rows x 128 contraction bytes (MN-major: swizzled over tile_n / 2 bytes)
   CUtensorMap tmD;             // D [M, N] (bf16, FP32 or FP8 bytes), box 32 x 32, for the epilogue's bulk stores
   uint32_t M, N, Kc;
+  uint32_t tile_n;             // columns per tile
   uint32_t idesc;              // tcgen05 instruction descriptor (formats, majors, shape)
-  uint32_t a_mn, b_mn;         // operand given MN-major (as [Kc, M] / [Kc, N] bytes): paired variant only
+  uint32_t b_desc_hi, b_step;  // B's shared-memory descriptor: high word; address advance (16-byte units) per 32 contraction elements
+  uint32_t a_mn, b_mn;         // operand given MN-major (as [Kc, M] / [Kc, N] bytes)
   const float* alpha_a;
   const float* alpha_b;
   void* out;                   // bf16 or FP32 [M, N], row pitch ldo elements
@@ -113,10 +119,18 @@ struct GemmParams {
   CommitParams commit;         // performed by the last CTA to finish (commit.st != null)
 };
 
+// One GEMM as the launch builders take it: everything the kernel needs except what follows from the tile width, which
+// the launch chooses (tmA, tmB, tile_n, idesc, b_desc_hi and b_step are filled from the fields below).
+struct GemmDesc : GemmParams {
+  uint32_t a_fmt, b_fmt;       // 0 = E4M3, 1 = E5M2
+  const CUtensorMap* mapA;
+  const CUtensorMap* mapB;     // one map per tile width
+};
+
 // Up to eight independent GEMMs computed by one launch: tiles are numbered problem after problem.
 struct GemmGroupParams {
   uint32_t n;
-  uint32_t tile_end[8];        // cumulative tile counts (256 x 256 tiles)
+  uint32_t tile_end[8];        // cumulative tile counts
   uint32_t pad[7];
   GemmParams prob[8];
 };
@@ -152,14 +166,12 @@ Launch make_amax_pass1(const AmaxParams& p);
 Launch make_amax_pass2(const AmaxParams& p);
 Launch make_accumulate(const AccumParams& p);
 Launch make_arena_reduce(const ArenaReduceParams& p);
-Launch make_gemm(const GemmParams& p, int num_sms);
-// One launch for n = 2..8 GEMMs (each may carry its own commit tail); false if the group cannot be formed (a problem
-// needs the single-CTA variant), in which case the caller launches them one by one.
-bool make_gemm_group(const GemmParams* probs, uint32_t n, int num_sms, Launch* out);
+Launch make_gemm(const GemmDesc& p, int num_sms);
+// One launch for n = 2..8 GEMMs (each may carry its own commit tail); false if the group cannot be formed (a problem's M
+// is not a multiple of 256), in which case the caller launches them one by one.
+bool make_gemm_group(const GemmDesc* probs, uint32_t n, int num_sms, Launch* out);
 cudaError_t gemm_prepare();  // opt in to the dynamic shared memory the GEMM needs (once per device)
-uint32_t gemm_idesc(int a_fmt, int b_fmt, uint32_t M, bool a_mn = false, bool b_mn = false);
-bool gemm_uses_pair(uint32_t M);
-uint32_t gemm_b_box_rows(uint32_t M);  // rows of the B operand's TMA box for a GEMM with M rows (128 paired, 256 single)
+bool gemm_uses_pair(uint32_t M);  // whole 256-row tiles: may share launches and take MN-major operands
 constexpr uint32_t kAmaxPartials = 2048;
 
 }  // namespace qe

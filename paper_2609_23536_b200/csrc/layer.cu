@@ -108,15 +108,15 @@ int32_t qe_layer_create(qe_ctx* ctx, const qe_layer_config* cfg, void* ws, uint6
     if ((st = make_map(d, &L->tmGq_A[p], L->Gq[p], T, N, 128)) != QE_OK) break;   // dI: A = Gq  [T,N]
     if (xgT) {
       if ((st = make_map(d, &L->tmGqT_A[p], L->GqT[p], N, T, 128)) != QE_OK) break; // dW: A = Gq^T [N,T]
-      if ((st = make_map(d, &L->tmXqT_B[p], L->XqT[p], K, T, qe::gemm_b_box_rows(N))) != QE_OK) break; // dW: B = Xq^T [K,T]
-    } else {  // dW reads Gq [T,N] and Xq [T,K] as MN-major operands: 128 x 128 boxes over the row-major tensors
+      if ((st = make_b_maps(d, L->tmXqT_B[p], L->XqT[p], K, T, false)) != QE_OK) break; // dW: B = Xq^T [K,T]
+    } else {  // dW reads Gq [T,N] and Xq [T,K] as MN-major operands, over the row-major tensors
       if ((st = make_map(d, &L->tmGqT_A[p], L->Gq[p], T, N, 128)) != QE_OK) break;
-      if ((st = make_map(d, &L->tmXqT_B[p], L->Xq[p], T, K, 128)) != QE_OK) break;
+      if ((st = make_b_maps(d, L->tmXqT_B[p], L->Xq[p], K, T, true)) != QE_OK) break;
     }
   }
-  if (st == QE_OK) st = make_map(d, &L->tmWq_B, L->Wq, N, K, qe::gemm_b_box_rows(T));    // F:  B = Wq   [N,K]
+  if (st == QE_OK) st = make_b_maps(d, L->tmWq_B, L->Wq, N, K, false);    // F:  B = Wq   [N,K]
   if (st == QE_OK)  // dI: B = Wq^T [K,N], or Wq [N,K] itself as an MN-major operand
-    st = wT ? make_map(d, &L->tmWqT_B, L->WqT, K, N, qe::gemm_b_box_rows(T)) : make_map(d, &L->tmWq_B_mn, L->Wq, N, K, 128);
+    st = wT ? make_b_maps(d, L->tmWq_dI, L->WqT, K, N, false) : make_b_maps(d, L->tmWq_dI, L->Wq, K, N, true);
   if (st != QE_OK) { qe_contract_destroy(L->contract); delete L; return st; }
   // state: histories 0, scales 1, everything else 0
   qe::DevState init{};

@@ -29,17 +29,29 @@ int32_t device_info(int device, DeviceInfo** out) {
   return QE_OK;
 }
 
-// Tensor map over a contraction-major byte matrix [rows, inner]: box = 128 bytes x box_rows, 128-byte swizzle.
+// Tensor map over a row-major byte matrix [rows, inner]: box = box_rows x box_inner bytes (128, 64 or 32), swizzled over
+// box_inner.
 int32_t make_map(const DeviceInfo* d, CUtensorMap* map, const void* ptr, uint64_t rows, uint64_t inner,
-                 uint32_t box_rows) {
+                 uint32_t box_rows, uint32_t box_inner) {
   cuuint64_t gdim[2] = {inner, rows};
   cuuint64_t gstride[1] = {inner};
-  cuuint32_t box[2] = {128u, box_rows};
+  cuuint32_t box[2] = {box_inner, box_rows};
   cuuint32_t estr[2] = {1u, 1u};
+  const CUtensorMapSwizzle sw = box_inner == 128u ? CU_TENSOR_MAP_SWIZZLE_128B : box_inner == 64u ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B;
   CUresult r = d->encode(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, const_cast<void*>(ptr), gdim, gstride, box, estr,
-                         CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                         CU_TENSOR_MAP_INTERLEAVE_NONE, sw, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) return fail(QE_ERR_CUDA, "cuTensorMapEncodeTiled failed with %d", (int)r);
+  return QE_OK;
+}
+
+// The maps of a GEMM's B operand, one per tile width: contraction-major [N, Kc], or (mn) the operand given as [Kc, N].
+int32_t make_b_maps(const DeviceInfo* d, CUtensorMap* maps, const void* ptr, uint64_t N, uint64_t Kc, bool mn) {
+  for (uint32_t w = 0; w < qe::kNumTileWidths; ++w) {
+    const uint32_t per_cta = qe::kTileWidths[w] / 2;
+    const int32_t st = mn ? make_map(d, &maps[w], ptr, Kc, N, 128, per_cta) : make_map(d, &maps[w], ptr, N, Kc, per_cta);
+    if (st != QE_OK) return st;
+  }
   return QE_OK;
 }
 
@@ -428,17 +440,17 @@ void add_refresh(qe_layer* L, std::vector<qe::Launch>& ls) {
 // inverse-scale snapshot), so `next` needs no cast kernel; x == null means L's own input was deposited that way.
 // gemm_out != null: the GEMM is handed back instead of being queued (the caller puts it into a shared launch).
 void add_forward(qe_layer* L, uint32_t p, const void* x, void* y, std::vector<qe::Launch>& ls, qe_layer* next,
-                 uint32_t pn, qe::GemmParams* gemm_out, qe::QuantParams* cast_out) {
+                 uint32_t pn, qe::GemmDesc* gemm_out, qe::QuantParams* cast_out) {
   const uint32_t T = L->cfg.T, K = L->cfg.K, N = L->cfg.N;
   if (x && cast_out) *cast_out = quant_params(L, x, L->Xq[p], L->XqT[p], T, K, QE_CLASS_X, &L->st->slot_sinv_X[p], QE_E4M3);
   else if (x) ls.push_back(quant_launch(L, x, L->Xq[p], L->XqT[p], T, K, QE_CLASS_X, &L->st->slot_sinv_X[p], QE_E4M3));
-  qe::GemmParams gp{};
-  gp.tmA = L->tmXq_A[p];
-  gp.tmB = L->tmWq_B;
+  qe::GemmDesc gp{};
+  gp.mapA = &L->tmXq_A[p];
+  gp.mapB = L->tmWq_B;
   gp.M = T;
   gp.N = N;
   gp.Kc = K;
-  gp.idesc = qe::gemm_idesc(QE_E4M3, QE_E4M3, T);
+  gp.a_fmt = gp.b_fmt = QE_E4M3;
   gp.alpha_a = &L->st->slot_sinv_X[p];
   gp.alpha_b = &L->st->cache_sinv_W;
   gp.ldo = N;
@@ -467,18 +479,19 @@ void add_forward(qe_layer* L, uint32_t p, const void* x, void* y, std::vector<qe
 // Hand-off in the backward direction: the input gradient of `L` is the output gradient of the linear before it
 // (`prev`), emitted as E5M2 with prev's G scale into prev's tape slot pp; dy == null: L's own dY came that way.
 void add_dI(qe_layer* L, uint32_t p, const void* dy, void* dx, std::vector<qe::Launch>& ls, qe_layer* prev,
-            uint32_t pp, qe::GemmParams* gemm_out, qe::QuantParams* cast_out) {
+            uint32_t pp, qe::GemmDesc* gemm_out, qe::QuantParams* cast_out) {
   const uint32_t T = L->cfg.T, K = L->cfg.K, N = L->cfg.N;
   if (dy && cast_out) *cast_out = quant_params(L, dy, L->Gq[p], L->GqT[p], T, N, QE_CLASS_G, &L->st->slot_sinv_G[p], QE_E5M2);
   else if (dy) ls.push_back(quant_launch(L, dy, L->Gq[p], L->GqT[p], T, N, QE_CLASS_G, &L->st->slot_sinv_G[p], QE_E5M2));
-  qe::GemmParams gp{};
+  qe::GemmDesc gp{};
   const bool b_mn = L->WqT == nullptr;  // no transposed weight copy: Wq [N,K] is B in MN-major form
-  gp.tmA = L->tmGq_A[p];
-  gp.tmB = b_mn ? L->tmWq_B_mn : L->tmWqT_B;
+  gp.mapA = &L->tmGq_A[p];
+  gp.mapB = L->tmWq_dI;
   gp.M = T;
   gp.N = K;
   gp.Kc = N;
-  gp.idesc = qe::gemm_idesc(QE_E5M2, QE_E4M3, T, false, b_mn);
+  gp.a_fmt = QE_E5M2;
+  gp.b_fmt = QE_E4M3;
   gp.b_mn = b_mn;
   gp.alpha_a = &L->st->slot_sinv_G[p];
   gp.alpha_b = &L->st->cache_sinv_W;
@@ -507,16 +520,17 @@ void add_dI(qe_layer* L, uint32_t p, const void* dy, void* dx, std::vector<qe::L
 
 // The weight-gradient GEMM of slot p; dst = first element of the layer's gradient slice, temp != null makes it
 // write the temporary instead (copied-gradient comparison path).
-qe::GemmParams dW_gemm(qe_layer* L, uint32_t p, float* dst, int32_t accumulate, float* temp) {
+qe::GemmDesc dW_gemm(qe_layer* L, uint32_t p, float* dst, int32_t accumulate, float* temp) {
   const uint32_t T = L->cfg.T, K = L->cfg.K, N = L->cfg.N;
-  qe::GemmParams gp{};
+  qe::GemmDesc gp{};
   const bool mn = L->GqT[p] == nullptr;  // Gq [T,N] and Xq [T,K] themselves, read as MN-major operands
-  gp.tmA = L->tmGqT_A[p];
-  gp.tmB = L->tmXqT_B[p];
+  gp.mapA = &L->tmGqT_A[p];
+  gp.mapB = L->tmXqT_B[p];
   gp.M = N;
   gp.N = K;
   gp.Kc = T;
-  gp.idesc = qe::gemm_idesc(QE_E5M2, QE_E4M3, N, mn, mn);
+  gp.a_fmt = QE_E5M2;
+  gp.b_fmt = QE_E4M3;
   gp.a_mn = gp.b_mn = mn;
   gp.alpha_a = &L->st->slot_sinv_G[p];  // snapshots taken when dY_m and X_m were quantised, never the current state
   gp.alpha_b = &L->st->slot_sinv_X[p];
@@ -535,8 +549,8 @@ qe::GemmParams dW_gemm(qe_layer* L, uint32_t p, float* dst, int32_t accumulate, 
 }
 
 // Per-microbatch arena: the same GEMM writes bf16(D) into the microbatch's own view (no accumulation, no amax).
-qe::GemmParams dW_gemm_view(qe_layer* L, uint32_t p, void* view) {
-  qe::GemmParams gp = dW_gemm(L, p, nullptr, 0, nullptr);
+qe::GemmDesc dW_gemm_view(qe_layer* L, uint32_t p, void* view) {
+  qe::GemmDesc gp = dW_gemm(L, p, nullptr, 0, nullptr);
   gp.out = view;
   gp.epi = 0;
   make_out_map(L->ctx->dev, &gp.tmD, view, L->cfg.N, L->cfg.K, L->cfg.K, false);

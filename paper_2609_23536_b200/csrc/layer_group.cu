@@ -180,7 +180,7 @@ int32_t qe_forward_dI_pair(qe_layer* Lf, uint32_t mb, uint64_t gen, const void* 
   }
   std::vector<qe::Launch> ls;
   if (refresh) add_refresh(Lf, ls);
-  qe::GemmParams g[2];
+  qe::GemmDesc g[2];
   qe::QuantParams c[2];
   add_forward(Lf, p, x, y, ls, nullptr, 0, &g[0], &c[0]);  // hands the casts and the GEMMs back
   add_dI(Lb, pb, dy, dx, ls, nullptr, 0, &g[1], &c[1]);
@@ -189,7 +189,7 @@ int32_t qe_forward_dI_pair(qe_layer* Lf, uint32_t mb, uint64_t gen, const void* 
   if (qe::make_gemm_group(g, 2, ctx->dev->num_sms, &shared)) {
     ls.push_back(shared);
     ctx->stats.paired_f_di += 1;
-  } else {  // a shape that needs the single-CTA variant: one after the other
+  } else {  // T is an odd multiple of 128: one after the other
     ls.push_back(qe::make_gemm(g[0], ctx->dev->num_sms));
     ls.push_back(qe::make_gemm(g[1], ctx->dev->num_sms));
   }
@@ -246,19 +246,19 @@ int32_t together_prepare(qe_ctx* ctx, const qe_action* acts, uint32_t n, float* 
   return QE_OK;
 }
 
-// the launches: the casts in one launch, then every GEMM that can run on the paired variant in one launch
+// the launches: the casts in one launch, then every GEMM of whole 256-row tiles in one launch
 int32_t together_build(qe_ctx* ctx, const qe_action* acts, uint32_t n, const TogetherPrep& pr, float* grad,
                        std::vector<qe::Launch>& ls, Fnv* h) {
-  qe::GemmParams g[QE_MAX_TOGETHER];
+  qe::GemmDesc g[QE_MAX_TOGETHER];
   qe::QuantParams casts[QE_MAX_TOGETHER];
-  std::vector<qe::GemmParams> singles;
+  std::vector<qe::GemmDesc> singles;
   uint32_t ng = 0, n_chain = 0, n_dw = 0, n_casts = 0;
   for (int pass = 0; pass < 2; ++pass) {  // F and dI first (others wait for them), the weight gradients' tiles after theirs
     for (uint32_t i = 0; i < n; ++i) {
       const qe_action& a = acts[i];
       qe_layer* L = a.layer;
       if ((a.kind == QE_ACT_DW) != (pass == 1)) continue;
-      qe::GemmParams gp;
+      qe::GemmDesc gp;
       if (a.kind == QE_ACT_F) {
         if (L->dw_pending[pr.slot[i]]) {
           QE_CUDA(cudaStreamWaitEvent(ctx->exec_stream, L->ev_dw[pr.slot[i]], 0));
@@ -275,7 +275,7 @@ int32_t together_build(qe_ctx* ctx, const qe_action* acts, uint32_t n, const Tog
         g[ng++] = gp;
         (a.kind == QE_ACT_DW ? n_dw : n_chain) += 1;
       } else {
-        singles.push_back(gp);  // single-CTA variant: a launch of its own
+        singles.push_back(gp);  // a half-filled last row tile: a launch of its own
       }
       if (h) {
         h->mix(&a.kind, sizeof(a.kind));
@@ -287,11 +287,11 @@ int32_t together_build(qe_ctx* ctx, const qe_action* acts, uint32_t n, const Tog
   }
   // longest tiles first (their contraction length decides a tile's duration): the launch's last, partial wave is then
   // made of short tiles.  The weight gradients (contraction over T only) stay behind the others.
-  std::stable_sort(g, g + n_chain, [](const qe::GemmParams& x, const qe::GemmParams& y) { return x.Kc > y.Kc; });
-  std::stable_sort(g + n_chain, g + ng, [](const qe::GemmParams& x, const qe::GemmParams& y) { return x.Kc > y.Kc; });
+  std::stable_sort(g, g + n_chain, [](const qe::GemmDesc& x, const qe::GemmDesc& y) { return x.Kc > y.Kc; });
+  std::stable_sort(g + n_chain, g + ng, [](const qe::GemmDesc& x, const qe::GemmDesc& y) { return x.Kc > y.Kc; });
   if (n_casts >= 2) ls.push_back(qe::make_quantize_multi(casts, n_casts));  // all casts of the call in one launch
   else if (n_casts == 1) ls.push_back(qe::make_quantize(casts[0]));
-  for (const qe::GemmParams& gp : singles) ls.push_back(qe::make_gemm(gp, ctx->dev->num_sms));
+  for (const qe::GemmDesc& gp : singles) ls.push_back(qe::make_gemm(gp, ctx->dev->num_sms));
   qe::Launch shared;
   if (ng >= 2 && qe::make_gemm_group(g, ng, ctx->dev->num_sms, &shared)) {
     ls.push_back(shared);

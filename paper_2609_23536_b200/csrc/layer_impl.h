@@ -37,7 +37,9 @@ struct DeviceInfo {
 
 int32_t device_info(int device, DeviceInfo** out);
 int32_t current_device_info(DeviceInfo** d);
-int32_t make_map(const DeviceInfo* d, CUtensorMap* map, const void* ptr, uint64_t rows, uint64_t inner, uint32_t box_rows);
+int32_t make_map(const DeviceInfo* d, CUtensorMap* map, const void* ptr, uint64_t rows, uint64_t inner, uint32_t box_rows,
+                 uint32_t box_inner = 128);
+int32_t make_b_maps(const DeviceInfo* d, CUtensorMap* maps, const void* ptr, uint64_t N, uint64_t Kc, bool mn);
 int32_t make_out_map(const DeviceInfo* d, CUtensorMap* map, const void* ptr, uint64_t M, uint64_t N, uint64_t ldo, bool fp32);
 int32_t make_out_map_u8(const DeviceInfo* d, CUtensorMap* map, const void* ptr, uint64_t M, uint64_t N, uint64_t ld);
 inline uint64_t align_up(uint64_t v, uint64_t a) { return (v + a - 1) / a * a; }
@@ -90,9 +92,9 @@ struct qe_layer {
   uint8_t *Wq = nullptr, *WqT = nullptr;
   uint8_t *x_stage = nullptr, *dx_stage = nullptr, *y_stage = nullptr, *dy_stage = nullptr;  // host_io only
   uint8_t *Xq[QE_MAX_SLOTS], *XqT[QE_MAX_SLOTS], *Gq[QE_MAX_SLOTS], *GqT[QE_MAX_SLOTS];
-  // tensor maps: A-role boxes are 128 rows, B-role boxes 256 rows
-  CUtensorMap tmXq_A[QE_MAX_SLOTS], tmGq_A[QE_MAX_SLOTS], tmGqT_A[QE_MAX_SLOTS], tmXqT_B[QE_MAX_SLOTS];
-  CUtensorMap tmWq_B, tmWqT_B, tmWq_B_mn;
+  // tensor maps: one per tensor in the A role, one per tile width in the B role
+  CUtensorMap tmXq_A[QE_MAX_SLOTS], tmGq_A[QE_MAX_SLOTS], tmGqT_A[QE_MAX_SLOTS], tmXqT_B[QE_MAX_SLOTS][qe::kNumTileWidths];
+  CUtensorMap tmWq_B[qe::kNumTileWidths], tmWq_dI[qe::kNumTileWidths];  // B of the forward; B of dI (Wq^T, or Wq MN-major)
   ActionGraph gF[QE_MAX_SLOTS], gDI[QE_MAX_SLOTS], gDW[QE_MAX_SLOTS], gDWs[QE_MAX_SLOTS], gRefresh, gCommit;
   // QE_CTX_OVERLAP_DW: per slot, "dI of the tape in this slot has been enqueued" / "the dW that released it has"
   cudaEvent_t ev_di[QE_MAX_SLOTS] = {}, ev_dw[QE_MAX_SLOTS] = {};
@@ -131,18 +133,18 @@ qe::Launch quant_launch(qe_layer* L, const void* x, uint8_t* q, uint8_t* qT, uin
                         float* sinv_dst, int fmt, uint32_t commit_mask = 0);
 void add_refresh(qe_layer* L, std::vector<qe::Launch>& ls);
 void add_forward(qe_layer* L, uint32_t p, const void* x, void* y, std::vector<qe::Launch>& ls, qe_layer* next = nullptr,
-                 uint32_t pn = 0, qe::GemmParams* gemm_out = nullptr, qe::QuantParams* cast_out = nullptr);
+                 uint32_t pn = 0, qe::GemmDesc* gemm_out = nullptr, qe::QuantParams* cast_out = nullptr);
 void add_dI(qe_layer* L, uint32_t p, const void* dy, void* dx, std::vector<qe::Launch>& ls, qe_layer* prev = nullptr,
-            uint32_t pp = 0, qe::GemmParams* gemm_out = nullptr, qe::QuantParams* cast_out = nullptr);
-qe::GemmParams dW_gemm(qe_layer* L, uint32_t p, float* dst, int32_t accumulate, float* temp);
-qe::GemmParams dW_gemm_view(qe_layer* L, uint32_t p, void* view);
+            uint32_t pp = 0, qe::GemmDesc* gemm_out = nullptr, qe::QuantParams* cast_out = nullptr);
+qe::GemmDesc dW_gemm(qe_layer* L, uint32_t p, float* dst, int32_t accumulate, float* temp);
+qe::GemmDesc dW_gemm_view(qe_layer* L, uint32_t p, void* view);
 void add_dW(qe_layer* L, uint32_t p, float* dst, int32_t accumulate, float* temp, std::vector<qe::Launch>& ls);
 
 // Weight-gradient GEMMs of different layers that follow one another share one launch where the kernel allows it
 // (all on the paired variant): the persistent CTAs pack their tiles into common waves and the launch is paid once.
 // The layers' gradient slices are disjoint (destination registry), so the GEMMs are independent.
 struct DWBatch {
-  qe::GemmParams gp[4];
+  qe::GemmDesc gp[4];
   qe_layer* layer[4];
   uint32_t n = 0;
   bool has(const qe_layer* L) const {
@@ -151,7 +153,7 @@ struct DWBatch {
     return false;
   }
   void flush(qe_ctx* ctx, std::vector<qe::Launch>& ls) {
-    qe::GemmParams paired[4];
+    qe::GemmDesc paired[4];
     uint32_t np = 0;
     for (uint32_t i = 0; i < n; ++i)
       if (qe::gemm_uses_pair(gp[i].M)) paired[np++] = gp[i];
@@ -165,7 +167,7 @@ struct DWBatch {
       if (!grouped || !qe::gemm_uses_pair(gp[i].M)) ls.push_back(qe::make_gemm(gp[i], ctx->dev->num_sms));
     n = 0;
   }
-  void add(qe_ctx* ctx, qe_layer* L, const qe::GemmParams& g, std::vector<qe::Launch>& ls) {
+  void add(qe_ctx* ctx, qe_layer* L, const qe::GemmDesc& g, std::vector<qe::Launch>& ls) {
     if (n == 4 || has(L)) flush(ctx, ls);  // a layer's own GEMMs accumulate into one slice: never in one launch
     gp[n] = g;
     layer[n++] = L;

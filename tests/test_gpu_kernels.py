@@ -223,6 +223,36 @@ def test_gemm_mn_major_needs_the_paired_variant(qe):
     assert e.value.code == "UNSUPPORTED"
 
 
+# Tile widths 64, 128 and 256 (by how many tiles the shape gives), whole and half-filled last row tiles, every operand
+# major; the last shape reaches the next wider tile by one row tile.
+@pytest.mark.parametrize("M,Nn", [(128, 256), (256, 2048), (640, 768), (1024, 1152), (1024, 2048), (1152, 1920), (2048, 2048), (2304, 2176)])
+@pytest.mark.parametrize("a_mn,b_mn", [(False, False), (False, True), (True, True)])
+def test_gemm_tile_widths_and_half_filled_row_tiles_integer_exact(qe, M, Nn, a_mn, b_mn):
+    if (a_mn or b_mn) and M % 256:
+        pytest.skip("MN-major operands need whole row tiles")
+    rng = np.random.default_rng(M + Nn + 2 * a_mn + b_mn)
+    Kc = 384
+    A, Av = _int_codes(rng, (M, Kc), 8, fp8.E5M2)
+    B, Bv = _int_codes(rng, (Nn, Kc), 4, fp8.E4M3)
+    want = (Av.astype(np.float64) @ Bv.astype(np.float64).T).astype(np.float32)  # integers below 2^24: exact in any order
+    Ad = torch.from_numpy(np.ascontiguousarray(A.T) if a_mn else A).to(DEV)
+    Bd = torch.from_numpy(np.ascontiguousarray(B.T) if b_mn else B).to(DEV)
+    one = torch.ones(1, device=DEV)
+    status = torch.zeros(1, dtype=torch.int32, device=DEV)
+    amax = torch.zeros(1, device=DEV)
+    guard = torch.full((M + 128, Nn), 7.0, device=DEV)  # rows beyond M must stay as they are
+    bf = torch.full((M + 128, Nn), 7.0, dtype=torch.bfloat16, device=DEV)
+    qe.qe_gemm_fp8_ex(Ad, 1, a_mn, Bd, 0, b_mn, one, one, guard[:M], 1, None, status)
+    qe.qe_gemm_fp8_ex(Ad, 1, a_mn, Bd, 0, b_mn, one, one, guard[:M], 2, None, status)
+    qe.qe_gemm_fp8_ex(Ad, 1, a_mn, Bd, 0, b_mn, one, one, bf[:M], 0, amax, status)
+    torch.cuda.synchronize()
+    assert status.item() == 0
+    assert np.array_equal(guard[:M].cpu().numpy(), want + want) and bool((guard[M:] == 7.0).all())
+    wb = bf16.round_from_f64(want.astype(np.float64))
+    assert np.array_equal(inputs.bits(bf[:M].cpu()), wb) and bool((bf[M:] == 7.0).all())
+    assert amax.item() == float(np.abs(bf16.decode(wb)).max())
+
+
 # ------------------------------------------------------------------------------------------ arena reduction
 @pytest.mark.parametrize("M,n", [(1, 8), (2, 8 * 300), (5, 8 * 1031), (8, 1 << 20), (64, 8 * 512)])
 def test_arena_reduce_adds_views_in_order(qe, M, n):
