@@ -347,15 +347,18 @@ int32_t qe_next_slot(const qe_layer*, uint32_t* slot_out);
  * differ from the previous replay.  dW runs on the execution stream here (QE_CTX_OVERLAP_DW does not apply).
  * Independent actions share launches, with bit-identical results (only the slot a tape lands in may differ from the
  * one-by-one order).  The list is read as units -- runs of actions of one kind and microbatch over distinct layers: a
- * forward, input-gradient or weight-gradient unit of the stage -- and cut into rounds of up to QE_MAX_TOGETHER actions
- * whose predecessors were issued in earlier rounds (the previous layer of the own unit for F and dI, the same layer of
- * the previous unit of the kind, F before dI before dW of a (layer, microbatch), a free tape slot), looking
- * qe_ctx_config.step_window units ahead of the earliest unfinished one; a round is issued as qe_run_together would.
+ * forward, input-gradient or weight-gradient unit of the stage -- and cut into rounds of actions whose predecessors were
+ * issued in earlier rounds (the previous layer of the own unit for F and dI, the same layer's previous action of the
+ * kind, F before dI before dW of a (layer, microbatch), a free tape slot): up to QE_MAX_TOGETHER F and dI actions,
+ * looking qe_ctx_config.step_window F and dI units ahead of the earliest unfinished one.  A layer's weight gradients
+ * wait until a forward needs one of their slots, or no more are to come, or there are enough of them; those that are
+ * ready then go out in one launch that adds their products up in microbatch order and writes the gradient slice once
+ * (bit for bit what one accumulating launch per microbatch leaves there).  A round is issued as qe_run_together would.
  * With temp_dev, with step_window 1, or when the list admits no such plan, actions go one by one and only
  * consecutive dW actions of different layers share launches (as in qe_backward_dW_multi).
  * (The plan honours dependencies, not positions: an action listed before a predecessor that lies within the look-ahead
  * simply runs after it.)
- * If a check fails at action k (the first action of the failing round), the kernels issued so far still run (device and host state stay in step),
+ * If a check fails at action k, the kernels issued so far still run (device and host state stay in step),
  * then every layer of the list is aborted as at a failure boundary (Sec. 4.5) and the failing check's status is
  * returned; qe_arena_rebuild restarts the epoch. */
 typedef struct qe_step_action { uint32_t kind; uint32_t layer; uint32_t mb; uint32_t reserved; } qe_step_action;
@@ -364,11 +367,18 @@ typedef struct qe_step_io { const void* x_dev; void* y_dev; const void* dy_dev; 
 int32_t qe_step_run(qe_ctx* ctx, qe_layer* const* layers, uint32_t n_layers, const qe_step_action* actions,
                     uint32_t n_actions, uint32_t microbatches, const qe_step_io* io, float* grad_buf_dev,
                     uint64_t grad_buf_elems, const uint64_t* offsets, float* temp_dev, void* caller_stream);
-/* The issue plan qe_step_run makes, as host logic of its own (no device needed): cuts actions[0..n) into rounds as
- * described above.  slots[l]: tape slots of layer l; live_now[l]: tapes of layer l alive before the list (NULL: none);
- * window >= 1 units of look-ahead; max_group actions per round.  round_of_action[i] receives the round of action i
- * (rounds are numbered from 0 in issue order), *n_rounds_out their number.  ORDER if the list admits no plan (an
- * action whose predecessors never become ready, or a pool too small), BAD_ARG for a malformed action. */
+/* Issue plans as host logic of their own (no device needed): both cut actions[0..n) into rounds.  slots[l]: tape slots of
+ * layer l; live_now[l]: tapes of layer l alive before the list (NULL: none); window >= 1 units of look-ahead; max_group
+ * actions per round.  round_of_action[i] receives the round of action i (rounds are numbered from 0 in issue order),
+ * *n_rounds_out their number.  ORDER if the list admits no plan (an action whose predecessors never become ready, or a
+ * pool too small), BAD_ARG for a malformed action.
+ * qe_plan_rounds: rounds that qe_run_together takes (at most one action of a kind per layer), all kinds in the window.
+ * qe_plan_step: the plan qe_step_run makes, as described above -- at most max_group F and dI actions and as many layers'
+ * weight gradients in a round, of a layer up to max_sum microbatches, of all layers QE_STEP_MAX_PRODUCTS. */
+#define QE_STEP_MAX_PRODUCTS 32
+int32_t qe_plan_step(const qe_step_action* actions, uint32_t n_actions, uint32_t n_layers, uint32_t microbatches,
+                     const uint32_t* slots, const uint32_t* live_now, uint32_t window, uint32_t max_group,
+                     uint32_t max_sum, uint32_t* round_of_action, uint32_t* n_rounds_out);
 int32_t qe_plan_rounds(const qe_step_action* actions, uint32_t n_actions, uint32_t n_layers, uint32_t microbatches,
                        const uint32_t* slots, const uint32_t* live_now, uint32_t window, uint32_t max_group,
                        uint32_t* round_of_action, uint32_t* n_rounds_out);

@@ -2,6 +2,7 @@
 // (Algorithm 1: a check precedes its action, the transition commits only after the action succeeded).
 #include "contract.h"
 
+#include <algorithm>
 #include <cstring>
 #include <new>
 #include <vector>
@@ -359,6 +360,109 @@ int32_t qe_plan_rounds(const qe_step_action* actions, uint32_t n_actions, uint32
       if (!all) break;
       ++first;
     }
+  }
+  *n_rounds_out = round;
+  return QE_OK;
+}
+
+// ---- issue plan of the whole-step call.  F and dI as in qe_plan_rounds (but the window counts F and dI units only, and
+// each layer sees its actions of a kind strictly in list order); dW actions wait and go out several microbatches at once.
+int32_t qe_plan_step(const qe_step_action* actions, uint32_t n_actions, uint32_t n_layers, uint32_t microbatches,
+                     const uint32_t* slots, const uint32_t* live_now, uint32_t window, uint32_t max_group,
+                     uint32_t max_sum, uint32_t* round_of_action, uint32_t* n_rounds_out) {
+  if (!actions || !slots || !round_of_action || !n_rounds_out) return fail(QE_ERR_BAD_ARG, "null argument");
+  if (n_actions == 0 || n_layers == 0 || microbatches == 0 || window == 0 || max_group == 0 || max_sum == 0) return fail(QE_ERR_BAD_ARG, "empty list or zero limit");
+  const uint32_t M = microbatches;
+  struct Unit { uint32_t kind, begin, end; };  // end: one past its last action; begin advances as they go out
+  std::vector<Unit> units;
+  struct LayerLists { std::vector<uint32_t> of[3]; uint32_t next[3] = {0, 0, 0}; };  // action indices per kind, list order
+  std::vector<LayerLists> lists(n_layers);
+  std::vector<uint8_t> in_unit(n_layers, 0);
+  for (uint32_t i = 0; i < n_actions; ++i) {
+    const qe_step_action& a = actions[i];
+    if (a.kind > QE_ACT_DW || a.layer >= n_layers || a.mb >= M) return fail(QE_ERR_BAD_ARG, "action %u: kind %u layer %u mb %u", i, a.kind, a.layer, a.mb);
+    const bool fresh = i == 0 || actions[i - 1].kind != a.kind || actions[i - 1].mb != a.mb || in_unit[a.layer];
+    if (fresh) std::fill(in_unit.begin(), in_unit.end(), (uint8_t)0);
+    in_unit[a.layer] = 1;
+    if (a.kind != QE_ACT_DW) {
+      if (fresh) units.push_back(Unit{a.kind, i, i});
+      units.back().end = i + 1;
+    }
+    lists[a.layer].of[a.kind].push_back(i);
+  }
+  constexpr uint32_t kNever = UINT32_MAX;
+  std::vector<uint32_t> f_round((size_t)n_layers * M, kNever), di_round((size_t)n_layers * M, kNever);
+  std::vector<uint32_t> live(n_layers, 0), freed(n_layers, 0);
+  for (uint32_t l = 0; live_now && l < n_layers; ++l) live[l] = live_now[l];
+  std::vector<uint8_t> blocked(n_layers, 0);
+  uint32_t round = 0, left = n_actions;
+  size_t first = 0;
+  for (; left; ++round) {
+    uint32_t group = 0;
+    std::fill(blocked.begin(), blocked.end(), (uint8_t)0);
+    for (size_t ui = first; ui < units.size() && ui < first + window && group < max_group; ++ui) {
+      Unit& u = units[ui];
+      if (u.begin == u.end) continue;
+      const uint32_t i = u.begin;  // a unit walks its layers in list order: only this action can be ready
+      const qe_step_action& a = actions[i];
+      LayerLists& q = lists[a.layer];
+      if (q.of[a.kind][q.next[a.kind]] != i) continue;  // an earlier action of the kind on this layer comes first
+      // predecessors must have been issued in earlier rounds (same-kind ones of this layer too)
+      if (q.next[a.kind]) {
+        const uint32_t before = q.of[a.kind][q.next[a.kind] - 1];
+        if (round_of_action[before] == round) continue;
+      }
+      const size_t u_mb = (size_t)a.layer * M + a.mb;
+      if (a.kind == QE_ACT_F) {
+        if (f_round[u_mb] != kNever) return fail(QE_ERR_ORDER, "action %u: second forward of layer %u microbatch %u", i, a.layer, a.mb);
+        if (live[a.layer] >= slots[a.layer]) {
+          blocked[a.layer] = 1;
+          continue;
+        }
+        f_round[u_mb] = round;
+        live[a.layer] += 1;
+      } else {
+        if (di_round[u_mb] != kNever) return fail(QE_ERR_ORDER, "action %u: second input gradient of layer %u microbatch %u", i, a.layer, a.mb);
+        if (f_round[u_mb] == kNever || f_round[u_mb] == round) continue;
+        di_round[u_mb] = round;
+      }
+      q.next[a.kind] += 1;
+      round_of_action[i] = round;
+      u.begin += 1;
+      ++group;
+    }
+    // Weight gradients: those of a layer that are ready (dI in an earlier round) go out together when a forward needs
+    // their slots, when there are max_sum of them, when no more are to come, or when nothing else can run.
+    const bool idle = group == 0;
+    uint32_t n_dw = 0, products = 0;
+    for (uint32_t l = 0; l < n_layers && n_dw < max_group && products < QE_STEP_MAX_PRODUCTS; ++l) {
+      LayerLists& q = lists[l];
+      const std::vector<uint32_t>& of = q.of[QE_ACT_DW];
+      uint32_t ready = 0;
+      while (q.next[QE_ACT_DW] + ready < of.size() && ready < max_sum) {
+        const qe_step_action& a = actions[of[q.next[QE_ACT_DW] + ready]];
+        const uint32_t r = di_round[(size_t)l * M + a.mb];
+        if (r == kNever || r == round) break;
+        ++ready;
+      }
+      if (!ready) continue;
+      const bool need = blocked[l] || (live[l] >= slots[l] && q.next[QE_ACT_F] < q.of[QE_ACT_F].size());
+      const bool last = q.next[QE_ACT_DW] + ready == of.size();
+      if (!need && !last && ready < max_sum && !idle) continue;
+      if (ready > QE_STEP_MAX_PRODUCTS - products) ready = QE_STEP_MAX_PRODUCTS - products;
+      for (uint32_t j = 0; j < ready; ++j) round_of_action[of[q.next[QE_ACT_DW] + j]] = round;
+      q.next[QE_ACT_DW] += ready;
+      freed[l] = ready;
+      products += ready;
+      ++n_dw;
+    }
+    if (group == 0 && n_dw == 0) return fail(QE_ERR_ORDER, "no action of round %u is ready: the list is not a legal schedule for these pools", round);
+    for (uint32_t l = 0; n_dw && l < n_layers; ++l) {  // released slots are visible to later rounds only
+      live[l] -= freed[l] < live[l] ? freed[l] : live[l];
+      freed[l] = 0;
+    }
+    left -= group + products;
+    while (first < units.size() && units[first].begin == units[first].end) ++first;
   }
   *n_rounds_out = round;
   return QE_OK;

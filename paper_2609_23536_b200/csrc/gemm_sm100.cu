@@ -2,21 +2,23 @@
 // stored contraction-major ([rows, Kc]) or MN-major ([Kc, rows]: the transposed view of a row-major tensor, read by the
 // tensor cores directly), FP32 accumulation in tensor memory.
 //
-// Structure: persistent clusters of two CTAs on neighbouring SMs, 320 threads each, that compute one tile of 256 rows
+// Structure: persistent clusters of two CTAs on neighbouring SMs, 320 or 384 threads each, that compute one tile of 256 rows
 // and 256, 128 or 64 columns together with tcgen05.mma.cta_group::2:
 //   warp 0      TMA producer: cp.async.bulk.tensor 2D tiles into a six-stage shared-memory ring; per 128-byte K block
 //               each CTA loads its own 128 rows of A and its own half of the tile's B rows
 //   warp 1      allocates tensor memory, then one lane of the even CTA issues tcgen05.mma (256 x tile_n x 32 per
 //               instruction) and tcgen05.commit, which multicasts stage-free / accumulator-ready arrivals to both CTAs
-//   warps 2-9   epilogue: tcgen05.ld the CTA's 128 x tile_n FP32 accumulator (two warps per 32-lane quadrant, half of
+//   8 warps     epilogue: tcgen05.ld the CTA's 128 x tile_n FP32 accumulator (two warps per 32-lane quadrant, half of
 //               the columns each) in 32 x 32 blocks, scale, write each block into a swizzled per-warp shared-memory
 //               tile and hand it to the bulk-store unit: a bulk tensor store for bf16 (+ max|D| reduced by warp
 //               shuffles, one atomicMax per warp and tile) and for FP32 overwrite; a bulk tensor reduction (.add) for
 //               FP32 accumulation straight into the destination (direct gradient placement): the addition is done in
 //               L2, one per element and launch, and the destination tile is prefetched into L2 while the tile's
 //               main loop runs.  The reduction is a plain round-to-nearest FP32 addition (subnormal values kept).
-//   The launch may also carry up to eight independent problems (grouped launch): tiles are numbered problem after
+//   The launch may also carry up to sixteen independent problems (grouped launch): tiles are numbered problem after
 //   problem and each role looks its tile's problem up, so that one set of persistent CTAs packs them all.
+//   A problem may be the sum of several products (the deferred weight gradients of several microbatches): each gets an
+//   accumulator of its own, and the epilogue adds them up in registers before the one store.
 // Rows beyond M (M is a multiple of 128; a tile has 256) are read as zeros by TMA and never stored.
 // Scale commits (fold a pending amax into its history, update the scale) ride along, so that no extra launch is needed:
 // classes whose amax an earlier kernel completed (X of a forward, G of an input gradient) are committed by an idle
@@ -52,8 +54,11 @@ constexpr int STAGES = 6;                      // faster at 64 columns: the ring
 constexpr uint32_t TMEM_COLS = 512;
 constexpr uint32_t EPI_BUF_BYTES = 4096;                     // per epilogue warp: one FP32 or two bf16 32 x 32 output tiles
                                                              // (1 KB-aligned, swizzled) that the bulk-store unit reads
-constexpr int THREADS = 320;
 constexpr int EPI_WARPS = 8, EPI_THREADS = EPI_WARPS * 32;
+// Threads of a CTA: warps 0 and 1, then the epilogue's eight.  The variant that sums several products keeps a tile row of
+// 128 FP32 per epilogue thread: its epilogue warps are two whole warpgroups (warps 2 and 3 idle), which take over
+// registers that the first warpgroup hands back (launched with 168 a thread; 40 + 2 * 224 <= 3 * 168).
+constexpr int threads_of(bool sums) { return sums ? 384 : 320; }
 static_assert(EPI_WARPS == 8, "shared-memory budget below assumes 8 epilogue warps");
 constexpr uint32_t SMEM_BYTES = STAGES * STAGE_BYTES + 1024 /*alignment slack*/ + 256 /*barriers, flags*/ + 8 * EPI_BUF_BYTES;
 constexpr long long WAIT_BUDGET_CYCLES = 4000000000ll;  // ~2 s at the maximum SM clock
@@ -184,7 +189,28 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
       : "r"(taddr)
       : "memory");
 }
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr)
+      : "memory");
+}
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+
+// One row of a 32 x 32 FP32 tile for the bulk-store unit: 128-byte rows, 128-byte swizzle (chunk c of row r sits at
+// c ^ (r & 7)).
+__device__ __forceinline__ void st_tile_f32(uint32_t buf, int row, const float (&v)[32]) {
+#pragma unroll
+  for (int c = 0; c < 8; ++c) {
+    const uint32_t dst = buf + (uint32_t)row * 128u + (((uint32_t)c ^ ((uint32_t)row & 7u)) << 4);
+    asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(dst), "f"(v[4 * c]), "f"(v[4 * c + 1]), "f"(v[4 * c + 2]),
+                 "f"(v[4 * c + 3])
+                 : "memory");
+  }
+}
 
 __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
   __nv_bfloat162 v = __floats2bfloat162_rn(a, b);  // .x = a in the low half
@@ -222,38 +248,52 @@ __device__ __forceinline__ uint32_t snake_tile(uint32_t w, uint32_t first, uint3
 }
 
 // ------------------------------------------------------------------------------------------------ problem lookup
-// A launch computes one GEMM, or (grouped launch) up to four independent ones whose tiles are numbered one after the
+// A launch computes one GEMM, or (grouped launch) several independent ones whose tiles are numbered one after the
 // other, so that one set of persistent CTAs packs them into common waves and the launch overhead is paid once.
-struct OneProblem {
-  const GemmParams& p;
-  __device__ __forceinline__ uint32_t total_tiles() const { return ((p.M + TILE_M - 1) / TILE_M) * ((p.N + p.tile_n - 1) / p.tile_n); }
-  __device__ __forceinline__ const GemmParams& at(uint32_t tile, uint32_t& local) const {
-    local = tile;
-    return p;
-  }
-  __device__ __forceinline__ const GemmParams& first() const { return p; }
-  __device__ __forceinline__ uint32_t count() const { return 1; }
-  __device__ __forceinline__ const CommitParams& commit(uint32_t) const { return p.commit; }
-  __device__ __forceinline__ uint32_t* status_of(uint32_t) const { return p.status; }
-};
-struct ProblemGroup {
-  const GemmGroupParams& g;
-  __device__ __forceinline__ uint32_t total_tiles() const { return g.tile_end[g.n - 1]; }
+template <int NP, int NOPS>
+struct Problems {
+  static constexpr bool SUMS = NOPS > NP;  // problems may have several products
+  const GemmLaunchParams<NP, NOPS>& g;
+  __device__ __forceinline__ uint32_t count() const { return NP == 1 ? 1u : g.n; }
+  __device__ __forceinline__ uint32_t total_tiles() const { return g.tile_end[count() - 1]; }
   __device__ __forceinline__ const GemmParams& at(uint32_t tile, uint32_t& local) const {
     uint32_t i = 0, base = 0;
-    while (i + 1 < g.n && tile >= g.tile_end[i]) base = g.tile_end[i++];
+    while (i + 1 < count() && tile >= g.tile_end[i]) base = g.tile_end[i++];
     local = tile - base;
     return g.prob[i];
   }
+  __device__ __forceinline__ const GemmOperands& operands(const GemmParams& p, uint32_t seg) const {
+    return g.op[NOPS == 1 ? 0u : p.op0 + seg];
+  }
   __device__ __forceinline__ const GemmParams& first() const { return g.prob[0]; }
-  __device__ __forceinline__ uint32_t count() const { return g.n; }
   __device__ __forceinline__ const CommitParams& commit(uint32_t i) const { return g.prob[i].commit; }
   __device__ __forceinline__ uint32_t* status_of(uint32_t i) const { return g.prob[i].status; }
 };
 
+// 32 floats of one row, read from L2 (the destination of an accumulating launch; earlier launches wrote it there).
+__device__ __forceinline__ void ld_row32(const float* src, float* v) {
+  if ((reinterpret_cast<uintptr_t>(src) & 31u) == 0) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      asm volatile("ld.relaxed.gpu.global.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                   : "=f"(v[8 * j]), "=f"(v[8 * j + 1]), "=f"(v[8 * j + 2]), "=f"(v[8 * j + 3]), "=f"(v[8 * j + 4]),
+                     "=f"(v[8 * j + 5]), "=f"(v[8 * j + 6]), "=f"(v[8 * j + 7])
+                   : "l"(src + 8 * j)
+                   : "memory");
+  } else {
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      const float4 q = __ldcg(reinterpret_cast<const float4*>(src) + j);
+      v[4 * j] = q.x, v[4 * j + 1] = q.y, v[4 * j + 2] = q.z, v[4 * j + 3] = q.w;
+    }
+  }
+}
+
 // ------------------------------------------------------------------------------------------------ kernel
 template <class PS>
 __device__ __forceinline__ void gemm_body(const PS& ps) {
+  constexpr bool SUMS = PS::SUMS;
+  constexpr int EPI_WARP0 = SUMS ? 4 : 2;  // first epilogue warp
   extern __shared__ uint8_t smem_raw[];
   const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   const uint32_t epi_base = smem_base + STAGES * STAGE_BYTES;  // 1 KB-aligned
@@ -283,8 +323,8 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
 
   if (threadIdx.x == 32) {  // descriptor fetch overlaps the rest of the prologue (and the predecessor's tail)
     const GemmParams& q = ps.first();  // (a group's other descriptors are fetched on first use)
-    asm volatile("prefetch.tensormap [%0];" ::"l"(&q.tmA) : "memory");
-    asm volatile("prefetch.tensormap [%0];" ::"l"(&q.tmB) : "memory");
+    asm volatile("prefetch.tensormap [%0];" ::"l"(&ps.operands(q, 0).tmA) : "memory");
+    asm volatile("prefetch.tensormap [%0];" ::"l"(&ps.operands(q, 0).tmB) : "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(&q.tmD) : "memory");
   }
   if (threadIdx.x == 0) {
@@ -320,21 +360,22 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
     uint32_t m0, n0;
     tile_coords(local_tile, tiles_m, tiles_n, m_fastest, tile_n, m0, n0);
     const int rb = (int)(n0 + rank * (tile_n / 2));
+    const CUtensorMap* tmB = &ps.operands(p, 0).tmB;
     for (uint32_t kb = 0; kb < num_kb && kb < (uint32_t)STAGES; ++kb) {
       const int ka = (int)(kb * BK);
-      if (p.b_mn) tma_prefetch_2d(&p.tmB, rb, ka);
-      else tma_prefetch_2d(&p.tmB, ka, rb);
+      if (p.b_mn) tma_prefetch_2d(tmB, rb, ka);
+      else tma_prefetch_2d(tmB, ka, rb);
     }
   }
   // Everything above (barriers, tensor memory) touched no data a predecessor produces and may overlap the previous
   // kernel's tail; operands, scales and the destination may come from it, so wait for it here.
   grid_dep_wait();
   grid_dep_launch();
-  if (blockIdx.x == 0 && threadIdx.x == 64) {  // FP8 hand-off: the consumer's tape snapshot of its inverse scale
+  if (blockIdx.x == 0 && threadIdx.x == EPI_WARP0 * 32) {  // FP8 hand-off: the consumer's tape snapshot of its inverse scale
     const GemmParams& q = ps.first();
     if (q.epi == 3 && q.sinv_dst) *q.sinv_dst = *q.sinv_src;
   }
-  if (warp == 9 && blockIdx.x < ps.count()) {  // (every launch has at least two CTAs per problem)
+  if (warp == EPI_WARP0 + 7 && blockIdx.x < ps.count()) {  // (every launch has at least two CTAs per problem)
     // The classes whose amax an EARLIER kernel reduced (the cast that made this GEMM's A operand) are committed here,
     // by an epilogue warp that has nothing to drain yet: nothing this launch computes reads their scale (its alphas
     // are snapshots), so only the output's class is left for the launch's tail.
@@ -345,6 +386,12 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
     }
   }
 
+  // (The roles are one flat choice: with producer and issuer nested under a choice of their own, or written as lambdas, the
+  // same code ran 4 % slower, small launches and large ones alike.)
+  if (SUMS) {
+    __syncwarp();
+    if (warp < EPI_WARP0) asm volatile("setmaxnreg.dec.sync.aligned.u32 40;");
+  }
   if (warp == 0) {
     // ---------------------------------------------------------------- TMA producer
     if (lane == 0) {
@@ -356,20 +403,23 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
         uint32_t m0, n0;
         tile_coords(local_tile, tiles_m, tiles_n, m_fastest, tile_n, m0, n0);
         const int ra = (int)(m0 + rank * BM), rb = (int)(n0 + rank * (tile_n / 2));
-        for (uint32_t kb = 0; kb < num_kb; ++kb) {
-          if (!(ok = mbar_wait(empty_bar(s), ph ^ 1u, abort_flag, status, ERR_PRODUCER))) break;
-          const uint32_t a_dst = smem_base + s * STAGE_BYTES, b_dst = a_dst + A_BYTES;
-          // both CTAs credit the even CTA's barrier, which expects the bytes of the whole pair
-          if (rank == 0) mbar_expect_tx(full_bar(s), 2 * A_BYTES + tile_n * BK);
-          const uint32_t bar = map_to_cta(full_bar(s), 0);
-          // contraction-major operand: box = 128 K-bytes x rows at (k, row); MN-major operand (stored as [Kc, rows]):
-          // box = row-bytes x 128 K-rows at (row, k).  Either way 128 bytes per row land in shared memory.
-          const int ka = (int)(kb * BK);
-          if (p.a_mn) tma_load_2d_pair(a_dst, &p.tmA, bar, ra, ka);
-          else tma_load_2d_pair(a_dst, &p.tmA, bar, ka, ra);
-          if (p.b_mn) tma_load_2d_pair(b_dst, &p.tmB, bar, rb, ka);
-          else tma_load_2d_pair(b_dst, &p.tmB, bar, ka, rb);
-          if (++s == STAGES) { s = 0; ph ^= 1u; }
+        for (uint32_t seg = 0; ok && seg < (SUMS ? p.nseg : 1u); ++seg) {
+          const GemmOperands& op = ps.operands(p, seg);
+          for (uint32_t kb = 0; kb < num_kb; ++kb) {
+            if (!(ok = mbar_wait(empty_bar(s), ph ^ 1u, abort_flag, status, ERR_PRODUCER))) break;
+            const uint32_t a_dst = smem_base + s * STAGE_BYTES, b_dst = a_dst + A_BYTES;
+            // both CTAs credit the even CTA's barrier, which expects the bytes of the whole pair
+            if (rank == 0) mbar_expect_tx(full_bar(s), 2 * A_BYTES + tile_n * BK);
+            const uint32_t bar = map_to_cta(full_bar(s), 0);
+            // contraction-major operand: box = 128 K-bytes x rows at (k, row); MN-major operand (stored as [Kc, rows]):
+            // box = row-bytes x 128 K-rows at (row, k).  Either way 128 bytes per row land in shared memory.
+            const int ka = (int)(kb * BK);
+            if (p.a_mn) tma_load_2d_pair(a_dst, &op.tmA, bar, ra, ka);
+            else tma_load_2d_pair(a_dst, &op.tmA, bar, ka, ra);
+            if (p.b_mn) tma_load_2d_pair(b_dst, &op.tmB, bar, rb, ka);
+            else tma_load_2d_pair(b_dst, &op.tmB, bar, ka, rb);
+            if (++s == STAGES) { s = 0; ph ^= 1u; }
+          }
         }
       }
       if (!ok) {
@@ -387,34 +437,37 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
       for (uint32_t wave = 0, tile = first_tile; ok && tile < num_tiles; ++wave, tile = snake_tile(wave, first_tile, tile_step)) {
         QE_TILE_PROBLEM();
         (void)tiles_m; (void)tiles_n; (void)m_fastest;
-        if (!(ok = mbar_wait(tempty_bar(acc), acc_ph ^ 1u, abort_flag, status, ERR_MMA))) break;
-        tc_fence_after();
-        const uint32_t d_tmem = tmem_base + acc * ACC_COLS;
         const uint32_t idesc = p.idesc, b_hi = p.b_desc_hi, a_step = p.a_mn ? 256u : 2u, b_step = p.b_step;
-        for (uint32_t kb = 0; kb < num_kb; ++kb) {
-          if (!(ok = mbar_wait(full_bar(s), ph, abort_flag, status, ERR_MMA))) break;
+        for (uint32_t seg = 0; ok && seg < (SUMS ? p.nseg : 1u); ++seg) {  // an accumulator of its own for each product
+          if (!(ok = mbar_wait(tempty_bar(acc), acc_ph ^ 1u, abort_flag, status, ERR_MMA))) break;
           tc_fence_after();
-          const uint32_t a_src = smem_base + s * STAGE_BYTES, b_src = a_src + A_BYTES;
-          const uint64_t adesc = make_desc(a_src, A_DESC_HI), bdesc = make_desc(b_src, b_hi);
+          const uint32_t d_tmem = tmem_base + acc * ACC_COLS;
+          for (uint32_t kb = 0; kb < num_kb; ++kb) {
+            if (!(ok = mbar_wait(full_bar(s), ph, abort_flag, status, ERR_MMA))) break;
+            tc_fence_after();
+            const uint32_t a_src = smem_base + s * STAGE_BYTES, b_src = a_src + A_BYTES;
+            const uint64_t adesc = make_desc(a_src, A_DESC_HI), bdesc = make_desc(b_src, b_hi);
 #pragma unroll
-          for (int k = 0; k < (int)BK / UMMA_K; ++k)
-            // advancing 32 along the contraction: 32 bytes inside the 128-byte swizzle row for a contraction-major
-            // tile (+2 in the address field), 32 rows for an MN-major one (+256 with rows of 128 bytes)
-            tc_mma_f8_pair(d_tmem, adesc + a_step * k, bdesc + b_step * k, idesc, (kb | (uint32_t)k) != 0u);
-          tc_commit_pair(empty_bar(s));  // stage reusable (in both CTAs) once these MMAs have read it
-          if (++s == STAGES) { s = 0; ph ^= 1u; }
+            for (int k = 0; k < (int)BK / UMMA_K; ++k)
+              // advancing 32 along the contraction: 32 bytes inside the 128-byte swizzle row for a contraction-major
+              // tile (+2 in the address field), 32 rows for an MN-major one (+256 with rows of 128 bytes)
+              tc_mma_f8_pair(d_tmem, adesc + a_step * k, bdesc + b_step * k, idesc, (kb | (uint32_t)k) != 0u);
+            tc_commit_pair(empty_bar(s));  // stage reusable (in both CTAs) once these MMAs have read it
+            if (++s == STAGES) { s = 0; ph ^= 1u; }
+          }
+          if (!ok) break;
+          tc_commit_pair(tfull_bar(acc));  // accumulator complete (each CTA holds its 128 rows)
+          if (++acc == 2) { acc = 0; acc_ph ^= 1u; }
         }
-        if (!ok) break;
-        tc_commit_pair(tfull_bar(acc));  // accumulator complete (each CTA holds its 128 rows)
-        if (++acc == 2) { acc = 0; acc_ph ^= 1u; }
       }
     }
-  } else {
-    // ---------------------------------------------------------------- epilogue (warps 2..9)
+  } else if (!SUMS || warp >= EPI_WARP0) {
+    // ---------------------------------------------------------------- epilogue
+    if (SUMS) asm volatile("setmaxnreg.inc.sync.aligned.u32 224;");
     const uint32_t quad = (uint32_t)warp & 3u;          // tensor-memory lane quadrant this warp may read
-    const uint32_t half = ((uint32_t)warp - 2u) >> 2;   // which half of the tile's columns
-    const int etid = (int)threadIdx.x - 64;
-    const uint32_t epi_smem = epi_base + (uint32_t)(warp - 2) * EPI_BUF_BYTES;  // this warp's two output tiles
+    const uint32_t half = (uint32_t)(warp - EPI_WARP0) >> 2;   // which half of the tile's columns
+    const int etid = (int)threadIdx.x - EPI_WARP0 * 32;
+    const uint32_t epi_smem = epi_base + (uint32_t)(warp - EPI_WARP0) * EPI_BUF_BYTES;  // this warp's two output tiles
     uint32_t n_groups = 0;  // bulk-store groups this warp has committed (buffer parity)
     uint32_t acc = 0, acc_ph = 0;
     bool ok = true;
@@ -422,13 +475,63 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
     for (uint32_t wave = 0, tile = first_tile; ok && tile < num_tiles; ++wave, tile = snake_tile(wave, first_tile, tile_step)) {
       QE_TILE_PROBLEM();
       (void)num_kb;
-      const float alpha = __fmul_rn(*p.alpha_a, *p.alpha_b);
       uint32_t m0, n0;
       tile_coords(local_tile, tiles_m, tiles_n, m_fastest, tile_n, m0, n0);
       const uint32_t blk_row0 = m0 + rank * BM + quad * 32u;
       const uint32_t col0 = n0 + half * (tile_n / 2);
       // 32 x 32 blocks of this warp: none in rows beyond M, fewer in a ragged last column tile; warp-uniform
       const uint32_t nch = blk_row0 >= p.M || col0 >= p.N ? 0u : min(tile_n / 64u, (p.N - col0) / 32u);
+      if (SUMS && p.nseg > 1) {
+        // Several products for one FP32 tile (the weight gradients of several microbatches): the tile's running value
+        // stays in registers and every product is added to it in order, each with its own scale -- the additions
+        // launches of their own would have done in L2, at one read and one write of the destination instead of one
+        // per product.  What is added to is fetched while the first product is being computed.
+        float v[4][32];
+        if (p.epi == 2) {
+          const float* src = reinterpret_cast<const float*>(p.out) + (size_t)(blk_row0 + lane) * p.ldo + col0;
+#pragma unroll
+          for (int ch = 0; ch < 4; ++ch)
+            if ((uint32_t)ch < nch) ld_row32(src + ch * 32, v[ch]);
+        }
+        for (uint32_t seg = 0; seg < (SUMS ? p.nseg : 1u); ++seg) {
+          const GemmOperands& op = ps.operands(p, seg);
+          const float alpha = __fmul_rn(*op.alpha_a, *op.alpha_b);
+          const bool overwrite = seg == 0 && p.epi == 1;
+          if (!(ok = mbar_wait(tfull_bar(acc), acc_ph, abort_flag, status, ERR_EPILOGUE))) break;
+          tc_fence_after();
+          const uint32_t t_row = tmem_base + ((quad * 32u) << 16) + acc * ACC_COLS + half * (tile_n / 2);
+#pragma unroll
+          for (int h = 0; h < 8; ++h) {
+            if ((uint32_t)h >= 2 * nch) break;
+            uint32_t rc[16];
+            tmem_ld16(t_row + h * 16u, rc);
+            tmem_ld_wait();
+#pragma unroll
+            for (int j = 0; j < 16; ++j) {
+              float& t = v[h / 2][(h & 1) * 16 + j];
+              const float d = __fmul_rn(__uint_as_float(rc[j]), alpha);
+              t = overwrite ? d : __fadd_rn(t, d);
+            }
+          }
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive_cluster(acc ? tempty_leader1 : tempty_leader0);
+          if (++acc == 2) { acc = 0; acc_ph ^= 1u; }
+        }
+        if (!ok) break;
+#pragma unroll
+        for (int ch = 0; ch < 4; ++ch) {
+          if ((uint32_t)ch >= nch) break;
+          if (lane == 0) tma_store_wait_read<0>();
+          __syncwarp();
+          st_tile_f32(epi_smem, lane, v[ch]);
+          fence_async_smem();
+          __syncwarp();
+          if (lane == 0) tma_store_2d(&p.tmD, epi_smem, (int)(col0 + ch * 32u), (int)blk_row0);
+        }
+        continue;
+      }
+      const float alpha = __fmul_rn(*ps.operands(p, 0).alpha_a, *ps.operands(p, 0).alpha_b);
       if (p.epi == 2) {
         // accumulate: pull this thread's destination row segment into L2, where the reduction will add to it, while
         // the MMAs of the tile run
@@ -457,7 +560,10 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
         // adds them to the destination where it lives, in L2 (FP32 accumulate: one addition per element and launch).
         if (p.epi == 0) {
           const uint32_t buf = epi_smem + (n_groups & 1u) * 2048u;  // two tiles: the previous store may still read
-          if (lane == 0) tma_store_wait_read<1>();
+          if (lane == 0) {  // (a tile before this one may have used the buffer as a whole)
+            if (ch == 0) tma_store_wait_read<0>();
+            else tma_store_wait_read<1>();
+          }
           __syncwarp();
           uint32_t o[16];
 #pragma unroll
@@ -516,14 +622,10 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
           const uint32_t buf = epi_smem;
           if (lane == 0) tma_store_wait_read<0>();
           __syncwarp();
+          float o[32];
 #pragma unroll
-          for (int c = 0; c < 8; ++c) {  // 128-byte rows, 128-byte swizzle: chunk c of row r sits at c ^ (r & 7)
-            const uint32_t dst = buf + (uint32_t)lane * 128u + (((uint32_t)c ^ ((uint32_t)lane & 7u)) << 4);
-            asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(dst),
-                         "f"(__fmul_rn(__uint_as_float(rc[4 * c]), alpha)), "f"(__fmul_rn(__uint_as_float(rc[4 * c + 1]), alpha)),
-                         "f"(__fmul_rn(__uint_as_float(rc[4 * c + 2]), alpha)), "f"(__fmul_rn(__uint_as_float(rc[4 * c + 3]), alpha))
-                         : "memory");
-          }
+          for (int j = 0; j < 32; ++j) o[j] = __fmul_rn(__uint_as_float(rc[j]), alpha);
+          st_tile_f32(buf, lane, o);
           fence_async_smem();
           __syncwarp();
           if (lane == 0) {
@@ -555,7 +657,7 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
       if (!ticket && ps.commit(i).st && ps.commit(i).class_mask) ticket = &ps.commit(i).st->ticket;
     if (ticket && last_block(ticket, gridDim.x, etid, last_flag, epi_bar_sync)) {
       // one epilogue warp per problem, side by side
-      for (uint32_t i = (uint32_t)warp - 2u; i < ps.count(); i += EPI_WARPS) {
+      for (uint32_t i = (uint32_t)(warp - EPI_WARP0); i < ps.count(); i += EPI_WARPS) {
         CommitParams c = ps.commit(i);
         c.bump_token = 0;  // (counted by the early part)
         if (c.st && c.class_mask) commit_classes_warp(c, lane);
@@ -584,15 +686,25 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
 
 #undef QE_TILE_PROBLEM
 
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
-    gemm_fp8_pair_kernel(const __grid_constant__ GemmParams p) {
-  gemm_body(OneProblem{p});
+using OneParams = GemmLaunchParams<1, 1>;
+using GroupParams = GemmLaunchParams<8, 8>;
+using WideParams = GemmLaunchParams<kMaxProblems, kMaxOperands>;
+
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(threads_of(false), 1)
+    gemm_fp8_pair_kernel(const __grid_constant__ OneParams p) {
+  gemm_body(Problems<1, 1>{p});
 }
 
 // Up to eight independent GEMMs in one launch.
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
-    gemm_fp8_pair_group_kernel(const __grid_constant__ GemmGroupParams g) {
-  gemm_body(ProblemGroup{g});
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(threads_of(false), 1)
+    gemm_fp8_pair_group_kernel(const __grid_constant__ GroupParams g) {
+  gemm_body(Problems<8, 8>{g});
+}
+
+// More problems, or problems of several products each.  (The parameter block is three times as large.)
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(threads_of(true), 1)
+    gemm_fp8_pair_wide_kernel(const __grid_constant__ WideParams g) {
+  gemm_body(Problems<kMaxProblems, kMaxOperands>{g});
 }
 
 uint32_t tiles_of(const GemmDesc& d, uint32_t tile_n) { return ((d.M + TILE_M - 1) / TILE_M) * ((d.N + tile_n - 1) / tile_n); }
@@ -615,12 +727,12 @@ uint32_t choose_width(const GemmDesc* d, uint32_t n, uint32_t pairs) {
   return w;
 }
 
-// The device's parameter block of one problem at a tile width.
-void fill_problem(const GemmDesc& d, uint32_t w, GemmParams* p) {
+// The device's parameter block of one problem at a tile width, its operand pairs appended to op[].
+void fill_problem(const GemmDesc& d, uint32_t w, GemmParams* p, GemmOperands* op, uint32_t* nops) {
   *p = d;
   const uint32_t tile_n = kTileWidths[w], per_cta = tile_n / 2;
-  p->tmA = *d.mapA;
-  p->tmB = d.mapB[w];
+  p->op0 = *nops;
+  for (uint32_t i = 0; i < d.nseg; ++i) op[(*nops)++] = GemmOperands{*d.ops[i].mapA, d.ops[i].mapB[w], d.ops[i].alpha_a, d.ops[i].alpha_b};
   p->tile_n = tile_n;
   // bits 4-5: accumulator format (1 = FP32); 7-9 / 10-12: A / B format (0 = E4M3, 1 = E5M2); 15 / 16: A / B major
   // (0 = contraction-major); 17-22: N >> 3; 24-28: M >> 4 (256 for a CTA pair).
@@ -631,50 +743,55 @@ void fill_problem(const GemmDesc& d, uint32_t w, GemmParams* p) {
   p->b_step = d.b_mn ? 32u * row / 16u : 2u;
 }
 
+template <int NP, int NOPS>
+Launch make_launch(const GemmDesc* probs, uint32_t n, int num_sms, const void* func) {
+  GemmLaunchParams<NP, NOPS> g{};
+  const uint32_t pairs = (uint32_t)num_sms / 2u, w = choose_width(probs, n, pairs);
+  uint32_t tiles = 0, nops = 0;
+  for (uint32_t i = 0; i < n; ++i) {
+    tiles += tiles_of(probs[i], kTileWidths[w]);
+    g.tile_end[i] = tiles;
+    fill_problem(probs[i], w, &g.prob[i], g.op, &nops);
+  }
+  g.n = n;
+  Launch l;
+  l.func = func;
+  l.grid = dim3(2u * (tiles < pairs ? tiles : pairs), 1, 1);
+  l.block = dim3(threads_of(NOPS > NP), 1, 1);
+  l.smem = SMEM_BYTES;
+  l.set(g);
+  return l;
+}
+
+Launch make_any(const GemmDesc* probs, uint32_t n, uint32_t nops, int num_sms) {
+  if (n == 1 && nops == 1) return make_launch<1, 1>(probs, n, num_sms, (const void*)gemm_fp8_pair_kernel);
+  if (n <= 8 && nops == n) return make_launch<8, 8>(probs, n, num_sms, (const void*)gemm_fp8_pair_group_kernel);
+  return make_launch<kMaxProblems, kMaxOperands>(probs, n, num_sms, (const void*)gemm_fp8_pair_wide_kernel);
+}
+
 }  // namespace
 
 bool gemm_uses_pair(uint32_t M) { return M % 256 == 0; }
 
 cudaError_t gemm_prepare() {
-  cudaError_t e = cudaFuncSetAttribute((const void*)gemm_fp8_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES);
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute((const void*)gemm_fp8_pair_group_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)SMEM_BYTES);
+  for (const void* f : {(const void*)gemm_fp8_pair_kernel, (const void*)gemm_fp8_pair_group_kernel, (const void*)gemm_fp8_pair_wide_kernel}) {
+    const cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 bool make_gemm_group(const GemmDesc* probs, uint32_t n, int num_sms, Launch* out) {
-  if (n < 2 || n > 8) return false;
-  GemmGroupParams g{};
-  const uint32_t pairs = (uint32_t)num_sms / 2u, w = choose_width(probs, n, pairs);
-  uint32_t tiles = 0;
+  uint32_t nops = 0;
   for (uint32_t i = 0; i < n; ++i) {
     if (!gemm_uses_pair(probs[i].M)) return false;
-    tiles += tiles_of(probs[i], kTileWidths[w]);
-    g.tile_end[i] = tiles;
-    fill_problem(probs[i], w, &g.prob[i]);
+    nops += probs[i].nseg;
   }
-  g.n = n;
-  Launch l;
-  l.func = (const void*)gemm_fp8_pair_group_kernel;
-  l.grid = dim3(2u * (tiles < pairs ? tiles : pairs), 1, 1);
-  l.block = dim3(THREADS, 1, 1);
-  l.smem = SMEM_BYTES;
-  l.set(g);
-  *out = l;
+  if (n < 2 || n > kMaxProblems || nops > kMaxOperands) return false;
+  *out = make_any(probs, n, nops, num_sms);
   return true;
 }
 
-Launch make_gemm(const GemmDesc& d, int num_sms) {
-  const uint32_t pairs = (uint32_t)num_sms / 2u, w = choose_width(&d, 1, pairs), tiles = tiles_of(d, kTileWidths[w]);
-  GemmParams p;
-  fill_problem(d, w, &p);
-  Launch l;
-  l.func = (const void*)gemm_fp8_pair_kernel;
-  l.grid = dim3(2u * (tiles < pairs ? tiles : pairs), 1, 1);
-  l.block = dim3(THREADS, 1, 1);
-  l.smem = SMEM_BYTES;
-  l.set(p);
-  return l;
-}
+Launch make_gemm(const GemmDesc& d, int num_sms) { return make_any(&d, 1, d.nseg, num_sms); }
 
 }  // namespace qe

@@ -7,6 +7,7 @@
 #include <cuda_runtime.h>
 
 #include <cstdint>
+#include <vector>
 
 namespace qe {
 
@@ -91,27 +92,32 @@ struct ArenaReduceParams {
 constexpr uint32_t kNumTileWidths = 3;
 constexpr uint32_t kTileWidths[kNumTileWidths] = {256, 128, 64};
 
-struct GemmParams {
+// One pair of operands: D = (A . B^T) * (*alpha_a * *alpha_b).
+struct GemmOperands {
   CUtensorMap tmA;             // A: 128 rows x 128 contraction bytes, 128-byte swizzle
   CUtensorMap tmB;             // B: tile_n / 2 rows x 128 contraction bytes (MN-major: swizzled over tile_n / 2 bytes)
+  const float* alpha_a;
+  const float* alpha_b;
+};
+
+struct GemmParams {
   CUtensorMap tmD;             // D [M, N] (bf16, FP32 or FP8 bytes), box 32 x 32, for the epilogue's bulk stores
   uint32_t M, N, Kc;
   uint32_t tile_n;             // columns per tile
+  uint32_t op0, nseg;          // its operand pairs in the launch's list; more than one: an FP32 output (epi 1, 2) that
+                               // receives the products one after the other, as nseg launches would have added them
   uint32_t idesc;              // tcgen05 instruction descriptor (formats, majors, shape)
   uint32_t b_desc_hi, b_step;  // B's shared-memory descriptor: high word; address advance (16-byte units) per 32 contraction elements
   uint32_t a_mn, b_mn;         // operand given MN-major (as [Kc, M] / [Kc, N] bytes)
-  const float* alpha_a;
-  const float* alpha_b;
-  void* out;                   // bf16 or FP32 [M, N], row pitch ldo elements
   uint32_t ldo;
-  int32_t epi;                 // 0 bf16 (+amax), 1 FP32 overwrite, 2 FP32 accumulate, 3 FP8 hand-off (below)
+  void* out;                   // bf16 or FP32 [M, N], row pitch ldo elements
   uint32_t* amax_bits;         // or null
   // epi 3: the bf16-rounded result is not stored; it is quantised for the consuming linear as that linear's own
   // cast kernel would have done: q = fp8(fp32(bf16(D)) * *out_scale), max|bf16(D)| also into *amax_bits2, and
   // *sinv_dst = *sinv_src (the consumer's tape snapshot)
   const float* out_scale;
   int32_t out_fmt;             // 0 = E4M3, 1 = E5M2
-  uint32_t pad0;
+  int32_t epi;                 // 0 bf16 (+amax), 1 FP32 overwrite, 2 FP32 accumulate, 3 FP8 hand-off (above)
   uint32_t* amax_bits2;        // or null
   const float* sinv_src;
   float* sinv_dst;
@@ -119,21 +125,30 @@ struct GemmParams {
   CommitParams commit;         // performed by the last CTA to finish (commit.st != null)
 };
 
-// One GEMM as the launch builders take it: everything the kernel needs except what follows from the tile width, which
-// the launch chooses (tmA, tmB, tile_n, idesc, b_desc_hi and b_step are filled from the fields below).
+constexpr uint32_t kMaxSegments = 8;
+
+// One GEMM as the launch builders take it: everything the kernel needs except what follows from the tile width and the
+// place in the launch (operand list, tile_n, idesc, b_desc_hi, b_step), which is filled from the fields below.
 struct GemmDesc : GemmParams {
   uint32_t a_fmt, b_fmt;       // 0 = E4M3, 1 = E5M2
-  const CUtensorMap* mapA;
-  const CUtensorMap* mapB;     // one map per tile width
+  struct Operands {
+    const CUtensorMap* mapA;
+    const CUtensorMap* mapB;   // one map per tile width
+    const float* alpha_a;
+    const float* alpha_b;
+  } ops[kMaxSegments];
+  GemmDesc() : GemmParams{}, a_fmt(0), b_fmt(0), ops{} { nseg = 1; }
 };
 
-// Up to eight independent GEMMs computed by one launch: tiles are numbered problem after problem.
-struct GemmGroupParams {
+// Independent GEMMs computed by one launch: tiles are numbered problem after problem.
+template <int NP, int NOPS>
+struct GemmLaunchParams {
   uint32_t n;
-  uint32_t tile_end[8];        // cumulative tile counts
-  uint32_t pad[7];
-  GemmParams prob[8];
+  uint32_t tile_end[NP];       // cumulative tile counts
+  GemmParams prob[NP];
+  GemmOperands op[NOPS];
 };
+constexpr uint32_t kMaxProblems = 16, kMaxOperands = 40;  // of the largest launch
 
 // ORs the status words of up to 64 layers into *out (first chunk: out = OR; later chunks: out |= OR).
 struct StatusGatherParams {
@@ -148,13 +163,11 @@ struct Launch {
   const void* func = nullptr;
   dim3 grid{1, 1, 1}, block{1, 1, 1};
   uint32_t smem = 0;
-  uint32_t nbytes = 0;
-  alignas(64) unsigned char params[4864];
+  std::vector<unsigned char> params;
   template <class P>
   void set(const P& p) {
-    static_assert(sizeof(P) <= sizeof(params), "parameter block too large");
-    nbytes = sizeof(P);
-    __builtin_memcpy(params, &p, sizeof(P));
+    const unsigned char* b = reinterpret_cast<const unsigned char*>(&p);
+    params.assign(b, b + sizeof(P));
   }
 };
 
@@ -167,8 +180,9 @@ Launch make_amax_pass2(const AmaxParams& p);
 Launch make_accumulate(const AccumParams& p);
 Launch make_arena_reduce(const ArenaReduceParams& p);
 Launch make_gemm(const GemmDesc& p, int num_sms);
-// One launch for n = 2..8 GEMMs (each may carry its own commit tail); false if the group cannot be formed (a problem's M
-// is not a multiple of 256), in which case the caller launches them one by one.
+// One launch for n = 2..kMaxProblems GEMMs of kMaxOperands operand pairs at most (each may carry its own commit tail);
+// false if the group cannot be formed (a problem's M is not a multiple of 256), in which case the caller launches them
+// one by one.
 bool make_gemm_group(const GemmDesc* probs, uint32_t n, int num_sms, Launch* out);
 cudaError_t gemm_prepare();  // opt in to the dynamic shared memory the GEMM needs (once per device)
 bool gemm_uses_pair(uint32_t M);  // whole 256-row tiles: may share launches and take MN-major operands

@@ -147,7 +147,7 @@ cudaError_t launch_pdl(const qe::Launch& l, cudaStream_t stream) {
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  void* args[1] = {const_cast<unsigned char*>(l.params)};
+  void* args[1] = {const_cast<unsigned char*>(l.params.data())};
   return cudaLaunchKernelExC(&cfg, l.func, args);
 }
 
@@ -226,13 +226,13 @@ int32_t replay_graph(qe_ctx* ctx, ActionGraph* g, const std::vector<qe::Launch>&
   for (size_t i = 0; i < ls.size(); ++i) {
     const qe::Launch& now = ls[i];
     qe::Launch& was = g->launches[i];
-    const bool same = now.func == was.func && now.nbytes == was.nbytes && now.smem == was.smem &&
+    const bool same = now.func == was.func && now.params.size() == was.params.size() && now.smem == was.smem &&
                       now.grid.x == was.grid.x && now.grid.y == was.grid.y && now.block.x == was.block.x &&
-                      std::memcmp(now.params, was.params, now.nbytes) == 0;
+                      std::memcmp(now.params.data(), was.params.data(), now.params.size()) == 0;
     if (same) continue;
     // caller-visible pointers (x, y, gradient destination) or the accumulate flag changed: patch the node in place
     cudaKernelNodeParams np{};
-    void* args[1] = {const_cast<unsigned char*>(now.params)};
+    void* args[1] = {const_cast<unsigned char*>(now.params.data())};
     np.func = const_cast<void*>(now.func);
     np.gridDim = now.grid;
     np.blockDim = now.block;
@@ -444,15 +444,12 @@ void add_forward(qe_layer* L, uint32_t p, const void* x, void* y, std::vector<qe
   const uint32_t T = L->cfg.T, K = L->cfg.K, N = L->cfg.N;
   if (x && cast_out) *cast_out = quant_params(L, x, L->Xq[p], L->XqT[p], T, K, QE_CLASS_X, &L->st->slot_sinv_X[p], QE_E4M3);
   else if (x) ls.push_back(quant_launch(L, x, L->Xq[p], L->XqT[p], T, K, QE_CLASS_X, &L->st->slot_sinv_X[p], QE_E4M3));
-  qe::GemmDesc gp{};
-  gp.mapA = &L->tmXq_A[p];
-  gp.mapB = L->tmWq_B;
+  qe::GemmDesc gp;
+  gp.ops[0] = {&L->tmXq_A[p], L->tmWq_B, &L->st->slot_sinv_X[p], &L->st->cache_sinv_W};
   gp.M = T;
   gp.N = N;
   gp.Kc = K;
   gp.a_fmt = gp.b_fmt = QE_E4M3;
-  gp.alpha_a = &L->st->slot_sinv_X[p];
-  gp.alpha_b = &L->st->cache_sinv_W;
   gp.ldo = N;
   if (next) {
     gp.out = next->Xq[pn];
@@ -483,18 +480,15 @@ void add_dI(qe_layer* L, uint32_t p, const void* dy, void* dx, std::vector<qe::L
   const uint32_t T = L->cfg.T, K = L->cfg.K, N = L->cfg.N;
   if (dy && cast_out) *cast_out = quant_params(L, dy, L->Gq[p], L->GqT[p], T, N, QE_CLASS_G, &L->st->slot_sinv_G[p], QE_E5M2);
   else if (dy) ls.push_back(quant_launch(L, dy, L->Gq[p], L->GqT[p], T, N, QE_CLASS_G, &L->st->slot_sinv_G[p], QE_E5M2));
-  qe::GemmDesc gp{};
+  qe::GemmDesc gp;
   const bool b_mn = L->WqT == nullptr;  // no transposed weight copy: Wq [N,K] is B in MN-major form
-  gp.mapA = &L->tmGq_A[p];
-  gp.mapB = L->tmWq_dI;
+  gp.ops[0] = {&L->tmGq_A[p], L->tmWq_dI, &L->st->slot_sinv_G[p], &L->st->cache_sinv_W};
   gp.M = T;
   gp.N = K;
   gp.Kc = N;
   gp.a_fmt = QE_E5M2;
   gp.b_fmt = QE_E4M3;
   gp.b_mn = b_mn;
-  gp.alpha_a = &L->st->slot_sinv_G[p];
-  gp.alpha_b = &L->st->cache_sinv_W;
   gp.ldo = K;
   if (prev) {
     gp.out = prev->Gq[pp];
@@ -522,18 +516,16 @@ void add_dI(qe_layer* L, uint32_t p, const void* dy, void* dx, std::vector<qe::L
 // write the temporary instead (copied-gradient comparison path).
 qe::GemmDesc dW_gemm(qe_layer* L, uint32_t p, float* dst, int32_t accumulate, float* temp) {
   const uint32_t T = L->cfg.T, K = L->cfg.K, N = L->cfg.N;
-  qe::GemmDesc gp{};
+  qe::GemmDesc gp;
   const bool mn = L->GqT[p] == nullptr;  // Gq [T,N] and Xq [T,K] themselves, read as MN-major operands
-  gp.mapA = &L->tmGqT_A[p];
-  gp.mapB = L->tmXqT_B[p];
+  // (scales: the snapshots taken when dY_m and X_m were quantised, never the current state)
+  gp.ops[0] = {&L->tmGqT_A[p], L->tmXqT_B[p], &L->st->slot_sinv_G[p], &L->st->slot_sinv_X[p]};
   gp.M = N;
   gp.N = K;
   gp.Kc = T;
   gp.a_fmt = QE_E5M2;
   gp.b_fmt = QE_E4M3;
   gp.a_mn = gp.b_mn = mn;
-  gp.alpha_a = &L->st->slot_sinv_G[p];  // snapshots taken when dY_m and X_m were quantised, never the current state
-  gp.alpha_b = &L->st->slot_sinv_X[p];
   gp.ldo = K;
   gp.amax_bits = nullptr;
   gp.status = &L->st->status;

@@ -209,9 +209,12 @@ int32_t qe_forward_dI_pair(qe_layer* Lf, uint32_t mb, uint64_t gen, const void* 
 
 // ------------------------------------------------------------------------------------------------ independent actions
 namespace {
+constexpr uint32_t kMaxRound = QE_MAX_TOGETHER + QE_STEP_MAX_PRODUCTS;  // actions of a round of the whole-step call
+static_assert(2 * QE_MAX_TOGETHER <= qe::kMaxProblems && kMaxRound <= qe::kMaxOperands, "a round fits into one launch");
+
 struct TogetherPrep {
-  int32_t refresh[QE_MAX_TOGETHER] = {}, acc[QE_MAX_TOGETHER] = {};
-  uint32_t slot[QE_MAX_TOGETHER] = {};
+  int32_t refresh[kMaxRound] = {}, acc[kMaxRound] = {};
+  uint32_t slot[kMaxRound] = {};
   bool any_dw = false;
 };
 
@@ -246,12 +249,15 @@ int32_t together_prepare(qe_ctx* ctx, const qe_action* acts, uint32_t n, float* 
   return QE_OK;
 }
 
-// the launches: the casts in one launch, then every GEMM of whole 256-row tiles in one launch
+// the launches: the casts in one launch, then every GEMM of whole 256-row tiles in one launch; weight gradients of
+// several microbatches of one layer (whole-step call only) become one GEMM that adds their products up
 int32_t together_build(qe_ctx* ctx, const qe_action* acts, uint32_t n, const TogetherPrep& pr, float* grad,
                        std::vector<qe::Launch>& ls, Fnv* h) {
-  qe::GemmDesc g[QE_MAX_TOGETHER];
+  qe::GemmDesc g[2 * QE_MAX_TOGETHER];
+  const qe_layer* owner[2 * QE_MAX_TOGETHER];
   qe::QuantParams casts[QE_MAX_TOGETHER];
   std::vector<qe::GemmDesc> singles;
+  std::vector<const qe_layer*> single_owner;
   uint32_t ng = 0, n_chain = 0, n_dw = 0, n_casts = 0;
   for (int pass = 0; pass < 2; ++pass) {  // F and dI first (others wait for them), the weight gradients' tiles after theirs
     for (uint32_t i = 0; i < n; ++i) {
@@ -271,11 +277,23 @@ int32_t together_build(qe_ctx* ctx, const qe_action* acts, uint32_t n, const Tog
       } else {
         gp = dW_gemm(L, pr.slot[i], grad + a.grad_offset, pr.acc[i], nullptr);
       }
-      if (qe::gemm_uses_pair(gp.M)) {
+      const bool paired = qe::gemm_uses_pair(gp.M);
+      if (paired) (a.kind == QE_ACT_DW ? n_dw : n_chain) += 1;
+      qe::GemmDesc* sum = nullptr;  // this layer's weight gradient of an earlier microbatch, which takes this one in
+      if (a.kind == QE_ACT_DW) {
+        for (uint32_t j = n_chain; paired && j < ng; ++j)
+          if (owner[j] == L) sum = &g[j];
+        for (size_t j = 0; !paired && j < singles.size(); ++j)
+          if (single_owner[j] == L && singles[j].epi != 0) sum = &singles[j];
+      }
+      if (sum) {
+        sum->ops[sum->nseg++] = gp.ops[0];
+      } else if (paired) {
+        owner[ng] = L;
         g[ng++] = gp;
-        (a.kind == QE_ACT_DW ? n_dw : n_chain) += 1;
       } else {
         singles.push_back(gp);  // a half-filled last row tile: a launch of its own
+        single_owner.push_back(L);
       }
       if (h) {
         h->mix(&a.kind, sizeof(a.kind));
@@ -288,7 +306,7 @@ int32_t together_build(qe_ctx* ctx, const qe_action* acts, uint32_t n, const Tog
   // longest tiles first (their contraction length decides a tile's duration): the launch's last, partial wave is then
   // made of short tiles.  The weight gradients (contraction over T only) stay behind the others.
   std::stable_sort(g, g + n_chain, [](const qe::GemmDesc& x, const qe::GemmDesc& y) { return x.Kc > y.Kc; });
-  std::stable_sort(g + n_chain, g + ng, [](const qe::GemmDesc& x, const qe::GemmDesc& y) { return x.Kc > y.Kc; });
+  std::stable_sort(g + n_chain, g + ng, [](const qe::GemmDesc& x, const qe::GemmDesc& y) { return x.Kc * x.nseg > y.Kc * y.nseg; });
   if (n_casts >= 2) ls.push_back(qe::make_quantize_multi(casts, n_casts));  // all casts of the call in one launch
   else if (n_casts == 1) ls.push_back(qe::make_quantize(casts[0]));
   for (const qe::GemmDesc& gp : singles) ls.push_back(qe::make_gemm(gp, ctx->dev->num_sms));
@@ -410,6 +428,14 @@ int32_t qe_step_run(qe_ctx* ctx, qe_layer* const* layers, uint32_t n_layers, con
   // the kind, F before dI before dW of a (layer, microbatch), a free tape slot -- looking `window` units ahead, and a
   // round goes out as qe_run_together would issue it.  If no such plan exists (an illegal list) the action-by-action
   // pass below runs instead and reports the failing action.
+  // Weight gradients: qe_plan_step collects a layer's and lets one launch add them up, as far as a sum stays within 8192
+  // tokens.  Few tokens make the destination's traffic the cost of a weight gradient: eight microbatches of 256 tokens
+  // through a 4096 / 11008 layer 2860 -> 1890 us a step.  With 2048 tokens a sum of four gains 2 %, of two or eight
+  // nothing; with 4096 the traffic is small, and tiles that last several times as long leave more of the chip idle at the
+  // end of a launch (a 4096 / 14336 block: 20.5 ms one by one, 21.2 ms in sums), so there they go out one by one.
+  uint32_t T_max = 0;
+  for (uint32_t l = 0; l < n_layers; ++l) T_max = std::max(T_max, layers[l]->cfg.T);
+  const uint32_t max_sum = T_max >= 4096 ? 1u : std::min(qe::kMaxSegments, 8192u / T_max);
   std::vector<std::vector<uint32_t>> rounds;  // indices into actions[]
   if (!temp && ctx->step_window > 1) {
     std::vector<uint32_t> slots(n_layers), live(n_layers), round_of(n_actions);
@@ -418,29 +444,59 @@ int32_t qe_step_run(qe_ctx* ctx, qe_layer* const* layers, uint32_t n_layers, con
       live[l] = layers[l]->contract->live_tapes();
     }
     uint32_t n_rounds = 0;
-    if (qe_plan_rounds(actions, n_actions, n_layers, M, slots.data(), live.data(), ctx->step_window, QE_MAX_TOGETHER,
+    if ((max_sum > 1 && qe_plan_step(actions, n_actions, n_layers, M, slots.data(), live.data(), ctx->step_window,
+                                     QE_MAX_TOGETHER, max_sum, round_of.data(), &n_rounds) == QE_OK) ||
+        qe_plan_rounds(actions, n_actions, n_layers, M, slots.data(), live.data(), ctx->step_window, QE_MAX_TOGETHER,
                        round_of.data(), &n_rounds) == QE_OK) {
       rounds.resize(n_rounds);
       for (uint32_t i = 0; i < n_actions; ++i) rounds[round_of[i]].push_back(i);
     }
   }
   for (size_t r = 0; r < rounds.size() && st == QE_OK; ++r) {
-    qe_action acts[QE_MAX_TOGETHER];
-    uint32_t na = 0;
-    for (uint32_t gi : rounds[r]) {
-      const qe_step_action& a = actions[gi];
-      const size_t u = (size_t)a.layer * M + a.mb;
-      qe_layer* L = layers[a.layer];
-      if (a.kind == QE_ACT_F) acts[na++] = qe_action{QE_ACT_F, a.mb, L->contract->e_W, L, io[u].x_dev, io[u].y_dev, &tapes[u], 0};
-      else if (a.kind == QE_ACT_DI) acts[na++] = qe_action{QE_ACT_DI, 0, 0, L, io[u].dy_dev, io[u].dx_dev, &tapes[u], 0};
-      else acts[na++] = qe_action{QE_ACT_DW, 0, 0, L, nullptr, nullptr, &tapes[u], offsets[a.layer]};
-    }
+    // check -> commit per action (all F first: a slot that a dW of the round releases is not theirs to take), then the
+    // launches of those that passed
+    qe_action acts[kMaxRound];
     TogetherPrep pr;
-    if ((st = together_prepare(ctx, acts, na, grad, grad_elems, &pr)) != QE_OK || (st = together_build(ctx, acts, na, pr, grad, ls, nullptr)) != QE_OK) {
-      k = rounds[r][0];  // (reported as the index of the first action of the failing round)
-      break;
+    uint32_t na = 0;
+    for (uint32_t kind = QE_ACT_F; kind <= QE_ACT_DW && st == QE_OK; ++kind) {
+      for (uint32_t gi : rounds[r]) {
+        const qe_step_action& a = actions[gi];
+        if (a.kind != kind) continue;
+        const size_t u = (size_t)a.layer * M + a.mb;
+        qe_layer* L = layers[a.layer];
+        const uint64_t slice = (uint64_t)L->cfg.N * L->cfg.K;
+        const void* in = a.kind == QE_ACT_F ? io[u].x_dev : io[u].dy_dev;
+        void* out = a.kind == QE_ACT_F ? io[u].y_dev : io[u].dx_dev;
+        if (a.kind == QE_ACT_DW) {
+          st = !grad ? fail(QE_ERR_BAD_ARG, "gradient buffer is null")
+                     : qe_contract_dW_check(L->contract, &tapes[u], (uint64_t)(uintptr_t)grad, grad_elems, offsets[a.layer], slice, &pr.acc[na]);
+          pr.slot[na] = tapes[u].ref.slot;
+          if (st == QE_OK) st = qe_contract_dW_commit(L->contract, &tapes[u], (uint64_t)(uintptr_t)grad, offsets[a.layer], slice);
+        } else if (!in || !out || (((uintptr_t)in | (uintptr_t)out) & 15u)) {
+          st = fail(QE_ERR_BAD_ARG, "input / output null or misaligned");
+        } else if (a.kind == QE_ACT_F) {
+          st = qe_contract_forward_check(L->contract, a.mb, L->contract->e_W, &pr.refresh[na], &pr.slot[na]);
+          if (st == QE_OK) st = qe_contract_forward_commit(L->contract, a.mb, &tapes[u]);
+        } else {
+          st = qe_contract_dI_check(L->contract, &tapes[u]);
+          pr.slot[na] = tapes[u].ref.slot;
+          if (st == QE_OK) st = qe_contract_dI_commit(L->contract, &tapes[u]);
+        }
+        if (st != QE_OK) {
+          k = gi;
+          break;
+        }
+        acts[na++] = qe_action{a.kind, a.mb, 0, L, in, out, &tapes[u], offsets[a.layer]};
+      }
     }
-    st = together_commit(acts, na, grad, pr);
+    char why[512];  // (a build can only fail on a CUDA error, which then is the one to report)
+    if (st != QE_OK) std::snprintf(why, sizeof(why), "%s", qe_last_error());
+    const int32_t built = na ? together_build(ctx, acts, na, pr, grad, ls, nullptr) : QE_OK;
+    if (st != QE_OK) st = fail(st, "%s", why);
+    else if (built != QE_OK) {
+      st = built;
+      k = rounds[r][0];
+    }
   }
   if (!rounds.empty()) k = st == QE_OK ? n_actions : k;
 

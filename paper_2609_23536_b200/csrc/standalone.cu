@@ -66,7 +66,7 @@ int32_t qe_arena_reduce(const void* views, uint64_t view_elems, uint32_t M, floa
 
 // A standalone GEMM with its operand maps (the descriptor points at them).
 struct StandaloneGemm {
-  qe::GemmDesc desc{};
+  qe::GemmDesc desc;
   CUtensorMap mapA, mapB[qe::kNumTileWidths];
 };
 
@@ -87,8 +87,7 @@ static int32_t standalone_gemm(DeviceInfo* dev, const void* a, uint32_t a_fmt, u
   st = a_mn ? make_map(dev, &sg->mapA, a, Kc, M, 128) : make_map(dev, &sg->mapA, a, M, Kc, 128);
   if (st != QE_OK) return st;
   if ((st = make_b_maps(dev, sg->mapB, b, Nn, Kc, b_mn != 0)) != QE_OK) return st;
-  gp.mapA = &sg->mapA;
-  gp.mapB = sg->mapB;
+  gp.ops[0] = {&sg->mapA, sg->mapB, alpha_a, alpha_b};
   gp.M = M;
   gp.N = Nn;
   gp.Kc = Kc;
@@ -96,8 +95,6 @@ static int32_t standalone_gemm(DeviceInfo* dev, const void* a, uint32_t a_fmt, u
   gp.b_fmt = b_fmt;
   gp.a_mn = a_mn;
   gp.b_mn = b_mn;
-  gp.alpha_a = alpha_a;
-  gp.alpha_b = alpha_b;
   gp.out = d;
   gp.ldo = Nn;
   gp.epi = (int32_t)out_kind;

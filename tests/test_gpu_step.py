@@ -637,3 +637,37 @@ def test_run_together_host_equals_device_buffers_bitwise(qe):
     with pytest.raises(qe.QEError) as e:
         qe.run_together(ctx, [("F", L, 0, 0, torch.zeros((T, 256), dtype=torch.bfloat16).pin_memory(), None)], host=True)
     assert e.value.code == "BAD_ARG"
+
+
+@pytest.mark.parametrize("mode", [0, 1], ids=["eager", "graph"])
+@pytest.mark.parametrize("M,w,d,slots", [(3, 3, 0, 3), (9, 1, 8, 9), (12, 2, 3, 6)])
+def test_step_call_sums_of_weight_gradients_equal_one_launch_each_bitwise(qe, mode, M, w, d, slots):
+    """Sums of up to eight products, with and without a destination to add to, on whole and half-filled row tiles, ragged
+    column tiles and a gradient slice that is 16- but not 32-byte aligned."""
+    T, shapes = 384, [(256, 512), (640, 384), (1152, 2304)]
+    s = sched(M, w, d)
+    acts = _actions(s, len(shapes))
+    offs, total = [], 4
+    for K, N in shapes:
+        offs.append(total)
+        total += K * N + 4
+    results = []
+    for step_window in (1, 6):  # 1: action by action
+        ctx = qe.Context(mode, step_window=step_window)
+        layers = [qe.Layer(ctx, T, K, N, 4, 0, max(slots, peak_live(s)), inputs.weights("SU", 0, j, N, K).to(DEV), unit=j) for j, (K, N) in enumerate(shapes)]
+        X = [[inputs.activations("SU", 0, 0, j, m, T, K).to(DEV) for j, (K, N) in enumerate(shapes)] for m in range(M)]
+        dY = [[inputs.upstream_grads("SU", 0, 0, j, m, T, N).to(DEV) for j, (K, N) in enumerate(shapes)] for m in range(M)]
+        Y = [[torch.zeros((T, N), dtype=torch.bfloat16, device=DEV) for K, N in shapes] for m in range(M)]
+        dX = [[torch.zeros((T, K), dtype=torch.bfloat16, device=DEV) for K, N in shapes] for m in range(M)]
+        grad = torch.full((total,), 3.0, device=DEV)
+        plan = qe.StepPlan(ctx, layers, acts, M, X, Y, dY, dX, grad, offs)
+        for _ in range(2):
+            plan.run()
+            qe.optimizer_boundary_all(layers, M)
+        results.append(_snapshot(layers, Y, dX, grad))
+        for j, (K, N) in enumerate(shapes):  # nothing outside the slices was touched
+            assert bool((grad[offs[j] - 4:offs[j]] == 3.0).all())
+    for a, b in zip(*(r[0] + r[1] + [r[2].view(np.uint32)] for r in results)):
+        assert np.array_equal(a, b)
+    for a, b in zip(results[0][3], results[1][3]):
+        assert state_equal({**a, "slots": []}, {**b, "slots": []})

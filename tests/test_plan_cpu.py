@@ -100,3 +100,54 @@ def test_native_planner_refuses_lists_without_a_plan(qe):
     assert len(qe.plan_rounds([("F", 0, 0), ("dI", 0, 0), ("dW", 0, 0)], 1, 1, 2, 4, 8, live_now=[1])) == 3
     with pytest.raises(qe.QEError):
         qe.plan_rounds([("F", 0, 0), ("dI", 0, 0), ("dW", 0, 0)], 1, 1, 2, 4, 8, live_now=[2])
+
+
+# ------------------------------------------------------------------------------------------ the whole-step call's plan
+@pytest.mark.parametrize("M,w,d", [(4, 1, 0), (8, 3, 3), (8, 1, 2), (6, 2, 1), (32, 3, 3), (5, 5, 5)])
+@pytest.mark.parametrize("n", [1, 3, 12])
+@pytest.mark.parametrize("window,group,sums", [(2, 4, 1), (4, 8, 2), (6, 8, 8)])
+def test_step_plan_is_legal_and_sums_weight_gradients(qe, M, w, d, n, window, group, sums):
+    s = sched(M, w, d)
+    slots = peak_live(s)
+    rounds = qe.plan_rounds(_actions(s, n), n, M, slots, window, group, max_sum=sums)
+    acts = [x for g in rounds for x in g]
+    assert sorted(acts) == sorted(_actions(s, n))
+    when = {x: r for r, g in enumerate(rounds) for x in g}
+    live = [0] * n
+    for r, g in enumerate(rounds):
+        chain = [x for x in g if x[0] != "dW"]
+        assert len(chain) <= group and len({(a, l) for a, l, m in chain}) == len(chain)
+        of = {}
+        for a, l, m in g:
+            if a == "dW":
+                of.setdefault(l, []).append(m)
+        assert len(of) <= group and all(len(v) <= sums for v in of.values()) and sum(map(len, of.values())) <= 32
+        for l, ms in of.items():
+            assert ms == list(range(ms[0], ms[0] + len(ms)))                 # consecutive, in microbatch order
+            assert ms[0] == 0 or when[("dW", l, ms[0] - 1)] < r
+            assert all(when[("dI", l, m)] < r for m in ms)
+        for a, l, m in chain:
+            if a == "F":
+                assert (l == 0 or when[("F", l - 1, m)] < r) and (m == 0 or when[("F", l, m - 1)] < r)
+                live[l] += 1
+                assert live[l] <= slots
+            else:
+                assert when[("F", l, m)] < r and (l == n - 1 or when[("dI", l + 1, m)] < r) and (m == 0 or when[("dI", l, m - 1)] < r)
+        for l, ms in of.items():
+            live[l] -= len(ms)
+    batches = sum(len({l for a, l, m in g if a == "dW"}) for g in rounds)
+    if (M, w, d) == (8, 3, 3) and sums == 8:
+        assert batches == 2 * n  # four microbatches at a time: seven slots, three of them in flight
+    with pytest.raises(qe.QEError) as e:  # tapes that another list left alive fill the pool
+        qe.plan_rounds(_actions(s, n), n, M, slots, window, group, max_sum=sums, live_now=[slots] * n)
+    assert e.value.code == "ORDER"
+
+
+def test_step_plan_refuses_repeated_and_malformed_actions(qe):
+    ok = [("F", 0, 0), ("dI", 0, 0), ("dW", 0, 0)]
+    assert qe.plan_rounds(ok, 1, 1, 1, 4, 8, max_sum=8) == [[x] for x in ok]
+    for bad, code in (([("F", 0, 0)] + ok, "ORDER"), (ok[:2] + [("dI", 0, 0)], "ORDER"), ([("dW", 0, 0)], "ORDER"),
+                      ([("F", 3, 0)], "BAD_ARG"), ([("F", 0, 1)], "BAD_ARG")):
+        with pytest.raises(qe.QEError) as e:
+            qe.plan_rounds(bad, 1, 1, 2, 4, 8, max_sum=8)
+        assert e.value.code == code
