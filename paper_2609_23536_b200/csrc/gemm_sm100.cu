@@ -36,6 +36,7 @@
 // word, raises a CTA-wide abort flag that all other waits observe, and the CTA falls through to its common exit
 // where tensor memory is released.
 #include <cuda_bf16.h>
+#include <type_traits>
 #include <cuda_fp8.h>
 
 #include "commit.cuh"
@@ -103,8 +104,11 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
   }
 }
 
-__device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_bar) {  // barrier may live in the peer CTA
-  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_bar) : "memory");
+// Arrival on a barrier that may live in the peer CTA.  What it announces are tensor-memory reads, ordered by the
+// tcgen05 fences on both sides, so it need not be a release at cluster scope: that waits for the thread's outstanding
+// stores too, ~1000 clocks per drained accumulator.
+__device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_bar) {
+  asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_bar) : "memory");
 }
 // Address of the same shared-memory location in CTA `rank` of the cluster (shared::cluster window).
 __device__ __forceinline__ uint32_t map_to_cta(uint32_t saddr, uint32_t rank) {
@@ -189,23 +193,14 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
       : "r"(taddr)
       : "memory");
 }
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-      : "r"(taddr)
-      : "memory");
-}
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
 // One row of a 32 x 32 FP32 tile for the bulk-store unit: 128-byte rows, 128-byte swizzle (chunk c of row r sits at
 // c ^ (r & 7)).
-__device__ __forceinline__ void st_tile_f32(uint32_t buf, int row, const float (&v)[32]) {
+__device__ __forceinline__ void st_tile_f32(uint32_t buf, uint32_t row, const float (&v)[32]) {
 #pragma unroll
   for (int c = 0; c < 8; ++c) {
-    const uint32_t dst = buf + (uint32_t)row * 128u + (((uint32_t)c ^ ((uint32_t)row & 7u)) << 4);
+    const uint32_t dst = buf + row * 128u + (((uint32_t)c ^ (row & 7u)) << 4);
     asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(dst), "f"(v[4 * c]), "f"(v[4 * c + 1]), "f"(v[4 * c + 2]),
                  "f"(v[4 * c + 3])
                  : "memory");
@@ -405,6 +400,7 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
         const int ra = (int)(m0 + rank * BM), rb = (int)(n0 + rank * (tile_n / 2));
         for (uint32_t seg = 0; ok && seg < (SUMS ? p.nseg : 1u); ++seg) {
           const GemmOperands& op = ps.operands(p, seg);
+          const CUtensorMap *tmA = &op.tmA, *tmB = &op.tmB;
           for (uint32_t kb = 0; kb < num_kb; ++kb) {
             if (!(ok = mbar_wait(empty_bar(s), ph ^ 1u, abort_flag, status, ERR_PRODUCER))) break;
             const uint32_t a_dst = smem_base + s * STAGE_BYTES, b_dst = a_dst + A_BYTES;
@@ -414,10 +410,10 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
             // contraction-major operand: box = 128 K-bytes x rows at (k, row); MN-major operand (stored as [Kc, rows]):
             // box = row-bytes x 128 K-rows at (row, k).  Either way 128 bytes per row land in shared memory.
             const int ka = (int)(kb * BK);
-            if (p.a_mn) tma_load_2d_pair(a_dst, &op.tmA, bar, ra, ka);
-            else tma_load_2d_pair(a_dst, &op.tmA, bar, ka, ra);
-            if (p.b_mn) tma_load_2d_pair(b_dst, &op.tmB, bar, rb, ka);
-            else tma_load_2d_pair(b_dst, &op.tmB, bar, ka, rb);
+            if (p.a_mn) tma_load_2d_pair(a_dst, tmA, bar, ra, ka);
+            else tma_load_2d_pair(a_dst, tmA, bar, ka, ra);
+            if (p.b_mn) tma_load_2d_pair(b_dst, tmB, bar, rb, ka);
+            else tma_load_2d_pair(b_dst, tmB, bar, ka, rb);
             if (++s == STAGES) { s = 0; ph ^= 1u; }
           }
         }
@@ -481,56 +477,81 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
       const uint32_t col0 = n0 + half * (tile_n / 2);
       // 32 x 32 blocks of this warp: none in rows beyond M, fewer in a ragged last column tile; warp-uniform
       const uint32_t nch = blk_row0 >= p.M || col0 >= p.N ? 0u : min(tile_n / 64u, (p.N - col0) / 32u);
+      auto prefetch_next = [&] {  // the destination rows that this thread adds to in its next tile, towards L2
+        const uint32_t tile = snake_tile(wave + 1, first_tile, tile_step);
+        if (tile >= num_tiles) return;
+        QE_TILE_PROBLEM();
+        (void)num_kb;
+        if (p.nseg == 1 || p.epi != 2) return;
+        uint32_t m0, n0;
+        tile_coords(local_tile, tiles_m, tiles_n, m_fastest, tile_n, m0, n0);
+        const uint32_t row = m0 + rank * BM + quad * 32u + (uint32_t)lane, col = n0 + half * (tile_n / 2);
+        if (row >= p.M || col >= p.N) return;
+        const char* d = reinterpret_cast<const char*>(reinterpret_cast<const float*>(p.out) + (size_t)row * p.ldo + col);
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if (j * 32u < min(tile_n / 2, p.N - col)) asm volatile("prefetch.global.L2 [%0];" ::"l"(d + 128 * j));
+      };
       if (SUMS && p.nseg > 1) {
         // Several products for one FP32 tile (the weight gradients of several microbatches): the tile's running value
         // stays in registers and every product is added to it in order, each with its own scale -- the additions
         // launches of their own would have done in L2, at one read and one write of the destination instead of one
         // per product.  What is added to is fetched while the first product is being computed.
         float v[4][32];
+        float* const dst = reinterpret_cast<float*>(p.out) + (size_t)(blk_row0 + lane) * p.ldo + col0;
         if (p.epi == 2) {
-          const float* src = reinterpret_cast<const float*>(p.out) + (size_t)(blk_row0 + lane) * p.ldo + col0;
 #pragma unroll
           for (int ch = 0; ch < 4; ++ch)
-            if ((uint32_t)ch < nch) ld_row32(src + ch * 32, v[ch]);
+            if ((uint32_t)ch < nch) ld_row32(dst + ch * 32, v[ch]);
         }
-        for (uint32_t seg = 0; seg < (SUMS ? p.nseg : 1u); ++seg) {
-          const GemmOperands& op = ps.operands(p, seg);
-          const float alpha = __fmul_rn(*op.alpha_a, *op.alpha_b);
-          const bool overwrite = seg == 0 && p.epi == 1;
-          if (!(ok = mbar_wait(tfull_bar(acc), acc_ph, abort_flag, status, ERR_EPILOGUE))) break;
+        prefetch_next();
+        // (lane i fetches the scales of product i: one chain of dependent loads per tile instead of one per product)
+        float my_alpha = 0.0f;
+        if ((uint32_t)lane < p.nseg) {
+          const GemmOperands& op = ps.operands(p, (uint32_t)lane);
+          my_alpha = __fmul_rn(*op.alpha_a, *op.alpha_b);
+        }
+        auto take = [&](uint32_t seg, auto first) {
+          const float alpha = __shfl_sync(0xffffffffu, my_alpha, (int)seg);
+          if (!(ok = mbar_wait(tfull_bar(acc), acc_ph, abort_flag, status, ERR_EPILOGUE))) return;
           tc_fence_after();
           const uint32_t t_row = tmem_base + ((quad * 32u) << 16) + acc * ACC_COLS + half * (tile_n / 2);
 #pragma unroll
-          for (int h = 0; h < 8; ++h) {
-            if ((uint32_t)h >= 2 * nch) break;
-            uint32_t rc[16];
-            tmem_ld16(t_row + h * 16u, rc);
+          for (int ch = 0; ch < 4; ++ch) {
+            if ((uint32_t)ch >= nch) break;
+            uint32_t rc[32];
+            tmem_ld32(t_row + ch * 32u, rc);
             tmem_ld_wait();
 #pragma unroll
-            for (int j = 0; j < 16; ++j) {
-              float& t = v[h / 2][(h & 1) * 16 + j];
+            for (int j = 0; j < 32; ++j) {
               const float d = __fmul_rn(__uint_as_float(rc[j]), alpha);
-              t = overwrite ? d : __fadd_rn(t, d);
+              v[ch][j] = decltype(first)::value ? d : __fadd_rn(v[ch][j], d);
             }
           }
           tc_fence_before();
           __syncwarp();
           if (lane == 0) mbar_arrive_cluster(acc ? tempty_leader1 : tempty_leader0);
           if (++acc == 2) { acc = 0; acc_ph ^= 1u; }
-        }
+        };
+        if (p.epi == 1) take(0, std::true_type{});
+        else take(0, std::false_type{});
+        for (uint32_t seg = 1; ok && seg < p.nseg; ++seg) take(seg, std::false_type{});
         if (!ok) break;
 #pragma unroll
         for (int ch = 0; ch < 4; ++ch) {
           if ((uint32_t)ch >= nch) break;
           if (lane == 0) tma_store_wait_read<0>();
           __syncwarp();
-          st_tile_f32(epi_smem, lane, v[ch]);
+          st_tile_f32(epi_smem, (uint32_t)lane, v[ch]);
           fence_async_smem();
           __syncwarp();
           if (lane == 0) tma_store_2d(&p.tmD, epi_smem, (int)(col0 + ch * 32u), (int)blk_row0);
         }
         continue;
       }
+      // (the variant that sums keeps no shared-memory addresses across its tiles: it needs the registers)
+      uint32_t ln = (uint32_t)lane;
+      if (SUMS) asm volatile("" : "+r"(ln));
       const float alpha = __fmul_rn(*ps.operands(p, 0).alpha_a, *ps.operands(p, 0).alpha_b);
       if (p.epi == 2) {
         // accumulate: pull this thread's destination row segment into L2, where the reduction will add to it, while
@@ -573,7 +594,7 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
           }
 #pragma unroll
           for (int c = 0; c < 4; ++c) {  // 64-byte rows, 64-byte swizzle: 16-byte chunk c of row r sits at c ^ ((r >> 1) & 3)
-            const uint32_t dst = buf + (uint32_t)lane * 64u + (((uint32_t)c ^ (((uint32_t)lane >> 1) & 3u)) << 4);
+            const uint32_t dst = buf + ln * 64u + (((uint32_t)c ^ ((ln >> 1) & 3u)) << 4);
             asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dst), "r"(o[4 * c]), "r"(o[4 * c + 1]),
                          "r"(o[4 * c + 2]), "r"(o[4 * c + 3])
                          : "memory");
@@ -608,7 +629,7 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
           }
 #pragma unroll
           for (int c = 0; c < 2; ++c) {
-            const uint32_t dst = buf + (uint32_t)lane * 32u + ((uint32_t)c << 4);
+            const uint32_t dst = buf + ln * 32u + ((uint32_t)c << 4);
             asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dst), "r"(q[4 * c]), "r"(q[4 * c + 1]),
                          "r"(q[4 * c + 2]), "r"(q[4 * c + 3])
                          : "memory");
@@ -625,7 +646,7 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
           float o[32];
 #pragma unroll
           for (int j = 0; j < 32; ++j) o[j] = __fmul_rn(__uint_as_float(rc[j]), alpha);
-          st_tile_f32(buf, lane, o);
+          st_tile_f32(buf, ln, o);
           fence_async_smem();
           __syncwarp();
           if (lane == 0) {
