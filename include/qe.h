@@ -342,9 +342,9 @@ int32_t qe_next_slot(const qe_layer*, uint32_t* slot_out);
  * All layers must belong to ctx.  io[layer * microbatches + mb] holds the device pointers of that unit (x, y for F;
  * dy, dx for dI).  Layer l's gradient slice is grad_buf_dev + offsets[l].  Every action is checked and committed on
  * the host exactly like the single calls; the kernels of the whole list are then issued behind ONE caller->execution
- * wait and ONE execution->caller event: in eager mode as plain launches, in graph mode as one captured graph that is
- * cached per (layers, actions) and replayed, with kernel-node parameters patched where pointers or the accumulate flag
- * differ from the previous replay.  dW runs on the execution stream here (QE_CTX_OVERLAP_DW does not apply).
+ * wait and ONE execution->caller event: in eager mode as plain launches, in graph mode as one captured graph (a list of more
+ * than 64 launches: several, issued one after the other while the next is prepared) that is cached per (layers, actions)
+ * and replayed, with kernel-node parameters patched where pointers or the accumulate flag differ from the previous replay.  dW runs on the execution stream here (QE_CTX_OVERLAP_DW does not apply).
  * Independent actions share launches, with bit-identical results (only the slot a tape lands in may differ from the
  * one-by-one order).  The list is read as units -- runs of actions of one kind and microbatch over distinct layers: a
  * forward, input-gradient or weight-gradient unit of the stage -- and cut into rounds of actions whose predecessors were

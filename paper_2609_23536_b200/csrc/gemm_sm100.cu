@@ -39,6 +39,9 @@
 #include <type_traits>
 #include <cuda_fp8.h>
 
+#include <cstddef>
+#include <cstring>
+
 #include "commit.cuh"
 #include "kernels.h"
 
@@ -748,46 +751,55 @@ uint32_t choose_width(const GemmDesc* d, uint32_t n, uint32_t pairs) {
   return w;
 }
 
-// The device's parameter block of one problem at a tile width, its operand pairs appended to op[].
-void fill_problem(const GemmDesc& d, uint32_t w, GemmParams* p, GemmOperands* op, uint32_t* nops) {
-  *p = d;
+// The device's parameter block of one problem at a tile width; its operand pairs start at op0.
+GemmParams problem_of(const GemmDesc& d, uint32_t w, uint32_t op0) {
+  GemmParams p = d;
   const uint32_t tile_n = kTileWidths[w], per_cta = tile_n / 2;
-  p->op0 = *nops;
-  for (uint32_t i = 0; i < d.nseg; ++i) op[(*nops)++] = GemmOperands{*d.ops[i].mapA, d.ops[i].mapB[w], d.ops[i].alpha_a, d.ops[i].alpha_b};
-  p->tile_n = tile_n;
+  p.op0 = op0;
+  p.tile_n = tile_n;
   // bits 4-5: accumulator format (1 = FP32); 7-9 / 10-12: A / B format (0 = E4M3, 1 = E5M2); 15 / 16: A / B major
   // (0 = contraction-major); 17-22: N >> 3; 24-28: M >> 4 (256 for a CTA pair).
-  p->idesc = (1u << 4) | (d.a_fmt << 7) | (d.b_fmt << 10) | (d.a_mn << 15) | (d.b_mn << 16) | ((tile_n >> 3) << 17) | ((TILE_M >> 4) << 24);
+  p.idesc = (1u << 4) | (d.a_fmt << 7) | (d.b_fmt << 10) | (d.a_mn << 15) | (d.b_mn << 16) | ((tile_n >> 3) << 17) | ((TILE_M >> 4) << 24);
   // An MN-major B tile has rows of per_cta bytes, swizzled over exactly that width; a contraction-major one rows of 128.
   const uint32_t row = d.b_mn ? per_cta : 128u;
-  p->b_desc_hi = desc_hi(row);
-  p->b_step = d.b_mn ? 32u * row / 16u : 2u;
+  p.b_desc_hi = desc_hi(row);
+  p.b_step = d.b_mn ? 32u * row / 16u : 2u;
+  return p;
 }
 
 template <int NP, int NOPS>
-Launch make_launch(const GemmDesc* probs, uint32_t n, int num_sms, const void* func) {
-  GemmLaunchParams<NP, NOPS> g{};
+Launch make_launch(const GemmDesc* probs, uint32_t n, uint32_t nops, int num_sms, const void* func) {
+  using P = GemmLaunchParams<NP, NOPS>;
+  static_assert(sizeof(P) <= sizeof(Launch::Block), "parameter block too large");
+  Launch l;
+  l.nbytes = sizeof(P);
+  l.params.resize(offsetof(P, op) + nops * sizeof(GemmOperands));  // (a step has hundreds of launches: no unused operands)
+  unsigned char* at = l.params.data();
   const uint32_t pairs = (uint32_t)num_sms / 2u, w = choose_width(probs, n, pairs);
-  uint32_t tiles = 0, nops = 0;
+  uint32_t tiles = 0, op = 0;
   for (uint32_t i = 0; i < n; ++i) {
     tiles += tiles_of(probs[i], kTileWidths[w]);
-    g.tile_end[i] = tiles;
-    fill_problem(probs[i], w, &g.prob[i], g.op, &nops);
+    std::memcpy(at + offsetof(P, tile_end) + i * sizeof(uint32_t), &tiles, sizeof(tiles));
+    const GemmParams p = problem_of(probs[i], w, op);
+    std::memcpy(at + offsetof(P, prob) + i * sizeof(GemmParams), &p, sizeof(p));
+    for (uint32_t j = 0; j < probs[i].nseg; ++j, ++op) {
+      const GemmDesc::Operands& d = probs[i].ops[j];
+      const GemmOperands o{*d.mapA, d.mapB[w], d.alpha_a, d.alpha_b};
+      std::memcpy(at + offsetof(P, op) + op * sizeof(GemmOperands), &o, sizeof(o));
+    }
   }
-  g.n = n;
-  Launch l;
+  std::memcpy(at + offsetof(P, n), &n, sizeof(n));
   l.func = func;
   l.grid = dim3(2u * (tiles < pairs ? tiles : pairs), 1, 1);
   l.block = dim3(threads_of(NOPS > NP), 1, 1);
   l.smem = SMEM_BYTES;
-  l.set(g);
   return l;
 }
 
 Launch make_any(const GemmDesc* probs, uint32_t n, uint32_t nops, int num_sms) {
-  if (n == 1 && nops == 1) return make_launch<1, 1>(probs, n, num_sms, (const void*)gemm_fp8_pair_kernel);
-  if (n <= 8 && nops == n) return make_launch<8, 8>(probs, n, num_sms, (const void*)gemm_fp8_pair_group_kernel);
-  return make_launch<kMaxProblems, kMaxOperands>(probs, n, num_sms, (const void*)gemm_fp8_pair_wide_kernel);
+  if (n == 1 && nops == 1) return make_launch<1, 1>(probs, n, nops, num_sms, (const void*)gemm_fp8_pair_kernel);
+  if (n <= 8 && nops == n) return make_launch<8, 8>(probs, n, nops, num_sms, (const void*)gemm_fp8_pair_group_kernel);
+  return make_launch<kMaxProblems, kMaxOperands>(probs, n, nops, num_sms, (const void*)gemm_fp8_pair_wide_kernel);
 }
 
 }  // namespace

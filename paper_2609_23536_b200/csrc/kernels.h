@@ -56,7 +56,7 @@ struct QuantParams {
 
 
 struct QuantMultiParams {
-  QuantParams q[8];            // none carries a commit tail
+  QuantParams q[8];
   uint32_t block_end[8];       // cumulative block counts
   uint32_t n;
   uint32_t pad[3];
@@ -163,11 +163,20 @@ struct Launch {
   const void* func = nullptr;
   dim3 grid{1, 1, 1}, block{1, 1, 1};
   uint32_t smem = 0;
-  std::vector<unsigned char> params;
+  std::vector<unsigned char> params;  // the parameter block, without an unused tail ...
+  uint32_t nbytes = 0;                // ... of a block of this size
   template <class P>
   void set(const P& p) {
     const unsigned char* b = reinterpret_cast<const unsigned char*>(&p);
     params.assign(b, b + sizeof(P));
+    nbytes = sizeof(P);
+  }
+  // The whole block as the runtime wants it (valid as long as the launch and the buffer are).
+  struct Block { alignas(64) unsigned char bytes[20480]; };
+  void* args_block(Block* tmp) const {
+    if (params.size() == nbytes) return const_cast<unsigned char*>(params.data());
+    __builtin_memcpy(tmp->bytes, params.data(), params.size());
+    return tmp->bytes;
   }
 };
 

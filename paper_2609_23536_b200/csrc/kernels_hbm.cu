@@ -125,9 +125,10 @@ __global__ void __launch_bounds__(kQuantThreads) quantize_kernel(const __grid_co
 }
 
 // Two to eight independent casts in one launch (the X of forward units and the dY of input-gradient units that go out
-// together): the blocks are dealt to the casts one cast after the other.  No commit tails.
+// together, the weights of a stage at the start of its step): the blocks are dealt to the casts one cast after the other.
 __global__ void __launch_bounds__(kQuantThreads) quantize_multi_kernel(const __grid_constant__ QuantMultiParams mp) {
   __shared__ uint32_t wmax[kQuantThreads / 32];
+  __shared__ uint32_t last_flag;
   grid_dep_wait();
   grid_dep_launch();
   uint32_t which = 0, base = 0;
@@ -136,6 +137,11 @@ __global__ void __launch_bounds__(kQuantThreads) quantize_multi_kernel(const __g
   const uint32_t b = blockIdx.x - base, bxn = p.cols / 64u;
   if (p.fmt == 0) quantize_block<0>(p, b % bxn, b / bxn, wmax);
   else quantize_block<1>(p, b % bxn, b / bxn, wmax);
+  if (p.commit.st) {  // the last block of this cast
+    auto sync = [] { __syncthreads(); };
+    if (last_block(&p.commit.st->ticket, mp.block_end[which] - base, threadIdx.x, &last_flag, sync))
+      commit_classes(p.commit, threadIdx.x, wmax, sync);
+  }
 }
 
 Launch make_quantize_multi(const QuantParams* casts, uint32_t n) {

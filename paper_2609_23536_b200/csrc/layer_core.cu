@@ -147,7 +147,8 @@ cudaError_t launch_pdl(const qe::Launch& l, cudaStream_t stream) {
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  void* args[1] = {const_cast<unsigned char*>(l.params.data())};
+  qe::Launch::Block tmp;
+  void* args[1] = {l.args_block(&tmp)};
   return cudaLaunchKernelExC(&cfg, l.func, args);
 }
 
@@ -232,7 +233,8 @@ int32_t replay_graph(qe_ctx* ctx, ActionGraph* g, const std::vector<qe::Launch>&
     if (same) continue;
     // caller-visible pointers (x, y, gradient destination) or the accumulate flag changed: patch the node in place
     cudaKernelNodeParams np{};
-    void* args[1] = {const_cast<unsigned char*>(now.params.data())};
+    qe::Launch::Block tmp;
+    void* args[1] = {now.args_block(&tmp)};
     np.func = const_cast<void*>(now.func);
     np.gridDim = now.grid;
     np.blockDim = now.block;
@@ -429,11 +431,11 @@ qe::Launch quant_launch(qe_layer* L, const void* x, uint8_t* q, uint8_t* qT, uin
 
 
 // ---- the launches of each action (shared by the per-action calls and the whole-step call)
-void add_refresh(qe_layer* L, std::vector<qe::Launch>& ls) {
-  // Invariant 3: first forward of the epoch re-quantises the weight; the kernel's last block commits its amax
-  ls.push_back(quant_launch(L, L->cfg.weight_dev, L->Wq, L->WqT, L->cfg.N, L->cfg.K, QE_CLASS_W, &L->st->cache_sinv_W,
-                            QE_E4M3, 1u << QE_CLASS_W));
+// Invariant 3: first forward of the epoch re-quantises the weight; the kernel's last block commits its amax
+qe::QuantParams refresh_params(qe_layer* L) {
+  return quant_params(L, L->cfg.weight_dev, L->Wq, L->WqT, L->cfg.N, L->cfg.K, QE_CLASS_W, &L->st->cache_sinv_W, QE_E4M3, 1u << QE_CLASS_W);
 }
+void add_refresh(qe_layer* L, std::vector<qe::Launch>& ls) { ls.push_back(qe::make_quantize(refresh_params(L))); }
 
 // FP8 hand-off between directly chained linears: the forward GEMM of `L` emits its output as the E4M3 input of
 // `next` (quantised with next's current X scale, straight into next's tape slot pn, with next's X amax and

@@ -131,6 +131,7 @@ qe::QuantParams quant_params(qe_layer* L, const void* x, uint8_t* q, uint8_t* qT
                              float* sinv_dst, int fmt, uint32_t commit_mask = 0);
 qe::Launch quant_launch(qe_layer* L, const void* x, uint8_t* q, uint8_t* qT, uint32_t rows, uint32_t cols, int cls,
                         float* sinv_dst, int fmt, uint32_t commit_mask = 0);
+qe::QuantParams refresh_params(qe_layer* L);
 void add_refresh(qe_layer* L, std::vector<qe::Launch>& ls);
 void add_forward(qe_layer* L, uint32_t p, const void* x, void* y, std::vector<qe::Launch>& ls, qe_layer* next = nullptr,
                  uint32_t pn = 0, qe::GemmDesc* gemm_out = nullptr, qe::QuantParams* cast_out = nullptr);
