@@ -281,7 +281,7 @@ int32_t qe_run_together_host(qe_ctx*, qe_action* actions, uint32_t n, float* gra
  * the same in the backward direction (tapes[] in layer order): dy_dev bf16 [T, N_{n-1}] in, dx_dev bf16 [T, K_0]
  * out, each input gradient handed to the layer before it as E5M2 with that layer's G scale.  Every layer's contract
  * check is made before anything runs; dW of each layer follows through qe_backward_dW / _multi as usual.
- * UNSUPPORTED when a receiving layer keeps transposed FP8 copies (T and N multiples of 256 are required). */
+ * UNSUPPORTED when a layer's N is not a multiple of 256. */
 #define QE_MAX_CHAIN 16
 int32_t qe_forward_chain(qe_layer* const* layers, uint32_t n, uint32_t mb, uint64_t gen, const void* x_dev,
                          void* y_dev, void* caller_stream, qe_tape* tapes_out);

@@ -87,9 +87,7 @@ int32_t qe_layer_create(qe_ctx* ctx, const qe_layer_config* cfg, void* ws, uint6
   uint8_t* base = (uint8_t*)ws;
   L->st = (qe::DevState*)base;
   L->hist = (float*)(base + k.hist);
-  const bool wT = !qe::gemm_uses_pair(cfg->T), xgT = !qe::gemm_uses_pair(cfg->N);
   L->Wq = base + k.Wq;
-  L->WqT = wT ? base + k.WqT : nullptr;
   if (cfg->host_io) {
     L->x_stage = base + k.stage_tk;
     L->dx_stage = L->x_stage + align_up(2ull * cfg->T * cfg->K, 1024);
@@ -101,22 +99,15 @@ int32_t qe_layer_create(qe_ctx* ctx, const qe_layer_config* cfg, void* ws, uint6
   for (uint32_t p = 0; p < cfg->slots; ++p) {
     uint8_t* s = base + k.slot0 + k.per_slot * p;
     L->Xq[p] = s + k.xq;
-    L->XqT[p] = xgT ? s + k.xqT : nullptr;
     L->Gq[p] = s + k.gq;
-    L->GqT[p] = xgT ? s + k.gqT : nullptr;
     if ((st = make_map(d, &L->tmXq_A[p], L->Xq[p], T, K, 128)) != QE_OK) break;   // F:  A = Xq  [T,K]
     if ((st = make_map(d, &L->tmGq_A[p], L->Gq[p], T, N, 128)) != QE_OK) break;   // dI: A = Gq  [T,N]
-    if (xgT) {
-      if ((st = make_map(d, &L->tmGqT_A[p], L->GqT[p], N, T, 128)) != QE_OK) break; // dW: A = Gq^T [N,T]
-      if ((st = make_b_maps(d, L->tmXqT_B[p], L->XqT[p], K, T, false)) != QE_OK) break; // dW: B = Xq^T [K,T]
-    } else {  // dW reads Gq [T,N] and Xq [T,K] as MN-major operands, over the row-major tensors
-      if ((st = make_map(d, &L->tmGqT_A[p], L->Gq[p], T, N, 128)) != QE_OK) break;
-      if ((st = make_b_maps(d, L->tmXqT_B[p], L->Xq[p], K, T, true)) != QE_OK) break;
-    }
+    // dW reads Gq [T,N] and Xq [T,K] as MN-major operands
+    if ((st = make_map(d, &L->tmGq_dW[p], L->Gq[p], T, N, 128)) != QE_OK) break;
+    if ((st = make_b_maps(d, L->tmXq_dW[p], L->Xq[p], K, T, true)) != QE_OK) break;
   }
-  if (st == QE_OK) st = make_b_maps(d, L->tmWq_B, L->Wq, N, K, false);    // F:  B = Wq   [N,K]
-  if (st == QE_OK)  // dI: B = Wq^T [K,N], or Wq [N,K] itself as an MN-major operand
-    st = wT ? make_b_maps(d, L->tmWq_dI, L->WqT, K, N, false) : make_b_maps(d, L->tmWq_dI, L->Wq, K, N, true);
+  if (st == QE_OK) st = make_b_maps(d, L->tmWq_B, L->Wq, N, K, false);   // F:  B = Wq [N,K]
+  if (st == QE_OK) st = make_b_maps(d, L->tmWq_dI, L->Wq, K, N, true);   // dI: B = Wq as an MN-major operand
   if (st != QE_OK) { qe_contract_destroy(L->contract); delete L; return st; }
   // state: histories 0, scales 1, everything else 0
   qe::DevState init{};
@@ -448,13 +439,23 @@ int32_t qe_read_fp8(qe_layer* L, uint32_t which, uint32_t slot, void* host_out, 
   if (!L || !host_out) return fail(QE_ERR_BAD_ARG, "null argument");
   const uint64_t tk = (uint64_t)L->cfg.T * L->cfg.K, tn = (uint64_t)L->cfg.T * L->cfg.N, nk = (uint64_t)L->cfg.N * L->cfg.K;
   if (which > 5 || (which < 4 && slot >= L->cfg.slots)) return fail(QE_ERR_BAD_ARG, "which %u slot %u", which, slot);
-  const uint8_t* src = which == 0 ? L->Xq[slot] : which == 1 ? L->XqT[slot] : which == 2 ? L->Gq[slot]
-                     : which == 3 ? L->GqT[slot] : which == 4 ? L->Wq : L->WqT;
-  if (!src) return fail(QE_ERR_UNSUPPORTED, "this layer keeps no transposed copy %u (its GEMM reads the row-major tensor directly)", which);
+  const bool transposed = which & 1u;  // 1, 3, 5: the transposes of 0, 2, 4
+  const uint8_t* src = which < 2 ? L->Xq[slot] : which < 4 ? L->Gq[slot] : L->Wq;
+  // (offered for the layers whose GEMMs have half-filled row tiles; made here, no kernel reads one)
+  if (transposed && qe::gemm_uses_pair(which == 5 ? L->cfg.T : L->cfg.N))
+    return fail(QE_ERR_UNSUPPORTED, "this layer keeps no transposed copy %u (its GEMM reads the row-major tensor directly)", which);
   const uint64_t need = which < 2 ? tk : which < 4 ? tn : nk;
   if (bytes != need) return fail(QE_ERR_BAD_ARG, "bytes %llu, tensor has %llu", (unsigned long long)bytes, (unsigned long long)need);
   QE_CUDA(cudaStreamSynchronize(L->ctx->exec_stream));
-  QE_CUDA(cudaMemcpy(host_out, src, need, cudaMemcpyDeviceToHost));
+  if (!transposed) {
+    QE_CUDA(cudaMemcpy(host_out, src, need, cudaMemcpyDeviceToHost));
+    return QE_OK;
+  }
+  const uint64_t rows = which == 5 ? L->cfg.N : L->cfg.T, cols = need / rows;
+  std::vector<uint8_t> m(need);
+  QE_CUDA(cudaMemcpy(m.data(), src, need, cudaMemcpyDeviceToHost));
+  for (uint64_t c = 0; c < cols; ++c)
+    for (uint64_t r = 0; r < rows; ++r) ((uint8_t*)host_out)[c * rows + r] = m[r * cols + c];
   return QE_OK;
 }
 

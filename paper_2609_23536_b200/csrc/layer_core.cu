@@ -360,19 +360,13 @@ Carve carve(const qe_layer_config& c) {
   k.hist = o;
   o = align_up(o + 4ull * c.history_len * sizeof(float), 1024);
   const uint64_t nk = (uint64_t)c.N * c.K, tk = (uint64_t)c.T * c.K, tn = (uint64_t)c.T * c.N;
-  // Transposed FP8 copies exist only where a GEMM cannot take the row-major tensor as an MN-major operand: the dI
-  // GEMM (M = T) needs Wq^T, the dW GEMM (M = N) needs Xq^T and Gq^T, when that M is not a multiple of 256.
-  const bool wT = !qe::gemm_uses_pair(c.T), xgT = !qe::gemm_uses_pair(c.N);
+  // One FP8 copy of every tensor, row-major: the GEMMs read it contraction-major or MN-major, as each of them needs.
   k.Wq = o;
   o += align_up(nk, 1024);
-  k.WqT = o;
-  if (wT) o += align_up(nk, 1024);
   k.slot0 = o;
   k.xq = 0;
-  k.xqT = align_up(tk, 1024);
-  k.gq = k.xqT + (xgT ? align_up(tk, 1024) : 0);
-  k.gqT = k.gq + align_up(tn, 1024);
-  k.per_slot = k.gqT + (xgT ? align_up(tn, 1024) : 0);
+  k.gq = align_up(tk, 1024);
+  k.per_slot = k.gq + align_up(tn, 1024);
   o += k.per_slot * c.slots;
   if (c.host_io) {  // x / dx [T,K] and y / dy [T,N] bf16 staging for the host-buffer entry points
     k.stage_tk = o;
@@ -408,12 +402,11 @@ qe::CommitParams commit_params(qe_layer* L, uint32_t mask, uint32_t bump, const 
 }
 
 // commit_mask != 0: the kernel's last block also commits those classes (used for the weight refresh)
-qe::QuantParams quant_params(qe_layer* L, const void* x, uint8_t* q, uint8_t* qT, uint32_t rows, uint32_t cols, int cls,
+qe::QuantParams quant_params(qe_layer* L, const void* x, uint8_t* q, uint32_t rows, uint32_t cols, int cls,
                              float* sinv_dst, int fmt, uint32_t commit_mask) {
   qe::QuantParams qp{};
   qp.x = (const uint16_t*)x;
   qp.q = q;
-  qp.qT = qT;
   qp.rows = rows;
   qp.cols = cols;
   qp.scale = &L->st->scale[cls];
@@ -424,16 +417,16 @@ qe::QuantParams quant_params(qe_layer* L, const void* x, uint8_t* q, uint8_t* qT
   if (commit_mask) qp.commit = commit_params(L, commit_mask, 0, nullptr);
   return qp;
 }
-qe::Launch quant_launch(qe_layer* L, const void* x, uint8_t* q, uint8_t* qT, uint32_t rows, uint32_t cols, int cls,
+qe::Launch quant_launch(qe_layer* L, const void* x, uint8_t* q, uint32_t rows, uint32_t cols, int cls,
                         float* sinv_dst, int fmt, uint32_t commit_mask) {
-  return qe::make_quantize(quant_params(L, x, q, qT, rows, cols, cls, sinv_dst, fmt, commit_mask));
+  return qe::make_quantize(quant_params(L, x, q, rows, cols, cls, sinv_dst, fmt, commit_mask));
 }
 
 
 // ---- the launches of each action (shared by the per-action calls and the whole-step call)
 // Invariant 3: first forward of the epoch re-quantises the weight; the kernel's last block commits its amax
 qe::QuantParams refresh_params(qe_layer* L) {
-  return quant_params(L, L->cfg.weight_dev, L->Wq, L->WqT, L->cfg.N, L->cfg.K, QE_CLASS_W, &L->st->cache_sinv_W, QE_E4M3, 1u << QE_CLASS_W);
+  return quant_params(L, L->cfg.weight_dev, L->Wq, L->cfg.N, L->cfg.K, QE_CLASS_W, &L->st->cache_sinv_W, QE_E4M3, 1u << QE_CLASS_W);
 }
 void add_refresh(qe_layer* L, std::vector<qe::Launch>& ls) { ls.push_back(qe::make_quantize(refresh_params(L))); }
 
@@ -444,8 +437,8 @@ void add_refresh(qe_layer* L, std::vector<qe::Launch>& ls) { ls.push_back(qe::ma
 void add_forward(qe_layer* L, uint32_t p, const void* x, void* y, std::vector<qe::Launch>& ls, qe_layer* next,
                  uint32_t pn, qe::GemmDesc* gemm_out, qe::QuantParams* cast_out) {
   const uint32_t T = L->cfg.T, K = L->cfg.K, N = L->cfg.N;
-  if (x && cast_out) *cast_out = quant_params(L, x, L->Xq[p], L->XqT[p], T, K, QE_CLASS_X, &L->st->slot_sinv_X[p], QE_E4M3);
-  else if (x) ls.push_back(quant_launch(L, x, L->Xq[p], L->XqT[p], T, K, QE_CLASS_X, &L->st->slot_sinv_X[p], QE_E4M3));
+  if (x && cast_out) *cast_out = quant_params(L, x, L->Xq[p], T, K, QE_CLASS_X, &L->st->slot_sinv_X[p], QE_E4M3);
+  else if (x) ls.push_back(quant_launch(L, x, L->Xq[p], T, K, QE_CLASS_X, &L->st->slot_sinv_X[p], QE_E4M3));
   qe::GemmDesc gp;
   gp.ops[0] = {&L->tmXq_A[p], L->tmWq_B, &L->st->slot_sinv_X[p], &L->st->cache_sinv_W};
   gp.M = T;
@@ -480,17 +473,16 @@ void add_forward(qe_layer* L, uint32_t p, const void* x, void* y, std::vector<qe
 void add_dI(qe_layer* L, uint32_t p, const void* dy, void* dx, std::vector<qe::Launch>& ls, qe_layer* prev,
             uint32_t pp, qe::GemmDesc* gemm_out, qe::QuantParams* cast_out) {
   const uint32_t T = L->cfg.T, K = L->cfg.K, N = L->cfg.N;
-  if (dy && cast_out) *cast_out = quant_params(L, dy, L->Gq[p], L->GqT[p], T, N, QE_CLASS_G, &L->st->slot_sinv_G[p], QE_E5M2);
-  else if (dy) ls.push_back(quant_launch(L, dy, L->Gq[p], L->GqT[p], T, N, QE_CLASS_G, &L->st->slot_sinv_G[p], QE_E5M2));
+  if (dy && cast_out) *cast_out = quant_params(L, dy, L->Gq[p], T, N, QE_CLASS_G, &L->st->slot_sinv_G[p], QE_E5M2);
+  else if (dy) ls.push_back(quant_launch(L, dy, L->Gq[p], T, N, QE_CLASS_G, &L->st->slot_sinv_G[p], QE_E5M2));
   qe::GemmDesc gp;
-  const bool b_mn = L->WqT == nullptr;  // no transposed weight copy: Wq [N,K] is B in MN-major form
   gp.ops[0] = {&L->tmGq_A[p], L->tmWq_dI, &L->st->slot_sinv_G[p], &L->st->cache_sinv_W};
   gp.M = T;
   gp.N = K;
   gp.Kc = N;
   gp.a_fmt = QE_E5M2;
   gp.b_fmt = QE_E4M3;
-  gp.b_mn = b_mn;
+  gp.b_mn = 1;  // Wq [N,K] itself: B in MN-major form
   gp.ldo = K;
   if (prev) {
     gp.out = prev->Gq[pp];
@@ -519,15 +511,14 @@ void add_dI(qe_layer* L, uint32_t p, const void* dy, void* dx, std::vector<qe::L
 qe::GemmDesc dW_gemm(qe_layer* L, uint32_t p, float* dst, int32_t accumulate, float* temp) {
   const uint32_t T = L->cfg.T, K = L->cfg.K, N = L->cfg.N;
   qe::GemmDesc gp;
-  const bool mn = L->GqT[p] == nullptr;  // Gq [T,N] and Xq [T,K] themselves, read as MN-major operands
   // (scales: the snapshots taken when dY_m and X_m were quantised, never the current state)
-  gp.ops[0] = {&L->tmGqT_A[p], L->tmXqT_B[p], &L->st->slot_sinv_G[p], &L->st->slot_sinv_X[p]};
+  gp.ops[0] = {&L->tmGq_dW[p], L->tmXq_dW[p], &L->st->slot_sinv_G[p], &L->st->slot_sinv_X[p]};
   gp.M = N;
   gp.N = K;
   gp.Kc = T;
   gp.a_fmt = QE_E5M2;
   gp.b_fmt = QE_E4M3;
-  gp.a_mn = gp.b_mn = mn;
+  gp.a_mn = gp.b_mn = 1;  // Gq [T,N] and Xq [T,K] themselves, read as MN-major operands
   gp.ldo = K;
   gp.amax_bits = nullptr;
   gp.status = &L->st->status;

@@ -81,10 +81,9 @@ static int32_t check_chain(qe_layer* const* layers, uint32_t n) {
       return fail(QE_ERR_SHAPE, "layer %u does not take layer %u's output ([%u, %u] after [%u, %u])", i, i - 1, layers[i]->cfg.T,
                   layers[i]->cfg.K, layers[i - 1]->cfg.T, layers[i - 1]->cfg.N);
   }
-  // a deposited FP8 tensor is the row-major one only: every layer that receives one must run without transposed copies
-  for (uint32_t i = 0; i < n; ++i)
-    if ((i > 0 && layers[i]->XqT[0]) || (i + 1 < n && layers[i]->GqT[0]))
-      return fail(QE_ERR_UNSUPPORTED, "layer %u keeps transposed FP8 copies (T and N must be multiples of 256 for the hand-off)", i);
+  // (whole 256-row tiles only, as for the shared launches)
+  for (uint32_t i = 0; n > 1 && i < n; ++i)
+    if (!qe::gemm_uses_pair(layers[i]->cfg.N)) return fail(QE_ERR_UNSUPPORTED, "layer %u: N must be a multiple of 256 for the hand-off", i);
   return QE_OK;
 }
 

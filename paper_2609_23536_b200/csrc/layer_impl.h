@@ -89,12 +89,12 @@ struct qe_layer {
   uint64_t ws_bytes = 0;
   qe::DevState* st = nullptr;
   float* hist = nullptr;
-  uint8_t *Wq = nullptr, *WqT = nullptr;
+  uint8_t* Wq = nullptr;
   uint8_t *x_stage = nullptr, *dx_stage = nullptr, *y_stage = nullptr, *dy_stage = nullptr;  // host_io only
-  uint8_t *Xq[QE_MAX_SLOTS], *XqT[QE_MAX_SLOTS], *Gq[QE_MAX_SLOTS], *GqT[QE_MAX_SLOTS];
+  uint8_t *Xq[QE_MAX_SLOTS], *Gq[QE_MAX_SLOTS];
   // tensor maps: one per tensor in the A role, one per tile width in the B role
-  CUtensorMap tmXq_A[QE_MAX_SLOTS], tmGq_A[QE_MAX_SLOTS], tmGqT_A[QE_MAX_SLOTS], tmXqT_B[QE_MAX_SLOTS][qe::kNumTileWidths];
-  CUtensorMap tmWq_B[qe::kNumTileWidths], tmWq_dI[qe::kNumTileWidths];  // B of the forward; B of dI (Wq^T, or Wq MN-major)
+  CUtensorMap tmXq_A[QE_MAX_SLOTS], tmGq_A[QE_MAX_SLOTS], tmGq_dW[QE_MAX_SLOTS], tmXq_dW[QE_MAX_SLOTS][qe::kNumTileWidths];
+  CUtensorMap tmWq_B[qe::kNumTileWidths], tmWq_dI[qe::kNumTileWidths];  // B of the forward; B of dI (MN-major)
   ActionGraph gF[QE_MAX_SLOTS], gDI[QE_MAX_SLOTS], gDW[QE_MAX_SLOTS], gDWs[QE_MAX_SLOTS], gRefresh, gCommit;
   // QE_CTX_OVERLAP_DW: per slot, "dI of the tape in this slot has been enqueued" / "the dW that released it has"
   cudaEvent_t ev_di[QE_MAX_SLOTS] = {}, ev_dw[QE_MAX_SLOTS] = {};
@@ -122,14 +122,14 @@ int32_t run_keyed(qe_ctx* ctx, uint64_t key, const std::vector<qe::Launch>& ls);
 
 // ---- workspace and launch builders
 struct Carve {
-  uint64_t hist, Wq, WqT, slot0, per_slot, xq, xqT, gq, gqT, total, stage_tk = 0, stage_tn = 0;
+  uint64_t hist, Wq, slot0, per_slot, xq, gq, total, stage_tk = 0, stage_tn = 0;
 };
 Carve carve(const qe_layer_config& c);
 int32_t check_config(const qe_layer_config* c);
 qe::CommitParams commit_params(qe_layer* L, uint32_t mask, uint32_t bump, const float* override_amax);
-qe::QuantParams quant_params(qe_layer* L, const void* x, uint8_t* q, uint8_t* qT, uint32_t rows, uint32_t cols, int cls,
+qe::QuantParams quant_params(qe_layer* L, const void* x, uint8_t* q, uint32_t rows, uint32_t cols, int cls,
                              float* sinv_dst, int fmt, uint32_t commit_mask = 0);
-qe::Launch quant_launch(qe_layer* L, const void* x, uint8_t* q, uint8_t* qT, uint32_t rows, uint32_t cols, int cls,
+qe::Launch quant_launch(qe_layer* L, const void* x, uint8_t* q, uint32_t rows, uint32_t cols, int cls,
                         float* sinv_dst, int fmt, uint32_t commit_mask = 0);
 qe::QuantParams refresh_params(qe_layer* L);
 void add_refresh(qe_layer* L, std::vector<qe::Launch>& ls);
@@ -142,7 +142,7 @@ qe::GemmDesc dW_gemm_view(qe_layer* L, uint32_t p, void* view);
 void add_dW(qe_layer* L, uint32_t p, float* dst, int32_t accumulate, float* temp, std::vector<qe::Launch>& ls);
 
 // Weight-gradient GEMMs of different layers that follow one another share one launch where the kernel allows it
-// (all on the paired variant): the persistent CTAs pack their tiles into common waves and the launch is paid once.
+// (all of whole 256-row tiles): the persistent CTAs pack their tiles into common waves and the launch is paid once.
 // The layers' gradient slices are disjoint (destination registry), so the GEMMs are independent.
 struct DWBatch {
   qe::GemmDesc gp[4];
