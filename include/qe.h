@@ -234,7 +234,7 @@ int32_t qe_backward_dW_staged(qe_layer*, const qe_tape*, float* grad_buf_dev, ui
  * holds a forward unit and an input-gradient unit at once; their chains through the layers are independent).  The
  * same checks, results (bit for bit) and state transitions as qe_forward(layer_f, mb, gen, x_dev, y_dev, stream,
  * tape_out) followed by qe_backward_dI(layer_b, tape_b, dy_dev, dx_dev, stream), with the two GEMMs in one kernel
- * launch where both can run on the paired-CTA variant (T a multiple of 256).  layer_f != layer_b, one context.  Both
+ * launch where both have whole 256-row tiles (T a multiple of 256).  layer_f != layer_b, one context.  Both
  * checks are made before anything runs: on a contract error nothing ran and neither layer's state changed. */
 int32_t qe_forward_dI_pair(qe_layer* layer_f, uint32_t mb, uint64_t gen, const void* x_dev, void* y_dev,
                            qe_tape* tape_out, qe_layer* layer_b, const qe_tape* tape_b, const void* dy_dev,
@@ -243,7 +243,7 @@ int32_t qe_forward_dI_pair(qe_layer* layer_f, uint32_t mb, uint64_t gen, const v
  * the steady state of a split-backward schedule a stage holds a forward unit, an input-gradient unit and a deferred
  * weight-gradient unit at once (Sec. 4.2), none of which depends on another.  The result -- outputs, gradient
  * buffer, scale state, tapes -- is bit for bit that of issuing the actions one after the other in the order given;
- * all GEMMs that can run on the paired-CTA variant share one kernel launch (forward and input-gradient tiles
+ * all GEMMs of whole 256-row tiles share one kernel launch (forward and input-gradient tiles
  * first, weight-gradient tiles after them).  1 <= n <= QE_MAX_TOGETHER; at most one
  * action of a kind per layer; a dW action's tape must already have had its dI (ORDER otherwise, also when that dI
  * is part of the same call).  Every check is made before anything runs, against the state before the call: on a
@@ -306,9 +306,9 @@ int32_t qe_arena_finalize(qe_layer*, const void* arena_dev, uint64_t arena_elems
 int32_t qe_arena_reduce(const void* views_dev, uint64_t view_elems, uint32_t M, float* dst_dev, void* stream);
 /* The W action of Sec. 4.2 for several layers of the stage at once (typically one microbatch's deferred weight
  * gradients): the same checks, results (bit for bit) and state transitions as qe_backward_dW(layers[i], &tapes[i],
- * grad_buf_dev, grad_buf_elems, offsets[i], stream) for i = 0..n-1, but the GEMMs of up to four layers at a time share one
- * kernel launch where each of them can run on the paired-CTA variant (N_i a multiple of 256); the others are
- * launched one by one inside the same call.  layers[] (host array) distinct and of one context, 1 <= n <=
+ * grad_buf_dev, grad_buf_elems, offsets[i], stream) for i = 0..n-1, but the GEMMs of up to four layers at a time (of up to
+ * sixteen in calls of more than eight) share one kernel launch where each has whole 256-row tiles (N_i a multiple of
+ * 256); the others are launched one by one inside the same call.  layers[] (host array) distinct and of one context, 1 <= n <=
  * QE_MAX_MULTI_DW; tapes[] and offsets[] host arrays of n entries.  All n checks are made before anything runs: on
  * a contract error nothing ran and no layer's state changed.  A bounded wait that expires inside a shared launch
  * is recorded in the status word of every layer that has a GEMM in that launch. */
@@ -443,8 +443,8 @@ uint32_t qe_amax_partials(void);
 int32_t qe_accumulate(float* dst_dev, const float* src_dev, uint64_t n, int32_t accumulate, void* stream);
 /* One FP8 GEMM on the tensor cores: D[m,n] = (sum_k A[m,k] B[n,k]) * *alpha_a_dev * *alpha_b_dev with A [M,Kc] and
  * B [Nn,Kc] both contraction-major bytes.  out_kind 0: bf16 D (amax_dev optional, as in qe_quantize); 1: FP32
- * D overwrite; 2: FP32 D accumulate.  M, Kc multiples of 128 (>= 128), Nn a multiple of 128 (>= 256).  A 256-row paired-CTA variant runs when
- * M is a multiple of 256, a single-CTA 128-row variant otherwise.  status_dev: one uint32 the kernel ORs error
+ * D overwrite; 2: FP32 D accumulate.  M, Kc multiples of 128 (>= 128), Nn a multiple of 128 (>= 256).  Tiles
+ * have 256 rows; a last one that M fills by half is computed with zero rows that are not stored.  status_dev: one uint32 the kernel ORs error
  * bits into (caller zeroes it). */
 int32_t qe_gemm_fp8(const void* a_dev, uint32_t a_format, const void* b_dev, uint32_t b_format, uint32_t M,
                     uint32_t Nn, uint32_t Kc, const float* alpha_a_dev, const float* alpha_b_dev, void* d_dev,

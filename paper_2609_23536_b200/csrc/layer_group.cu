@@ -35,7 +35,7 @@ int32_t qe_backward_dW_multi(qe_layer* const* layers, const qe_tape* tapes, uint
     return st;
   }
   std::vector<qe::Launch> ls;
-  DWBatch dwb;
+  DWBatch dwb(n);
   Fnv h;
   h.mix("dWmulti", 8);
   for (uint32_t i = 0; i < n; ++i) {
@@ -558,10 +558,10 @@ int32_t qe_step_run(qe_ctx* ctx, qe_layer* const* layers, uint32_t n_layers, con
   if (!rounds.empty()) k = st == QE_OK ? n_actions : k;
 
   // ---- host pass: check -> collect launches -> commit, action by action (Algorithm 1)
-  DWBatch dwb;
+  DWBatch dwb(n_layers);
   for (; rounds.empty() && k < n_actions && st == QE_OK; ++k) {
     const qe_step_action& a = actions[k];
-    if (a.kind != QE_ACT_DW && dwb.n) dwb.flush(ctx, ls);
+    if (a.kind != QE_ACT_DW) dwb.flush(ctx, ls);
     if (a.layer >= n_layers || a.mb >= M || a.kind > QE_ACT_DW) {
       st = fail(QE_ERR_BAD_ARG, "action %u: kind %u layer %u mb %u", k, a.kind, a.layer, a.mb);
       break;
@@ -598,7 +598,7 @@ int32_t qe_step_run(qe_ctx* ctx, qe_layer* const* layers, uint32_t n_layers, con
       st = qe_contract_dW_commit(L->contract, &tapes[u], (uint64_t)(uintptr_t)grad, offsets[a.layer], slice);
     }
   }
-  if (dwb.n) dwb.flush(ctx, ls);
+  dwb.flush(ctx, ls);
   const int32_t check_status = st;
   char saved_msg[512];
   std::snprintf(saved_msg, sizeof(saved_msg), "%s", qe_last_error());

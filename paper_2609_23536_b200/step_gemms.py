@@ -40,7 +40,7 @@ def build(cfg, device, max_group=8):
                 ps.append((Gq[m][i], 1, 1, Xq[m][i], 0, 1, one, one, grad[i], 2, None))
                 nbytes += T * N + T * K + 8 * N * K
         pairable = [q for q in ps if q[8].shape[0] % 256 == 0]
-        launches += [[q] for q in ps if q[8].shape[0] % 256]  # single-CTA variant: a launch of its own, as in the layer
+        launches += [[q] for q in ps if q[8].shape[0] % 256]  # half-filled last row tile: a launch of its own, as in the layer
         if len(pairable) >= 2:
             launches.append(pairable)
         else:
