@@ -471,7 +471,12 @@ int32_t qe_step_run(qe_ctx* ctx, qe_layer* const* layers, uint32_t n_layers, con
   // end of a launch (a 4096 / 14336 block: 20.5 ms one by one, 21.2 ms in sums), so there they go out one by one.
   uint32_t T_max = 0;
   for (uint32_t l = 0; l < n_layers; ++l) T_max = std::max(T_max, layers[l]->cfg.T);
-  const uint32_t max_sum = T_max >= 4096 ? 1u : std::min(qe::kMaxSegments, 8192u / T_max);
+  // A layer that the list names by more than one index is planned without sums (a sum belongs to one index), and two of its
+  // actions of a kind may not meet in a round: the round's launch would commit the layer's scales twice.
+  std::vector<qe_layer*> by_address(layers, layers + n_layers);
+  std::sort(by_address.begin(), by_address.end());
+  const bool repeated = std::adjacent_find(by_address.begin(), by_address.end()) != by_address.end();
+  const uint32_t max_sum = repeated || T_max >= 4096 ? 1u : std::min(qe::kMaxSegments, 8192u / T_max);
   std::vector<std::vector<uint32_t>> rounds;  // indices into actions[]
   if (!temp && ctx->step_window > 1) {
     std::vector<uint32_t> slots(n_layers), live(n_layers), round_of(n_actions);
@@ -506,6 +511,13 @@ int32_t qe_step_run(qe_ctx* ctx, qe_layer* const* layers, uint32_t n_layers, con
     qe_action acts[kMaxRound];
     TogetherPrep pr;
     uint32_t na = 0;
+    for (size_t i = 0; repeated && i < rounds[r].size(); ++i)
+      for (size_t j = 0; j < i; ++j) {
+        const qe_step_action &a = actions[rounds[r][j]], &b = actions[rounds[r][i]];
+        if (a.kind == b.kind && layers[a.layer] == layers[b.layer])
+          st = fail(QE_ERR_BAD_ARG, "actions %u and %u: same kind on the same layer", rounds[r][j], rounds[r][i]);
+      }
+    if (st != QE_OK) k = rounds[r][0];
     for (uint32_t kind = QE_ACT_F; kind <= QE_ACT_DW && st == QE_OK; ++kind) {
       for (uint32_t gi : rounds[r]) {
         const qe_step_action& a = actions[gi];
