@@ -163,8 +163,9 @@ static int32_t forward_impl(qe_layer* L, uint32_t mb, uint64_t gen, const void* 
   if (st != QE_OK) return st;
   qe_ctx* ctx = L->ctx;
   cudaStream_t caller = (cudaStream_t)caller_stream;
+  Handshake handshake(ctx, caller);
   const uint32_t T = L->cfg.T, K = L->cfg.K, N = L->cfg.N;
-  if ((st = handoff_in(ctx, caller)) != QE_OK) return st;
+  if ((st = handshake.in()) != QE_OK) return st;
   if (x_host && (st = host_upload(ctx, const_cast<void*>(x), x_host, 2ull * T * K, caller)) != QE_OK) return st;
   if (L->dw_pending[p]) {  // the slot's buffers are still being read by the dW that released it (other stream)
     QE_CUDA(cudaStreamWaitEvent(ctx->exec_stream, L->ev_dw[p], 0));
@@ -179,7 +180,7 @@ static int32_t forward_impl(qe_layer* L, uint32_t mb, uint64_t gen, const void* 
   add_forward(L, p, x, y, ls);
   if ((st = run_action(ctx, &L->gF[p], ls)) != QE_OK) return st;  // ... run ...
   if (x_host && (st = host_download(ctx, y_host, y, 2ull * T * N)) != QE_OK) return st;
-  if ((st = handoff_out(ctx, caller)) != QE_OK) return st;
+  if ((st = handshake.out()) != QE_OK) return st;
   return qe_contract_forward_commit(L->contract, mb, tape_out);  // ... commit
 }
 
@@ -203,15 +204,16 @@ static int32_t backward_dI_impl(qe_layer* L, const qe_tape* tape, const void* dy
   if (st != QE_OK) return st;
   qe_ctx* ctx = L->ctx;
   cudaStream_t caller = (cudaStream_t)caller_stream;
+  Handshake handshake(ctx, caller);
   const uint32_t p = tape->ref.slot, T = L->cfg.T, K = L->cfg.K, N = L->cfg.N;
-  if ((st = handoff_in(ctx, caller)) != QE_OK) return st;
+  if ((st = handshake.in()) != QE_OK) return st;
   if (dy_host && (st = host_upload(ctx, const_cast<void*>(dy), dy_host, 2ull * T * N, caller)) != QE_OK) return st;
   std::vector<qe::Launch> ls;
   add_dI(L, p, dy, dx, ls);
   if ((st = run_action(ctx, &L->gDI[p], ls)) != QE_OK) return st;
   if (ctx->dw_stream) QE_CUDA(cudaEventRecord(L->ev_di[p], ctx->exec_stream));
   if (dy_host && (st = host_download(ctx, dx_host, dx, 2ull * T * K)) != QE_OK) return st;
-  if ((st = handoff_out(ctx, caller)) != QE_OK) return st;
+  if ((st = handshake.out()) != QE_OK) return st;
   return qe_contract_dI_commit(L->contract, tape);
 }
 
@@ -239,6 +241,7 @@ static int32_t backward_dW_impl(qe_layer* L, const qe_tape* tape, float* grad, u
   if (st != QE_OK) return st;
   qe_ctx* ctx = L->ctx;
   cudaStream_t caller = (cudaStream_t)caller_stream;
+  Handshake handshake(ctx, caller);
   const uint32_t p = tape->ref.slot;
   cudaStream_t run_on = ctx->exec_stream;
   if (ctx->dw_stream) {
@@ -248,7 +251,7 @@ static int32_t backward_dW_impl(qe_layer* L, const qe_tape* tape, float* grad, u
     QE_CUDA(cudaStreamWaitEvent(run_on, ctx->ev_dw_in, 0));
     QE_CUDA(cudaStreamWaitEvent(run_on, L->ev_di[p], 0));
     ctx->stats.handoffs += 1;
-  } else if ((st = handoff_in(ctx, caller)) != QE_OK) {
+  } else if ((st = handshake.in()) != QE_OK) {
     return st;
   }
   std::vector<qe::Launch> ls;
@@ -259,7 +262,7 @@ static int32_t backward_dW_impl(qe_layer* L, const qe_tape* tape, float* grad, u
   if (ctx->dw_stream) {  // joined at the optimizer boundary and before the slot's next forward
     QE_CUDA(cudaEventRecord(L->ev_dw[p], run_on));
     L->dw_pending[p] = true;
-  } else if ((st = handoff_out(ctx, caller)) != QE_OK) {
+  } else if ((st = handshake.out()) != QE_OK) {
     return st;
   }
   return qe_contract_dW_commit(L->contract, tape, (uint64_t)(uintptr_t)grad, off, slice);
@@ -303,7 +306,8 @@ int32_t qe_arena_finalize(qe_layer* L, const void* arena, uint64_t arena_elems, 
   if (off > grad_elems || n > grad_elems - off || ((uintptr_t)(grad + off) & 15u)) return fail(QE_ERR_DEST, "gradient slice out of range or misaligned");
   qe_ctx* ctx = L->ctx;
   cudaStream_t caller = (cudaStream_t)caller_stream;
-  int32_t st = handoff_in(ctx, caller);
+  Handshake handshake(ctx, caller);
+  int32_t st = handshake.in();
   if (st != QE_OK) return st;
   if (ctx->dw_stream) {  // the views were written on the second stream
     QE_CUDA(cudaEventRecord(ctx->ev_dw_in, ctx->dw_stream));
@@ -315,7 +319,7 @@ int32_t qe_arena_finalize(qe_layer* L, const void* arena, uint64_t arena_elems, 
   ap.view_vec = n / 8;
   ap.M = microbatches;
   if ((st = launch_eager(ctx, qe::make_arena_reduce(ap), ctx->exec_stream)) != QE_OK) return st;
-  return handoff_out(ctx, caller);
+  return handshake.out();
 }
 
 static int32_t read_status(qe_layer* L, uint32_t* status) {
@@ -372,12 +376,13 @@ int32_t qe_scale_commit(qe_layer* L, uint32_t cls, const float* amax_dev, void* 
   if (cls > QE_CLASS_Y) return fail(QE_ERR_BAD_ARG, "tensor_class %u", cls);
   qe_ctx* ctx = L->ctx;
   cudaStream_t caller = (cudaStream_t)caller_stream;
+  Handshake handshake(ctx, caller);
   int32_t st;
-  if ((st = handoff_in(ctx, caller)) != QE_OK) return st;
+  if ((st = handshake.in()) != QE_OK) return st;
   std::vector<qe::Launch> ls;
   ls.push_back(qe::make_commit(commit_params(L, 1u << cls, 0, amax_dev)));
   if ((st = run_action(ctx, &L->gCommit, ls)) != QE_OK) return st;
-  return handoff_out(ctx, caller);
+  return handshake.out();
 }
 
 int32_t qe_abort_step(qe_layer* L) {

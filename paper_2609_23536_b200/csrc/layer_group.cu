@@ -24,6 +24,7 @@ int32_t qe_backward_dW_multi(qe_layer* const* layers, const qe_tape* tapes, uint
       return st;
   }
   cudaStream_t caller = (cudaStream_t)caller_stream;
+  Handshake handshake(ctx, caller);
   cudaStream_t run_on = ctx->exec_stream;
   if (ctx->dw_stream) {
     run_on = ctx->dw_stream;
@@ -31,7 +32,7 @@ int32_t qe_backward_dW_multi(qe_layer* const* layers, const qe_tape* tapes, uint
     QE_CUDA(cudaStreamWaitEvent(run_on, ctx->ev_dw_in, 0));
     for (uint32_t i = 0; i < n; ++i) QE_CUDA(cudaStreamWaitEvent(run_on, layers[i]->ev_di[tapes[i].ref.slot], 0));
     ctx->stats.handoffs += 1;
-  } else if ((st = handoff_in(ctx, caller)) != QE_OK) {
+  } else if ((st = handshake.in()) != QE_OK) {
     return st;
   }
   std::vector<qe::Launch> ls;
@@ -60,7 +61,7 @@ int32_t qe_backward_dW_multi(qe_layer* const* layers, const qe_tape* tapes, uint
       QE_CUDA(cudaEventRecord(layers[i]->ev_dw[p], run_on));
       layers[i]->dw_pending[p] = true;
     }
-  } else if ((st = handoff_out(ctx, caller)) != QE_OK) {
+  } else if ((st = handshake.out()) != QE_OK) {
     return st;
   }
   for (uint32_t i = 0; i < n; ++i) {
@@ -99,7 +100,8 @@ int32_t qe_forward_chain(qe_layer* const* layers, uint32_t n, uint32_t mb, uint6
     if ((st = qe_contract_forward_check(layers[i]->contract, mb, gen, &refresh[i], &p[i])) != QE_OK) return st;
   qe_ctx* ctx = layers[0]->ctx;
   cudaStream_t caller = (cudaStream_t)caller_stream;
-  if ((st = handoff_in(ctx, caller)) != QE_OK) return st;
+  Handshake handshake(ctx, caller);
+  if ((st = handshake.in()) != QE_OK) return st;
   std::vector<qe::Launch> ls;
   Fnv h;
   h.mix("Fchain", 7);
@@ -119,7 +121,7 @@ int32_t qe_forward_chain(qe_layer* const* layers, uint32_t n, uint32_t mb, uint6
     add_forward(layers[i], p[i], i == 0 ? x : nullptr, last ? y : nullptr, ls, last ? nullptr : layers[i + 1], last ? 0 : p[i + 1]);
   }
   if ((st = run_keyed(ctx, h.key, ls)) != QE_OK) return st;
-  if ((st = handoff_out(ctx, caller)) != QE_OK) return st;
+  if ((st = handshake.out()) != QE_OK) return st;
   for (uint32_t i = 0; i < n; ++i)
     if ((st = qe_contract_forward_commit(layers[i]->contract, mb, &tapes_out[i])) != QE_OK) return st;
   return QE_OK;
@@ -135,7 +137,8 @@ int32_t qe_backward_dI_chain(qe_layer* const* layers, const qe_tape* tapes, uint
     if ((st = qe_contract_dI_check(layers[i]->contract, &tapes[i])) != QE_OK) return st;
   qe_ctx* ctx = layers[0]->ctx;
   cudaStream_t caller = (cudaStream_t)caller_stream;
-  if ((st = handoff_in(ctx, caller)) != QE_OK) return st;
+  Handshake handshake(ctx, caller);
+  if ((st = handshake.in()) != QE_OK) return st;
   std::vector<qe::Launch> ls;
   Fnv h;
   h.mix("Bchain", 7);
@@ -149,7 +152,7 @@ int32_t qe_backward_dI_chain(qe_layer* const* layers, const qe_tape* tapes, uint
   if ((st = run_keyed(ctx, h.key, ls)) != QE_OK) return st;
   if (ctx->dw_stream)
     for (uint32_t i = 0; i < n; ++i) QE_CUDA(cudaEventRecord(layers[i]->ev_di[tapes[i].ref.slot], ctx->exec_stream));
-  if ((st = handoff_out(ctx, caller)) != QE_OK) return st;
+  if ((st = handshake.out()) != QE_OK) return st;
   for (uint32_t i = 0; i < n; ++i)
     if ((st = qe_contract_dI_commit(layers[i]->contract, &tapes[i])) != QE_OK) return st;
   return QE_OK;
@@ -171,8 +174,9 @@ int32_t qe_forward_dI_pair(qe_layer* Lf, uint32_t mb, uint64_t gen, const void* 
   if ((st = qe_contract_dI_check(Lb->contract, tape_b)) != QE_OK) return st;
   qe_ctx* ctx = Lf->ctx;
   cudaStream_t caller = (cudaStream_t)caller_stream;
+  Handshake handshake(ctx, caller);
   const uint32_t pb = tape_b->ref.slot;
-  if ((st = handoff_in(ctx, caller)) != QE_OK) return st;
+  if ((st = handshake.in()) != QE_OK) return st;
   if (Lf->dw_pending[p]) {
     QE_CUDA(cudaStreamWaitEvent(ctx->exec_stream, Lf->ev_dw[p], 0));
     Lf->dw_pending[p] = false;
@@ -201,7 +205,7 @@ int32_t qe_forward_dI_pair(qe_layer* Lf, uint32_t mb, uint64_t gen, const void* 
   h.mix(&refresh, sizeof(refresh));
   if ((st = run_keyed(ctx, h.key, ls)) != QE_OK) return st;
   if (ctx->dw_stream) QE_CUDA(cudaEventRecord(Lb->ev_di[pb], ctx->exec_stream));
-  if ((st = handoff_out(ctx, caller)) != QE_OK) return st;
+  if ((st = handshake.out()) != QE_OK) return st;
   if ((st = qe_contract_forward_commit(Lf->contract, mb, tape_out)) != QE_OK) return st;
   return qe_contract_dI_commit(Lb->contract, tape_b);
 }
@@ -365,7 +369,8 @@ static int32_t run_together_impl(qe_ctx* ctx, qe_action* acts, uint32_t n, float
   int32_t st = together_prepare(ctx, dev, n, grad, grad_elems, &pr);  // check (every action, before anything runs)
   if (st != QE_OK) return st;
   cudaStream_t caller = (cudaStream_t)caller_stream;
-  if ((st = handoff_in(ctx, caller)) != QE_OK) return st;
+  Handshake handshake(ctx, caller);
+  if ((st = handshake.in()) != QE_OK) return st;
   if (host)
     for (uint32_t i = 0; i < n; ++i) {
       if (acts[i].kind > QE_ACT_DI) continue;
@@ -392,7 +397,7 @@ static int32_t run_together_impl(qe_ctx* ctx, qe_action* acts, uint32_t n, float
   if (ctx->dw_stream)
     for (uint32_t i = 0; i < n; ++i)
       if (acts[i].kind == QE_ACT_DI) QE_CUDA(cudaEventRecord(acts[i].layer->ev_di[pr.slot[i]], ctx->exec_stream));
-  if ((st = handoff_out(ctx, caller)) != QE_OK) return st;
+  if ((st = handshake.out()) != QE_OK) return st;
   return together_commit(dev, n, grad, pr);  // ... commit (the tapes are written through the callers' pointers)
 }
 
@@ -414,6 +419,7 @@ int32_t qe_step_run(qe_ctx* ctx, qe_layer* const* layers, uint32_t n_layers, con
   for (uint32_t l = 0; l < n_layers; ++l)
     if (!layers[l] || layers[l]->ctx != ctx) return fail(QE_ERR_BAD_ARG, "layer %u is null or belongs to another context", l);
   cudaStream_t caller = (cudaStream_t)caller_stream;
+  Handshake handshake(ctx, caller);
 
   std::vector<qe_tape> tapes((size_t)n_layers * M);
   std::vector<uint8_t> have((size_t)n_layers * M, 0);
@@ -434,7 +440,7 @@ int32_t qe_step_run(qe_ctx* ctx, qe_layer* const* layers, uint32_t n_layers, con
   constexpr size_t kPieceLaunches = 64;
   auto run_piece = [&](const std::vector<qe::Launch>& piece, bool as_graph) -> int32_t {
     if (pieces++ == 0) {
-      const int32_t hs = handoff_in(ctx, caller);
+      const int32_t hs = handshake.in();
       if (hs != QE_OK) return hs;
       if (ctx->dw_stream) {
         // weight-gradient work issued earlier through the overlapped per-action path must finish first: this list's
@@ -617,7 +623,7 @@ int32_t qe_step_run(qe_ctx* ctx, qe_layer* const* layers, uint32_t n_layers, con
 
   // ---- device pass: the launches of every action that passed (in graph mode the ones that are not on their way yet)
   if (run_status == QE_OK && !ls.empty()) run_status = run_piece(ls, check_status == QE_OK);
-  if (run_status == QE_OK && pieces) run_status = handoff_out(ctx, caller);
+  if (run_status == QE_OK && pieces) run_status = handshake.out();
   if (check_status != QE_OK || run_status != QE_OK) {
     // failure boundary: outstanding tapes aborted, arenas unusable for the epoch
     for (uint32_t l = 0; l < n_layers; ++l) qe_contract_abort(layers[l]->contract);

@@ -114,6 +114,31 @@ int32_t build_graph(qe_ctx* ctx, ActionGraph* g, const std::vector<qe::Launch>& 
 int32_t replay_graph(qe_ctx* ctx, ActionGraph* g, const std::vector<qe::Launch>& ls, cudaStream_t stream);
 int32_t handoff_in(qe_ctx* ctx, cudaStream_t caller);
 int32_t handoff_out(qe_ctx* ctx, cudaStream_t caller);
+// The handshake around a call's work.  A call that an error ends in between may have kernels and copies of its own in
+// flight: the caller's stream is ordered after those as well, and the error that ended the call stays the one reported.
+class Handshake {
+ public:
+  Handshake(qe_ctx* ctx, cudaStream_t caller) : ctx_(ctx), caller_(caller) {}
+  Handshake(const Handshake&) = delete;
+  ~Handshake() {
+    if (open_ && caller_ != ctx_->exec_stream && !ctx_->one_way && cudaEventRecord(ctx_->ev_out, ctx_->exec_stream) == cudaSuccess)
+      cudaStreamWaitEvent(caller_, ctx_->ev_out, 0);
+  }
+  int32_t in() {
+    const int32_t st = handoff_in(ctx_, caller_);
+    open_ = st == QE_OK;
+    return st;
+  }
+  int32_t out() {
+    open_ = false;
+    return handoff_out(ctx_, caller_);
+  }
+
+ private:
+  qe_ctx* ctx_;
+  cudaStream_t caller_;
+  bool open_ = false;
+};
 int32_t host_upload(qe_ctx* ctx, void* dst, const void* src_host, size_t bytes, cudaStream_t caller);
 int32_t host_download(qe_ctx* ctx, void* dst_host, const void* src, size_t bytes);
 int32_t run_action(qe_ctx* ctx, ActionGraph* g, const std::vector<qe::Launch>& ls, cudaStream_t stream = nullptr);

@@ -30,3 +30,71 @@ def test_one_layer_under_two_indices_never_shares_a_launch_with_itself(lib):
     s = fake_runtime.Stage(lib, [(256, 256)], M=2, slots=2, window=1)  # action by action the list is a legal one
     assert s.step([("F", 0, 0), ("F", 1, 1), ("dI", 0, 0), ("dI", 1, 1), ("dW", 0, 0), ("dW", 1, 1)], layers=[0, 0]) == 0
     s.close()
+
+
+def _actions(M, n):
+    return [(k, l, m) for m in range(M) for k, order in (("F", range(n)), ("dI", range(n - 1, -1, -1)), ("dW", range(n - 1, -1, -1)))
+            for l in order]
+
+
+@pytest.mark.parametrize("mode,fn,nth", [(1, "cudaGraphInstantiate", 2), (1, "cudaGraphLaunch", 2), (1, "cudaStreamBeginCapture", 2),
+                                         (0, "cudaLaunchKernelExC", 5), (0, "cudaLaunchKernelExC", 90)])
+def test_a_step_that_fails_part_way_leaves_the_callers_stream_behind_what_is_running(lib, mode, fn, nth):
+    s = fake_runtime.Stage(lib, [(256, 256)] * 20, M=4, slots=4, mode=mode, window=4)
+    lib.fake_reset()
+    lib.fake_fail(fn.encode(), nth)
+    assert s.step(_actions(4, 20)) == CUDA
+    order = fake_runtime.Order(lib.fake_log().decode())
+    launches = order.of("launch")
+    assert launches and all(order.seen_by(fake_runtime.CALLER, x) for x in launches)
+    s.close()
+
+
+def _calls(s, lib):
+    """One after the other the calls that put work on the execution stream; the status of each."""
+    import ctypes as C
+
+    from paper_2609_23536_b200 import binding as qe
+
+    T, (K, N) = s.T, s.shapes[0]
+    x, y, grad, at = s.buffer(2 * T * K), s.buffer(2 * T * N), s.grad, fake_runtime.CALLER
+    n = len(s.layers)
+    hs, offs = (C.c_void_p * n)(*[h.value for h in s.layers]), (C.c_uint64 * n)(*s.offsets)
+    tapes, t2 = (qe.qe_tape * n)(), (qe.qe_tape * n)()
+    yield "qe_forward_chain", lambda: lib.qe_forward_chain(hs, n, 0, 0, x, y, at, tapes)
+    yield "qe_backward_dI_chain", lambda: lib.qe_backward_dI_chain(hs, tapes, n, y, x, at)
+    yield "qe_backward_dW_multi", lambda: lib.qe_backward_dW_multi(hs, tapes, n, grad, s.elems, offs, at)
+    for i in range(n):
+        yield "qe_forward", lambda: lib.qe_forward(hs[i], 1, 0, x, y, at, C.byref(t2[i]))
+    acts = (qe.qe_action * 1)(qe.qe_action(1, 1, 0, hs[0], y, x, C.pointer(t2[0]), 0))
+    yield "qe_run_together", lambda: lib.qe_run_together(s.ctx, acts, 1, grad, s.elems, at)
+    yield "qe_backward_dI", lambda: lib.qe_backward_dI(hs[1], C.byref(t2[1]), y, x, at)
+    temp = s.buffer(4 * N * K)
+    yield "qe_backward_dW_staged", lambda: lib.qe_backward_dW_staged(hs[0], C.byref(t2[0]), grad, s.elems, offs[0], temp, at)
+    yield "qe_backward_dW", lambda: lib.qe_backward_dW(hs[1], C.byref(t2[1]), grad, s.elems, offs[1], at)
+    yield "qe_forward", lambda: lib.qe_forward(hs[0], 2, 0, x, y, at, C.byref(t2[0]))
+    yield "qe_forward_dI_pair", lambda: lib.qe_forward_dI_pair(hs[1], 2, 0, x, y, C.byref(t2[1]), hs[0], C.byref(t2[0]), y, x, at)
+
+
+def test_a_call_whose_last_launch_fails_leaves_the_callers_stream_behind_the_others(lib):
+    shapes = [(256, 256)] * 3
+    plain = fake_runtime.Stage(lib, shapes, slots=4)
+    for i, (name, call) in enumerate(_calls(plain, lib)):
+        lib.fake_reset()
+        assert call() == 0, (name, plain.error())
+        n = len(fake_runtime.Order(lib.fake_log().decode()).of("launch"))
+        if n < 2:
+            continue
+        s = fake_runtime.Stage(lib, shapes, slots=4)
+        for j, (_, other) in enumerate(_calls(s, lib)):
+            if j == i:
+                lib.fake_reset()
+                lib.fake_fail(b"cudaLaunchKernelExC", n)
+                assert other() == CUDA
+                break
+            assert other() == 0
+        order = fake_runtime.Order(lib.fake_log().decode())
+        assert len(order.of("launch")) == n - 1
+        assert all(order.seen_by(fake_runtime.CALLER, x) for x in order.of("launch")), name
+        s.close()
+    plain.close()
