@@ -214,9 +214,13 @@ int32_t qe_backward_dI(qe_layer*, const qe_tape*, const void* dy_dev, void* dx_d
  * the staging buffers -- in graph mode the graph's addresses therefore never change -- and the output is copied
  * device-to-host before the execution->caller edge, so it is complete for work the caller queues after the call (or
  * after synchronising caller_stream on the host).  The two copies run on copy streams of the context, ordered with
- * the execution stream by events: the upload of a call overlaps the read-back of the call before it (the host link
- * is full duplex), the kernels wait for both.  Pinned host memory makes the copies asynchronous; y_host / dx_host
- * may be NULL to skip the read-back.  Same checks, state transitions and results as qe_forward / qe_backward_dI. */
+ * the execution stream by events; the kernels wait for both.  Where caller_stream is the context's execution stream,
+ * the upload of a call overlaps the read-back of the call before it (the host link is full duplex), unless that
+ * read-back writes what the upload reads, which is then uploaded after it; other work of the caller's on that stream
+ * that writes a host input must be complete when the call is made.  With any other caller_stream the upload waits for
+ * all that the stream holds, the read-backs of its earlier calls among it.  Pinned host memory makes the copies
+ * asynchronous; y_host / dx_host may be NULL to skip the read-back.  Same checks, state transitions and results as
+ * qe_forward / qe_backward_dI. */
 int32_t qe_forward_host(qe_layer*, uint32_t mb, uint64_t gen, const void* x_host, void* y_host, void* caller_stream,
                         qe_tape* tape_out);
 int32_t qe_backward_dI_host(qe_layer*, const qe_tape*, const void* dy_host, void* dx_host, void* caller_stream);
@@ -267,7 +271,7 @@ int32_t qe_run_together(qe_ctx*, qe_action* actions, uint32_t n, float* grad_buf
 /* The same with HOST buffers for the F and dI actions (layers created with host_io = 1): in_dev / out_dev then hold
  * host pointers (out may be NULL to skip the read-back); every input is uploaded into its layer's staging buffer
  * first, the kernels run on the staging buffers, the outputs are read back afterwards -- copies on the context's
- * two copy streams as in qe_forward_host, so the uploads of a call overlap the read-backs of the call before it. */
+ * two copy streams, ordered as those of qe_forward_host. */
 int32_t qe_run_together_host(qe_ctx*, qe_action* actions, uint32_t n, float* grad_buf_dev, uint64_t grad_buf_elems,
                              void* caller_stream);
 /* FP8 hand-off between directly chained linears (layers[i+1] consumes layers[i]'s output: same T,

@@ -272,7 +272,14 @@ int32_t handoff_out(qe_ctx* ctx, cudaStream_t caller) {
 // ---- host-buffer calls.  The upload of an action runs on one copy stream and the read-back of its result on
 // another, so that the upload of action k+1 overlaps the read-back of action k (the host link is full duplex); the
 // kernels stay on the execution stream, which waits for the upload before them and for the read-back after them
-// (a caller that synchronises after the call finds its host buffer complete).
+// (a caller that synchronises after the call finds its host buffer complete).  An upload comes after every earlier
+// read-back that writes what it reads.
+static int32_t uploads_after_readbacks(qe_ctx* ctx) {
+  QE_CUDA(cudaStreamWaitEvent(ctx->h2d_stream, ctx->ev_d2h, 0));  // recorded after the latest of them
+  ctx->readbacks.clear();
+  return QE_OK;
+}
+
 int32_t host_upload(qe_ctx* ctx, void* dst, const void* src_host, size_t bytes, cudaStream_t caller) {
   if (!ctx->h2d_stream) {
     cudaError_t e = cudaStreamCreateWithFlags(&ctx->h2d_stream, cudaStreamNonBlocking);
@@ -284,7 +291,18 @@ int32_t host_upload(qe_ctx* ctx, void* dst, const void* src_host, size_t bytes, 
   }
   // the staging buffer was last read by the kernels of an earlier host-buffer call
   if (ctx->kernels_recorded) QE_CUDA(cudaStreamWaitEvent(ctx->h2d_stream, ctx->ev_kernels, 0));
-  if (caller != ctx->exec_stream) QE_CUDA(cudaStreamWaitEvent(ctx->h2d_stream, ctx->ev_in, 0));  // recorded by handoff_in
+  if (caller != ctx->exec_stream) {
+    QE_CUDA(cudaStreamWaitEvent(ctx->h2d_stream, ctx->ev_in, 0));  // recorded by handoff_in, after the read-backs of earlier calls
+  } else {
+    // (the execution stream itself: waiting for all of it would keep uploads and read-backs from overlapping)
+    const uintptr_t lo = (uintptr_t)src_host, hi = lo + bytes;
+    for (const qe_ctx::HostRange& r : ctx->readbacks)
+      if (r.lo < hi && lo < r.hi) {
+        const int32_t st = uploads_after_readbacks(ctx);
+        if (st != QE_OK) return st;
+        break;
+      }
+  }
   QE_CUDA(cudaMemcpyAsync(dst, src_host, bytes, cudaMemcpyHostToDevice, ctx->h2d_stream));
   QE_CUDA(cudaEventRecord(ctx->ev_h2d, ctx->h2d_stream));
   QE_CUDA(cudaStreamWaitEvent(ctx->exec_stream, ctx->ev_h2d, 0));
@@ -295,6 +313,11 @@ int32_t host_download(qe_ctx* ctx, void* dst_host, const void* src, size_t bytes
   QE_CUDA(cudaEventRecord(ctx->ev_kernels, ctx->exec_stream));
   ctx->kernels_recorded = true;
   if (!dst_host) return QE_OK;
+  if (ctx->readbacks.size() == 256) {
+    const int32_t st = uploads_after_readbacks(ctx);
+    if (st != QE_OK) return st;
+  }
+  ctx->readbacks.push_back({(uintptr_t)dst_host, (uintptr_t)dst_host + bytes});
   QE_CUDA(cudaStreamWaitEvent(ctx->d2h_stream, ctx->ev_kernels, 0));
   QE_CUDA(cudaMemcpyAsync(dst_host, src, bytes, cudaMemcpyDeviceToHost, ctx->d2h_stream));
   QE_CUDA(cudaEventRecord(ctx->ev_d2h, ctx->d2h_stream));

@@ -71,6 +71,8 @@ struct qe_ctx {
   cudaStream_t h2d_stream = nullptr, d2h_stream = nullptr;
   cudaEvent_t ev_h2d = nullptr, ev_kernels = nullptr, ev_d2h = nullptr;
   bool kernels_recorded = false;
+  struct HostRange { uintptr_t lo, hi; };
+  std::vector<HostRange> readbacks;  // host memory that read-backs write which no upload has been ordered after yet
   qe_registry* registry = nullptr;
   qe_stats stats{};
   // Layers keep their context alive: it is released when the caller has destroyed it AND its last layer is gone,

@@ -98,3 +98,38 @@ def test_a_call_whose_last_launch_fails_leaves_the_callers_stream_behind_the_oth
         assert all(order.seen_by(fake_runtime.CALLER, x) for x in order.of("launch")), name
         s.close()
     plain.close()
+
+
+@pytest.mark.parametrize("own_stream", [True, False], ids=["callers-stream", "execution-stream"])
+def test_a_host_input_that_an_earlier_call_reads_back_is_uploaded_after_that(lib, own_stream):
+    import ctypes as C
+
+    from paper_2609_23536_b200 import binding as qe
+
+    s = fake_runtime.Stage(lib, [(256, 256)] * 3, host_io=True, slots=4, exec_stream=None if own_stream else fake_runtime.CALLER)
+    a, b, c, d = (s.buffer(2 * s.T * 256) for _ in range(4))
+    tape = qe.qe_tape()
+
+    def forward(layer, mb, x, y):
+        assert lib.qe_forward_host(s.layers[layer], mb, 0, x, y, fake_runtime.CALLER, C.byref(tape)) == 0
+
+    lib.fake_reset()
+    forward(0, 0, a, b)
+    forward(1, 0, b, c)                        # the whole buffer
+    forward(2, 0, c + 2 * 256 * 255, a)        # its last row
+    order = fake_runtime.Order(lib.fake_log().decode())
+    up, down = order.of("h2d"), order.of("d2h")
+    assert order.before(down[0], up[1]) and order.before(down[1], up[2])
+    lib.fake_reset()
+    forward(0, 1, a, b)
+    forward(1, 1, d, c)                        # other memory: the link is used in both directions at once
+    order = fake_runtime.Order(lib.fake_log().decode())
+    assert order.before(order.of("d2h")[0], order.of("h2d")[1]) == own_stream
+    lib.fake_reset()
+    for i in range(600):                       # however many read-backs lie in between
+        assert lib.qe_abort_step(s.layers[0]) == 0 and lib.qe_arena_rebuild(s.layers[0]) == 0
+        forward(0, 0, a, b if i == 0 else d)
+    forward(2, 1, b, c)
+    order = fake_runtime.Order(lib.fake_log().decode())
+    assert order.before(order.of("d2h")[0], order.of("h2d")[-1])
+    s.close()
