@@ -771,6 +771,7 @@ template <int NP, int NOPS>
 Launch make_launch(const GemmDesc* probs, uint32_t n, uint32_t nops, int num_sms, const void* func) {
   using P = GemmLaunchParams<NP, NOPS>;
   static_assert(sizeof(P) <= sizeof(Launch::Block), "parameter block too large");
+  static_assert(NP > 1 || sizeof(P) <= ParamBytes::kInline, "a launch of one problem takes no heap memory");
   Launch l;
   l.nbytes = sizeof(P);
   l.params.resize(offsetof(P, op) + nops * sizeof(GemmOperands));  // (a step has hundreds of launches: no unused operands)

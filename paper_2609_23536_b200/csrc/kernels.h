@@ -6,7 +6,9 @@
 #include <cuda.h>
 #include <cuda_runtime.h>
 
+#include <cstddef>
 #include <cstdint>
+#include <utility>
 #include <vector>
 
 namespace qe {
@@ -158,17 +160,55 @@ struct StatusGatherParams {
   uint32_t accumulate;
 };
 
+// Bytes of a parameter block.  Those of a launch of one problem live inside the object: the standalone calls, and with
+// them the one that promises to touch no allocator, take no heap memory.
+class ParamBytes {
+ public:
+  static constexpr size_t kInline = 768;
+  ParamBytes() = default;
+  ParamBytes(const ParamBytes& o) { *this = o; }
+  ParamBytes(ParamBytes&& o) noexcept { *this = std::move(o); }
+  ParamBytes& operator=(const ParamBytes& o) {
+    if (this == &o) return *this;
+    if (o.n_ > kInline) more_.assign(o.more_.begin(), o.more_.end());
+    else __builtin_memcpy(here_, o.here_, o.n_);
+    n_ = o.n_;
+    return *this;
+  }
+  ParamBytes& operator=(ParamBytes&& o) noexcept {
+    if (this == &o) return *this;
+    if (o.n_ > kInline) more_ = std::move(o.more_);
+    else __builtin_memcpy(here_, o.here_, o.n_);
+    n_ = o.n_;
+    o.n_ = 0;
+    return *this;
+  }
+  void resize(size_t n) {  // all bytes zero
+    if (n > kInline) more_.assign(n, 0);
+    else __builtin_memset(here_, 0, n);
+    n_ = n;
+  }
+  size_t size() const { return n_; }
+  unsigned char* data() { return n_ > kInline ? more_.data() : here_; }
+  const unsigned char* data() const { return n_ > kInline ? more_.data() : here_; }
+
+ private:
+  size_t n_ = 0;
+  alignas(64) unsigned char here_[kInline];
+  std::vector<unsigned char> more_;
+};
+
 // One launch, self-contained.
 struct Launch {
   const void* func = nullptr;
   dim3 grid{1, 1, 1}, block{1, 1, 1};
   uint32_t smem = 0;
-  std::vector<unsigned char> params;  // the parameter block, without an unused tail ...
-  uint32_t nbytes = 0;                // ... of a block of this size
+  ParamBytes params;    // the parameter block, without an unused tail ...
+  uint32_t nbytes = 0;  // ... of a block of this size
   template <class P>
   void set(const P& p) {
-    const unsigned char* b = reinterpret_cast<const unsigned char*>(&p);
-    params.assign(b, b + sizeof(P));
+    params.resize(sizeof(P));
+    __builtin_memcpy(params.data(), &p, sizeof(P));
     nbytes = sizeof(P);
   }
   // The whole block as the runtime wants it (valid as long as the launch and the buffer are).

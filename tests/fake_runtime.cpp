@@ -189,7 +189,8 @@ Launch named(const char* fmt, ...) {
   va_end(a);
   Launch l;
   l.func = kKernels;
-  l.params.assign(b, b + sizeof(b));
+  l.params.resize(sizeof(b));
+  std::memcpy(l.params.data(), b, sizeof(b));
   l.nbytes = sizeof(b);
   return l;
 }

@@ -133,3 +133,14 @@ def test_a_host_input_that_an_earlier_call_reads_back_is_uploaded_after_that(lib
     order = fake_runtime.Order(lib.fake_log().decode())
     assert order.before(order.of("d2h")[0], order.of("h2d")[-1])
     s.close()
+
+
+def test_the_call_that_must_not_allocate_takes_no_heap_memory(lib):
+    import ctypes as C
+
+    buf = (C.c_char * (1 << 20))()
+    a = (C.addressof(buf) + 255) // 256 * 256
+    call = lambda: lib.qe_gemm_fp8_staged_noalloc(a, 0, a, 0, 256, 256, 256, a, a, a, 0, a, None)  # noqa: E731
+    assert call() == 0  # the warm-up, which may
+    lib.fake_fail_alloc(1)
+    assert call() == 0 and lib.fake_alloc_left() == 1
