@@ -4,6 +4,7 @@
 
 #include <algorithm>
 #include <cstring>
+#include <memory>
 #include <new>
 #include <vector>
 
@@ -44,32 +45,35 @@ int32_t qe_contract::resolve(const qe_tape* t, uint32_t* p_out) const {
 
 extern "C" {
 
-int32_t qe_registry_create(qe_registry** out) {
+int32_t qe_registry_create(qe_registry** out) try {
   if (!out) return fail(QE_ERR_BAD_ARG, "out is null");
-  *out = new (std::nothrow) qe_registry();
-  if (!*out) return fail(QE_ERR_BAD_ARG, "out of host memory");
-  (*out)->state = std::make_shared<qe::RegistryState>();
+  auto r = std::make_unique<qe_registry>();
+  r->state = std::make_shared<qe::RegistryState>();
+  *out = r.release();
   return QE_OK;
-}
+} QE_NO_MEMORY
 int32_t qe_registry_destroy(qe_registry* r) {
   delete r;
   return QE_OK;
 }
 
 int32_t qe_contract_create(uint32_t slots, uint32_t stage, uint32_t unit, uint32_t inv, qe_registry* registry,
-                           qe_contract** out) {
+                           qe_contract** out) try {
   if (!out) return fail(QE_ERR_BAD_ARG, "out is null");
   if (slots < 1 || slots > QE_MAX_SLOTS) return fail(QE_ERR_BAD_ARG, "slots %u not in [1, %u]", slots, QE_MAX_SLOTS);
-  qe_contract* c = new (std::nothrow) qe_contract();
-  if (!c) return fail(QE_ERR_BAD_ARG, "out of host memory");
+  auto c = std::make_unique<qe_contract>();
   c->P = slots;
   c->stage = stage;
   c->unit = unit;
   c->inv = inv;
-  if (registry) c->registry = registry->state;
-  *out = c;
+  if (registry) {  // its entry (an empty range) is made here: a commit must not fail
+    std::lock_guard<std::mutex> g(registry->state->mu);
+    registry->state->bound[c.get()] = {};
+    c->registry = registry->state;
+  }
+  *out = c.release();
   return QE_OK;
-}
+} QE_NO_MEMORY
 
 int32_t qe_contract_destroy(qe_contract* c) {
   if (c && c->registry) {
@@ -213,7 +217,7 @@ int32_t qe_contract_boundary(qe_contract* c, uint32_t expected) {
   c->has_dest = false;
   if (c->registry) {
     std::lock_guard<std::mutex> g(c->registry->mu);
-    c->registry->bound.erase(c);
+    c->registry->bound[c] = {};
   }
   return QE_OK;
 }
@@ -236,7 +240,7 @@ int32_t qe_contract_rebuild(qe_contract* c) {
   c->has_dest = false;
   if (c->registry) {
     std::lock_guard<std::mutex> g(c->registry->mu);
-    c->registry->bound.erase(c);
+    c->registry->bound[c] = {};
   }
   return QE_OK;
 }
@@ -264,7 +268,7 @@ int32_t qe_contract_restore(qe_contract* c, uint64_t e_W) {
   c->has_dest = false;
   if (c->registry) {
     std::lock_guard<std::mutex> g(c->registry->mu);
-    c->registry->bound.erase(c);
+    c->registry->bound[c] = {};
   }
   return QE_OK;
 }
@@ -292,7 +296,7 @@ int32_t qe_contract_get(const qe_contract* c, qe_contract_view* v) {
 // ---- issue plan of a whole-step action list (host logic only; used by qe_step_run)
 int32_t qe_plan_rounds(const qe_step_action* actions, uint32_t n_actions, uint32_t n_layers, uint32_t microbatches,
                        const uint32_t* slots, const uint32_t* live_now, uint32_t window, uint32_t max_group,
-                       uint32_t* round_of_action, uint32_t* n_rounds_out) {
+                       uint32_t* round_of_action, uint32_t* n_rounds_out) try {
   if (!actions || !slots || !round_of_action || !n_rounds_out) return fail(QE_ERR_BAD_ARG, "null argument");
   if (n_actions == 0 || n_layers == 0 || microbatches == 0 || window == 0 || max_group == 0) return fail(QE_ERR_BAD_ARG, "empty list or zero limit");
   const uint32_t M = microbatches;
@@ -363,13 +367,13 @@ int32_t qe_plan_rounds(const qe_step_action* actions, uint32_t n_actions, uint32
   }
   *n_rounds_out = round;
   return QE_OK;
-}
+} QE_NO_MEMORY
 
 // ---- issue plan of the whole-step call.  F and dI as in qe_plan_rounds (but the window counts F and dI units only, and
 // each layer sees its actions of a kind strictly in list order); dW actions wait and go out several microbatches at once.
 int32_t qe_plan_step(const qe_step_action* actions, uint32_t n_actions, uint32_t n_layers, uint32_t microbatches,
                      const uint32_t* slots, const uint32_t* live_now, uint32_t window, uint32_t max_group,
-                     uint32_t max_sum, uint32_t* round_of_action, uint32_t* n_rounds_out) {
+                     uint32_t max_sum, uint32_t* round_of_action, uint32_t* n_rounds_out) try {
   if (!actions || !slots || !round_of_action || !n_rounds_out) return fail(QE_ERR_BAD_ARG, "null argument");
   if (n_actions == 0 || n_layers == 0 || microbatches == 0 || window == 0 || max_group == 0 || max_sum == 0) return fail(QE_ERR_BAD_ARG, "empty list or zero limit");
   const uint32_t M = microbatches;
@@ -466,6 +470,6 @@ int32_t qe_plan_step(const qe_step_action* actions, uint32_t n_actions, uint32_t
   }
   *n_rounds_out = round;
   return QE_OK;
-}
+} QE_NO_MEMORY
 
 }  // extern "C"

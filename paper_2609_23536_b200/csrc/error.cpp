@@ -17,6 +17,7 @@ int32_t fail(int32_t status, const char* fmt, ...) {
   return status;
 }
 void clear_error() { g_msg[0] = 0; }
+int32_t out_of_memory() { return fail(QE_ERR_BAD_ARG, "out of host memory"); }
 }  // namespace qe
 
 extern "C" const char* qe_last_error(void) { return qe::g_msg; }

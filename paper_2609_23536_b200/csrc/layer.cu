@@ -185,18 +185,18 @@ static int32_t forward_impl(qe_layer* L, uint32_t mb, uint64_t gen, const void* 
 }
 
 int32_t qe_forward(qe_layer* L, uint32_t mb, uint64_t gen, const void* x, void* y, void* caller_stream,
-                   qe_tape* tape_out) {
+                   qe_tape* tape_out) try {
   if (!L || !x || !y || !tape_out) return fail(QE_ERR_BAD_ARG, "null argument");
   if (((uintptr_t)x | (uintptr_t)y) & 15u) return fail(QE_ERR_BAD_ARG, "x and y must be 16-byte aligned");
   return forward_impl(L, mb, gen, x, y, caller_stream, tape_out, nullptr, nullptr);
-}
+} QE_NO_MEMORY
 
 int32_t qe_forward_host(qe_layer* L, uint32_t mb, uint64_t gen, const void* x_host, void* y_host, void* caller_stream,
-                        qe_tape* tape_out) {
+                        qe_tape* tape_out) try {
   if (!L || !x_host || !tape_out) return fail(QE_ERR_BAD_ARG, "null argument");
   if (!L->x_stage) return fail(QE_ERR_BAD_ARG, "layer was created without host_io");
   return forward_impl(L, mb, gen, L->x_stage, L->y_stage, caller_stream, tape_out, x_host, y_host);
-}
+} QE_NO_MEMORY
 
 static int32_t backward_dI_impl(qe_layer* L, const qe_tape* tape, const void* dy, void* dx, void* caller_stream,
                                 const void* dy_host, void* dx_host) {
@@ -217,17 +217,17 @@ static int32_t backward_dI_impl(qe_layer* L, const qe_tape* tape, const void* dy
   return qe_contract_dI_commit(L->contract, tape);
 }
 
-int32_t qe_backward_dI(qe_layer* L, const qe_tape* tape, const void* dy, void* dx, void* caller_stream) {
+int32_t qe_backward_dI(qe_layer* L, const qe_tape* tape, const void* dy, void* dx, void* caller_stream) try {
   if (!L || !tape || !dy || !dx) return fail(QE_ERR_BAD_ARG, "null argument");
   if (((uintptr_t)dy | (uintptr_t)dx) & 15u) return fail(QE_ERR_BAD_ARG, "dy and dx must be 16-byte aligned");
   return backward_dI_impl(L, tape, dy, dx, caller_stream, nullptr, nullptr);
-}
+} QE_NO_MEMORY
 
-int32_t qe_backward_dI_host(qe_layer* L, const qe_tape* tape, const void* dy_host, void* dx_host, void* caller_stream) {
+int32_t qe_backward_dI_host(qe_layer* L, const qe_tape* tape, const void* dy_host, void* dx_host, void* caller_stream) try {
   if (!L || !tape || !dy_host) return fail(QE_ERR_BAD_ARG, "null argument");
   if (!L->dy_stage) return fail(QE_ERR_BAD_ARG, "layer was created without host_io");
   return backward_dI_impl(L, tape, L->dy_stage, L->dx_stage, caller_stream, dy_host, dx_host);
-}
+} QE_NO_MEMORY
 
 // view != null: per-microbatch arena mode; grad / elems / off / slice then describe the layer's whole region of the
 // arena in 4-byte units (what the contract core's destination rules are written in) and view is this microbatch's.
@@ -268,18 +268,18 @@ static int32_t backward_dW_impl(qe_layer* L, const qe_tape* tape, float* grad, u
   return qe_contract_dW_commit(L->contract, tape, (uint64_t)(uintptr_t)grad, off, slice);
 }
 
-int32_t qe_backward_dW(qe_layer* L, const qe_tape* tape, float* grad, uint64_t elems, uint64_t off, void* stream) {
+int32_t qe_backward_dW(qe_layer* L, const qe_tape* tape, float* grad, uint64_t elems, uint64_t off, void* stream) try {
   return backward_dW_impl(L, tape, grad, elems, off, nullptr, stream);
-}
+} QE_NO_MEMORY
 
 int32_t qe_backward_dW_staged(qe_layer* L, const qe_tape* tape, float* grad, uint64_t elems, uint64_t off,
-                              float* temp, void* stream) {
+                              float* temp, void* stream) try {
   if (!temp || ((uintptr_t)temp & 15u)) return fail(QE_ERR_BAD_ARG, "temp_dev must be non-null and 16-byte aligned");
   return backward_dW_impl(L, tape, grad, elems, off, temp, stream);
-}
+} QE_NO_MEMORY
 
 int32_t qe_backward_dW_arena(qe_layer* L, const qe_tape* tape, void* arena, uint64_t arena_elems, uint64_t layer_offset,
-                             uint32_t microbatches, void* stream) {
+                             uint32_t microbatches, void* stream) try {
   if (!L || !tape || !arena) return fail(QE_ERR_BAD_ARG, "null argument");
   if (microbatches < 1 || microbatches > QE_MAX_MICROBATCHES) return fail(QE_ERR_BAD_ARG, "microbatches %u", microbatches);
   const uint64_t n = (uint64_t)L->cfg.N * L->cfg.K;
@@ -288,10 +288,10 @@ int32_t qe_backward_dW_arena(qe_layer* L, const qe_tape* tape, void* arena, uint
   uint16_t* view = (uint16_t*)arena + layer_offset + (uint64_t)tape->key.mb * n;
   // 2-byte elements expressed in the contract core's 4-byte units (n is even: N and K are multiples of 128)
   return backward_dW_impl(L, tape, (float*)arena, arena_elems / 2, layer_offset / 2, nullptr, stream, view, microbatches * n / 2);
-}
+} QE_NO_MEMORY
 
 int32_t qe_arena_finalize(qe_layer* L, const void* arena, uint64_t arena_elems, uint64_t layer_offset, uint32_t microbatches,
-                          float* grad, uint64_t grad_elems, uint64_t off, void* caller_stream) {
+                          float* grad, uint64_t grad_elems, uint64_t off, void* caller_stream) try {
   if (!L || !arena || !grad) return fail(QE_ERR_BAD_ARG, "null argument");
   if (microbatches < 1 || microbatches > QE_MAX_MICROBATCHES) return fail(QE_ERR_BAD_ARG, "microbatches %u", microbatches);
   const qe_contract* c = L->contract;
@@ -320,7 +320,7 @@ int32_t qe_arena_finalize(qe_layer* L, const void* arena, uint64_t arena_elems, 
   ap.M = microbatches;
   if ((st = launch_eager(ctx, qe::make_arena_reduce(ap), ctx->exec_stream)) != QE_OK) return st;
   return handshake.out();
-}
+} QE_NO_MEMORY
 
 static int32_t read_status(qe_layer* L, uint32_t* status) {
   QE_CUDA(cudaStreamSynchronize(L->ctx->exec_stream));
@@ -338,7 +338,7 @@ int32_t qe_optimizer_boundary(qe_layer* L, uint32_t expected) {
   return qe_contract_boundary(L->contract, expected);
 }
 
-int32_t qe_optimizer_boundary_all(qe_layer* const* layers, uint32_t n, uint32_t expected) {
+int32_t qe_optimizer_boundary_all(qe_layer* const* layers, uint32_t n, uint32_t expected) try {
   if (!layers || n < 1 || n > 4096) return fail(QE_ERR_BAD_ARG, "layers null or n = %u out of range", n);
   for (uint32_t i = 0; i < n; ++i) {
     if (!layers[i]) return fail(QE_ERR_BAD_ARG, "layers[%u] is null", i);
@@ -369,9 +369,9 @@ int32_t qe_optimizer_boundary_all(qe_layer* const* layers, uint32_t n, uint32_t 
   }
   for (uint32_t i = 0; i < n; ++i) qe_contract_boundary(layers[i]->contract, expected);
   return QE_OK;
-}
+} QE_NO_MEMORY
 
-int32_t qe_scale_commit(qe_layer* L, uint32_t cls, const float* amax_dev, void* caller_stream) {
+int32_t qe_scale_commit(qe_layer* L, uint32_t cls, const float* amax_dev, void* caller_stream) try {
   if (!L) return fail(QE_ERR_BAD_ARG, "layer is null");
   if (cls > QE_CLASS_Y) return fail(QE_ERR_BAD_ARG, "tensor_class %u", cls);
   qe_ctx* ctx = L->ctx;
@@ -383,7 +383,7 @@ int32_t qe_scale_commit(qe_layer* L, uint32_t cls, const float* amax_dev, void* 
   ls.push_back(qe::make_commit(commit_params(L, 1u << cls, 0, amax_dev)));
   if ((st = run_action(ctx, &L->gCommit, ls)) != QE_OK) return st;
   return handshake.out();
-}
+} QE_NO_MEMORY
 
 int32_t qe_abort_step(qe_layer* L) {
   if (!L) return fail(QE_ERR_BAD_ARG, "layer is null");
@@ -405,7 +405,7 @@ int32_t qe_next_slot(const qe_layer* L, uint32_t* slot_out) {
   return QE_OK;
 }
 
-int32_t qe_get_state(qe_layer* L, qe_state_view* out, float* window_out, float* slot_sinv_out) {
+int32_t qe_get_state(qe_layer* L, qe_state_view* out, float* window_out, float* slot_sinv_out) try {
   if (!L || !out) return fail(QE_ERR_BAD_ARG, "null argument");
   QE_CUDA(cudaStreamSynchronize(L->ctx->exec_stream));
   if (L->ctx->dw_stream) QE_CUDA(cudaStreamSynchronize(L->ctx->dw_stream));
@@ -438,9 +438,9 @@ int32_t qe_get_state(qe_layer* L, qe_state_view* out, float* window_out, float* 
       slot_sinv_out[P + p] = h.slot_sinv_G[p];
     }
   return QE_OK;
-}
+} QE_NO_MEMORY
 
-int32_t qe_read_fp8(qe_layer* L, uint32_t which, uint32_t slot, void* host_out, uint64_t bytes) {
+int32_t qe_read_fp8(qe_layer* L, uint32_t which, uint32_t slot, void* host_out, uint64_t bytes) try {
   if (!L || !host_out) return fail(QE_ERR_BAD_ARG, "null argument");
   const uint64_t tk = (uint64_t)L->cfg.T * L->cfg.K, tn = (uint64_t)L->cfg.T * L->cfg.N, nk = (uint64_t)L->cfg.N * L->cfg.K;
   if (which > 5 || (which < 4 && slot >= L->cfg.slots)) return fail(QE_ERR_BAD_ARG, "which %u slot %u", which, slot);
@@ -457,12 +457,16 @@ int32_t qe_read_fp8(qe_layer* L, uint32_t which, uint32_t slot, void* host_out, 
     return QE_OK;
   }
   const uint64_t rows = which == 5 ? L->cfg.N : L->cfg.T, cols = need / rows;
-  std::vector<uint8_t> m(need);
-  QE_CUDA(cudaMemcpy(m.data(), src, need, cudaMemcpyDeviceToHost));
-  for (uint64_t c = 0; c < cols; ++c)
-    for (uint64_t r = 0; r < rows; ++r) ((uint8_t*)host_out)[c * rows + r] = m[r * cols + c];
+  const uint64_t band = std::min<uint64_t>(rows, std::max<uint64_t>(1, (16ull << 20) / cols));  // rows at a time
+  std::vector<uint8_t> m(band * cols);
+  for (uint64_t r0 = 0; r0 < rows; r0 += band) {
+    const uint64_t n = std::min(band, rows - r0);
+    QE_CUDA(cudaMemcpy(m.data(), src + r0 * cols, n * cols, cudaMemcpyDeviceToHost));
+    for (uint64_t c = 0; c < cols; ++c)
+      for (uint64_t r = 0; r < n; ++r) ((uint8_t*)host_out)[c * rows + r0 + r] = m[r * cols + c];
+  }
   return QE_OK;
-}
+} QE_NO_MEMORY
 
 // ------------------------------------------------------------------------------------------------ checkpoint
 namespace {

@@ -163,6 +163,9 @@ int32_t launch_eager(qe_ctx* ctx, const qe::Launch& l, cudaStream_t stream) {
 // launch order by walking the (linear) dependency chain from the root.
 int32_t build_graph(qe_ctx* ctx, ActionGraph* g, const std::vector<qe::Launch>& ls, cudaStream_t stream) {
   const auto t0 = std::chrono::steady_clock::now();
+  std::vector<qe::Launch> kept = ls;  // (all memory before the capture: nothing below fails for lack of it)
+  std::vector<cudaGraphNode_t> chain;
+  chain.reserve(ls.size());
   QE_CUDA(cudaStreamBeginCapture(stream, cudaStreamCaptureModeThreadLocal));
   cudaError_t err = cudaSuccess;
   for (const qe::Launch& l : ls) {
@@ -182,7 +185,6 @@ int32_t build_graph(qe_ctx* ctx, ActionGraph* g, const std::vector<qe::Launch>& 
     cudaGraphDestroy(graph);
     return fail(QE_ERR_CUDA, "captured %zu nodes for %zu launches", n, ls.size());
   }
-  std::vector<cudaGraphNode_t> chain;
   size_t nroot = 1;
   cudaGraphNode_t cur = nullptr;
   QE_CUDA(cudaGraphGetRootNodes(graph, &cur, &nroot));
@@ -214,8 +216,8 @@ int32_t build_graph(qe_ctx* ctx, ActionGraph* g, const std::vector<qe::Launch>& 
   }
   g->graph = graph;
   g->exec = exec;
-  g->nodes = chain;
-  g->launches = ls;
+  g->nodes = std::move(chain);
+  g->launches = std::move(kept);
   g->built = true;
   ctx->stats.graphs_built += 1;
   ctx->stats.capture_host_ms += std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
@@ -282,6 +284,7 @@ static int32_t uploads_after_readbacks(qe_ctx* ctx) {
 
 int32_t host_upload(qe_ctx* ctx, void* dst, const void* src_host, size_t bytes, cudaStream_t caller) {
   if (!ctx->h2d_stream) {
+    ctx->readbacks.reserve(256);
     cudaError_t e = cudaStreamCreateWithFlags(&ctx->h2d_stream, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&ctx->d2h_stream, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ctx->ev_h2d, cudaEventDisableTiming);
@@ -352,6 +355,7 @@ ActionGraph* keyed_graph(qe_ctx* ctx, uint64_t key, size_t n_launches) {
     sg->g = ActionGraph();
   }
   if (!sg) {
+    ctx->step_graphs.reserve(ctx->step_graphs.size() + 1);
     sg = new (std::nothrow) qe_ctx::StepGraph();
     if (!sg) return nullptr;
     sg->key = key;

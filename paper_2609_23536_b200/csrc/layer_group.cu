@@ -7,7 +7,7 @@ using namespace qe_impl;
 extern "C" {
 
 int32_t qe_backward_dW_multi(qe_layer* const* layers, const qe_tape* tapes, uint32_t n, float* grad, uint64_t elems,
-                             const uint64_t* offsets, void* caller_stream) {
+                             const uint64_t* offsets, void* caller_stream) try {
   if (!layers || !tapes || !offsets || n == 0 || n > QE_MAX_MULTI_DW) return fail(QE_ERR_BAD_ARG, "null argument or bad count %u", n);
   qe_ctx* ctx = layers[0] ? layers[0]->ctx : nullptr;
   for (uint32_t i = 0; i < n; ++i) {
@@ -69,7 +69,7 @@ int32_t qe_backward_dW_multi(qe_layer* const* layers, const qe_tape* tapes, uint
     if ((st = qe_contract_dW_commit(layers[i]->contract, &tapes[i], (uint64_t)(uintptr_t)grad, offsets[i], slice)) != QE_OK) return st;
   }
   return QE_OK;
-}
+} QE_NO_MEMORY
 
 // ------------------------------------------------------------------------------------------------ chained linears
 static int32_t check_chain(qe_layer* const* layers, uint32_t n) {
@@ -89,7 +89,7 @@ static int32_t check_chain(qe_layer* const* layers, uint32_t n) {
 }
 
 int32_t qe_forward_chain(qe_layer* const* layers, uint32_t n, uint32_t mb, uint64_t gen, const void* x, void* y,
-                         void* caller_stream, qe_tape* tapes_out) {
+                         void* caller_stream, qe_tape* tapes_out) try {
   int32_t st = check_chain(layers, n);
   if (st != QE_OK) return st;
   if (!x || !y || !tapes_out) return fail(QE_ERR_BAD_ARG, "null argument");
@@ -125,10 +125,10 @@ int32_t qe_forward_chain(qe_layer* const* layers, uint32_t n, uint32_t mb, uint6
   for (uint32_t i = 0; i < n; ++i)
     if ((st = qe_contract_forward_commit(layers[i]->contract, mb, &tapes_out[i])) != QE_OK) return st;
   return QE_OK;
-}
+} QE_NO_MEMORY
 
 int32_t qe_backward_dI_chain(qe_layer* const* layers, const qe_tape* tapes, uint32_t n, const void* dy, void* dx,
-                             void* caller_stream) {
+                             void* caller_stream) try {
   int32_t st = check_chain(layers, n);
   if (st != QE_OK) return st;
   if (!tapes || !dy || !dx) return fail(QE_ERR_BAD_ARG, "null argument");
@@ -156,14 +156,14 @@ int32_t qe_backward_dI_chain(qe_layer* const* layers, const qe_tape* tapes, uint
   for (uint32_t i = 0; i < n; ++i)
     if ((st = qe_contract_dI_commit(layers[i]->contract, &tapes[i])) != QE_OK) return st;
   return QE_OK;
-}
+} QE_NO_MEMORY
 
 // ------------------------------------------------------------------------------------------------ F and dI together
 // In the steady state of a split-backward schedule a stage holds a forward unit (microbatch m + k) and an input-
 // gradient unit (microbatch m) at the same time.  Their chains through the layers are independent, so F of layer i
 // and dI of layer j (two different layers) can share one GEMM launch: one fixed cost and common waves.
 int32_t qe_forward_dI_pair(qe_layer* Lf, uint32_t mb, uint64_t gen, const void* x, void* y, qe_tape* tape_out,
-                           qe_layer* Lb, const qe_tape* tape_b, const void* dy, void* dx, void* caller_stream) {
+                           qe_layer* Lb, const qe_tape* tape_b, const void* dy, void* dx, void* caller_stream) try {
   if (!Lf || !Lb || !x || !y || !tape_out || !tape_b || !dy || !dx) return fail(QE_ERR_BAD_ARG, "null argument");
   if (Lf == Lb || Lf->ctx != Lb->ctx) return fail(QE_ERR_BAD_ARG, "the two layers must be different layers of one context");
   if (((uintptr_t)x | (uintptr_t)y | (uintptr_t)dy | (uintptr_t)dx) & 15u) return fail(QE_ERR_BAD_ARG, "tensors must be 16-byte aligned");
@@ -208,7 +208,7 @@ int32_t qe_forward_dI_pair(qe_layer* Lf, uint32_t mb, uint64_t gen, const void* 
   if ((st = handshake.out()) != QE_OK) return st;
   if ((st = qe_contract_forward_commit(Lf->contract, mb, tape_out)) != QE_OK) return st;
   return qe_contract_dI_commit(Lb->contract, tape_b);
-}
+} QE_NO_MEMORY
 
 // ------------------------------------------------------------------------------------------------ independent actions
 namespace {
@@ -401,18 +401,18 @@ static int32_t run_together_impl(qe_ctx* ctx, qe_action* acts, uint32_t n, float
   return together_commit(dev, n, grad, pr);  // ... commit (the tapes are written through the callers' pointers)
 }
 
-int32_t qe_run_together(qe_ctx* ctx, qe_action* acts, uint32_t n, float* grad, uint64_t grad_elems, void* caller_stream) {
+int32_t qe_run_together(qe_ctx* ctx, qe_action* acts, uint32_t n, float* grad, uint64_t grad_elems, void* caller_stream) try {
   return run_together_impl(ctx, acts, n, grad, grad_elems, caller_stream, 0);
-}
+} QE_NO_MEMORY
 
-int32_t qe_run_together_host(qe_ctx* ctx, qe_action* acts, uint32_t n, float* grad, uint64_t grad_elems, void* caller_stream) {
+int32_t qe_run_together_host(qe_ctx* ctx, qe_action* acts, uint32_t n, float* grad, uint64_t grad_elems, void* caller_stream) try {
   return run_together_impl(ctx, acts, n, grad, grad_elems, caller_stream, 1);
-}
+} QE_NO_MEMORY
 
 // ------------------------------------------------------------------------------------------------ whole-step call
 int32_t qe_step_run(qe_ctx* ctx, qe_layer* const* layers, uint32_t n_layers, const qe_step_action* actions,
                     uint32_t n_actions, uint32_t M, const qe_step_io* io, float* grad, uint64_t grad_elems,
-                    const uint64_t* offsets, float* temp, void* caller_stream) {
+                    const uint64_t* offsets, float* temp, void* caller_stream) try {
   if (!ctx || !layers || !actions || !io || !offsets) return fail(QE_ERR_BAD_ARG, "null argument");
   if (n_layers == 0 || n_actions == 0 || M == 0 || M > QE_MAX_MICROBATCHES) return fail(QE_ERR_BAD_ARG, "empty list or bad microbatch count");
   if (temp && ((uintptr_t)temp & 15u)) return fail(QE_ERR_BAD_ARG, "temp_dev must be 16-byte aligned");
@@ -631,6 +631,9 @@ int32_t qe_step_run(qe_ctx* ctx, qe_layer* const* layers, uint32_t n_layers, con
     return run_status;
   }
   return QE_OK;
+} catch (const std::bad_alloc&) {  // (the layers were looked at before anything was allocated)
+  for (uint32_t l = 0; l < n_layers; ++l) qe_contract_abort(layers[l]->contract);
+  return qe::out_of_memory();
 }
 
 }  // extern "C"

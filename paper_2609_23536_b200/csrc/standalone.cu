@@ -115,7 +115,7 @@ int32_t qe_gemm_fp8_ex(const void* a, uint32_t a_fmt, uint32_t a_mn, const void*
   return launch_on(qe::make_gemm(sg.desc, dev->num_sms), (cudaStream_t)stream);
 }
 
-int32_t qe_gemm_fp8_group(const qe_gemm_desc* descs, uint32_t n, uint32_t* status_dev, void* stream) {
+int32_t qe_gemm_fp8_group(const qe_gemm_desc* descs, uint32_t n, uint32_t* status_dev, void* stream) try {
   if (!descs || !status_dev) return fail(QE_ERR_BAD_ARG, "null argument");
   if (n < 2 || n > 8) return fail(QE_ERR_BAD_ARG, "a group holds 2 to 8 problems, got %u", n);
   DeviceInfo* dev = nullptr;
@@ -134,7 +134,7 @@ int32_t qe_gemm_fp8_group(const qe_gemm_desc* descs, uint32_t n, uint32_t* statu
   qe::Launch l;
   if (!qe::make_gemm_group(gp, n, dev->num_sms, &l)) return fail(QE_ERR_UNSUPPORTED, "the problems cannot share a launch");
   return launch_on(l, (cudaStream_t)stream);
-}
+} QE_NO_MEMORY
 
 int32_t qe_gemm_fp8(const void* a, uint32_t a_fmt, const void* b, uint32_t b_fmt, uint32_t M, uint32_t Nn, uint32_t Kc,
                     const float* alpha_a, const float* alpha_b, void* d, uint32_t out_kind, float* amax_dev,

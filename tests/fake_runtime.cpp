@@ -69,14 +69,18 @@ const char kKernels[8] = {};  // addresses that stand for kernels
 }  // namespace
 
 // the library's own allocations (it is linked so that its calls come here)
-void* operator new(size_t n) {
+static void* allocate(size_t n, size_t align) {
   if (g && g->alloc_in > 0 && --g->alloc_in == 0) throw std::bad_alloc();
-  void* p = std::malloc(n ? n : 1);
+  void* p = std::aligned_alloc(align, (n + align) / align * align);
   if (!p) throw std::bad_alloc();
   return p;
 }
+void* operator new(size_t n) { return allocate(n, 16); }
+void* operator new(size_t n, std::align_val_t a) { return allocate(n, (size_t)a); }
 void operator delete(void* p) noexcept { std::free(p); }
 void operator delete(void* p, size_t) noexcept { std::free(p); }
+void operator delete(void* p, std::align_val_t) noexcept { std::free(p); }
+void operator delete(void* p, size_t, std::align_val_t) noexcept { std::free(p); }
 
 extern "C" {
 const char* fake_log() { return s().log.c_str(); }

@@ -144,3 +144,60 @@ def test_the_call_that_must_not_allocate_takes_no_heap_memory(lib):
     assert call() == 0  # the warm-up, which may
     lib.fake_fail_alloc(1)
     assert call() == 0 and lib.fake_alloc_left() == 1
+
+
+def out_of_memory(so):
+    """(runs in a process of its own) Every allocation of every call fails in turn: the call says so, leaves the caller's
+    stream behind what it issued and works when it is made again."""
+    lib = fake_runtime.load(so)
+
+    def attempts(call, again=None):
+        nth = 0
+        while True:
+            nth += 1
+            lib.fake_reset()
+            lib.fake_fail_alloc(nth)
+            st = call()
+            if lib.fake_alloc_left() > 0:
+                assert st == 0, (nth, st, lib.qe_last_error())
+                lib.fake_reset()
+                return nth
+            # (a step that finds no memory for one issue plan may still run by another)
+            assert st == BAD_ARG and b"out of host memory" in lib.qe_last_error() or (st == 0 and again), (st, lib.qe_last_error())
+            order = fake_runtime.Order(lib.fake_log().decode())
+            assert all(order.seen_by(fake_runtime.CALLER, x) for x in order.of("launch"))
+            if again:
+                again()
+
+    import ctypes as C
+
+    from paper_2609_23536_b200 import binding as qe
+
+    for mode in (0, 1):
+        s = fake_runtime.Stage(lib, [(256, 256)] * 3, T=384, slots=4, mode=mode)
+        for name, call in _calls(s, lib):
+            assert attempts(call) > 1, name
+        view, window = qe.qe_state_view(), (C.c_float * 16)()
+        attempts(lambda: lib.qe_get_state(s.layers[0], C.byref(view), window, None))
+        out = (C.c_char * 65536)()
+        attempts(lambda: lib.qe_read_fp8(s.layers[0], 5, 0, out, 65536))
+        s.close()
+        s = fake_runtime.Stage(lib, [(256, 256)] * 12, M=4, slots=4, mode=mode)
+        rebuild = lambda: [lib.qe_arena_rebuild(h) for h in s.layers]  # noqa: E731
+        assert attempts(lambda: s.step(_actions(4, 12)), rebuild) > 100
+        s.close()
+    h, c, reg = C.c_void_p(), C.c_void_p(), C.c_void_p()
+    attempts(lambda: lib.qe_registry_create(C.byref(reg)))
+    attempts(lambda: lib.qe_contract_create(4, 0, 0, 0, reg, C.byref(c)))
+    print("all attempts made")
+
+
+def test_no_allocation_that_fails_ends_the_process(lib):
+    import os
+    import subprocess
+    import sys
+
+    here = os.path.dirname(os.path.abspath(__file__))
+    code = "import sys; sys.path[:0] = sys.argv[2:]; import test_host_paths_cpu as t; t.out_of_memory(sys.argv[1])"
+    r = subprocess.run([sys.executable, "-c", code, lib._name, here, os.path.dirname(here)], capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0 and "all attempts made" in r.stdout, r.stderr[-2000:]
