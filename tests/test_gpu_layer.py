@@ -728,3 +728,32 @@ def test_arena_variant_contract_errors(qe):
     torch.cuda.synchronize()
     L.optimizer_boundary(M)
     assert L.state()["e_W"] == 1
+
+
+@pytest.mark.parametrize("H", [1, 2, 3, 4, 7, 33, 127, 128, 130, 1024, 4095, 4096])
+def test_commits_that_scan_the_ring_find_its_maximum(qe, H):
+    """The GEMM launches' own commits when the entry that leaves is the ring's maximum and the new one is smaller, at every
+    remainder of the scan's loads; the scale is the closed form of the window."""
+    T, M = 256, 3
+    ctx, L = _mk_layer(qe, 1, T, 256, 256, H, 0, 1)
+    g = torch.Generator().manual_seed(H)
+    L.weight.copy_(torch.eye(256))
+    pushed = 8.0 + (H - torch.arange(H)).float() / 512.0  # falling, all above the inputs: the oldest is the largest
+    for cls in (qe.CLASS_X, qe.CLASS_G, qe.CLASS_Y):
+        for v in pushed.to(DEV):
+            L.scale_commit(cls, v.reshape(1))
+    x = torch.randn((T, 256), generator=g).to(torch.bfloat16).to(DEV)
+    y, dx = torch.empty_like(x), torch.empty_like(x)
+    grad = torch.zeros(256 * 256, device=DEV)
+    for m in range(M):
+        t = L.forward(m, 0, x, y)
+        L.backward_dI(t, x, dx)
+        L.backward_dW(t, grad, 0)
+        st = L.state()["classes"]
+        for c, top in (("X", 448.0), ("G", 57344.0), ("Y", 448.0)):
+            window = np.asarray(st[c]["window"])
+            want = [float(v) for v in pushed[m + 1:].flip(0)]  # what is left of the pushed entries, newest first
+            assert list(window[m + 1:]) == want[:max(0, H - m - 1)] and st[c]["count"] == H + m + 1
+            assert np.float32(st[c]["scale"]) == np.float32(top) / np.float32(window.max())
+        amax = float(x.float().abs().max())
+        assert st["X"]["window"][0] == amax and st["G"]["window"][0] == amax and 0 < st["Y"]["window"][0] < 8
