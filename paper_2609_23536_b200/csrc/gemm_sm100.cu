@@ -19,7 +19,9 @@
 //   problem and each role looks its tile's problem up, so that one set of persistent CTAs packs them all.
 //   A problem may be the sum of several products (the deferred weight gradients of several microbatches): each gets an
 //   accumulator of its own, and the epilogue adds them up in registers before the one store.
-// Rows beyond M (M is a multiple of 128; a tile has 256) are read as zeros by TMA and never stored.
+//   A launch of one GEMM with an odd number of 128-row tiles may run without clusters, a CTA to a tile of 128 x 256
+//   (gemm_fp8_kernel: the same roles, four stages of 128 rows of A and 256 of B, tcgen05.mma.cta_group::1; see one_cta).
+// Rows beyond M (M is a multiple of 128; a pair's tile has 256) are read as zeros by TMA and never stored.
 // Scale commits (fold a pending amax into its history, update the scale) ride along, so that no extra launch is needed:
 // classes whose amax an earlier kernel completed (X of a forward, G of an input gradient) are committed by an idle
 // epilogue warp while the first tile is being computed; only the class the epilogue itself reduces (Y) waits for the
@@ -30,7 +32,7 @@
 // No TMA multicast is used.
 // Each output element is produced by exactly one thread with a fixed contraction order and reaches its destination
 // by exactly one store or one addition per launch, so results do not depend on the grid size or on how tiles are
-// scheduled, nor on how wide they are (no split-K; launches that add to the same destination are ordered by their stream).
+// scheduled, nor on how wide they are or how many CTAs compute one (no split-K; launches that add to the same destination are ordered by their stream).
 //
 // Every wait on an mbarrier is bounded by a clock budget; on expiry the thread ORs an error bit into the status
 // word, raises a CTA-wide abort flag that all other waits observe, and the CTA falls through to its common exit
@@ -49,12 +51,21 @@ namespace qe {
 namespace {
 
 constexpr uint32_t BM = 128, BK = 128;  // rows per CTA; bytes (= FP8 elements) per stage along the contraction
-constexpr uint32_t TILE_M = 2 * BM;     // rows of D per tile (per CTA pair)
 constexpr uint32_t ACC_COLS = 256;      // tensor-memory columns between the two accumulators (the widest tile)
 constexpr int UMMA_K = 32;
 constexpr uint32_t A_BYTES = BM * BK;
-constexpr uint32_t STAGE_BYTES = 2 * A_BYTES;  // A and at most as many rows of B (nine stages of 20 KB measured no
-constexpr int STAGES = 6;                      // faster at 64 columns: the ring's latency is covered)
+// CTAs that work on one tile, and what follows from it.
+template <bool PAIR>
+struct Form {
+  static constexpr uint32_t CTAS = PAIR ? 2 : 1;
+  static constexpr uint32_t TILE_M = CTAS * BM;  // rows of D per tile
+  // A and this CTA's rows of B: at most 128 in a pair, 256 alone.  (Nine stages of 20 KB measured no faster than six at 64
+  // columns: the ring's latency is covered.)
+  static constexpr uint32_t STAGE_BYTES = PAIR ? 2 * A_BYTES : 3 * A_BYTES;
+  static constexpr int STAGES = PAIR ? 6 : 4;
+};
+constexpr uint32_t RING_BYTES = 12 * A_BYTES;
+static_assert(Form<true>::STAGES * Form<true>::STAGE_BYTES == RING_BYTES && Form<false>::STAGES * Form<false>::STAGE_BYTES == RING_BYTES, "");
 constexpr uint32_t TMEM_COLS = 512;
 constexpr uint32_t EPI_BUF_BYTES = 4096;                     // per epilogue warp: one FP32 or two bf16 32 x 32 output tiles
                                                              // (1 KB-aligned, swizzled) that the bulk-store unit reads
@@ -64,7 +75,7 @@ constexpr int EPI_WARPS = 8, EPI_THREADS = EPI_WARPS * 32;
 // registers that the first warpgroup hands back (launched with 168 a thread; 40 + 2 * 224 <= 3 * 168).
 constexpr int threads_of(bool sums) { return sums ? 384 : 320; }
 static_assert(EPI_WARPS == 8, "shared-memory budget below assumes 8 epilogue warps");
-constexpr uint32_t SMEM_BYTES = STAGES * STAGE_BYTES + 1024 /*alignment slack*/ + 256 /*barriers, flags*/ + 8 * EPI_BUF_BYTES;
+constexpr uint32_t SMEM_BYTES = RING_BYTES + 1024 /*alignment slack*/ + 256 /*barriers, flags*/ + 8 * EPI_BUF_BYTES;
 constexpr long long WAIT_BUDGET_CYCLES = 4000000000ll;  // ~2 s at the maximum SM clock
 
 constexpr uint32_t ERR_PRODUCER = 1u, ERR_MMA = 2u, ERR_EPILOGUE = 4u;
@@ -113,6 +124,9 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_bar) {
   asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_bar) : "memory");
 }
+__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
+}
 // Address of the same shared-memory location in CTA `rank` of the cluster (shared::cluster window).
 __device__ __forceinline__ uint32_t map_to_cta(uint32_t saddr, uint32_t rank) {
   uint32_t r;
@@ -135,6 +149,17 @@ __device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap
       ::"r"(dst), "l"(map), "r"(bar), "r"(c0), "r"(c1)
       : "memory");
 }
+__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, uint32_t bar, int c0, int c1) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.shared::cta.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
+      ::"r"(dst), "l"(map), "r"(bar), "r"(c0), "r"(c1)
+      : "memory");
+}
+template <bool PAIR>
+__device__ __forceinline__ void tma_load(uint32_t dst, const CUtensorMap* map, uint32_t bar, int c0, int c1) {
+  if (PAIR) tma_load_2d_pair(dst, map, bar, c0, c1);
+  else tma_load_2d(dst, map, bar, c0, c1);
+}
 __device__ __forceinline__ void tc_commit_pair(uint32_t bar) {  // arrives on `bar` in both CTAs of the pair
   asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
                ::"r"(bar), "h"((uint16_t)3)
@@ -148,6 +173,29 @@ __device__ __forceinline__ void tc_mma_f8_pair(uint32_t d_tmem, uint64_t adesc, 
       "tcgen05.mma.cta_group::2.kind::f8f6f4 [%0], %1, %2, %3, p;\n\t}"
       ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
       : "memory");
+}
+
+__device__ __forceinline__ void tc_commit_one(uint32_t bar) {
+  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void tc_mma_f8_one(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+                                              uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %1, %2, %3, p;\n\t}"
+      ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+      : "memory");
+}
+template <bool PAIR>
+__device__ __forceinline__ void tc_commit(uint32_t bar) {
+  if (PAIR) tc_commit_pair(bar);
+  else tc_commit_one(bar);
+}
+template <bool PAIR>
+__device__ __forceinline__ void tc_mma_f8(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
+  if (PAIR) tc_mma_f8_pair(d_tmem, adesc, bdesc, idesc, accumulate);
+  else tc_mma_f8_one(d_tmem, adesc, bdesc, idesc, accumulate);
 }
 
 __device__ __forceinline__ void tma_prefetch_2d(const CUtensorMap* map, int c0, int c1) {
@@ -177,11 +225,11 @@ __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.a
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
-// Shared-memory matrix descriptor: start address (>>4) in bits 0-13; leading byte offset (unused: one swizzle atom in
-// that direction) 1 in bits 16-29; the high word (stride byte offset >>4 in bits 32-45, descriptor version 1 in bits
+// Shared-memory matrix descriptor: start address (>>4) in bits 0-13; leading byte offset (>>4) in bits 16-29: from one swizzle
+// atom of an MN-major tile's rows to the next, 1 (unused) where there is only one; the high word (stride byte offset >>4 in bits 32-45, descriptor version 1 in bits
 // 46-47, swizzle mode in bits 61-63) comes from the host: desc_hi() below.
-__device__ __forceinline__ uint64_t make_desc(uint32_t saddr, uint32_t hi) {
-  return (uint64_t)((saddr & 0x3ffffu) >> 4) | (1ull << 16) | ((uint64_t)hi << 32);
+__device__ __forceinline__ uint64_t make_desc(uint32_t saddr, uint32_t hi, uint32_t leading = 1u) {
+  return (uint64_t)((saddr & 0x3ffffu) >> 4) | ((uint64_t)leading << 16) | ((uint64_t)hi << 32);
 }
 
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
@@ -218,6 +266,7 @@ __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
 // Tile order.  The CTAs running at the same time take consecutive tiles.  Walking the dimension of the SMALLER
 // operand fastest means that operand is swept again and again (from L2, where it fits) while the larger one is
 // streamed from HBM once.
+template <uint32_t TILE_M>
 __device__ __forceinline__ void tile_coords(uint32_t tile, uint32_t tiles_m, uint32_t tiles_n, bool m_fastest,
                                             uint32_t tile_n, uint32_t& m0, uint32_t& n0) {
   if (m_fastest) {
@@ -288,8 +337,10 @@ __device__ __forceinline__ void ld_row32(const float* src, float* v) {
 }
 
 // ------------------------------------------------------------------------------------------------ kernel
-template <class PS>
+template <bool PAIR, class PS>
 __device__ __forceinline__ void gemm_body(const PS& ps) {
+  constexpr uint32_t CTAS = Form<PAIR>::CTAS, TILE_M = Form<PAIR>::TILE_M, STAGE_BYTES = Form<PAIR>::STAGE_BYTES;
+  constexpr int STAGES = Form<PAIR>::STAGES;
   constexpr bool SUMS = PS::SUMS;
   constexpr int EPI_WARP0 = SUMS ? 4 : 2;  // first epilogue warp
   extern __shared__ uint8_t smem_raw[];
@@ -307,9 +358,9 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
   uint32_t* last_flag = tmem_slot + 2;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const uint32_t rank = cluster_ctarank();  // position in the CTA pair; rank 0 issues the MMAs
+  const uint32_t rank = PAIR ? cluster_ctarank() : 0u;  // position in the CTA pair; rank 0 issues the MMAs
   const uint32_t num_tiles = ps.total_tiles();
-  const uint32_t first_tile = blockIdx.x / 2u, tile_step = gridDim.x / 2u;
+  const uint32_t first_tile = blockIdx.x / CTAS, tile_step = gridDim.x / CTAS;
   uint32_t* const status = ps.first().status;
 // per tile: which problem it belongs to (`p`), its index inside that problem and the problem's tiling
 #define QE_TILE_PROBLEM()                                                                                     \
@@ -332,22 +383,28 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
     }
     for (int a = 0; a < 2; ++a) {
       mbar_init(tfull_bar(a), 1);
-      mbar_init(tempty_bar(a), EPI_WARPS * 2);  // the epilogue warps of both CTAs of the pair
+      mbar_init(tempty_bar(a), EPI_WARPS * CTAS);  // the epilogue warps of every CTA of the tile
     }
     *abort_flag = 0u;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
   if (warp == 1) {
-    // same warp in both CTAs of the pair
-    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
-                 "r"(TMEM_COLS)
-                 : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    if (PAIR) {  // same warp in both CTAs of the pair
+      asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
+                   "r"(TMEM_COLS)
+                   : "memory");
+      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    } else {
+      asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
+                   "r"(TMEM_COLS)
+                   : "memory");
+      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
   }
   tc_fence_before();
   __syncthreads();
-  cluster_sync_all();  // the peer's barriers are initialised before anything signals them
+  if (PAIR) cluster_sync_all();  // the peer's barriers are initialised before anything signals them
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
   if (warp == 0 && lane == 0 && first_tile < num_tiles) {
@@ -356,13 +413,15 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
     const uint32_t tile = first_tile;
     QE_TILE_PROBLEM();
     uint32_t m0, n0;
-    tile_coords(local_tile, tiles_m, tiles_n, m_fastest, tile_n, m0, n0);
+    tile_coords<TILE_M>(local_tile, tiles_m, tiles_n, m_fastest, tile_n, m0, n0);
     const int rb = (int)(n0 + rank * (tile_n / 2));
     const CUtensorMap* tmB = &ps.operands(p, 0).tmB;
     for (uint32_t kb = 0; kb < num_kb && kb < (uint32_t)STAGES; ++kb) {
       const int ka = (int)(kb * BK);
-      if (p.b_mn) tma_prefetch_2d(tmB, rb, ka);
-      else tma_prefetch_2d(tmB, ka, rb);
+      for (int b = 0; b < (PAIR ? 1 : 2); ++b) {
+        if (p.b_mn) tma_prefetch_2d(tmB, rb + b * (int)BM, ka);
+        else tma_prefetch_2d(tmB, ka, rb + b * (int)BM);
+      }
     }
   }
   // Everything above (barriers, tensor memory) touched no data a predecessor produces and may overlap the previous
@@ -373,7 +432,7 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
     const GemmParams& q = ps.first();
     if (q.epi == 3 && q.sinv_dst) *q.sinv_dst = *q.sinv_src;
   }
-  if (warp == EPI_WARP0 + 7 && blockIdx.x < ps.count()) {  // (every launch has at least two CTAs per problem)
+  if (warp == EPI_WARP0 + 7 && blockIdx.x < ps.count()) {  // (every launch has at least one CTA per problem)
     // The classes whose amax an EARLIER kernel reduced (the cast that made this GEMM's A operand) are committed here,
     // by an epilogue warp that has nothing to drain yet: nothing this launch computes reads their scale (its alphas
     // are snapshots), so only the output's class is left for the launch's tail.
@@ -399,7 +458,7 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
       for (uint32_t wave = 0, tile = first_tile; ok && tile < num_tiles; ++wave, tile = snake_tile(wave, first_tile, tile_step)) {
         QE_TILE_PROBLEM();
         uint32_t m0, n0;
-        tile_coords(local_tile, tiles_m, tiles_n, m_fastest, tile_n, m0, n0);
+        tile_coords<TILE_M>(local_tile, tiles_m, tiles_n, m_fastest, tile_n, m0, n0);
         const int ra = (int)(m0 + rank * BM), rb = (int)(n0 + rank * (tile_n / 2));
         for (uint32_t seg = 0; ok && seg < (SUMS ? p.nseg : 1u); ++seg) {
           const GemmOperands& op = ps.operands(p, seg);
@@ -407,16 +466,20 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
           for (uint32_t kb = 0; kb < num_kb; ++kb) {
             if (!(ok = mbar_wait(empty_bar(s), ph ^ 1u, abort_flag, status, ERR_PRODUCER))) break;
             const uint32_t a_dst = smem_base + s * STAGE_BYTES, b_dst = a_dst + A_BYTES;
-            // both CTAs credit the even CTA's barrier, which expects the bytes of the whole pair
-            if (rank == 0) mbar_expect_tx(full_bar(s), 2 * A_BYTES + tile_n * BK);
-            const uint32_t bar = map_to_cta(full_bar(s), 0);
+            // both CTAs of a pair credit the even CTA's barrier, which expects the bytes of the whole pair
+            if (rank == 0) mbar_expect_tx(full_bar(s), CTAS * A_BYTES + tile_n * BK);
+            const uint32_t bar = PAIR ? map_to_cta(full_bar(s), 0) : full_bar(s);
             // contraction-major operand: box = 128 K-bytes x rows at (k, row); MN-major operand (stored as [Kc, rows]):
             // box = row-bytes x 128 K-rows at (row, k).  Either way 128 bytes per row land in shared memory.
             const int ka = (int)(kb * BK);
-            if (p.a_mn) tma_load_2d_pair(a_dst, tmA, bar, ra, ka);
-            else tma_load_2d_pair(a_dst, tmA, bar, ka, ra);
-            if (p.b_mn) tma_load_2d_pair(b_dst, tmB, bar, rb, ka);
-            else tma_load_2d_pair(b_dst, tmB, bar, ka, rb);
+            if (p.a_mn) tma_load<PAIR>(a_dst, tmA, bar, ra, ka);
+            else tma_load<PAIR>(a_dst, tmA, bar, ka, ra);
+            // (a CTA on its own loads the tile's 256 rows of B as two boxes of 128, one behind the other)
+#pragma unroll
+            for (int b = 0; b < (PAIR ? 1 : 2); ++b) {
+              if (p.b_mn) tma_load<PAIR>(b_dst + b * A_BYTES, tmB, bar, rb + b * (int)BM, ka);
+              else tma_load<PAIR>(b_dst + b * A_BYTES, tmB, bar, ka, rb + b * (int)BM);
+            }
             if (++s == STAGES) { s = 0; ph ^= 1u; }
           }
         }
@@ -445,17 +508,18 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
             if (!(ok = mbar_wait(full_bar(s), ph, abort_flag, status, ERR_MMA))) break;
             tc_fence_after();
             const uint32_t a_src = smem_base + s * STAGE_BYTES, b_src = a_src + A_BYTES;
-            const uint64_t adesc = make_desc(a_src, A_DESC_HI), bdesc = make_desc(b_src, b_hi);
+            const uint64_t adesc = make_desc(a_src, A_DESC_HI);
+            const uint64_t bdesc = make_desc(b_src, b_hi, PAIR || !p.b_mn ? 1u : A_BYTES / 16u);
 #pragma unroll
             for (int k = 0; k < (int)BK / UMMA_K; ++k)
               // advancing 32 along the contraction: 32 bytes inside the 128-byte swizzle row for a contraction-major
               // tile (+2 in the address field), 32 rows for an MN-major one (+256 with rows of 128 bytes)
-              tc_mma_f8_pair(d_tmem, adesc + a_step * k, bdesc + b_step * k, idesc, (kb | (uint32_t)k) != 0u);
-            tc_commit_pair(empty_bar(s));  // stage reusable (in both CTAs) once these MMAs have read it
+              tc_mma_f8<PAIR>(d_tmem, adesc + a_step * k, bdesc + b_step * k, idesc, (kb | (uint32_t)k) != 0u);
+            tc_commit<PAIR>(empty_bar(s));  // stage reusable (in both CTAs) once these MMAs have read it
             if (++s == STAGES) { s = 0; ph ^= 1u; }
           }
           if (!ok) break;
-          tc_commit_pair(tfull_bar(acc));  // accumulator complete (each CTA holds its 128 rows)
+          tc_commit<PAIR>(tfull_bar(acc));  // accumulator complete (each CTA holds its 128 rows)
           if (++acc == 2) { acc = 0; acc_ph ^= 1u; }
         }
       }
@@ -470,12 +534,13 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
     uint32_t n_groups = 0;  // bulk-store groups this warp has committed (buffer parity)
     uint32_t acc = 0, acc_ph = 0;
     bool ok = true;
-    const uint32_t tempty_leader0 = map_to_cta(tempty_bar(0), 0), tempty_leader1 = map_to_cta(tempty_bar(1), 0);
+    const uint32_t tempty_leader0 = PAIR ? map_to_cta(tempty_bar(0), 0) : tempty_bar(0);
+    const uint32_t tempty_leader1 = PAIR ? map_to_cta(tempty_bar(1), 0) : tempty_bar(1);
     for (uint32_t wave = 0, tile = first_tile; ok && tile < num_tiles; ++wave, tile = snake_tile(wave, first_tile, tile_step)) {
       QE_TILE_PROBLEM();
       (void)num_kb;
       uint32_t m0, n0;
-      tile_coords(local_tile, tiles_m, tiles_n, m_fastest, tile_n, m0, n0);
+      tile_coords<TILE_M>(local_tile, tiles_m, tiles_n, m_fastest, tile_n, m0, n0);
       const uint32_t blk_row0 = m0 + rank * BM + quad * 32u;
       const uint32_t col0 = n0 + half * (tile_n / 2);
       // 32 x 32 blocks of this warp: none in rows beyond M, fewer in a ragged last column tile; warp-uniform
@@ -487,7 +552,7 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
         (void)num_kb;
         if (p.nseg == 1 || p.epi != 2) return;
         uint32_t m0, n0;
-        tile_coords(local_tile, tiles_m, tiles_n, m_fastest, tile_n, m0, n0);
+        tile_coords<TILE_M>(local_tile, tiles_m, tiles_n, m_fastest, tile_n, m0, n0);
         const uint32_t row = m0 + rank * BM + quad * 32u + (uint32_t)lane, col = n0 + half * (tile_n / 2);
         if (row >= p.M || col >= p.N) return;
         const char* d = reinterpret_cast<const char*>(reinterpret_cast<const float*>(p.out) + (size_t)row * p.ldo + col);
@@ -662,7 +727,10 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
       // accumulator drained: hand it back to the MMA warp
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive_cluster(acc ? tempty_leader1 : tempty_leader0);  // the MMA issuer waits in the even CTA
+      if (lane == 0) {  // the MMA issuer of a pair waits in the even CTA
+        if (PAIR) mbar_arrive_cluster(acc ? tempty_leader1 : tempty_leader0);
+        else mbar_arrive(acc ? tempty_leader1 : tempty_leader0);
+      }
       if ((p.epi == 0 || p.epi == 3) && (p.amax_bits || p.amax_bits2)) {
         // two packed bf16 magnitudes -> FP32 bit pattern of the larger
         const uint32_t w = __reduce_max_sync(0xffffffffu, max(amax_bits & 0xffffu, amax_bits >> 16) << 16);
@@ -701,10 +769,11 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
     for (uint32_t i = 1; i < ps.count(); ++i)
       if (ps.status_of(i) && ps.status_of(i) != status) atomicOr(ps.status_of(i), bits);
   }
-  cluster_sync_all();  // no arrival may still be on its way to a CTA that has left
+  if (PAIR) cluster_sync_all();  // no arrival may still be on its way to a CTA that has left
   if (warp == 1) {
     tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TMEM_COLS) : "memory");
+    if (PAIR) asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TMEM_COLS) : "memory");
+    else asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TMEM_COLS) : "memory");
   }
 }
 
@@ -716,22 +785,29 @@ using WideParams = GemmLaunchParams<kMaxProblems, kMaxOperands>;
 
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(threads_of(false), 1)
     gemm_fp8_pair_kernel(const __grid_constant__ OneParams p) {
-  gemm_body(Problems<1, 1>{p});
+  gemm_body<true>(Problems<1, 1>{p});
+}
+
+// One GEMM with an odd number of 128-row tiles, a CTA to a tile.
+__global__ void __launch_bounds__(threads_of(false), 1) gemm_fp8_kernel(const __grid_constant__ OneParams p) {
+  gemm_body<false>(Problems<1, 1>{p});
 }
 
 // Up to eight independent GEMMs in one launch.
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(threads_of(false), 1)
     gemm_fp8_pair_group_kernel(const __grid_constant__ GroupParams g) {
-  gemm_body(Problems<8, 8>{g});
+  gemm_body<true>(Problems<8, 8>{g});
 }
 
 // More problems, or problems of several products each.  (The parameter block is three times as large.)
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(threads_of(true), 1)
     gemm_fp8_pair_wide_kernel(const __grid_constant__ WideParams g) {
-  gemm_body(Problems<kMaxProblems, kMaxOperands>{g});
+  gemm_body<true>(Problems<kMaxProblems, kMaxOperands>{g});
 }
 
-uint32_t tiles_of(const GemmDesc& d, uint32_t tile_n) { return ((d.M + TILE_M - 1) / TILE_M) * ((d.N + tile_n - 1) / tile_n); }
+constexpr uint32_t PAIR_M = Form<true>::TILE_M;
+uint32_t ceil_div(uint32_t a, uint32_t b) { return (a + b - 1) / b; }
+uint32_t tiles_of(const GemmDesc& d, uint32_t tile_n) { return ceil_div(d.M, PAIR_M) * ceil_div(d.N, tile_n); }
 
 // Columns per tile of a launch's problems (index into kTileWidths).  A tile's main loop takes 0.27 us per 128-byte K
 // block at ANY width (four dependent MMAs of ~128 clocks each), so width is free only as long as every CTA pair has a
@@ -751,16 +827,36 @@ uint32_t choose_width(const GemmDesc* d, uint32_t n, uint32_t pairs) {
   return w;
 }
 
+// Whether a GEMM goes out with a CTA to a 128 x 256 tile instead of a pair to a 256-row one.  With an odd number of 128-row
+// tiles the pairs' last row tile is half empty, and the launch may need a wave more; a CTA on its own loads half as much
+// again per K block, so that its waves take up to a fifth longer (M x N x contraction, one CTA to a tile against pairs):
+//   1 wave for 2    1152 x 4096 x 4096 15.0 us for 24.7, 384 x 11008 x 4096 14.6 for 24.6, 3712 x 1280 x 1024 8.2 for 11.5
+//   2 for 3         640 x 12800 x 4096 29.1 for 34.7, 3712 x 2560 x 1024 12.2 for 13.5
+//   3 for 4         3968 x 3584 x 4096 43.5 for 47.6;  4 for 5: 1152 x 15360 x 4096 61.9 for 62.8
+//   5 for 6         3712 x 6400 x 4096 74.6 for 74.5;  7 for 8: 3968 x 8448 x 4096 104.7 for 101.5;  4 for 4: 64.8 for 60.8
+// With one wave either way the CTAs, which wait for no peer, start and finish 1 us earlier (384 x 9472 x 4096 14.5 for 15.3),
+// which the loads of a long contraction eat up (1920 x 2176, cast included: 23.7 for 25.3 at 4096, 31.6 for 32.3 at 6528,
+// 39.2 for 38.8 at 8192); at 128 rows the pair's empty half still shares the loads of B (128 x 16384 x 4096, FP32: 17.6
+// for 16.9).  Even row counts have no empty half.
+bool one_cta(const GemmDesc& d, int num_sms) {
+  const uint32_t pairs = (uint32_t)num_sms / 2u;
+  if (d.M % PAIR_M == 0 || choose_width(&d, 1, pairs) != 0) return false;
+  const uint32_t waves_pairs = ceil_div(tiles_of(d, 256), pairs);
+  const uint32_t waves_ctas = ceil_div((d.M / BM) * ceil_div(d.N, 256), (uint32_t)num_sms);
+  return 6 * waves_ctas < 5 * waves_pairs || (waves_pairs == 1 && d.M > BM && d.Kc <= 6144);
+}
+
 // The device's parameter block of one problem at a tile width; its operand pairs start at op0.
-GemmParams problem_of(const GemmDesc& d, uint32_t w, uint32_t op0) {
+GemmParams problem_of(const GemmDesc& d, uint32_t w, uint32_t op0, uint32_t tile_m) {
   GemmParams p = d;
   const uint32_t tile_n = kTileWidths[w], per_cta = tile_n / 2;
   p.op0 = op0;
   p.tile_n = tile_n;
   // bits 4-5: accumulator format (1 = FP32); 7-9 / 10-12: A / B format (0 = E4M3, 1 = E5M2); 15 / 16: A / B major
-  // (0 = contraction-major); 17-22: N >> 3; 24-28: M >> 4 (256 for a CTA pair).
-  p.idesc = (1u << 4) | (d.a_fmt << 7) | (d.b_fmt << 10) | (d.a_mn << 15) | (d.b_mn << 16) | ((tile_n >> 3) << 17) | ((TILE_M >> 4) << 24);
-  // An MN-major B tile has rows of per_cta bytes, swizzled over exactly that width; a contraction-major one rows of 128.
+  // (0 = contraction-major); 17-22: N >> 3; 24-28: M >> 4 (of the whole tile).
+  p.idesc = (1u << 4) | (d.a_fmt << 7) | (d.b_fmt << 10) | (d.a_mn << 15) | (d.b_mn << 16) | ((tile_n >> 3) << 17) | ((tile_m >> 4) << 24);
+  // An MN-major B tile has rows of per_cta bytes (a CTA alone: two boxes of 128), swizzled over exactly that width; a
+  // contraction-major one rows of 128.
   const uint32_t row = d.b_mn ? per_cta : 128u;
   p.b_desc_hi = desc_hi(row);
   p.b_step = d.b_mn ? 32u * row / 16u : 2u;
@@ -768,7 +864,7 @@ GemmParams problem_of(const GemmDesc& d, uint32_t w, uint32_t op0) {
 }
 
 template <int NP, int NOPS>
-Launch make_launch(const GemmDesc* probs, uint32_t n, uint32_t nops, int num_sms, const void* func) {
+Launch make_launch(const GemmDesc* probs, uint32_t n, uint32_t nops, int num_sms, const void* func, bool alone = false) {
   using P = GemmLaunchParams<NP, NOPS>;
   static_assert(sizeof(P) <= sizeof(Launch::Block), "parameter block too large");
   static_assert(NP > 1 || sizeof(P) <= ParamBytes::kInline, "a launch of one problem takes no heap memory");
@@ -776,12 +872,13 @@ Launch make_launch(const GemmDesc* probs, uint32_t n, uint32_t nops, int num_sms
   l.nbytes = sizeof(P);
   l.params.resize(offsetof(P, op) + nops * sizeof(GemmOperands));  // (a step has hundreds of launches: no unused operands)
   unsigned char* at = l.params.data();
-  const uint32_t pairs = (uint32_t)num_sms / 2u, w = choose_width(probs, n, pairs);
+  const uint32_t tile_m = alone ? BM : PAIR_M, ctas = alone ? 1u : 2u, most = (uint32_t)num_sms / ctas;
+  const uint32_t w = alone ? 0u : choose_width(probs, n, most);
   uint32_t tiles = 0, op = 0;
   for (uint32_t i = 0; i < n; ++i) {
-    tiles += tiles_of(probs[i], kTileWidths[w]);
+    tiles += ceil_div(probs[i].M, tile_m) * ceil_div(probs[i].N, kTileWidths[w]);
     std::memcpy(at + offsetof(P, tile_end) + i * sizeof(uint32_t), &tiles, sizeof(tiles));
-    const GemmParams p = problem_of(probs[i], w, op);
+    const GemmParams p = problem_of(probs[i], w, op, tile_m);
     std::memcpy(at + offsetof(P, prob) + i * sizeof(GemmParams), &p, sizeof(p));
     for (uint32_t j = 0; j < probs[i].nseg; ++j, ++op) {
       const GemmDesc::Operands& d = probs[i].ops[j];
@@ -791,14 +888,17 @@ Launch make_launch(const GemmDesc* probs, uint32_t n, uint32_t nops, int num_sms
   }
   std::memcpy(at + offsetof(P, n), &n, sizeof(n));
   l.func = func;
-  l.grid = dim3(2u * (tiles < pairs ? tiles : pairs), 1, 1);
+  l.grid = dim3(ctas * (tiles < most ? tiles : most), 1, 1);
   l.block = dim3(threads_of(NOPS > NP), 1, 1);
   l.smem = SMEM_BYTES;
   return l;
 }
 
 Launch make_any(const GemmDesc* probs, uint32_t n, uint32_t nops, int num_sms) {
-  if (n == 1 && nops == 1) return make_launch<1, 1>(probs, n, nops, num_sms, (const void*)gemm_fp8_pair_kernel);
+  if (n == 1 && nops == 1) {
+    const bool alone = one_cta(*probs, num_sms);
+    return make_launch<1, 1>(probs, n, nops, num_sms, alone ? (const void*)gemm_fp8_kernel : (const void*)gemm_fp8_pair_kernel, alone);
+  }
   if (n <= 8 && nops == n) return make_launch<8, 8>(probs, n, nops, num_sms, (const void*)gemm_fp8_pair_group_kernel);
   return make_launch<kMaxProblems, kMaxOperands>(probs, n, nops, num_sms, (const void*)gemm_fp8_pair_wide_kernel);
 }
@@ -808,7 +908,7 @@ Launch make_any(const GemmDesc* probs, uint32_t n, uint32_t nops, int num_sms) {
 bool gemm_uses_pair(uint32_t M) { return M % 256 == 0; }
 
 cudaError_t gemm_prepare() {
-  for (const void* f : {(const void*)gemm_fp8_pair_kernel, (const void*)gemm_fp8_pair_group_kernel, (const void*)gemm_fp8_pair_wide_kernel}) {
+  for (const void* f : {(const void*)gemm_fp8_kernel, (const void*)gemm_fp8_pair_kernel, (const void*)gemm_fp8_pair_group_kernel, (const void*)gemm_fp8_pair_wide_kernel}) {
     const cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES);
     if (e != cudaSuccess) return e;
   }

@@ -1,5 +1,7 @@
 """FP8 hand-off between directly chained linears (qe_forward_chain / qe_backward_dI_chain): bit for bit the result of
 running the layers one by one through bf16 tensors, and within tolerance of the oracle's composition."""
+import sys
+
 import numpy as np
 import pytest
 import torch
@@ -104,6 +106,23 @@ def test_chained_equals_layer_by_layer_bitwise(qe, mode, overlap):
     # two cast kernels per microbatch and direction are gone
     steps, M, n = 2, 3, len(CHAIN)
     assert a["stats"]["kernels_launched"] - b["stats"]["kernels_launched"] == steps * M * 2 * (n - 1)
+
+
+@pytest.mark.parametrize("tokens", [384, 640, 1152])
+def test_chain_of_odd_token_counts_equals_layer_by_layer_bitwise(qe, tokens, monkeypatch):
+    """The hand-off on half-filled row tiles; the wide linear's outputs go out a CTA to a tile at 1152 tokens."""
+    monkeypatch.setattr(sys.modules[__name__], "T", tokens)
+    monkeypatch.setattr(sys.modules[__name__], "CHAIN", [(256, 512), (512, 4096), (4096, 256), (256, 768)])
+    a = _run(qe, 1, chained=False)
+    b = _run(qe, 1, chained=True)
+    for key in ("Y", "dX", "mg"):
+        for u, v in zip(a[key], b[key]):
+            assert np.array_equal(u.view(np.uint8), v.view(np.uint8)), key
+    for key in ("Xq", "Gq"):
+        for u, v in zip(a[key], b[key]):
+            assert all(np.array_equal(x, y) for x, y in zip(u, v)), key
+    for u, v in zip(a["state"], b["state"]):
+        assert all(state_equal(x, y) and x["device_token"] == y["device_token"] and x["device_status"] == 0 for x, y in zip(u, v))
 
 
 def test_chain_against_the_oracle_composition(qe):

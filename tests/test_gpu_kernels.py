@@ -223,13 +223,15 @@ def test_gemm_mn_major_needs_the_paired_variant(qe):
     assert e.value.code == "UNSUPPORTED"
 
 
-# Tile widths 64, 128 and 256 (by how many tiles the shape gives), whole and half-filled last row tiles, every operand
-# major; the last shape reaches the next wider tile by one row tile.
-@pytest.mark.parametrize("M,Nn", [(128, 256), (256, 2048), (640, 768), (1024, 1152), (1024, 2048), (1152, 1920), (2048, 2048), (2304, 2176)])
-@pytest.mark.parametrize("a_mn,b_mn", [(False, False), (False, True), (True, True)])
+# Tile widths 64, 128 and 256 (by how many tiles the shape gives), whole and half-filled last row tiles, odd row counts that a
+# CTA to a tile needs fewer waves for (1152 x 8192: two for three; 384 x 11008: one for two) or as many (2176 x 2304), every
+# operand major (with an odd row count the call takes contraction-major ones only; the layer tests cover the others).
+@pytest.mark.parametrize("M,Nn,a_mn,b_mn", [
+    (M, Nn, a_mn, b_mn)
+    for M, Nn in [(128, 256), (256, 2048), (640, 768), (1024, 1152), (1024, 2048), (1152, 1920), (2048, 2048), (2304, 2176),
+                  (1152, 8192), (384, 11008), (2176, 2304), (128, 16384)]
+    for a_mn, b_mn in [(False, False), (False, True), (True, True)] if M % 256 == 0 or not b_mn])
 def test_gemm_tile_widths_and_half_filled_row_tiles_integer_exact(qe, M, Nn, a_mn, b_mn):
-    if (a_mn or b_mn) and M % 256:
-        pytest.skip("MN-major operands need whole row tiles")
     rng = np.random.default_rng(M + Nn + 2 * a_mn + b_mn)
     Kc = 384
     A, Av = _int_codes(rng, (M, Kc), 8, fp8.E5M2)
@@ -251,6 +253,26 @@ def test_gemm_tile_widths_and_half_filled_row_tiles_integer_exact(qe, M, Nn, a_m
     wb = bf16.round_from_f64(want.astype(np.float64))
     assert np.array_equal(inputs.bits(bf[:M].cpu()), wb) and bool((bf[M:] == 7.0).all())
     assert amax.item() == float(np.abs(bf16.decode(wb)).max())
+
+
+@pytest.mark.parametrize("M,Nn,Kc", [(1152, 8192, 640), (384, 11008, 384), (1152, 1920, 2176)])
+@pytest.mark.parametrize("kind", [0, 1, 2])
+def test_odd_row_counts_give_the_bits_of_even_ones(qe, M, Nn, Kc, kind):
+    """A CTA to a tile (M odd in units of 128) against a pair to a tile (the same rows and 128 more): weight gradients may
+    go out either way, alone or as sums, and are promised to be the same bits."""
+    g = torch.Generator(device=DEV).manual_seed(M + kind)
+    fp8_of = lambda shape, t: torch.randn(shape, generator=g, device=DEV).to(t).view(torch.uint8)  # noqa: E731
+    A, B = fp8_of((M + 128, Kc), torch.float8_e5m2), fp8_of((Nn, Kc), torch.float8_e4m3fn)
+    scale = [torch.tensor([v], device=DEV) for v in (0.37, 1.91)]
+    status = torch.zeros(1, dtype=torch.int32, device=DEV)
+    start = torch.randn((M + 128, Nn), generator=g, device=DEV).to(torch.float32 if kind else torch.bfloat16)
+    odd, even = start.clone(), start.clone()
+    qe.qe_gemm_fp8_ex(A[:M], 1, False, B, 0, False, *scale, odd[:M], kind, None, status)
+    qe.qe_gemm_fp8_ex(A, 1, False, B, 0, False, *scale, even, kind, None, status)
+    torch.cuda.synchronize()
+    assert status.item() == 0 and torch.equal(odd[M:], start[M:])
+    bits = torch.int32 if kind else torch.int16
+    assert torch.equal(odd[:M].view(bits), even[:M].view(bits)) and not torch.equal(odd[:M], start[:M])
 
 
 # ------------------------------------------------------------------------------------------ arena reduction

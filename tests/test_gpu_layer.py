@@ -757,3 +757,40 @@ def test_commits_that_scan_the_ring_find_its_maximum(qe, H):
             assert np.float32(st[c]["scale"]) == np.float32(top) / np.float32(window.max())
         amax = float(x.float().abs().max())
         assert st["X"]["window"][0] == amax and st["G"]["window"][0] == amax and 0 < st["Y"]["window"][0] < 8
+
+
+@pytest.mark.parametrize("T,K,N", [
+    (1152, 2176, 1920),   # F, dI and dW: a CTA to a 128 x 256 tile, one wave, a last column tile of 128
+    (1152, 8192, 1152),   # dI and dW: two waves of such tiles (three of paired ones)
+    (384, 256, 11008),    # F: one wave instead of two
+    (2176, 2304, 2176),   # as many waves either way: pairs
+])
+def test_odd_row_counts_are_exact_on_integers(qe, T, K, N):
+    """Every GEMM of a layer whose row counts are odd multiples of 128, both operand majors, overwrite and accumulate.
+    Integers up to 7 with scales that are powers of two are FP8 numbers, and their sums stay below 2^24: exact."""
+    ctx, L = _mk_layer(qe, 0, T, K, N, 4, 0, 2)
+    g = torch.Generator(device=DEV).manual_seed(T + K + N)
+
+    def ints(shape, top):
+        t = torch.randint(-top, top + 1, shape, generator=g, device=DEV).to(torch.bfloat16)
+        t.view(-1)[0] = top  # amax 7: the next scale is 448 / 7 = 64 (E4M3) or 57344 / 7 = 8192 (E5M2)
+        return t
+
+    W = ints((N, K), 4)
+    L.weight.copy_(W)
+    grad = torch.full((N * K + 8,), 3.0, device=DEV)
+    want = torch.zeros((N, K), dtype=torch.float64, device=DEV)
+    tapes = []
+    for m in range(2):
+        x, y = ints((T, K), 7), torch.full((T + 128, N), 9.0, dtype=torch.bfloat16, device=DEV)
+        dy, dx = ints((T, N), 7), torch.full((T + 128, K), 9.0, dtype=torch.bfloat16, device=DEV)
+        t = L.forward(m, 0, x, y[:T])
+        L.backward_dI(t, dy, dx[:T])
+        L.backward_dW(t, grad, 4)
+        assert torch.equal(y[:T], (x.double() @ W.double().T).float().to(torch.bfloat16)) and bool((y[T:] == 9.0).all())
+        assert torch.equal(dx[:T], (dy.double() @ W.double()).float().to(torch.bfloat16)) and bool((dx[T:] == 9.0).all())
+        want += dy.double().T @ x.double()
+        assert torch.equal(grad[4:-4].view(N, K).double(), want) and bool((grad[:4] == 3.0).all()) and bool((grad[-4:] == 3.0).all())
+        assert L.state()["classes"]["Y"]["window"][0] == float(y[:T].float().abs().max())
+    assert L.state()["device_status"] == 0
+    L.optimizer_boundary(2)

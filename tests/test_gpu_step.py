@@ -643,8 +643,9 @@ def test_run_together_host_equals_device_buffers_bitwise(qe):
 @pytest.mark.parametrize("M,w,d,slots", [(3, 3, 0, 3), (9, 1, 8, 9), (12, 2, 3, 6)])
 def test_step_call_sums_of_weight_gradients_equal_one_launch_each_bitwise(qe, mode, M, w, d, slots):
     """Sums of up to eight products, with and without a destination to add to, on whole and half-filled row tiles, ragged
-    column tiles and a gradient slice that is 16- but not 32-byte aligned."""
-    T, shapes = 384, [(256, 512), (640, 384), (1152, 2304)]
+    column tiles and a gradient slice that is 16- but not 32-byte aligned; the last linear's gradients go out a CTA to a tile
+    where they go out one by one."""
+    T, shapes = 384, [(256, 512), (640, 384), (1152, 2304), (2176, 1920)]
     s = sched(M, w, d)
     acts = _actions(s, len(shapes))
     offs, total = [], 4
