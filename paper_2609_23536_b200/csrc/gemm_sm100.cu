@@ -873,7 +873,7 @@ Launch make_launch(const GemmDesc* probs, uint32_t n, uint32_t nops, int num_sms
   l.params.resize(offsetof(P, op) + nops * sizeof(GemmOperands));  // (a step has hundreds of launches: no unused operands)
   unsigned char* at = l.params.data();
   const uint32_t tile_m = alone ? BM : PAIR_M, ctas = alone ? 1u : 2u, most = (uint32_t)num_sms / ctas;
-  const uint32_t w = alone ? 0u : choose_width(probs, n, most);
+  const uint32_t w = choose_width(probs, n, (uint32_t)num_sms / 2u);  // (alone: 0, see one_cta)
   uint32_t tiles = 0, op = 0;
   for (uint32_t i = 0; i < n; ++i) {
     tiles += ceil_div(probs[i].M, tile_m) * ceil_div(probs[i].N, kTileWidths[w]);
@@ -925,6 +925,8 @@ bool make_gemm_group(const GemmDesc* probs, uint32_t n, int num_sms, Launch* out
   *out = make_any(probs, n, nops, num_sms);
   return true;
 }
+
+uint32_t gemm_width(const GemmDesc* probs, uint32_t n, int num_sms) { return choose_width(probs, n, (uint32_t)num_sms / 2u); }
 
 Launch make_gemm(const GemmDesc& d, int num_sms) { return make_any(&d, 1, d.nseg, num_sms); }
 

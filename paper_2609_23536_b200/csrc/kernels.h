@@ -135,7 +135,7 @@ struct GemmDesc : GemmParams {
   uint32_t a_fmt, b_fmt;       // 0 = E4M3, 1 = E5M2
   struct Operands {
     const CUtensorMap* mapA;
-    const CUtensorMap* mapB;   // one map per tile width
+    const CUtensorMap* mapB;   // one map per tile width (the launch reads the one of the width it chooses: gemm_width)
     const float* alpha_a;
     const float* alpha_b;
   } ops[kMaxSegments];
@@ -233,6 +233,7 @@ Launch make_gemm(const GemmDesc& p, int num_sms);
 // false if the group cannot be formed (a problem's M is not a multiple of 256), in which case the caller launches them
 // one by one.
 bool make_gemm_group(const GemmDesc* probs, uint32_t n, int num_sms, Launch* out);
+uint32_t gemm_width(const GemmDesc* probs, uint32_t n, int num_sms);  // index of the tile width the launch of these will have
 cudaError_t gemm_prepare();  // opt in to the dynamic shared memory the GEMM needs (once per device)
 bool gemm_uses_pair(uint32_t M);  // whole 256-row tiles: may share launches and take MN-major operands
 constexpr uint32_t kAmaxPartials = 2048;

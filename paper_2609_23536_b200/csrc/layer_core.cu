@@ -45,11 +45,15 @@ int32_t make_map(const DeviceInfo* d, CUtensorMap* map, const void* ptr, uint64_
   return QE_OK;
 }
 
-// The maps of a GEMM's B operand, one per tile width: contraction-major [N, Kc], or (mn) the operand given as [Kc, N].
+// The map of a GEMM's B operand for one tile width: contraction-major [N, Kc], or (mn) the operand given as [Kc, N].
+int32_t make_b_map(const DeviceInfo* d, CUtensorMap* map, const void* ptr, uint64_t N, uint64_t Kc, bool mn, uint32_t width) {
+  const uint32_t per_cta = qe::kTileWidths[width] / 2;
+  return mn ? make_map(d, map, ptr, Kc, N, 128, per_cta) : make_map(d, map, ptr, N, Kc, per_cta);
+}
+// ... for all of them: operands that a layer keeps.
 int32_t make_b_maps(const DeviceInfo* d, CUtensorMap* maps, const void* ptr, uint64_t N, uint64_t Kc, bool mn) {
   for (uint32_t w = 0; w < qe::kNumTileWidths; ++w) {
-    const uint32_t per_cta = qe::kTileWidths[w] / 2;
-    const int32_t st = mn ? make_map(d, &maps[w], ptr, Kc, N, 128, per_cta) : make_map(d, &maps[w], ptr, N, Kc, per_cta);
+    const int32_t st = make_b_map(d, &maps[w], ptr, N, Kc, mn, w);
     if (st != QE_OK) return st;
   }
   return QE_OK;

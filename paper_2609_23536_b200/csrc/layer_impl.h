@@ -39,6 +39,7 @@ int32_t device_info(int device, DeviceInfo** out);
 int32_t current_device_info(DeviceInfo** d);
 int32_t make_map(const DeviceInfo* d, CUtensorMap* map, const void* ptr, uint64_t rows, uint64_t inner, uint32_t box_rows,
                  uint32_t box_inner = 128);
+int32_t make_b_map(const DeviceInfo* d, CUtensorMap* map, const void* ptr, uint64_t N, uint64_t Kc, bool mn, uint32_t width);
 int32_t make_b_maps(const DeviceInfo* d, CUtensorMap* maps, const void* ptr, uint64_t N, uint64_t Kc, bool mn);
 int32_t make_out_map(const DeviceInfo* d, CUtensorMap* map, const void* ptr, uint64_t M, uint64_t N, uint64_t ldo, bool fp32);
 int32_t make_out_map_u8(const DeviceInfo* d, CUtensorMap* map, const void* ptr, uint64_t M, uint64_t N, uint64_t ld);

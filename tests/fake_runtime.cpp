@@ -201,6 +201,7 @@ Launch named(const char* fmt, ...) {
 }  // namespace
 bool gemm_uses_pair(uint32_t M) { return M % 256 == 0; }
 cudaError_t gemm_prepare() { return cudaSuccess; }
+uint32_t gemm_width(const GemmDesc*, uint32_t, int) { return 1; }
 Launch make_quantize(const QuantParams&) { return named("cast 1"); }
 Launch make_quantize_multi(const QuantParams*, uint32_t n) { return named("cast %u", n); }
 Launch make_commit(const CommitParams&) { return named("commit"); }

@@ -201,3 +201,16 @@ def test_no_allocation_that_fails_ends_the_process(lib):
     code = "import sys; sys.path[:0] = sys.argv[2:]; import test_host_paths_cpu as t; t.out_of_memory(sys.argv[1])"
     r = subprocess.run([sys.executable, "-c", code, lib._name, here, os.path.dirname(here)], capture_output=True, text=True, timeout=300)
     assert r.returncode == 0 and "all attempts made" in r.stdout, r.stderr[-2000:]
+
+
+def test_standalone_gemms_encode_one_map_per_operand_and_output(lib):
+    import ctypes as C
+
+    from paper_2609_23536_b200 import binding as qe
+
+    buf = (C.c_char * (1 << 20))()
+    a = (C.addressof(buf) + 255) // 256 * 256
+    assert lib.qe_gemm_fp8_ex(a, 0, 0, a, 0, 1, 256, 256, 256, a, a, a, 0, a, a, None) == 0 and lib.fake_encodes() == 3
+    lib.fake_reset()
+    d = qe.qe_gemm_desc(a, a, a, a, a, a, 0, 0, 0, 0, 256, 256, 256, 0)
+    assert lib.qe_gemm_fp8_group((qe.qe_gemm_desc * 3)(d, d, d), 3, a, None) == 0 and lib.fake_encodes() == 9
