@@ -471,10 +471,12 @@ int32_t qe_step_run(qe_ctx* ctx, qe_layer* const* layers, uint32_t n_layers, con
   // round goes out as qe_run_together would issue it.  If no such plan exists (an illegal list) the action-by-action
   // pass below runs instead and reports the failing action.
   // Weight gradients: qe_plan_step collects a layer's and lets one launch add them up, as far as a sum stays within 8192
-  // tokens.  Few tokens make the destination's traffic the cost of a weight gradient: eight microbatches of 256 tokens
-  // through a 4096 / 11008 layer 2860 -> 1890 us a step.  With 2048 tokens a sum of four gains 2 %, of two or eight
-  // nothing; with 4096 the traffic is small, and tiles that last several times as long leave more of the chip idle at the
-  // end of a launch (a 4096 / 14336 block: 20.5 ms one by one, 21.2 ms in sums), so there they go out one by one.
+  // tokens and holds three products.  Few tokens make the destination's traffic the cost of a weight gradient: eight
+  // microbatches of 256 tokens through a 4096 / 11008 layer 2860 -> 1890 us a step.  With 2048 tokens a sum of four gains 2 %.
+  // Tiles that last several times as long leave more of the chip idle at the end of a launch, which sums of two do not make
+  // up for (blocks of eight microbatches, sums against launches one by one): hidden 2048, three products at 2176 tokens 3132 us
+  // for 3276, at 2432 3754 for 4013, at 2560 3368 for 3512; two at 3072 4178 for 4094, at 3584 4777 for 4641; hidden 4096, three
+  // at 2304 9116 for 9337, two at 2816 11150 for 11087; hidden 1024, three at 2560 1190 for 1181, two at 3584 1595 for 1561.
   uint32_t T_max = 0;
   for (uint32_t l = 0; l < n_layers; ++l) T_max = std::max(T_max, layers[l]->cfg.T);
   // A layer that the list names by more than one index is planned without sums (a sum belongs to one index), and two of its
@@ -482,7 +484,7 @@ int32_t qe_step_run(qe_ctx* ctx, qe_layer* const* layers, uint32_t n_layers, con
   std::vector<qe_layer*> by_address(layers, layers + n_layers);
   std::sort(by_address.begin(), by_address.end());
   const bool repeated = std::adjacent_find(by_address.begin(), by_address.end()) != by_address.end();
-  const uint32_t max_sum = repeated || T_max >= 4096 ? 1u : std::min(qe::kMaxSegments, 8192u / T_max);
+  const uint32_t fit = 8192u / T_max, max_sum = repeated || fit < 3 ? 1u : std::min(qe::kMaxSegments, fit);
   std::vector<std::vector<uint32_t>> rounds;  // indices into actions[]
   if (!temp && ctx->step_window > 1) {
     std::vector<uint32_t> slots(n_layers), live(n_layers), round_of(n_actions);

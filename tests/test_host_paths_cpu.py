@@ -214,3 +214,15 @@ def test_standalone_gemms_encode_one_map_per_operand_and_output(lib):
     lib.fake_reset()
     d = qe.qe_gemm_desc(a, a, a, a, a, a, 0, 0, 0, 0, 256, 256, 256, 0)
     assert lib.qe_gemm_fp8_group((qe.qe_gemm_desc * 3)(d, d, d), 3, a, None) == 0 and lib.fake_encodes() == 9
+
+
+@pytest.mark.parametrize("tokens,sums", [(256, True), (2048, True), (2688, True), (2816, False), (4096, False)])
+def test_step_sums_weight_gradients_where_three_products_fit(lib, tokens, sums):
+    s = fake_runtime.Stage(lib, [(256, 256)] * 2, T=tokens, M=6, slots=6)
+    lib.fake_reset()
+    acts = [a for a in _actions(6, 2) if a[0] != "dW"] + [("dW", l, m) for m in range(6) for l in (1, 0)]
+    assert s.step(acts) == 0
+    words = [w.split() for w in lib.fake_log().decode().splitlines() if " gemm " in w]  # launch STREAM gemm N products P
+    assert sum(int(w[5]) for w in words) == len(acts)
+    assert any(int(w[5]) > int(w[3]) for w in words) == sums
+    s.close()
