@@ -672,3 +672,108 @@ def test_step_call_sums_of_weight_gradients_equal_one_launch_each_bitwise(qe, mo
         assert np.array_equal(a, b)
     for a, b in zip(results[0][3], results[1][3]):
         assert state_equal({**a, "slots": []}, {**b, "slots": []})
+
+
+LONG = [(256, 512), (512, 256), (256, 256), (384, 256)] * 4
+
+
+def _long_stage(qe, mode, window, M, s, shapes=LONG, T=256, tag="LG"):
+    ctx = qe.Context(mode, step_window=window)
+    layers = [qe.Layer(ctx, T, K, N, 4, 0, peak_live(s), inputs.weights(tag, 0, j, N, K).to(DEV), unit=j) for j, (K, N) in enumerate(shapes)]
+    offs, total = inputs.grad_offsets([("l", K, N) for K, N in shapes])
+    X = [[inputs.activations(tag, 0, 0, j, m, T, K).to(DEV) for j, (K, N) in enumerate(shapes)] for m in range(M)]
+    dY = [[inputs.upstream_grads(tag, 0, 0, j, m, T, N).to(DEV) for j, (K, N) in enumerate(shapes)] for m in range(M)]
+    Y = [[torch.zeros((T, N), dtype=torch.bfloat16, device=DEV) for K, N in shapes] for m in range(M)]
+    dX = [[torch.zeros((T, K), dtype=torch.bfloat16, device=DEV) for K, N in shapes] for m in range(M)]
+    grad = torch.full((total,), 3.0, device=DEV)
+    return ctx, layers, offs, X, Y, dY, dX, grad
+
+
+def _same_snapshot(a, b):
+    for u, v in zip(a[0] + a[1] + [a[2].view(np.uint32)], b[0] + b[1] + [b[2].view(np.uint32)]):
+        assert np.array_equal(u, v)
+    for u, v in zip(a[3], b[3]):
+        assert state_equal({**u, "slots": []}, {**v, "slots": []}) and u["device_token"] == v["device_token"]
+
+
+@pytest.mark.parametrize("mode", [0, 1], ids=["eager", "graph"])
+def test_long_step_of_wide_launches_in_several_pieces_equals_single_actions_bitwise(qe, mode):
+    """Sixteen linears and twelve microbatches: launches of eight forwards and input gradients with sums of weight gradients
+    beside them, and in graph mode a list that goes out as several graphs."""
+    M, n = 12, len(LONG)
+    s = sched(M, 4, 4)
+    acts = _actions(s, n)
+    rounds = qe.plan_rounds(acts, n, M, peak_live(s), 16, 8, max_sum=8)
+    assert len(rounds) > 64 and any(sum(a != "dW" for a, l, m in g) == 8 and len({l for a, l, m in g if a == "dW"}) == 3 for g in rounds)
+    got = []
+    for window in (1, 16):
+        ctx, layers, offs, X, Y, dY, dX, grad = _long_stage(qe, mode, window, M, s)
+        plan = qe.StepPlan(ctx, layers, acts, M, X, Y, dY, dX, grad, offs)
+        for _ in range(3):
+            plan.run()
+            qe.optimizer_boundary_all(layers, M)
+        got.append(_snapshot(layers, Y, dX, grad))
+    _same_snapshot(*got)
+    if mode == 1:
+        st = ctx.stats()
+        assert st["graphs_built"] >= 2 and st["graph_replays"] == 3 * st["graphs_built"]  # several pieces, kept from step to step
+
+
+def test_check_that_fails_after_a_piece_is_out_leaves_the_state_that_eager_mode_leaves(qe):
+    M, n = 12, len(LONG)
+    s = sched(M, 4, 4)
+    acts = _actions(s, n)
+    got = []
+    for mode in (0, 1):
+        ctx, layers, offs, X, Y, dY, dX, grad = _long_stage(qe, mode, 16, M, s)
+        missing = [row[:] for row in dY]
+        missing[M - 1][2] = None  # one of the last input gradients has no dY
+        plan = qe.StepPlan(ctx, layers, acts, M, X, Y, missing, dX, grad, offs)
+        with pytest.raises(qe.QEError) as e:
+            plan.run()
+        assert e.value.code == "BAD_ARG" and "step aborted at action %d" % acts.index(("dI", 2, M - 1)) in str(e.value)
+        if mode == 1:
+            assert ctx.stats()["graph_replays"] >= 1  # a piece had gone out before the check
+        after = _snapshot(layers, Y, dX, grad)
+        for L in layers:
+            st = L.state()
+            assert st["aborted"] and st["device_token"] == st["token"] and not any(x["live"] for x in st["slots"])
+            L.arena_rebuild()
+        qe.StepPlan(ctx, layers, acts, M, X, Y, dY, dX, grad, offs).run()  # the epoch again, with every input
+        qe.optimizer_boundary_all(layers, M)
+        got.append((after, _snapshot(layers, Y, dX, grad)))
+    _same_snapshot(got[0][0], got[1][0])
+    _same_snapshot(got[0][1], got[1][1])
+
+
+@pytest.mark.parametrize("n", [5, 9, 16])
+def test_dW_multi_of_many_linears_equals_per_layer_calls_bitwise(qe, n):
+    """Overwriting and accumulating weight gradients of up to sixteen linears in one launch; one linear's N is an odd multiple
+    of 128, which goes out by itself."""
+    T, M = 384, 2
+    shapes = [(256 + 128 * (j % 3), 384 if j == 2 else 256 + 256 * (j % 2)) for j in range(n)]
+    offs, total = inputs.grad_offsets([("l", K, N) for K, N in shapes])
+    results = []
+    for multi in (False, True):
+        ctx = qe.Context(1)
+        layers = [qe.Layer(ctx, T, K, N, 4, 0, M, inputs.weights("MW", 0, j, N, K).to(DEV), unit=j) for j, (K, N) in enumerate(shapes)]
+        grad = torch.full((total,), -3.0, device=DEV)
+        for step in range(2):
+            tapes = {}
+            for m in range(M):
+                for j, (K, N) in enumerate(shapes):
+                    x, dy = inputs.activations("MW", 0, step, j, m, T, K).to(DEV), inputs.upstream_grads("MW", 0, step, j, m, T, N).to(DEV)
+                    tapes[j, m] = layers[j].forward(m, step, x, torch.empty((T, N), dtype=torch.bfloat16, device=DEV))
+                    layers[j].backward_dI(tapes[j, m], dy, torch.empty((T, K), dtype=torch.bfloat16, device=DEV))
+                if multi:
+                    qe.backward_dW_multi(layers, [tapes[j, m] for j in range(n)], grad, offs)
+                else:
+                    for j in range(n):
+                        layers[j].backward_dW(tapes[j, m], grad, offs[j])
+            torch.cuda.synchronize()
+            qe.optimizer_boundary_all(layers, M)
+        results.append((grad.cpu().numpy().view(np.uint32).copy(), [L.state() for L in layers], ctx.stats()))
+    (g0, s0, st0), (g1, s1, st1) = results
+    assert np.array_equal(g0, g1) and all(state_equal(a, b) for a, b in zip(s0, s1))
+    launches = 1 + (-(-n // 4) if n <= 8 else 1)  # the odd linear by itself, the others of every four (more than eight: of all) together
+    assert st0["kernels_launched"] - st1["kernels_launched"] == 2 * M * (n - launches)
