@@ -43,7 +43,7 @@ extern "C" {
 
 typedef enum qe_status {
   QE_OK = 0,
-  QE_ERR_BAD_ARG = -1,      /* null pointer, index out of range, unknown enum value                           */
+  QE_ERR_BAD_ARG = -1,      /* null pointer, index out of range, unknown enum value, out of host memory       */
   QE_ERR_SHAPE = -2,        /* T, K or N not a multiple of 128 or outside [256, 2^20]                         */
   QE_ERR_KEY_LIVE = -3,     /* forward: the same TapeKey already has a live tape (mapping must stay injective)*/
   QE_ERR_POOL_FULL = -4,    /* forward: no free slot; an occupied slot is never pre-empted                    */
@@ -200,14 +200,13 @@ int32_t qe_layer_create(qe_ctx*, const qe_layer_config*, void* workspace_dev, ui
 int32_t qe_layer_destroy(qe_layer*);
 
 /* F (Eq. 3).  x_dev bf16 [T,K] in, y_dev bf16 [T,N] out.  `gen` is the caller's view of the weight version and must
- * equal e_W.  On the first forward of an epoch the weight is re-quantised (E4M3; plus its transpose where dI needs one) and its amax
- * committed.  Then: X quantised to E4M3 with the current scale (amax taken in the same pass; the inverse scale is
- * snapshotted into the tape slot), Y = bf16((Xq Wq^T) * sinv_X * sinv_W) on the tensor cores with max|Y| reduced in
- * the epilogue, and the X and Y histories/scales updated.  *tape_out names the retained work. */
+ * equal e_W.  On the first forward of an epoch the weight is re-quantised (E4M3) and its amax committed.  Then: X
+ * quantised to E4M3 with the current scale (amax taken in the same pass; the inverse scale is snapshotted into the tape
+ * slot), Y = bf16((Xq Wq^T) * sinv_X * sinv_W) on the tensor cores with max|Y| reduced in the epilogue, and the X and Y
+ * histories/scales updated.  *tape_out names the retained work. */
 int32_t qe_forward(qe_layer*, uint32_t mb, uint64_t gen, const void* x_dev, void* y_dev, void* caller_stream,
                    qe_tape* tape_out);
-/* dI (Eq. 4).  dy_dev bf16 [T,N] in, dx_dev bf16 [T,K] out.  Quantises dY to E5M2 (and, where dW needs it, its transpose, retained for
- * dW), dX = bf16((Gq Wq) * sinv_G * sinv_W), commits the gradient amax/scale once. */
+/* dI (Eq. 4).  dy_dev bf16 [T,N] in, dx_dev bf16 [T,K] out.  Quantises dY to E5M2 (retained for dW), dX = bf16((Gq Wq) * sinv_G * sinv_W), commits the gradient amax/scale once. */
 int32_t qe_backward_dI(qe_layer*, const qe_tape*, const void* dy_dev, void* dx_dev, void* caller_stream);
 /* F and dI with HOST buffers (layer created with host_io = 1).  The input is copied host-to-device into the layer's
  * fixed staging buffer after the caller->execution edge (the dynamic-input copy of Sec. 4.4), the action runs on
@@ -348,7 +347,8 @@ int32_t qe_next_slot(const qe_layer*, uint32_t* slot_out);
  * the host exactly like the single calls; the kernels of the whole list are then issued behind ONE caller->execution
  * wait and ONE execution->caller event: in eager mode as plain launches, in graph mode as one captured graph (a list of more
  * than 64 launches: several, issued one after the other while the next is prepared) that is cached per (layers, actions)
- * and replayed, with kernel-node parameters patched where pointers or the accumulate flag differ from the previous replay.  dW runs on the execution stream here (QE_CTX_OVERLAP_DW does not apply).
+ * and replayed, with kernel-node parameters patched where pointers or the accumulate flag differ from the previous
+ * replay.  dW runs on the execution stream here (QE_CTX_OVERLAP_DW does not apply).
  * Independent actions share launches, with bit-identical results (only the slot a tape lands in may differ from the
  * one-by-one order).  The list is read as units -- runs of actions of one kind and microbatch over distinct layers: a
  * forward, input-gradient or weight-gradient unit of the stage -- and cut into rounds of actions whose predecessors were
@@ -406,8 +406,8 @@ typedef struct qe_state_view {
 int32_t qe_get_state(qe_layer*, qe_state_view* out, float* window_out, float* slot_sinv_out);
 /* Copies a slot's retained FP8 bytes to host memory (testing aid; synchronises).  which: 0 = Xq [T,K],
  * 1 = Xq^T [K,T], 2 = Gq [T,N], 3 = Gq^T [N,T], 4 = Wq [N,K] (slot ignored), 5 = Wq^T [K,N] (slot ignored).
- * Transposed copies exist only where a GEMM needs them: Wq^T when T is not a multiple of 256, Xq^T and Gq^T when N
- * is not (otherwise the tensor cores read the row-major tensor as an MN-major operand) -- QE_ERR_UNSUPPORTED if absent. */
+ * The layer keeps the row-major tensors only (every GEMM reads them as they are); the transposes are made on the host, and
+ * offered for Wq when T is not a multiple of 256 and for Xq and Gq when N is not -- QE_ERR_UNSUPPORTED otherwise. */
 int32_t qe_read_fp8(qe_layer*, uint32_t which, uint32_t slot, void* host_out, uint64_t bytes);
 
 /* Quiescent checkpoint (Sec. 3.5, Invariant 4).  The payload holds PERSISTENT state only: the static configuration
@@ -447,9 +447,10 @@ uint32_t qe_amax_partials(void);
 int32_t qe_accumulate(float* dst_dev, const float* src_dev, uint64_t n, int32_t accumulate, void* stream);
 /* One FP8 GEMM on the tensor cores: D[m,n] = (sum_k A[m,k] B[n,k]) * *alpha_a_dev * *alpha_b_dev with A [M,Kc] and
  * B [Nn,Kc] both contraction-major bytes.  out_kind 0: bf16 D (amax_dev optional, as in qe_quantize); 1: FP32
- * D overwrite; 2: FP32 D accumulate.  M, Kc multiples of 128 (>= 128), Nn a multiple of 128 (>= 256).  Tiles
- * have 256 rows; a last one that M fills by half is computed with zero rows that are not stored.  status_dev: one uint32 the kernel ORs error
- * bits into (caller zeroes it). */
+ * D overwrite; 2: FP32 D accumulate.  M, Kc multiples of 128 (>= 128), Nn a multiple of 128 (>= 256).  Tiles have 256
+ * rows, of which a last one that M fills by half computes 128 that are not stored; an odd number of 128-row tiles that
+ * would need another wave of them goes out in tiles of 128 rows.  status_dev: one uint32 the kernel ORs error bits into
+ * (caller zeroes it). */
 int32_t qe_gemm_fp8(const void* a_dev, uint32_t a_format, const void* b_dev, uint32_t b_format, uint32_t M,
                     uint32_t Nn, uint32_t Kc, const float* alpha_a_dev, const float* alpha_b_dev, void* d_dev,
                     uint32_t out_kind, float* amax_dev, uint32_t* status_dev, void* stream);

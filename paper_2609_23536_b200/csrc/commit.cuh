@@ -1,7 +1,8 @@
-// Amax-history reduction and scale update as a device function, shared by the standalone commit kernel and by the
-// tails of the quantise and GEMM kernels (where the last block to finish performs it, saving a launch).
+// Amax-history reduction and scale update as device functions: by a whole block in the standalone commit kernel and in the
+// tail of a weight's cast (its last block), by one warp in the GEMM launches (X and G at a launch's start, where an earlier
+// kernel has completed the amax; Y by the last CTA of the launch that computes it).  No launch is spent on a commit.
 //   hist[c][count mod H] = amax;  scale_c = fp8_max / max(hist[c]) / 2^margin;  scale_inv_c = 1 / scale_c
-// 256 threads take part: 64 per tensor class, all four classes in parallel, one barrier.  The ring's maximum is kept
+// The block form: 256 threads, 64 per tensor class, all four classes in parallel, one barrier.  The ring's maximum is kept
 // beside it so that a commit usually reads one entry instead of H.  The maximum is taken on
 // the bit patterns of the non-negative FP32 entries, which orders them like their values and lets a NaN or Inf
 // entry surface as "not finite" (scale then stays as it was, like for an all-zero window).

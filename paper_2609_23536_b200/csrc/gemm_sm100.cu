@@ -905,7 +905,7 @@ Launch make_any(const GemmDesc* probs, uint32_t n, uint32_t nops, int num_sms) {
 
 }  // namespace
 
-bool gemm_uses_pair(uint32_t M) { return M % 256 == 0; }
+bool whole_row_tiles(uint32_t M) { return M % 256 == 0; }
 
 cudaError_t gemm_prepare() {
   for (const void* f : {(const void*)gemm_fp8_kernel, (const void*)gemm_fp8_pair_kernel, (const void*)gemm_fp8_pair_group_kernel, (const void*)gemm_fp8_pair_wide_kernel}) {
@@ -918,7 +918,7 @@ cudaError_t gemm_prepare() {
 bool make_gemm_group(const GemmDesc* probs, uint32_t n, int num_sms, Launch* out) {
   uint32_t nops = 0;
   for (uint32_t i = 0; i < n; ++i) {
-    if (!gemm_uses_pair(probs[i].M)) return false;
+    if (!whole_row_tiles(probs[i].M)) return false;
     nops += probs[i].nseg;
   }
   if (n < 2 || n > kMaxProblems || nops > kMaxOperands) return false;

@@ -235,7 +235,9 @@ Launch make_gemm(const GemmDesc& p, int num_sms);
 bool make_gemm_group(const GemmDesc* probs, uint32_t n, int num_sms, Launch* out);
 uint32_t gemm_width(const GemmDesc* probs, uint32_t n, int num_sms);  // index of the tile width the launch of these will have
 cudaError_t gemm_prepare();  // opt in to the dynamic shared memory the GEMM needs (once per device)
-bool gemm_uses_pair(uint32_t M);  // whole 256-row tiles: may share launches and take MN-major operands
+// Whether M fills whole 256-row tiles.  The kernels take any multiple of 128, and the layers' MN-major operands come with any;
+// shared launches, the hand-off (of N) and MN-major operands of the standalone calls are offered for whole tiles only.
+bool whole_row_tiles(uint32_t M);
 constexpr uint32_t kAmaxPartials = 2048;
 
 }  // namespace qe

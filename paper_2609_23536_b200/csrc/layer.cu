@@ -446,9 +446,9 @@ int32_t qe_read_fp8(qe_layer* L, uint32_t which, uint32_t slot, void* host_out, 
   if (which > 5 || (which < 4 && slot >= L->cfg.slots)) return fail(QE_ERR_BAD_ARG, "which %u slot %u", which, slot);
   const bool transposed = which & 1u;  // 1, 3, 5: the transposes of 0, 2, 4
   const uint8_t* src = which < 2 ? L->Xq[slot] : which < 4 ? L->Gq[slot] : L->Wq;
-  // (offered for the layers whose GEMMs have half-filled row tiles; made here, no kernel reads one)
-  if (transposed && qe::gemm_uses_pair(which == 5 ? L->cfg.T : L->cfg.N))
-    return fail(QE_ERR_UNSUPPORTED, "this layer keeps no transposed copy %u (its GEMM reads the row-major tensor directly)", which);
+  // (offered where a GEMM has a half-filled row tile; made here, no kernel reads one)
+  if (transposed && qe::whole_row_tiles(which == 5 ? L->cfg.T : L->cfg.N))
+    return fail(QE_ERR_UNSUPPORTED, "no transposed view %u of this layer (offered for odd multiples of 128 only)", which);
   const uint64_t need = which < 2 ? tk : which < 4 ? tn : nk;
   if (bytes != need) return fail(QE_ERR_BAD_ARG, "bytes %llu, tensor has %llu", (unsigned long long)bytes, (unsigned long long)need);
   QE_CUDA(cudaStreamSynchronize(L->ctx->exec_stream));

@@ -84,7 +84,7 @@ static int32_t check_chain(qe_layer* const* layers, uint32_t n) {
   }
   // (whole 256-row tiles only, as for the shared launches)
   for (uint32_t i = 0; n > 1 && i < n; ++i)
-    if (!qe::gemm_uses_pair(layers[i]->cfg.N)) return fail(QE_ERR_UNSUPPORTED, "layer %u: N must be a multiple of 256 for the hand-off", i);
+    if (!qe::whole_row_tiles(layers[i]->cfg.N)) return fail(QE_ERR_UNSUPPORTED, "layer %u: N must be a multiple of 256 for the hand-off", i);
   return QE_OK;
 }
 
@@ -282,7 +282,7 @@ int32_t together_build(qe_ctx* ctx, const qe_action* acts, uint32_t n, const Tog
       } else {
         gp = dW_gemm(L, pr.slot[i], grad + a.grad_offset, pr.acc[i], nullptr);
       }
-      const bool paired = qe::gemm_uses_pair(gp.M);
+      const bool paired = qe::whole_row_tiles(gp.M);
       if (paired) (a.kind == QE_ACT_DW ? n_dw : n_chain) += 1;
       qe::GemmDesc* sum = nullptr;  // this layer's weight gradient of an earlier microbatch, which takes this one in
       if (a.kind == QE_ACT_DW) {

@@ -174,7 +174,10 @@ void add_dW(qe_layer* L, uint32_t p, float* dst, int32_t accumulate, float* temp
 // The layers' gradient slices are disjoint (destination registry), so the GEMMs are independent.
 // Up to eight layers go out four to a launch.  More go out sixteen to a launch: sixteen 1024 x 1024 gradients of 512 tokens
 // in four launches of 64 tiles leave CTA pairs idle and pay four starts and four last epilogues (chain of sixteen:
-// 2397 us a step in fours, 2316 in eights, 2304 in sixteens).
+// 2397 us a step in fours, 2316 in eights, 2304 in sixteens).  One call, accumulating, sixteen to a launch against fours:
+// nine of 1024 x 1024 35 us for 44, sixteen of 2048 x 2048 138 for 158 (2048 tokens: 182 for 197), twelve and sixteen of
+// 4096 x 4096 334 and 443 for 334 and 445 (446 and 596 for 450 and 601).  Sixteens are faster at five to eight layers
+// too (five of 1024 x 1024 30 for 33, eight of 2048 x 2048 76 for 86, eight of 4096 x 4096 at 2048 tokens 288 for 300).
 struct DWBatch {
   uint32_t limit;
   std::vector<qe::GemmDesc> gp;
@@ -184,7 +187,7 @@ struct DWBatch {
   void flush(qe_ctx* ctx, std::vector<qe::Launch>& ls) {
     std::vector<qe::GemmDesc> paired;
     for (const qe::GemmDesc& g : gp)
-      if (qe::gemm_uses_pair(g.M)) paired.push_back(g);
+      if (qe::whole_row_tiles(g.M)) paired.push_back(g);
     qe::Launch l;
     const bool grouped = paired.size() >= 2 && qe::make_gemm_group(paired.data(), (uint32_t)paired.size(), ctx->dev->num_sms, &l);
     if (grouped) {
@@ -192,7 +195,7 @@ struct DWBatch {
       ctx->stats.grouped_dw += paired.size();
     }
     for (const qe::GemmDesc& g : gp)
-      if (!grouped || !qe::gemm_uses_pair(g.M)) ls.push_back(qe::make_gemm(g, ctx->dev->num_sms));
+      if (!grouped || !qe::whole_row_tiles(g.M)) ls.push_back(qe::make_gemm(g, ctx->dev->num_sms));
     gp.clear();
     layer.clear();
   }

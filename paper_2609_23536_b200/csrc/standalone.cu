@@ -71,7 +71,8 @@ struct StandaloneGemm {
 };
 
 // Validates one standalone GEMM and fills its descriptor, up to the map of its B operand (standalone_map_b), whose box depends
-// on the launch's tile width: one map is encoded per operand (three for B cost the call 0.25 us of host time, which bounds it: 9.8 us for 9.6).
+// on the launch's tile width: one map is encoded per operand.  (Host time bounds the call; with three maps for B 512 x 4096 x
+// 4096 took 9.8 us of it, with one 9.6.)
 static int32_t standalone_gemm(DeviceInfo* dev, const void* a, uint32_t a_fmt, uint32_t a_mn, const void* b, uint32_t b_fmt,
                                uint32_t b_mn, uint32_t M, uint32_t Nn, uint32_t Kc, const float* alpha_a, const float* alpha_b,
                                void* d, uint32_t out_kind, float* amax_dev, uint32_t* status_dev, StandaloneGemm* sg) {
@@ -79,7 +80,7 @@ static int32_t standalone_gemm(DeviceInfo* dev, const void* a, uint32_t a_fmt, u
   if (a_fmt > QE_E5M2 || b_fmt > QE_E5M2 || out_kind > 2 || a_mn > 1 || b_mn > 1) return fail(QE_ERR_BAD_ARG, "bad enum");
   if (!shape_ok(M) && M != 128) return fail(QE_ERR_SHAPE, "M=%u", M);
   if (!shape_ok(Nn) || (!shape_ok(Kc) && Kc != 128)) return fail(QE_ERR_SHAPE, "N=%u Kc=%u", Nn, Kc);
-  if ((a_mn || b_mn) && !qe::gemm_uses_pair(M))
+  if ((a_mn || b_mn) && !qe::whole_row_tiles(M))
     return fail(QE_ERR_UNSUPPORTED, "MN-major operands need M to be a multiple of 256, M=%u", M);
   if ((((uintptr_t)a | (uintptr_t)b | (uintptr_t)d) & 15u)) return fail(QE_ERR_BAD_ARG, "misaligned pointer");
   int32_t st;
@@ -130,7 +131,7 @@ int32_t qe_gemm_fp8_group(const qe_gemm_desc* descs, uint32_t n, uint32_t* statu
   qe::GemmDesc gp[8];
   for (uint32_t i = 0; i < n; ++i) {
     const qe_gemm_desc& q = descs[i];
-    if (!qe::gemm_uses_pair(q.M)) return fail(QE_ERR_UNSUPPORTED, "problem %u: M=%u is not a multiple of 256", i, q.M);
+    if (!qe::whole_row_tiles(q.M)) return fail(QE_ERR_UNSUPPORTED, "problem %u: M=%u is not a multiple of 256", i, q.M);
     if ((st = standalone_gemm(dev, q.a_dev, q.a_format, q.a_mn, q.b_dev, q.b_format, q.b_mn, q.M, q.Nn, q.Kc, q.alpha_a_dev,
                               q.alpha_b_dev, q.d_dev, q.out_kind, q.amax_dev, status_dev, &sg[i])) != QE_OK)
       return st;

@@ -1,6 +1,6 @@
 """Small single-kernel cases for profiling (ncu) and quick timing.
 
-    python profile_case.py gemm_f|gemm_di|gemm_dw|gemm_microbatch|gemm_microbatch_grouped|gemm_step|quantize|quantize_t|amax|accumulate [--reps N]
+    python profile_case.py gemm_f|gemm_di|gemm_dw|gemm_narrow|gemm_odd|gemm_microbatch|gemm_microbatch_grouped|gemm_step|step_sums|quantize|quantize_t|amax|accumulate [--reps N]
 
 Each case holds well under 2 GB on the device, uses operands larger than the 126 MB L2 where DRAM traffic is
 the question, does 2 warm-up launches and then `reps` launches, and prints the CUDA-event time per launch.
@@ -82,10 +82,32 @@ def main():
 
         work = {"flop": sum(2.0 * M * N * Kc for M, N, Kc, *_ in shapes),
                 "bytes": sum(M * Kc + N * Kc + M * N * (2 if k == 0 else 8) for M, N, Kc, _, k, _, _ in shapes)}
+    elif a.case == "step_sums":
+        # one optimizer step of a 4096 / 11008 layer, eight microbatches of 256 tokens: the weight gradients go out as sums
+        # (gemm_fp8_pair_wide_kernel)
+        from paper_2609_23536_b200.schedules import peak_live, sched
+
+        t, M, shapes = 256, 8, [(4096, 12288), (4096, 4096), (4096, 11008), (11008, 4096)]
+        order = sched(M, 3, 3)
+        ctx = qe.Context(qe.EAGER, step_window=6)
+        rnd = lambda *shape: torch.randn(shape, device=dev).to(torch.bfloat16)
+        layers = [qe.Layer(ctx, t, K, N, 16, 0, peak_live(order), rnd(N, K).mul_(0.02), unit=u) for u, (K, N) in enumerate(shapes)]
+        tensors = [[[rnd(t, d[side]) for d in shapes] for _ in range(M)] for side in (0, 1, 1, 0)]
+        grad = torch.zeros(sum(K * N for K, N in shapes), device=dev)
+        acts = [(k, i, m) for k, m in order for i in (range(4) if k == "F" else range(3, -1, -1))]
+        plan = qe.StepPlan(ctx, layers, acts, M, *tensors, grad, [sum(K * N for K, N in shapes[:i]) for i in range(4)])
+
+        def fn():
+            plan.run()
+            qe.optimizer_boundary_all(layers, M)
+
+        work = {"flop": 6.0 * t * M * sum(K * N for K, N in shapes), "bytes": sum(4 * t * M * (K + N) + 6 * K * N for K, N in shapes)}
     elif a.case.startswith("gemm"):
-        # gate/up projection: F: [T,H]x[F,H]^T ; dI: [T,F]x[H,F]^T ; dW: [F,T]x[H,T]^T (FP32 accumulate)
+        # gate/up projection: F: [T,H]x[F,H]^T ; dI: [T,F]x[H,F]^T ; dW: [F,T]x[H,T]^T (FP32 accumulate); a weight
+        # gradient small enough for tiles of 64 columns; a forward of nine 128-row tiles, a CTA to a tile
         M, N, Kc, af, kind, amn, bmn = {"gemm_f": (T, F, H, 0, 0, 0, 0), "gemm_di": (T, H, F, 1, 0, 0, 1),
-                                        "gemm_dw": (F, H, T, 1, 2, 1, 1)}[a.case]
+                                        "gemm_dw": (F, H, T, 1, 2, 1, 1), "gemm_narrow": (1024, 512, 1024, 1, 2, 1, 1),
+                                        "gemm_odd": (1152, 4096, 4096, 0, 0, 0, 0)}[a.case]
         A = torch.randint(0, 120, (Kc, M) if amn else (M, Kc), dtype=torch.uint8, device=dev)
         B = torch.randint(0, 120, (Kc, N) if bmn else (N, Kc), dtype=torch.uint8, device=dev)
         D = torch.zeros((M, N), dtype=torch.bfloat16 if kind == 0 else torch.float32, device=dev)

@@ -199,7 +199,7 @@ Launch named(const char* fmt, ...) {
   return l;
 }
 }  // namespace
-bool gemm_uses_pair(uint32_t M) { return M % 256 == 0; }
+bool whole_row_tiles(uint32_t M) { return M % 256 == 0; }
 cudaError_t gemm_prepare() { return cudaSuccess; }
 uint32_t gemm_width(const GemmDesc*, uint32_t, int) { return 1; }
 Launch make_quantize(const QuantParams&) { return named("cast 1"); }

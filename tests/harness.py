@@ -185,8 +185,8 @@ def state_equal_except_Y(gpu: dict, orc: dict) -> bool:
 
 
 def transposed_or_none(layer, which, slot=0):
-    """A layer's transposed FP8 copy (which = 1, 3, 5), or None when the layer keeps none because its GEMMs read the
-    row-major tensor as an MN-major operand."""
+    """The transposed view of a layer's FP8 tensor (which = 1, 3, 5) that qe_read_fp8 makes on the host, or None where it
+    offers none."""
     from paper_2609_23536_b200 import binding as qe
 
     try:

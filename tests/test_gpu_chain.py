@@ -255,7 +255,7 @@ def test_chain_argument_checks(qe):
     with pytest.raises(qe.QEError) as e:
         qe.forward_chain([layers[0], layers[0]], 0, 0, x, y)
     assert e.value.code == "BAD_ARG"
-    odd = qe.Layer(ctx, T, 768, 384, 4, 0, 2, inputs.weights("CN", 0, 9, 384, 768).to(DEV), unit=9)  # N = 384 keeps transposed copies
+    odd = qe.Layer(ctx, T, 768, 384, 4, 0, 2, inputs.weights("CN", 0, 9, 384, 768).to(DEV), unit=9)  # N = 384: not offered
     tail = qe.Layer(ctx, T, 384, 256, 4, 0, 2, inputs.weights("CN", 0, 10, 256, 384).to(DEV), unit=10)
     with pytest.raises(qe.QEError) as e:
         qe.forward_chain(layers + [odd, tail], 0, 0, x, torch.zeros((T, 256), dtype=torch.bfloat16, device=DEV))

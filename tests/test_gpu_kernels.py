@@ -332,7 +332,7 @@ def test_gemm_group_equals_single_launches_bitwise(qe):
     for d1, d2, am1, am2, kind in outs:
         assert torch.equal(d1.view(torch.int16 if kind == 0 else torch.int32), d2.view(torch.int16 if kind == 0 else torch.int32))
         assert am1.item() == am2.item() and (kind != 0 or am1.item() > 0)
-    with pytest.raises(qe.QEError) as e:  # a problem that needs the single-CTA variant cannot join
+    with pytest.raises(qe.QEError) as e:  # a problem with a half-filled row tile cannot join
         A = torch.zeros((384, 128), dtype=torch.uint8, device=DEV)
         B = torch.zeros((256, 128), dtype=torch.uint8, device=DEV)
         d = torch.zeros((384, 256), device=DEV)

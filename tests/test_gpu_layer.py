@@ -73,7 +73,7 @@ def test_config1_every_action_against_oracle(qe, mode):
         assert state_equal_except_Y(g, ostate), (step, a, m)
         assert np.float32(g["cache_sinv_W"]).view(np.uint32) == np.float32(osinvW).view(np.uint32)
         assert np.array_equal(layer.read_fp8(4), oWq)
-        assert transposed_or_none(layer, 5) is None  # 256-multiples: the dI GEMM reads Wq itself, MN-major
+        assert transposed_or_none(layer, 5) is None  # 256-multiples: not offered
         for p, (Xq, Gq, sX, sG) in oslots.items():
             assert np.array_equal(layer.read_fp8(0, p), Xq) and transposed_or_none(layer, 1, p) is None
             assert g["slot_sinv_X"][p].view(np.uint32) == np.float32(sX).view(np.uint32)
@@ -163,7 +163,8 @@ def test_overlapped_dW_stream_gives_the_same_bits(qe, mode, staged):
 
 @pytest.mark.parametrize("mode", [0, 1], ids=["eager", "graph"])
 def test_shapes_that_take_the_single_cta_gemm_against_oracle(qe, mode):
-    # T and N multiples of 128 but not of 256: F, dI and dW all run the 128 x 256-tile variant, with ragged last tiles
+    # T and N multiples of 128 but not of 256: F, dI (B MN-major) and dW (both MN-major) with half-filled last row tiles and
+    # ragged last column tiles; the comparison with the oracle is what checks that no GEMM needs a transposed tensor
     T, K, N, M, H = 384, 640, 896, 3, 4
     s = sched(M, 2, 1)
     P = peak_live(s)
@@ -181,7 +182,7 @@ def test_shapes_that_take_the_single_cta_gemm_against_oracle(qe, mode):
         else:
             assert_gemm_close(got[k], want[k], k)
     assert state_equal_except_Y(L.state(), O.state())
-    # these shapes keep transposed copies (their dI / dW GEMMs take contraction-major operands only)
+    # the transposed views that qe_read_fp8 makes on the host for such shapes
     assert np.array_equal(L.read_fp8(5), O.Wq.T) and np.array_equal(L.read_fp8(4), O.Wq)
     assert L.read_fp8(1, 0).shape == (K, T) and L.read_fp8(3, 0).shape == (N, T)
 

@@ -302,7 +302,7 @@ def test_two_chunk_schedules_split_equals_full_and_match_the_oracle(qe, gen, mod
 def test_forward_dI_pair_equals_separate_calls_bitwise(qe, mode, overlap):
     """Steady state of a split-backward schedule: F(m + 2) of linear i together with dI(m) of linear n-1-i."""
     T, M = 256, 5
-    shapes = [(256, 512), (512, 256), (384, 384), (256, 768)]  # F and dI GEMMs have M = T = 256: all take the paired variant
+    shapes = [(256, 512), (512, 256), (384, 384), (256, 768)]  # F and dI GEMMs have M = T = 256: whole row tiles
     n = len(shapes)
     offs, total = inputs.grad_offsets([("l", K, N) for K, N in shapes])
     s = sched(M, 2, 2)
@@ -431,7 +431,7 @@ def test_run_together_equals_one_action_after_the_other_bitwise(qe, mode):
         assert state_equal({**u, "slots": []}, {**v, "slots": []}) and u["device_token"] == v["device_token"]
     n_triples = sum(1 for k in range(len(s) - 2) if s[k][0] == "F" and s[k + 1][0] == "dI" and s[k + 2][0] == "dW")
     assert n_triples == 3
-    # per triple call three GEMM launches became one, except for the 384-wide linear whose dW takes the single-CTA variant
+    # per triple call three GEMM launches became one, except for the 384-wide linear whose dW, with a half-filled row tile, goes out by itself
     assert a[4]["kernels_launched"] - b[4]["kernels_launched"] == 2 * n_triples * (2 * n - 1 + n)  # ... and the two casts became one
     assert b[4]["grouped_dw"] == 2 * n_triples * (n - 1)
 

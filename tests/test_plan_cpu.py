@@ -75,7 +75,8 @@ def _actions(schedule, n):
 @pytest.mark.parametrize("n", [1, 3, 4])
 @pytest.mark.parametrize("window,group", [(1, 4), (2, 4), (4, 8), (6, 8)])
 def test_native_planner_makes_the_same_legal_plan(qe, M, w, d, n, window, group):
-    """qe_plan_rounds (what qe_step_run uses; host logic, no device) against schedules.plan_rounds (what bench.py uses)."""
+    """qe_plan_rounds (what qe_step_run uses where it sums no weight gradients; host logic, no device) against
+    schedules.plan_rounds (what bench.py uses)."""
     s = sched(M, w, d)
     slots = peak_live(s)
     native = qe.plan_rounds(_actions(s, n), n, M, slots, window, group)
