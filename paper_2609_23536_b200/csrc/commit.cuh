@@ -61,59 +61,54 @@ __device__ __forceinline__ void commit_classes(const CommitParams& p, int tid, u
   if (tid == 0 && p.bump_token) st->token += 1ull;
 }
 
-// The same commit done by ONE warp, class after class (a GEMM launch hands it one: X or G at its start, Y in its tail).
+// The same commit of ONE class by one warp (class_mask has one bit: X or G at a GEMM launch's start, Y in its tail).
 // A grouped launch may carry sixteen problems, each committed by a warp of its own, side by side: a commit is a chain of
-// dependent global accesses, and one after the other the commits of a launch took as long as its tiles.  The rare ring
-// scan takes 16-byte loads over all lanes, eight in flight each: F, dI and dW of a 256 x 256 x 256 linear plus the boundary
-// take 57 us when no commit scans; when all three do, 62 us at 4096 entries (81 with 4-byte loads of eight lanes) and the
-// same as without at 1024 (60).  Same values as commit_classes; the token is bumped atomically because two problems of
-// one launch may belong to the same layer (its forward and its input gradient of different microbatches).
-__device__ __forceinline__ uint32_t ring_max(const uint32_t* h, uint32_t H, uint32_t pos, uint32_t newest, uint32_t lane) {
-  uint32_t m = newest, at = 0;  // (the entry at pos is the one that leaves)
-  if ((reinterpret_cast<uintptr_t>(h) & 15u) == 0) {
-    at = H & ~3u;
-#pragma unroll 8
-    for (uint32_t i = 4 * lane; i < at; i += 128) {
-      const uint4 q = __ldcg(reinterpret_cast<const uint4*>(h + i));
-      m = max(m, max(max(i == pos ? 0u : q.x, i + 1 == pos ? 0u : q.y), max(i + 2 == pos ? 0u : q.z, i + 3 == pos ? 0u : q.w)));
-    }
-  }
-#pragma unroll 8
-  for (uint32_t i = at + lane; i < H; i += 32) {
-    const uint32_t q = __ldcg(h + i);
-    m = max(m, i == pos ? 0u : q);
-  }
-  return __reduce_max_sync(0xffffffffu, m);
-}
-
-__device__ __forceinline__ void commit_classes_warp(const CommitParams& p, int lane) {
+// dependent global accesses, and one after the other the commits of a launch took as long as its tiles.  The code runs once
+// per launch, from cold instruction memory, so it is short: one loop for the rare ring scan, 16-byte loads over all lanes,
+// four in flight each (48 linears of 1024 x 1024: 13254 us a step; 13337 with the scan in two loops of eight loads, 13298
+// with eight lanes of 4-byte loads for each of four classes).  F, dI and dW of a 256 x 256 x 256 linear plus the boundary
+// take 55 us when no commit scans; when all three do, 60 us at 4096 entries (77 with the eight lanes) and the same as
+// without at 1024 (61).  Same values as commit_classes; the token is bumped atomically because two problems of one launch
+// may belong to the same layer (its forward and its input gradient of different microbatches).
+__device__ __forceinline__ void commit_class_warp(const CommitParams& p, int lane) {
   DevState* st = p.st;
-#pragma unroll 1
-  for (uint32_t left = p.class_mask; left; left &= left - 1) {
-    const int c = __ffs(left) - 1;
-    uint32_t* h = reinterpret_cast<uint32_t*>(p.hist + (size_t)c * p.H);
-    const uint32_t cnt = __ldcg(&st->count[c]);
-    const uint32_t newest = p.amax_override ? (__float_as_uint(__ldcg(p.amax_override)) & 0x7fffffffu) : __ldcg(&st->pending_amax[c]);
-    const uint32_t wmax = __ldcg(&st->wmax[c]);
-    const uint32_t pos = cnt % p.H;
-    const uint32_t evicted = __ldcg(h + pos);
-    const uint32_t m = newest >= wmax ? newest : evicted < wmax ? wmax : ring_max(h, p.H, pos, newest, (uint32_t)lane);
-    __syncwarp();  // every lane has read the entry that lane 0 replaces
-    if (lane == 0) {
-      h[pos] = newest;
-      st->count[c] = cnt + 1;
-      st->pending_amax[c] = 0;
-      st->wmax[c] = m;
-      if (m != 0 && m < 0x7f800000u) {
-        const float fp8_max = c == 2 ? 57344.0f : 448.0f;
-        float s = __fmul_rn(__fdiv_rn(fp8_max, __uint_as_float(m)), p.pow2_neg_margin);
-        if (isinf(s)) s = FLT_MAX;
-        st->scale[c] = s;
-        st->scale_inv[c] = __fdiv_rn(1.0f, s);
-      }
+  const int c = __ffs(p.class_mask) - 1;
+  uint32_t* h = reinterpret_cast<uint32_t*>(p.hist + (size_t)c * p.H);
+  const uint32_t cnt = __ldcg(&st->count[c]);
+  const uint32_t newest = p.amax_override ? (__float_as_uint(__ldcg(p.amax_override)) & 0x7fffffffu) : __ldcg(&st->pending_amax[c]);
+  const uint32_t wmax = __ldcg(&st->wmax[c]);
+  const uint32_t pos = cnt % p.H;
+  const uint32_t evicted = __ldcg(h + pos);
+  uint32_t m = newest >= wmax ? newest : wmax;
+  if (newest < wmax && evicted >= wmax) {  // the maximum leaves: scan what stays
+    m = newest;
+    auto take = [&](uint32_t i, uint32_t q) { m = max(m, i == pos ? 0u : q); };
+    const uint32_t head = min(p.H, (4u - ((uint32_t)(reinterpret_cast<uintptr_t>(h) >> 2) & 3u)) & 3u);  // up to a 16-byte boundary
+    const uint32_t vecs = (p.H - head) / 4, tail = p.H - head - 4 * vecs;
+    if ((uint32_t)lane < head) take((uint32_t)lane, __ldcg(h + lane));
+    if ((uint32_t)lane < tail) take(p.H - tail + (uint32_t)lane, __ldcg(h + p.H - tail + lane));
+#pragma unroll 4
+    for (uint32_t v = (uint32_t)lane; v < vecs; v += 32) {
+      const uint32_t i = head + 4 * v;
+      const uint4 q = __ldcg(reinterpret_cast<const uint4*>(h + i));
+      take(i, q.x), take(i + 1, q.y), take(i + 2, q.z), take(i + 3, q.w);
     }
+    m = __reduce_max_sync(0xffffffffu, m);
   }
-  if (lane == 0 && p.bump_token) atomicAdd(&st->token, 1ull);
+  if (lane == 0) {
+    h[pos] = newest;
+    st->count[c] = cnt + 1;
+    st->pending_amax[c] = 0;
+    st->wmax[c] = m;
+    if (m != 0 && m < 0x7f800000u) {
+      const float fp8_max = c == 2 ? 57344.0f : 448.0f;
+      float s = __fmul_rn(__fdiv_rn(fp8_max, __uint_as_float(m)), p.pow2_neg_margin);
+      if (isinf(s)) s = FLT_MAX;
+      st->scale[c] = s;
+      st->scale_inv[c] = __fdiv_rn(1.0f, s);
+    }
+    if (p.bump_token) atomicAdd(&st->token, 1ull);
+  }
 }
 
 // Returns true in every thread of exactly one block of the grid: the last one to get here.  Stores and atomics the

@@ -439,7 +439,7 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
     CommitParams c = ps.commit(blockIdx.x);
     if (c.st && c.early_mask) {
       c.class_mask = c.early_mask;
-      commit_classes_warp(c, lane);
+      commit_class_warp(c, lane);
     }
   }
 
@@ -752,7 +752,7 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
       for (uint32_t i = (uint32_t)(warp - EPI_WARP0); i < ps.count(); i += EPI_WARPS) {
         CommitParams c = ps.commit(i);
         c.bump_token = 0;  // (counted by the early part)
-        if (c.st && c.class_mask) commit_classes_warp(c, lane);
+        if (c.st && c.class_mask) commit_class_warp(c, lane);
       }
     }
     // The bulk-store unit has read this warp's last tiles out of shared memory; that the bytes are in global memory
