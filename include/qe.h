@@ -346,7 +346,7 @@ int32_t qe_next_slot(const qe_layer*, uint32_t* slot_out);
  * dy, dx for dI).  Layer l's gradient slice is grad_buf_dev + offsets[l].  Every action is checked and committed on
  * the host exactly like the single calls; the kernels of the whole list are then issued behind ONE caller->execution
  * wait and ONE execution->caller event: in eager mode as plain launches, in graph mode as one captured graph (a list of more
- * than 64 launches: several, issued one after the other while the next is prepared) that is cached per (layers, actions)
+ * than 96 actions: several, issued one after the other while the next is prepared) that is cached per (layers, actions)
  * and replayed, with kernel-node parameters patched where pointers or the accumulate flag differ from the previous
  * replay.  dW runs on the execution stream here (QE_CTX_OVERLAP_DW does not apply).
  * Independent actions share launches, with bit-identical results (only the slot a tape lands in may differ from the
@@ -358,6 +358,8 @@ int32_t qe_next_slot(const qe_layer*, uint32_t* slot_out);
  * wait until a forward needs one of their slots, or no more are to come, or there are enough of them; those that are
  * ready then go out in one launch that adds their products up in microbatch order and writes the gradient slice once
  * (bit for bit what one accumulating launch per microbatch leaves there).  A round is issued as qe_run_together would.
+ * Where nothing that the list writes (outputs, gradient slices) overlaps anything else that it reads or writes, the layers of
+ * a unit do not wait for one another: a round takes all F and dI actions within the look-ahead whose own layer is ready.
  * With temp_dev, with step_window 1, or when the list admits no such plan, actions go one by one and only
  * consecutive dW actions of different layers share launches (as in qe_backward_dW_multi).
  * (The plan honours dependencies, not positions: an action listed before a predecessor that lies within the look-ahead
@@ -380,6 +382,12 @@ int32_t qe_step_run(qe_ctx* ctx, qe_layer* const* layers, uint32_t n_layers, con
  * qe_plan_step: the plan qe_step_run makes, as described above -- at most max_group F and dI actions and as many layers'
  * weight gradients in a round, of a layer up to max_sum microbatches, of all layers QE_STEP_MAX_PRODUCTS. */
 #define QE_STEP_MAX_PRODUCTS 32
+/* qe_plan_step_apart: the same for a list whose tensors do not overlap, without the order of a unit's layers: a round takes
+ * all of its actions that are ready (QE_APART_MAX_PRODUCTS products of weight gradients). */
+#define QE_APART_MAX_PRODUCTS 512
+int32_t qe_plan_step_apart(const qe_step_action* actions, uint32_t n_actions, uint32_t n_layers, uint32_t microbatches,
+                           const uint32_t* slots, const uint32_t* live_now, uint32_t window, uint32_t max_group,
+                           uint32_t max_sum, uint32_t* round_of_action, uint32_t* n_rounds_out);
 int32_t qe_plan_step(const qe_step_action* actions, uint32_t n_actions, uint32_t n_layers, uint32_t microbatches,
                      const uint32_t* slots, const uint32_t* live_now, uint32_t window, uint32_t max_group,
                      uint32_t max_sum, uint32_t* round_of_action, uint32_t* n_rounds_out);

@@ -159,6 +159,8 @@ _SIGNATURES = {
                                    C.POINTER(C.c_uint32), C.c_uint32, C.c_uint32, C.POINTER(C.c_uint32), C.POINTER(C.c_uint32)]),
     "qe_plan_step": (C.c_int32, [C.POINTER(qe_step_action), C.c_uint32, C.c_uint32, C.c_uint32, C.POINTER(C.c_uint32),
                                  C.POINTER(C.c_uint32), C.c_uint32, C.c_uint32, C.c_uint32, C.POINTER(C.c_uint32), C.POINTER(C.c_uint32)]),
+    "qe_plan_step_apart": (C.c_int32, [C.POINTER(qe_step_action), C.c_uint32, C.c_uint32, C.c_uint32, C.POINTER(C.c_uint32),
+                                 C.POINTER(C.c_uint32), C.c_uint32, C.c_uint32, C.c_uint32, C.POINTER(C.c_uint32), C.POINTER(C.c_uint32)]),
     "qe_run_together": (C.c_int32, [_P, C.POINTER(qe_action), C.c_uint32, _P, C.c_uint64, _P]),
     "qe_forward_chain": (C.c_int32, [C.POINTER(_P), C.c_uint32, C.c_uint32, C.c_uint64, _P, _P, _P, C.POINTER(qe_tape)]),
     "qe_backward_dI_chain": (C.c_int32, [C.POINTER(_P), C.POINTER(qe_tape), C.c_uint32, _P, _P, _P]),
@@ -534,8 +536,8 @@ def qe_gemm_fp8_group(problems, status, stream=None):
     _check(lib.qe_gemm_fp8_group(arr, n, _ptr(status), _stream(stream)))
 
 
-def plan_rounds(actions, n_layers, microbatches, slots, window, max_group=8, live_now=None, max_sum=None):
-    """qe_plan_rounds (host only), or qe_plan_step when max_sum is given.  actions: (kind name, layer, mb) triples; returns
+def plan_rounds(actions, n_layers, microbatches, slots, window, max_group=8, live_now=None, max_sum=None, apart=False):
+    """qe_plan_rounds (host only), or qe_plan_step (apart: qe_plan_step_apart) when max_sum is given.  actions: (kind name, layer, mb) triples; returns
     the rounds as lists of triples."""
     n = len(actions)
     arr = (qe_step_action * n)(*[qe_step_action(ACT[k], l, m, 0) for k, l, m in actions])
@@ -546,7 +548,7 @@ def plan_rounds(actions, n_layers, microbatches, slots, window, max_group=8, liv
     if max_sum is None:
         _check(lib.qe_plan_rounds(arr, n, n_layers, microbatches, sl, lv, window, max_group, rnd, C.byref(nr)))
     else:
-        _check(lib.qe_plan_step(arr, n, n_layers, microbatches, sl, lv, window, max_group, max_sum, rnd, C.byref(nr)))
+        _check((lib.qe_plan_step_apart if apart else lib.qe_plan_step)(arr, n, n_layers, microbatches, sl, lv, window, max_group, max_sum, rnd, C.byref(nr)))
     out = [[] for _ in range(nr.value)]
     for i, a in enumerate(actions):
         out[rnd[i]].append(tuple(a))

@@ -1,5 +1,5 @@
 // Amax-history reduction and scale update as device functions: by a whole block in the standalone commit kernel and in the
-// tail of a weight's cast (its last block), by one warp in the GEMM launches (X and G at a launch's start, where an earlier
+// tail of a weight's cast (its last block), by one warp or lane in the GEMM launches (X and G at a launch's start, where an earlier
 // kernel has completed the amax; Y by the last CTA of the launch that computes it).  No launch is spent on a commit.
 //   hist[c][count mod H] = amax;  scale_c = fp8_max / max(hist[c]) / 2^margin;  scale_inv_c = 1 / scale_c
 // The block form: 256 threads, 64 per tensor class, all four classes in parallel, one barrier.  The ring's maximum is kept
@@ -61,41 +61,60 @@ __device__ __forceinline__ void commit_classes(const CommitParams& p, int tid, u
   if (tid == 0 && p.bump_token) st->token += 1ull;
 }
 
-// The same commit of ONE class by one warp (class_mask has one bit: X or G at a GEMM launch's start, Y in its tail).
-// A grouped launch may carry sixteen problems, each committed by a warp of its own, side by side: a commit is a chain of
-// dependent global accesses, and one after the other the commits of a launch took as long as its tiles.  The code runs once
-// per launch, from cold instruction memory, so it is short: one loop for the rare ring scan, 16-byte loads over all lanes,
-// four in flight each (48 linears of 1024 x 1024: 13254 us a step; 13337 with the scan in two loops of eight loads, 13298
-// with eight lanes of 4-byte loads for each of four classes).  F, dI and dW of a 256 x 256 x 256 linear plus the boundary
-// take 55 us when no commit scans; when all three do, 60 us at 4096 entries (77 with the eight lanes) and the same as
-// without at 1024 (61).  Same values as commit_classes; the token is bumped atomically because two problems of one launch
-// may belong to the same layer (its forward and its input gradient of different microbatches).
-__device__ __forceinline__ void commit_class_warp(const CommitParams& p, int lane) {
-  DevState* st = p.st;
-  const int c = __ffs(p.class_mask) - 1;
-  uint32_t* h = reinterpret_cast<uint32_t*>(p.hist + (size_t)c * p.H);
-  const uint32_t cnt = __ldcg(&st->count[c]);
-  const uint32_t newest = p.amax_override ? (__float_as_uint(__ldcg(p.amax_override)) & 0x7fffffffu) : __ldcg(&st->pending_amax[c]);
-  const uint32_t wmax = __ldcg(&st->wmax[c]);
-  const uint32_t pos = cnt % p.H;
-  const uint32_t evicted = __ldcg(h + pos);
-  uint32_t m = newest >= wmax ? newest : wmax;
-  if (newest < wmax && evicted >= wmax) {  // the maximum leaves: scan what stays
-    m = newest;
-    auto take = [&](uint32_t i, uint32_t q) { m = max(m, i == pos ? 0u : q); };
-    const uint32_t head = min(p.H, (4u - ((uint32_t)(reinterpret_cast<uintptr_t>(h) >> 2) & 3u)) & 3u);  // up to a 16-byte boundary
-    const uint32_t vecs = (p.H - head) / 4, tail = p.H - head - 4 * vecs;
-    if ((uint32_t)lane < head) take((uint32_t)lane, __ldcg(h + lane));
-    if ((uint32_t)lane < tail) take(p.H - tail + (uint32_t)lane, __ldcg(h + p.H - tail + lane));
+// Largest entry of a ring without the one at `hole`, by one warp: 16-byte loads over all lanes, four in flight each.
+__device__ __forceinline__ uint32_t ring_max(const uint32_t* ring, uint32_t n, uint32_t hole, int lane) {
+  uint32_t top = 0;
+  auto take = [&](uint32_t i, uint32_t q) { top = max(top, i == hole ? 0u : q); };
+  const uint32_t head = min(n, (4u - ((uint32_t)(reinterpret_cast<uintptr_t>(ring) >> 2) & 3u)) & 3u);  // up to a 16-byte boundary
+  const uint32_t vecs = (n - head) / 4, tail = n - head - 4 * vecs;
+  if ((uint32_t)lane < head) take((uint32_t)lane, __ldcg(ring + lane));
+  if ((uint32_t)lane < tail) take(n - tail + (uint32_t)lane, __ldcg(ring + n - tail + lane));
 #pragma unroll 4
-    for (uint32_t v = (uint32_t)lane; v < vecs; v += 32) {
-      const uint32_t i = head + 4 * v;
-      const uint4 q = __ldcg(reinterpret_cast<const uint4*>(h + i));
-      take(i, q.x), take(i + 1, q.y), take(i + 2, q.z), take(i + 3, q.w);
-    }
-    m = __reduce_max_sync(0xffffffffu, m);
+  for (uint32_t v = (uint32_t)lane; v < vecs; v += 32) {
+    const uint32_t i = head + 4 * v;
+    const uint4 q = __ldcg(reinterpret_cast<const uint4*>(ring + i));
+    take(i, q.x), take(i + 1, q.y), take(i + 2, q.z), take(i + 3, q.w);
   }
-  if (lane == 0) {
+  return __reduce_max_sync(0xffffffffu, top);
+}
+
+// The same commit of ONE class (class_mask has one bit: X or G at a GEMM launch's start, Y in its tail) by one warp; EACH: of a
+// class per lane, for lanes with `active`.  A grouped launch may carry dozens of problems, all committed side by side by lanes
+// of the epilogue's warps: a commit is a chain of dependent global accesses, and one after the other the commits of a launch
+// took as long as its tiles.  The code runs once per launch, from cold instruction memory, so it is short, with one loop for
+// the rare ring scan, which a whole warp makes for one lane after the other (launches of one problem keep the form without
+// lanes: with it twelve chained linears of 256 x 256 took 1402 us a step, without it 1389).  F, dI and dW of a 256 x 256 x 256
+// linear plus the boundary take 55 us when no commit scans; when all three do, 60 us at 4096 entries and the same as without
+// at 1024.  Same values as commit_classes; the token is bumped atomically because two problems of one launch may belong to
+// the same layer (its forward and its input gradient of different microbatches).
+template <bool EACH>
+__device__ __forceinline__ void commit_class(const CommitParams& p, uint32_t class_mask, bool bump, bool active, int lane) {
+  DevState* st = p.st;
+  const int c = !EACH || active ? __ffs(class_mask) - 1 : 0;
+  uint32_t* h = reinterpret_cast<uint32_t*>(p.hist + (size_t)c * p.H);
+  const uint32_t H = p.H;
+  uint32_t cnt = 0, newest = 0, m = 0, pos = 0;
+  bool scan = false;
+  if (!EACH || active) {
+    cnt = __ldcg(&st->count[c]);
+    newest = p.amax_override ? (__float_as_uint(__ldcg(p.amax_override)) & 0x7fffffffu) : __ldcg(&st->pending_amax[c]);
+    const uint32_t wmax = __ldcg(&st->wmax[c]);
+    pos = cnt % H;
+    const uint32_t evicted = __ldcg(h + pos);
+    m = newest >= wmax ? newest : wmax;
+    scan = newest < wmax && evicted >= wmax;  // the maximum leaves: scan what stays
+  }
+  if (!EACH) {
+    if (scan) m = max(newest, ring_max(h, H, pos, lane));
+  } else {
+    for (uint32_t left = __ballot_sync(0xffffffffu, scan); left; left &= left - 1) {
+      const int who = __ffs(left) - 1;
+      const uint32_t* ring = reinterpret_cast<const uint32_t*>(__shfl_sync(0xffffffffu, (unsigned long long)h, who));
+      const uint32_t top = ring_max(ring, __shfl_sync(0xffffffffu, H, who), __shfl_sync(0xffffffffu, pos, who), lane);
+      if (lane == who) m = max(newest, top);
+    }
+  }
+  if (EACH ? active : lane == 0) {
     h[pos] = newest;
     st->count[c] = cnt + 1;
     st->pending_amax[c] = 0;
@@ -107,7 +126,7 @@ __device__ __forceinline__ void commit_class_warp(const CommitParams& p, int lan
       st->scale[c] = s;
       st->scale_inv[c] = __fdiv_rn(1.0f, s);
     }
-    if (p.bump_token) atomicAdd(&st->token, 1ull);
+    if (bump) atomicAdd(&st->token, 1ull);
   }
 }
 

@@ -371,9 +371,11 @@ int32_t qe_plan_rounds(const qe_step_action* actions, uint32_t n_actions, uint32
 
 // ---- issue plan of the whole-step call.  F and dI as in qe_plan_rounds (but the window counts F and dI units only, and
 // each layer sees its actions of a kind strictly in list order); dW actions wait and go out several microbatches at once.
-int32_t qe_plan_step(const qe_step_action* actions, uint32_t n_actions, uint32_t n_layers, uint32_t microbatches,
-                     const uint32_t* slots, const uint32_t* live_now, uint32_t window, uint32_t max_group,
-                     uint32_t max_sum, uint32_t* round_of_action, uint32_t* n_rounds_out) try {
+// chained: the layers of a unit feed one another, so that one of its actions at most is ready at a time; otherwise all of
+// them are whose own layer is ready.
+static int32_t plan_step(const qe_step_action* actions, uint32_t n_actions, uint32_t n_layers, uint32_t microbatches,
+                         const uint32_t* slots, const uint32_t* live_now, uint32_t window, uint32_t max_group,
+                         uint32_t max_sum, uint32_t max_products, bool chained, uint32_t* round_of_action, uint32_t* n_rounds_out) {
   if (!actions || !slots || !round_of_action || !n_rounds_out) return fail(QE_ERR_BAD_ARG, "null argument");
   if (n_actions == 0 || n_layers == 0 || microbatches == 0 || window == 0 || max_group == 0 || max_sum == 0) return fail(QE_ERR_BAD_ARG, "empty list or zero limit");
   const uint32_t M = microbatches;
@@ -395,6 +397,7 @@ int32_t qe_plan_step(const qe_step_action* actions, uint32_t n_actions, uint32_t
     lists[a.layer].of[a.kind].push_back(i);
   }
   constexpr uint32_t kNever = UINT32_MAX;
+  std::fill(round_of_action, round_of_action + n_actions, kNever);
   std::vector<uint32_t> f_round((size_t)n_layers * M, kNever), di_round((size_t)n_layers * M, kNever);
   std::vector<uint32_t> live(n_layers, 0), freed(n_layers, 0);
   for (uint32_t l = 0; live_now && l < n_layers; ++l) live[l] = live_now[l];
@@ -406,40 +409,43 @@ int32_t qe_plan_step(const qe_step_action* actions, uint32_t n_actions, uint32_t
     std::fill(blocked.begin(), blocked.end(), (uint8_t)0);
     for (size_t ui = first; ui < units.size() && ui < first + window && group < max_group; ++ui) {
       Unit& u = units[ui];
-      if (u.begin == u.end) continue;
-      const uint32_t i = u.begin;  // a unit walks its layers in list order: only this action can be ready
-      const qe_step_action& a = actions[i];
-      LayerLists& q = lists[a.layer];
-      if (q.of[a.kind][q.next[a.kind]] != i) continue;  // an earlier action of the kind on this layer comes first
-      // predecessors must have been issued in earlier rounds (same-kind ones of this layer too)
-      if (q.next[a.kind]) {
-        const uint32_t before = q.of[a.kind][q.next[a.kind] - 1];
-        if (round_of_action[before] == round) continue;
-      }
-      const size_t u_mb = (size_t)a.layer * M + a.mb;
-      if (a.kind == QE_ACT_F) {
-        if (f_round[u_mb] != kNever) return fail(QE_ERR_ORDER, "action %u: second forward of layer %u microbatch %u", i, a.layer, a.mb);
-        if (live[a.layer] >= slots[a.layer]) {
-          blocked[a.layer] = 1;
-          continue;
+      // (a chained unit walks its layers in list order: only its first action that is left can be ready)
+      const uint32_t end = chained ? std::min(u.begin + 1, u.end) : u.end;
+      for (uint32_t i = u.begin; i < end && group < max_group; ++i) {
+        if (round_of_action[i] != kNever) continue;
+        const qe_step_action& a = actions[i];
+        LayerLists& q = lists[a.layer];
+        if (q.of[a.kind][q.next[a.kind]] != i) continue;  // an earlier action of the kind on this layer comes first
+        // predecessors must have been issued in earlier rounds (same-kind ones of this layer too)
+        if (q.next[a.kind]) {
+          const uint32_t before = q.of[a.kind][q.next[a.kind] - 1];
+          if (round_of_action[before] == round) continue;
         }
-        f_round[u_mb] = round;
-        live[a.layer] += 1;
-      } else {
-        if (di_round[u_mb] != kNever) return fail(QE_ERR_ORDER, "action %u: second input gradient of layer %u microbatch %u", i, a.layer, a.mb);
-        if (f_round[u_mb] == kNever || f_round[u_mb] == round) continue;
-        di_round[u_mb] = round;
+        const size_t u_mb = (size_t)a.layer * M + a.mb;
+        if (a.kind == QE_ACT_F) {
+          if (f_round[u_mb] != kNever) return fail(QE_ERR_ORDER, "action %u: second forward of layer %u microbatch %u", i, a.layer, a.mb);
+          if (live[a.layer] >= slots[a.layer]) {
+            blocked[a.layer] = 1;
+            continue;
+          }
+          f_round[u_mb] = round;
+          live[a.layer] += 1;
+        } else {
+          if (di_round[u_mb] != kNever) return fail(QE_ERR_ORDER, "action %u: second input gradient of layer %u microbatch %u", i, a.layer, a.mb);
+          if (f_round[u_mb] == kNever || f_round[u_mb] == round) continue;
+          di_round[u_mb] = round;
+        }
+        q.next[a.kind] += 1;
+        round_of_action[i] = round;
+        ++group;
       }
-      q.next[a.kind] += 1;
-      round_of_action[i] = round;
-      u.begin += 1;
-      ++group;
+      while (u.begin < u.end && round_of_action[u.begin] != kNever) u.begin += 1;
     }
     // Weight gradients: those of a layer that are ready (dI in an earlier round) go out together when a forward needs
     // their slots, when there are max_sum of them, when no more are to come, or when nothing else can run.
     const bool idle = group == 0;
     uint32_t n_dw = 0, products = 0;
-    for (uint32_t l = 0; l < n_layers && n_dw < max_group && products < QE_STEP_MAX_PRODUCTS; ++l) {
+    for (uint32_t l = 0; l < n_layers && n_dw < max_group && products < max_products; ++l) {
       LayerLists& q = lists[l];
       const std::vector<uint32_t>& of = q.of[QE_ACT_DW];
       uint32_t ready = 0;
@@ -453,7 +459,7 @@ int32_t qe_plan_step(const qe_step_action* actions, uint32_t n_actions, uint32_t
       const bool need = blocked[l] || (live[l] >= slots[l] && q.next[QE_ACT_F] < q.of[QE_ACT_F].size());
       const bool last = q.next[QE_ACT_DW] + ready == of.size();
       if (!need && !last && ready < max_sum && !idle) continue;
-      if (ready > QE_STEP_MAX_PRODUCTS - products) ready = QE_STEP_MAX_PRODUCTS - products;
+      if (ready > max_products - products) ready = max_products - products;
       for (uint32_t j = 0; j < ready; ++j) round_of_action[of[q.next[QE_ACT_DW] + j]] = round;
       q.next[QE_ACT_DW] += ready;
       freed[l] = ready;
@@ -470,6 +476,20 @@ int32_t qe_plan_step(const qe_step_action* actions, uint32_t n_actions, uint32_t
   }
   *n_rounds_out = round;
   return QE_OK;
+}
+
+int32_t qe_plan_step(const qe_step_action* actions, uint32_t n_actions, uint32_t n_layers, uint32_t microbatches,
+                     const uint32_t* slots, const uint32_t* live_now, uint32_t window, uint32_t max_group,
+                     uint32_t max_sum, uint32_t* round_of_action, uint32_t* n_rounds_out) try {
+  return plan_step(actions, n_actions, n_layers, microbatches, slots, live_now, window, max_group, max_sum, QE_STEP_MAX_PRODUCTS,
+                   true, round_of_action, n_rounds_out);
+} QE_NO_MEMORY
+
+int32_t qe_plan_step_apart(const qe_step_action* actions, uint32_t n_actions, uint32_t n_layers, uint32_t microbatches,
+                           const uint32_t* slots, const uint32_t* live_now, uint32_t window, uint32_t max_group,
+                           uint32_t max_sum, uint32_t* round_of_action, uint32_t* n_rounds_out) try {
+  return plan_step(actions, n_actions, n_layers, microbatches, slots, live_now, window, max_group, max_sum, QE_APART_MAX_PRODUCTS,
+                   false, round_of_action, n_rounds_out);
 } QE_NO_MEMORY
 
 }  // extern "C"

@@ -299,14 +299,18 @@ __device__ __forceinline__ uint32_t snake_tile(uint32_t w, uint32_t first, uint3
 // other, so that one set of persistent CTAs packs them into common waves and the launch overhead is paid once.
 template <int NP, int NOPS>
 struct Problems {
-  static constexpr bool SUMS = NOPS > NP;  // problems may have several products
+  static constexpr bool ONE = NP == 1, SUMS = NOPS > NP;  // one problem; problems may have several products
   const GemmLaunchParams<NP, NOPS>& g;
   __device__ __forceinline__ uint32_t count() const { return NP == 1 ? 1u : g.n; }
   __device__ __forceinline__ uint32_t total_tiles() const { return g.tile_end[count() - 1]; }
-  __device__ __forceinline__ const GemmParams& at(uint32_t tile, uint32_t& local) const {
-    uint32_t i = 0, base = 0;
-    while (i + 1 < count() && tile >= g.tile_end[i]) base = g.tile_end[i++];
-    local = tile - base;
+  // `i`: the problem of an earlier tile of the same role (its tiles come in ascending order), from which the search goes on
+  __device__ __forceinline__ const GemmParams& at(uint32_t tile, uint32_t& i, uint32_t& local) const {
+    if (NP == 1) {
+      local = tile;
+      return g.prob[0];
+    }
+    while (i + 1 < count() && tile >= g.tile_end[i]) ++i;
+    local = tile - (i ? g.tile_end[i - 1] : 0u);
     return g.prob[i];
   }
   __device__ __forceinline__ const GemmOperands& operands(const GemmParams& p, uint32_t seg) const {
@@ -314,6 +318,7 @@ struct Problems {
   }
   __device__ __forceinline__ const GemmParams& first() const { return g.prob[0]; }
   __device__ __forceinline__ const CommitParams& commit(uint32_t i) const { return g.prob[i].commit; }
+  __device__ __forceinline__ uint32_t* ticket() const { return g.ticket; }
   __device__ __forceinline__ uint32_t* status_of(uint32_t i) const { return g.prob[i].status; }
 };
 
@@ -365,7 +370,7 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
 // per tile: which problem it belongs to (`p`), its index inside that problem and the problem's tiling
 #define QE_TILE_PROBLEM()                                                                                     \
   uint32_t local_tile;                                                                                        \
-  const GemmParams& p = ps.at(tile, local_tile);                                                              \
+  const GemmParams& p = ps.at(tile, at_problem, local_tile);                                                  \
   const uint32_t tile_n = p.tile_n, tiles_m = (p.M + TILE_M - 1) / TILE_M, tiles_n = (p.N + tile_n - 1) / tile_n; \
   const uint32_t num_kb = p.Kc / BK;                                                                          \
   const bool m_fastest = p.M <= p.N
@@ -411,6 +416,7 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
     // While the predecessor drains: pull the first ring-full of B tiles of this CTA's first tile towards L2.  A
     // prefetch moves no data into the SM, so it is harmless even if the predecessor is still writing that operand.
     const uint32_t tile = first_tile;
+    uint32_t at_problem = 0;
     QE_TILE_PROBLEM();
     uint32_t m0, n0;
     tile_coords<TILE_M>(local_tile, tiles_m, tiles_n, m_fastest, tile_n, m0, n0);
@@ -436,11 +442,8 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
     // The classes whose amax an EARLIER kernel reduced (the cast that made this GEMM's A operand) are committed here,
     // by an epilogue warp that has nothing to drain yet: nothing this launch computes reads their scale (its alphas
     // are snapshots), so only the output's class is left for the launch's tail.
-    CommitParams c = ps.commit(blockIdx.x);
-    if (c.st && c.early_mask) {
-      c.class_mask = c.early_mask;
-      commit_class_warp(c, lane);
-    }
+    const CommitParams& c = ps.commit(blockIdx.x);
+    if (c.st && c.early_mask) commit_class<false>(c, c.early_mask, c.bump_token != 0, true, lane);
   }
 
   // (The roles are one flat choice: with producer and issuer nested under a choice of their own, or written as lambdas, the
@@ -453,7 +456,7 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
     // ---------------------------------------------------------------- TMA producer
     if (lane == 0) {
       int s = 0;
-      uint32_t ph = 0;
+      uint32_t ph = 0, at_problem = 0;
       bool ok = true;
       for (uint32_t wave = 0, tile = first_tile; ok && tile < num_tiles; ++wave, tile = snake_tile(wave, first_tile, tile_step)) {
         QE_TILE_PROBLEM();
@@ -494,7 +497,7 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
     // ---------------------------------------------------------------- MMA issuer
     if (lane == 0 && rank == 0) {
       int s = 0;
-      uint32_t ph = 0, acc = 0, acc_ph = 0;
+      uint32_t ph = 0, acc = 0, acc_ph = 0, at_problem = 0;
       bool ok = true;
       for (uint32_t wave = 0, tile = first_tile; ok && tile < num_tiles; ++wave, tile = snake_tile(wave, first_tile, tile_step)) {
         QE_TILE_PROBLEM();
@@ -532,7 +535,7 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
     const int etid = (int)threadIdx.x - EPI_WARP0 * 32;
     const uint32_t epi_smem = epi_base + (uint32_t)(warp - EPI_WARP0) * EPI_BUF_BYTES;  // this warp's two output tiles
     uint32_t n_groups = 0;  // bulk-store groups this warp has committed (buffer parity)
-    uint32_t acc = 0, acc_ph = 0;
+    uint32_t acc = 0, acc_ph = 0, at_problem = 0;
     bool ok = true;
     const uint32_t tempty_leader0 = PAIR ? map_to_cta(tempty_bar(0), 0) : tempty_bar(0);
     const uint32_t tempty_leader1 = PAIR ? map_to_cta(tempty_bar(1), 0) : tempty_bar(1);
@@ -548,6 +551,8 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
       auto prefetch_next = [&] {  // the destination rows that this thread adds to in its next tile, towards L2
         const uint32_t tile = snake_tile(wave + 1, first_tile, tile_step);
         if (tile >= num_tiles) return;
+        uint32_t from = at_problem;
+        uint32_t& at_problem = from;
         QE_TILE_PROBLEM();
         (void)num_kb;
         if (p.nseg == 1 || p.epi != 2) return;
@@ -744,15 +749,16 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
     // Every epilogue thread of every CTA gets here (also after a timeout); the last CTA commits the scale state of
     // every problem that asks for it.  The commit needs the amax atomics only, so it runs while this CTA's last
     // bulk stores are still draining.
-    uint32_t* ticket = nullptr;
-    for (uint32_t i = 0; i < ps.count(); ++i)
-      if (!ticket && ps.commit(i).st && ps.commit(i).class_mask) ticket = &ps.commit(i).st->ticket;
-    if (ticket && last_block(ticket, gridDim.x, etid, last_flag, epi_bar_sync)) {
-      // one epilogue warp per problem, side by side
-      for (uint32_t i = (uint32_t)(warp - EPI_WARP0); i < ps.count(); i += EPI_WARPS) {
-        CommitParams c = ps.commit(i);
-        c.bump_token = 0;  // (counted by the early part)
-        if (c.st && c.class_mask) commit_class_warp(c, lane);
+    if (ps.ticket() && last_block(ps.ticket(), gridDim.x, etid, last_flag, epi_bar_sync)) {
+      // (the token is counted by the early part)
+      const uint32_t ew = (uint32_t)(warp - EPI_WARP0);
+      if (PS::ONE) {
+        if (ew == 0) commit_class<false>(ps.commit(0), ps.commit(0).class_mask, false, true, lane);
+      } else if (ew < ps.count()) {  // a lane per problem, dealt to the epilogue's warps
+        static_assert(kMaxSingles <= EPI_WARPS * 32 && kMaxProblems <= EPI_WARPS * 32, "a lane for every problem");
+        const uint32_t i = ew + EPI_WARPS * (uint32_t)lane;
+        const CommitParams& c = ps.commit(i < ps.count() ? i : 0u);
+        commit_class<true>(c, c.class_mask, false, i < ps.count() && c.st && c.class_mask, lane);
       }
     }
     // The bulk-store unit has read this warp's last tiles out of shared memory; that the bytes are in global memory
@@ -781,6 +787,7 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
 
 using OneParams = GemmLaunchParams<1, 1>;
 using GroupParams = GemmLaunchParams<8, 8>;
+using ManyParams = GemmLaunchParams<kMaxSingles, kMaxSingles>;
 using WideParams = GemmLaunchParams<kMaxProblems, kMaxOperands>;
 
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(threads_of(false), 1)
@@ -799,7 +806,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(threads_of(false), 1
   gemm_body<true>(Problems<8, 8>{g});
 }
 
-// More problems, or problems of several products each.  (The parameter block is three times as large.)
+// Up to fifty: what the kernel's parameter space holds.
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(threads_of(false), 1)
+    gemm_fp8_pair_many_kernel(const __grid_constant__ ManyParams g) {
+  gemm_body<true>(Problems<kMaxSingles, kMaxSingles>{g});
+}
+
+// Problems of several products each.  (The parameter block is three times as large.)
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(threads_of(true), 1)
     gemm_fp8_pair_wide_kernel(const __grid_constant__ WideParams g) {
   gemm_body<true>(Problems<kMaxProblems, kMaxOperands>{g});
@@ -875,7 +888,9 @@ Launch make_launch(const GemmDesc* probs, uint32_t n, uint32_t nops, int num_sms
   const uint32_t tile_m = alone ? BM : PAIR_M, ctas = alone ? 1u : 2u, most = (uint32_t)num_sms / ctas;
   const uint32_t w = choose_width(probs, n, (uint32_t)num_sms / 2u);  // (alone: 0, see one_cta)
   uint32_t tiles = 0, op = 0;
+  uint32_t* ticket = nullptr;
   for (uint32_t i = 0; i < n; ++i) {
+    if (!ticket && probs[i].commit.st && probs[i].commit.class_mask) ticket = &probs[i].commit.st->ticket;
     tiles += ceil_div(probs[i].M, tile_m) * ceil_div(probs[i].N, kTileWidths[w]);
     std::memcpy(at + offsetof(P, tile_end) + i * sizeof(uint32_t), &tiles, sizeof(tiles));
     const GemmParams p = problem_of(probs[i], w, op, tile_m);
@@ -887,6 +902,7 @@ Launch make_launch(const GemmDesc* probs, uint32_t n, uint32_t nops, int num_sms
     }
   }
   std::memcpy(at + offsetof(P, n), &n, sizeof(n));
+  std::memcpy(at + offsetof(P, ticket), &ticket, sizeof(ticket));
   l.func = func;
   l.grid = dim3(ctas * (tiles < most ? tiles : most), 1, 1);
   l.block = dim3(threads_of(NOPS > NP), 1, 1);
@@ -900,6 +916,7 @@ Launch make_any(const GemmDesc* probs, uint32_t n, uint32_t nops, int num_sms) {
     return make_launch<1, 1>(probs, n, nops, num_sms, alone ? (const void*)gemm_fp8_kernel : (const void*)gemm_fp8_pair_kernel, alone);
   }
   if (n <= 8 && nops == n) return make_launch<8, 8>(probs, n, nops, num_sms, (const void*)gemm_fp8_pair_group_kernel);
+  if (nops == n) return make_launch<kMaxSingles, kMaxSingles>(probs, n, nops, num_sms, (const void*)gemm_fp8_pair_many_kernel);
   return make_launch<kMaxProblems, kMaxOperands>(probs, n, nops, num_sms, (const void*)gemm_fp8_pair_wide_kernel);
 }
 
@@ -908,7 +925,7 @@ Launch make_any(const GemmDesc* probs, uint32_t n, uint32_t nops, int num_sms) {
 bool whole_row_tiles(uint32_t M) { return M % 256 == 0; }
 
 cudaError_t gemm_prepare() {
-  for (const void* f : {(const void*)gemm_fp8_kernel, (const void*)gemm_fp8_pair_kernel, (const void*)gemm_fp8_pair_group_kernel, (const void*)gemm_fp8_pair_wide_kernel}) {
+  for (const void* f : {(const void*)gemm_fp8_kernel, (const void*)gemm_fp8_pair_kernel, (const void*)gemm_fp8_pair_group_kernel, (const void*)gemm_fp8_pair_many_kernel, (const void*)gemm_fp8_pair_wide_kernel}) {
     const cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES);
     if (e != cudaSuccess) return e;
   }
@@ -917,11 +934,8 @@ cudaError_t gemm_prepare() {
 
 bool make_gemm_group(const GemmDesc* probs, uint32_t n, int num_sms, Launch* out) {
   uint32_t nops = 0;
-  for (uint32_t i = 0; i < n; ++i) {
-    if (!whole_row_tiles(probs[i].M)) return false;
-    nops += probs[i].nseg;
-  }
-  if (n < 2 || n > kMaxProblems || nops > kMaxOperands) return false;
+  for (uint32_t i = 0; i < n; ++i) nops += probs[i].nseg;
+  if (n < 2 || (nops == n ? n > kMaxSingles : n > kMaxProblems || nops > kMaxOperands)) return false;
   *out = make_any(probs, n, nops, num_sms);
   return true;
 }

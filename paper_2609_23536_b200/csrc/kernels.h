@@ -57,9 +57,11 @@ struct QuantParams {
 };
 
 
+constexpr uint32_t kMaxCasts = 128;  // of one launch
+template <int N>
 struct QuantMultiParams {
-  QuantParams q[8];
-  uint32_t block_end[8];       // cumulative block counts
+  QuantParams q[N];
+  uint32_t block_end[N];       // cumulative block counts
   uint32_t n;
   uint32_t pad[3];
 };
@@ -147,10 +149,12 @@ template <int NP, int NOPS>
 struct GemmLaunchParams {
   uint32_t n;
   uint32_t tile_end[NP];       // cumulative tile counts
+  uint32_t* ticket;            // counts the CTAs that are done, where a problem has a commit in the tail; else null
   GemmParams prob[NP];
   GemmOperands op[NOPS];
 };
-constexpr uint32_t kMaxProblems = 16, kMaxOperands = 40;  // of the largest launch
+constexpr uint32_t kMaxProblems = 16, kMaxOperands = 40;  // of a launch in which a problem has several products
+constexpr uint32_t kMaxSingles = 50;                      // problems of a launch whose problems have one each
 
 // ORs the status words of up to 64 layers into *out (first chunk: out = OR; later chunks: out |= OR).
 struct StatusGatherParams {
@@ -212,7 +216,7 @@ struct Launch {
     nbytes = sizeof(P);
   }
   // The whole block as the runtime wants it (valid as long as the launch and the buffer are).
-  struct Block { alignas(64) unsigned char bytes[20480]; };
+  struct Block { alignas(64) unsigned char bytes[32768]; };
   void* args_block(Block* tmp) const {
     if (params.size() == nbytes) return const_cast<unsigned char*>(params.data());
     __builtin_memcpy(tmp->bytes, params.data(), params.size());
@@ -221,7 +225,7 @@ struct Launch {
 };
 
 Launch make_quantize(const QuantParams& p);
-Launch make_quantize_multi(const QuantParams* casts, uint32_t n);  // 2..8 independent casts in one launch
+Launch make_quantize_multi(const QuantParams* casts, uint32_t n);  // 2..kMaxCasts independent casts in one launch
 Launch make_commit(const CommitParams& p);
 Launch make_status_gather(const StatusGatherParams& p);
 Launch make_amax_pass1(const AmaxParams& p);
@@ -229,9 +233,8 @@ Launch make_amax_pass2(const AmaxParams& p);
 Launch make_accumulate(const AccumParams& p);
 Launch make_arena_reduce(const ArenaReduceParams& p);
 Launch make_gemm(const GemmDesc& p, int num_sms);
-// One launch for n = 2..kMaxProblems GEMMs of kMaxOperands operand pairs at most (each may carry its own commit tail);
-// false if the group cannot be formed (a problem's M is not a multiple of 256), in which case the caller launches them
-// one by one.
+// One launch for n = 2..kMaxSingles GEMMs of one operand pair each, or 2..kMaxProblems of kMaxOperands pairs at most (each
+// may carry its own commit tail); false if there are more.
 bool make_gemm_group(const GemmDesc* probs, uint32_t n, int num_sms, Launch* out);
 uint32_t gemm_width(const GemmDesc* probs, uint32_t n, int num_sms);  // index of the tile width the launch of these will have
 cudaError_t gemm_prepare();  // opt in to the dynamic shared memory the GEMM needs (once per device)

@@ -124,15 +124,21 @@ __global__ void __launch_bounds__(kQuantThreads) quantize_kernel(const __grid_co
   }
 }
 
-// Two to eight independent casts in one launch (the X of forward units and the dY of input-gradient units that go out
-// together, the weights of a stage at the start of its step): the blocks are dealt to the casts one cast after the other.
-__global__ void __launch_bounds__(kQuantThreads) quantize_multi_kernel(const __grid_constant__ QuantMultiParams mp) {
+// Independent casts in one launch (the X of forward units and the dY of input-gradient units that go out together, the
+// weights of a stage at the start of its step): the blocks are dealt to the casts one cast after the other.
+template <int N>
+__global__ void __launch_bounds__(kQuantThreads) quantize_multi_kernel(const __grid_constant__ QuantMultiParams<N> mp) {
   __shared__ uint32_t wmax[kQuantThreads / 32];
   __shared__ uint32_t last_flag;
+  uint32_t which = 0, end = mp.n;  // the first cast that ends behind this block
+  while (which + 1 < end) {
+    const uint32_t mid = (which + end) / 2;
+    if (blockIdx.x >= mp.block_end[mid - 1]) which = mid;
+    else end = mid;
+  }
+  const uint32_t base = which ? mp.block_end[which - 1] : 0u;
   grid_dep_wait();
   grid_dep_launch();
-  uint32_t which = 0, base = 0;
-  while (which + 1 < mp.n && blockIdx.x >= mp.block_end[which]) base = mp.block_end[which++];
   const QuantParams& p = mp.q[which];
   const uint32_t b = blockIdx.x - base, bxn = p.cols / 64u;
   if (p.fmt == 0) quantize_block<0>(p, b % bxn, b / bxn, wmax);
@@ -144,8 +150,9 @@ __global__ void __launch_bounds__(kQuantThreads) quantize_multi_kernel(const __g
   }
 }
 
-Launch make_quantize_multi(const QuantParams* casts, uint32_t n) {
-  QuantMultiParams mp{};
+template <int N>
+static Launch make_multi(const QuantParams* casts, uint32_t n) {
+  QuantMultiParams<N> mp{};
   uint32_t blocks = 0;
   for (uint32_t i = 0; i < n; ++i) {
     mp.q[i] = casts[i];
@@ -154,11 +161,15 @@ Launch make_quantize_multi(const QuantParams* casts, uint32_t n) {
   }
   mp.n = n;
   Launch l;
-  l.func = (const void*)quantize_multi_kernel;
+  l.func = (const void*)quantize_multi_kernel<N>;
   l.grid = dim3(blocks, 1, 1);
   l.block = dim3(kQuantThreads, 1, 1);
   l.set(mp);
   return l;
+}
+
+Launch make_quantize_multi(const QuantParams* casts, uint32_t n) {
+  return n <= 8 ? make_multi<8>(casts, n) : make_multi<kMaxCasts>(casts, n);
 }
 
 Launch make_quantize(const QuantParams& p) {

@@ -189,7 +189,7 @@ int32_t qe_forward_dI_pair(qe_layer* Lf, uint32_t mb, uint64_t gen, const void* 
   add_dI(Lb, pb, dy, dx, ls, nullptr, 0, &g[1], &c[1]);
   ls.push_back(qe::make_quantize_multi(c, 2));  // both casts in one launch
   qe::Launch shared;
-  if (qe::make_gemm_group(g, 2, ctx->dev->num_sms, &shared)) {
+  if (qe::whole_row_tiles(g[0].M) && qe::whole_row_tiles(g[1].M) && qe::make_gemm_group(g, 2, ctx->dev->num_sms, &shared)) {
     ls.push_back(shared);
     ctx->stats.paired_f_di += 1;
   } else {  // T is an odd multiple of 128: one after the other
@@ -212,17 +212,14 @@ int32_t qe_forward_dI_pair(qe_layer* Lf, uint32_t mb, uint64_t gen, const void* 
 
 // ------------------------------------------------------------------------------------------------ independent actions
 namespace {
-constexpr uint32_t kMaxRound = QE_MAX_TOGETHER + QE_STEP_MAX_PRODUCTS;  // actions of a round of the whole-step call
-static_assert(2 * QE_MAX_TOGETHER <= qe::kMaxProblems && kMaxRound <= qe::kMaxOperands, "a round fits into one launch");
-
-struct TogetherPrep {
-  int32_t refresh[kMaxRound] = {}, acc[kMaxRound] = {};
-  uint32_t slot[kMaxRound] = {};
-  bool any_dw = false;
+// An action on its way to the device: what its contract check said.
+struct Prepared : qe_action {
+  int32_t refresh = 0, acc = 0;
+  uint32_t slot = 0;
 };
 
 // argument rules and every action's contract check; nothing is changed
-int32_t together_prepare(qe_ctx* ctx, const qe_action* acts, uint32_t n, float* grad, uint64_t grad_elems, TogetherPrep* pr) {
+int32_t together_prepare(qe_ctx* ctx, Prepared* acts, uint32_t n, float* grad, uint64_t grad_elems, bool* any_dw) {
   if (!ctx || !acts || n == 0 || n > QE_MAX_TOGETHER) return fail(QE_ERR_BAD_ARG, "null argument or bad count %u", n);
   for (uint32_t i = 0; i < n; ++i) {
     const qe_action& a = acts[i];
@@ -231,113 +228,144 @@ int32_t together_prepare(qe_ctx* ctx, const qe_action* acts, uint32_t n, float* 
       return fail(QE_ERR_BAD_ARG, "action %u: input / output null or misaligned", i);
     for (uint32_t j = 0; j < i; ++j)
       if (acts[j].layer == a.layer && acts[j].kind == a.kind) return fail(QE_ERR_BAD_ARG, "actions %u and %u: same kind on the same layer", j, i);
-    pr->any_dw |= a.kind == QE_ACT_DW;
+    *any_dw |= a.kind == QE_ACT_DW;
   }
-  if (pr->any_dw && !grad) return fail(QE_ERR_BAD_ARG, "gradient buffer is null");
+  if (*any_dw && !grad) return fail(QE_ERR_BAD_ARG, "gradient buffer is null");
   for (uint32_t i = 0; i < n; ++i) {
-    const qe_action& a = acts[i];
+    Prepared& a = acts[i];
     qe_layer* L = a.layer;
     int32_t st;
     if (a.kind == QE_ACT_F) {
-      st = qe_contract_forward_check(L->contract, a.mb, a.gen, &pr->refresh[i], &pr->slot[i]);
+      st = qe_contract_forward_check(L->contract, a.mb, a.gen, &a.refresh, &a.slot);
     } else if (a.kind == QE_ACT_DI) {
       st = qe_contract_dI_check(L->contract, a.tape);
-      pr->slot[i] = a.tape->ref.slot;
+      a.slot = a.tape->ref.slot;
     } else {
-      st = qe_contract_dW_check(L->contract, a.tape, (uint64_t)(uintptr_t)grad, grad_elems, a.grad_offset, (uint64_t)L->cfg.N * L->cfg.K, &pr->acc[i]);
-      pr->slot[i] = a.tape->ref.slot;
+      st = qe_contract_dW_check(L->contract, a.tape, (uint64_t)(uintptr_t)grad, grad_elems, a.grad_offset, (uint64_t)L->cfg.N * L->cfg.K, &a.acc);
+      a.slot = a.tape->ref.slot;
     }
     if (st != QE_OK) return st;
   }
   return QE_OK;
 }
 
+// The GEMMs gemms[0..n) in as few launches as hold them, each launch with about as many.
+void push_gemms(qe_ctx* ctx, const qe::GemmDesc* gemms, uint32_t n, std::vector<qe::Launch>& ls) {
+  while (n) {
+    // what the next launch takes: an equal share of what is left, as far as its operand pairs fit
+    uint32_t nops = 0, share = 0;
+    bool sums = false;
+    for (uint32_t i = 0; i < n; ++i) nops += gemms[i].nseg, sums |= gemms[i].nseg > 1;
+    const uint32_t most = sums ? qe::kMaxProblems : qe::kMaxSingles, launches = std::max((n + most - 1) / most, sums ? (nops + qe::kMaxOperands - 1) / qe::kMaxOperands : 1u);
+    const uint32_t want = (n + launches - 1) / launches;
+    nops = 0;
+    while (share < want && (!sums || nops + gemms[share].nseg <= qe::kMaxOperands)) nops += gemms[share++].nseg;
+    qe::Launch l;
+    if (share >= 2 && qe::make_gemm_group(gemms, share, ctx->dev->num_sms, &l)) ls.push_back(std::move(l));
+    else for (uint32_t i = 0; i < share; ++i) ls.push_back(qe::make_gemm(gemms[i], ctx->dev->num_sms));
+    gemms += share;
+    n -= share;
+  }
+}
+
 // the launches: the casts in one launch, then every GEMM of whole 256-row tiles in one launch; weight gradients of
 // several microbatches of one layer (whole-step call only) become one GEMM that adds their products up
-// (refresh != null: the weight casts are collected there instead of being queued)
-int32_t together_build(qe_ctx* ctx, const qe_action* acts, uint32_t n, const TogetherPrep& pr, float* grad,
-                       std::vector<qe::Launch>& ls, Fnv* h, std::vector<qe::QuantParams>* refresh = nullptr) {
-  qe::GemmDesc g[2 * QE_MAX_TOGETHER];
-  const qe_layer* owner[2 * QE_MAX_TOGETHER];
-  qe::QuantParams casts[QE_MAX_TOGETHER];
-  std::vector<qe::GemmDesc> singles;
-  std::vector<const qe_layer*> single_owner;
-  uint32_t ng = 0, n_chain = 0, n_dw = 0, n_casts = 0;
+// (refresh != null: the weight casts are collected there instead of being queued; any_rows: half-filled last row tiles share
+// launches too)
+int32_t together_build(qe_ctx* ctx, const Prepared* acts, uint32_t n, float* grad, std::vector<qe::Launch>& ls, Fnv* h,
+                       std::vector<qe::QuantParams>* refresh = nullptr, bool any_rows = false) {
+  std::vector<qe::GemmDesc> chain, dw, singles;  // F and dI; weight gradients; those that go out one by one
+  std::vector<const qe_layer*> dw_owner, single_owner;
+  std::vector<qe::QuantParams> casts;
+  chain.reserve(n);
+  casts.reserve(n);
   for (int pass = 0; pass < 2; ++pass) {  // F and dI first (others wait for them), the weight gradients' tiles after theirs
     for (uint32_t i = 0; i < n; ++i) {
-      const qe_action& a = acts[i];
+      const Prepared& a = acts[i];
       qe_layer* L = a.layer;
       if ((a.kind == QE_ACT_DW) != (pass == 1)) continue;
-      qe::GemmDesc gp;
-      if (a.kind == QE_ACT_F) {
-        if (L->dw_pending[pr.slot[i]]) {
-          QE_CUDA(cudaStreamWaitEvent(ctx->exec_stream, L->ev_dw[pr.slot[i]], 0));
-          L->dw_pending[pr.slot[i]] = false;
-        }
-        if (pr.refresh[i] && refresh) refresh->push_back(refresh_params(L));
-        else if (pr.refresh[i]) add_refresh(L, ls);
-        add_forward(L, pr.slot[i], a.in_dev, a.out_dev, ls, nullptr, 0, &gp, &casts[n_casts++]);
-      } else if (a.kind == QE_ACT_DI) {
-        add_dI(L, pr.slot[i], a.in_dev, a.out_dev, ls, nullptr, 0, &gp, &casts[n_casts++]);
-      } else {
-        gp = dW_gemm(L, pr.slot[i], grad + a.grad_offset, pr.acc[i], nullptr);
-      }
-      const bool paired = qe::whole_row_tiles(gp.M);
-      if (paired) (a.kind == QE_ACT_DW ? n_dw : n_chain) += 1;
-      qe::GemmDesc* sum = nullptr;  // this layer's weight gradient of an earlier microbatch, which takes this one in
-      if (a.kind == QE_ACT_DW) {
-        for (uint32_t j = n_chain; paired && j < ng; ++j)
-          if (owner[j] == L) sum = &g[j];
-        for (size_t j = 0; !paired && j < singles.size(); ++j)
-          if (single_owner[j] == L && singles[j].epi != 0) sum = &singles[j];
-      }
-      if (sum) {
-        sum->ops[sum->nseg++] = gp.ops[0];
-      } else if (paired) {
-        owner[ng] = L;
-        g[ng++] = gp;
-      } else {
-        singles.push_back(gp);  // a half-filled last row tile: a launch of its own
-        single_owner.push_back(L);
-      }
       if (h) {
         h->mix(&a.kind, sizeof(a.kind));
         h->mix(&a.layer, sizeof(a.layer));
-        h->mix(&pr.slot[i], sizeof(uint32_t));
-        h->mix(&pr.refresh[i], sizeof(int32_t));
+        h->mix(&a.slot, sizeof(uint32_t));
+        h->mix(&a.refresh, sizeof(int32_t));
+      }
+      if (a.kind == QE_ACT_DW) {
+        const qe::GemmDesc gp = dW_gemm(L, a.slot, grad + a.grad_offset, a.acc, nullptr);
+        const bool apart = !any_rows && !qe::whole_row_tiles(gp.M);  // a half-filled last row tile: a launch of its own
+        std::vector<qe::GemmDesc>& to = apart ? singles : dw;
+        std::vector<const qe_layer*>& owner = apart ? single_owner : dw_owner;
+        const auto sum = std::find(owner.begin(), owner.end(), L);  // this layer's of an earlier microbatch takes this one in
+        if (sum != owner.end()) {
+          qe::GemmDesc& g = to[sum - owner.begin()];
+          g.ops[g.nseg++] = gp.ops[0];
+        } else {
+          to.push_back(gp);
+          owner.push_back(L);
+        }
+        continue;
+      }
+      qe::GemmDesc gp;
+      qe::QuantParams cast;
+      if (a.kind == QE_ACT_F) {
+        if (L->dw_pending[a.slot]) {
+          QE_CUDA(cudaStreamWaitEvent(ctx->exec_stream, L->ev_dw[a.slot], 0));
+          L->dw_pending[a.slot] = false;
+        }
+        if (a.refresh && refresh) refresh->push_back(refresh_params(L));
+        else if (a.refresh) add_refresh(L, ls);
+        add_forward(L, a.slot, a.in_dev, a.out_dev, ls, nullptr, 0, &gp, &cast);
+      } else {
+        add_dI(L, a.slot, a.in_dev, a.out_dev, ls, nullptr, 0, &gp, &cast);
+      }
+      casts.push_back(cast);
+      if (any_rows || qe::whole_row_tiles(gp.M)) {
+        chain.push_back(gp);
+      } else {
+        singles.push_back(gp);
+        single_owner.push_back(nullptr);
       }
     }
   }
   // longest tiles first (their contraction length decides a tile's duration): the launch's last, partial wave is then
   // made of short tiles.  The weight gradients (contraction over T only) stay behind the others.
-  std::stable_sort(g, g + n_chain, [](const qe::GemmDesc& x, const qe::GemmDesc& y) { return x.Kc > y.Kc; });
-  std::stable_sort(g + n_chain, g + ng, [](const qe::GemmDesc& x, const qe::GemmDesc& y) { return x.Kc * x.nseg > y.Kc * y.nseg; });
-  if (n_casts >= 2) ls.push_back(qe::make_quantize_multi(casts, n_casts));  // all casts of the call in one launch
-  else if (n_casts == 1) ls.push_back(qe::make_quantize(casts[0]));
-  for (const qe::GemmDesc& gp : singles) ls.push_back(qe::make_gemm(gp, ctx->dev->num_sms));
-  qe::Launch shared;
-  if (ng >= 2 && qe::make_gemm_group(g, ng, ctx->dev->num_sms, &shared)) {
-    ls.push_back(shared);
-    ctx->stats.grouped_dw += n_dw;
-    ctx->stats.paired_f_di += n_chain >= 1 ? 1 : 0;
-  } else {
-    for (uint32_t i = 0; i < ng; ++i) ls.push_back(qe::make_gemm(g[i], ctx->dev->num_sms));
+  std::stable_sort(chain.begin(), chain.end(), [](const qe::GemmDesc& x, const qe::GemmDesc& y) { return x.Kc > y.Kc; });
+  std::stable_sort(dw.begin(), dw.end(), [](const qe::GemmDesc& x, const qe::GemmDesc& y) { return x.Kc * x.nseg > y.Kc * y.nseg; });
+  for (size_t i = 0; i < casts.size(); i += qe::kMaxCasts) {  // all casts of the call in one launch
+    const uint32_t m = (uint32_t)std::min<size_t>(qe::kMaxCasts, casts.size() - i);
+    ls.push_back(m > 1 ? qe::make_quantize_multi(&casts[i], m) : qe::make_quantize(casts[i]));
   }
+  for (const qe::GemmDesc& gp : singles) ls.push_back(qe::make_gemm(gp, ctx->dev->num_sms));
+  if (chain.size() + dw.size() >= 2) {
+    ctx->stats.grouped_dw += dw.size();
+    ctx->stats.paired_f_di += !chain.empty() ? 1 : 0;
+  }
+  // one launch where it holds them all; else weight gradients, which add products up, have launches of their own
+  uint32_t nops = (uint32_t)chain.size();
+  bool sums = false;
+  for (const qe::GemmDesc& g : dw) nops += g.nseg, sums |= g.nseg > 1;
+  const size_t all = chain.size() + dw.size();
+  if (sums ? all <= qe::kMaxProblems && nops <= qe::kMaxOperands : all <= qe::kMaxSingles) {
+    chain.insert(chain.end(), dw.begin(), dw.end());
+    dw.clear();
+  }
+  push_gemms(ctx, chain.data(), (uint32_t)chain.size(), ls);
+  push_gemms(ctx, dw.data(), (uint32_t)dw.size(), ls);
   return QE_OK;
 }
 
 // Forward commits first: a forward's tape slot was chosen by its check, on the state before the call, and the kernels
 // used it; a weight-gradient commit of the same layer releases a slot and must not come in between.
-int32_t together_commit(const qe_action* acts, uint32_t n, float* grad, const TogetherPrep& pr) {
+int32_t together_commit(const Prepared* acts, uint32_t n, float* grad) {
   for (uint32_t kind = QE_ACT_F; kind <= QE_ACT_DW; ++kind) {
     for (uint32_t i = 0; i < n; ++i) {
-      const qe_action& a = acts[i];
+      const Prepared& a = acts[i];
       if (a.kind != kind) continue;
       qe_layer* L = a.layer;
       int32_t st;
       if (a.kind == QE_ACT_F) {
         st = qe_contract_forward_commit(L->contract, a.mb, a.tape);
-        if (st == QE_OK && a.tape->ref.slot != pr.slot[i]) return fail(QE_ERR_ORDER, "forward committed to slot %u, ran in slot %u", a.tape->ref.slot, pr.slot[i]);
+        if (st == QE_OK && a.tape->ref.slot != a.slot) return fail(QE_ERR_ORDER, "forward committed to slot %u, ran in slot %u", a.tape->ref.slot, a.slot);
       } else if (a.kind == QE_ACT_DI) {
         st = qe_contract_dI_commit(L->contract, a.tape);
       } else {
@@ -355,9 +383,9 @@ int32_t together_commit(const qe_action* acts, uint32_t n, float* grad, const To
 static int32_t run_together_impl(qe_ctx* ctx, qe_action* acts, uint32_t n, float* grad, uint64_t grad_elems, void* caller_stream,
                                  int host) {
   if (!ctx || !acts || n == 0 || n > QE_MAX_TOGETHER) return fail(QE_ERR_BAD_ARG, "null argument or bad count %u", n);
-  qe_action dev[QE_MAX_TOGETHER];
+  Prepared dev[QE_MAX_TOGETHER];
   for (uint32_t i = 0; i < n; ++i) {
-    dev[i] = acts[i];
+    static_cast<qe_action&>(dev[i]) = acts[i];
     if (!host || acts[i].kind > QE_ACT_DI || !acts[i].layer) continue;
     qe_layer* L = acts[i].layer;
     if (!L->x_stage) return fail(QE_ERR_BAD_ARG, "action %u: layer was created without host_io", i);
@@ -365,8 +393,8 @@ static int32_t run_together_impl(qe_ctx* ctx, qe_action* acts, uint32_t n, float
     dev[i].in_dev = acts[i].kind == QE_ACT_F ? L->x_stage : L->dy_stage;
     dev[i].out_dev = acts[i].kind == QE_ACT_F ? L->y_stage : L->dx_stage;
   }
-  TogetherPrep pr;
-  int32_t st = together_prepare(ctx, dev, n, grad, grad_elems, &pr);  // check (every action, before anything runs)
+  bool any_dw = false;
+  int32_t st = together_prepare(ctx, dev, n, grad, grad_elems, &any_dw);  // check (every action, before anything runs)
   if (st != QE_OK) return st;
   cudaStream_t caller = (cudaStream_t)caller_stream;
   Handshake handshake(ctx, caller);
@@ -378,14 +406,14 @@ static int32_t run_together_impl(qe_ctx* ctx, qe_action* acts, uint32_t n, float
       const size_t bytes = 2ull * c.T * (acts[i].kind == QE_ACT_F ? c.K : c.N);
       if ((st = host_upload(ctx, const_cast<void*>(dev[i].in_dev), acts[i].in_dev, bytes, caller)) != QE_OK) return st;
     }
-  if (pr.any_dw && ctx->dw_stream) {  // weight gradients issued earlier on the second stream accumulate into the same buffer
+  if (any_dw && ctx->dw_stream) {  // weight gradients issued earlier on the second stream accumulate into the same buffer
     QE_CUDA(cudaEventRecord(ctx->ev_dw_in, ctx->dw_stream));
     QE_CUDA(cudaStreamWaitEvent(ctx->exec_stream, ctx->ev_dw_in, 0));
   }
   std::vector<qe::Launch> ls;
   Fnv h;
   h.mix("together", 9);
-  if ((st = together_build(ctx, dev, n, pr, grad, ls, &h)) != QE_OK) return st;
+  if ((st = together_build(ctx, dev, n, grad, ls, &h)) != QE_OK) return st;
   if ((st = run_keyed(ctx, h.key, ls)) != QE_OK) return st;  // ... run ...
   if (host)
     for (uint32_t i = 0; i < n; ++i) {
@@ -396,9 +424,9 @@ static int32_t run_together_impl(qe_ctx* ctx, qe_action* acts, uint32_t n, float
     }
   if (ctx->dw_stream)
     for (uint32_t i = 0; i < n; ++i)
-      if (acts[i].kind == QE_ACT_DI) QE_CUDA(cudaEventRecord(acts[i].layer->ev_di[pr.slot[i]], ctx->exec_stream));
+      if (acts[i].kind == QE_ACT_DI) QE_CUDA(cudaEventRecord(acts[i].layer->ev_di[dev[i].slot], ctx->exec_stream));
   if ((st = handshake.out()) != QE_OK) return st;
-  return together_commit(dev, n, grad, pr);  // ... commit (the tapes are written through the callers' pointers)
+  return together_commit(dev, n, grad);  // ... commit (the tapes are written through the callers' pointers)
 }
 
 int32_t qe_run_together(qe_ctx* ctx, qe_action* acts, uint32_t n, float* grad, uint64_t grad_elems, void* caller_stream) try {
@@ -410,6 +438,60 @@ int32_t qe_run_together_host(qe_ctx* ctx, qe_action* acts, uint32_t n, float* gr
 } QE_NO_MEMORY
 
 // ------------------------------------------------------------------------------------------------ whole-step call
+namespace {
+struct Bytes { uintptr_t lo, hi; };
+
+// Whether nothing that the list's actions write -- outputs, gradient slices, workspaces -- overlaps anything else they read or
+// write: then only a layer's own order binds them, and the layers of a unit need not wait for one another.  (A null pointer: no.)
+bool tensors_apart(qe_layer* const* layers, uint32_t n_layers, const qe_step_action* actions, uint32_t n_actions, uint32_t M,
+                   const qe_step_io* io, const float* grad, const uint64_t* offsets) {
+  // runs of one kind of tensor in the order of the list: mostly ascending as they come
+  std::vector<Bytes> run[5];  // x, dy (read), weights (read), y, dx and the rest (written)
+  enum { kX, kDY, kY, kDX, kRest };
+  for (uint32_t i = 0; i < n_actions; ++i) {
+    const qe_step_action& a = actions[i];
+    if (a.kind > QE_ACT_DW || a.layer >= n_layers || a.mb >= M) return false;
+    if (a.kind == QE_ACT_DW) continue;
+    const qe_layer_config& c = layers[a.layer]->cfg;
+    const qe_step_io& b = io[(size_t)a.layer * M + a.mb];
+    const uintptr_t tk = 2ull * c.T * c.K, tn = 2ull * c.T * c.N;
+    const uintptr_t in = (uintptr_t)(a.kind == QE_ACT_F ? b.x_dev : b.dy_dev), out = (uintptr_t)(a.kind == QE_ACT_F ? b.y_dev : b.dx_dev);
+    if (!in || !out) return false;
+    run[a.kind == QE_ACT_F ? kX : kDY].push_back({in, in + (a.kind == QE_ACT_F ? tk : tn)});
+    run[a.kind == QE_ACT_F ? kY : kDX].push_back({out, out + (a.kind == QE_ACT_F ? tn : tk)});
+  }
+  std::vector<Bytes> weights;
+  for (uint32_t l = 0; l < n_layers; ++l) {
+    const qe_layer* L = layers[l];
+    const uintptr_t nk = (uintptr_t)L->cfg.N * L->cfg.K, w = (uintptr_t)L->cfg.weight_dev, g = (uintptr_t)(grad + offsets[l]);
+    weights.push_back({w, w + 2 * nk});
+    run[kRest].push_back({(uintptr_t)L->st, (uintptr_t)L->st + L->ws_bytes});
+    if (grad) run[kRest].push_back({g, g + 4 * nk});
+  }
+  run[kX].insert(run[kX].end(), weights.begin(), weights.end());
+  const auto less = [](const Bytes& a, const Bytes& b) { return a.lo < b.lo; };
+  for (std::vector<Bytes>& r : run)
+    if (!std::is_sorted(r.begin(), r.end(), less)) std::sort(r.begin(), r.end(), less);
+  // sweep by address: what is written may not begin before all that came before it has ended, nor anything before all that
+  // is written has
+  size_t at[5] = {};
+  uintptr_t read_to = 0, written_to = 0;
+  for (;;) {
+    int best = -1;
+    for (int k = 0; k < 5; ++k)
+      if (at[k] < run[k].size() && (best < 0 || run[k][at[k]].lo < run[best][at[best]].lo)) best = k;
+    if (best < 0) return true;
+    const Bytes& b = run[best][at[best]++];
+    const bool write = best >= kY;
+    if (b.lo < written_to || (write && b.lo < read_to)) return false;
+    (write ? written_to : read_to) = std::max(write ? written_to : read_to, b.hi);
+  }
+}
+
+// Actions of a round of a list whose tensors are apart: forwards and input gradients for two launches.
+constexpr uint32_t kApartGroup = 2 * qe::kMaxSingles;
+}  // namespace
+
 int32_t qe_step_run(qe_ctx* ctx, qe_layer* const* layers, uint32_t n_layers, const qe_step_action* actions,
                     uint32_t n_actions, uint32_t M, const qe_step_io* io, float* grad, uint64_t grad_elems,
                     const uint64_t* offsets, float* temp, void* caller_stream) try {
@@ -437,7 +519,6 @@ int32_t qe_step_run(qe_ctx* ctx, qe_layer* const* layers, uint32_t n_layers, con
     list_key.mix(actions, sizeof(qe_step_action) * n_actions);
     list_key.mix(&M, sizeof(M));
   }
-  constexpr size_t kPieceLaunches = 64;
   auto run_piece = [&](const std::vector<qe::Launch>& piece, bool as_graph) -> int32_t {
     if (pieces++ == 0) {
       const int32_t hs = handshake.in();
@@ -485,7 +566,14 @@ int32_t qe_step_run(qe_ctx* ctx, qe_layer* const* layers, uint32_t n_layers, con
   std::sort(by_address.begin(), by_address.end());
   const bool repeated = std::adjacent_find(by_address.begin(), by_address.end()) != by_address.end();
   const uint32_t fit = 8192u / T_max, max_sum = repeated || fit < 3 ? 1u : std::min(qe::kMaxSegments, fit);
+  // Where the list's tensors are apart (qe_plan_step_apart), a round takes every layer that is ready, not one of each unit: a
+  // unit of n layers is one round instead of n, and half-filled last row tiles share its launches (of the tiles' rows a
+  // sixteenth at 1920 tokens, a quarter at 384; launches of their own cost more).  us a step, layers in turn / at once:
+  // 48 linears of 1024 x 1024 at 512 tokens 13250 / 5340; six of 1536 x 1536 at 1152 tokens (odd) 889 / 351; eight of 2048 x
+  // 2048 at 768 1316 / 871; a 4096 / 11008 layer at 256 1776 / 1619; blocks of hidden 1024 at 3072 970 / 853, 2048 at 2048
+  // 2900 / 2795; hidden 4096 at 4096, which the power limit bounds, the same.
   std::vector<std::vector<uint32_t>> rounds;  // indices into actions[]
+  bool apart = false;
   if (!temp && ctx->step_window > 1) {
     std::vector<uint32_t> slots(n_layers), live(n_layers), round_of(n_actions);
     for (uint32_t l = 0; l < n_layers; ++l) {
@@ -493,7 +581,10 @@ int32_t qe_step_run(qe_ctx* ctx, qe_layer* const* layers, uint32_t n_layers, con
       live[l] = layers[l]->contract->live_tapes();
     }
     uint32_t n_rounds = 0;
-    if ((max_sum > 1 && qe_plan_step(actions, n_actions, n_layers, M, slots.data(), live.data(), ctx->step_window,
+    apart = !repeated && tensors_apart(layers, n_layers, actions, n_actions, M, io, grad, offsets) &&
+            qe_plan_step_apart(actions, n_actions, n_layers, M, slots.data(), live.data(), ctx->step_window, kApartGroup, max_sum,
+                               round_of.data(), &n_rounds) == QE_OK;
+    if (apart || (max_sum > 1 && qe_plan_step(actions, n_actions, n_layers, M, slots.data(), live.data(), ctx->step_window,
                                      QE_MAX_TOGETHER, max_sum, round_of.data(), &n_rounds) == QE_OK) ||
         qe_plan_rounds(actions, n_actions, n_layers, M, slots.data(), live.data(), ctx->step_window, QE_MAX_TOGETHER,
                        round_of.data(), &n_rounds) == QE_OK) {
@@ -501,24 +592,24 @@ int32_t qe_step_run(qe_ctx* ctx, qe_layer* const* layers, uint32_t n_layers, con
       for (uint32_t i = 0; i < n_actions; ++i) rounds[round_of[i]].push_back(i);
     }
   }
-  // Weights that are to be cast anew: the casts of a piece (below) go out together ahead of it, eight to a launch, instead of
-  // one by one between the rounds of the warm-up.
+  // Weights that are to be cast anew: the casts of a piece (below) go out together ahead of it instead of one by one between
+  // the rounds of the warm-up.
   std::vector<qe::QuantParams> refresh;
   auto put_refresh = [&] {
     std::vector<qe::Launch> first;
-    for (size_t i = 0; i < refresh.size(); i += 8) {
-      const uint32_t n = (uint32_t)std::min<size_t>(8, refresh.size() - i);
+    for (size_t i = 0; i < refresh.size(); i += qe::kMaxCasts) {
+      const uint32_t n = (uint32_t)std::min<size_t>(qe::kMaxCasts, refresh.size() - i);
       first.push_back(n > 1 ? qe::make_quantize_multi(&refresh[i], n) : qe::make_quantize(refresh[i]));
     }
     ls.insert(ls.begin(), std::make_move_iterator(first.begin()), std::make_move_iterator(first.end()));
     refresh.clear();
   };
+  uint32_t waiting = 0;  // actions in the piece that is being put together
+  std::vector<Prepared> acts;
   for (size_t r = 0; r < rounds.size() && st == QE_OK; ++r) {
     // check -> commit per action (all F first: a slot that a dW of the round releases is not theirs to take), then the
     // launches of those that passed
-    qe_action acts[kMaxRound];
-    TogetherPrep pr;
-    uint32_t na = 0;
+    acts.clear();
     for (size_t i = 0; repeated && i < rounds[r].size(); ++i)
       for (size_t j = 0; j < i; ++j) {
         const qe_step_action &a = actions[rounds[r][j]], &b = actions[rounds[r][i]];
@@ -533,44 +624,49 @@ int32_t qe_step_run(qe_ctx* ctx, qe_layer* const* layers, uint32_t n_layers, con
         const size_t u = (size_t)a.layer * M + a.mb;
         qe_layer* L = layers[a.layer];
         const uint64_t slice = (uint64_t)L->cfg.N * L->cfg.K;
+        Prepared p;
         const void* in = a.kind == QE_ACT_F ? io[u].x_dev : io[u].dy_dev;
         void* out = a.kind == QE_ACT_F ? io[u].y_dev : io[u].dx_dev;
         if (a.kind == QE_ACT_DW) {
           st = !grad ? fail(QE_ERR_BAD_ARG, "gradient buffer is null")
-                     : qe_contract_dW_check(L->contract, &tapes[u], (uint64_t)(uintptr_t)grad, grad_elems, offsets[a.layer], slice, &pr.acc[na]);
-          pr.slot[na] = tapes[u].ref.slot;
+                     : qe_contract_dW_check(L->contract, &tapes[u], (uint64_t)(uintptr_t)grad, grad_elems, offsets[a.layer], slice, &p.acc);
+          p.slot = tapes[u].ref.slot;
           if (st == QE_OK) st = qe_contract_dW_commit(L->contract, &tapes[u], (uint64_t)(uintptr_t)grad, offsets[a.layer], slice);
         } else if (!in || !out || (((uintptr_t)in | (uintptr_t)out) & 15u)) {
           st = fail(QE_ERR_BAD_ARG, "input / output null or misaligned");
         } else if (a.kind == QE_ACT_F) {
-          st = qe_contract_forward_check(L->contract, a.mb, L->contract->e_W, &pr.refresh[na], &pr.slot[na]);
+          st = qe_contract_forward_check(L->contract, a.mb, L->contract->e_W, &p.refresh, &p.slot);
           if (st == QE_OK) st = qe_contract_forward_commit(L->contract, a.mb, &tapes[u]);
         } else {
           st = qe_contract_dI_check(L->contract, &tapes[u]);
-          pr.slot[na] = tapes[u].ref.slot;
+          p.slot = tapes[u].ref.slot;
           if (st == QE_OK) st = qe_contract_dI_commit(L->contract, &tapes[u]);
         }
         if (st != QE_OK) {
           k = gi;
           break;
         }
-        acts[na++] = qe_action{a.kind, a.mb, 0, L, in, out, &tapes[u], offsets[a.layer]};
+        static_cast<qe_action&>(p) = qe_action{a.kind, a.mb, 0, L, in, out, &tapes[u], offsets[a.layer]};
+        acts.push_back(p);
       }
     }
     char why[512];  // (a build can only fail on a CUDA error, which then is the one to report)
     if (st != QE_OK) std::snprintf(why, sizeof(why), "%s", qe_last_error());
-    const int32_t built = na ? together_build(ctx, acts, na, pr, grad, ls, nullptr, &refresh) : QE_OK;
+    const int32_t built = acts.empty() ? QE_OK : together_build(ctx, acts.data(), (uint32_t)acts.size(), grad, ls, nullptr, &refresh, apart);
     if (st != QE_OK) st = fail(st, "%s", why);
     else if (built != QE_OK) {
       st = built;
       k = rounds[r][0];
     }
-    // In graph mode a long list goes out in pieces, each a graph of its own, so that the device works on one while the
-    // host builds the next (48 linears, 32 microbatches: 3.4 of 16.4 ms were host time ahead of the one launch).
-    if (st == QE_OK && ctx->exec_mode == QE_EXEC_GRAPH && ls.size() >= kPieceLaunches && r + 1 < rounds.size()) {
+    // A long list goes out in pieces (in graph mode each a graph of its own), so that the device works on one while the host
+    // prepares the next: a first one soon, later ones so long that the gaps between graphs do not count (48 linears, 32
+    // microbatches: 3.4 of 16.4 ms were host time ahead of the one launch).
+    waiting += (uint32_t)acts.size();
+    if (st == QE_OK && waiting >= (pieces ? 384u : 96u) && r + 1 < rounds.size()) {
       put_refresh();
       run_status = run_piece(ls, true);
       ls.clear();
+      waiting = 0;
       if (run_status != QE_OK) break;
     }
   }

@@ -51,12 +51,13 @@ class Stage:
 
     def __init__(self, lib, shapes, T=256, M=2, slots=2, mode=0, window=4, flags=0, host_io=False, exec_stream=None):
         self.lib, self.M, self.T, self.shapes = lib, M, T, shapes
-        self.ctx, self.keep, self.layers = C.c_void_p(), [], []
+        self.ctx, self.keep, self.layers, self.weights = C.c_void_p(), [], [], []
         cfg = qe.qe_ctx_config(exec_mode=mode, device=0, exec_stream=exec_stream, flags=flags, step_window=window)
         assert lib.qe_ctx_create(C.byref(cfg), C.byref(self.ctx)) == 0
         for u, (K, N) in enumerate(shapes):
+            self.weights.append(self.buffer(2 * N * K))
             lc = qe.qe_layer_config(T=T, K=K, N=N, history_len=4, margin=0, slots=slots, unit=u, host_io=int(host_io),
-                                    weight_dev=self.buffer(2 * N * K))
+                                    weight_dev=self.weights[-1])
             need = C.c_uint64()
             assert lib.qe_layer_workspace_bytes(C.byref(lc), C.byref(need)) == 0
             h = C.c_void_p()
@@ -71,8 +72,9 @@ class Stage:
         self.keep.append(b)
         return (C.addressof(b) + 255) // 256 * 256
 
-    def step(self, actions, layers=None, stream=CALLER):
-        """qe_step_run over (kind, layer index, microbatch) triples; the status."""
+    def step(self, actions, layers=None, stream=CALLER, apart=False):
+        """qe_step_run over (kind, layer index, microbatch) triples; the status.  apart: every unit has tensors of its own (a
+        function of the layer and the microbatch: which buffers it has); otherwise a layer's outputs are its inputs."""
         idx = list(range(len(self.layers))) if layers is None else layers
         n = len(idx)
         hs = (C.c_void_p * n)(*[self.layers[i].value for i in idx])
@@ -82,7 +84,7 @@ class Stage:
             K, N = self.shapes[i]
             x, y = self.buffer(2 * self.T * K), self.buffer(2 * self.T * N)
             for m in range(self.M):
-                io[l * self.M + m] = qe.qe_step_io(x, y, y, x)
+                io[l * self.M + m] = qe.qe_step_io(*(apart(l, m) if apart else (x, y, y, x)))
         offs = (C.c_uint64 * n)(*[self.offsets[i] for i in idx])
         return self.lib.qe_step_run(self.ctx, hs, n, acts, len(actions), self.M, io, self.grad, self.elems, offs, None, stream)
 

@@ -777,3 +777,32 @@ def test_dW_multi_of_many_linears_equals_per_layer_calls_bitwise(qe, n):
     assert np.array_equal(g0, g1) and all(state_equal(a, b) for a, b in zip(s0, s1))
     launches = 1 + (-(-n // 4) if n <= 8 else 1)  # the odd linear by itself, the others of every four (more than eight: of all) together
     assert st0["kernels_launched"] - st1["kernels_launched"] == 2 * M * (n - launches)
+
+
+@pytest.mark.parametrize("T,n,slots", [(384, 53, 4), (256, 9, 2)])
+def test_step_of_linears_that_do_not_feed_one_another_equals_single_actions_bitwise(qe, T, n, slots):
+    """More than fifty linears (two launches of forwards and input gradients, two of sums) and few; half-filled row tiles of tokens and
+    of features; inputs whose maxima fall, so that lanes of one warp scan their rings."""
+    M, steps = 4, 2
+    shapes = [((256, 384, 512)[j % 3], (256, 640)[j % 2]) for j in range(n)]
+    s = sched(M, 2, 1)
+    acts = _actions(s, n)
+    slots = max(slots, peak_live(s))
+    assert max(map(len, qe.plan_rounds(acts, n, M, slots, 4, 100, max_sum=8, apart=True))) >= min(2 * n, 100)
+    got = []
+    for window in (1, 4):
+        ctx = qe.Context(1, step_window=window)
+        layers = [qe.Layer(ctx, T, K, N, 3, j % 2, slots, inputs.weights("AP", 0, j, N, K).to(DEV), unit=j) for j, (K, N) in enumerate(shapes)]
+        offs, total = inputs.grad_offsets([("l", K, N) for K, N in shapes])
+        X = [[(inputs.activations("AP", 0, 0, j, m, T, K) * 0.5 ** ((m + j) % 5)).to(DEV) for j, (K, N) in enumerate(shapes)] for m in range(M)]
+        dY = [[(inputs.upstream_grads("AP", 0, 0, j, m, T, N) * 0.5 ** ((2 * m + j) % 5)).to(DEV) for j, (K, N) in enumerate(shapes)] for m in range(M)]
+        Y = [[torch.zeros((T, N), dtype=torch.bfloat16, device=DEV) for K, N in shapes] for m in range(M)]
+        dX = [[torch.zeros((T, K), dtype=torch.bfloat16, device=DEV) for K, N in shapes] for m in range(M)]
+        grad = torch.full((total,), 3.0, device=DEV)
+        plan = qe.StepPlan(ctx, layers, acts, M, X, Y, dY, dX, grad, offs)
+        for _ in range(steps):
+            plan.run()
+            qe.optimizer_boundary_all(layers, M)
+        got.append((_snapshot(layers, Y, dX, grad), ctx.stats()["kernels_launched"]))
+    _same_snapshot(got[0][0], got[1][0])
+    assert got[1][1] < got[0][1] / 4

@@ -226,3 +226,36 @@ def test_step_sums_weight_gradients_where_three_products_fit(lib, tokens, sums):
     assert sum(int(w[5]) for w in words) == len(acts)
     assert any(int(w[5]) > int(w[3]) for w in words) == sums
     s.close()
+
+
+def test_step_takes_all_layers_of_a_unit_at_once_only_where_its_tensors_are_apart(lib):
+    """Forty linears in one round, cast by one launch, their GEMMs in two; as soon as one tensor that an action writes overlaps
+    what another reads or writes, or a weight, or a gradient, the layers go one after the other."""
+    n, M, K = 40, 2, 256
+    s = fake_runtime.Stage(lib, [(K, K)] * n, M=M, slots=M, window=4)
+    size = 2 * s.T * K
+    base = s.buffer(4 * n * M * size)
+    own = lambda l, m: [base + ((l * M + m) * 4 + j) * size for j in range(4)]  # noqa: E731
+    acts = [a for a in _actions(M, n)]
+
+    def casts(io):
+        lib.fake_reset()
+        assert s.step(acts, apart=io) == 0
+        for h in s.layers:
+            assert lib.qe_optimizer_boundary(h, M) == 0
+        return max(int(w.split()[3]) for w in lib.fake_log().decode().splitlines() if " cast " in w)
+
+    assert casts(own) == 2 * n  # the second forward and the first input gradient of every layer; the weights' casts are n
+    words = [w.split() for w in lib.fake_log().decode().splitlines() if " gemm " in w]
+    assert max(int(w[3]) for w in words) <= 50 and sum(int(w[5]) for w in words) == 3 * n * M
+    where = {"y on another x": (3, 1, 7, 0, 0), "dx on another dy": (3, 1, 7, 0, 2), "y on another y": (3, 1, 7, 1, 1), "dx on its own x": (3, 3, 3, 0, 0)}
+    for name, (l, j, l2, m2, j2) in where.items():
+        def io(a, b):
+            t = own(a, b)
+            if (a, b) == (l, 0):
+                t[j] = own(l2, m2)[j2] + (0 if l2 == l else size - 16)
+            return t
+        assert casts(io) < 2 * n, name
+    for name, at in (("weight", s.weights[9]), ("gradient", s.grad + 4 * s.offsets[5])):
+        assert casts(lambda a, b: own(a, b)[:1] + [at - size + 16] + own(a, b)[2:] if (a, b) == (3, 0) else own(a, b)) < 2 * n, name
+    s.close()

@@ -152,3 +152,31 @@ def test_step_plan_refuses_repeated_and_malformed_actions(qe):
         with pytest.raises(qe.QEError) as e:
             qe.plan_rounds(bad, 1, 1, 2, 4, 8, max_sum=8)
         assert e.value.code == code
+
+
+@pytest.mark.parametrize("M,w,d,extra", [(4, 1, 0, 0), (8, 3, 3, 0), (6, 2, 1, 2), (32, 3, 3, 0)])
+@pytest.mark.parametrize("n,group,sums", [(1, 8, 1), (5, 100, 8), (48, 100, 2), (48, 20, 4)])
+def test_step_plan_of_layers_that_do_not_feed_one_another(qe, M, w, d, extra, n, group, sums):
+    s = sched(M, w, d)
+    slots = peak_live(s) + extra
+    rounds = qe.plan_rounds(_actions(s, n), n, M, slots, 6, group, max_sum=sums, apart=True)
+    assert sorted(x for g in rounds for x in g) == sorted(_actions(s, n))
+    when = {x: r for r, g in enumerate(rounds) for x in g}
+    live = [0] * n
+    for r, g in enumerate(rounds):
+        chain = [x for x in g if x[0] != "dW"]
+        assert len(chain) <= group and len({(a, l) for a, l, m in chain}) == len(chain)
+        for a, l, m in g:
+            if a == "F":
+                live[l] += 1
+                assert live[l] <= slots and (m == 0 or when["F", l, m - 1] < r)
+            elif a == "dI":
+                assert when["F", l, m] < r and (m == 0 or when["dI", l, m - 1] < r)
+            else:
+                assert when["dI", l, m] < r and (m == 0 or when["dW", l, m - 1] <= r)
+        for l in range(n):
+            ms = [m for a, k, m in g if a == "dW" and k == l]
+            assert len(ms) <= sums and ms == list(range(ms[0], ms[0] + len(ms))) if ms else True
+            live[l] -= len(ms)
+    if n == 5 and (w, d) == (3, 3):  # a unit is a round: the last forward in round M - 1 at the earliest
+        assert when["F", 4, M - 1] <= M
