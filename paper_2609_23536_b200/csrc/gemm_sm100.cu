@@ -4,9 +4,10 @@
 //
 // Structure: persistent clusters of two CTAs on neighbouring SMs, 320 or 384 threads each, that compute one tile of 256 rows
 // and 256, 128 or 64 columns together with tcgen05.mma.cta_group::2:
-//   warp 0      TMA producer: cp.async.bulk.tensor 2D tiles into a six-stage shared-memory ring; per 128-byte K block
-//               each CTA loads its own 128 rows of A and its own half of the tile's B rows
-//   warp 1      allocates tensor memory, then one lane of the even CTA issues tcgen05.mma (256 x tile_n x 32 per
+//   warp 0      TMA producer: cp.async.bulk.tensor boxes into a shared-memory ring (six stages of a 128-byte K block, or four
+//               of two blocks for tiles of 128 or 64 columns); each CTA loads its own 128 rows of A and its own half of the
+//               tile's B rows
+//   warp 1      allocates tensor memory, then one elected lane of the even CTA issues tcgen05.mma (256 x tile_n x 32 per
 //               instruction) and tcgen05.commit, which multicasts stage-free / accumulator-ready arrivals to both CTAs
 //   8 warps     epilogue: tcgen05.ld the CTA's 128 x tile_n FP32 accumulator (two warps per 32-lane quadrant, half of
 //               the columns each) in 32 x 32 blocks, scale, write each block into a swizzled per-warp shared-memory
@@ -52,20 +53,29 @@ namespace {
 
 constexpr uint32_t BM = 128, BK = 128;  // rows per CTA; bytes (= FP8 elements) per stage along the contraction
 constexpr uint32_t ACC_COLS = 256;      // tensor-memory columns between the two accumulators (the widest tile)
-constexpr int UMMA_K = 32;
+constexpr uint32_t UMMA_K = 32;
 constexpr uint32_t A_BYTES = BM * BK;
 // CTAs that work on one tile, and what follows from it.
 template <bool PAIR>
 struct Form {
   static constexpr uint32_t CTAS = PAIR ? 2 : 1;
   static constexpr uint32_t TILE_M = CTAS * BM;  // rows of D per tile
-  // A and this CTA's rows of B: at most 128 in a pair, 256 alone.  (Nine stages of 20 KB measured no faster than six at 64
-  // columns: the ring's latency is covered.)
-  static constexpr uint32_t STAGE_BYTES = PAIR ? 2 * A_BYTES : 3 * A_BYTES;
-  static constexpr int STAGES = PAIR ? 6 : 4;
 };
+// The ring of operand stages: A and this CTA's rows of B, for one K block of 128 bytes (tiles of 256 columns) or two of them
+// (narrower tiles of a pair).  A stage costs the producer about 270 clocks and the issuer of the MMAs about 130 whatever its size
+// (barrier operations; 45 to 90 for another load), while the MMAs of a K block take 240 to 260 clocks at up to 128 columns: with
+// stages of one K block, tiles of 64 columns ran at 387 clocks a block, now at 339 (256 x 2048 x 8192: 15.9 -> 14.1 us).  There
+// shared memory bounds them: 20 KB written and 20 to 24 KB read a block at 128 bytes a clock.
 constexpr uint32_t RING_BYTES = 12 * A_BYTES;
-static_assert(Form<true>::STAGES * Form<true>::STAGE_BYTES == RING_BYTES && Form<false>::STAGES * Form<false>::STAGE_BYTES == RING_BYTES, "");
+constexpr int MAX_STAGES = 6;
+template <bool PAIR>
+struct Ring {
+  uint32_t blocks, stages, stage_bytes;  // K blocks of a stage, stages, bytes of one
+  __device__ __forceinline__ explicit Ring(uint32_t tile_n)
+      : blocks(PAIR && tile_n < 256u ? 2u : 1u), stages(PAIR && tile_n == 256u ? 6u : 4u), stage_bytes(RING_BYTES / stages) {}
+  __device__ __forceinline__ uint32_t b_offset() const { return blocks * A_BYTES; }
+};
+static_assert(RING_BYTES / 4 >= 2 * A_BYTES + 2 * 64 * BK && RING_BYTES / 4 >= 3 * A_BYTES && RING_BYTES / 6 >= 2 * A_BYTES, "");
 constexpr uint32_t TMEM_COLS = 512;
 constexpr uint32_t EPI_BUF_BYTES = 4096;                     // per epilogue warp: one FP32 or two bf16 32 x 32 output tiles
                                                              // (1 KB-aligned, swizzled) that the bulk-store unit reads
@@ -142,23 +152,31 @@ __device__ __forceinline__ void cluster_sync_all() {
   asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
-// TMA load whose completion is credited to a barrier that may live in the peer CTA of the pair.
-__device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap* map, uint32_t bar, int c0, int c1) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cta.global.tile.mbarrier::complete_tx::bytes.cta_group::2 [%0], [%1, {%3, %4}], [%2];"
-      ::"r"(dst), "l"(map), "r"(bar), "r"(c0), "r"(c1)
-      : "memory");
-}
-__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, uint32_t bar, int c0, int c1) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cta.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
-      ::"r"(dst), "l"(map), "r"(bar), "r"(c0), "r"(c1)
-      : "memory");
-}
+// TMA load of a box of an operand; in a pair its completion may be credited to a barrier of the peer CTA.
 template <bool PAIR>
-__device__ __forceinline__ void tma_load(uint32_t dst, const CUtensorMap* map, uint32_t bar, int c0, int c1) {
-  if (PAIR) tma_load_2d_pair(dst, map, bar, c0, c1);
-  else tma_load_2d(dst, map, bar, c0, c1);
+__device__ __forceinline__ void tma_load(uint32_t dst, const CUtensorMap* map, uint32_t bar, int c0, int c1, int c2) {
+  if (PAIR)
+    asm volatile(
+        "cp.async.bulk.tensor.3d.shared::cta.global.tile.mbarrier::complete_tx::bytes.cta_group::2 [%0], [%1, {%3, %4, %5}], [%2];"
+        ::"r"(dst), "l"(map), "r"(bar), "r"(c0), "r"(c1), "r"(c2)
+        : "memory");
+  else
+    asm volatile(
+        "cp.async.bulk.tensor.3d.shared::cta.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];"
+        ::"r"(dst), "l"(map), "r"(bar), "r"(c0), "r"(c1), "r"(c2)
+        : "memory");
+}
+// One lane of a converged warp, the same one every time.  The producer's and the issuer's loops run on whole warps, so that
+// addresses and descriptors stay in uniform registers, and this lane issues: on one lane of a divergent warp the same loops
+// took 65 clocks an MMA instead of 48 (64 columns) and twice as long a load (8192 x 256 x 2048: 21.1 us, now 15.9).
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile(
+      "{\n\t.reg .pred q;\n\t"
+      "elect.sync _|q, 0xffffffff;\n\t"
+      "selp.u32 %0, 1, 0, q;\n\t}"
+      : "=r"(p));
+  return p != 0;
 }
 __device__ __forceinline__ void tc_commit_pair(uint32_t bar) {  // arrives on `bar` in both CTAs of the pair
   asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
@@ -198,8 +216,8 @@ __device__ __forceinline__ void tc_mma_f8(uint32_t d_tmem, uint64_t adesc, uint6
   else tc_mma_f8_one(d_tmem, adesc, bdesc, idesc, accumulate);
 }
 
-__device__ __forceinline__ void tma_prefetch_2d(const CUtensorMap* map, int c0, int c1) {
-  asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global.tile [%0, {%1, %2}];" ::"l"(map), "r"(c0), "r"(c1) : "memory");
+__device__ __forceinline__ void tma_prefetch(const CUtensorMap* map, int c0, int c1, int c2) {
+  asm volatile("cp.async.bulk.prefetch.tensor.3d.L2.global.tile [%0, {%1, %2, %3}];" ::"l"(map), "r"(c0), "r"(c1), "r"(c2) : "memory");
 }
 
 // Bulk tensor store of a shared-memory tile (issued by one lane), with group tracking.
@@ -344,27 +362,27 @@ __device__ __forceinline__ void ld_row32(const float* src, float* v) {
 // ------------------------------------------------------------------------------------------------ kernel
 template <bool PAIR, class PS>
 __device__ __forceinline__ void gemm_body(const PS& ps) {
-  constexpr uint32_t CTAS = Form<PAIR>::CTAS, TILE_M = Form<PAIR>::TILE_M, STAGE_BYTES = Form<PAIR>::STAGE_BYTES;
-  constexpr int STAGES = Form<PAIR>::STAGES;
+  constexpr uint32_t CTAS = Form<PAIR>::CTAS, TILE_M = Form<PAIR>::TILE_M;
   constexpr bool SUMS = PS::SUMS;
   constexpr int EPI_WARP0 = SUMS ? 4 : 2;  // first epilogue warp
   extern __shared__ uint8_t smem_raw[];
   const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
-  const uint32_t epi_base = smem_base + STAGES * STAGE_BYTES;  // 1 KB-aligned
+  const uint32_t epi_base = smem_base + RING_BYTES;  // 1 KB-aligned
   const uint32_t bar_base = epi_base + 8 * EPI_BUF_BYTES;
-  // barrier block: full[STAGES], empty[STAGES], tmem_full[2], tmem_empty[2], then tmem address + abort flag
-  auto full_bar = [&](int s) { return bar_base + 8u * s; };
-  auto empty_bar = [&](int s) { return bar_base + 8u * (STAGES + s); };
-  auto tfull_bar = [&](int a) { return bar_base + 8u * (2 * STAGES + a); };
-  auto tempty_bar = [&](int a) { return bar_base + 8u * (2 * STAGES + 2 + a); };
+  // barrier block: full[MAX_STAGES], empty[MAX_STAGES], tmem_full[2], tmem_empty[2], then tmem address + abort flag
+  auto full_bar = [&](uint32_t s) { return bar_base + 8u * s; };
+  auto empty_bar = [&](uint32_t s) { return bar_base + 8u * (MAX_STAGES + s); };
+  auto tfull_bar = [&](int a) { return bar_base + 8u * (2 * MAX_STAGES + a); };
+  auto tempty_bar = [&](int a) { return bar_base + 8u * (2 * MAX_STAGES + 2 + a); };
   uint8_t* gen_base = smem_raw + (smem_base - smem_u32(smem_raw));
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(gen_base + STAGES * STAGE_BYTES + 8 * EPI_BUF_BYTES + 8 * (2 * STAGES + 4));
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(gen_base + RING_BYTES + 8 * EPI_BUF_BYTES + 8 * (2 * MAX_STAGES + 4));
   volatile uint32_t* abort_flag = tmem_slot + 1;
   uint32_t* last_flag = tmem_slot + 2;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = PAIR ? cluster_ctarank() : 0u;  // position in the CTA pair; rank 0 issues the MMAs
   const uint32_t num_tiles = ps.total_tiles();
+  const Ring<PAIR> ring(ps.first().tile_n);  // (one tile width per launch)
   const uint32_t first_tile = blockIdx.x / CTAS, tile_step = gridDim.x / CTAS;
   uint32_t* const status = ps.first().status;
 // per tile: which problem it belongs to (`p`), its index inside that problem and the problem's tiling
@@ -382,7 +400,7 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
     asm volatile("prefetch.tensormap [%0];" ::"l"(&q.tmD) : "memory");
   }
   if (threadIdx.x == 0) {
-    for (int s = 0; s < STAGES; ++s) {
+    for (uint32_t s = 0; s < MAX_STAGES; ++s) {
       mbar_init(full_bar(s), 1);
       mbar_init(empty_bar(s), 1);
     }
@@ -422,13 +440,8 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
     tile_coords<TILE_M>(local_tile, tiles_m, tiles_n, m_fastest, tile_n, m0, n0);
     const int rb = (int)(n0 + rank * (tile_n / 2));
     const CUtensorMap* tmB = &ps.operands(p, 0).tmB;
-    for (uint32_t kb = 0; kb < num_kb && kb < (uint32_t)STAGES; ++kb) {
-      const int ka = (int)(kb * BK);
-      for (int b = 0; b < (PAIR ? 1 : 2); ++b) {
-        if (p.b_mn) tma_prefetch_2d(tmB, rb + b * (int)BM, ka);
-        else tma_prefetch_2d(tmB, ka, rb + b * (int)BM);
-      }
-    }
+    for (uint32_t kb = 0; kb < num_kb && kb < ring.blocks * ring.stages; kb += ring.blocks)
+      for (int b = 0; b < (PAIR ? 1 : 2); ++b) tma_prefetch(tmB, p.b_mn ? rb + b * (int)BM : 0, p.b_mn ? 0 : rb + b * (int)BM, (int)kb);
   }
   // Everything above (barriers, tensor memory) touched no data a predecessor produces and may overlap the previous
   // kernel's tail; operands, scales and the destination may come from it, so wait for it here.
@@ -454,75 +467,81 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
   }
   if (warp == 0) {
     // ---------------------------------------------------------------- TMA producer
-    if (lane == 0) {
-      int s = 0;
-      uint32_t ph = 0, at_problem = 0;
-      bool ok = true;
-      for (uint32_t wave = 0, tile = first_tile; ok && tile < num_tiles; ++wave, tile = snake_tile(wave, first_tile, tile_step)) {
-        QE_TILE_PROBLEM();
-        uint32_t m0, n0;
-        tile_coords<TILE_M>(local_tile, tiles_m, tiles_n, m_fastest, tile_n, m0, n0);
-        const int ra = (int)(m0 + rank * BM), rb = (int)(n0 + rank * (tile_n / 2));
-        for (uint32_t seg = 0; ok && seg < (SUMS ? p.nseg : 1u); ++seg) {
-          const GemmOperands& op = ps.operands(p, seg);
-          const CUtensorMap *tmA = &op.tmA, *tmB = &op.tmB;
-          for (uint32_t kb = 0; kb < num_kb; ++kb) {
-            if (!(ok = mbar_wait(empty_bar(s), ph ^ 1u, abort_flag, status, ERR_PRODUCER))) break;
-            const uint32_t a_dst = smem_base + s * STAGE_BYTES, b_dst = a_dst + A_BYTES;
-            // both CTAs of a pair credit the even CTA's barrier, which expects the bytes of the whole pair
-            if (rank == 0) mbar_expect_tx(full_bar(s), CTAS * A_BYTES + tile_n * BK);
+    const bool elected = elect_one();
+    uint32_t s = 0, ph = 0, at_problem = 0;
+    bool ok = true;
+    for (uint32_t wave = 0, tile = first_tile; ok && tile < num_tiles; ++wave, tile = snake_tile(wave, first_tile, tile_step)) {
+      QE_TILE_PROBLEM();
+      uint32_t m0, n0;
+      tile_coords<TILE_M>(local_tile, tiles_m, tiles_n, m_fastest, tile_n, m0, n0);
+      // contraction-major operand: box = 128 K-bytes x rows x blocks at (0, row, block); MN-major operand (stored as [Kc, rows]):
+      // box = row-bytes x 128 K-rows x blocks at (row, 0, block).  Either way 128 bytes per row and block land in shared memory.
+      const int ra = (int)(m0 + rank * BM), rb = (int)(n0 + rank * (tile_n / 2));
+      const int a0 = p.a_mn ? ra : 0, a1 = p.a_mn ? 0 : ra, b0 = p.b_mn ? rb : 0, b1 = p.b_mn ? 0 : rb;
+      // both CTAs of a pair credit the even CTA's barrier, which expects the bytes of the whole pair (blocks beyond the
+      // contraction are filled with zeros and counted)
+      const uint32_t bytes = ring.blocks * (CTAS * A_BYTES + tile_n * BK);
+      for (uint32_t seg = 0; ok && seg < (SUMS ? p.nseg : 1u); ++seg) {
+        const GemmOperands& op = ps.operands(p, seg);
+        const CUtensorMap *tmA = &op.tmA, *tmB = &op.tmB;
+        for (uint32_t kb = 0; kb < num_kb; kb += ring.blocks) {
+          if (!(ok = mbar_wait(empty_bar(s), ph ^ 1u, abort_flag, status, ERR_PRODUCER))) break;
+          const uint32_t a_dst = smem_base + s * ring.stage_bytes, b_dst = a_dst + ring.b_offset();
+          if (elected) {
+            if (rank == 0) mbar_expect_tx(full_bar(s), bytes);
             const uint32_t bar = PAIR ? map_to_cta(full_bar(s), 0) : full_bar(s);
-            // contraction-major operand: box = 128 K-bytes x rows at (k, row); MN-major operand (stored as [Kc, rows]):
-            // box = row-bytes x 128 K-rows at (row, k).  Either way 128 bytes per row land in shared memory.
-            const int ka = (int)(kb * BK);
-            if (p.a_mn) tma_load<PAIR>(a_dst, tmA, bar, ra, ka);
-            else tma_load<PAIR>(a_dst, tmA, bar, ka, ra);
+            tma_load<PAIR>(a_dst, tmA, bar, a0, a1, (int)kb);
+            tma_load<PAIR>(b_dst, tmB, bar, b0, b1, (int)kb);
             // (a CTA on its own loads the tile's 256 rows of B as two boxes of 128, one behind the other)
-#pragma unroll
-            for (int b = 0; b < (PAIR ? 1 : 2); ++b) {
-              if (p.b_mn) tma_load<PAIR>(b_dst + b * A_BYTES, tmB, bar, rb + b * (int)BM, ka);
-              else tma_load<PAIR>(b_dst + b * A_BYTES, tmB, bar, ka, rb + b * (int)BM);
-            }
-            if (++s == STAGES) { s = 0; ph ^= 1u; }
+            if (!PAIR) tma_load<PAIR>(b_dst + A_BYTES, tmB, bar, p.b_mn ? rb + (int)BM : 0, p.b_mn ? 0 : rb + (int)BM, (int)kb);
           }
+          if (++s == ring.stages) { s = 0; ph ^= 1u; }
         }
       }
-      if (!ok) {
-        // give copies already in flight a bounded chance to land before the CTA's shared memory goes away
-        const long long t0 = clock64();
-        while (clock64() - t0 < 2000000ll) { }
-      }
+    }
+    if (!ok) {
+      // give copies already in flight a bounded chance to land before the CTA's shared memory goes away
+      const long long t0 = clock64();
+      while (clock64() - t0 < 2000000ll) { }
     }
   } else if (warp == 1) {
     // ---------------------------------------------------------------- MMA issuer
-    if (lane == 0 && rank == 0) {
-      int s = 0;
-      uint32_t ph = 0, acc = 0, acc_ph = 0, at_problem = 0;
+    if (rank == 0) {
+      const bool elected = elect_one();
+      uint32_t s = 0, ph = 0, acc = 0, acc_ph = 0, at_problem = 0;
       bool ok = true;
       for (uint32_t wave = 0, tile = first_tile; ok && tile < num_tiles; ++wave, tile = snake_tile(wave, first_tile, tile_step)) {
         QE_TILE_PROBLEM();
         (void)tiles_m; (void)tiles_n; (void)m_fastest;
         const uint32_t idesc = p.idesc, b_hi = p.b_desc_hi, a_step = p.a_mn ? 256u : 2u, b_step = p.b_step;
+        const uint32_t b_block = tile_n / CTAS * BK / 16u;  // from one block of B in a stage to the next
         for (uint32_t seg = 0; ok && seg < (SUMS ? p.nseg : 1u); ++seg) {  // an accumulator of its own for each product
           if (!(ok = mbar_wait(tempty_bar(acc), acc_ph ^ 1u, abort_flag, status, ERR_MMA))) break;
           tc_fence_after();
           const uint32_t d_tmem = tmem_base + acc * ACC_COLS;
-          for (uint32_t kb = 0; kb < num_kb; ++kb) {
+          for (uint32_t kb = 0; kb < num_kb; kb += ring.blocks) {
             if (!(ok = mbar_wait(full_bar(s), ph, abort_flag, status, ERR_MMA))) break;
             tc_fence_after();
-            const uint32_t a_src = smem_base + s * STAGE_BYTES, b_src = a_src + A_BYTES;
+            const uint32_t a_src = smem_base + s * ring.stage_bytes, b_src = a_src + ring.b_offset();
             const uint64_t adesc = make_desc(a_src, A_DESC_HI);
             const uint64_t bdesc = make_desc(b_src, b_hi, PAIR || !p.b_mn ? 1u : A_BYTES / 16u);
+            if (elected) {
 #pragma unroll
-            for (int k = 0; k < (int)BK / UMMA_K; ++k)
-              // advancing 32 along the contraction: 32 bytes inside the 128-byte swizzle row for a contraction-major
-              // tile (+2 in the address field), 32 rows for an MN-major one (+256 with rows of 128 bytes)
-              tc_mma_f8<PAIR>(d_tmem, adesc + a_step * k, bdesc + b_step * k, idesc, (kb | (uint32_t)k) != 0u);
-            tc_commit<PAIR>(empty_bar(s));  // stage reusable (in both CTAs) once these MMAs have read it
-            if (++s == STAGES) { s = 0; ph ^= 1u; }
+              for (uint32_t k = 0; k < BK / UMMA_K; ++k)
+                // advancing 32 along the contraction: 32 bytes inside the 128-byte swizzle row for a contraction-major
+                // tile (+2 in the address field), 32 rows for an MN-major one (+256 with rows of 128 bytes)
+                tc_mma_f8<PAIR>(d_tmem, adesc + a_step * k, bdesc + b_step * k, idesc, k ? 1u : kb);
+              if (PAIR && ring.blocks == 2 && kb + 1 < num_kb) {
+#pragma unroll
+                for (uint32_t k = 0; k < BK / UMMA_K; ++k)
+                  tc_mma_f8<PAIR>(d_tmem, adesc + A_BYTES / 16u + a_step * k, bdesc + b_block + b_step * k, idesc, 1u);
+              }
+              tc_commit<PAIR>(empty_bar(s));  // stage reusable (in both CTAs) once these MMAs have read it
+            }
+            if (++s == ring.stages) { s = 0; ph ^= 1u; }
           }
           if (!ok) break;
-          tc_commit<PAIR>(tfull_bar(acc));  // accumulator complete (each CTA holds its 128 rows)
+          if (elected) tc_commit<PAIR>(tfull_bar(acc));  // accumulator complete (each CTA holds its 128 rows)
           if (++acc == 2) { acc = 0; acc_ph ^= 1u; }
         }
       }
@@ -822,13 +841,14 @@ constexpr uint32_t PAIR_M = Form<true>::TILE_M;
 uint32_t ceil_div(uint32_t a, uint32_t b) { return (a + b - 1) / b; }
 uint32_t tiles_of(const GemmDesc& d, uint32_t tile_n) { return ceil_div(d.M, PAIR_M) * ceil_div(d.N, tile_n); }
 
-// Columns per tile of a launch's problems (index into kTileWidths).  A tile's main loop takes 0.27 us per 128-byte K
-// block at ANY width (four dependent MMAs of ~128 clocks each), so width is free only as long as every CTA pair has a
-// tile; a launch that leaves pairs idle takes narrower tiles for their shorter epilogue: 256 columns against 64, back to
-// back, 5.0 -> 4.1 us (256 x 256 x 256), 7.4 -> 6.4 us (512 x 1024 x 1024, dI), 8.5 -> 6.6 us (1024 x 1024 x 512, FP32
-// accumulate); 256 against 128: 15.8 -> 14.7 us (256 x 8192 x 4096).  The narrowest only up to half the pairs: beyond,
-// the next launch's CTAs find no free SM to start on before this one ends (1024 x 1024 x 1024: 6.9 us at 128, 7.2 at 64).
-// More tiles than pairs lose at once (256 x 8192 x 4096 at 64 columns: 23.4 us).
+// Columns per tile of a launch's problems (index into kTileWidths).  A tile's main loop takes 340, 460 or 530 clocks per 128-byte
+// K block at 64, 128 or 256 columns (shared memory is read and written for A whatever the width; an MMA of up to 64 columns
+// takes 48 clocks, one of 128 takes 64), so narrower tiles gain nothing unless every CTA pair has one: a launch that leaves
+// pairs idle takes narrower ones, which also shortens its epilogue.  us at 256 / 128 / 64 columns, back to back: 256 x 256 x
+// 256 4.5 / 3.7 / 3.2, 512 x 1024 x 1024 6.4 / 4.8 / 4.1, 256 x 2048 x 8192 22.4 / 15.6 / 13.9, 512 x 4096 x 4096 13.8 / 10.8
+// (two waves of 64: 14.6).  The narrowest only up to half the pairs: beyond, the next launch's CTAs find no free SM to start on
+// before this one ends, which costs what the width gains (1024 x 1024 x 1024 6.5 / 4.96 / 5.01, 768 x 1536 x 1536 7.7 / 5.63 /
+// 5.76, 512 x 2048 x 2048 9.0 / 6.4 / 6.2).  More tiles than pairs lose at once (256 x 8192 x 4096 14.9 / 12.0 / 15.2).
 uint32_t choose_width(const GemmDesc* d, uint32_t n, uint32_t pairs) {
   uint32_t w = 0;
   while (w + 1 < kNumTileWidths) {
@@ -897,7 +917,7 @@ Launch make_launch(const GemmDesc* probs, uint32_t n, uint32_t nops, int num_sms
     std::memcpy(at + offsetof(P, prob) + i * sizeof(GemmParams), &p, sizeof(p));
     for (uint32_t j = 0; j < probs[i].nseg; ++j, ++op) {
       const GemmDesc::Operands& d = probs[i].ops[j];
-      const GemmOperands o{*d.mapA, d.mapB[w], d.alpha_a, d.alpha_b};
+      const GemmOperands o{d.mapA[a_map_of(w)], d.mapB[w], d.alpha_a, d.alpha_b};
       std::memcpy(at + offsetof(P, op) + op * sizeof(GemmOperands), &o, sizeof(o));
     }
   }

@@ -95,11 +95,15 @@ struct ArenaReduceParams {
 // Tile widths the GEMM can be run with: the B operand's TMA box has half as many rows (each CTA of a pair loads half).
 constexpr uint32_t kNumTileWidths = 3;
 constexpr uint32_t kTileWidths[kNumTileWidths] = {256, 128, 64};
+// K blocks of 128 that a box of an operand holds: one where tiles are 256 columns wide, else two; an operand in the A role has
+// a map for either.
+constexpr uint32_t blocks_of(uint32_t width) { return width ? 2u : 1u; }
+constexpr uint32_t a_map_of(uint32_t width) { return width ? 1u : 0u; }
 
 // One pair of operands: D = (A . B^T) * (*alpha_a * *alpha_b).
 struct GemmOperands {
-  CUtensorMap tmA;             // A: 128 rows x 128 contraction bytes, 128-byte swizzle
-  CUtensorMap tmB;             // B: tile_n / 2 rows x 128 contraction bytes (MN-major: swizzled over tile_n / 2 bytes)
+  CUtensorMap tmA;             // A: 128 rows x 128 contraction bytes x blocks_of(width), 128-byte swizzle
+  CUtensorMap tmB;             // B: tile_n / 2 rows, likewise (MN-major: swizzled over tile_n / 2 bytes)
   const float* alpha_a;
   const float* alpha_b;
 };
@@ -136,8 +140,8 @@ constexpr uint32_t kMaxSegments = 8;
 struct GemmDesc : GemmParams {
   uint32_t a_fmt, b_fmt;       // 0 = E4M3, 1 = E5M2
   struct Operands {
-    const CUtensorMap* mapA;
-    const CUtensorMap* mapB;   // one map per tile width (the launch reads the one of the width it chooses: gemm_width)
+    const CUtensorMap* mapA;   // [2]: a_map_of(width); the launch reads those of the width it chooses (gemm_width)
+    const CUtensorMap* mapB;   // [kNumTileWidths]
     const float* alpha_a;
     const float* alpha_b;
   } ops[kMaxSegments];

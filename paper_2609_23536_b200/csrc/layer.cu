@@ -100,10 +100,10 @@ int32_t qe_layer_create(qe_ctx* ctx, const qe_layer_config* cfg, void* ws, uint6
     uint8_t* s = base + k.slot0 + k.per_slot * p;
     L->Xq[p] = s + k.xq;
     L->Gq[p] = s + k.gq;
-    if ((st = make_map(d, &L->tmXq_A[p], L->Xq[p], T, K, 128)) != QE_OK) break;   // F:  A = Xq  [T,K]
-    if ((st = make_map(d, &L->tmGq_A[p], L->Gq[p], T, N, 128)) != QE_OK) break;   // dI: A = Gq  [T,N]
+    if ((st = make_a_maps(d, L->tmXq_A[p], L->Xq[p], T, K, false)) != QE_OK) break;   // F:  A = Xq  [T,K]
+    if ((st = make_a_maps(d, L->tmGq_A[p], L->Gq[p], T, N, false)) != QE_OK) break;   // dI: A = Gq  [T,N]
     // dW reads Gq [T,N] and Xq [T,K] as MN-major operands
-    if ((st = make_map(d, &L->tmGq_dW[p], L->Gq[p], T, N, 128)) != QE_OK) break;
+    if ((st = make_a_maps(d, L->tmGq_dW[p], L->Gq[p], N, T, true)) != QE_OK) break;
     if ((st = make_b_maps(d, L->tmXq_dW[p], L->Xq[p], K, T, true)) != QE_OK) break;
   }
   if (st == QE_OK) st = make_b_maps(d, L->tmWq_B, L->Wq, N, K, false);   // F:  B = Wq [N,K]

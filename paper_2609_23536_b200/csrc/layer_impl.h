@@ -37,9 +37,9 @@ struct DeviceInfo {
 
 int32_t device_info(int device, DeviceInfo** out);
 int32_t current_device_info(DeviceInfo** d);
-int32_t make_map(const DeviceInfo* d, CUtensorMap* map, const void* ptr, uint64_t rows, uint64_t inner, uint32_t box_rows,
-                 uint32_t box_inner = 128);
+int32_t make_a_map(const DeviceInfo* d, CUtensorMap* map, const void* ptr, uint64_t M, uint64_t Kc, bool mn, uint32_t width);
 int32_t make_b_map(const DeviceInfo* d, CUtensorMap* map, const void* ptr, uint64_t N, uint64_t Kc, bool mn, uint32_t width);
+int32_t make_a_maps(const DeviceInfo* d, CUtensorMap* maps, const void* ptr, uint64_t M, uint64_t Kc, bool mn);
 int32_t make_b_maps(const DeviceInfo* d, CUtensorMap* maps, const void* ptr, uint64_t N, uint64_t Kc, bool mn);
 int32_t make_out_map(const DeviceInfo* d, CUtensorMap* map, const void* ptr, uint64_t M, uint64_t N, uint64_t ldo, bool fp32);
 int32_t make_out_map_u8(const DeviceInfo* d, CUtensorMap* map, const void* ptr, uint64_t M, uint64_t N, uint64_t ld);
@@ -95,8 +95,8 @@ struct qe_layer {
   uint8_t* Wq = nullptr;
   uint8_t *x_stage = nullptr, *dx_stage = nullptr, *y_stage = nullptr, *dy_stage = nullptr;  // host_io only
   uint8_t *Xq[QE_MAX_SLOTS], *Gq[QE_MAX_SLOTS];
-  // tensor maps: one per tensor in the A role, one per tile width in the B role
-  CUtensorMap tmXq_A[QE_MAX_SLOTS], tmGq_A[QE_MAX_SLOTS], tmGq_dW[QE_MAX_SLOTS], tmXq_dW[QE_MAX_SLOTS][qe::kNumTileWidths];
+  // tensor maps: two per tensor in the A role (a_map_of), one per tile width in the B role
+  CUtensorMap tmXq_A[QE_MAX_SLOTS][2], tmGq_A[QE_MAX_SLOTS][2], tmGq_dW[QE_MAX_SLOTS][2], tmXq_dW[QE_MAX_SLOTS][qe::kNumTileWidths];
   CUtensorMap tmWq_B[qe::kNumTileWidths], tmWq_dI[qe::kNumTileWidths];  // B of the forward; B of dI (MN-major)
   ActionGraph gF[QE_MAX_SLOTS], gDI[QE_MAX_SLOTS], gDW[QE_MAX_SLOTS], gDWs[QE_MAX_SLOTS], gRefresh, gCommit;
   // QE_CTX_OVERLAP_DW: per slot, "dI of the tape in this slot has been enqueued" / "the dW that released it has"

@@ -67,10 +67,10 @@ int32_t qe_arena_reduce(const void* views, uint64_t view_elems, uint32_t M, floa
 // A standalone GEMM with its operand maps (the descriptor points at them).
 struct StandaloneGemm {
   qe::GemmDesc desc;
-  CUtensorMap mapA, mapB[qe::kNumTileWidths];
+  CUtensorMap mapA[2], mapB[qe::kNumTileWidths];
 };
 
-// Validates one standalone GEMM and fills its descriptor, up to the map of its B operand (standalone_map_b), whose box depends
+// Validates one standalone GEMM and fills its descriptor, up to the maps of its operands (standalone_maps), whose boxes depend
 // on the launch's tile width: one map is encoded per operand.  (Host time bounds the call; with three maps for B 512 x 4096 x
 // 4096 took 9.8 us of it, with one 9.6.)
 static int32_t standalone_gemm(DeviceInfo* dev, const void* a, uint32_t a_fmt, uint32_t a_mn, const void* b, uint32_t b_fmt,
@@ -85,10 +85,7 @@ static int32_t standalone_gemm(DeviceInfo* dev, const void* a, uint32_t a_fmt, u
   if ((((uintptr_t)a | (uintptr_t)b | (uintptr_t)d) & 15u)) return fail(QE_ERR_BAD_ARG, "misaligned pointer");
   int32_t st;
   qe::GemmDesc& gp = sg->desc;
-  // contraction-major operand: [rows, Kc]; MN-major operand: [Kc, rows]
-  st = a_mn ? make_map(dev, &sg->mapA, a, Kc, M, 128) : make_map(dev, &sg->mapA, a, M, Kc, 128);
-  if (st != QE_OK) return st;
-  gp.ops[0] = {&sg->mapA, sg->mapB, alpha_a, alpha_b};
+  gp.ops[0] = {sg->mapA, sg->mapB, alpha_a, alpha_b};
   gp.M = M;
   gp.N = Nn;
   gp.Kc = Kc;
@@ -105,8 +102,9 @@ static int32_t standalone_gemm(DeviceInfo* dev, const void* a, uint32_t a_fmt, u
   return QE_OK;
 }
 
-static int32_t standalone_map_b(DeviceInfo* dev, StandaloneGemm* sg, const void* b, uint32_t width) {
-  return make_b_map(dev, &sg->mapB[width], b, sg->desc.N, sg->desc.Kc, sg->desc.b_mn != 0, width);
+static int32_t standalone_maps(DeviceInfo* dev, StandaloneGemm* sg, const void* a, const void* b, uint32_t width) {
+  const int32_t st = make_a_map(dev, &sg->mapA[qe::a_map_of(width)], a, sg->desc.M, sg->desc.Kc, sg->desc.a_mn != 0, width);
+  return st != QE_OK ? st : make_b_map(dev, &sg->mapB[width], b, sg->desc.N, sg->desc.Kc, sg->desc.b_mn != 0, width);
 }
 
 int32_t qe_gemm_fp8_ex(const void* a, uint32_t a_fmt, uint32_t a_mn, const void* b, uint32_t b_fmt, uint32_t b_mn,
@@ -117,7 +115,7 @@ int32_t qe_gemm_fp8_ex(const void* a, uint32_t a_fmt, uint32_t a_mn, const void*
   if (st != QE_OK) return st;
   StandaloneGemm sg;
   if ((st = standalone_gemm(dev, a, a_fmt, a_mn, b, b_fmt, b_mn, M, Nn, Kc, alpha_a, alpha_b, d, out_kind, amax_dev, status_dev, &sg)) != QE_OK) return st;
-  if ((st = standalone_map_b(dev, &sg, b, qe::gemm_width(&sg.desc, 1, dev->num_sms))) != QE_OK) return st;
+  if ((st = standalone_maps(dev, &sg, a, b, qe::gemm_width(&sg.desc, 1, dev->num_sms))) != QE_OK) return st;
   return launch_on(qe::make_gemm(sg.desc, dev->num_sms), (cudaStream_t)stream);
 }
 
@@ -139,7 +137,7 @@ int32_t qe_gemm_fp8_group(const qe_gemm_desc* descs, uint32_t n, uint32_t* statu
   }
   const uint32_t width = qe::gemm_width(gp, n, dev->num_sms);
   for (uint32_t i = 0; i < n; ++i)
-    if ((st = standalone_map_b(dev, &sg[i], descs[i].b_dev, width)) != QE_OK) return st;
+    if ((st = standalone_maps(dev, &sg[i], descs[i].a_dev, descs[i].b_dev, width)) != QE_OK) return st;
   qe::Launch l;
   if (!qe::make_gemm_group(gp, n, dev->num_sms, &l)) return fail(QE_ERR_UNSUPPORTED, "the problems cannot share a launch");
   return launch_on(l, (cudaStream_t)stream);

@@ -255,6 +255,19 @@ def test_gemm_tile_widths_and_half_filled_row_tiles_integer_exact(qe, M, Nn, a_m
     assert amax.item() == float(np.abs(bf16.decode(wb)).max())
 
 
+@pytest.mark.parametrize("M,Nn", [(256, 256), (512, 1152), (256, 8192)])  # 64 and 128 columns: two K blocks to a stage
+@pytest.mark.parametrize("Kc", [128, 256, 1024, 1152, 2176])                # half a stage; the ring's length; its last stage half filled
+@pytest.mark.parametrize("a_mn,b_mn", [(0, 0), (0, 1), (1, 1)])
+def test_gemm_narrow_tiles_of_any_contraction_integer_exact(qe, M, Nn, Kc, a_mn, b_mn):
+    g = torch.Generator(device=DEV).manual_seed(M + Nn + Kc)
+    a, b = (torch.randint(-3, 4, shape, generator=g, device=DEV).float() for shape in ((M, Kc), (Nn, Kc)))
+    to8 = lambda t, mn: (t.t() if mn else t).contiguous().to(torch.float8_e4m3fn).view(torch.uint8)  # noqa: E731
+    one, status = torch.ones(1, device=DEV), torch.zeros(1, dtype=torch.int32, device=DEV)
+    out = torch.full((M, Nn), 7.0, device=DEV)
+    qe.qe_gemm_fp8_ex(to8(a, a_mn), 0, a_mn, to8(b, b_mn), 0, b_mn, one, one, out, 1, None, status)
+    assert torch.equal(out.double(), a.double() @ b.double().t()) and status.item() == 0  # sums below 2^24: exact
+
+
 @pytest.mark.parametrize("M,Nn,Kc", [(1152, 8192, 640), (384, 11008, 384), (1152, 1920, 2176)])
 @pytest.mark.parametrize("kind", [0, 1, 2])
 def test_odd_row_counts_give_the_bits_of_even_ones(qe, M, Nn, Kc, kind):
