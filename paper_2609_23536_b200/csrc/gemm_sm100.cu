@@ -446,7 +446,8 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
   // Everything above (barriers, tensor memory) touched no data a predecessor produces and may overlap the previous
   // kernel's tail; operands, scales and the destination may come from it, so wait for it here.
   grid_dep_wait();
-  grid_dep_launch();
+  const bool hold = blockIdx.x < ps.count() && ps.commit(blockIdx.x).hold_trigger;
+  if (!hold) grid_dep_launch();
   if (blockIdx.x == 0 && threadIdx.x == EPI_WARP0 * 32) {  // FP8 hand-off: the consumer's tape snapshot of its inverse scale
     const GemmParams& q = ps.first();
     if (q.epi == 3 && q.sinv_dst) *q.sinv_dst = *q.sinv_src;
@@ -457,6 +458,11 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
     // are snapshots), so only the output's class is left for the launch's tail.
     const CommitParams& c = ps.commit(blockIdx.x);
     if (c.st && c.early_mask) commit_class<false>(c, c.early_mask, c.bump_token != 0, true, lane);
+    if (hold) {
+      __threadfence();
+      __syncwarp();
+      grid_dep_launch();
+    }
   }
 
   // (The roles are one flat choice: with producer and issuer nested under a choice of their own, or written as lambdas, the
@@ -819,14 +825,21 @@ __global__ void __launch_bounds__(threads_of(false), 1) gemm_fp8_kernel(const __
   gemm_body<false>(Problems<1, 1>{p});
 }
 
+// The whole-step call's casts may run beside these launches (quantize_multi_kernel, `early`), a block of eight warps of 40
+// registers on each SM: three GEMM warps share a sub-partition's 16384 registers with two of the cast's, which leaves each 144.
+// The bound is that of 448 threads (128 registers taken, none spilled; 168 without it).  A block of hidden 2048 at 2048 tokens:
+// 2389 us a step with the casts between the GEMMs, 2340 with their blocks starting on SMs that a GEMM launch has left, 2116
+// beside its CTAs; eight linears of 2048 x 2048 at 768 tokens 803 / 778 / 749.
+constexpr int SHARED_SM_THREADS = 448;
+
 // Up to eight independent GEMMs in one launch.
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(threads_of(false), 1)
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(SHARED_SM_THREADS, 1)
     gemm_fp8_pair_group_kernel(const __grid_constant__ GroupParams g) {
   gemm_body<true>(Problems<8, 8>{g});
 }
 
 // Up to fifty: what the kernel's parameter space holds.
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(threads_of(false), 1)
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(SHARED_SM_THREADS, 1)
     gemm_fp8_pair_many_kernel(const __grid_constant__ ManyParams g) {
   gemm_body<true>(Problems<kMaxSingles, kMaxSingles>{g});
 }

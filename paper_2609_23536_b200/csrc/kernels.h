@@ -40,6 +40,8 @@ struct CommitParams {
   uint32_t early_mask;         // GEMM launches: classes whose amax is complete when the launch starts (committed then, with
                                // the token); class_mask holds the ones its own epilogue completes
   uint32_t bump_token;         // 1 for F and dI, 0 otherwise
+  uint32_t hold_trigger;       // GEMM launches: the next kernel in the stream may start before this one ends, and reads what the
+                               // early part commits: it is let go after that
   const float* amax_override;  // if non-null: value to push for the single class in class_mask
 };
 
@@ -53,6 +55,7 @@ struct QuantParams {
   float* sinv_dst;
   uint32_t* amax_bits;         // atomicMax target or null
   int32_t fmt;                 // 0 = E4M3, 1 = E5M2
+  uint32_t early;              // of the first cast of a launch: the launch may overlap the kernel before it (quantize_multi_kernel)
   CommitParams commit;         // performed by the last block to finish (commit.st != null)
 };
 
@@ -229,7 +232,7 @@ struct Launch {
 };
 
 Launch make_quantize(const QuantParams& p);
-Launch make_quantize_multi(const QuantParams* casts, uint32_t n);  // 2..kMaxCasts independent casts in one launch
+Launch make_quantize_multi(const QuantParams* casts, uint32_t n);  // 1..kMaxCasts independent casts in one launch
 Launch make_commit(const CommitParams& p);
 Launch make_status_gather(const StatusGatherParams& p);
 Launch make_amax_pass1(const AmaxParams& p);

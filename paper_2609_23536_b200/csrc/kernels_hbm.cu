@@ -64,8 +64,8 @@ __device__ __forceinline__ void quantize_block(const QuantParams& p, uint32_t bx
   const int rb = lane >> 3, cv = lane & 7;
   const uint32_t row0 = by * 256u + warp * 32u + rb * 8u;
   const uint32_t col0 = bx * 64u + cv * 8u;
-  const float scale = *p.scale;
-  if (bx == 0 && by == 0 && threadIdx.x == 0 && p.sinv_dst) *p.sinv_dst = *p.sinv_src;
+  const float scale = __ldcg(p.scale);
+  if (bx == 0 && by == 0 && threadIdx.x == 0 && p.sinv_dst) *p.sinv_dst = __ldcg(p.sinv_src);
 
   uint32_t m = 0;
   if (row0 < p.rows) {  // warp-uniform up to rb; rows is a multiple of 8 so a thread's 8 rows are all in or out
@@ -126,8 +126,14 @@ __global__ void __launch_bounds__(kQuantThreads) quantize_kernel(const __grid_co
 
 // Independent casts in one launch (the X of forward units and the dY of input-gradient units that go out together, the
 // weights of a stage at the start of its step): the blocks are dealt to the casts one cast after the other.
+//
+// early: the casts' inputs, scales and destinations belong to no part of the kernel before this one that is still running (a
+// GEMM launch of the whole-step call, whose tiles leave DRAM bandwidth unused): the blocks do not wait for that kernel.  They
+// start when all of its CTAs have let its dependents go, which they do after their own wait, so that everything before it is
+// complete, and after the commits that these casts read.  One block waits at the end, so that this launch ends after that
+// kernel does and whoever waits for this launch has waited for both.  A block fits beside a GEMM CTA: 40 registers a thread.
 template <int N>
-__global__ void __launch_bounds__(kQuantThreads) quantize_multi_kernel(const __grid_constant__ QuantMultiParams<N> mp) {
+__global__ void __launch_bounds__(kQuantThreads, 6) quantize_multi_kernel(const __grid_constant__ QuantMultiParams<N> mp) {
   __shared__ uint32_t wmax[kQuantThreads / 32];
   __shared__ uint32_t last_flag;
   uint32_t which = 0, end = mp.n;  // the first cast that ends behind this block
@@ -137,7 +143,7 @@ __global__ void __launch_bounds__(kQuantThreads) quantize_multi_kernel(const __g
     else end = mid;
   }
   const uint32_t base = which ? mp.block_end[which - 1] : 0u;
-  grid_dep_wait();
+  if (!mp.q[0].early) grid_dep_wait();
   grid_dep_launch();
   const QuantParams& p = mp.q[which];
   const uint32_t b = blockIdx.x - base, bxn = p.cols / 64u;
@@ -148,6 +154,7 @@ __global__ void __launch_bounds__(kQuantThreads) quantize_multi_kernel(const __g
     if (last_block(&p.commit.st->ticket, mp.block_end[which] - base, threadIdx.x, &last_flag, sync))
       commit_classes(p.commit, threadIdx.x, wmax, sync);
   }
+  if (mp.q[0].early && blockIdx.x == gridDim.x - 1) grid_dep_wait();
 }
 
 template <int N>

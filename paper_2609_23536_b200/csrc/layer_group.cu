@@ -270,10 +270,11 @@ void push_gemms(qe_ctx* ctx, const qe::GemmDesc* gemms, uint32_t n, std::vector<
 
 // the launches: the casts in one launch, then every GEMM of whole 256-row tiles in one launch; weight gradients of
 // several microbatches of one layer (whole-step call only) become one GEMM that adds their products up
-// (refresh != null: the weight casts are collected there instead of being queued; any_rows: half-filled last row tiles share
-// launches too)
+// (refresh != null: the weight casts are collected there instead of being queued; apart: a round of a list whose tensors are
+// apart: half-filled last row tiles share launches too, and the next round's casts may overlap its GEMMs; early: its own casts
+// may overlap what is before them)
 int32_t together_build(qe_ctx* ctx, const Prepared* acts, uint32_t n, float* grad, std::vector<qe::Launch>& ls, Fnv* h,
-                       std::vector<qe::QuantParams>* refresh = nullptr, bool any_rows = false) {
+                       std::vector<qe::QuantParams>* refresh = nullptr, bool apart = false, bool early = false) {
   std::vector<qe::GemmDesc> chain, dw, singles;  // F and dI; weight gradients; those that go out one by one
   std::vector<const qe_layer*> dw_owner, single_owner;
   std::vector<qe::QuantParams> casts;
@@ -292,9 +293,9 @@ int32_t together_build(qe_ctx* ctx, const Prepared* acts, uint32_t n, float* gra
       }
       if (a.kind == QE_ACT_DW) {
         const qe::GemmDesc gp = dW_gemm(L, a.slot, grad + a.grad_offset, a.acc, nullptr);
-        const bool apart = !any_rows && !qe::whole_row_tiles(gp.M);  // a half-filled last row tile: a launch of its own
-        std::vector<qe::GemmDesc>& to = apart ? singles : dw;
-        std::vector<const qe_layer*>& owner = apart ? single_owner : dw_owner;
+        const bool single = !apart && !qe::whole_row_tiles(gp.M);  // a half-filled last row tile: a launch of its own
+        std::vector<qe::GemmDesc>& to = single ? singles : dw;
+        std::vector<const qe_layer*>& owner = single ? single_owner : dw_owner;
         const auto sum = std::find(owner.begin(), owner.end(), L);  // this layer's of an earlier microbatch takes this one in
         if (sum != owner.end()) {
           qe::GemmDesc& g = to[sum - owner.begin()];
@@ -319,7 +320,8 @@ int32_t together_build(qe_ctx* ctx, const Prepared* acts, uint32_t n, float* gra
         add_dI(L, a.slot, a.in_dev, a.out_dev, ls, nullptr, 0, &gp, &cast);
       }
       casts.push_back(cast);
-      if (any_rows || qe::whole_row_tiles(gp.M)) {
+      gp.commit.hold_trigger = apart;
+      if (apart || qe::whole_row_tiles(gp.M)) {
         chain.push_back(gp);
       } else {
         singles.push_back(gp);
@@ -333,7 +335,8 @@ int32_t together_build(qe_ctx* ctx, const Prepared* acts, uint32_t n, float* gra
   std::stable_sort(dw.begin(), dw.end(), [](const qe::GemmDesc& x, const qe::GemmDesc& y) { return x.Kc * x.nseg > y.Kc * y.nseg; });
   for (size_t i = 0; i < casts.size(); i += qe::kMaxCasts) {  // all casts of the call in one launch
     const uint32_t m = (uint32_t)std::min<size_t>(qe::kMaxCasts, casts.size() - i);
-    ls.push_back(m > 1 ? qe::make_quantize_multi(&casts[i], m) : qe::make_quantize(casts[i]));
+    casts[i].early = early;
+    ls.push_back(m > 1 || early ? qe::make_quantize_multi(&casts[i], m) : qe::make_quantize(casts[i]));
   }
   for (const qe::GemmDesc& gp : singles) ls.push_back(qe::make_gemm(gp, ctx->dev->num_sms));
   if (chain.size() + dw.size() >= 2) {
@@ -605,11 +608,15 @@ int32_t qe_step_run(qe_ctx* ctx, qe_layer* const* layers, uint32_t n_layers, con
     refresh.clear();
   };
   uint32_t waiting = 0;  // actions in the piece that is being put together
+  std::vector<uint64_t> freed(n_layers, 0), freed_before(n_layers, 0);  // slots that the weight gradients of a round release
   std::vector<Prepared> acts;
   for (size_t r = 0; r < rounds.size() && st == QE_OK; ++r) {
     // check -> commit per action (all F first: a slot that a dW of the round releases is not theirs to take), then the
     // launches of those that passed
     acts.clear();
+    bool early = apart && r > 0;
+    freed_before.swap(freed);
+    std::fill(freed.begin(), freed.end(), 0);
     for (size_t i = 0; repeated && i < rounds[r].size(); ++i)
       for (size_t j = 0; j < i; ++j) {
         const qe_step_action &a = actions[rounds[r][j]], &b = actions[rounds[r][i]];
@@ -632,11 +639,13 @@ int32_t qe_step_run(qe_ctx* ctx, qe_layer* const* layers, uint32_t n_layers, con
                      : qe_contract_dW_check(L->contract, &tapes[u], (uint64_t)(uintptr_t)grad, grad_elems, offsets[a.layer], slice, &p.acc);
           p.slot = tapes[u].ref.slot;
           if (st == QE_OK) st = qe_contract_dW_commit(L->contract, &tapes[u], (uint64_t)(uintptr_t)grad, offsets[a.layer], slice);
+          freed[a.layer] |= 1ull << (p.slot & 63u);
         } else if (!in || !out || (((uintptr_t)in | (uintptr_t)out) & 15u)) {
           st = fail(QE_ERR_BAD_ARG, "input / output null or misaligned");
         } else if (a.kind == QE_ACT_F) {
           st = qe_contract_forward_check(L->contract, a.mb, L->contract->e_W, &p.refresh, &p.slot);
           if (st == QE_OK) st = qe_contract_forward_commit(L->contract, a.mb, &tapes[u]);
+          early = early && !(freed_before[a.layer] >> (p.slot & 63u) & 1u);  // the GEMMs of the round before still read this slot
         } else {
           st = qe_contract_dI_check(L->contract, &tapes[u]);
           p.slot = tapes[u].ref.slot;
@@ -652,7 +661,7 @@ int32_t qe_step_run(qe_ctx* ctx, qe_layer* const* layers, uint32_t n_layers, con
     }
     char why[512];  // (a build can only fail on a CUDA error, which then is the one to report)
     if (st != QE_OK) std::snprintf(why, sizeof(why), "%s", qe_last_error());
-    const int32_t built = acts.empty() ? QE_OK : together_build(ctx, acts.data(), (uint32_t)acts.size(), grad, ls, nullptr, &refresh, apart);
+    const int32_t built = acts.empty() ? QE_OK : together_build(ctx, acts.data(), (uint32_t)acts.size(), grad, ls, nullptr, &refresh, apart, early);
     if (st != QE_OK) st = fail(st, "%s", why);
     else if (built != QE_OK) {
       st = built;

@@ -203,7 +203,7 @@ bool whole_row_tiles(uint32_t M) { return M % 256 == 0; }
 cudaError_t gemm_prepare() { return cudaSuccess; }
 uint32_t gemm_width(const GemmDesc*, uint32_t, int) { return 1; }
 Launch make_quantize(const QuantParams&) { return named("cast 1"); }
-Launch make_quantize_multi(const QuantParams*, uint32_t n) { return named("cast %u", n); }
+Launch make_quantize_multi(const QuantParams* q, uint32_t n) { return named("cast %u%s", n, q[0].early ? " early" : ""); }
 Launch make_commit(const CommitParams&) { return named("commit"); }
 Launch make_status_gather(const StatusGatherParams&) { return named("status"); }
 Launch make_amax_pass1(const AmaxParams&) { return named("amax1"); }

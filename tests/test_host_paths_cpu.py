@@ -259,3 +259,31 @@ def test_step_takes_all_layers_of_a_unit_at_once_only_where_its_tensors_are_apar
     for name, at in (("weight", s.weights[9]), ("gradient", s.grad + 4 * s.offsets[5])):
         assert casts(lambda a, b: own(a, b)[:1] + [at - size + 16] + own(a, b)[2:] if (a, b) == (3, 0) else own(a, b)) < 2 * n, name
     s.close()
+
+
+@pytest.mark.parametrize("slots", [1, 2, 3, 4, 7])
+def test_step_casts_overlap_the_gemms_before_them_unless_those_read_the_slot(lib, slots):
+    """The casts of a round may run beside the GEMMs of the one before, except the first round's and those of a forward into a
+    slot that a weight gradient of the round before releases."""
+    from paper_2609_23536_b200 import binding as qe
+
+    M, n = 7, 3
+    s = fake_runtime.Stage(lib, [(256, 256)] * n, M=M, slots=slots, window=4)
+    size = 2 * s.T * 256
+    base = s.buffer(4 * n * M * size)
+    lib.fake_reset()
+    assert s.step(_actions(M, n), apart=lambda l, m: [base + ((l * M + m) * 4 + j) * size for j in range(4)]) == 0
+    casts = [w.split() for w in lib.fake_log().decode().splitlines() if " cast " in w][1:]  # (the weights' come first)
+    want, free, held, last = [], set(range(slots)), {}, set()
+    for r, g in enumerate(qe.plan_rounds(_actions(M, n), n, M, slots, 4, 100, max_sum=8, apart=True)):
+        mine = [(a, m) for a, l, m in g if l == 0]  # the layers go alike
+        for a, m in mine:
+            if a == "F":
+                held[m] = min(free)
+                free.remove(held[m])
+        if any(a != "dW" for a, m in mine):
+            want.append(r > 0 and not any(a == "F" and held[m] in last for a, m in mine))
+        last = {held[m] for a, m in mine if a == "dW"}
+        free |= last
+    assert ["early" in w for w in casts] == want and any(want) and (slots == 7 or not all(want[1:]))
+    s.close()
