@@ -154,16 +154,16 @@ __device__ __forceinline__ void cluster_sync_all() {
 }
 // TMA load of a box of an operand; in a pair its completion may be credited to a barrier of the peer CTA.
 template <bool PAIR>
-__device__ __forceinline__ void tma_load(uint32_t dst, const CUtensorMap* map, uint32_t bar, int c0, int c1, int c2) {
+__device__ __forceinline__ void tma_load(uint32_t dst, const CUtensorMap* map, uint32_t bar, int c0, int c1, int c2, int c3) {
   if (PAIR)
     asm volatile(
-        "cp.async.bulk.tensor.3d.shared::cta.global.tile.mbarrier::complete_tx::bytes.cta_group::2 [%0], [%1, {%3, %4, %5}], [%2];"
-        ::"r"(dst), "l"(map), "r"(bar), "r"(c0), "r"(c1), "r"(c2)
+        "cp.async.bulk.tensor.4d.shared::cta.global.tile.mbarrier::complete_tx::bytes.cta_group::2 [%0], [%1, {%3, %4, %5, %6}], [%2];"
+        ::"r"(dst), "l"(map), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "r"(c3)
         : "memory");
   else
     asm volatile(
-        "cp.async.bulk.tensor.3d.shared::cta.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];"
-        ::"r"(dst), "l"(map), "r"(bar), "r"(c0), "r"(c1), "r"(c2)
+        "cp.async.bulk.tensor.4d.shared::cta.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2];"
+        ::"r"(dst), "l"(map), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "r"(c3)
         : "memory");
 }
 // One lane of a converged warp, the same one every time.  The producer's and the issuer's loops run on whole warps, so that
@@ -216,8 +216,8 @@ __device__ __forceinline__ void tc_mma_f8(uint32_t d_tmem, uint64_t adesc, uint6
   else tc_mma_f8_one(d_tmem, adesc, bdesc, idesc, accumulate);
 }
 
-__device__ __forceinline__ void tma_prefetch(const CUtensorMap* map, int c0, int c1, int c2) {
-  asm volatile("cp.async.bulk.prefetch.tensor.3d.L2.global.tile [%0, {%1, %2, %3}];" ::"l"(map), "r"(c0), "r"(c1), "r"(c2) : "memory");
+__device__ __forceinline__ void tma_prefetch(const CUtensorMap* map, int c0, int c1, int c2, int c3) {
+  asm volatile("cp.async.bulk.prefetch.tensor.4d.L2.global.tile [%0, {%1, %2, %3, %4}];" ::"l"(map), "r"(c0), "r"(c1), "r"(c2), "r"(c3) : "memory");
 }
 
 // Bulk tensor store of a shared-memory tile (issued by one lane), with group tracking.
@@ -315,10 +315,10 @@ __device__ __forceinline__ uint32_t snake_tile(uint32_t w, uint32_t first, uint3
 // ------------------------------------------------------------------------------------------------ problem lookup
 // A launch computes one GEMM, or (grouped launch) several independent ones whose tiles are numbered one after the
 // other, so that one set of persistent CTAs packs them into common waves and the launch overhead is paid once.
-template <int NP, int NOPS>
+template <int NP, bool SEVERAL>
 struct Problems {
-  static constexpr bool ONE = NP == 1, SUMS = NOPS > NP;  // one problem; problems may have several products
-  const GemmLaunchParams<NP, NOPS>& g;
+  static constexpr bool ONE = NP == 1, SUMS = SEVERAL;  // one problem; problems may have several products
+  const GemmLaunchParams<NP>& g;
   __device__ __forceinline__ uint32_t count() const { return NP == 1 ? 1u : g.n; }
   __device__ __forceinline__ uint32_t total_tiles() const { return g.tile_end[count() - 1]; }
   // `i`: the problem of an earlier tile of the same role (its tiles come in ascending order), from which the search goes on
@@ -330,9 +330,6 @@ struct Problems {
     while (i + 1 < count() && tile >= g.tile_end[i]) ++i;
     local = tile - (i ? g.tile_end[i - 1] : 0u);
     return g.prob[i];
-  }
-  __device__ __forceinline__ const GemmOperands& operands(const GemmParams& p, uint32_t seg) const {
-    return g.op[NOPS == 1 ? 0u : p.op0 + seg];
   }
   __device__ __forceinline__ const GemmParams& first() const { return g.prob[0]; }
   __device__ __forceinline__ const CommitParams& commit(uint32_t i) const { return g.prob[i].commit; }
@@ -395,8 +392,8 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
 
   if (threadIdx.x == 32) {  // descriptor fetch overlaps the rest of the prologue (and the predecessor's tail)
     const GemmParams& q = ps.first();  // (a group's other descriptors are fetched on first use)
-    asm volatile("prefetch.tensormap [%0];" ::"l"(&ps.operands(q, 0).tmA) : "memory");
-    asm volatile("prefetch.tensormap [%0];" ::"l"(&ps.operands(q, 0).tmB) : "memory");
+    asm volatile("prefetch.tensormap [%0];" ::"l"(&q.tmA) : "memory");
+    asm volatile("prefetch.tensormap [%0];" ::"l"(&q.tmB) : "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(&q.tmD) : "memory");
   }
   if (threadIdx.x == 0) {
@@ -439,9 +436,9 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
     uint32_t m0, n0;
     tile_coords<TILE_M>(local_tile, tiles_m, tiles_n, m_fastest, tile_n, m0, n0);
     const int rb = (int)(n0 + rank * (tile_n / 2));
-    const CUtensorMap* tmB = &ps.operands(p, 0).tmB;
+    const CUtensorMap* tmB = &p.tmB;
     for (uint32_t kb = 0; kb < num_kb && kb < ring.blocks * ring.stages; kb += ring.blocks)
-      for (int b = 0; b < (PAIR ? 1 : 2); ++b) tma_prefetch(tmB, p.b_mn ? rb + b * (int)BM : 0, p.b_mn ? 0 : rb + b * (int)BM, (int)kb);
+      for (int b = 0; b < (PAIR ? 1 : 2); ++b) tma_prefetch(tmB, p.b_mn ? rb + b * (int)BM : 0, p.b_mn ? 0 : rb + b * (int)BM, (int)kb, p.slot_b[0]);
   }
   // Everything above (barriers, tensor memory) touched no data a predecessor produces and may overlap the previous
   // kernel's tail; operands, scales and the destination may come from it, so wait for it here.
@@ -488,18 +485,18 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
       // contraction are filled with zeros and counted)
       const uint32_t bytes = ring.blocks * (CTAS * A_BYTES + tile_n * BK);
       for (uint32_t seg = 0; ok && seg < (SUMS ? p.nseg : 1u); ++seg) {
-        const GemmOperands& op = ps.operands(p, seg);
-        const CUtensorMap *tmA = &op.tmA, *tmB = &op.tmB;
+        const CUtensorMap *tmA = &p.tmA, *tmB = &p.tmB;
+        const int sa = p.slot_a[SUMS ? seg : 0u], sb = p.slot_b[SUMS ? seg : 0u];
         for (uint32_t kb = 0; kb < num_kb; kb += ring.blocks) {
           if (!(ok = mbar_wait(empty_bar(s), ph ^ 1u, abort_flag, status, ERR_PRODUCER))) break;
           const uint32_t a_dst = smem_base + s * ring.stage_bytes, b_dst = a_dst + ring.b_offset();
           if (elected) {
             if (rank == 0) mbar_expect_tx(full_bar(s), bytes);
             const uint32_t bar = PAIR ? map_to_cta(full_bar(s), 0) : full_bar(s);
-            tma_load<PAIR>(a_dst, tmA, bar, a0, a1, (int)kb);
-            tma_load<PAIR>(b_dst, tmB, bar, b0, b1, (int)kb);
+            tma_load<PAIR>(a_dst, tmA, bar, a0, a1, (int)kb, sa);
+            tma_load<PAIR>(b_dst, tmB, bar, b0, b1, (int)kb, sb);
             // (a CTA on its own loads the tile's 256 rows of B as two boxes of 128, one behind the other)
-            if (!PAIR) tma_load<PAIR>(b_dst + A_BYTES, tmB, bar, p.b_mn ? rb + (int)BM : 0, p.b_mn ? 0 : rb + (int)BM, (int)kb);
+            if (!PAIR) tma_load<PAIR>(b_dst + A_BYTES, tmB, bar, p.b_mn ? rb + (int)BM : 0, p.b_mn ? 0 : rb + (int)BM, (int)kb, sb);
           }
           if (++s == ring.stages) { s = 0; ph ^= 1u; }
         }
@@ -605,10 +602,7 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
         prefetch_next();
         // (lane i fetches the scales of product i: one chain of dependent loads per tile instead of one per product)
         float my_alpha = 0.0f;
-        if ((uint32_t)lane < p.nseg) {
-          const GemmOperands& op = ps.operands(p, (uint32_t)lane);
-          my_alpha = __fmul_rn(*op.alpha_a, *op.alpha_b);
-        }
+        if ((uint32_t)lane < p.nseg) my_alpha = __fmul_rn(p.alpha_a[p.slot_a[lane]], p.alpha_b[p.slot_b[lane]]);
         auto take = [&](uint32_t seg, auto first) {
           const float alpha = __shfl_sync(0xffffffffu, my_alpha, (int)seg);
           if (!(ok = mbar_wait(tfull_bar(acc), acc_ph, abort_flag, status, ERR_EPILOGUE))) return;
@@ -650,7 +644,7 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
       // (the variant that sums keeps no shared-memory addresses across its tiles: it needs the registers)
       uint32_t ln = (uint32_t)lane;
       if (SUMS) asm volatile("" : "+r"(ln));
-      const float alpha = __fmul_rn(*ps.operands(p, 0).alpha_a, *ps.operands(p, 0).alpha_b);
+      const float alpha = __fmul_rn(p.alpha_a[p.slot_a[0]], p.alpha_b[p.slot_b[0]]);
       if (p.epi == 2) {
         // accumulate: pull this thread's destination row segment into L2, where the reduction will add to it, while
         // the MMAs of the tile run
@@ -780,7 +774,7 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
       if (PS::ONE) {
         if (ew == 0) commit_class<false>(ps.commit(0), ps.commit(0).class_mask, false, true, lane);
       } else if (ew < ps.count()) {  // a lane per problem, dealt to the epilogue's warps
-        static_assert(kMaxSingles <= EPI_WARPS * 32 && kMaxProblems <= EPI_WARPS * 32, "a lane for every problem");
+        static_assert(kMaxProblems <= EPI_WARPS * 32, "a lane for every problem");
         const uint32_t i = ew + EPI_WARPS * (uint32_t)lane;
         const CommitParams& c = ps.commit(i < ps.count() ? i : 0u);
         commit_class<true>(c, c.class_mask, false, i < ps.count() && c.st && c.class_mask, lane);
@@ -810,19 +804,14 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
 
 #undef QE_TILE_PROBLEM
 
-using OneParams = GemmLaunchParams<1, 1>;
-using GroupParams = GemmLaunchParams<8, 8>;
-using ManyParams = GemmLaunchParams<kMaxSingles, kMaxSingles>;
-using WideParams = GemmLaunchParams<kMaxProblems, kMaxOperands>;
-
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(threads_of(false), 1)
-    gemm_fp8_pair_kernel(const __grid_constant__ OneParams p) {
-  gemm_body<true>(Problems<1, 1>{p});
+    gemm_fp8_pair_kernel(const __grid_constant__ GemmLaunchParams<1> p) {
+  gemm_body<true>(Problems<1, false>{p});
 }
 
 // One GEMM with an odd number of 128-row tiles, a CTA to a tile.
-__global__ void __launch_bounds__(threads_of(false), 1) gemm_fp8_kernel(const __grid_constant__ OneParams p) {
-  gemm_body<false>(Problems<1, 1>{p});
+__global__ void __launch_bounds__(threads_of(false), 1) gemm_fp8_kernel(const __grid_constant__ GemmLaunchParams<1> p) {
+  gemm_body<false>(Problems<1, false>{p});
 }
 
 // The whole-step call's casts may run beside these launches (quantize_multi_kernel, `early`), a block of eight warps of 40
@@ -832,22 +821,18 @@ __global__ void __launch_bounds__(threads_of(false), 1) gemm_fp8_kernel(const __
 // beside its CTAs; eight linears of 2048 x 2048 at 768 tokens 803 / 778 / 749.
 constexpr int SHARED_SM_THREADS = 448;
 
-// Up to eight independent GEMMs in one launch.
+// Several independent GEMMs in one launch: up to eight (a parameter block of 5 KB), or what the parameter space holds.
+template <int NP>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(SHARED_SM_THREADS, 1)
-    gemm_fp8_pair_group_kernel(const __grid_constant__ GroupParams g) {
-  gemm_body<true>(Problems<8, 8>{g});
+    gemm_fp8_pair_group_kernel(const __grid_constant__ GemmLaunchParams<NP> g) {
+  gemm_body<true>(Problems<NP, false>{g});
 }
 
-// Up to fifty: what the kernel's parameter space holds.
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(SHARED_SM_THREADS, 1)
-    gemm_fp8_pair_many_kernel(const __grid_constant__ ManyParams g) {
-  gemm_body<true>(Problems<kMaxSingles, kMaxSingles>{g});
-}
-
-// Problems of several products each.  (The parameter block is three times as large.)
+// The same where problems have several products each.
+template <int NP>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(threads_of(true), 1)
-    gemm_fp8_pair_wide_kernel(const __grid_constant__ WideParams g) {
-  gemm_body<true>(Problems<kMaxProblems, kMaxOperands>{g});
+    gemm_fp8_pair_wide_kernel(const __grid_constant__ GemmLaunchParams<NP> g) {
+  gemm_body<true>(Problems<NP, true>{g});
 }
 
 constexpr uint32_t PAIR_M = Form<true>::TILE_M;
@@ -892,11 +877,12 @@ bool one_cta(const GemmDesc& d, int num_sms) {
   return 6 * waves_ctas < 5 * waves_pairs || (waves_pairs == 1 && d.M > BM && d.Kc <= 6144);
 }
 
-// The device's parameter block of one problem at a tile width; its operand pairs start at op0.
-GemmParams problem_of(const GemmDesc& d, uint32_t w, uint32_t op0, uint32_t tile_m) {
+// The device's parameter block of one problem at a tile width.
+GemmParams problem_of(const GemmDesc& d, uint32_t w, uint32_t tile_m) {
   GemmParams p = d;
   const uint32_t tile_n = kTileWidths[w], per_cta = tile_n / 2;
-  p.op0 = op0;
+  p.tmA = d.mapA[a_map_of(w)];
+  p.tmB = d.mapB[w];
   p.tile_n = tile_n;
   // bits 4-5: accumulator format (1 = FP32); 7-9 / 10-12: A / B format (0 = E4M3, 1 = E5M2); 15 / 16: A / B major
   // (0 = contraction-major); 17-22: N >> 3; 24-28: M >> 4 (of the whole tile).
@@ -909,48 +895,48 @@ GemmParams problem_of(const GemmDesc& d, uint32_t w, uint32_t op0, uint32_t tile
   return p;
 }
 
-template <int NP, int NOPS>
-Launch make_launch(const GemmDesc* probs, uint32_t n, uint32_t nops, int num_sms, const void* func, bool alone = false) {
-  using P = GemmLaunchParams<NP, NOPS>;
-  static_assert(sizeof(P) <= sizeof(Launch::Block), "parameter block too large");
+template <int NP>
+Launch make_launch(const GemmDesc* probs, uint32_t n, int num_sms, const void* func, bool sums, bool alone = false) {
+  using P = GemmLaunchParams<NP>;
+  static_assert(sizeof(P) <= sizeof(Launch::Block) && sizeof(P) <= 32764, "parameter block too large");
   static_assert(NP > 1 || sizeof(P) <= ParamBytes::kInline, "a launch of one problem takes no heap memory");
   Launch l;
   l.nbytes = sizeof(P);
-  l.params.resize(offsetof(P, op) + nops * sizeof(GemmOperands));  // (a step has hundreds of launches: no unused operands)
+  l.params.resize(offsetof(P, prob) + n * sizeof(GemmParams));  // (no unused problems)
   unsigned char* at = l.params.data();
   const uint32_t tile_m = alone ? BM : PAIR_M, ctas = alone ? 1u : 2u, most = (uint32_t)num_sms / ctas;
   const uint32_t w = choose_width(probs, n, (uint32_t)num_sms / 2u);  // (alone: 0, see one_cta)
-  uint32_t tiles = 0, op = 0;
+  uint32_t tiles = 0;
   uint32_t* ticket = nullptr;
   for (uint32_t i = 0; i < n; ++i) {
     if (!ticket && probs[i].commit.st && probs[i].commit.class_mask) ticket = &probs[i].commit.st->ticket;
     tiles += ceil_div(probs[i].M, tile_m) * ceil_div(probs[i].N, kTileWidths[w]);
     std::memcpy(at + offsetof(P, tile_end) + i * sizeof(uint32_t), &tiles, sizeof(tiles));
-    const GemmParams p = problem_of(probs[i], w, op, tile_m);
+    const GemmParams p = problem_of(probs[i], w, tile_m);
     std::memcpy(at + offsetof(P, prob) + i * sizeof(GemmParams), &p, sizeof(p));
-    for (uint32_t j = 0; j < probs[i].nseg; ++j, ++op) {
-      const GemmDesc::Operands& d = probs[i].ops[j];
-      const GemmOperands o{d.mapA[a_map_of(w)], d.mapB[w], d.alpha_a, d.alpha_b};
-      std::memcpy(at + offsetof(P, op) + op * sizeof(GemmOperands), &o, sizeof(o));
-    }
   }
   std::memcpy(at + offsetof(P, n), &n, sizeof(n));
   std::memcpy(at + offsetof(P, ticket), &ticket, sizeof(ticket));
   l.func = func;
   l.grid = dim3(ctas * (tiles < most ? tiles : most), 1, 1);
-  l.block = dim3(threads_of(NOPS > NP), 1, 1);
+  l.block = dim3(threads_of(sums), 1, 1);
   l.smem = SMEM_BYTES;
   return l;
 }
 
-Launch make_any(const GemmDesc* probs, uint32_t n, uint32_t nops, int num_sms) {
-  if (n == 1 && nops == 1) {
+constexpr uint32_t kFew = 8, kFewSums = 16;  // problems of a launch with a small parameter block
+
+Launch make_any(const GemmDesc* probs, uint32_t n, int num_sms) {
+  bool sums = false;
+  for (uint32_t i = 0; i < n; ++i) sums |= probs[i].nseg > 1;
+  if (n == 1 && !sums) {
     const bool alone = one_cta(*probs, num_sms);
-    return make_launch<1, 1>(probs, n, nops, num_sms, alone ? (const void*)gemm_fp8_kernel : (const void*)gemm_fp8_pair_kernel, alone);
+    return make_launch<1>(probs, n, num_sms, alone ? (const void*)gemm_fp8_kernel : (const void*)gemm_fp8_pair_kernel, false, alone);
   }
-  if (n <= 8 && nops == n) return make_launch<8, 8>(probs, n, nops, num_sms, (const void*)gemm_fp8_pair_group_kernel);
-  if (nops == n) return make_launch<kMaxSingles, kMaxSingles>(probs, n, nops, num_sms, (const void*)gemm_fp8_pair_many_kernel);
-  return make_launch<kMaxProblems, kMaxOperands>(probs, n, nops, num_sms, (const void*)gemm_fp8_pair_wide_kernel);
+  if (!sums && n <= kFew) return make_launch<kFew>(probs, n, num_sms, (const void*)gemm_fp8_pair_group_kernel<kFew>, false);
+  if (!sums) return make_launch<kMaxProblems>(probs, n, num_sms, (const void*)gemm_fp8_pair_group_kernel<kMaxProblems>, false);
+  if (n <= kFewSums) return make_launch<kFewSums>(probs, n, num_sms, (const void*)gemm_fp8_pair_wide_kernel<kFewSums>, true);
+  return make_launch<kMaxProblems>(probs, n, num_sms, (const void*)gemm_fp8_pair_wide_kernel<kMaxProblems>, true);
 }
 
 }  // namespace
@@ -958,7 +944,9 @@ Launch make_any(const GemmDesc* probs, uint32_t n, uint32_t nops, int num_sms) {
 bool whole_row_tiles(uint32_t M) { return M % 256 == 0; }
 
 cudaError_t gemm_prepare() {
-  for (const void* f : {(const void*)gemm_fp8_kernel, (const void*)gemm_fp8_pair_kernel, (const void*)gemm_fp8_pair_group_kernel, (const void*)gemm_fp8_pair_many_kernel, (const void*)gemm_fp8_pair_wide_kernel}) {
+  for (const void* f : {(const void*)gemm_fp8_kernel, (const void*)gemm_fp8_pair_kernel, (const void*)gemm_fp8_pair_group_kernel<kFew>,
+                        (const void*)gemm_fp8_pair_group_kernel<kMaxProblems>, (const void*)gemm_fp8_pair_wide_kernel<kFewSums>,
+                        (const void*)gemm_fp8_pair_wide_kernel<kMaxProblems>}) {
     const cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES);
     if (e != cudaSuccess) return e;
   }
@@ -966,15 +954,13 @@ cudaError_t gemm_prepare() {
 }
 
 bool make_gemm_group(const GemmDesc* probs, uint32_t n, int num_sms, Launch* out) {
-  uint32_t nops = 0;
-  for (uint32_t i = 0; i < n; ++i) nops += probs[i].nseg;
-  if (n < 2 || (nops == n ? n > kMaxSingles : n > kMaxProblems || nops > kMaxOperands)) return false;
-  *out = make_any(probs, n, nops, num_sms);
+  if (n < 2 || n > kMaxProblems) return false;
+  *out = make_any(probs, n, num_sms);
   return true;
 }
 
 uint32_t gemm_width(const GemmDesc* probs, uint32_t n, int num_sms) { return choose_width(probs, n, (uint32_t)num_sms / 2u); }
 
-Launch make_gemm(const GemmDesc& d, int num_sms) { return make_any(&d, 1, d.nseg, num_sms); }
+Launch make_gemm(const GemmDesc& d, int num_sms) { return make_any(&d, 1, num_sms); }
 
 }  // namespace qe

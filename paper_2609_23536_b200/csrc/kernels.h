@@ -103,20 +103,21 @@ constexpr uint32_t kTileWidths[kNumTileWidths] = {256, 128, 64};
 constexpr uint32_t blocks_of(uint32_t width) { return width ? 2u : 1u; }
 constexpr uint32_t a_map_of(uint32_t width) { return width ? 1u : 0u; }
 
-// One pair of operands: D = (A . B^T) * (*alpha_a * *alpha_b).
-struct GemmOperands {
-  CUtensorMap tmA;             // A: 128 rows x 128 contraction bytes x blocks_of(width), 128-byte swizzle
-  CUtensorMap tmB;             // B: tile_n / 2 rows, likewise (MN-major: swizzled over tile_n / 2 bytes)
-  const float* alpha_a;
-  const float* alpha_b;
-};
+constexpr uint32_t kMaxSegments = 8;
 
+// D = (A . B^T) * (*alpha_a * *alpha_b), or the sum of several such products over tensors of the same shape at equal distances
+// (the tape slots of a layer): an operand's map spans all of them.
 struct GemmParams {
+  CUtensorMap tmA;             // A: boxes of 128 rows x 128 contraction bytes x blocks_of(width), 128-byte swizzle
+  CUtensorMap tmB;             // B: tile_n / 2 rows, likewise (MN-major: swizzled over tile_n / 2 bytes)
   CUtensorMap tmD;             // D [M, N] (bf16, FP32 or FP8 bytes), box 32 x 32, for the epilogue's bulk stores
+  const float* alpha_a;        // [slot]
+  const float* alpha_b;
+  uint8_t slot_a[kMaxSegments], slot_b[kMaxSegments];  // of each product
   uint32_t M, N, Kc;
   uint32_t tile_n;             // columns per tile
-  uint32_t op0, nseg;          // its operand pairs in the launch's list; more than one: an FP32 output (epi 1, 2) that
-                               // receives the products one after the other, as nseg launches would have added them
+  uint32_t nseg;               // products; more than one: an FP32 output (epi 1, 2) that receives them one after the other, as
+                               // nseg launches would have added them
   uint32_t idesc;              // tcgen05 instruction descriptor (formats, majors, shape)
   uint32_t b_desc_hi, b_step;  // B's shared-memory descriptor: high word; address advance (16-byte units) per 32 contraction elements
   uint32_t a_mn, b_mn;         // operand given MN-major (as [Kc, M] / [Kc, N] bytes)
@@ -136,32 +137,32 @@ struct GemmParams {
   CommitParams commit;         // performed by the last CTA to finish (commit.st != null)
 };
 
-constexpr uint32_t kMaxSegments = 8;
-
-// One GEMM as the launch builders take it: everything the kernel needs except what follows from the tile width and the
-// place in the launch (operand list, tile_n, idesc, b_desc_hi, b_step), which is filled from the fields below.
+// One GEMM as the launch builders take it: everything the kernel needs except what follows from the tile width (tmA, tmB,
+// tile_n, idesc, b_desc_hi, b_step), which is filled from the fields below.
 struct GemmDesc : GemmParams {
   uint32_t a_fmt, b_fmt;       // 0 = E4M3, 1 = E5M2
-  struct Operands {
-    const CUtensorMap* mapA;   // [2]: a_map_of(width); the launch reads those of the width it chooses (gemm_width)
-    const CUtensorMap* mapB;   // [kNumTileWidths]
-    const float* alpha_a;
-    const float* alpha_b;
-  } ops[kMaxSegments];
-  GemmDesc() : GemmParams{}, a_fmt(0), b_fmt(0), ops{} { nseg = 1; }
+  const CUtensorMap* mapA;     // [2]: a_map_of(width); the launch reads those of the width it chooses (gemm_width)
+  const CUtensorMap* mapB;     // [kNumTileWidths]
+  GemmDesc() : GemmParams{}, a_fmt(0), b_fmt(0), mapA(nullptr), mapB(nullptr) { nseg = 1; }
+  void operands(const CUtensorMap* a, const float* alphas_a, uint32_t slot_of_a, const CUtensorMap* b, const float* alphas_b, uint32_t slot_of_b) {
+    mapA = a, mapB = b, alpha_a = alphas_a, alpha_b = alphas_b;
+    slot_a[0] = (uint8_t)slot_of_a, slot_b[0] = (uint8_t)slot_of_b;
+  }
+  void add_product(const GemmDesc& d) {  // of another slot
+    slot_a[nseg] = d.slot_a[0], slot_b[nseg] = d.slot_b[0];
+    ++nseg;
+  }
 };
 
 // Independent GEMMs computed by one launch: tiles are numbered problem after problem.
-template <int NP, int NOPS>
+template <int NP>
 struct GemmLaunchParams {
   uint32_t n;
   uint32_t tile_end[NP];       // cumulative tile counts
   uint32_t* ticket;            // counts the CTAs that are done, where a problem has a commit in the tail; else null
   GemmParams prob[NP];
-  GemmOperands op[NOPS];
 };
-constexpr uint32_t kMaxProblems = 16, kMaxOperands = 40;  // of a launch in which a problem has several products
-constexpr uint32_t kMaxSingles = 50;                      // problems of a launch whose problems have one each
+constexpr uint32_t kMaxProblems = 56;  // of a launch: what a kernel's parameter space of 32764 bytes holds
 
 // ORs the status words of up to 64 layers into *out (first chunk: out = OR; later chunks: out |= OR).
 struct StatusGatherParams {
@@ -240,8 +241,7 @@ Launch make_amax_pass2(const AmaxParams& p);
 Launch make_accumulate(const AccumParams& p);
 Launch make_arena_reduce(const ArenaReduceParams& p);
 Launch make_gemm(const GemmDesc& p, int num_sms);
-// One launch for n = 2..kMaxSingles GEMMs of one operand pair each, or 2..kMaxProblems of kMaxOperands pairs at most (each
-// may carry its own commit tail); false if there are more.
+// One launch for n = 2..kMaxProblems GEMMs (each may carry its own commit tail); false if there are more.
 bool make_gemm_group(const GemmDesc* probs, uint32_t n, int num_sms, Launch* out);
 uint32_t gemm_width(const GemmDesc* probs, uint32_t n, int num_sms);  // index of the tile width the launch of these will have
 cudaError_t gemm_prepare();  // opt in to the dynamic shared memory the GEMM needs (once per device)

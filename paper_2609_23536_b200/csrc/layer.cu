@@ -100,14 +100,15 @@ int32_t qe_layer_create(qe_ctx* ctx, const qe_layer_config* cfg, void* ws, uint6
     uint8_t* s = base + k.slot0 + k.per_slot * p;
     L->Xq[p] = s + k.xq;
     L->Gq[p] = s + k.gq;
-    if ((st = make_a_maps(d, L->tmXq_A[p], L->Xq[p], T, K, false)) != QE_OK) break;   // F:  A = Xq  [T,K]
-    if ((st = make_a_maps(d, L->tmGq_A[p], L->Gq[p], T, N, false)) != QE_OK) break;   // dI: A = Gq  [T,N]
-    // dW reads Gq [T,N] and Xq [T,K] as MN-major operands
-    if ((st = make_a_maps(d, L->tmGq_dW[p], L->Gq[p], N, T, true)) != QE_OK) break;
-    if ((st = make_b_maps(d, L->tmXq_dW[p], L->Xq[p], K, T, true)) != QE_OK) break;
   }
-  if (st == QE_OK) st = make_b_maps(d, L->tmWq_B, L->Wq, N, K, false);   // F:  B = Wq [N,K]
-  if (st == QE_OK) st = make_b_maps(d, L->tmWq_dI, L->Wq, K, N, true);   // dI: B = Wq as an MN-major operand
+  // Wq [N,K], and of every slot Xq [T,K] and Gq [T,N], as the GEMMs read them: contraction-major or MN-major
+  const Slots X{L->Xq[0], cfg->slots, k.per_slot}, G{L->Gq[0], cfg->slots, k.per_slot}, W{L->Wq};
+  st = make_a_maps(d, L->tmXq_A, X, T, K, false);
+  if (st == QE_OK) st = make_b_maps(d, L->tmWq_B, W, N, K, false);
+  if (st == QE_OK) st = make_a_maps(d, L->tmGq_A, G, T, N, false);
+  if (st == QE_OK) st = make_b_maps(d, L->tmWq_dI, W, K, N, true);
+  if (st == QE_OK) st = make_a_maps(d, L->tmGq_dW, G, N, T, true);
+  if (st == QE_OK) st = make_b_maps(d, L->tmXq_dW, X, K, T, true);
   if (st != QE_OK) { qe_contract_destroy(L->contract); delete L; return st; }
   // state: histories 0, scales 1, everything else 0
   qe::DevState init{};

@@ -31,15 +31,16 @@ int32_t device_info(int device, DeviceInfo** out) {
 
 // Tensor map over a GEMM operand of `rows` rows: contraction-major bytes [rows, Kc], or (mn) [Kc, rows].  Its box holds box_rows
 // (128, 64 or 32) rows of `blocks` K blocks of 128, one block behind the other: dimensions (byte of the block, row, block) or
-// (row, K row of the block, block).  128 contraction bytes (mn: box_rows bytes) lie together, swizzled over that length.
-int32_t make_map(const DeviceInfo* d, CUtensorMap* map, const void* ptr, uint64_t rows, uint64_t Kc, bool mn, uint32_t box_rows,
+// (row, K row of the block, block), and the tensor's number among those of the same shape that follow at `apart` bytes.  128
+// contraction bytes (mn: box_rows bytes) lie together, swizzled over that length.
+int32_t make_map(const DeviceInfo* d, CUtensorMap* map, const Slots& t, uint64_t rows, uint64_t Kc, bool mn, uint32_t box_rows,
                  uint32_t blocks) {
-  cuuint64_t gdim[3] = {mn ? rows : 128u, mn ? 128u : rows, Kc / 128u};
-  cuuint64_t gstride[2] = {mn ? rows : Kc, mn ? 128u * rows : 128u};
-  cuuint32_t box[3] = {mn ? box_rows : 128u, mn ? 128u : box_rows, blocks};
-  cuuint32_t estr[3] = {1u, 1u, 1u};
+  cuuint64_t gdim[4] = {mn ? rows : 128u, mn ? 128u : rows, Kc / 128u, t.count};
+  cuuint64_t gstride[3] = {mn ? rows : Kc, mn ? 128u * rows : 128u, t.count > 1 ? t.apart : rows * Kc};
+  cuuint32_t box[4] = {mn ? box_rows : 128u, mn ? 128u : box_rows, blocks, 1u};
+  cuuint32_t estr[4] = {1u, 1u, 1u, 1u};
   const CUtensorMapSwizzle sw = box[0] == 128u ? CU_TENSOR_MAP_SWIZZLE_128B : box[0] == 64u ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B;
-  CUresult r = d->encode(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 3, const_cast<void*>(ptr), gdim, gstride, box, estr,
+  CUresult r = d->encode(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 4, const_cast<void*>(t.first), gdim, gstride, box, estr,
                          CU_TENSOR_MAP_INTERLEAVE_NONE, sw, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) return fail(QE_ERR_CUDA, "cuTensorMapEncodeTiled failed with %d", (int)r);
@@ -47,23 +48,23 @@ int32_t make_map(const DeviceInfo* d, CUtensorMap* map, const void* ptr, uint64_
 }
 
 // The map of a GEMM's A operand for launches of one tile width, or of its B operand.
-int32_t make_a_map(const DeviceInfo* d, CUtensorMap* map, const void* ptr, uint64_t M, uint64_t Kc, bool mn, uint32_t width) {
-  return make_map(d, map, ptr, M, Kc, mn, 128, qe::blocks_of(width));
+int32_t make_a_map(const DeviceInfo* d, CUtensorMap* map, const Slots& t, uint64_t M, uint64_t Kc, bool mn, uint32_t width) {
+  return make_map(d, map, t, M, Kc, mn, 128, qe::blocks_of(width));
 }
-int32_t make_b_map(const DeviceInfo* d, CUtensorMap* map, const void* ptr, uint64_t N, uint64_t Kc, bool mn, uint32_t width) {
-  return make_map(d, map, ptr, N, Kc, mn, qe::kTileWidths[width] / 2, qe::blocks_of(width));
+int32_t make_b_map(const DeviceInfo* d, CUtensorMap* map, const Slots& t, uint64_t N, uint64_t Kc, bool mn, uint32_t width) {
+  return make_map(d, map, t, N, Kc, mn, qe::kTileWidths[width] / 2, qe::blocks_of(width));
 }
 // ... for all of them: operands that a layer keeps.
-int32_t make_a_maps(const DeviceInfo* d, CUtensorMap* maps, const void* ptr, uint64_t M, uint64_t Kc, bool mn) {
+int32_t make_a_maps(const DeviceInfo* d, CUtensorMap* maps, const Slots& t, uint64_t M, uint64_t Kc, bool mn) {
   for (uint32_t w = 0; w < 2; ++w) {
-    const int32_t st = make_a_map(d, &maps[qe::a_map_of(w)], ptr, M, Kc, mn, w);
+    const int32_t st = make_a_map(d, &maps[qe::a_map_of(w)], t, M, Kc, mn, w);
     if (st != QE_OK) return st;
   }
   return QE_OK;
 }
-int32_t make_b_maps(const DeviceInfo* d, CUtensorMap* maps, const void* ptr, uint64_t N, uint64_t Kc, bool mn) {
+int32_t make_b_maps(const DeviceInfo* d, CUtensorMap* maps, const Slots& t, uint64_t N, uint64_t Kc, bool mn) {
   for (uint32_t w = 0; w < qe::kNumTileWidths; ++w) {
-    const int32_t st = make_b_map(d, &maps[w], ptr, N, Kc, mn, w);
+    const int32_t st = make_b_map(d, &maps[w], t, N, Kc, mn, w);
     if (st != QE_OK) return st;
   }
   return QE_OK;
@@ -481,7 +482,7 @@ void add_forward(qe_layer* L, uint32_t p, const void* x, void* y, std::vector<qe
   if (x && cast_out) *cast_out = quant_params(L, x, L->Xq[p], T, K, QE_CLASS_X, &L->st->slot_sinv_X[p], QE_E4M3);
   else if (x) ls.push_back(quant_launch(L, x, L->Xq[p], T, K, QE_CLASS_X, &L->st->slot_sinv_X[p], QE_E4M3));
   qe::GemmDesc gp;
-  gp.ops[0] = {L->tmXq_A[p], L->tmWq_B, &L->st->slot_sinv_X[p], &L->st->cache_sinv_W};
+  gp.operands(L->tmXq_A, L->st->slot_sinv_X, p, L->tmWq_B, &L->st->cache_sinv_W, 0);
   gp.M = T;
   gp.N = N;
   gp.Kc = K;
@@ -517,7 +518,7 @@ void add_dI(qe_layer* L, uint32_t p, const void* dy, void* dx, std::vector<qe::L
   if (dy && cast_out) *cast_out = quant_params(L, dy, L->Gq[p], T, N, QE_CLASS_G, &L->st->slot_sinv_G[p], QE_E5M2);
   else if (dy) ls.push_back(quant_launch(L, dy, L->Gq[p], T, N, QE_CLASS_G, &L->st->slot_sinv_G[p], QE_E5M2));
   qe::GemmDesc gp;
-  gp.ops[0] = {L->tmGq_A[p], L->tmWq_dI, &L->st->slot_sinv_G[p], &L->st->cache_sinv_W};
+  gp.operands(L->tmGq_A, L->st->slot_sinv_G, p, L->tmWq_dI, &L->st->cache_sinv_W, 0);
   gp.M = T;
   gp.N = K;
   gp.Kc = N;
@@ -553,7 +554,7 @@ qe::GemmDesc dW_gemm(qe_layer* L, uint32_t p, float* dst, int32_t accumulate, fl
   const uint32_t T = L->cfg.T, K = L->cfg.K, N = L->cfg.N;
   qe::GemmDesc gp;
   // (scales: the snapshots taken when dY_m and X_m were quantised, never the current state)
-  gp.ops[0] = {L->tmGq_dW[p], L->tmXq_dW[p], &L->st->slot_sinv_G[p], &L->st->slot_sinv_X[p]};
+  gp.operands(L->tmGq_dW, L->st->slot_sinv_G, p, L->tmXq_dW, L->st->slot_sinv_X, p);
   gp.M = N;
   gp.N = K;
   gp.Kc = T;

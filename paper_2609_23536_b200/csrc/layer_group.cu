@@ -251,20 +251,11 @@ int32_t together_prepare(qe_ctx* ctx, Prepared* acts, uint32_t n, float* grad, u
 
 // The GEMMs gemms[0..n) in as few launches as hold them, each launch with about as many.
 void push_gemms(qe_ctx* ctx, const qe::GemmDesc* gemms, uint32_t n, std::vector<qe::Launch>& ls) {
-  while (n) {
-    // what the next launch takes: an equal share of what is left, as far as its operand pairs fit
-    uint32_t nops = 0, share = 0;
-    bool sums = false;
-    for (uint32_t i = 0; i < n; ++i) nops += gemms[i].nseg, sums |= gemms[i].nseg > 1;
-    const uint32_t most = sums ? qe::kMaxProblems : qe::kMaxSingles, launches = std::max((n + most - 1) / most, sums ? (nops + qe::kMaxOperands - 1) / qe::kMaxOperands : 1u);
-    const uint32_t want = (n + launches - 1) / launches;
-    nops = 0;
-    while (share < want && (!sums || nops + gemms[share].nseg <= qe::kMaxOperands)) nops += gemms[share++].nseg;
+  for (uint32_t launches = (n + qe::kMaxProblems - 1) / qe::kMaxProblems, share; launches; --launches, gemms += share, n -= share) {
+    share = (n + launches - 1) / launches;
     qe::Launch l;
     if (share >= 2 && qe::make_gemm_group(gemms, share, ctx->dev->num_sms, &l)) ls.push_back(std::move(l));
     else for (uint32_t i = 0; i < share; ++i) ls.push_back(qe::make_gemm(gemms[i], ctx->dev->num_sms));
-    gemms += share;
-    n -= share;
   }
 }
 
@@ -298,8 +289,7 @@ int32_t together_build(qe_ctx* ctx, const Prepared* acts, uint32_t n, float* gra
         std::vector<const qe_layer*>& owner = single ? single_owner : dw_owner;
         const auto sum = std::find(owner.begin(), owner.end(), L);  // this layer's of an earlier microbatch takes this one in
         if (sum != owner.end()) {
-          qe::GemmDesc& g = to[sum - owner.begin()];
-          g.ops[g.nseg++] = gp.ops[0];
+          to[sum - owner.begin()].add_product(gp);
         } else {
           to.push_back(gp);
           owner.push_back(L);
@@ -344,11 +334,7 @@ int32_t together_build(qe_ctx* ctx, const Prepared* acts, uint32_t n, float* gra
     ctx->stats.paired_f_di += !chain.empty() ? 1 : 0;
   }
   // one launch where it holds them all; else weight gradients, which add products up, have launches of their own
-  uint32_t nops = (uint32_t)chain.size();
-  bool sums = false;
-  for (const qe::GemmDesc& g : dw) nops += g.nseg, sums |= g.nseg > 1;
-  const size_t all = chain.size() + dw.size();
-  if (sums ? all <= qe::kMaxProblems && nops <= qe::kMaxOperands : all <= qe::kMaxSingles) {
+  if (chain.size() + dw.size() <= qe::kMaxProblems) {
     chain.insert(chain.end(), dw.begin(), dw.end());
     dw.clear();
   }
@@ -492,7 +478,7 @@ bool tensors_apart(qe_layer* const* layers, uint32_t n_layers, const qe_step_act
 }
 
 // Actions of a round of a list whose tensors are apart: forwards and input gradients for two launches.
-constexpr uint32_t kApartGroup = 2 * qe::kMaxSingles;
+constexpr uint32_t kApartGroup = 2 * qe::kMaxProblems;
 }  // namespace
 
 int32_t qe_step_run(qe_ctx* ctx, qe_layer* const* layers, uint32_t n_layers, const qe_step_action* actions,

@@ -37,10 +37,16 @@ struct DeviceInfo {
 
 int32_t device_info(int device, DeviceInfo** out);
 int32_t current_device_info(DeviceInfo** d);
-int32_t make_a_map(const DeviceInfo* d, CUtensorMap* map, const void* ptr, uint64_t M, uint64_t Kc, bool mn, uint32_t width);
-int32_t make_b_map(const DeviceInfo* d, CUtensorMap* map, const void* ptr, uint64_t N, uint64_t Kc, bool mn, uint32_t width);
-int32_t make_a_maps(const DeviceInfo* d, CUtensorMap* maps, const void* ptr, uint64_t M, uint64_t Kc, bool mn);
-int32_t make_b_maps(const DeviceInfo* d, CUtensorMap* maps, const void* ptr, uint64_t N, uint64_t Kc, bool mn);
+// Operand tensors of one shape, `apart` bytes from one to the next (one tensor: any).
+struct Slots {
+  const void* first;
+  uint32_t count = 1;
+  uint64_t apart = 0;
+};
+int32_t make_a_map(const DeviceInfo* d, CUtensorMap* map, const Slots& t, uint64_t M, uint64_t Kc, bool mn, uint32_t width);
+int32_t make_b_map(const DeviceInfo* d, CUtensorMap* map, const Slots& t, uint64_t N, uint64_t Kc, bool mn, uint32_t width);
+int32_t make_a_maps(const DeviceInfo* d, CUtensorMap* maps, const Slots& t, uint64_t M, uint64_t Kc, bool mn);
+int32_t make_b_maps(const DeviceInfo* d, CUtensorMap* maps, const Slots& t, uint64_t N, uint64_t Kc, bool mn);
 int32_t make_out_map(const DeviceInfo* d, CUtensorMap* map, const void* ptr, uint64_t M, uint64_t N, uint64_t ldo, bool fp32);
 int32_t make_out_map_u8(const DeviceInfo* d, CUtensorMap* map, const void* ptr, uint64_t M, uint64_t N, uint64_t ld);
 inline uint64_t align_up(uint64_t v, uint64_t a) { return (v + a - 1) / a * a; }
@@ -95,9 +101,8 @@ struct qe_layer {
   uint8_t* Wq = nullptr;
   uint8_t *x_stage = nullptr, *dx_stage = nullptr, *y_stage = nullptr, *dy_stage = nullptr;  // host_io only
   uint8_t *Xq[QE_MAX_SLOTS], *Gq[QE_MAX_SLOTS];
-  // tensor maps: two per tensor in the A role (a_map_of), one per tile width in the B role
-  CUtensorMap tmXq_A[QE_MAX_SLOTS][2], tmGq_A[QE_MAX_SLOTS][2], tmGq_dW[QE_MAX_SLOTS][2], tmXq_dW[QE_MAX_SLOTS][qe::kNumTileWidths];
-  CUtensorMap tmWq_B[qe::kNumTileWidths], tmWq_dI[qe::kNumTileWidths];  // B of the forward; B of dI (MN-major)
+  // tensor maps over all slots (A and B roles: a_map_of, tile widths): forward, input gradient, weight gradient (MN-major)
+  CUtensorMap tmXq_A[2], tmWq_B[qe::kNumTileWidths], tmGq_A[2], tmWq_dI[qe::kNumTileWidths], tmGq_dW[2], tmXq_dW[qe::kNumTileWidths];
   ActionGraph gF[QE_MAX_SLOTS], gDI[QE_MAX_SLOTS], gDW[QE_MAX_SLOTS], gDWs[QE_MAX_SLOTS], gRefresh, gCommit;
   // QE_CTX_OVERLAP_DW: per slot, "dI of the tape in this slot has been enqueued" / "the dW that released it has"
   cudaEvent_t ev_di[QE_MAX_SLOTS] = {}, ev_dw[QE_MAX_SLOTS] = {};
@@ -182,7 +187,7 @@ struct DWBatch {
   uint32_t limit;
   std::vector<qe::GemmDesc> gp;
   std::vector<qe_layer*> layer;
-  explicit DWBatch(uint32_t n_layers) : limit(n_layers > 8 ? qe::kMaxProblems : 4) {}
+  explicit DWBatch(uint32_t n_layers) : limit(n_layers > 8 ? QE_MAX_MULTI_DW : 4) {}
   bool has(const qe_layer* L) const { return std::find(layer.begin(), layer.end(), L) != layer.end(); }
   void flush(qe_ctx* ctx, std::vector<qe::Launch>& ls) {
     std::vector<qe::GemmDesc> paired;

@@ -85,7 +85,7 @@ static int32_t standalone_gemm(DeviceInfo* dev, const void* a, uint32_t a_fmt, u
   if ((((uintptr_t)a | (uintptr_t)b | (uintptr_t)d) & 15u)) return fail(QE_ERR_BAD_ARG, "misaligned pointer");
   int32_t st;
   qe::GemmDesc& gp = sg->desc;
-  gp.ops[0] = {sg->mapA, sg->mapB, alpha_a, alpha_b};
+  gp.operands(sg->mapA, alpha_a, 0, sg->mapB, alpha_b, 0);
   gp.M = M;
   gp.N = Nn;
   gp.Kc = Kc;
@@ -103,8 +103,8 @@ static int32_t standalone_gemm(DeviceInfo* dev, const void* a, uint32_t a_fmt, u
 }
 
 static int32_t standalone_maps(DeviceInfo* dev, StandaloneGemm* sg, const void* a, const void* b, uint32_t width) {
-  const int32_t st = make_a_map(dev, &sg->mapA[qe::a_map_of(width)], a, sg->desc.M, sg->desc.Kc, sg->desc.a_mn != 0, width);
-  return st != QE_OK ? st : make_b_map(dev, &sg->mapB[width], b, sg->desc.N, sg->desc.Kc, sg->desc.b_mn != 0, width);
+  const int32_t st = make_a_map(dev, &sg->mapA[qe::a_map_of(width)], Slots{a}, sg->desc.M, sg->desc.Kc, sg->desc.a_mn != 0, width);
+  return st != QE_OK ? st : make_b_map(dev, &sg->mapB[width], Slots{b}, sg->desc.N, sg->desc.Kc, sg->desc.b_mn != 0, width);
 }
 
 int32_t qe_gemm_fp8_ex(const void* a, uint32_t a_fmt, uint32_t a_mn, const void* b, uint32_t b_fmt, uint32_t b_mn,
