@@ -165,7 +165,10 @@ int32_t qe_contract_dW_check(const qe_contract* c, const qe_tape* t, uint64_t de
     return fail(QE_ERR_DEST, "differs from the destination bound for this epoch");
   if (c->registry) {
     std::lock_guard<std::mutex> g(c->registry->mu);
-    for (const auto& kv : c->registry->bound)
+    const auto own = c->registry->bound.find(c);
+    // (a range that is bound already was compared when it was, and every later one with it)
+    const bool bound = own != c->registry->bound.end() && own->second.lo == lo && own->second.hi == hi;
+    if (!bound) for (const auto& kv : c->registry->bound)
       if (kv.first != c && kv.second.lo < hi && lo < kv.second.hi)
         return fail(QE_ERR_DEST, "destination aliases another layer's slice");
   }

@@ -16,7 +16,7 @@
 //               FP32 accumulation straight into the destination (direct gradient placement): the addition is done in
 //               L2, one per element and launch, and the destination tile is prefetched into L2 while the tile's
 //               main loop runs.  The reduction is a plain round-to-nearest FP32 addition (subnormal values kept).
-//   The launch may also carry up to sixteen independent problems (grouped launch): tiles are numbered problem after
+//   The launch may also carry up to fifty-six independent problems (grouped launch): tiles are numbered problem after
 //   problem and each role looks its tile's problem up, so that one set of persistent CTAs packs them all.
 //   A problem may be the sum of several products (the deferred weight gradients of several microbatches): each gets an
 //   accumulator of its own, and the epilogue adds them up in registers before the one store.

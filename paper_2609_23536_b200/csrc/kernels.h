@@ -148,8 +148,8 @@ struct GemmDesc : GemmParams {
     mapA = a, mapB = b, alpha_a = alphas_a, alpha_b = alphas_b;
     slot_a[0] = (uint8_t)slot_of_a, slot_b[0] = (uint8_t)slot_of_b;
   }
-  void add_product(const GemmDesc& d) {  // of another slot
-    slot_a[nseg] = d.slot_a[0], slot_b[nseg] = d.slot_b[0];
+  void add_product(uint32_t slot_of_a, uint32_t slot_of_b) {
+    slot_a[nseg] = (uint8_t)slot_of_a, slot_b[nseg] = (uint8_t)slot_of_b;
     ++nseg;
   }
 };

@@ -481,7 +481,8 @@ void add_forward(qe_layer* L, uint32_t p, const void* x, void* y, std::vector<qe
   const uint32_t T = L->cfg.T, K = L->cfg.K, N = L->cfg.N;
   if (x && cast_out) *cast_out = quant_params(L, x, L->Xq[p], T, K, QE_CLASS_X, &L->st->slot_sinv_X[p], QE_E4M3);
   else if (x) ls.push_back(quant_launch(L, x, L->Xq[p], T, K, QE_CLASS_X, &L->st->slot_sinv_X[p], QE_E4M3));
-  qe::GemmDesc gp;
+  qe::GemmDesc own;
+  qe::GemmDesc& gp = gemm_out ? *gemm_out : own;  // (as it was made: nothing set yet)
   gp.operands(L->tmXq_A, L->st->slot_sinv_X, p, L->tmWq_B, &L->st->cache_sinv_W, 0);
   gp.M = T;
   gp.N = N;
@@ -506,8 +507,7 @@ void add_forward(qe_layer* L, uint32_t p, const void* x, void* y, std::vector<qe
   gp.status = &L->st->status;
   gp.commit = commit_params(L, 1u << QE_CLASS_Y, 1, nullptr);  // done by the GEMM's last CTA ...
   gp.commit.early_mask = 1u << QE_CLASS_X;                     // ... and by its first, once the cast before it is complete
-  if (gemm_out) *gemm_out = gp;
-  else ls.push_back(qe::make_gemm(gp, L->ctx->dev->num_sms));
+  if (!gemm_out) ls.push_back(qe::make_gemm(gp, L->ctx->dev->num_sms));
 }
 
 // Hand-off in the backward direction: the input gradient of `L` is the output gradient of the linear before it
@@ -517,7 +517,8 @@ void add_dI(qe_layer* L, uint32_t p, const void* dy, void* dx, std::vector<qe::L
   const uint32_t T = L->cfg.T, K = L->cfg.K, N = L->cfg.N;
   if (dy && cast_out) *cast_out = quant_params(L, dy, L->Gq[p], T, N, QE_CLASS_G, &L->st->slot_sinv_G[p], QE_E5M2);
   else if (dy) ls.push_back(quant_launch(L, dy, L->Gq[p], T, N, QE_CLASS_G, &L->st->slot_sinv_G[p], QE_E5M2));
-  qe::GemmDesc gp;
+  qe::GemmDesc own;
+  qe::GemmDesc& gp = gemm_out ? *gemm_out : own;  // (as it was made: nothing set yet)
   gp.operands(L->tmGq_A, L->st->slot_sinv_G, p, L->tmWq_dI, &L->st->cache_sinv_W, 0);
   gp.M = T;
   gp.N = K;
@@ -544,8 +545,7 @@ void add_dI(qe_layer* L, uint32_t p, const void* dy, void* dx, std::vector<qe::L
   gp.status = &L->st->status;
   gp.commit = commit_params(L, 0, 1, nullptr);  // backward amax/scale updated exactly once, here: the cast (or the
   gp.commit.early_mask = 1u << QE_CLASS_G;      // hand-off) that made Gq has completed the amax before this GEMM starts
-  if (gemm_out) *gemm_out = gp;
-  else ls.push_back(qe::make_gemm(gp, L->ctx->dev->num_sms));
+  if (!gemm_out) ls.push_back(qe::make_gemm(gp, L->ctx->dev->num_sms));
 }
 
 // The weight-gradient GEMM of slot p; dst = first element of the layer's gradient slice, temp != null makes it

@@ -266,15 +266,19 @@ void push_gemms(qe_ctx* ctx, const qe::GemmDesc* gemms, uint32_t n, std::vector<
 // may overlap what is before them)
 int32_t together_build(qe_ctx* ctx, const Prepared* acts, uint32_t n, float* grad, std::vector<qe::Launch>& ls, Fnv* h,
                        std::vector<qe::QuantParams>* refresh = nullptr, bool apart = false, bool early = false) {
-  std::vector<qe::GemmDesc> chain, dw, singles;  // F and dI; weight gradients; those that go out one by one
-  std::vector<const qe_layer*> dw_owner, single_owner;
-  std::vector<qe::QuantParams> casts;
-  chain.reserve(n);
-  casts.reserve(n);
-  for (int pass = 0; pass < 2; ++pass) {  // F and dI first (others wait for them), the weight gradients' tiles after theirs
+  // The order of the launches' problems is settled before they are built: F and dI first (others wait for them), the weight
+  // gradients' tiles after theirs; the longest tiles first (their contraction length decides a tile's duration), so that a
+  // launch's last, partial wave is made of short ones (weight gradients: contraction over the tokens of all products).
+  struct Product { const Prepared* first; uint32_t n; };  // a weight gradient: its first microbatch's action, its products
+  std::vector<const Prepared*> chain_of;
+  std::vector<Product> dw_of;
+  const auto dw_product = [&](const qe_layer* L) {
+    return std::find_if(dw_of.begin(), dw_of.end(), [&](const Product& d) { return d.first->layer == L; });
+  };
+  chain_of.reserve(n);
+  for (int pass = 0; pass < 2; ++pass)
     for (uint32_t i = 0; i < n; ++i) {
       const Prepared& a = acts[i];
-      qe_layer* L = a.layer;
       if ((a.kind == QE_ACT_DW) != (pass == 1)) continue;
       if (h) {
         h->mix(&a.kind, sizeof(a.kind));
@@ -282,64 +286,64 @@ int32_t together_build(qe_ctx* ctx, const Prepared* acts, uint32_t n, float* gra
         h->mix(&a.slot, sizeof(uint32_t));
         h->mix(&a.refresh, sizeof(int32_t));
       }
-      if (a.kind == QE_ACT_DW) {
-        const qe::GemmDesc gp = dW_gemm(L, a.slot, grad + a.grad_offset, a.acc, nullptr);
-        const bool single = !apart && !qe::whole_row_tiles(gp.M);  // a half-filled last row tile: a launch of its own
-        std::vector<qe::GemmDesc>& to = single ? singles : dw;
-        std::vector<const qe_layer*>& owner = single ? single_owner : dw_owner;
-        const auto sum = std::find(owner.begin(), owner.end(), L);  // this layer's of an earlier microbatch takes this one in
-        if (sum != owner.end()) {
-          to[sum - owner.begin()].add_product(gp);
-        } else {
-          to.push_back(gp);
-          owner.push_back(L);
-        }
-        continue;
-      }
-      qe::GemmDesc gp;
-      qe::QuantParams cast;
-      if (a.kind == QE_ACT_F) {
-        if (L->dw_pending[a.slot]) {
-          QE_CUDA(cudaStreamWaitEvent(ctx->exec_stream, L->ev_dw[a.slot], 0));
-          L->dw_pending[a.slot] = false;
-        }
-        if (a.refresh && refresh) refresh->push_back(refresh_params(L));
-        else if (a.refresh) add_refresh(L, ls);
-        add_forward(L, a.slot, a.in_dev, a.out_dev, ls, nullptr, 0, &gp, &cast);
+      if (pass == 0) {
+        chain_of.push_back(&a);
       } else {
-        add_dI(L, a.slot, a.in_dev, a.out_dev, ls, nullptr, 0, &gp, &cast);
-      }
-      casts.push_back(cast);
-      gp.commit.hold_trigger = apart;
-      if (apart || qe::whole_row_tiles(gp.M)) {
-        chain.push_back(gp);
-      } else {
-        singles.push_back(gp);
-        single_owner.push_back(nullptr);
+        const auto sum = dw_product(a.layer);  // this layer's of an earlier microbatch takes this one in
+        if (sum != dw_of.end()) sum->n += 1;
+        else dw_of.push_back({&a, 1});
       }
     }
+  const auto contraction = [](const Prepared* a) { return a->kind == QE_ACT_F ? a->layer->cfg.K : a->layer->cfg.N; };
+  std::stable_sort(chain_of.begin(), chain_of.end(), [&](const Prepared* x, const Prepared* y) { return contraction(x) > contraction(y); });
+  std::stable_sort(dw_of.begin(), dw_of.end(), [](const Product& x, const Product& y) { return x.first->layer->cfg.T * x.n > y.first->layer->cfg.T * y.n; });
+  std::vector<qe::GemmDesc> gemms, singles;  // those that share launches; those that go out one by one: half-filled last row tiles
+  std::vector<qe::QuantParams> casts(chain_of.size());
+  gemms.reserve(chain_of.size() + dw_of.size());
+  const auto place = [&](uint32_t M) -> qe::GemmDesc& {
+    std::vector<qe::GemmDesc>& to = apart || qe::whole_row_tiles(M) ? gemms : singles;
+    to.emplace_back();
+    return to.back();
+  };
+  for (size_t i = 0; i < chain_of.size(); ++i) {
+    const Prepared& a = *chain_of[i];
+    qe_layer* L = a.layer;
+    qe::GemmDesc& gp = place(L->cfg.T);
+    if (a.kind == QE_ACT_F) {
+      if (L->dw_pending[a.slot]) {
+        QE_CUDA(cudaStreamWaitEvent(ctx->exec_stream, L->ev_dw[a.slot], 0));
+        L->dw_pending[a.slot] = false;
+      }
+      if (a.refresh && refresh) refresh->push_back(refresh_params(L));
+      else if (a.refresh) add_refresh(L, ls);
+      add_forward(L, a.slot, a.in_dev, a.out_dev, ls, nullptr, 0, &gp, &casts[i]);
+    } else {
+      add_dI(L, a.slot, a.in_dev, a.out_dev, ls, nullptr, 0, &gp, &casts[i]);
+    }
+    gp.commit.hold_trigger = apart;
   }
-  // longest tiles first (their contraction length decides a tile's duration): the launch's last, partial wave is then
-  // made of short tiles.  The weight gradients (contraction over T only) stay behind the others.
-  std::stable_sort(chain.begin(), chain.end(), [](const qe::GemmDesc& x, const qe::GemmDesc& y) { return x.Kc > y.Kc; });
-  std::stable_sort(dw.begin(), dw.end(), [](const qe::GemmDesc& x, const qe::GemmDesc& y) { return x.Kc * x.nseg > y.Kc * y.nseg; });
+  const uint32_t n_chain = (uint32_t)gemms.size();
+  for (const Product& d : dw_of) {
+    qe::GemmDesc& gp = place(d.first->layer->cfg.N);
+    gp = dW_gemm(d.first->layer, d.first->slot, grad + d.first->grad_offset, d.first->acc, nullptr);
+    for (const Prepared* a = d.first + 1; gp.nseg < d.n; ++a)
+      if (a->kind == QE_ACT_DW && a->layer == d.first->layer) gp.add_product(a->slot, a->slot);
+  }
+  const uint32_t n_gemms = (uint32_t)gemms.size();
   for (size_t i = 0; i < casts.size(); i += qe::kMaxCasts) {  // all casts of the call in one launch
     const uint32_t m = (uint32_t)std::min<size_t>(qe::kMaxCasts, casts.size() - i);
     casts[i].early = early;
     ls.push_back(m > 1 || early ? qe::make_quantize_multi(&casts[i], m) : qe::make_quantize(casts[i]));
   }
   for (const qe::GemmDesc& gp : singles) ls.push_back(qe::make_gemm(gp, ctx->dev->num_sms));
-  if (chain.size() + dw.size() >= 2) {
-    ctx->stats.grouped_dw += dw.size();
-    ctx->stats.paired_f_di += !chain.empty() ? 1 : 0;
+  if (n_gemms >= 2) {
+    ctx->stats.grouped_dw += n_gemms - n_chain;
+    ctx->stats.paired_f_di += n_chain ? 1 : 0;
   }
   // one launch where it holds them all; else weight gradients, which add products up, have launches of their own
-  if (chain.size() + dw.size() <= qe::kMaxProblems) {
-    chain.insert(chain.end(), dw.begin(), dw.end());
-    dw.clear();
-  }
-  push_gemms(ctx, chain.data(), (uint32_t)chain.size(), ls);
-  push_gemms(ctx, dw.data(), (uint32_t)dw.size(), ls);
+  const uint32_t together = n_gemms <= qe::kMaxProblems ? n_gemms : n_chain;
+  push_gemms(ctx, gemms.data(), together, ls);
+  push_gemms(ctx, gemms.data() + together, n_gemms - together, ls);
   return QE_OK;
 }
 
@@ -654,10 +658,10 @@ int32_t qe_step_run(qe_ctx* ctx, qe_layer* const* layers, uint32_t n_layers, con
       k = rounds[r][0];
     }
     // A long list goes out in pieces (in graph mode each a graph of its own), so that the device works on one while the host
-    // prepares the next: a first one soon, later ones so long that the gaps between graphs do not count (48 linears, 32
-    // microbatches: 3.4 of 16.4 ms were host time ahead of the one launch).
+    // prepares the next: a first one soon, the next while that one runs, later ones so long that the gaps between graphs do
+    // not count (48 linears, 32 microbatches: 3.4 of 16.4 ms were host time ahead of the one launch).
     waiting += (uint32_t)acts.size();
-    if (st == QE_OK && waiting >= (pieces ? 384u : 96u) && r + 1 < rounds.size()) {
+    if (st == QE_OK && waiting >= (pieces < 2 ? 96u << pieces : 384u) && r + 1 < rounds.size()) {
       put_refresh();
       run_status = run_piece(ls, true);
       ls.clear();
