@@ -334,6 +334,7 @@ struct Problems {
   __device__ __forceinline__ const GemmParams& first() const { return g.prob[0]; }
   __device__ __forceinline__ const CommitParams& commit(uint32_t i) const { return g.prob[i].commit; }
   __device__ __forceinline__ uint32_t* ticket() const { return g.ticket; }
+  __device__ __forceinline__ const CommitParams& before() const { return g.before; }
   __device__ __forceinline__ uint32_t* status_of(uint32_t i) const { return g.prob[i].status; }
 };
 
@@ -461,6 +462,10 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
       grid_dep_launch();
     }
   }
+
+  // The output's class of a chained forward before this one: its amax is complete too, and no tail of its own was spent on it.
+  if (PS::ONE && warp == EPI_WARP0 + 6 && blockIdx.x == 0 && ps.before().st)
+    commit_class<false>(ps.before(), ps.before().class_mask, false, true, lane);
 
   // (The roles are one flat choice: with producer and issuer nested under a choice of their own, or written as lambdas, the
   // same code ran 4 % slower, small launches and large ones alike.)
@@ -917,6 +922,7 @@ Launch make_launch(const GemmDesc* probs, uint32_t n, int num_sms, const void* f
   }
   std::memcpy(at + offsetof(P, n), &n, sizeof(n));
   std::memcpy(at + offsetof(P, ticket), &ticket, sizeof(ticket));
+  if (NP == 1) std::memcpy(at + offsetof(P, before), &probs->before, sizeof(CommitParams));
   l.func = func;
   l.grid = dim3(ctas * (tiles < most ? tiles : most), 1, 1);
   l.block = dim3(threads_of(sums), 1, 1);

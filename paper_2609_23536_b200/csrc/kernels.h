@@ -143,6 +143,7 @@ struct GemmDesc : GemmParams {
   uint32_t a_fmt, b_fmt;       // 0 = E4M3, 1 = E5M2
   const CUtensorMap* mapA;     // [2]: a_map_of(width); the launch reads those of the width it chooses (gemm_width)
   const CUtensorMap* mapB;     // [kNumTileWidths]
+  CommitParams before{};       // of a launch of its own: GemmLaunchParams::before
   GemmDesc() : GemmParams{}, a_fmt(0), b_fmt(0), mapA(nullptr), mapB(nullptr) { nseg = 1; }
   void operands(const CUtensorMap* a, const float* alphas_a, uint32_t slot_of_a, const CUtensorMap* b, const float* alphas_b, uint32_t slot_of_b) {
     mapA = a, mapB = b, alpha_a = alphas_a, alpha_b = alphas_b;
@@ -160,6 +161,7 @@ struct GemmLaunchParams {
   uint32_t n;
   uint32_t tile_end[NP];       // cumulative tile counts
   uint32_t* ticket;            // counts the CTAs that are done, where a problem has a commit in the tail; else null
+  CommitParams before;         // launches of one problem: a class whose amax the launch before completed (before.st != null)
   GemmParams prob[NP];
 };
 constexpr uint32_t kMaxProblems = 56;  // of a launch: what a kernel's parameter space of 32764 bytes holds
