@@ -57,15 +57,16 @@ __device__ __forceinline__ void transpose4x4(const uint32_t a0, const uint32_t a
 // bytes of every output row of the transposed copy).
 constexpr int kQuantThreads = 256;
 
-// One block's share (256 rows x 64 columns at block coordinates bx, by) of a cast; wmax: 8 shared words.
-template <int FMT>
+// One block's share (256 rows x 64 columns at block coordinates bx, by) of a cast; wmax: 8 shared words.  L2: the scale is read
+// there (a launch that does not wait for the kernel before it); a lone cast, whose reads it would slow, does not.
+template <int FMT, bool L2 = false>
 __device__ __forceinline__ void quantize_block(const QuantParams& p, uint32_t bx, uint32_t by, uint32_t* wmax) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int rb = lane >> 3, cv = lane & 7;
   const uint32_t row0 = by * 256u + warp * 32u + rb * 8u;
   const uint32_t col0 = bx * 64u + cv * 8u;
-  const float scale = __ldcg(p.scale);
-  if (bx == 0 && by == 0 && threadIdx.x == 0 && p.sinv_dst) *p.sinv_dst = __ldcg(p.sinv_src);
+  const float scale = L2 ? __ldcg(p.scale) : *p.scale;
+  if (bx == 0 && by == 0 && threadIdx.x == 0 && p.sinv_dst) *p.sinv_dst = L2 ? __ldcg(p.sinv_src) : *p.sinv_src;
 
   uint32_t m = 0;
   if (row0 < p.rows) {  // warp-uniform up to rb; rows is a multiple of 8 so a thread's 8 rows are all in or out
@@ -147,8 +148,8 @@ __global__ void __launch_bounds__(kQuantThreads, 6) quantize_multi_kernel(const 
   grid_dep_launch();
   const QuantParams& p = mp.q[which];
   const uint32_t b = blockIdx.x - base, bxn = p.cols / 64u;
-  if (p.fmt == 0) quantize_block<0>(p, b % bxn, b / bxn, wmax);
-  else quantize_block<1>(p, b % bxn, b / bxn, wmax);
+  if (p.fmt == 0) quantize_block<0, true>(p, b % bxn, b / bxn, wmax);
+  else quantize_block<1, true>(p, b % bxn, b / bxn, wmax);
   if (p.commit.st) {  // the last block of this cast
     auto sync = [] { __syncthreads(); };
     if (last_block(&p.commit.st->ticket, mp.block_end[which] - base, threadIdx.x, &last_flag, sync))
