@@ -128,6 +128,14 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
   }
 }
 
+// The same wait by a whole warp (converged).  Its lanes leave it together and with one answer: a lane that was still polling
+// while the elected one went on to issue could find the barrier a phase further, take that for the phase it waits for not being
+// over, and wait on; no lane may give up alone either.
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile uint32_t* abort_flag, uint32_t* status,
+                                               uint32_t err_bit) {
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag, status, err_bit));
+}
+
 // Arrival on a barrier that may live in the peer CTA.  What it announces are tensor-memory reads, ordered by the
 // tcgen05 fences on both sides, so it need not be a release at cluster scope: that waits for the thread's outstanding
 // stores too, ~1000 clocks per drained accumulator.
@@ -493,7 +501,7 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
         const CUtensorMap *tmA = &p.tmA, *tmB = &p.tmB;
         const int sa = p.slot_a[SUMS ? seg : 0u], sb = p.slot_b[SUMS ? seg : 0u];
         for (uint32_t kb = 0; kb < num_kb; kb += ring.blocks) {
-          if (!(ok = mbar_wait(empty_bar(s), ph ^ 1u, abort_flag, status, ERR_PRODUCER))) break;
+          if (!(ok = mbar_wait_warp(empty_bar(s), ph ^ 1u, abort_flag, status, ERR_PRODUCER))) break;
           const uint32_t a_dst = smem_base + s * ring.stage_bytes, b_dst = a_dst + ring.b_offset();
           if (elected) {
             if (rank == 0) mbar_expect_tx(full_bar(s), bytes);
@@ -524,11 +532,11 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
         const uint32_t idesc = p.idesc, b_hi = p.b_desc_hi, a_step = p.a_mn ? 256u : 2u, b_step = p.b_step;
         const uint32_t b_block = tile_n / CTAS * BK / 16u;  // from one block of B in a stage to the next
         for (uint32_t seg = 0; ok && seg < (SUMS ? p.nseg : 1u); ++seg) {  // an accumulator of its own for each product
-          if (!(ok = mbar_wait(tempty_bar(acc), acc_ph ^ 1u, abort_flag, status, ERR_MMA))) break;
+          if (!(ok = mbar_wait_warp(tempty_bar(acc), acc_ph ^ 1u, abort_flag, status, ERR_MMA))) break;
           tc_fence_after();
           const uint32_t d_tmem = tmem_base + acc * ACC_COLS;
           for (uint32_t kb = 0; kb < num_kb; kb += ring.blocks) {
-            if (!(ok = mbar_wait(full_bar(s), ph, abort_flag, status, ERR_MMA))) break;
+            if (!(ok = mbar_wait_warp(full_bar(s), ph, abort_flag, status, ERR_MMA))) break;
             tc_fence_after();
             const uint32_t a_src = smem_base + s * ring.stage_bytes, b_src = a_src + ring.b_offset();
             const uint64_t adesc = make_desc(a_src, A_DESC_HI);

@@ -268,6 +268,22 @@ def test_gemm_narrow_tiles_of_any_contraction_integer_exact(qe, M, Nn, Kc, a_mn,
     assert torch.equal(out.double(), a.double() @ b.double().t()) and status.item() == 0  # sums below 2^24: exact
 
 
+@pytest.mark.parametrize("M,Nn", [(256, 256), (512, 4096), (256, 16384), (1152, 4096)])  # 64, 128, 256 columns; a CTA to a tile
+def test_gemm_goes_round_the_ring_of_stages_many_times(qe, M, Nn):
+    """Producer and issuer meet at every barrier some forty times, without one lane of theirs falling behind the others."""
+    g = torch.Generator(device=DEV).manual_seed(M + Nn)
+    a, b = (torch.randint(-3, 4, shape, generator=g, device=DEV).float() for shape in ((M, 16384), (Nn, 16384)))
+    to8 = lambda t: t.to(torch.float8_e4m3fn).view(torch.uint8)  # noqa: E731
+    one, status = torch.ones(1, device=DEV), torch.zeros(1, dtype=torch.int32, device=DEV)
+    A, B, want = to8(a), to8(b), (a.double() @ b.double().t()).float()  # sums below 2^24: exact
+    out = torch.zeros((M, Nn), device=DEV)
+    for _ in range(50):
+        qe.qe_gemm_fp8_ex(A, 0, False, B, 0, False, one, one, out, 1, None, status)
+        assert torch.equal(out, want)
+        out.zero_()
+    assert status.item() == 0
+
+
 @pytest.mark.parametrize("M,Nn,Kc", [(1152, 8192, 640), (384, 11008, 384), (1152, 1920, 2176)])
 @pytest.mark.parametrize("kind", [0, 1, 2])
 def test_odd_row_counts_give_the_bits_of_even_ones(qe, M, Nn, Kc, kind):
