@@ -342,6 +342,8 @@ struct Problems {
   __device__ __forceinline__ const GemmParams& first() const { return g.prob[0]; }
   __device__ __forceinline__ const CommitParams& commit(uint32_t i) const { return g.prob[i].commit; }
   __device__ __forceinline__ uint32_t* ticket() const { return g.ticket; }
+  __device__ __forceinline__ uint32_t* commits() const { return g.commits; }
+  __device__ __forceinline__ uint32_t commits_op() const { return g.commits_op; }
   __device__ __forceinline__ const CommitParams& before() const { return g.before; }
   __device__ __forceinline__ uint32_t* status_of(uint32_t i) const { return g.prob[i].status; }
 };
@@ -452,7 +454,7 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
   // Everything above (barriers, tensor memory) touched no data a predecessor produces and may overlap the previous
   // kernel's tail; operands, scales and the destination may come from it, so wait for it here.
   grid_dep_wait();
-  const bool hold = blockIdx.x < ps.count() && ps.commit(blockIdx.x).hold_trigger;
+  const bool hold = blockIdx.x < ps.count() && ps.commits_op() == 1u;
   if (!hold) grid_dep_launch();
   if (blockIdx.x == 0 && threadIdx.x == EPI_WARP0 * 32) {  // FP8 hand-off: the consumer's tape snapshot of its inverse scale
     const GemmParams& q = ps.first();
@@ -464,8 +466,14 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
     // are snapshots), so only the output's class is left for the launch's tail.
     const CommitParams& c = ps.commit(blockIdx.x);
     if (c.st && c.early_mask) commit_class<false>(c, c.early_mask, c.bump_token != 0, true, lane);
+    if (ps.commits_op() && lane == 0) {
+      if (!hold) *ps.commits() = 0u;
+      else {
+        __threadfence();
+        atomicAdd(ps.commits(), 1u);
+      }
+    }
     if (hold) {
-      __threadfence();
       __syncwarp();
       grid_dep_launch();
     }
@@ -972,6 +980,21 @@ bool make_gemm_group(const GemmDesc* probs, uint32_t n, int num_sms, Launch* out
   *out = make_any(probs, n, num_sms);
   return true;
 }
+
+// (the fields stand at the front of every launch's parameter block)
+static void set_commits(Launch* l, uint32_t* word, uint32_t op) {
+  using P = GemmLaunchParams<1>;
+  static_assert(offsetof(P, commits) == 0 && offsetof(P, n) == offsetof(GemmLaunchParams<kMaxProblems>, n), "");
+  std::memcpy(l->params.data() + offsetof(P, commits), &word, sizeof(word));
+  std::memcpy(l->params.data() + offsetof(P, commits_op), &op, sizeof(op));
+}
+uint32_t announce_commits(Launch* gemm, uint32_t* word) {
+  set_commits(gemm, word, 1u);
+  uint32_t n;
+  std::memcpy(&n, gemm->params.data() + offsetof(GemmLaunchParams<1>, n), sizeof(n));
+  return n;
+}
+void withdraw_commits(Launch* gemm, uint32_t* word) { set_commits(gemm, word, 2u); }
 
 uint32_t gemm_width(const GemmDesc* probs, uint32_t n, int num_sms) { return choose_width(probs, n, (uint32_t)num_sms / 2u); }
 

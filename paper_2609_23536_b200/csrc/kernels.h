@@ -27,7 +27,8 @@ struct DevState {
   uint32_t ticket;             // "last CTA" counter of the kernel whose tail performs the commit; self-resetting
   uint32_t wmax[4];            // bit pattern of max(history ring) per class, kept by the commit (derived state)
   uint32_t status_all;         // scratch of the multi-layer boundary: OR of several layers' status words
-  uint32_t pad[38];            // header is 768 bytes; history rings [4][H] follow
+  uint32_t commits;            // whole-step calls whose first layer this is: Announce::word
+  uint32_t pad[37];            // header is 768 bytes; history rings [4][H] follow
 };
 static_assert(sizeof(DevState) == 768, "DevState layout");
 
@@ -40,8 +41,7 @@ struct CommitParams {
   uint32_t early_mask;         // GEMM launches: classes whose amax is complete when the launch starts (committed then, with
                                // the token); class_mask holds the ones its own epilogue completes
   uint32_t bump_token;         // 1 for F and dI, 0 otherwise
-  uint32_t hold_trigger;       // GEMM launches: the next kernel in the stream may start before this one ends, and reads what the
-                               // early part commits: it is let go after that
+  uint32_t pad;
   const float* amax_override;  // if non-null: value to push for the single class in class_mask
 };
 
@@ -55,10 +55,17 @@ struct QuantParams {
   float* sinv_dst;
   uint32_t* amax_bits;         // atomicMax target or null
   int32_t fmt;                 // 0 = E4M3, 1 = E5M2
-  uint32_t early;              // of the first cast of a launch: the launch may overlap the kernel before it (quantize_multi_kernel)
+  uint32_t pad;
   CommitParams commit;         // performed by the last block to finish (commit.st != null)
 };
 
+
+// A launch of casts that need not wait for the GEMM launch before it, which is only to have made its early commits (it counts
+// the problems that have, in *word; announce_commits).  Null: the casts wait.
+struct Announce {
+  uint32_t* word = nullptr;
+  uint32_t count = 0;          // what *word has come to by then
+};
 
 constexpr uint32_t kMaxCasts = 128;  // of one launch
 template <int N>
@@ -66,7 +73,8 @@ struct QuantMultiParams {
   QuantParams q[N];
   uint32_t block_end[N];       // cumulative block counts
   uint32_t n;
-  uint32_t pad[3];
+  uint32_t commits_count;      // Announce
+  const uint32_t* commits;
 };
 
 struct AmaxParams {
@@ -158,6 +166,8 @@ struct GemmDesc : GemmParams {
 // Independent GEMMs computed by one launch: tiles are numbered problem after problem.
 template <int NP>
 struct GemmLaunchParams {
+  uint32_t* commits;           // Announce: the next kernel in the stream may start before this one ends and reads what the early
+  uint32_t commits_op;         // part commits.  1: a problem is counted after that and the next kernel let go; 2: set to zero
   uint32_t n;
   uint32_t tile_end[NP];       // cumulative tile counts
   uint32_t* ticket;            // counts the CTAs that are done, where a problem has a commit in the tail; else null
@@ -235,7 +245,7 @@ struct Launch {
 };
 
 Launch make_quantize(const QuantParams& p);
-Launch make_quantize_multi(const QuantParams* casts, uint32_t n);  // 1..kMaxCasts independent casts in one launch
+Launch make_quantize_multi(const QuantParams* casts, uint32_t n, const Announce& early = {});  // 1..kMaxCasts independent casts in one launch
 Launch make_commit(const CommitParams& p);
 Launch make_status_gather(const StatusGatherParams& p);
 Launch make_amax_pass1(const AmaxParams& p);
@@ -245,6 +255,8 @@ Launch make_arena_reduce(const ArenaReduceParams& p);
 Launch make_gemm(const GemmDesc& p, int num_sms);
 // One launch for n = 2..kMaxProblems GEMMs (each may carry its own commit tail); false if there are more.
 bool make_gemm_group(const GemmDesc* probs, uint32_t n, int num_sms, Launch* out);
+uint32_t announce_commits(Launch* gemm, uint32_t* word);  // the launch is to count its problems in *word; how many that are
+void withdraw_commits(Launch* gemm, uint32_t* word);      // the launch is to set *word to zero
 uint32_t gemm_width(const GemmDesc* probs, uint32_t n, int num_sms);  // index of the tile width the launch of these will have
 cudaError_t gemm_prepare();  // opt in to the dynamic shared memory the GEMM needs (once per device)
 // Whether M fills whole 256-row tiles.  The kernels take any multiple of 128, and the layers' MN-major operands come with any;

@@ -128,11 +128,14 @@ __global__ void __launch_bounds__(kQuantThreads) quantize_kernel(const __grid_co
 // Independent casts in one launch (the X of forward units and the dY of input-gradient units that go out together, the
 // weights of a stage at the start of its step): the blocks are dealt to the casts one cast after the other.
 //
-// early: the casts' inputs, scales and destinations belong to no part of the kernel before this one that is still running (a
-// GEMM launch of the whole-step call, whose tiles leave DRAM bandwidth unused): the blocks do not wait for that kernel.  They
-// start when all of its CTAs have let its dependents go, which they do after their own wait, so that everything before it is
-// complete, and after the commits that these casts read.  One block waits at the end, so that this launch ends after that
-// kernel does and whoever waits for this launch has waited for both.  A block fits beside a GEMM CTA: 40 registers a thread.
+// commits (Announce): the casts' inputs, scales and destinations belong to no part of the kernel before this one that is still
+// running (a GEMM launch of the whole-step call, whose tiles leave DRAM bandwidth unused), and the blocks do not wait for that
+// kernel.  What they need of it and of those before it is that every problem's CTA has waited for its predecessors and
+// committed the scales that these casts read: it then counts itself, and a block that finds all of them counted goes ahead (a
+// release on the one side, an acquire on the other).  That the launch starts after the CTAs have let their dependents go makes
+// this the usual case, but nothing rests on it: a block that finds less waits for the whole kernel.  One block waits at the
+// end, so that this launch ends after that kernel does and whoever waits for this launch has waited for both.
+// A block fits beside a CTA of a GEMM launch without sums (40 registers a thread); behind others, blocks start as SMs come free.
 template <int N>
 __global__ void __launch_bounds__(kQuantThreads, 6) quantize_multi_kernel(const __grid_constant__ QuantMultiParams<N> mp) {
   __shared__ uint32_t wmax[kQuantThreads / 32];
@@ -144,7 +147,7 @@ __global__ void __launch_bounds__(kQuantThreads, 6) quantize_multi_kernel(const 
     else end = mid;
   }
   const uint32_t base = which ? mp.block_end[which - 1] : 0u;
-  if (!mp.q[0].early) grid_dep_wait();
+  if (!mp.commits || (int32_t)(ld_acquire(mp.commits) - mp.commits_count) < 0) grid_dep_wait();
   grid_dep_launch();
   const QuantParams& p = mp.q[which];
   const uint32_t b = blockIdx.x - base, bxn = p.cols / 64u;
@@ -155,11 +158,11 @@ __global__ void __launch_bounds__(kQuantThreads, 6) quantize_multi_kernel(const 
     if (last_block(&p.commit.st->ticket, mp.block_end[which] - base, threadIdx.x, &last_flag, sync))
       commit_classes(p.commit, threadIdx.x, wmax, sync);
   }
-  if (mp.q[0].early && blockIdx.x == gridDim.x - 1) grid_dep_wait();
+  if (mp.commits && blockIdx.x == gridDim.x - 1) grid_dep_wait();
 }
 
 template <int N>
-static Launch make_multi(const QuantParams* casts, uint32_t n) {
+static Launch make_multi(const QuantParams* casts, uint32_t n, const Announce& early) {
   QuantMultiParams<N> mp{};
   uint32_t blocks = 0;
   for (uint32_t i = 0; i < n; ++i) {
@@ -168,6 +171,8 @@ static Launch make_multi(const QuantParams* casts, uint32_t n) {
     mp.block_end[i] = blocks;
   }
   mp.n = n;
+  mp.commits = early.word;
+  mp.commits_count = early.count;
   Launch l;
   l.func = (const void*)quantize_multi_kernel<N>;
   l.grid = dim3(blocks, 1, 1);
@@ -176,8 +181,8 @@ static Launch make_multi(const QuantParams* casts, uint32_t n) {
   return l;
 }
 
-Launch make_quantize_multi(const QuantParams* casts, uint32_t n) {
-  return n <= 8 ? make_multi<8>(casts, n) : make_multi<kMaxCasts>(casts, n);
+Launch make_quantize_multi(const QuantParams* casts, uint32_t n, const Announce& early) {
+  return n <= 8 ? make_multi<8>(casts, n, early) : make_multi<kMaxCasts>(casts, n, early);
 }
 
 Launch make_quantize(const QuantParams& p) {

@@ -269,10 +269,9 @@ void push_gemms(qe_ctx* ctx, const qe::GemmDesc* gemms, uint32_t n, std::vector<
 // the launches: the casts in one launch, then every GEMM of whole 256-row tiles in one launch; weight gradients of
 // several microbatches of one layer (whole-step call only) become one GEMM that adds their products up
 // (refresh != null: the weight casts are collected there instead of being queued; apart: a round of a list whose tensors are
-// apart: half-filled last row tiles share launches too, and the next round's casts may overlap its GEMMs; early: its own casts
-// may overlap what is before them)
+// apart: half-filled last row tiles share launches too; early: its casts may overlap what is before them)
 int32_t together_build(qe_ctx* ctx, const Prepared* acts, uint32_t n, float* grad, std::vector<qe::Launch>& ls, Fnv* h,
-                       std::vector<qe::QuantParams>* refresh = nullptr, bool apart = false, bool early = false) {
+                       std::vector<qe::QuantParams>* refresh = nullptr, bool apart = false, const qe::Announce& early = {}) {
   // The order of the launches' problems is settled before they are built: F and dI first (others wait for them), the weight
   // gradients' tiles after theirs; the longest tiles first (their contraction length decides a tile's duration), so that a
   // launch's last, partial wave is made of short ones (weight gradients: contraction over the tokens of all products).
@@ -327,7 +326,6 @@ int32_t together_build(qe_ctx* ctx, const Prepared* acts, uint32_t n, float* gra
     } else {
       add_dI(L, a.slot, a.in_dev, a.out_dev, ls, nullptr, 0, &gp, &casts[i]);
     }
-    gp.commit.hold_trigger = apart;
   }
   const uint32_t n_chain = (uint32_t)gemms.size();
   for (const Product& d : dw_of) {
@@ -339,8 +337,7 @@ int32_t together_build(qe_ctx* ctx, const Prepared* acts, uint32_t n, float* gra
   const uint32_t n_gemms = (uint32_t)gemms.size();
   for (size_t i = 0; i < casts.size(); i += qe::kMaxCasts) {  // all casts of the call in one launch
     const uint32_t m = (uint32_t)std::min<size_t>(qe::kMaxCasts, casts.size() - i);
-    casts[i].early = early;
-    ls.push_back(m > 1 || early ? qe::make_quantize_multi(&casts[i], m) : qe::make_quantize(casts[i]));
+    ls.push_back(m > 1 || early.word ? qe::make_quantize_multi(&casts[i], m, early) : qe::make_quantize(casts[i]));
   }
   for (const qe::GemmDesc& gp : singles) ls.push_back(qe::make_gemm(gp, ctx->dev->num_sms));
   if (n_gemms >= 2) {
@@ -605,13 +602,23 @@ int32_t qe_step_run(qe_ctx* ctx, qe_layer* const* layers, uint32_t n_layers, con
     refresh.clear();
   };
   uint32_t waiting = 0;  // actions in the piece that is being put together
+  // Commits that GEMM launches announce to casts (Announce), and what their count has come to.  In graph mode the numbers are
+  // the piece's own, the same at every replay, and its last launch sets the count back; in eager mode they go on.
+  uint32_t* const commits = &layers[0]->st->commits;
+  const bool by_graphs = ctx->exec_mode == QE_EXEC_GRAPH;
+  uint32_t announced = by_graphs ? 0 : layers[0]->commits;
+  auto end_of_piece = [&] {
+    if (by_graphs && announced) qe::withdraw_commits(&ls.back(), commits);
+    if (by_graphs) announced = 0;
+    else layers[0]->commits = announced;
+  };
   std::vector<uint64_t> freed(n_layers, 0), freed_before(n_layers, 0);  // slots that the weight gradients of a round release
   std::vector<Prepared> acts;
   for (size_t r = 0; r < rounds.size() && st == QE_OK; ++r) {
     // check -> commit per action (all F first: a slot that a dW of the round releases is not theirs to take), then the
     // launches of those that passed
     acts.clear();
-    bool early = apart && r > 0;
+    bool early = apart && !ls.empty() && !ctx->launch_failed, casts = false;
     freed_before.swap(freed);
     std::fill(freed.begin(), freed.end(), 0);
     for (size_t i = 0; repeated && i < rounds[r].size(); ++i)
@@ -642,11 +649,13 @@ int32_t qe_step_run(qe_ctx* ctx, qe_layer* const* layers, uint32_t n_layers, con
         } else if (a.kind == QE_ACT_F) {
           st = qe_contract_forward_check(L->contract, a.mb, L->contract->e_W, &p.refresh, &p.slot);
           if (st == QE_OK) st = qe_contract_forward_commit(L->contract, a.mb, &tapes[u]);
+          casts = true;
           early = early && !(freed_before[a.layer] >> (p.slot & 63u) & 1u);  // the GEMMs of the round before still read this slot
         } else {
           st = qe_contract_dI_check(L->contract, &tapes[u]);
           p.slot = tapes[u].ref.slot;
           if (st == QE_OK) st = qe_contract_dI_commit(L->contract, &tapes[u]);
+          casts = true;
         }
         if (st != QE_OK) {
           k = gi;
@@ -658,7 +667,9 @@ int32_t qe_step_run(qe_ctx* ctx, qe_layer* const* layers, uint32_t n_layers, con
     }
     char why[512];  // (a build can only fail on a CUDA error, which then is the one to report)
     if (st != QE_OK) std::snprintf(why, sizeof(why), "%s", qe_last_error());
-    const int32_t built = acts.empty() ? QE_OK : together_build(ctx, acts.data(), (uint32_t)acts.size(), grad, ls, nullptr, &refresh, apart, early);
+    qe::Announce before;  // (the launch at the end of the list is the GEMM launch that these casts come after)
+    if (early && casts && !acts.empty()) before = {commits, announced += qe::announce_commits(&ls.back(), commits)};
+    const int32_t built = acts.empty() ? QE_OK : together_build(ctx, acts.data(), (uint32_t)acts.size(), grad, ls, nullptr, &refresh, apart, before);
     if (st != QE_OK) st = fail(st, "%s", why);
     else if (built != QE_OK) {
       st = built;
@@ -669,6 +680,7 @@ int32_t qe_step_run(qe_ctx* ctx, qe_layer* const* layers, uint32_t n_layers, con
     // not count (48 linears, 32 microbatches: 3.4 of 16.4 ms were host time ahead of the one launch).
     waiting += (uint32_t)acts.size();
     if (st == QE_OK && waiting >= (pieces < 2 ? 96u << pieces : 384u) && r + 1 < rounds.size()) {
+      end_of_piece();
       put_refresh();
       run_status = run_piece(ls, true);
       ls.clear();
@@ -676,6 +688,7 @@ int32_t qe_step_run(qe_ctx* ctx, qe_layer* const* layers, uint32_t n_layers, con
       if (run_status != QE_OK) break;
     }
   }
+  end_of_piece();
   put_refresh();
   if (!rounds.empty()) k = st == QE_OK ? n_actions : k;
 
@@ -727,6 +740,7 @@ int32_t qe_step_run(qe_ctx* ctx, qe_layer* const* layers, uint32_t n_layers, con
 
   // ---- device pass: the launches of every action that passed (in graph mode the ones that are not on their way yet)
   if (run_status == QE_OK && !ls.empty()) run_status = run_piece(ls, check_status == QE_OK);
+  ctx->launch_failed |= run_status != QE_OK;
   if (run_status == QE_OK && pieces) run_status = handshake.out();
   if (check_status != QE_OK || run_status != QE_OK) {
     // failure boundary: outstanding tapes aborted, arenas unusable for the epoch

@@ -70,6 +70,7 @@ struct qe_ctx {
   cudaStream_t exec_stream = nullptr;
   bool owns_stream = true;
   bool one_way = false;              // QE_CTX_UNSAFE_ONE_WAY_HANDOFF
+  bool launch_failed = false;        // a whole-step call's: counts of commits in device memory may not be what they should be
   uint32_t step_window = 4;          // qe_step_run: units looked ahead when planning rounds (1: action by action)
   cudaStream_t dw_stream = nullptr;  // only with QE_CTX_OVERLAP_DW
   cudaEvent_t ev_dw_in = nullptr;
@@ -97,6 +98,7 @@ struct qe_layer {
   qe_contract* contract = nullptr;
   uint64_t ws_bytes = 0;
   qe::DevState* st = nullptr;
+  uint32_t commits = 0;  // eager mode: what DevState::commits has come to when all that was issued has run
   float* hist = nullptr;
   uint8_t* Wq = nullptr;
   uint8_t *x_stage = nullptr, *dx_stage = nullptr, *y_stage = nullptr, *dy_stage = nullptr;  // host_io only

@@ -19,10 +19,10 @@
 namespace {
 struct Event { int id; };
 struct Stream { int id; };
-struct Node { size_t at; struct Graph* of; };
+struct Node { size_t at; struct Graph* of; char what[256]; };
 struct Graph { std::vector<Node*> nodes; };
 struct State {
-  std::string log;
+  std::string log, replayed;  // replayed: the launches of the graphs, one by one
   std::map<std::string, long> fail_in;  // function -> calls until one fails
   long alloc_in = -1;
   int events = 0, streams = 100;
@@ -84,7 +84,8 @@ void operator delete(void* p, size_t, std::align_val_t) noexcept { std::free(p);
 
 extern "C" {
 const char* fake_log() { return s().log.c_str(); }
-void fake_reset() { s().log.clear(); s().fail_in.clear(); s().alloc_in = -1; s().encodes = 0; }
+const char* fake_replayed() { return s().replayed.c_str(); }
+void fake_reset() { s().log.clear(); s().replayed.clear(); s().fail_in.clear(); s().alloc_in = -1; s().encodes = 0; }
 void fake_fail(const char* fn, long nth) { s().fail_in[fn] = nth; }
 void fake_fail_alloc(long nth) { s().alloc_in = nth; }
 long fake_alloc_left() { return s().alloc_in; }
@@ -137,7 +138,9 @@ cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void*, void**
   if (s().capturing && c->stream == s().capturing) {
     const long keep = s().alloc_in;
     s().alloc_in = -1;
-    s().graph->nodes.push_back(plain_new<Node>(s().graph->nodes.size(), s().graph));
+    Node* nd = plain_new<Node>(s().graph->nodes.size(), s().graph);
+    std::snprintf(nd->what, sizeof(nd->what), "%s", (const char*)args[0]);
+    s().graph->nodes.push_back(nd);
     s().alloc_in = keep;
   } else {
     note("launch %ld %s", sid(c->stream), (const char*)args[0]);
@@ -173,10 +176,18 @@ cudaError_t cudaGraphInstantiate(cudaGraphExec_t* e, cudaGraph_t gr, unsigned lo
   *e = (cudaGraphExec_t)gr;
   return cudaSuccess;
 }
-cudaError_t cudaGraphExecKernelNodeSetParams(cudaGraphExec_t, cudaGraphNode_t, const cudaKernelNodeParams*) { return cudaSuccess; }
+cudaError_t cudaGraphExecKernelNodeSetParams(cudaGraphExec_t, cudaGraphNode_t nd, const cudaKernelNodeParams* p) {
+  std::snprintf(((Node*)nd)->what, sizeof(Node::what), "%s", (const char*)p->kernelParams[0]);
+  return cudaSuccess;
+}
 cudaError_t cudaGraphLaunch(cudaGraphExec_t e, cudaStream_t st) {
   FAILS(cudaGraphLaunch);
   note("launch %ld graph %zu", sid(st), ((Graph*)e)->nodes.size());
+  const long keep = s().alloc_in;
+  s().alloc_in = -1;
+  s().replayed += "graph\n";
+  for (const Node* nd : ((Graph*)e)->nodes) s().replayed += std::string("launch - ") + nd->what + '\n';
+  s().alloc_in = keep;
   return cudaSuccess;
 }
 cudaError_t cudaGraphExecDestroy(cudaGraphExec_t) { return cudaSuccess; }
@@ -203,7 +214,15 @@ bool whole_row_tiles(uint32_t M) { return M % 256 == 0; }
 cudaError_t gemm_prepare() { return cudaSuccess; }
 uint32_t gemm_width(const GemmDesc*, uint32_t, int) { return 1; }
 Launch make_quantize(const QuantParams&) { return named("cast 1"); }
-Launch make_quantize_multi(const QuantParams* q, uint32_t n) { return named("cast %u%s", n, q[0].early ? " early" : ""); }
+Launch make_quantize_multi(const QuantParams*, uint32_t n, const Announce& early) {
+  return early.word ? named("cast %u early %u", n, early.count) : named("cast %u", n);
+}
+// (a GEMM launch is "gemm <problems> products <products>", and then what it does with the count of commits)
+uint32_t announce_commits(Launch* l, uint32_t*) {
+  std::strcat((char*)l->params.data(), " announces");
+  return (uint32_t)std::atoi((char*)l->params.data() + 5);
+}
+void withdraw_commits(Launch* l, uint32_t*) { std::strcat((char*)l->params.data(), " withdraws"); }
 Launch make_commit(const CommitParams&) { return named("commit"); }
 Launch make_status_gather(const StatusGatherParams&) { return named("status"); }
 Launch make_amax_pass1(const AmaxParams&) { return named("amax1"); }

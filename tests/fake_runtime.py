@@ -38,7 +38,7 @@ def load(so):
     for name, (res, args) in qe._SIGNATURES.items():
         fn = getattr(lib, name)
         fn.restype, fn.argtypes = res, args
-    lib.fake_log.restype = C.c_char_p
+    lib.fake_log.restype = lib.fake_replayed.restype = C.c_char_p
     lib.fake_fail.argtypes = [C.c_char_p, C.c_long]
     lib.fake_fail_alloc.argtypes = [C.c_long]
     lib.fake_alloc_left.restype = lib.fake_encodes.restype = C.c_long

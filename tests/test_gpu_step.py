@@ -806,3 +806,38 @@ def test_step_of_linears_that_do_not_feed_one_another_equals_single_actions_bitw
         got.append((_snapshot(layers, Y, dX, grad), ctx.stats()["kernels_launched"]))
     _same_snapshot(got[0][0], got[1][0])
     assert got[1][1] < got[0][1] / 4
+
+
+@pytest.mark.parametrize("mode", [0, 1], ids=["eager", "graph"])
+@pytest.mark.parametrize("n,H", [(4, 1), (4, 3), (12, 2)])
+def test_casts_beside_long_gemms_read_the_scales_those_commit(qe, mode, n, H):
+    """Small casts behind GEMMs of few tiles and long contractions, which they overlap for most of their time; scales that every
+    commit changes, no slot to spare, many steps.  From the third step on every step's results are those of the third made
+    action by action (the history holds fewer entries than a step makes)."""
+    T, M = 256, 6
+    s = sched(M, 3, 1)
+    shapes = [((4096, 256), (512, 4096))[j % 2] for j in range(n)]
+    acts = _actions(s, n)
+    X = [[(inputs.activations("EC", 0, 0, j, m, T, K) * 4.0 ** ((3 * m + j) % 5)).to(DEV) for j, (K, N) in enumerate(shapes)] for m in range(M)]
+    dY = [[(inputs.upstream_grads("EC", 0, 0, j, m, T, N) * 4.0 ** ((2 * m + j) % 5)).to(DEV) for j, (K, N) in enumerate(shapes)] for m in range(M)]
+    offs, total = inputs.grad_offsets([("l", K, N) for K, N in shapes])
+    want = None
+    for window in (1, 4):
+        ctx = qe.Context(mode, step_window=window)
+        layers = [qe.Layer(ctx, T, K, N, H, 0, peak_live(s), inputs.weights("EC", 0, j, N, K).to(DEV), unit=j) for j, (K, N) in enumerate(shapes)]
+        Y = [[torch.zeros((T, N), dtype=torch.bfloat16, device=DEV) for K, N in shapes] for m in range(M)]
+        dX = [[torch.zeros((T, K), dtype=torch.bfloat16, device=DEV) for K, N in shapes] for m in range(M)]
+        grad = torch.full((total,), 3.0, device=DEV)
+        plan = qe.StepPlan(ctx, layers, acts, M, X, Y, dY, dX, grad, offs)
+        results = [t for row in Y + dX for t in row] + [grad]
+        for step in range(3 if window == 1 else 40):
+            plan.run()
+            qe.optimizer_boundary_all(layers, M)
+            if window == 4 and step >= 2:
+                assert all(torch.equal(a, b) for a, b in zip(results, want)), step
+        if window == 1:
+            torch.cuda.synchronize()
+            want = [t.clone() for t in results]
+            single = ctx.stats()["kernels_launched"]
+        else:
+            assert ctx.stats()["kernels_launched"] * 3 < single * 40

@@ -287,3 +287,42 @@ def test_step_casts_overlap_the_gemms_before_them_unless_those_read_the_slot(lib
         free |= last
     assert ["early" in w for w in casts] == want and any(want) and (slots == 7 or not all(want[1:]))
     s.close()
+
+
+@pytest.mark.parametrize("mode", [0, 1], ids=["eager", "graph"])
+def test_casts_that_overlap_go_ahead_on_a_count_of_commits(lib, mode):
+    """A cast that does not wait for the GEMM launch before it is told how many problems will have committed by then, and that
+    launch counts its own: numbers that go on from call to call, or start anew in every graph, whose last launch sets the count
+    back.  Nothing counts for a cast that waits."""
+    M, n = 12, 20
+    s = fake_runtime.Stage(lib, [(256, 256)] * n, M=M, slots=6, mode=mode, window=4)
+    size = 2 * s.T * 256
+    base = s.buffer(4 * n * M * size)
+    total = early = 0
+    for _ in range(3):
+        lib.fake_reset()
+        assert s.step(_actions(M, n), apart=lambda l, m: [base + ((l * M + m) * 4 + j) * size for j in range(4)]) == 0
+        for h in s.layers:
+            assert lib.qe_optimizer_boundary(h, M) == 0
+        log = (lib.fake_replayed() if mode else lib.fake_log()).decode()
+        for piece in log.split("graph\n")[1:] if mode else [log]:
+            launches = [w.split() for w in piece.splitlines() if " cast " in w or " gemm " in w]
+            start = total
+            for before, w in zip([[]] + launches, launches):
+                if "early" in w:
+                    assert before[2] == "gemm" and before[-1] == "announces"
+                    total += int(before[3])
+                    assert int(w[-1]) == total
+                    early += 1
+                else:
+                    assert "announces" not in before
+            assert [("withdraws" in w) for w in launches] == [False] * (len(launches) - 1) + [mode == 1 and total > start]
+            total = total if mode == 0 else 0
+    assert early > 15
+    lib.fake_reset()
+    lib.fake_fail(b"cudaGraphLaunch" if mode else b"cudaLaunchKernelExC", 2 if mode else 30)  # some of the counting is lost
+    own = lambda l, m: [base + ((l * M + m) * 4 + j) * size for j in range(4)]  # noqa: E731
+    assert s.step(_actions(M, n), apart=own) == CUDA and all(lib.qe_arena_rebuild(h) == 0 for h in s.layers)
+    lib.fake_reset()
+    assert s.step(_actions(M, n), apart=own) == 0 and b"early" not in lib.fake_log() + lib.fake_replayed()
+    s.close()
