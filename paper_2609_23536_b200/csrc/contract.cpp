@@ -144,9 +144,10 @@ int32_t qe_contract_dI_commit(qe_contract* c, const qe_tape* t) {
   return QE_OK;
 }
 
-// Sec. 3.4: destination validated; microbatch 0 initialises; duplicate / aliased writes fail.
-int32_t qe_contract_dW_check(const qe_contract* c, const qe_tape* t, uint64_t dest_addr, uint64_t dest_elems,
-                             uint64_t offset, uint64_t slice_elems, int32_t* accumulate_out) {
+// Sec. 3.4: destination validated; microbatch 0 initialises; duplicate / aliased writes fail.  bind: the destination is bound
+// in the same breath, so that of two threads whose slices overlap one at most gets through.
+static int32_t dW_validate(const qe_contract* c, const qe_tape* t, uint64_t dest_addr, uint64_t dest_elems, uint64_t offset,
+                           uint64_t slice_elems, int32_t* accumulate_out, bool bind) {
   if (!c) return fail(QE_ERR_BAD_ARG, "contract is null");
   if (c->aborted) return fail(QE_ERR_ABORTED, "step aborted; arena unusable for this epoch");
   uint32_t p;
@@ -163,8 +164,9 @@ int32_t qe_contract_dW_check(const qe_contract* c, const qe_tape* t, uint64_t de
   if (lo % 16 != 0) return fail(QE_ERR_DEST, "destination slice not 16-byte aligned");
   if (c->has_dest && (c->dest_addr != dest_addr || c->dest_off != offset))
     return fail(QE_ERR_DEST, "differs from the destination bound for this epoch");
+  std::unique_lock<std::mutex> g;
   if (c->registry) {
-    std::lock_guard<std::mutex> g(c->registry->mu);
+    g = std::unique_lock<std::mutex>(c->registry->mu);
     const auto own = c->registry->bound.find(c);
     // (a range that is bound already was compared when it was, and every later one with it)
     const bool bound = own != c->registry->bound.end() && own->second.lo == lo && own->second.hi == hi;
@@ -176,22 +178,23 @@ int32_t qe_contract_dW_check(const qe_contract* c, const qe_tape* t, uint64_t de
   if ((c->write_mask >> mb) & 1ull) return fail(QE_ERR_DUP_WRITE, "microbatch %u already wrote this epoch", mb);
   if (c->write_mask == 0 && mb != 0) return fail(QE_ERR_ORDER, "first write of the epoch must be microbatch 0, got %u", mb);
   if (accumulate_out) *accumulate_out = c->write_mask == 0 ? 0 : 1;
+  if (bind && c->registry) c->registry->bound[c] = qe::RegistryState::Range{lo, hi};
   return QE_OK;
+}
+
+int32_t qe_contract_dW_check(const qe_contract* c, const qe_tape* t, uint64_t dest_addr, uint64_t dest_elems,
+                             uint64_t offset, uint64_t slice_elems, int32_t* accumulate_out) {
+  return dW_validate(c, t, dest_addr, dest_elems, offset, slice_elems, accumulate_out, false);
 }
 
 int32_t qe_contract_dW_commit(qe_contract* c, const qe_tape* t, uint64_t dest_addr, uint64_t offset,
                               uint64_t slice_elems) {
   // re-validate everything that does not depend on the buffer length (already checked before the action)
-  int32_t st = qe_contract_dW_check(c, t, dest_addr, UINT64_MAX, offset, slice_elems, nullptr);
+  int32_t st = dW_validate(c, t, dest_addr, UINT64_MAX, offset, slice_elems, nullptr, true);
   if (st != QE_OK) return st;
   c->has_dest = true;
   c->dest_addr = dest_addr;
   c->dest_off = offset;
-  if (c->registry) {
-    std::lock_guard<std::mutex> g(c->registry->mu);
-    const uint64_t lo = dest_addr + 4ull * offset;
-    c->registry->bound[c] = qe::RegistryState::Range{lo, lo + 4ull * slice_elems};
-  }
   qe_contract::Slot& s = c->slot[t->ref.slot];
   c->write_mask |= 1ull << t->key.mb;
   s.bits |= qe::kDWBit;

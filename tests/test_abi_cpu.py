@@ -167,6 +167,38 @@ def test_destination_rules(qe):
     a.dW_check(t, BUF, ELEMS, 2048, SLICE)
 
 
+def test_of_two_threads_that_bind_overlapping_slices_one_at_most_gets_through(qe):
+    import threading
+
+    reg = qe.Registry()
+    others = [qe.Contract(1, unit=2 + i, registry=reg) for i in range(2000)]  # (so many that both threads look through them at once)
+    a, b = qe.Contract(1, unit=0, registry=reg), qe.Contract(1, unit=1, registry=reg)
+    for trial in range(200):
+        start, done = threading.Barrier(2), []
+
+        def bind(c, offset):
+            t = c.forward_commit(0)
+            c.dI_commit(t)
+            c.dW_check(t, BUF, ELEMS, offset, SLICE)
+            start.wait()
+            try:
+                c.dW_commit(t, BUF, offset, SLICE)
+                done.append(c)
+            except qe.QEError as e:
+                assert e.code == "DEST"
+
+        threads = [threading.Thread(target=bind, args=x) for x in ((a, 0), (b, 512))]
+        for t in threads:
+            t.start()
+        for t in threads:
+            t.join()
+        assert len(done) == 1, trial
+        for c in (a, b):
+            c.abort()
+            c.rebuild()
+    del others
+
+
 @settings(max_examples=80, deadline=None)
 @given(st.lists(st.tuples(st.sampled_from(["F", "dI", "dW", "stale", "boundary", "abort"]), st.integers(0, 4)), max_size=50))
 def test_contract_core_matches_oracle_state_machine(qe, ops):
