@@ -460,7 +460,7 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
     const GemmParams& q = ps.first();
     if (q.epi == 3 && q.sinv_dst) *q.sinv_dst = *q.sinv_src;
   }
-  if (warp == EPI_WARP0 + 7 && blockIdx.x < ps.count()) {  // (every launch has at least one CTA per problem)
+  if (warp == EPI_WARP0 + 7 && blockIdx.x < ps.count()) {  // (a launch with early commits has a CTA per problem at least: most_committing)
     // The classes whose amax an EARLIER kernel reduced (the cast that made this GEMM's A operand) are committed here,
     // by an epilogue warp that has nothing to drain yet: nothing this launch computes reads their scale (its alphas
     // are snapshots), so only the output's class is left for the launch's tail.
@@ -977,6 +977,8 @@ cudaError_t gemm_prepare() {
 
 bool make_gemm_group(const GemmDesc* probs, uint32_t n, int num_sms, Launch* out) {
   if (n < 2 || n > kMaxProblems) return false;
+  for (uint32_t i = 0; i < n && n > most_committing(num_sms); ++i)
+    if (probs[i].commit.st && probs[i].commit.early_mask) return false;
   *out = make_any(probs, n, num_sms);
   return true;
 }

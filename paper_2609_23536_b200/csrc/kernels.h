@@ -175,6 +175,11 @@ struct GemmLaunchParams {
   GemmParams prob[NP];
 };
 constexpr uint32_t kMaxProblems = 56;  // of a launch: what a kernel's parameter space of 32764 bytes holds
+// ... and of one whose problems commit scales at its start, a CTA each: the grid has that many at least
+inline uint32_t most_committing(int num_sms) {
+  const uint32_t ctas = num_sms < 4 ? 2u : (uint32_t)num_sms / 2u * 2u;
+  return ctas < kMaxProblems ? ctas : kMaxProblems;
+}
 
 // ORs the status words of up to 64 layers into *out (first chunk: out = OR; later chunks: out |= OR).
 struct StatusGatherParams {
@@ -254,6 +259,7 @@ Launch make_accumulate(const AccumParams& p);
 Launch make_arena_reduce(const ArenaReduceParams& p);
 Launch make_gemm(const GemmDesc& p, int num_sms);
 // One launch for n = 2..kMaxProblems GEMMs (each may carry its own commit tail); false if there are more.
+// (most_committing, where they commit scales at the launch's start)
 bool make_gemm_group(const GemmDesc* probs, uint32_t n, int num_sms, Launch* out);
 uint32_t announce_commits(Launch* gemm, uint32_t* word);  // the launch is to count its problems in *word; how many that are
 void withdraw_commits(Launch* gemm, uint32_t* word);      // the launch is to set *word to zero

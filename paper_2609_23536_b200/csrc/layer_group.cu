@@ -258,7 +258,8 @@ int32_t together_prepare(qe_ctx* ctx, Prepared* acts, uint32_t n, float* grad, u
 
 // The GEMMs gemms[0..n) in as few launches as hold them, each launch with about as many.
 void push_gemms(qe_ctx* ctx, const qe::GemmDesc* gemms, uint32_t n, std::vector<qe::Launch>& ls) {
-  for (uint32_t launches = (n + qe::kMaxProblems - 1) / qe::kMaxProblems, share; launches; --launches, gemms += share, n -= share) {
+  const uint32_t most = qe::most_committing(ctx->dev->num_sms);
+  for (uint32_t launches = (n + most - 1) / most, share; launches; --launches, gemms += share, n -= share) {
     share = (n + launches - 1) / launches;
     qe::Launch l;
     if (share >= 2 && qe::make_gemm_group(gemms, share, ctx->dev->num_sms, &l)) ls.push_back(std::move(l));
@@ -345,7 +346,7 @@ int32_t together_build(qe_ctx* ctx, const Prepared* acts, uint32_t n, float* gra
     ctx->stats.paired_f_di += n_chain ? 1 : 0;
   }
   // one launch where it holds them all; else weight gradients, which add products up, have launches of their own
-  const uint32_t together = n_gemms <= qe::kMaxProblems ? n_gemms : n_chain;
+  const uint32_t together = n_gemms <= qe::most_committing(ctx->dev->num_sms) ? n_gemms : n_chain;
   push_gemms(ctx, gemms.data(), together, ls);
   push_gemms(ctx, gemms.data() + together, n_gemms - together, ls);
   return QE_OK;

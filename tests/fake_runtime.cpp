@@ -29,6 +29,7 @@ struct State {
   cudaStream_t capturing = nullptr;
   Graph* graph = nullptr;
   long encodes = 0;
+  int sms = 148;
 };
 State* g = nullptr;  // (never freed: the library may be used until the process ends)
 State& s() {
@@ -89,6 +90,7 @@ void fake_reset() { s().log.clear(); s().replayed.clear(); s().fail_in.clear(); 
 void fake_fail(const char* fn, long nth) { s().fail_in[fn] = nth; }
 void fake_fail_alloc(long nth) { s().alloc_in = nth; }
 long fake_alloc_left() { return s().alloc_in; }
+void fake_sms(int n) { s().sms = n; }  // before the library has looked at the device
 long fake_encodes() { return s().encodes; }
 
 cudaError_t cudaGetDeviceCount(int* n) { *n = 1; return cudaSuccess; }
@@ -97,7 +99,7 @@ cudaError_t cudaGetDevice(int* d) { *d = 0; return cudaSuccess; }
 cudaError_t cudaGetDeviceProperties_v2(cudaDeviceProp* p, int) {
   std::memset(p, 0, sizeof(*p));
   p->major = 10;
-  p->multiProcessorCount = 148;
+  p->multiProcessorCount = s().sms;
   return cudaSuccess;
 }
 cudaError_t cudaGetDriverEntryPoint(const char*, void** fn, unsigned long long, cudaDriverEntryPointQueryResult* q) {

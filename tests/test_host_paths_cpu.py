@@ -326,3 +326,21 @@ def test_casts_that_overlap_go_ahead_on_a_count_of_commits(lib, mode):
     lib.fake_reset()
     assert s.step(_actions(M, n), apart=own) == 0 and b"early" not in lib.fake_log() + lib.fake_replayed()
     s.close()
+
+
+@pytest.mark.parametrize("sms", [20, 57, 148])
+def test_launches_that_commit_scales_hold_a_problem_per_cta_at_most(lib, tmp_path, sms):
+    """A problem's early commit is made by the CTA of its number: a device of few SMs gets more launches, not lost commits."""
+    import shutil
+
+    lib = fake_runtime.load(shutil.copy(lib._name, tmp_path / "few_sms.so"))
+    lib.fake_sms(sms)
+    n, M = 57, 2
+    s = fake_runtime.Stage(lib, [(256, 256)] * n, M=M, slots=M, window=4)
+    size = 2 * s.T * 256
+    base = s.buffer(4 * n * M * size)
+    lib.fake_reset()
+    assert s.step(_actions(M, n), apart=lambda l, m: [base + ((l * M + m) * 4 + j) * size for j in range(4)]) == 0
+    words = [w.split() for w in lib.fake_log().decode().splitlines() if " gemm " in w]  # launch STREAM gemm N products P
+    assert max(int(w[3]) for w in words) <= min(56, sms // 2 * 2) and sum(int(w[5]) for w in words) == 3 * n * M
+    s.close()
