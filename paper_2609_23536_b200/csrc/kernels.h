@@ -48,7 +48,7 @@ struct CommitParams {
 struct QuantParams {
   const uint16_t* x;           // bf16 [rows, cols]
   uint8_t* q;                  // fp8 [rows, cols]
-  uint8_t* qT;                 // fp8 [cols, rows] or null
+  uint8_t* qT;                 // fp8 [cols, rows] or null (a launch of its own only)
   uint32_t rows, cols;
   const float* scale;          // device scalar read by every thread
   const float* sinv_src;       // if non-null, block 0 copies *sinv_src to *sinv_dst (tape snapshot)
@@ -250,7 +250,7 @@ struct Launch {
 };
 
 Launch make_quantize(const QuantParams& p);
-Launch make_quantize_multi(const QuantParams* casts, uint32_t n, const Announce& early = {});  // 1..kMaxCasts independent casts in one launch
+Launch make_quantize_multi(const QuantParams* casts, uint32_t n, const Announce& early = {});  // 1..kMaxCasts independent casts without transposed copies in one launch
 Launch make_commit(const CommitParams& p);
 Launch make_status_gather(const StatusGatherParams& p);
 Launch make_amax_pass1(const AmaxParams& p);

@@ -57,16 +57,17 @@ __device__ __forceinline__ void transpose4x4(const uint32_t a0, const uint32_t a
 // bytes of every output row of the transposed copy).
 constexpr int kQuantThreads = 256;
 
-// One block's share (256 rows x 64 columns at block coordinates bx, by) of a cast; wmax: 8 shared words.  L2: the scale is read
-// there (a launch that does not wait for the kernel before it); a lone cast, whose reads it would slow, does not.
-template <int FMT, bool L2 = false>
+// One block's share (256 rows x 64 columns at block coordinates bx, by) of a cast; wmax: 8 shared words.  SHARED: one of a
+// launch's several casts: no transposed copy, which leaves a thread 40 registers without a spill, and the scale is read from L2
+// (the launch may overlap the kernel before it; a lone cast, whose reads that would slow, does not).
+template <int FMT, bool SHARED = false>
 __device__ __forceinline__ void quantize_block(const QuantParams& p, uint32_t bx, uint32_t by, uint32_t* wmax) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int rb = lane >> 3, cv = lane & 7;
   const uint32_t row0 = by * 256u + warp * 32u + rb * 8u;
   const uint32_t col0 = bx * 64u + cv * 8u;
-  const float scale = L2 ? __ldcg(p.scale) : *p.scale;
-  if (bx == 0 && by == 0 && threadIdx.x == 0 && p.sinv_dst) *p.sinv_dst = L2 ? __ldcg(p.sinv_src) : *p.sinv_src;
+  const float scale = SHARED ? __ldcg(p.scale) : *p.scale;
+  if (bx == 0 && by == 0 && threadIdx.x == 0 && p.sinv_dst) *p.sinv_dst = SHARED ? __ldcg(p.sinv_src) : *p.sinv_src;
 
   uint32_t m = 0;
   if (row0 < p.rows) {  // warp-uniform up to rb; rows is a multiple of 8 so a thread's 8 rows are all in or out
@@ -84,7 +85,7 @@ __device__ __forceinline__ void quantize_block(const QuantParams& p, uint32_t bx
     uint8_t* dst = p.q + (size_t)row0 * p.cols + col0;
 #pragma unroll
     for (int i = 0; i < 8; ++i) *reinterpret_cast<uint2*>(dst + (size_t)i * p.cols) = make_uint2(lo[i], hi[i]);
-    if (p.qT) {
+    if (!SHARED && p.qT) {
       uint32_t t00[4], t10[4], t01[4], t11[4];  // t<rowhalf><colhalf>
       transpose4x4(lo[0], lo[1], lo[2], lo[3], t00);
       transpose4x4(lo[4], lo[5], lo[6], lo[7], t10);

@@ -1,6 +1,7 @@
-"""What the kernels' sources state about synchronisation that no run can show to be missing."""
+"""What the kernels' sources state that no run would show to be missing: synchronisation, registers."""
 import os
 import re
+import subprocess
 
 from paper_2609_23536_b200 import build
 
@@ -17,3 +18,12 @@ def test_whole_warp_roles_of_the_gemm_leave_every_wait_together():
     roles = raw[raw.index("-- TMA producer"):raw.index("-- epilogue")]
     assert len(re.findall(r"\bmbar_wait_warp\(", roles)) == 3 and not re.findall(r"\bmbar_wait\(", roles)
     assert re.search(r"bool mbar_wait_warp\([^{]*\{\s*return __all_sync\(0xffffffffu, mbar_wait\(", _source("gemm_sm100.cu"))
+
+
+def test_casts_that_share_a_launch_fit_beside_a_gemm_cta(tmp_path):
+    """A block of theirs has the registers that a GEMM CTA leaves on its SM, 40 a thread, and needs no more."""
+    cmd = [build._nvcc(), "-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-std=c++17", "-Xptxas", "-v", "-I", build.INCLUDE,
+           "-I", build.CSRC, "-c", os.path.join(build.CSRC, "kernels_hbm.cu"), "-o", str(tmp_path / "k.o")]
+    said = subprocess.run(cmd, check=True, capture_output=True, text=True).stderr
+    kernels = re.findall(r"Compiling entry function '\w*quantize_multi_kernel.*?(\d+) bytes spill stores.*?Used (\d+) registers", said, re.S)
+    assert len(kernels) == 2 and all(int(spilled) == 0 and int(used) <= 40 for spilled, used in kernels)
