@@ -698,13 +698,13 @@ def _same_snapshot(a, b):
 
 @pytest.mark.parametrize("mode", [0, 1], ids=["eager", "graph"])
 def test_long_step_of_wide_launches_in_several_pieces_equals_single_actions_bitwise(qe, mode):
-    """Sixteen linears and twelve microbatches: launches of eight forwards and input gradients with sums of weight gradients
-    beside them, and in graph mode a list that goes out as several graphs."""
+    """Sixteen linears and twelve microbatches: launches of all forwards and input gradients that are ready with sums of weight
+    gradients beside them, and in graph mode a list that goes out as several graphs."""
     M, n = 12, len(LONG)
     s = sched(M, 4, 4)
     acts = _actions(s, n)
-    rounds = qe.plan_rounds(acts, n, M, peak_live(s), 16, 8, max_sum=8)
-    assert len(rounds) > 64 and any(sum(a != "dW" for a, l, m in g) == 8 and len({l for a, l, m in g if a == "dW"}) == 3 for g in rounds)
+    rounds = qe.plan_rounds(acts, n, M, peak_live(s), 16, 112, max_sum=8, apart=True)
+    assert any(sum(a != "dW" for a, l, m in g) == 2 * n and len({l for a, l, m in g if a == "dW"}) == n for g in rounds)
     got = []
     for window in (1, 16):
         ctx, layers, offs, X, Y, dY, dX, grad = _long_stage(qe, mode, window, M, s)
@@ -779,16 +779,18 @@ def test_dW_multi_of_many_linears_equals_per_layer_calls_bitwise(qe, n):
     assert st0["kernels_launched"] - st1["kernels_launched"] == 2 * M * (n - launches)
 
 
-@pytest.mark.parametrize("T,n,slots", [(384, 53, 4), (256, 9, 2)])
+@pytest.mark.parametrize("T,n,slots", [(384, 53, 4), (256, 9, 2), (256, 112, 4)])
 def test_step_of_linears_that_do_not_feed_one_another_equals_single_actions_bitwise(qe, T, n, slots):
-    """More than fifty linears (two launches of forwards and input gradients, two of sums) and few; half-filled row tiles of tokens and
-    of features; inputs whose maxima fall, so that lanes of one warp scan their rings."""
+    """Fifty-three linears (two launches of forwards and input gradients, one of sums), few, and a hundred and
+    twelve (launches of 56, two of them of sums); half-filled row tiles of tokens and of features; inputs whose maxima fall, so that lanes of one warp scan their rings."""
     M, steps = 4, 2
     shapes = [((256, 384, 512)[j % 3], (256, 640)[j % 2]) for j in range(n)]
     s = sched(M, 2, 1)
     acts = _actions(s, n)
     slots = max(slots, peak_live(s))
-    assert max(map(len, qe.plan_rounds(acts, n, M, slots, 4, 100, max_sum=8, apart=True))) >= min(2 * n, 100)
+    rounds = qe.plan_rounds(acts, n, M, slots, 4, 112, max_sum=8, apart=True)
+    assert max(sum(a != "dW" for a, l, m in g) for g in rounds) == min(2 * n, 112)
+    assert (max(len({l for a, l, m in g if a == "dW"}) for g in rounds) > 56) == (n == 112)
     got = []
     for window in (1, 4):
         ctx = qe.Context(1, step_window=window)
@@ -841,3 +843,39 @@ def test_casts_beside_long_gemms_read_the_scales_those_commit(qe, mode, n, H):
             single = ctx.stats()["kernels_launched"]
         else:
             assert ctx.stats()["kernels_launched"] * 3 < single * 40
+
+
+@pytest.mark.parametrize("mode", [0, 1], ids=["eager", "graph"])
+@pytest.mark.parametrize("T,widths,M,w,d,window,sums", [
+    (384, [256, 512, 640, 256, 384], 9, 1, 8, 6, 8),           # half-filled row tiles, sums of up to eight products
+    (256, [256, 512, 256, 256, 256] * 3 + [384], 12, 4, 4, 16, 8),  # several pieces
+    (2816, [256, 512, 384, 256], 3, 2, 1, 4, None),            # too many tokens for sums
+])
+def test_step_of_linears_that_feed_one_another_equals_single_actions_bitwise(qe, mode, T, widths, M, w, d, window, sums):
+    """Each linear's output is the next one's input and each input gradient the upstream gradient of the one before: a linear
+    that ran too early would read what an earlier step left there, or nothing."""
+    shapes = list(zip(widths, widths[1:]))
+    n, steps = len(shapes), 3
+    s = sched(M, w, d)
+    acts = _actions(s, n)
+    rounds = qe.plan_rounds(acts, n, M, peak_live(s), window, 8, max_sum=sums)
+    assert (sums is not None) == any(len({l for a, l, m in g if a == "dW"}) < sum(a == "dW" for a, l, m in g) for g in rounds)
+    offs, total = inputs.grad_offsets([("l", K, N) for K, N in shapes])
+    got = []
+    for step_window in (1, window):
+        ctx = qe.Context(mode, step_window=step_window)
+        layers = [qe.Layer(ctx, T, K, N, 4, 0, peak_live(s), inputs.weights("FD", 0, j, N, K).to(DEV), unit=j) for j, (K, N) in enumerate(shapes)]
+        act = [[torch.full((T, f), 7.0, dtype=torch.bfloat16, device=DEV) for f in widths] for m in range(M)]
+        dact = [[torch.full((T, f), 7.0, dtype=torch.bfloat16, device=DEV) for f in widths] for m in range(M)]
+        grad = torch.full((total,), 3.0, device=DEV)
+        plan = qe.StepPlan(ctx, layers, acts, M, [r[:-1] for r in act], [r[1:] for r in act], [r[1:] for r in dact], [r[:-1] for r in dact], grad, offs)
+        for step in range(steps):
+            for m in range(M):
+                act[m][0].copy_(inputs.activations("FD", 0, step, 0, m, T, widths[0]))
+                dact[m][-1].copy_(inputs.upstream_grads("FD", 0, step, n - 1, m, T, widths[-1]))
+            plan.run()
+            qe.optimizer_boundary_all(layers, M)
+        got.append((_snapshot(layers, [r[1:] for r in act], [r[:-1] for r in dact], grad), ctx.stats()["kernels_launched"]))
+    _same_snapshot(got[0][0], got[1][0])
+    # (a round of casts and GEMMs is two launches at least; with all layers at once there would be far fewer rounds)
+    assert steps * len(rounds) < got[1][1] < got[0][1]

@@ -229,7 +229,7 @@ def test_step_sums_weight_gradients_where_three_products_fit(lib, tokens, sums):
 
 
 def test_step_takes_all_layers_of_a_unit_at_once_only_where_its_tensors_are_apart(lib):
-    """Forty linears in one round, cast by one launch, their GEMMs in two; as soon as one tensor that an action writes overlaps
+    """Forty linears in one round, cast by one launch, their eighty GEMMs in two; as soon as one tensor that an action writes overlaps
     what another reads or writes, or a weight, or a gradient, the layers go one after the other."""
     n, M, K = 40, 2, 256
     s = fake_runtime.Stage(lib, [(K, K)] * n, M=M, slots=M, window=4)
@@ -247,7 +247,7 @@ def test_step_takes_all_layers_of_a_unit_at_once_only_where_its_tensors_are_apar
 
     assert casts(own) == 2 * n  # the second forward and the first input gradient of every layer; the weights' casts are n
     words = [w.split() for w in lib.fake_log().decode().splitlines() if " gemm " in w]
-    assert max(int(w[3]) for w in words) <= 50 and sum(int(w[5]) for w in words) == 3 * n * M
+    assert max(int(w[3]) for w in words) == n and sum(int(w[5]) for w in words) == 3 * n * M
     where = {"y on another x": (3, 1, 7, 0, 0), "dx on another dy": (3, 1, 7, 0, 2), "y on another y": (3, 1, 7, 1, 1), "dx on its own x": (3, 3, 3, 0, 0)}
     for name, (l, j, l2, m2, j2) in where.items():
         def io(a, b):
@@ -344,3 +344,40 @@ def test_launches_that_commit_scales_hold_a_problem_per_cta_at_most(lib, tmp_pat
     words = [w.split() for w in lib.fake_log().decode().splitlines() if " gemm " in w]  # launch STREAM gemm N products P
     assert max(int(w[3]) for w in words) <= min(56, sms // 2 * 2) and sum(int(w[5]) for w in words) == 3 * n * M
     s.close()
+
+
+@pytest.mark.parametrize("n,M,w,d", [(56, 2, 2, 0), (57, 2, 2, 0), (100, 4, 1, 1), (112, 2, 1, 0), (113, 2, 1, 0)])
+def test_launches_of_a_round_hold_fifty_six_problems_and_split_evenly(lib, n, M, w, d):
+    """A round has 112 forwards and input gradients at most; what does not fit one launch goes out in launches of about the same
+    size, weight gradients then in launches of their own."""
+    from paper_2609_23536_b200 import binding as qe
+    from paper_2609_23536_b200.schedules import peak_live, sched
+
+    s = sched(M, w, d)
+    acts = [(a, l, m) for a, m in s for l in (range(n) if a == "F" else range(n - 1, -1, -1))]
+    stage = fake_runtime.Stage(lib, [(256, 256)] * n, T=256, M=M, slots=peak_live(s), window=4)
+    size = 2 * 256 * 256
+    base = stage.buffer(4 * n * M * size)
+    lib.fake_reset()
+    assert stage.step(acts, apart=lambda l, m: [base + ((l * M + m) * 4 + j) * size for j in range(4)]) == 0
+    got = [tuple(map(int, w.split()[3:6:2])) for w in lib.fake_log().decode().splitlines() if " gemm " in w]
+    stage.close()
+    rounds, want = qe.plan_rounds(acts, n, M, peak_live(s), 4, 112, max_sum=8, apart=True), []
+
+    def shares(k):
+        launches = -(-k // 56)
+        return [k // launches + (i < k % launches) for i in range(launches)]
+
+    for g in rounds:
+        chain = sum(a != "dW" for a, l, m in g)
+        sums = {l: sum((a, x) == ("dW", l) for a, x, m in g) for a, l, m in g if a == "dW"}
+        if chain + len(sums) <= 56:
+            want.append((chain + len(sums), len(g)))
+        else:
+            want += [(k, k) for k in shares(chain)]
+            products = set(sums.values())
+            assert len(products) < 2
+            want += [(k, k * max(products)) for k in shares(len(sums))] if sums else []
+    assert got == want
+    assert {56: want[0] == (56, 56), 57: want[:2] == [(29, 29), (28, 28)], 100: (50, 50) in want, 112: want[-2:] == [(56, 112)] * 2,
+            113: (1, 1) not in want and max(want) < (57, 0)}[n]
