@@ -850,10 +850,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(SHARED_SM_THREADS, 1
 }
 
 // The same where problems have several products each.
-template <int NP>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(threads_of(true), 1)
-    gemm_fp8_pair_wide_kernel(const __grid_constant__ GemmLaunchParams<NP> g) {
-  gemm_body<true>(Problems<NP, true>{g});
+    gemm_fp8_pair_wide_kernel(const __grid_constant__ GemmLaunchParams<kMaxProblems> g) {
+  gemm_body<true>(Problems<kMaxProblems, true>{g});
 }
 
 constexpr uint32_t PAIR_M = Form<true>::TILE_M;
@@ -946,7 +945,11 @@ Launch make_launch(const GemmDesc* probs, uint32_t n, int num_sms, const void* f
   return l;
 }
 
-constexpr uint32_t kFew = 8, kFewSums = 16;  // problems of a launch with a small parameter block
+// Problems of a launch with a parameter block of 5 KB instead of 32, whose copies cost the host 2 to 3 us a launch: two problems of
+// 256 x 256 x 256 by qe_gemm_fp8_group 12.9 us for 15.3, eight 24 for 27; F, dI and dW of four such linears, their calls sharing
+// launches, 123 for 132 (a graph keeps its blocks: 114 either way).  Blocks of up to sixteen gain nothing over eight, nor do
+// small blocks for sums, which go out a few times a step: 5 KB and 32 within 1 % on steps of 2 to 64 linears.
+constexpr uint32_t kFew = 8;
 
 Launch make_any(const GemmDesc* probs, uint32_t n, int num_sms) {
   bool sums = false;
@@ -957,8 +960,7 @@ Launch make_any(const GemmDesc* probs, uint32_t n, int num_sms) {
   }
   if (!sums && n <= kFew) return make_launch<kFew>(probs, n, num_sms, (const void*)gemm_fp8_pair_group_kernel<kFew>, false);
   if (!sums) return make_launch<kMaxProblems>(probs, n, num_sms, (const void*)gemm_fp8_pair_group_kernel<kMaxProblems>, false);
-  if (n <= kFewSums) return make_launch<kFewSums>(probs, n, num_sms, (const void*)gemm_fp8_pair_wide_kernel<kFewSums>, true);
-  return make_launch<kMaxProblems>(probs, n, num_sms, (const void*)gemm_fp8_pair_wide_kernel<kMaxProblems>, true);
+  return make_launch<kMaxProblems>(probs, n, num_sms, (const void*)gemm_fp8_pair_wide_kernel, true);
 }
 
 }  // namespace
@@ -967,8 +969,7 @@ bool whole_row_tiles(uint32_t M) { return M % 256 == 0; }
 
 cudaError_t gemm_prepare() {
   for (const void* f : {(const void*)gemm_fp8_kernel, (const void*)gemm_fp8_pair_kernel, (const void*)gemm_fp8_pair_group_kernel<kFew>,
-                        (const void*)gemm_fp8_pair_group_kernel<kMaxProblems>, (const void*)gemm_fp8_pair_wide_kernel<kFewSums>,
-                        (const void*)gemm_fp8_pair_wide_kernel<kMaxProblems>}) {
+                        (const void*)gemm_fp8_pair_group_kernel<kMaxProblems>, (const void*)gemm_fp8_pair_wide_kernel}) {
     const cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES);
     if (e != cudaSuccess) return e;
   }
