@@ -16,7 +16,8 @@ namespace qe {
 // Programmatic dependent launch.  Every kernel of the library is launched with programmatic stream serialization, so
 // the next kernel in the stream may be scheduled while this one drains.  grid_dep_wait() returns once every kernel
 // this one depends on has completed and its writes are visible: it must precede the first access to anything a
-// predecessor produced.  grid_dep_launch() lets the successor's blocks start (they stop at their own wait).
+// predecessor produced (or, for a cast that may overlap it, an acquire of its commits: Announce).  grid_dep_launch() lets the
+// successor's blocks start (they stop at their own wait).
 __device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ uint32_t ld_acquire(const uint32_t* p) {

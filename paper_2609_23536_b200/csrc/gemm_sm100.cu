@@ -835,11 +835,12 @@ __global__ void __launch_bounds__(threads_of(false), 1) gemm_fp8_kernel(const __
   gemm_body<false>(Problems<1, false>{p});
 }
 
-// The whole-step call's casts may run beside these launches (quantize_multi_kernel, `early`), a block of eight warps of 40
+// The whole-step call's casts may run beside these launches (quantize_multi_kernel, Announce), a block of eight warps of 40
 // registers on each SM: three GEMM warps share a sub-partition's 16384 registers with two of the cast's, which leaves each 144.
-// The bound is that of 448 threads (128 registers taken, none spilled; 168 without it).  A block of hidden 2048 at 2048 tokens:
-// 2389 us a step with the casts between the GEMMs, 2340 with their blocks starting on SMs that a GEMM launch has left, 2116
-// beside its CTAs; eight linears of 2048 x 2048 at 768 tokens 803 / 778 / 749.
+// The bound is that of 448 threads (128 registers taken, none spilled; 168 without it).  us a step with the casts between the
+// GEMMs / with their blocks starting on SMs that a GEMM launch has left (168 registers) / beside its CTAs, under the power limit:
+// a block of hidden 2048 at 2048 tokens 2620 / 2575 / 2510, 48 linears of 1024 4990 / 4910 / 4880, a 4096 / 11008 layer at 256
+// tokens 1564 / 1536 / 1536.
 constexpr int SHARED_SM_THREADS = 448;
 
 // Several independent GEMMs in one launch: up to eight (a parameter block of 5 KB), or what the parameter space holds.

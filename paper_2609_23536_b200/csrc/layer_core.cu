@@ -150,7 +150,8 @@ void ctx_release(qe_ctx* c) {
 
 
 // One launch with programmatic stream serialization: the kernel may be scheduled while its predecessor in the stream
-// drains; every kernel of the library waits for its predecessors (griddepcontrol.wait) before touching their data.
+// drains; every kernel of the library waits for its predecessors (griddepcontrol.wait) before touching their data, or, a
+// cast that may overlap a GEMM launch, acquires that launch's commits (Announce).
 cudaError_t launch_pdl(const qe::Launch& l, cudaStream_t stream) {
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = l.grid;

@@ -486,7 +486,9 @@ bool tensors_apart(qe_layer* const* layers, uint32_t n_layers, const qe_step_act
   }
 }
 
-// Actions of a round of a list whose tensors are apart: forwards and input gradients for two launches.
+// Actions of a round of a list whose tensors are apart: forwards and input gradients for two launches (us a step with 28 / 56 / 112:
+// 48 linears of 1024 at 512 tokens 5310 / 5240 / 4640, at 256 993 / 905 / 863; 64 of 512 at 512 1000 / 848 / 882; steps of up to
+// 32 linears the same).
 constexpr uint32_t kApartGroup = 2 * qe::kMaxProblems;
 }  // namespace
 
@@ -551,11 +553,13 @@ int32_t qe_step_run(qe_ctx* ctx, qe_layer* const* layers, uint32_t n_layers, con
   // pass below runs instead and reports the failing action.
   // Weight gradients: qe_plan_step collects a layer's and lets one launch add them up, as far as a sum stays within 8192
   // tokens and holds three products.  Few tokens make the destination's traffic the cost of a weight gradient: eight
-  // microbatches of 256 tokens through a 4096 / 11008 layer 2860 -> 1890 us a step.  With 2048 tokens a sum of four gains 2 %.
-  // Tiles that last several times as long leave more of the chip idle at the end of a launch, which sums of two do not make
-  // up for (blocks of eight microbatches, sums against launches one by one): hidden 2048, three products at 2176 tokens 3132 us
-  // for 3276, at 2432 3754 for 4013, at 2560 3368 for 3512; two at 3072 4178 for 4094, at 3584 4777 for 4641; hidden 4096, three
-  // at 2304 9116 for 9337, two at 2816 11150 for 11087; hidden 1024, three at 2560 1190 for 1181, two at 3584 1595 for 1561.
+  // microbatches of 256 tokens through a 4096 / 11008 layer 2860 -> 1890 us a step.  Blocks of eight microbatches, sums against
+  // launches one by one: four products at 2048 tokens, hidden 1024 705 us for 794, 2048 2180 for 2410, 4096 9320 for 10310;
+  // three at 2688, hidden 4096 13310 for 13970.  Tiles that last several times as long leave more of the chip idle at the end of
+  // a launch; with the casts between the launches sums of two did not make up for that (hidden 2048 at 3072 tokens 4178 for 4094,
+  // at 3584 4777 for 4641; hidden 4096 at 2816 11150 for 11087), which is where the line was drawn.  With the casts beside the
+  // launches they do where tensors are apart (two products, hidden 4096 at 2816 14000 for 14600, at 3584 17270 for 17890; hidden
+  // 2048 3460 for 3430 and 4140 for 4530): the line lies lower than it could there.
   uint32_t T_max = 0;
   for (uint32_t l = 0; l < n_layers; ++l) T_max = std::max(T_max, layers[l]->cfg.T);
   // A layer that the list names by more than one index is planned without sums (a sum belongs to one index), and two of its
@@ -569,7 +573,7 @@ int32_t qe_step_run(qe_ctx* ctx, qe_layer* const* layers, uint32_t n_layers, con
   // sixteenth at 1920 tokens, a quarter at 384; launches of their own cost more).  us a step, layers in turn / at once:
   // 48 linears of 1024 x 1024 at 512 tokens 13250 / 5340; six of 1536 x 1536 at 1152 tokens (odd) 889 / 351; eight of 2048 x
   // 2048 at 768 1316 / 871; a 4096 / 11008 layer at 256 1776 / 1619; blocks of hidden 1024 at 3072 970 / 853, 2048 at 2048
-  // 2900 / 2795; hidden 4096 at 4096, which the power limit bounds, the same.
+  // 2900 / 2795; hidden 4096 at 4096, which the power limit bounds, the same.  (Both sides with the casts between the GEMMs.)
   std::vector<std::vector<uint32_t>> rounds;  // indices into actions[]
   bool apart = false;
   if (!temp && ctx->step_window > 1) {
@@ -678,7 +682,9 @@ int32_t qe_step_run(qe_ctx* ctx, qe_layer* const* layers, uint32_t n_layers, con
     }
     // A long list goes out in pieces (in graph mode each a graph of its own), so that the device works on one while the host
     // prepares the next: a first one soon, the next while that one runs, later ones so long that the gaps between graphs do
-    // not count (48 linears, 32 microbatches: 3.4 of 16.4 ms were host time ahead of the one launch).
+    // not count.  us a step as one graph / in pieces of 96 / of 384 / of 96, 192 and then 384 actions: 48 linears of 1024, 32
+    // microbatches of 512 tokens 5350 / 4685 / 4685 / 4670, eight of 256 1040 / 880 / 938 / 862; blocks, which are two or three
+    // pieces, the same.
     waiting += (uint32_t)acts.size();
     if (st == QE_OK && waiting >= (pieces < 2 ? 96u << pieces : 384u) && r + 1 < rounds.size()) {
       end_of_piece();

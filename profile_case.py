@@ -1,6 +1,6 @@
 """Small single-kernel cases for profiling (ncu) and quick timing.
 
-    python profile_case.py gemm_f|gemm_di|gemm_dw|gemm_narrow|gemm_odd|gemm_microbatch|gemm_microbatch_grouped|gemm_step|step_sums|quantize|quantize_t|amax|accumulate [--reps N]
+    python profile_case.py gemm_f|gemm_di|gemm_dw|gemm_narrow|gemm_odd|gemm_microbatch|gemm_microbatch_grouped|gemm_step|step_sums|step_many|step_block|quantize|quantize_t|amax|accumulate [--reps N] [--timeline]
 
 Each case holds well under 2 GB on the device, uses operands larger than the 126 MB L2 where DRAM traffic is
 the question, does 2 warm-up launches and then `reps` launches, and prints the CUDA-event time per launch.
@@ -27,6 +27,7 @@ def main():
     ap = argparse.ArgumentParser()
     ap.add_argument("case")
     ap.add_argument("--reps", type=int, default=3)
+    ap.add_argument("--timeline", action="store_true", help="one more call under torch.profiler: every kernel's start, duration and what it overlaps")
     ap.add_argument("--small", action="store_true", help="Llama-block (hidden 2048) shapes instead of Llama-3-8B ones")
     a = ap.parse_args()
     dev = torch.device("cuda", 0)
@@ -82,20 +83,24 @@ def main():
 
         work = {"flop": sum(2.0 * M * N * Kc for M, N, Kc, *_ in shapes),
                 "bytes": sum(M * Kc + N * Kc + M * N * (2 if k == 0 else 8) for M, N, Kc, _, k, _, _ in shapes)}
-    elif a.case == "step_sums":
-        # one optimizer step of a 4096 / 11008 layer, eight microbatches of 256 tokens: the weight gradients go out as sums
-        # (gemm_fp8_pair_wide_kernel)
+    elif a.case.startswith("step_"):
+        # one optimizer step in one call.  step_sums: a 4096 / 11008 layer, eight microbatches of 256 tokens, the weight gradients
+        # go out as sums (gemm_fp8_pair_wide_kernel); step_many: 56 linears of 1024 x 1024, four microbatches of 512, launches of 56
+        # problems; step_block: a block of hidden 2048, eight microbatches of 2048
         from paper_2609_23536_b200.schedules import peak_live, sched
 
-        t, M, shapes = 256, 8, [(4096, 12288), (4096, 4096), (4096, 11008), (11008, 4096)]
+        t, M, shapes = {"step_sums": (256, 8, [(4096, 12288), (4096, 4096), (4096, 11008), (11008, 4096)]),
+                        "step_many": (512, 4, [(1024, 1024)] * 56),
+                        "step_block": (2048, 8, [(2048, 6144), (2048, 2048), (2048, 11264), (5632, 2048)])}[a.case]
+        n = len(shapes)
         order = sched(M, 3, 3)
         ctx = qe.Context(qe.EAGER, step_window=6)
         rnd = lambda *shape: torch.randn(shape, device=dev).to(torch.bfloat16)
         layers = [qe.Layer(ctx, t, K, N, 16, 0, peak_live(order), rnd(N, K).mul_(0.02), unit=u) for u, (K, N) in enumerate(shapes)]
         tensors = [[[rnd(t, d[side]) for d in shapes] for _ in range(M)] for side in (0, 1, 1, 0)]
         grad = torch.zeros(sum(K * N for K, N in shapes), device=dev)
-        acts = [(k, i, m) for k, m in order for i in (range(4) if k == "F" else range(3, -1, -1))]
-        plan = qe.StepPlan(ctx, layers, acts, M, *tensors, grad, [sum(K * N for K, N in shapes[:i]) for i in range(4)])
+        acts = [(k, i, m) for k, m in order for i in (range(n) if k == "F" else range(n - 1, -1, -1))]
+        plan = qe.StepPlan(ctx, layers, acts, M, *tensors, grad, [sum(K * N for K, N in shapes[:i]) for i in range(n)])
 
         def fn():
             plan.run()
@@ -152,6 +157,19 @@ def main():
         out["TFLOP/s"] = round(work["flop"] / ms / 1e9, 1)
     out["GB/s_algorithmic"] = round(work["bytes"] / ms / 1e6, 1)
     print(json.dumps(out))
+    if a.timeline:
+        from torch.profiler import ProfilerActivity, profile
+
+        with profile(activities=[ProfilerActivity.CUDA, ProfilerActivity.CPU]) as p:
+            fn()
+            torch.cuda.synchronize()
+        ks = sorted((e.start_ns() / 1e3, e.duration_ns() / 1e3, e.name()) for e in p.profiler.kineto_results.events()
+                    if "CUDA" in str(e.device_type()) and e.duration_ns() > 0)
+        end = ks[0][0]
+        for start, dur, name in ks:  # start and duration in us, and how much of it lies before the end of what started earlier
+            name = name.replace("(anonymous namespace)::", "").replace("void ", "").replace("qe::", "").split("(")[0]
+            print("%9.1f %7.1f %7.1f  %s" % (start - ks[0][0], dur, max(0.0, min(end, start + dur) - start), name))
+            end = max(end, start + dur)
 
 
 if __name__ == "__main__":
