@@ -128,9 +128,10 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
   }
 }
 
-// The same wait by a whole warp (converged).  Its lanes leave it together and with one answer: a lane that was still polling
-// while the elected one went on to issue could find the barrier a phase further, take that for the phase it waits for not being
-// over, and wait on; no lane may give up alone either.
+// The same wait by a whole warp (converged), as every role makes it.  Its lanes leave it together and with one answer: in the
+// roles that issue from an elected lane, a lane that was still polling while that one went on could find the barrier a phase
+// further, take that for the phase it waits for not being over, and wait on; and where one lane gives up (the launch is being
+// abandoned) while another finds the phase complete, the warp may not go on to its next aligned instruction in parts.
 __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile uint32_t* abort_flag, uint32_t* status,
                                                uint32_t err_bit) {
   return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag, status, err_bit));
@@ -626,7 +627,7 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
         if ((uint32_t)lane < p.nseg) my_alpha = __fmul_rn(p.alpha_a[p.slot_a[lane]], p.alpha_b[p.slot_b[lane]]);
         auto take = [&](uint32_t seg, auto first) {
           const float alpha = __shfl_sync(0xffffffffu, my_alpha, (int)seg);
-          if (!(ok = mbar_wait(tfull_bar(acc), acc_ph, abort_flag, status, ERR_EPILOGUE))) return;
+          if (!(ok = mbar_wait_warp(tfull_bar(acc), acc_ph, abort_flag, status, ERR_EPILOGUE))) return;
           tc_fence_after();
           const uint32_t t_row = tmem_base + ((quad * 32u) << 16) + acc * ACC_COLS + half * (tile_n / 2);
 #pragma unroll
@@ -675,7 +676,7 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
           if ((uint32_t)j < nch) asm volatile("prefetch.global.L2 [%0];" ::"l"(d + 128 * j));
       }
       uint32_t r[2][32];
-      if (!(ok = mbar_wait(tfull_bar(acc), acc_ph, abort_flag, status, ERR_EPILOGUE))) break;
+      if (!(ok = mbar_wait_warp(tfull_bar(acc), acc_ph, abort_flag, status, ERR_EPILOGUE))) break;
       tc_fence_after();
       const uint32_t t_row = tmem_base + ((quad * 32u) << 16) + acc * ACC_COLS + half * (tile_n / 2);
       uint32_t amax_bits = 0;
