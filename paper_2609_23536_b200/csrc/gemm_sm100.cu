@@ -17,9 +17,9 @@
 //               L2, one per element and launch, and the destination tile is prefetched into L2 while the tile's
 //               main loop runs.  The reduction is a plain round-to-nearest FP32 addition (subnormal values kept).
 //   The launch may also carry up to fifty-six independent problems (grouped launch): tiles are numbered problem after
-//   problem and each role looks its tile's problem up, so that one set of persistent CTAs packs them all.
+//   problem and a warp of its own tells the roles what each tile is, so that one set of persistent CTAs packs them all.
 //   A problem may be the sum of several products (the deferred weight gradients of several microbatches): each gets an
-//   accumulator of its own, and the epilogue adds them up in registers before the one store.
+//   accumulator of its own, the epilogue adds them up in registers, and a warp of its own stores the result.
 //   A launch of one GEMM with an odd number of 128-row tiles may run without clusters, a CTA to a tile of 128 x 256
 //   (gemm_fp8_kernel: the same roles, four stages of 128 rows of A and 256 of B, tcgen05.mma.cta_group::1; see one_cta).
 // Rows beyond M (M is a multiple of 128; a pair's tile has 256) are read as zeros by TMA and never stored.
@@ -66,26 +66,37 @@ struct Form {
 // (barrier operations; 45 to 90 for another load), while the MMAs of a K block take 240 to 260 clocks at up to 128 columns: with
 // stages of one K block, tiles of 64 columns ran at 387 clocks a block, now at 339 (256 x 2048 x 8192: 15.9 -> 14.1 us).  There
 // shared memory bounds them: 20 KB written and 20 to 24 KB read a block at 128 bytes a clock.
-constexpr uint32_t RING_BYTES = 12 * A_BYTES;
-constexpr int MAX_STAGES = 6;
-template <bool PAIR>
-struct Ring {
-  uint32_t blocks, stages, stage_bytes;  // K blocks of a stage, stages, bytes of one
-  __device__ __forceinline__ explicit Ring(uint32_t tile_n)
-      : blocks(PAIR && tile_n < 256u ? 2u : 1u), stages(PAIR && tile_n == 256u ? 6u : 4u), stage_bytes(RING_BYTES / stages) {}
-  __device__ __forceinline__ uint32_t b_offset() const { return blocks * A_BYTES; }
-};
-static_assert(RING_BYTES / 4 >= 2 * A_BYTES + 2 * 64 * BK && RING_BYTES / 4 >= 3 * A_BYTES && RING_BYTES / 6 >= 2 * A_BYTES, "");
-constexpr uint32_t TMEM_COLS = 512;
 constexpr uint32_t EPI_BUF_BYTES = 4096;                     // per epilogue warp: one FP32 or two bf16 32 x 32 output tiles
                                                              // (1 KB-aligned, swizzled) that the bulk-store unit reads
+constexpr uint32_t RING_AND_BUFS = 14 * A_BYTES;
+constexpr int MAX_STAGES = 6;
+template <bool PAIR, uint32_t BUFS>
+struct Ring {
+  static constexpr uint32_t BYTES = RING_AND_BUFS - 8 * BUFS * EPI_BUF_BYTES;
+  uint32_t blocks, stages, stage_bytes;  // K blocks of a stage, stages, bytes of one
+  __device__ __forceinline__ explicit Ring(uint32_t tile_n)
+      : blocks(PAIR && tile_n < 256u ? 2u : 1u),
+        stages(PAIR && tile_n == 256u ? BYTES / (2 * A_BYTES) : BYTES / (3 * A_BYTES)),
+        stage_bytes(PAIR && tile_n == 256u ? 2 * A_BYTES : 3 * A_BYTES) {}
+  __device__ __forceinline__ uint32_t b_offset() const { return blocks * A_BYTES; }
+};
+static_assert(2 * A_BYTES + 2 * 64 * BK <= 3 * A_BYTES && Ring<true, 1>::BYTES / (2 * A_BYTES) <= MAX_STAGES, "");
+constexpr uint32_t TMEM_COLS = 512;
 constexpr int EPI_WARPS = 8, EPI_THREADS = EPI_WARPS * 32;
-// Threads of a CTA: warps 0 and 1, then the epilogue's eight.  The variant that sums several products keeps a tile row of
-// 128 FP32 per epilogue thread: its epilogue warps are two whole warpgroups (warps 2 and 3 idle), which take over
-// registers that the first warpgroup hands back (launched with 168 a thread; 40 + 2 * 224 <= 3 * 168).
-constexpr int threads_of(bool sums) { return sums ? 384 : 320; }
+// Threads of a CTA: warps 0 and 1, then the epilogue's eight, and where a launch has several problems one for the tile records.
+// The variant that sums several products keeps a tile row of 128 FP32 per epilogue thread: its epilogue warps are two whole
+// warpgroups (warps 2 and 3 make records and store results), which take over registers that the first warpgroup hands back
+// (launched with 168 a thread; 56 + 2 * 224 <= 3 * 168).
+constexpr int threads_of(bool sums, bool several) { return sums ? 384 : several ? 352 : 320; }
 static_assert(EPI_WARPS == 8, "shared-memory budget below assumes 8 epilogue warps");
-constexpr uint32_t SMEM_BYTES = RING_BYTES + 1024 /*alignment slack*/ + 256 /*barriers, flags*/ + 8 * EPI_BUF_BYTES;
+// Launches of several problems: what the roles need to know of a tile is put into a small ring of records by a warp of its own,
+// some tiles ahead.  Looked up by each role, it is a chain of reads of the parameter block, which no constant cache holds: 800
+// to 2300 clocks a tile and role, where the MMAs of a tile of eight K blocks take 4100 (the records: 300 to 450).
+constexpr uint32_t INFO_SLOTS = 4, INFO_BYTES = 128;
+constexpr uint32_t BARS_BYTES = 512;
+// (What the SM has left has to hold a block of the casts that run beside these launches: 1 KB that the system takes and 36 bytes.)
+constexpr uint32_t SMEM_BYTES = RING_AND_BUFS + BARS_BYTES /*barriers, flags*/ + INFO_SLOTS * INFO_BYTES;
+static_assert(SMEM_BYTES + 1024 + 2048 <= 228 * 1024, "no room for a cast beside a GEMM launch");
 constexpr long long WAIT_BUDGET_CYCLES = 4000000000ll;  // ~2 s at the maximum SM clock
 
 constexpr uint32_t ERR_PRODUCER = 1u, ERR_MMA = 2u, ERR_EPILOGUE = 4u;
@@ -225,6 +236,13 @@ __device__ __forceinline__ void tc_mma_f8(uint32_t d_tmem, uint64_t adesc, uint6
   else tc_mma_f8_one(d_tmem, adesc, bdesc, idesc, accumulate);
 }
 
+// Load of a 32 x 32 block of an output.
+__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, uint32_t bar, int c0, int c1) {
+  asm volatile("cp.async.bulk.tensor.2d.shared::cta.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
+               ::"r"(dst), "l"(map), "r"(bar), "r"(c0), "r"(c1)
+               : "memory");
+}
+
 __device__ __forceinline__ void tma_prefetch(const CUtensorMap* map, int c0, int c1, int c2, int c3) {
   asm volatile("cp.async.bulk.prefetch.tensor.4d.L2.global.tile [%0, {%1, %2, %3, %4}];" ::"l"(map), "r"(c0), "r"(c1), "r"(c2), "r"(c3) : "memory");
 }
@@ -285,6 +303,40 @@ __device__ __forceinline__ void st_tile_f32(uint32_t buf, uint32_t row, const fl
   }
 }
 
+// Two FP32 values at a time.
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pack2(uint32_t lo, uint32_t hi) {
+  f32x2 v;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "r"(lo), "r"(hi));
+  return v;
+}
+// a * b, rounded by itself.  (Written as mul.rn, ptxas makes a multiply-add of it and the addition that follows, which rounds
+// once.  So it is one already, with a -0 that ptxas cannot see: that changes no product, not even the sign of a zero.)
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b, f32x2 minus_zero) {
+  f32x2 v;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(v) : "l"(a), "l"(b), "l"(minus_zero));
+  return v;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+  f32x2 v;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(v) : "l"(a), "l"(b));
+  return v;
+}
+__device__ __forceinline__ void st_tile_f32x2(uint32_t buf, uint32_t row, const f32x2 (&v)[16]) {
+#pragma unroll
+  for (int c = 0; c < 8; ++c) {
+    const uint32_t dst = buf + row * 128u + (((uint32_t)c ^ (row & 7u)) << 4);
+    asm volatile("st.shared.v2.b64 [%0], {%1, %2};" ::"r"(dst), "l"(v[2 * c]), "l"(v[2 * c + 1]) : "memory");
+  }
+}
+__device__ __forceinline__ void ld_tile_f32x2(uint32_t buf, uint32_t row, f32x2 (&v)[16]) {
+#pragma unroll
+  for (int c = 0; c < 8; ++c) {
+    const uint32_t src = buf + row * 128u + (((uint32_t)c ^ (row & 7u)) << 4);
+    asm volatile("ld.shared.v2.b64 {%0, %1}, [%2];" : "=l"(v[2 * c]), "=l"(v[2 * c + 1]) : "r"(src) : "memory");
+  }
+}
+
 __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
   __nv_bfloat162 v = __floats2bfloat162_rn(a, b);  // .x = a in the low half
   return *reinterpret_cast<uint32_t*>(&v);
@@ -324,22 +376,25 @@ __device__ __forceinline__ uint32_t snake_tile(uint32_t w, uint32_t first, uint3
 // ------------------------------------------------------------------------------------------------ problem lookup
 // A launch computes one GEMM, or (grouped launch) several independent ones whose tiles are numbered one after the
 // other, so that one set of persistent CTAs packs them into common waves and the launch overhead is paid once.
-template <int NP, bool SEVERAL>
+template <int NP, bool SEVERAL, uint32_t EPI_BUFS = 1>
 struct Problems {
   static constexpr bool ONE = NP == 1, SUMS = SEVERAL;  // one problem; problems may have several products
+  static constexpr uint32_t BUFS = EPI_BUFS;            // output buffers of an epilogue warp
   const GemmLaunchParams<NP>& g;
   __device__ __forceinline__ uint32_t count() const { return NP == 1 ? 1u : g.n; }
   __device__ __forceinline__ uint32_t total_tiles() const { return g.tile_end[count() - 1]; }
   // `i`: the problem of an earlier tile of the same role (its tiles come in ascending order), from which the search goes on
   __device__ __forceinline__ const GemmParams& at(uint32_t tile, uint32_t& i, uint32_t& local) const {
-    if (NP == 1) {
+    if constexpr (NP == 1) {
       local = tile;
       return g.prob[0];
+    } else {
+      while (i + 1 < g.n && tile >= g.tile_end[i]) ++i;
+      local = tile - (i ? g.tile_end[i - 1] : 0u);
+      return g.prob[i];
     }
-    while (i + 1 < count() && tile >= g.tile_end[i]) ++i;
-    local = tile - (i ? g.tile_end[i - 1] : 0u);
-    return g.prob[i];
   }
+  __device__ __forceinline__ const GemmParams& problem(uint32_t i) const { return g.prob[NP == 1 ? 0u : i]; }
   __device__ __forceinline__ const GemmParams& first() const { return g.prob[0]; }
   __device__ __forceinline__ const CommitParams& commit(uint32_t i) const { return g.prob[i].commit; }
   __device__ __forceinline__ uint32_t* ticket() const { return g.ticket; }
@@ -349,58 +404,115 @@ struct Problems {
   __device__ __forceinline__ uint32_t* status_of(uint32_t i) const { return g.prob[i].status; }
 };
 
-// 32 floats of one row, read from L2 (the destination of an accumulating launch; earlier launches wrote it there).
-__device__ __forceinline__ void ld_row32(const float* src, float* v) {
-  if ((reinterpret_cast<uintptr_t>(src) & 31u) == 0) {
-#pragma unroll
-    for (int j = 0; j < 4; ++j)
-      asm volatile("ld.relaxed.gpu.global.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-                   : "=f"(v[8 * j]), "=f"(v[8 * j + 1]), "=f"(v[8 * j + 2]), "=f"(v[8 * j + 3]), "=f"(v[8 * j + 4]),
-                     "=f"(v[8 * j + 5]), "=f"(v[8 * j + 6]), "=f"(v[8 * j + 7])
-                   : "l"(src + 8 * j)
-                   : "memory");
-  } else {
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const float4 q = __ldcg(reinterpret_cast<const float4*>(src) + j);
-      v[4 * j] = q.x, v[4 * j + 1] = q.y, v[4 * j + 2] = q.z, v[4 * j + 3] = q.w;
-    }
-  }
-}
+// What the roles need to know of a tile (INFO_BYTES of shared memory at most).  `alpha` is filled in later than the rest: scales
+// come from kernels before this one.
+struct TileInfo {
+  uint32_t problem, m0, n0, num_kb;
+  uint32_t nseg, epi, a_mn, b_mn;
+  uint32_t idesc, b_desc_hi, b_step, ldo;
+  uint32_t M, N;
+  unsigned long long out;
+  unsigned long long amax_bits;
+  uint8_t slot_a[kMaxSegments], slot_b[kMaxSegments];
+  float alpha[kMaxSegments];
+  uint32_t minus_zero;  // see mul2; 0 where the tile is no sum
+};
+static_assert(sizeof(TileInfo) <= INFO_BYTES && offsetof(TileInfo, alpha) % 4 == 0, "");
+// The same value in every lane, and known to be: kept in a uniform register, as the instructions of the issuing roles want it.
+__device__ __forceinline__ uint32_t uniform(uint32_t v) { return __reduce_or_sync(0xffffffffu, v); }
 
 // ------------------------------------------------------------------------------------------------ kernel
 template <bool PAIR, class PS>
 __device__ __forceinline__ void gemm_body(const PS& ps) {
   constexpr uint32_t CTAS = Form<PAIR>::CTAS, TILE_M = Form<PAIR>::TILE_M;
-  constexpr bool SUMS = PS::SUMS;
-  constexpr int EPI_WARP0 = SUMS ? 4 : 2;  // first epilogue warp
-  extern __shared__ uint8_t smem_raw[];
-  const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
+  constexpr bool SUMS = PS::SUMS, ONE = PS::ONE;
+  constexpr int EPI_WARP0 = SUMS ? 4 : 2;    // first epilogue warp
+  constexpr int INFO_WARP = SUMS ? 2 : 10;  // (launches of several problems)
+  constexpr int STORE_WARP = 3;             // (sums)
+  constexpr uint32_t BUFS = PS::BUFS, RING_BYTES = Ring<PAIR, BUFS>::BYTES;
+  extern __shared__ __align__(1024) uint8_t smem_raw[];
+  const uint32_t smem_base = smem_u32(smem_raw);
   const uint32_t epi_base = smem_base + RING_BYTES;  // 1 KB-aligned
-  const uint32_t bar_base = epi_base + 8 * EPI_BUF_BYTES;
-  // barrier block: full[MAX_STAGES], empty[MAX_STAGES], tmem_full[2], tmem_empty[2], then tmem address + abort flag
+  const uint32_t bar_base = smem_base + RING_AND_BUFS;
+  // barrier block: full[MAX_STAGES], empty[MAX_STAGES], tmem_full[2], tmem_empty[2], tmem address + abort flag + last-CTA flag,
+  // of the tile records full, scales and empty[INFO_SLOTS], of the buffers of sums ready and result[2][BUFS]
   auto full_bar = [&](uint32_t s) { return bar_base + 8u * s; };
   auto empty_bar = [&](uint32_t s) { return bar_base + 8u * (MAX_STAGES + s); };
   auto tfull_bar = [&](int a) { return bar_base + 8u * (2 * MAX_STAGES + a); };
   auto tempty_bar = [&](int a) { return bar_base + 8u * (2 * MAX_STAGES + 2 + a); };
-  uint8_t* gen_base = smem_raw + (smem_base - smem_u32(smem_raw));
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(gen_base + RING_BYTES + 8 * EPI_BUF_BYTES + 8 * (2 * MAX_STAGES + 4));
+  uint8_t* const gen_base = smem_raw;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(gen_base + RING_AND_BUFS + 8 * (2 * MAX_STAGES + 4));
+  constexpr uint32_t INFO_BARS = 8 * (2 * MAX_STAGES + 4) + 16;
+  constexpr uint32_t BUF_BARS = INFO_BARS + 8 * 3 * INFO_SLOTS;
+  static_assert(BUF_BARS + 8 * 4 * BUFS <= BARS_BYTES, "barrier block too large");
+  // sums: buffer b of a half of the tile's columns (128 rows x 32 columns) is the epilogue's again (free, or holding what the
+  // tile is added to) / is the storing warp's
+  auto ready_bar = [&](uint32_t h, uint32_t b) { return bar_base + BUF_BARS + 8u * (h * BUFS + b); };
+  auto result_bar = [&](uint32_t h, uint32_t b) { return ready_bar(h, b) + 16u * BUFS; };
+  auto info_bar = [&](uint32_t n) { return bar_base + INFO_BARS + 8u * (n % INFO_SLOTS); };  // of the CTA's n-th tile
+  auto scales_bar = [&](uint32_t n) { return info_bar(n) + 8u * INFO_SLOTS; };
+  auto taken_bar = [&](uint32_t n) { return info_bar(n) + 16u * INFO_SLOTS; };
+  auto info_of = [&](uint32_t n) { return reinterpret_cast<TileInfo*>(gen_base + RING_AND_BUFS + BARS_BYTES + INFO_BYTES * (n % INFO_SLOTS)); };
+  auto info_parity = [](uint32_t n) { return n / INFO_SLOTS & 1u; };
   volatile uint32_t* abort_flag = tmem_slot + 1;
   uint32_t* last_flag = tmem_slot + 2;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = PAIR ? cluster_ctarank() : 0u;  // position in the CTA pair; rank 0 issues the MMAs
   const uint32_t num_tiles = ps.total_tiles();
-  const Ring<PAIR> ring(ps.first().tile_n);  // (one tile width per launch)
+  const Ring<PAIR, BUFS> ring(ps.first().tile_n);  // (one tile width per launch)
   const uint32_t first_tile = blockIdx.x / CTAS, tile_step = gridDim.x / CTAS;
   uint32_t* const status = ps.first().status;
-// per tile: which problem it belongs to (`p`), its index inside that problem and the problem's tiling
-#define QE_TILE_PROBLEM()                                                                                     \
-  uint32_t local_tile;                                                                                        \
-  const GemmParams& p = ps.at(tile, at_problem, local_tile);                                                  \
-  const uint32_t tile_n = p.tile_n, tiles_m = (p.M + TILE_M - 1) / TILE_M, tiles_n = (p.N + tile_n - 1) / tile_n; \
-  const uint32_t num_kb = p.Kc / BK;                                                                          \
-  const bool m_fastest = p.M <= p.N
+  const uint32_t tile_n = ps.first().tile_n;  // (of the whole launch)
+  // which problem a tile belongs to and where it lies in it; `at_problem` as in Problems::at
+  auto look_up = [&](uint32_t tile, uint32_t& at_problem, TileInfo& t) -> const GemmParams& {
+    uint32_t local_tile;
+    const GemmParams& p = ps.at(tile, at_problem, local_tile);
+    tile_coords<TILE_M>(local_tile, (p.M + TILE_M - 1) / TILE_M, (p.N + tile_n - 1) / tile_n, p.M <= p.N, tile_n, t.m0, t.n0);
+    t.problem = at_problem;
+    t.num_kb = p.Kc / BK;
+    t.nseg = SUMS ? p.nseg : 1u;
+    t.epi = (uint32_t)p.epi;
+    t.a_mn = p.a_mn;
+    t.b_mn = p.b_mn;
+    t.idesc = p.idesc;
+    t.b_desc_hi = p.b_desc_hi;
+    t.b_step = p.b_step;
+    t.ldo = p.ldo;
+    t.M = p.M;
+    t.N = p.N;
+    t.out = (unsigned long long)p.out;
+    t.amax_bits = (unsigned long long)p.amax_bits;
+    return p;
+  };
+  // ... from the records that the info warp makes of it, for the CTA's n-th tile: one role's reading of it, and that it has
+  auto await = [&](uint32_t bar, uint32_t parity, uint32_t err_bit) { return mbar_wait_warp(bar, parity, abort_flag, status, err_bit); };
+  auto await_tile = [&](uint32_t n, uint32_t err_bit) { return await(info_bar(n), info_parity(n), err_bit); };
+  auto took_tile = [&](uint32_t n) {
+    __syncwarp();
+    if (lane == 0) mbar_arrive(taken_bar(n));
+  };
+  // info warp: makes the record of the CTA's n-th tile
+  auto announce = [&](uint32_t n, uint32_t tile, uint32_t& at_problem) {
+    const uint32_t before = at_problem;
+    TileInfo t;
+    const GemmParams& p = look_up(tile, at_problem, t);
+    if ((n == 0 || at_problem != before) && lane < 3)
+      asm volatile("prefetch.tensormap [%0];" ::"l"(lane == 0 ? &p.tmA : lane == 1 ? &p.tmB : &p.tmD) : "memory");
+    TileInfo* const to = info_of(n);
+    if (lane == 0) {
+      uint4* const w = reinterpret_cast<uint4*>(to);
+      const uint4* const v = reinterpret_cast<const uint4*>(&t);
+#pragma unroll
+      for (uint32_t i = 0; i < offsetof(TileInfo, amax_bits) / 16; ++i) w[i] = v[i];
+      to->amax_bits = t.amax_bits;
+      if (SUMS) to->minus_zero = p.sum ? 0x80000000u : 0u;
+    }
+    if (SUMS && (uint32_t)lane < kMaxSegments) to->slot_a[lane] = p.slot_a[lane], to->slot_b[lane] = p.slot_b[lane];
+    if (!SUMS && lane == 0) to->slot_a[0] = p.slot_a[0], to->slot_b[0] = p.slot_b[0];
+    __syncwarp();
+    if (lane == 0) mbar_arrive(info_bar(n));
+  };
 
   if (threadIdx.x == 32) {  // descriptor fetch overlaps the rest of the prologue (and the predecessor's tail)
     const GemmParams& q = ps.first();  // (a group's other descriptors are fetched on first use)
@@ -416,6 +528,17 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
     for (int a = 0; a < 2; ++a) {
       mbar_init(tfull_bar(a), 1);
       mbar_init(tempty_bar(a), EPI_WARPS * CTAS);  // the epilogue warps of every CTA of the tile
+    }
+    if (SUMS)
+      for (uint32_t i = 0; i < 2 * BUFS; ++i) {
+        mbar_init(ready_bar(0, 0) + 8u * i, 1);
+        mbar_init(result_bar(0, 0) + 8u * i, EPI_WARPS / 2);
+      }
+    if (!ONE)
+      for (uint32_t i = 0; i < INFO_SLOTS; ++i) {
+      mbar_init(info_bar(i), 1);
+      mbar_init(scales_bar(i), 1);
+      mbar_init(taken_bar(i), EPI_WARPS + 1 + (SUMS ? 1u : 0u) + (rank == 0 ? 1u : 0u));  // epilogue, producer, storing warp, MMA issuer
     }
     *abort_flag = 0u;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -439,18 +562,23 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
   if (PAIR) cluster_sync_all();  // the peer's barriers are initialised before anything signals them
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
-  if (warp == 0 && lane == 0 && first_tile < num_tiles) {
+  if (warp == (ONE ? 0 : INFO_WARP) && first_tile < num_tiles) {
     // While the predecessor drains: pull the first ring-full of B tiles of this CTA's first tile towards L2.  A
     // prefetch moves no data into the SM, so it is harmless even if the predecessor is still writing that operand.
-    const uint32_t tile = first_tile;
     uint32_t at_problem = 0;
-    QE_TILE_PROBLEM();
-    uint32_t m0, n0;
-    tile_coords<TILE_M>(local_tile, tiles_m, tiles_n, m_fastest, tile_n, m0, n0);
-    const int rb = (int)(n0 + rank * (tile_n / 2));
-    const CUtensorMap* tmB = &p.tmB;
-    for (uint32_t kb = 0; kb < num_kb && kb < ring.blocks * ring.stages; kb += ring.blocks)
-      for (int b = 0; b < (PAIR ? 1 : 2); ++b) tma_prefetch(tmB, p.b_mn ? rb + b * (int)BM : 0, p.b_mn ? 0 : rb + b * (int)BM, (int)kb, p.slot_b[0]);
+    TileInfo t;
+    const GemmParams& p = look_up(first_tile, at_problem, t);
+    if (lane == 0) {
+      const int rb = (int)(t.n0 + rank * (tile_n / 2));
+      const CUtensorMap* tmB = &p.tmB;
+      for (uint32_t kb = 0; kb < t.num_kb && kb < ring.blocks * ring.stages; kb += ring.blocks)
+        for (int b = 0; b < (PAIR ? 1 : 2); ++b)
+          tma_prefetch(tmB, p.b_mn ? rb + b * (int)BM : 0, p.b_mn ? 0 : rb + b * (int)BM, (int)kb, p.slot_b[0]);
+    }
+    // (and the first records)
+    if (!ONE)
+      for (uint32_t n = 0, tile = first_tile, from = 0; n < INFO_SLOTS && tile < num_tiles; ++n, tile = snake_tile(n, first_tile, tile_step))
+        announce(n, tile, from);
   }
   // Everything above (barriers, tensor memory) touched no data a predecessor produces and may overlap the previous
   // kernel's tail; operands, scales and the destination may come from it, so wait for it here.
@@ -488,28 +616,44 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
   // same code ran 4 % slower, small launches and large ones alike.)
   if (SUMS) {
     __syncwarp();
-    if (warp < EPI_WARP0) asm volatile("setmaxnreg.dec.sync.aligned.u32 40;");
+    if (warp < EPI_WARP0) asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
   }
   if (warp == 0) {
     // ---------------------------------------------------------------- TMA producer
     const bool elected = elect_one();
-    uint32_t s = 0, ph = 0, at_problem = 0;
+    uint32_t s = 0, ph = 0;
     bool ok = true;
-    for (uint32_t wave = 0, tile = first_tile; ok && tile < num_tiles; ++wave, tile = snake_tile(wave, first_tile, tile_step)) {
-      QE_TILE_PROBLEM();
-      uint32_t m0, n0;
-      tile_coords<TILE_M>(local_tile, tiles_m, tiles_n, m_fastest, tile_n, m0, n0);
+    for (uint32_t n = 0, tile = first_tile; ok && tile < num_tiles; ++n, tile = snake_tile(n, first_tile, tile_step)) {
+      TileInfo t;
+      unsigned long long slots_a = 0, slots_b = 0;  // a byte per product
+      if (ONE) {
+        uint32_t at_problem = 0;
+        const GemmParams& p = look_up(tile, at_problem, t);
+        slots_a = p.slot_a[0], slots_b = p.slot_b[0];
+      } else {
+        if (!(ok = await_tile(n, ERR_PRODUCER))) break;
+        const TileInfo& r = *info_of(n);
+        t.problem = uniform(r.problem), t.m0 = uniform(r.m0), t.n0 = uniform(r.n0), t.num_kb = uniform(r.num_kb);
+        t.nseg = SUMS ? uniform(r.nseg) : 1u, t.a_mn = uniform(r.a_mn), t.b_mn = uniform(r.b_mn);
+        if (SUMS) {
+          slots_a = *reinterpret_cast<const unsigned long long*>(r.slot_a), slots_b = *reinterpret_cast<const unsigned long long*>(r.slot_b);
+        } else {
+          slots_a = uniform(r.slot_a[0]), slots_b = uniform(r.slot_b[0]);
+        }
+        took_tile(n);
+      }
+      const GemmParams& p = ps.problem(t.problem);
       // contraction-major operand: box = 128 K-bytes x rows x blocks at (0, row, block); MN-major operand (stored as [Kc, rows]):
       // box = row-bytes x 128 K-rows x blocks at (row, 0, block).  Either way 128 bytes per row and block land in shared memory.
-      const int ra = (int)(m0 + rank * BM), rb = (int)(n0 + rank * (tile_n / 2));
-      const int a0 = p.a_mn ? ra : 0, a1 = p.a_mn ? 0 : ra, b0 = p.b_mn ? rb : 0, b1 = p.b_mn ? 0 : rb;
+      const int ra = (int)(t.m0 + rank * BM), rb = (int)(t.n0 + rank * (tile_n / 2));
+      const int a0 = t.a_mn ? ra : 0, a1 = t.a_mn ? 0 : ra, b0 = t.b_mn ? rb : 0, b1 = t.b_mn ? 0 : rb;
       // both CTAs of a pair credit the even CTA's barrier, which expects the bytes of the whole pair (blocks beyond the
       // contraction are filled with zeros and counted)
       const uint32_t bytes = ring.blocks * (CTAS * A_BYTES + tile_n * BK);
-      for (uint32_t seg = 0; ok && seg < (SUMS ? p.nseg : 1u); ++seg) {
+      for (uint32_t seg = 0; ok && seg < t.nseg; ++seg, slots_a >>= 8, slots_b >>= 8) {
         const CUtensorMap *tmA = &p.tmA, *tmB = &p.tmB;
-        const int sa = p.slot_a[SUMS ? seg : 0u], sb = p.slot_b[SUMS ? seg : 0u];
-        for (uint32_t kb = 0; kb < num_kb; kb += ring.blocks) {
+        const int sa = SUMS ? (int)uniform((uint32_t)slots_a & 255u) : (int)slots_a, sb = SUMS ? (int)uniform((uint32_t)slots_b & 255u) : (int)slots_b;
+        for (uint32_t kb = 0; kb < t.num_kb; kb += ring.blocks) {
           if (!(ok = mbar_wait_warp(empty_bar(s), ph ^ 1u, abort_flag, status, ERR_PRODUCER))) break;
           const uint32_t a_dst = smem_base + s * ring.stage_bytes, b_dst = a_dst + ring.b_offset();
           if (elected) {
@@ -518,7 +662,7 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
             tma_load<PAIR>(a_dst, tmA, bar, a0, a1, (int)kb, sa);
             tma_load<PAIR>(b_dst, tmB, bar, b0, b1, (int)kb, sb);
             // (a CTA on its own loads the tile's 256 rows of B as two boxes of 128, one behind the other)
-            if (!PAIR) tma_load<PAIR>(b_dst + A_BYTES, tmB, bar, p.b_mn ? rb + (int)BM : 0, p.b_mn ? 0 : rb + (int)BM, (int)kb, sb);
+            if (!PAIR) tma_load<PAIR>(b_dst + A_BYTES, tmB, bar, t.b_mn ? rb + (int)BM : 0, t.b_mn ? 0 : rb + (int)BM, (int)kb, sb);
           }
           if (++s == ring.stages) { s = 0; ph ^= 1u; }
         }
@@ -533,14 +677,24 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
     // ---------------------------------------------------------------- MMA issuer
     if (rank == 0) {
       const bool elected = elect_one();
-      uint32_t s = 0, ph = 0, acc = 0, acc_ph = 0, at_problem = 0;
+      uint32_t s = 0, ph = 0, acc = 0, acc_ph = 0;
       bool ok = true;
-      for (uint32_t wave = 0, tile = first_tile; ok && tile < num_tiles; ++wave, tile = snake_tile(wave, first_tile, tile_step)) {
-        QE_TILE_PROBLEM();
-        (void)tiles_m; (void)tiles_n; (void)m_fastest;
-        const uint32_t idesc = p.idesc, b_hi = p.b_desc_hi, a_step = p.a_mn ? 256u : 2u, b_step = p.b_step;
+      for (uint32_t n = 0, tile = first_tile; ok && tile < num_tiles; ++n, tile = snake_tile(n, first_tile, tile_step)) {
+        TileInfo t;
+        if (ONE) {
+          uint32_t at_problem = 0;
+          look_up(tile, at_problem, t);
+        } else {
+          if (!(ok = await_tile(n, ERR_MMA))) break;
+          const TileInfo& r = *info_of(n);
+          t.num_kb = uniform(r.num_kb), t.nseg = SUMS ? uniform(r.nseg) : 1u;
+          t.idesc = uniform(r.idesc), t.b_desc_hi = uniform(r.b_desc_hi), t.b_step = uniform(r.b_step);
+          t.a_mn = uniform(r.a_mn), t.b_mn = uniform(r.b_mn);
+          took_tile(n);
+        }
+        const uint32_t idesc = t.idesc, b_hi = t.b_desc_hi, a_step = t.a_mn ? 256u : 2u, b_step = t.b_step, num_kb = t.num_kb;
         const uint32_t b_block = tile_n / CTAS * BK / 16u;  // from one block of B in a stage to the next
-        for (uint32_t seg = 0; ok && seg < (SUMS ? p.nseg : 1u); ++seg) {  // an accumulator of its own for each product
+        for (uint32_t seg = 0; ok && seg < t.nseg; ++seg) {  // an accumulator of its own for each product
           if (!(ok = mbar_wait_warp(tempty_bar(acc), acc_ph ^ 1u, abort_flag, status, ERR_MMA))) break;
           tc_fence_after();
           const uint32_t d_tmem = tmem_base + acc * ACC_COLS;
@@ -549,7 +703,7 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
             tc_fence_after();
             const uint32_t a_src = smem_base + s * ring.stage_bytes, b_src = a_src + ring.b_offset();
             const uint64_t adesc = make_desc(a_src, A_DESC_HI);
-            const uint64_t bdesc = make_desc(b_src, b_hi, PAIR || !p.b_mn ? 1u : A_BYTES / 16u);
+            const uint64_t bdesc = make_desc(b_src, b_hi, PAIR || !t.b_mn ? 1u : A_BYTES / 16u);
             if (elected) {
 #pragma unroll
               for (uint32_t k = 0; k < BK / UMMA_K; ++k)
@@ -571,110 +725,192 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
         }
       }
     }
+  } else if (!ONE && warp == INFO_WARP) {
+    // ---------------------------------------------------------------- tile records
+    uint32_t at_problem = 0, announced = 0, fetched_to = 0, last = 0;
+    bool ok = true;
+    auto fetch_rows = [&](uint32_t tile, uint32_t& from) {
+      TileInfo t;
+      look_up(tile, from, t);
+      if (t.epi != 2 || !ps.problem(from).sum) return;
+      const uint32_t rows = min(BM, t.M - min(t.M, t.m0 + rank * BM)), lines = min(tile_n, t.N - t.n0) / 32u;
+      const char* d = reinterpret_cast<const char*>(reinterpret_cast<const float*>(t.out) + (size_t)(t.m0 + rank * BM) * t.ldo + t.n0);
+      for (uint32_t i = (uint32_t)lane; i < rows * lines; i += 32)
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(d + (size_t)(i / lines) * t.ldo * 4u + 128u * (i % lines)));
+    };
+    for (uint32_t n = 0, tile = first_tile; ok && tile < num_tiles; ++n, tile = snake_tile(n, first_tile, tile_step)) {
+      if (n >= INFO_SLOTS) {
+        if (!(ok = await(taken_bar(n), info_parity(n) ^ 1u, ERR_PRODUCER))) break;
+        announce(n, tile, announced);
+      }
+      uint32_t local_tile;
+      const GemmParams& p = ps.at(tile, at_problem, local_tile);
+      // (of the products' scales a lane each)
+      if ((uint32_t)lane < (SUMS ? p.nseg : 1u)) info_of(n)->alpha[lane] = __fmul_rn(p.alpha_a[p.slot_a[lane]], p.alpha_b[p.slot_b[lane]]);
+      __syncwarp();
+      if (lane == 0) mbar_arrive(scales_bar(n));
+      // Sums that start from what is there: towards L2, two tiles ahead (this warp is four ahead).
+      if (SUMS && n >= INFO_SLOTS / 2) fetch_rows(snake_tile(n - INFO_SLOTS / 2, first_tile, tile_step), fetched_to);
+      last = n;
+    }
+    for (uint32_t n = last < INFO_SLOTS / 2 ? 0 : last - INFO_SLOTS / 2 + 1; SUMS && ok && n <= last && first_tile < num_tiles; ++n)
+      fetch_rows(snake_tile(n, first_tile, tile_step), fetched_to);
+  } else if (SUMS && warp == STORE_WARP) {
+    // ---------------------------------------------------------------- stores of sums
+    // An SM writes 32 bytes a clock to L2 at most, by whichever unit: the 128 KB of a tile take 4130 clocks, and after a few
+    // stores the thread that issues them waits for that.  So that is this warp's and not the epilogue's, which goes on to the next
+    // tile: 11000 by 4096 gradients of 256 tokens, five products overwriting, 13000 -> 11500 clocks a tile.  Boxes of 16 KB: by
+    // boxes of 4 KB the warp's own 500 clocks for each would bound it.  It also loads what a tile is added to into the buffers,
+    // as they come free (by the epilogue's threads, a row each, that took as long as the stores).
+    uint32_t result_ph = 0;    // a bit per buffer, the same for both halves
+    bool ok = true, first = true;
+    const uint32_t all = tile_n / 64u;
+    struct Place {
+      uint32_t sum, epi, problem, row, col;
+      bool rows;  // not beyond M
+      uint32_t N;
+    };
+    auto place_of = [&](uint32_t n) {
+      const TileInfo& r = *info_of(n);
+      const uint32_t row = r.m0 + rank * BM;
+      return Place{r.minus_zero, r.epi, r.problem, row, r.n0, row < r.M, r.N};
+    };
+    auto result = [&](uint32_t h, uint32_t b) {
+      const bool got = await(result_bar(h, b), result_ph >> b & 1u, ERR_EPILOGUE);
+      if (h) result_ph ^= 1u << b;
+      return got;
+    };
+    auto buf_of = [&](uint32_t h, uint32_t b) { return epi_base + (h * BUFS + b) * (4 * EPI_BUF_BYTES); };
+    auto hand_on = [&](const Place& t, uint32_t h, uint32_t block) {  // block's buffer, for that block of tile t
+      const uint32_t b = block % BUFS, col = t.col + h * (tile_n / 2) + block * 32u;
+      if (t.sum && t.epi == 2 && t.rows && col < t.N) {
+        fence_async_smem();
+        mbar_expect_tx(ready_bar(h, b), 4 * EPI_BUF_BYTES);
+        tma_load_2d(buf_of(h, b), &ps.problem(t.problem).tmD, ready_bar(h, b), (int)col, (int)t.row);
+      } else {
+        mbar_arrive(ready_bar(h, b));
+      }
+    };
+    Place t{}, next{};
+    if (first_tile < num_tiles && (ok = await_tile(0, ERR_EPILOGUE))) next = place_of(0);
+    for (uint32_t n = 0, tile = first_tile; ok && tile < num_tiles; ++n) {
+      tile = snake_tile(n + 1, first_tile, tile_step);
+      t = next;
+      took_tile(n);
+      next.sum = 0;
+      if (tile < num_tiles) {
+        if (!(ok = await_tile(n + 1, ERR_EPILOGUE))) break;
+        next = place_of(n + 1);
+      }
+      if (!t.sum) continue;
+      for (uint32_t i = 0; ok && first && i < 2 * min(BUFS, all); ++i)
+        if ((ok = result(i & 1u, i / 2)) && lane == 0) hand_on(t, i & 1u, i / 2);
+      first = false;
+      for (uint32_t i = 0; ok && t.epi == 2 && i / 2 + BUFS < all; ++i)
+        if ((ok = result(i & 1u, i / 2 % BUFS)) && lane == 0) hand_on(t, i & 1u, i / 2 + BUFS);
+      auto stored = [&](uint32_t i) {  // the i-th block has been read out of its buffer
+        const uint32_t block = i / 2;
+        if (block + BUFS < all) mbar_arrive(ready_bar(i & 1u, block % BUFS));
+        else hand_on(next, i & 1u, block % BUFS);
+      };
+      for (uint32_t i = 0; i < 2 * all; ++i) {
+        const uint32_t h = i & 1u, block = i / 2;
+        if (!(ok = ok && result(h, block % BUFS))) break;
+        if (lane == 0) {
+          const uint32_t col = t.col + h * (tile_n / 2) + block * 32u;
+          if (t.rows && col < t.N) tma_store_2d(&ps.problem(t.problem).tmD, buf_of(h, block % BUFS), (int)col, (int)t.row);
+          else asm volatile("cp.async.bulk.commit_group;" ::: "memory");  // (a group for every block)
+          if (i) {
+            tma_store_wait_read<1>();
+            stored(i - 1);
+          }
+        }
+      }
+      if (ok && lane == 0) {
+        tma_store_wait_read<0>();
+        stored(2 * all - 1);
+      }
+    }
+    if (lane == 0) tma_store_wait_read<0>();
   } else if (!SUMS || warp >= EPI_WARP0) {
     // ---------------------------------------------------------------- epilogue
     if (SUMS) asm volatile("setmaxnreg.inc.sync.aligned.u32 224;");
     const uint32_t quad = (uint32_t)warp & 3u;          // tensor-memory lane quadrant this warp may read
     const uint32_t half = (uint32_t)(warp - EPI_WARP0) >> 2;   // which half of the tile's columns
     const int etid = (int)threadIdx.x - EPI_WARP0 * 32;
-    const uint32_t epi_smem = epi_base + (uint32_t)(warp - EPI_WARP0) * EPI_BUF_BYTES;  // this warp's two output tiles
+    // this warp's output tiles; sums: the first of its quarters of its half's buffers
+    const uint32_t epi_smem = epi_base + ((uint32_t)half * 4 * BUFS + (uint32_t)(warp - EPI_WARP0) % 4u) * EPI_BUF_BYTES;
     uint32_t n_groups = 0;  // bulk-store groups this warp has committed (buffer parity)
-    uint32_t acc = 0, acc_ph = 0, at_problem = 0;
+    const uint32_t ready = ready_bar(half, 0), result = result_bar(half, 0);
+    uint32_t ready_ph = 0;  // a bit per buffer
+    auto give_buf = [&](uint32_t b) {  // sums: to the storing warp
+      __syncwarp();
+      if (lane == 0) mbar_arrive(result + 8u * b);
+    };
+    auto await_buf = [&](uint32_t b) {  // ... and back
+      const bool got = await(ready + 8u * b, ready_ph >> b & 1u, ERR_EPILOGUE);
+      ready_ph ^= 1u << b;
+      return got;
+    };
+    uint32_t acc = 0, acc_ph = 0;
     bool ok = true;
     const uint32_t tempty_leader0 = PAIR ? map_to_cta(tempty_bar(0), 0) : tempty_bar(0);
     const uint32_t tempty_leader1 = PAIR ? map_to_cta(tempty_bar(1), 0) : tempty_bar(1);
-    for (uint32_t wave = 0, tile = first_tile; ok && tile < num_tiles; ++wave, tile = snake_tile(wave, first_tile, tile_step)) {
-      QE_TILE_PROBLEM();
-      (void)num_kb;
-      uint32_t m0, n0;
-      tile_coords<TILE_M>(local_tile, tiles_m, tiles_n, m_fastest, tile_n, m0, n0);
-      const uint32_t blk_row0 = m0 + rank * BM + quad * 32u;
-      const uint32_t col0 = n0 + half * (tile_n / 2);
-      // 32 x 32 blocks of this warp: none in rows beyond M, fewer in a ragged last column tile; warp-uniform
-      const uint32_t nch = blk_row0 >= p.M || col0 >= p.N ? 0u : min(tile_n / 64u, (p.N - col0) / 32u);
-      auto prefetch_next = [&] {  // the destination rows that this thread adds to in its next tile, towards L2
-        const uint32_t tile = snake_tile(wave + 1, first_tile, tile_step);
-        if (tile >= num_tiles) return;
-        uint32_t from = at_problem;
-        uint32_t& at_problem = from;
-        QE_TILE_PROBLEM();
-        (void)num_kb;
-        if (p.nseg == 1 || p.epi != 2) return;
-        uint32_t m0, n0;
-        tile_coords<TILE_M>(local_tile, tiles_m, tiles_n, m_fastest, tile_n, m0, n0);
-        const uint32_t row = m0 + rank * BM + quad * 32u + (uint32_t)lane, col = n0 + half * (tile_n / 2);
-        if (row >= p.M || col >= p.N) return;
-        const char* d = reinterpret_cast<const char*>(reinterpret_cast<const float*>(p.out) + (size_t)row * p.ldo + col);
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-          if (j * 32u < min(tile_n / 2, p.N - col)) asm volatile("prefetch.global.L2 [%0];" ::"l"(d + 128 * j));
-      };
-      if (SUMS && p.nseg > 1) {
-        // Several products for one FP32 tile (the weight gradients of several microbatches): the tile's running value
-        // stays in registers and every product is added to it in order, each with its own scale -- the additions
-        // launches of their own would have done in L2, at one read and one write of the destination instead of one
-        // per product.  What is added to is fetched while the first product is being computed.
-        float v[4][32];
-        float* const dst = reinterpret_cast<float*>(p.out) + (size_t)(blk_row0 + lane) * p.ldo + col0;
-        if (p.epi == 2) {
-#pragma unroll
-          for (int ch = 0; ch < 4; ++ch)
-            if ((uint32_t)ch < nch) ld_row32(dst + ch * 32, v[ch]);
-        }
-        prefetch_next();
-        // (lane i fetches the scales of product i: one chain of dependent loads per tile instead of one per product)
-        float my_alpha = 0.0f;
-        if ((uint32_t)lane < p.nseg) my_alpha = __fmul_rn(p.alpha_a[p.slot_a[lane]], p.alpha_b[p.slot_b[lane]]);
-        auto take = [&](uint32_t seg, auto first) {
-          const float alpha = __shfl_sync(0xffffffffu, my_alpha, (int)seg);
-          if (!(ok = mbar_wait_warp(tfull_bar(acc), acc_ph, abort_flag, status, ERR_EPILOGUE))) return;
-          tc_fence_after();
-          const uint32_t t_row = tmem_base + ((quad * 32u) << 16) + acc * ACC_COLS + half * (tile_n / 2);
-#pragma unroll
-          for (int ch = 0; ch < 4; ++ch) {
-            if ((uint32_t)ch >= nch) break;
-            uint32_t rc[32];
-            tmem_ld32(t_row + ch * 32u, rc);
-            tmem_ld_wait();
-#pragma unroll
-            for (int j = 0; j < 32; ++j) {
-              const float d = __fmul_rn(__uint_as_float(rc[j]), alpha);
-              v[ch][j] = decltype(first)::value ? d : __fadd_rn(v[ch][j], d);
-            }
-          }
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive_cluster(acc ? tempty_leader1 : tempty_leader0);
-          if (++acc == 2) { acc = 0; acc_ph ^= 1u; }
-        };
-        if (p.epi == 1) take(0, std::true_type{});
-        else take(0, std::false_type{});
-        for (uint32_t seg = 1; ok && seg < p.nseg; ++seg) take(seg, std::false_type{});
-        if (!ok) break;
-#pragma unroll
-        for (int ch = 0; ch < 4; ++ch) {
-          if ((uint32_t)ch >= nch) break;
-          if (lane == 0) tma_store_wait_read<0>();
-          __syncwarp();
-          st_tile_f32(epi_smem, (uint32_t)lane, v[ch]);
-          fence_async_smem();
-          __syncwarp();
-          if (lane == 0) tma_store_2d(&p.tmD, epi_smem, (int)(col0 + ch * 32u), (int)blk_row0);
-        }
-        continue;
+    // Of a tile: this warp's part of it.
+    struct Part {
+      uint32_t problem, epi, nseg, row, col, blocks;  // 32 x 32 blocks: none in rows beyond M, fewer in a ragged last column tile
+      float* dst;                                     // FP32 results: this thread's row
+      uint32_t* amax_bits;
+      float alpha;                                    // SUMS: lane i has the scale of product i
+      uint32_t minus_zero;
+    };
+    auto part_of = [&](const TileInfo& r) {
+      Part t;
+      t.problem = r.problem;
+      t.epi = r.epi;
+      t.nseg = SUMS ? r.nseg : 1u;
+      t.row = r.m0 + rank * BM + quad * 32u;
+      t.col = r.n0 + half * (tile_n / 2);
+      t.blocks = t.row >= r.M || t.col >= r.N ? 0u : min(tile_n / 64u, (r.N - t.col) / 32u);
+      t.dst = reinterpret_cast<float*>(r.out) + (size_t)(t.row + lane) * r.ldo + t.col;
+      t.amax_bits = reinterpret_cast<uint32_t*>(r.amax_bits);
+      return t;
+    };
+    auto take_part = [&](uint32_t n, Part& t) {  // of the CTA's n-th tile
+      if (ONE) {
+        uint32_t at_problem = 0;
+        TileInfo r;
+        const GemmParams& p = look_up(snake_tile(n, first_tile, tile_step), at_problem, r);
+        t = part_of(r);
+        t.alpha = __fmul_rn(p.alpha_a[p.slot_a[0]], p.alpha_b[p.slot_b[0]]);
+        return true;
       }
-      // (the variant that sums keeps no shared-memory addresses across its tiles: it needs the registers)
-      uint32_t ln = (uint32_t)lane;
-      if (SUMS) asm volatile("" : "+r"(ln));
-      const float alpha = __fmul_rn(p.alpha_a[p.slot_a[0]], p.alpha_b[p.slot_b[0]]);
-      if (p.epi == 2) {
-        // accumulate: pull this thread's destination row segment into L2, where the reduction will add to it, while
-        // the MMAs of the tile run
-        const char* d = reinterpret_cast<const char*>(reinterpret_cast<const float*>(p.out) + (size_t)(blk_row0 + lane) * p.ldo + col0);
+      if (!await(scales_bar(n), info_parity(n), ERR_EPILOGUE)) return false;
+      const TileInfo& r = *info_of(n);
+      t = part_of(r);
+      t.alpha = r.alpha[SUMS ? (uint32_t)lane % kMaxSegments : 0u];
+      t.minus_zero = r.minus_zero;
+      took_tile(n);
+      return true;
+    };
+    auto prefetch_rows = [&](const Part& t) {  // what this thread's row will be added to, towards L2
 #pragma unroll
-        for (int j = 0; j < 4; ++j)
-          if ((uint32_t)j < nch) asm volatile("prefetch.global.L2 [%0];" ::"l"(d + 128 * j));
-      }
+      for (uint32_t j = 0; j < 4; ++j)
+        if (j < t.blocks) asm volatile("prefetch.global.L2 [%0];" ::"l"(t.dst + 32 * j));
+    };
+    Part now;
+    ok = first_tile < num_tiles && take_part(0, now);
+    uint32_t n = 0, tile = first_tile;
+    for (; ok && tile < num_tiles && !(SUMS && now.minus_zero); ++n) {  // (sums come after all others)
+      tile = snake_tile(n + 1, first_tile, tile_step);
+      const Part t = now;
+      const uint32_t nch = t.blocks, blk_row0 = t.row, col0 = t.col;
+      const GemmParams& p = ps.problem(t.problem);
+      const uint32_t ln = (uint32_t)lane;
+      const float alpha = SUMS ? __shfl_sync(0xffffffffu, t.alpha, 0) : t.alpha;
+      // accumulate: pull this thread's destination row segment into L2, where the reduction will add to it, while the MMAs of
+      // the tile run
+      if (t.epi == 2) prefetch_rows(t);
       uint32_t r[2][32];
       if (!(ok = mbar_wait_warp(tfull_bar(acc), acc_ph, abort_flag, status, ERR_EPILOGUE))) break;
       tc_fence_after();
@@ -693,7 +929,7 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
         // Each lane (= row) writes its 32 columns into a swizzled shared-memory tile (conflict-free); one lane hands
         // the 32 x 32 tile to the bulk-store unit, which writes full rows to global memory (bf16, FP32 overwrite) or
         // adds them to the destination where it lives, in L2 (FP32 accumulate: one addition per element and launch).
-        if (p.epi == 0) {
+        if (t.epi == 0) {
           const uint32_t buf = epi_smem + (n_groups & 1u) * 2048u;  // two tiles: the previous store may still read
           if (lane == 0) {  // (a tile before this one may have used the buffer as a whole)
             if (ch == 0) tma_store_wait_read<0>();
@@ -716,7 +952,7 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
           fence_async_smem();
           __syncwarp();
           if (lane == 0) tma_store_2d(&p.tmD, buf, (int)col, (int)blk_row0);
-        } else if (p.epi == 3) {
+        } else if (ONE && t.epi == 3) {  // (chained linears go out one by one)
           // FP8 hand-off to the consuming linear: round to bf16 (the value that linear would have read), take its
           // magnitude for the amax, multiply by the consumer's scale in FP32 and convert -- the consumer's cast
           // kernel, applied to registers.  32 bytes per row; two 1 KB tiles per warp.
@@ -764,7 +1000,7 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
           fence_async_smem();
           __syncwarp();
           if (lane == 0) {
-            if (p.epi == 2) tma_reduce_add_2d(&p.tmD, buf, (int)col, (int)blk_row0);
+            if (t.epi == 2) tma_reduce_add_2d(&p.tmD, buf, (int)col, (int)blk_row0);
             else tma_store_2d(&p.tmD, buf, (int)col, (int)blk_row0);
           }
         }
@@ -777,15 +1013,80 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
         if (PAIR) mbar_arrive_cluster(acc ? tempty_leader1 : tempty_leader0);
         else mbar_arrive(acc ? tempty_leader1 : tempty_leader0);
       }
-      if ((p.epi == 0 || p.epi == 3) && (p.amax_bits || p.amax_bits2)) {
+      uint32_t* const also = ONE ? p.amax_bits2 : nullptr;  // (hand-off)
+      if ((t.epi == 0 || (ONE && t.epi == 3)) && (t.amax_bits || also)) {
         // two packed bf16 magnitudes -> FP32 bit pattern of the larger
         const uint32_t w = __reduce_max_sync(0xffffffffu, max(amax_bits & 0xffffu, amax_bits >> 16) << 16);
         if (lane == 0 && w) {
-          if (p.amax_bits) atomicMax(p.amax_bits, w);
-          if (p.amax_bits2) atomicMax(p.amax_bits2, w);
+          if (t.amax_bits) atomicMax(t.amax_bits, w);
+          if (also) atomicMax(also, w);
         }
       }
       if (++acc == 2) { acc = 0; acc_ph ^= 1u; }
+      if (tile < num_tiles && !(ok = take_part(n + 1, now))) break;
+    }
+    if constexpr (SUMS) {
+      // A tile's running value stays in registers and every product (the weight gradient of a microbatch) is added to it in
+      // order, each with its own scale -- the additions that launches of their own would have done in L2, at one read and one
+      // write of the destination instead of one per product.  (A loop of its own behind the other tiles': in one loop with them
+      // the values did not fit the registers, and the few bytes of them in local memory, for which shared memory leaves no L1,
+      // cost more than all that is saved here.)
+      f32x2 v[4][16];                    // this thread's row
+      const uint32_t all = tile_n / 64u;  // blocks of a tile that is not ragged: what buffers are handed on for
+      if (lane == 0) tma_store_wait_read<0>();
+      for (uint32_t b = 0; b < BUFS && b < all; ++b) give_buf(b);
+      for (; ok && tile < num_tiles; ++n) {
+          const uint32_t nch = now.blocks, nseg = now.nseg;
+          const bool adds = now.epi == 2;
+          const f32x2 minus_zero = pack2(now.minus_zero, now.minus_zero);
+          auto take = [&](uint32_t seg, auto first) {
+            const float alpha = __shfl_sync(0xffffffffu, now.alpha, (int)seg);
+            const f32x2 alpha2 = pack2(__float_as_uint(alpha), __float_as_uint(alpha));
+            if (!(ok = await(tfull_bar(acc), acc_ph, ERR_EPILOGUE))) return;
+            tc_fence_after();
+            const uint32_t t_row = tmem_base + ((quad * 32u) << 16) + acc * ACC_COLS + half * (tile_n / 2);
+#pragma unroll
+            for (int ch = 0; ch < 4; ++ch) {
+              if ((uint32_t)ch >= nch) break;
+              uint32_t r[32];
+              tmem_ld32(t_row + ch * 32u, r);
+              tmem_ld_wait();
+#pragma unroll
+              for (int j = 0; j < 16; ++j) {
+                const f32x2 d = mul2(pack2(r[2 * j], r[2 * j + 1]), alpha2, minus_zero);
+                v[ch][j] = decltype(first)::value ? d : add2(v[ch][j], d);
+              }
+            }
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive_cluster(acc ? tempty_leader1 : tempty_leader0);
+            if (++acc == 2) { acc = 0; acc_ph ^= 1u; }
+          };
+          if (!adds) {
+            take(0, std::true_type{});
+          } else {
+#pragma unroll
+            for (int ch = 0; ch < 4; ++ch) {
+              if ((uint32_t)ch >= all || !(ok = await_buf(ch % BUFS))) break;
+              if ((uint32_t)ch < nch) ld_tile_f32x2(epi_smem + (ch % BUFS) * (4 * EPI_BUF_BYTES), (uint32_t)lane, v[ch]);
+              if (ch + BUFS < all) give_buf(ch % BUFS);
+            }
+            if (ok) take(0, std::false_type{});
+          }
+          for (uint32_t seg = 1; ok && seg < nseg; ++seg) take(seg, std::false_type{});
+          if (!ok) break;
+#pragma unroll
+          for (int ch = 0; ch < 4; ++ch) {
+            if ((uint32_t)ch >= all) break;
+            if ((!adds || ch >= (int)BUFS) && !(ok = await_buf(ch % BUFS))) break;
+            if ((uint32_t)ch < nch) st_tile_f32x2(epi_smem + (ch % BUFS) * (4 * EPI_BUF_BYTES), (uint32_t)lane, v[ch]);
+            fence_async_smem();
+            give_buf(ch % BUFS);
+          }
+          if (!ok) break;
+          tile = snake_tile(n + 1, first_tile, tile_step);
+          if (tile < num_tiles && !(ok = take_part(n + 1, now))) break;
+      }
     }
     // Every epilogue thread of every CTA gets here (also after a timeout); the last CTA commits the scale state of
     // every problem that asks for it.  The commit needs the amax atomics only, so it runs while this CTA's last
@@ -824,15 +1125,13 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
   }
 }
 
-#undef QE_TILE_PROBLEM
-
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(threads_of(false), 1)
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(threads_of(false, false), 1)
     gemm_fp8_pair_kernel(const __grid_constant__ GemmLaunchParams<1> p) {
   gemm_body<true>(Problems<1, false>{p});
 }
 
 // One GEMM with an odd number of 128-row tiles, a CTA to a tile.
-__global__ void __launch_bounds__(threads_of(false), 1) gemm_fp8_kernel(const __grid_constant__ GemmLaunchParams<1> p) {
+__global__ void __launch_bounds__(threads_of(false, false), 1) gemm_fp8_kernel(const __grid_constant__ GemmLaunchParams<1> p) {
   gemm_body<false>(Problems<1, false>{p});
 }
 
@@ -852,9 +1151,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(SHARED_SM_THREADS, 1
 }
 
 // The same where problems have several products each.
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(threads_of(true), 1)
+template <uint32_t EPI_BUFS>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(threads_of(true, true), 1)
     gemm_fp8_pair_wide_kernel(const __grid_constant__ GemmLaunchParams<kMaxProblems> g) {
-  gemm_body<true>(Problems<kMaxProblems, true>{g});
+  gemm_body<true>(Problems<kMaxProblems, true, EPI_BUFS>{g});
 }
 
 constexpr uint32_t PAIR_M = Form<true>::TILE_M;
@@ -942,7 +1242,7 @@ Launch make_launch(const GemmDesc* probs, uint32_t n, int num_sms, const void* f
   if (NP == 1) std::memcpy(at + offsetof(P, before), &probs->before, sizeof(CommitParams));
   l.func = func;
   l.grid = dim3(ctas * (tiles < most ? tiles : most), 1, 1);
-  l.block = dim3(threads_of(sums), 1, 1);
+  l.block = dim3(threads_of(sums, NP > 1), 1, 1);
   l.smem = SMEM_BYTES;
   return l;
 }
@@ -953,16 +1253,20 @@ Launch make_launch(const GemmDesc* probs, uint32_t n, int num_sms, const void* f
 // small blocks for sums, which go out a few times a step: 5 KB and 32 within 1 % on steps of 2 to 64 linears.
 constexpr uint32_t kFew = 8;
 
+
 Launch make_any(const GemmDesc* probs, uint32_t n, int num_sms) {
-  bool sums = false;
-  for (uint32_t i = 0; i < n; ++i) sums |= probs[i].nseg > 1;
+  const bool sums = probs[n - 1].sum;  // (they are the last ones)
   if (n == 1 && !sums) {
     const bool alone = one_cta(*probs, num_sms);
     return make_launch<1>(probs, n, num_sms, alone ? (const void*)gemm_fp8_kernel : (const void*)gemm_fp8_pair_kernel, false, alone);
   }
   if (!sums && n <= kFew) return make_launch<kFew>(probs, n, num_sms, (const void*)gemm_fp8_pair_group_kernel<kFew>, false);
   if (!sums) return make_launch<kMaxProblems>(probs, n, num_sms, (const void*)gemm_fp8_pair_group_kernel<kMaxProblems>, false);
-  return make_launch<kMaxProblems>(probs, n, num_sms, (const void*)gemm_fp8_pair_wide_kernel, true);
+  uint32_t longest = 0;
+  for (uint32_t i = 0; i < n; ++i)
+    if (probs[i].sum && probs[i].Kc > longest) longest = probs[i].Kc;
+  return make_launch<kMaxProblems>(probs, n, num_sms, longest <= 256 ? (const void*)gemm_fp8_pair_wide_kernel<4>
+                                   : longest <= 768 ? (const void*)gemm_fp8_pair_wide_kernel<3> : (const void*)gemm_fp8_pair_wide_kernel<1>, true);
 }
 
 }  // namespace
@@ -971,7 +1275,8 @@ bool whole_row_tiles(uint32_t M) { return M % 256 == 0; }
 
 cudaError_t gemm_prepare() {
   for (const void* f : {(const void*)gemm_fp8_kernel, (const void*)gemm_fp8_pair_kernel, (const void*)gemm_fp8_pair_group_kernel<kFew>,
-                        (const void*)gemm_fp8_pair_group_kernel<kMaxProblems>, (const void*)gemm_fp8_pair_wide_kernel}) {
+                        (const void*)gemm_fp8_pair_group_kernel<kMaxProblems>, (const void*)gemm_fp8_pair_wide_kernel<1>,
+                        (const void*)gemm_fp8_pair_wide_kernel<3>, (const void*)gemm_fp8_pair_wide_kernel<4>}) {
     const cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES);
     if (e != cudaSuccess) return e;
   }

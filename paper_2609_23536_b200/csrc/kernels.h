@@ -118,7 +118,7 @@ constexpr uint32_t kMaxSegments = 8;
 struct GemmParams {
   CUtensorMap tmA;             // A: boxes of 128 rows x 128 contraction bytes x blocks_of(width), 128-byte swizzle
   CUtensorMap tmB;             // B: tile_n / 2 rows, likewise (MN-major: swizzled over tile_n / 2 bytes)
-  CUtensorMap tmD;             // D [M, N] (bf16, FP32 or FP8 bytes), box 32 x 32, for the epilogue's bulk stores
+  CUtensorMap tmD;             // D [M, N] (bf16, FP32 or FP8 bytes), box 32 x 32 (sum: 128 x 32), for the epilogue's bulk stores
   const float* alpha_a;        // [slot]
   const float* alpha_b;
   uint8_t slot_a[kMaxSegments], slot_b[kMaxSegments];  // of each product
@@ -128,7 +128,9 @@ struct GemmParams {
                                // nseg launches would have added them
   uint32_t idesc;              // tcgen05 instruction descriptor (formats, majors, shape)
   uint32_t b_desc_hi, b_step;  // B's shared-memory descriptor: high word; address advance (16-byte units) per 32 contraction elements
-  uint32_t a_mn, b_mn;         // operand given MN-major (as [Kc, M] / [Kc, N] bytes)
+  uint8_t a_mn, b_mn;          // operand given MN-major (as [Kc, M] / [Kc, N] bytes)
+  uint8_t sum, pad;            // FP32 result of one product or several that gemm_fp8_pair_wide_kernel keeps in registers: after all
+                               // other problems of the launch; tmD's box has 128 rows
   uint32_t ldo;
   void* out;                   // bf16 or FP32 [M, N], row pitch ldo elements
   uint32_t* amax_bits;         // or null

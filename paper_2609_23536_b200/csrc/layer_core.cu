@@ -70,13 +70,13 @@ int32_t make_b_maps(const DeviceInfo* d, CUtensorMap* maps, const Slots& t, uint
   return QE_OK;
 }
 
-// Tensor map over the output D [M, N] (row pitch ldo elements) for the epilogue's bulk stores: 32 x 32 boxes; bf16
-// rows of a box are 64 bytes (64-byte swizzle), FP32 rows 128 bytes (128-byte swizzle).
+// Tensor map over the output D [M, N] (row pitch ldo elements) for the epilogue's bulk stores: boxes of 32 columns and 32 rows
+// (FP32 sums of products: 128); bf16 rows of a box are 64 bytes (64-byte swizzle), FP32 rows 128 bytes (128-byte swizzle).
 int32_t make_out_map(const DeviceInfo* d, CUtensorMap* map, const void* ptr, uint64_t M, uint64_t N, uint64_t ldo,
-                     bool fp32) {
+                     bool fp32, uint32_t rows) {
   cuuint64_t gdim[2] = {N, M};
   cuuint64_t gstride[1] = {ldo * (fp32 ? 4u : 2u)};
-  cuuint32_t box[2] = {32u, 32u};
+  cuuint32_t box[2] = {32u, rows};
   cuuint32_t estr[2] = {1u, 1u};
   CUresult r = d->encode(map, fp32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2,
                          const_cast<void*>(ptr), gdim, gstride, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
@@ -550,8 +550,8 @@ void add_dI(qe_layer* L, uint32_t p, const void* dy, void* dx, std::vector<qe::L
 }
 
 // The weight-gradient GEMM of slot p; dst = first element of the layer's gradient slice, temp != null makes it
-// write the temporary instead (copied-gradient comparison path).
-qe::GemmDesc dW_gemm(qe_layer* L, uint32_t p, float* dst, int32_t accumulate, float* temp) {
+// write the temporary instead (copied-gradient comparison path); sum: products of other slots are going to be added.
+qe::GemmDesc dW_gemm(qe_layer* L, uint32_t p, float* dst, int32_t accumulate, float* temp, bool sum) {
   const uint32_t T = L->cfg.T, K = L->cfg.K, N = L->cfg.N;
   qe::GemmDesc gp;
   // (scales: the snapshots taken when dY_m and X_m were quantised, never the current state)
@@ -565,7 +565,8 @@ qe::GemmDesc dW_gemm(qe_layer* L, uint32_t p, float* dst, int32_t accumulate, fl
   gp.ldo = K;
   gp.amax_bits = nullptr;
   gp.status = &L->st->status;
-  make_out_map(L->ctx->dev, &gp.tmD, temp ? temp : dst, N, K, K, true);  // used by the overwrite epilogue
+  make_out_map(L->ctx->dev, &gp.tmD, temp ? temp : dst, N, K, K, true, sum ? 128 : 32);
+  gp.sum = sum;
   if (!temp) {
     gp.out = dst;  // direct placement: the epilogue reads, adds and writes the destination itself
     gp.epi = accumulate ? 2 : 1;

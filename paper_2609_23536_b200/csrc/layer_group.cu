@@ -329,9 +329,12 @@ int32_t together_build(qe_ctx* ctx, const Prepared* acts, uint32_t n, float* gra
     }
   }
   const uint32_t n_chain = (uint32_t)gemms.size();
+  // (a launch in which one adds products up computes all its weight gradients as sums)
+  const auto shares = [&](const Product& d) { return apart || qe::whole_row_tiles(d.first->layer->cfg.N); };
+  const bool sums = std::any_of(dw_of.begin(), dw_of.end(), [&](const Product& d) { return d.n > 1 && shares(d); });
   for (const Product& d : dw_of) {
     qe::GemmDesc& gp = place(d.first->layer->cfg.N);
-    gp = dW_gemm(d.first->layer, d.first->slot, grad + d.first->grad_offset, d.first->acc, nullptr);
+    gp = dW_gemm(d.first->layer, d.first->slot, grad + d.first->grad_offset, d.first->acc, nullptr, d.n > 1 || (sums && shares(d)));
     for (const Prepared* a = d.first + 1; gp.nseg < d.n; ++a)
       if (a->kind == QE_ACT_DW && a->layer == d.first->layer) gp.add_product(a->slot, a->slot);
   }

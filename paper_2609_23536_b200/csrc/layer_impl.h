@@ -47,7 +47,7 @@ int32_t make_a_map(const DeviceInfo* d, CUtensorMap* map, const Slots& t, uint64
 int32_t make_b_map(const DeviceInfo* d, CUtensorMap* map, const Slots& t, uint64_t N, uint64_t Kc, bool mn, uint32_t width);
 int32_t make_a_maps(const DeviceInfo* d, CUtensorMap* maps, const Slots& t, uint64_t M, uint64_t Kc, bool mn);
 int32_t make_b_maps(const DeviceInfo* d, CUtensorMap* maps, const Slots& t, uint64_t N, uint64_t Kc, bool mn);
-int32_t make_out_map(const DeviceInfo* d, CUtensorMap* map, const void* ptr, uint64_t M, uint64_t N, uint64_t ldo, bool fp32);
+int32_t make_out_map(const DeviceInfo* d, CUtensorMap* map, const void* ptr, uint64_t M, uint64_t N, uint64_t ldo, bool fp32, uint32_t rows = 32);
 int32_t make_out_map_u8(const DeviceInfo* d, CUtensorMap* map, const void* ptr, uint64_t M, uint64_t N, uint64_t ld);
 inline uint64_t align_up(uint64_t v, uint64_t a) { return (v + a - 1) / a * a; }
 inline bool shape_ok(uint32_t v) { return v >= 256 && v % 128 == 0 && v <= (1u << 20); }
@@ -172,7 +172,7 @@ void add_forward(qe_layer* L, uint32_t p, const void* x, void* y, std::vector<qe
                  uint32_t pn = 0, qe::GemmDesc* gemm_out = nullptr, qe::QuantParams* cast_out = nullptr);
 void add_dI(qe_layer* L, uint32_t p, const void* dy, void* dx, std::vector<qe::Launch>& ls, qe_layer* prev = nullptr,
             uint32_t pp = 0, qe::GemmDesc* gemm_out = nullptr, qe::QuantParams* cast_out = nullptr);
-qe::GemmDesc dW_gemm(qe_layer* L, uint32_t p, float* dst, int32_t accumulate, float* temp);
+qe::GemmDesc dW_gemm(qe_layer* L, uint32_t p, float* dst, int32_t accumulate, float* temp, bool sum = false);
 qe::GemmDesc dW_gemm_view(qe_layer* L, uint32_t p, void* view);
 void add_dW(qe_layer* L, uint32_t p, float* dst, int32_t accumulate, float* temp, std::vector<qe::Launch>& ls);
 

@@ -696,6 +696,25 @@ def _same_snapshot(a, b):
         assert state_equal({**u, "slots": []}, {**v, "slots": []}) and u["device_token"] == v["device_token"]
 
 
+@pytest.mark.parametrize("T", [256, 384, 768, 896])
+@pytest.mark.parametrize("shapes", [[(2176, 3200), (384, 640)], [(1152, 1152), (256, 256)], [(256, 384)]], ids=["wide", "middle", "narrow"])
+def test_sums_of_short_and_long_products_equal_single_actions_bitwise(qe, T, shapes):
+    """Products of 256, up to 768 and more tokens have four, three and one output buffers a warp and operand rings to match; tiles of
+    256, 128 and 64 columns, half-filled row tiles and ragged column tiles, sums that overwrite and that add, with F and dI
+    in the same launches."""
+    M = 7
+    s = sched(M, 2, 2)
+    got = []
+    for window in (1, 6):
+        ctx, layers, offs, X, Y, dY, dX, grad = _long_stage(qe, 1, window, M, s, shapes, T, "SB")
+        plan = qe.StepPlan(ctx, layers, _actions(s, len(shapes)), M, X, Y, dY, dX, grad, offs)
+        for _ in range(2):
+            plan.run()
+            qe.optimizer_boundary_all(layers, M)
+        got.append(_snapshot(layers, Y, dX, grad))
+    _same_snapshot(*got)
+
+
 @pytest.mark.parametrize("mode", [0, 1], ids=["eager", "graph"])
 def test_long_step_of_wide_launches_in_several_pieces_equals_single_actions_bitwise(qe, mode):
     """Sixteen linears and twelve microbatches: launches of all forwards and input gradients that are ready with sums of weight
