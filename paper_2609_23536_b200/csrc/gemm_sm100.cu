@@ -42,6 +42,7 @@
 #include <type_traits>
 #include <cuda_fp8.h>
 
+#include <algorithm>
 #include <cstddef>
 #include <cstring>
 
@@ -146,6 +147,35 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
 __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile uint32_t* abort_flag, uint32_t* status,
                                                uint32_t err_bit) {
   return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag, status, err_bit));
+}
+
+// Wait of a warp until `count` CTAs have said that they have stored their part of some rows (chained problems), bounded likewise.
+// What they stored is then there for bulk loads too.
+__device__ __forceinline__ bool rows_wait(const uint32_t* done, uint32_t count, volatile uint32_t* abort_flag, uint32_t* status) {
+  const long long t0 = clock64();
+  bool there = ld_acquire(done) >= count;
+  while (!there) {
+    there = ld_acquire(done) >= count;
+    if (there || *abort_flag) break;
+    if (clock64() - t0 > WAIT_BUDGET_CYCLES) {
+      *abort_flag = 1u;
+      atomicOr(status, ERR_PRODUCER);
+      break;
+    }
+  }
+  asm volatile("fence.proxy.async;" ::: "memory");
+  return __all_sync(0xffffffffu, there);
+}
+
+// ... and how they say it: the last warp of a CTA to get here, for all of them.  (An addition of each warp's own, behind a fence of
+// each lane, took 3500 clocks from a tile's last store until its rows were seen to be there; now 2000.)
+__device__ __forceinline__ bool last_of_cta(uint32_t* count /* shared */, uint32_t warps) {
+  uint32_t before;
+  asm volatile("atom.acq_rel.cta.shared::cta.add.u32 %0, [%1], 1;" : "=r"(before) : "r"(smem_u32(count)) : "memory");
+  return (before + 1) % warps == 0;
+}
+__device__ __forceinline__ void add_release(uint32_t* p, uint32_t v) {
+  asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
 // Arrival on a barrier that may live in the peer CTA.  What it announces are tensor-memory reads, ordered by the
@@ -376,8 +406,9 @@ __device__ __forceinline__ uint32_t snake_tile(uint32_t w, uint32_t first, uint3
 // ------------------------------------------------------------------------------------------------ problem lookup
 // A launch computes one GEMM, or (grouped launch) several independent ones whose tiles are numbered one after the
 // other, so that one set of persistent CTAs packs them into common waves and the launch overhead is paid once.
-template <int NP, bool SEVERAL, uint32_t EPI_BUFS = 1>
+template <int NP, bool SEVERAL, uint32_t EPI_BUFS = 1, bool CHAINED = false>
 struct Problems {
+  static constexpr bool CHAIN = CHAINED;                // each problem's A is the result of the one before
   static constexpr bool ONE = NP == 1, SUMS = SEVERAL;  // one problem; problems may have several products
   static constexpr uint32_t BUFS = EPI_BUFS;            // output buffers of an epilogue warp
   const GemmLaunchParams<NP>& g;
@@ -425,7 +456,7 @@ __device__ __forceinline__ uint32_t uniform(uint32_t v) { return __reduce_or_syn
 template <bool PAIR, class PS>
 __device__ __forceinline__ void gemm_body(const PS& ps) {
   constexpr uint32_t CTAS = Form<PAIR>::CTAS, TILE_M = Form<PAIR>::TILE_M;
-  constexpr bool SUMS = PS::SUMS, ONE = PS::ONE;
+  constexpr bool SUMS = PS::SUMS, ONE = PS::ONE, CHAIN = PS::CHAIN;
   constexpr int EPI_WARP0 = SUMS ? 4 : 2;    // first epilogue warp
   constexpr int INFO_WARP = SUMS ? 2 : 10;  // (launches of several problems)
   constexpr int STORE_WARP = 3;             // (sums)
@@ -456,6 +487,7 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
   auto info_parity = [](uint32_t n) { return n / INFO_SLOTS & 1u; };
   volatile uint32_t* abort_flag = tmem_slot + 1;
   uint32_t* last_flag = tmem_slot + 2;
+  uint32_t* stored_count = tmem_slot + 3;  // chained problems: epilogue warps that have stored their part of a tile
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = PAIR ? cluster_ctarank() : 0u;  // position in the CTA pair; rank 0 issues the MMAs
@@ -463,12 +495,14 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
   const Ring<PAIR, BUFS> ring(ps.first().tile_n);  // (one tile width per launch)
   const uint32_t first_tile = blockIdx.x / CTAS, tile_step = gridDim.x / CTAS;
   uint32_t* const status = ps.first().status;
+  // the n-th tile of this cluster.  (Chained problems: in order, so that what a tile waits for is on its way before it.)
+  auto tile_of = [&](uint32_t n) { return CHAIN ? first_tile + n * tile_step : snake_tile(n, first_tile, tile_step); };
   const uint32_t tile_n = ps.first().tile_n;  // (of the whole launch)
   // which problem a tile belongs to and where it lies in it; `at_problem` as in Problems::at
   auto look_up = [&](uint32_t tile, uint32_t& at_problem, TileInfo& t) -> const GemmParams& {
     uint32_t local_tile;
     const GemmParams& p = ps.at(tile, at_problem, local_tile);
-    tile_coords<TILE_M>(local_tile, (p.M + TILE_M - 1) / TILE_M, (p.N + tile_n - 1) / tile_n, p.M <= p.N, tile_n, t.m0, t.n0);
+    tile_coords<TILE_M>(local_tile, (p.M + TILE_M - 1) / TILE_M, (p.N + tile_n - 1) / tile_n, !CHAIN && p.M <= p.N, tile_n, t.m0, t.n0);
     t.problem = at_problem;
     t.num_kb = p.Kc / BK;
     t.nseg = SUMS ? p.nseg : 1u;
@@ -541,6 +575,7 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
       mbar_init(taken_bar(i), EPI_WARPS + 1 + (SUMS ? 1u : 0u) + (rank == 0 ? 1u : 0u));  // epilogue, producer, storing warp, MMA issuer
     }
     *abort_flag = 0u;
+    *stored_count = 0u;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
@@ -577,7 +612,7 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
     }
     // (and the first records)
     if (!ONE)
-      for (uint32_t n = 0, tile = first_tile, from = 0; n < INFO_SLOTS && tile < num_tiles; ++n, tile = snake_tile(n, first_tile, tile_step))
+      for (uint32_t n = 0, tile = first_tile, from = 0; n < INFO_SLOTS && tile < num_tiles; ++n, tile = tile_of(n))
         announce(n, tile, from);
   }
   // Everything above (barriers, tensor memory) touched no data a predecessor produces and may overlap the previous
@@ -585,11 +620,11 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
   grid_dep_wait();
   const bool hold = blockIdx.x < ps.count() && ps.commits_op() == 1u;
   if (!hold) grid_dep_launch();
-  if (blockIdx.x == 0 && threadIdx.x == EPI_WARP0 * 32) {  // FP8 hand-off: the consumer's tape snapshot of its inverse scale
-    const GemmParams& q = ps.first();
+  if (blockIdx.x == 0 && warp == EPI_WARP0 && (uint32_t)lane < (CHAIN ? ps.count() : 1u)) {  // FP8 hand-off: the consumer's tape snapshot of its inverse scale
+    const GemmParams& q = ps.problem((uint32_t)lane);
     if (q.epi == 3 && q.sinv_dst) *q.sinv_dst = *q.sinv_src;
   }
-  if (warp == EPI_WARP0 + 7 && blockIdx.x < ps.count()) {  // (a launch with early commits has a CTA per problem at least: most_committing)
+  if (!CHAIN && warp == EPI_WARP0 + 7 && blockIdx.x < ps.count()) {  // (a launch with early commits has a CTA per problem at least: most_committing)
     // The classes whose amax an EARLIER kernel reduced (the cast that made this GEMM's A operand) are committed here,
     // by an epilogue warp that has nothing to drain yet: nothing this launch computes reads their scale (its alphas
     // are snapshots), so only the output's class is left for the launch's tail.
@@ -623,7 +658,7 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
     const bool elected = elect_one();
     uint32_t s = 0, ph = 0;
     bool ok = true;
-    for (uint32_t n = 0, tile = first_tile; ok && tile < num_tiles; ++n, tile = snake_tile(n, first_tile, tile_step)) {
+    for (uint32_t n = 0, tile = first_tile; ok && tile < num_tiles; ++n, tile = tile_of(n)) {
       TileInfo t;
       unsigned long long slots_a = 0, slots_b = 0;  // a byte per product
       if (ONE) {
@@ -653,7 +688,26 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
       for (uint32_t seg = 0; ok && seg < t.nseg; ++seg, slots_a >>= 8, slots_b >>= 8) {
         const CUtensorMap *tmA = &p.tmA, *tmB = &p.tmB;
         const int sa = SUMS ? (int)uniform((uint32_t)slots_a & 255u) : (int)slots_a, sb = SUMS ? (int)uniform((uint32_t)slots_b & 255u) : (int)slots_b;
-        for (uint32_t kb = 0; kb < t.num_kb; kb += ring.blocks) {
+        uint32_t kb = 0;
+        if (CHAIN && t.problem) {
+          // A is being made by other CTAs: B first, as far as the ring goes, then A when its rows are there.
+          const uint32_t s0 = s;
+          for (uint32_t j = 0; ok && j < ring.stages && kb < t.num_kb; ++j, kb += ring.blocks) {
+            if (!(ok = await(empty_bar(s), ph ^ 1u, ERR_PRODUCER))) break;
+            if (elected) {
+              if (rank == 0) mbar_expect_tx(full_bar(s), bytes);
+              tma_load<PAIR>(smem_base + s * ring.stage_bytes + ring.b_offset(), tmB, PAIR ? map_to_cta(full_bar(s), 0) : full_bar(s), b0, b1, (int)kb, sb);
+            }
+            if (++s == ring.stages) { s = 0; ph ^= 1u; }
+          }
+          const GemmParams& q = ps.problem(t.problem - 1);
+          if (!(ok = ok && rows_wait(&q.commit.st->rows_done[t.m0 / TILE_M], (q.N + tile_n - 1) / tile_n * CTAS, abort_flag, status))) break;
+          for (uint32_t j = s0, at = 0; at < kb; at += ring.blocks) {
+            if (elected) tma_load<PAIR>(smem_base + j * ring.stage_bytes, tmA, PAIR ? map_to_cta(full_bar(j), 0) : full_bar(j), a0, a1, (int)at, sa);
+            if (++j == ring.stages) j = 0;
+          }
+        }
+        for (; kb < t.num_kb; kb += ring.blocks) {
           if (!(ok = mbar_wait_warp(empty_bar(s), ph ^ 1u, abort_flag, status, ERR_PRODUCER))) break;
           const uint32_t a_dst = smem_base + s * ring.stage_bytes, b_dst = a_dst + ring.b_offset();
           if (elected) {
@@ -679,7 +733,7 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
       const bool elected = elect_one();
       uint32_t s = 0, ph = 0, acc = 0, acc_ph = 0;
       bool ok = true;
-      for (uint32_t n = 0, tile = first_tile; ok && tile < num_tiles; ++n, tile = snake_tile(n, first_tile, tile_step)) {
+      for (uint32_t n = 0, tile = first_tile; ok && tile < num_tiles; ++n, tile = tile_of(n)) {
         TileInfo t;
         if (ONE) {
           uint32_t at_problem = 0;
@@ -738,7 +792,7 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
       for (uint32_t i = (uint32_t)lane; i < rows * lines; i += 32)
         asm volatile("prefetch.global.L2 [%0];" ::"l"(d + (size_t)(i / lines) * t.ldo * 4u + 128u * (i % lines)));
     };
-    for (uint32_t n = 0, tile = first_tile; ok && tile < num_tiles; ++n, tile = snake_tile(n, first_tile, tile_step)) {
+    for (uint32_t n = 0, tile = first_tile; ok && tile < num_tiles; ++n, tile = tile_of(n)) {
       if (n >= INFO_SLOTS) {
         if (!(ok = await(taken_bar(n), info_parity(n) ^ 1u, ERR_PRODUCER))) break;
         announce(n, tile, announced);
@@ -746,15 +800,22 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
       uint32_t local_tile;
       const GemmParams& p = ps.at(tile, at_problem, local_tile);
       // (of the products' scales a lane each)
-      if ((uint32_t)lane < (SUMS ? p.nseg : 1u)) info_of(n)->alpha[lane] = __fmul_rn(p.alpha_a[p.slot_a[lane]], p.alpha_b[p.slot_b[lane]]);
+      if (CHAIN) {  // (the tape's copy of A's scale is being made; its source stays as it is until the launch's last commits)
+        const bool later = at_problem > 0;
+        const GemmParams& q = ps.problem(later ? at_problem - 1 : 0u);
+        if (lane == 0) info_of(n)->alpha[0] = __fmul_rn(later ? *q.sinv_src : p.alpha_a[p.slot_a[0]], p.alpha_b[p.slot_b[0]]);
+        if (lane == 1 && p.epi == 3) info_of(n)->alpha[1] = *p.out_scale;
+      } else if ((uint32_t)lane < (SUMS ? p.nseg : 1u)) {
+        info_of(n)->alpha[lane] = __fmul_rn(p.alpha_a[p.slot_a[lane]], p.alpha_b[p.slot_b[lane]]);
+      }
       __syncwarp();
       if (lane == 0) mbar_arrive(scales_bar(n));
       // Sums that start from what is there: towards L2, two tiles ahead (this warp is four ahead).
-      if (SUMS && n >= INFO_SLOTS / 2) fetch_rows(snake_tile(n - INFO_SLOTS / 2, first_tile, tile_step), fetched_to);
+      if (SUMS && n >= INFO_SLOTS / 2) fetch_rows(tile_of(n - INFO_SLOTS / 2), fetched_to);
       last = n;
     }
     for (uint32_t n = last < INFO_SLOTS / 2 ? 0 : last - INFO_SLOTS / 2 + 1; SUMS && ok && n <= last && first_tile < num_tiles; ++n)
-      fetch_rows(snake_tile(n, first_tile, tile_step), fetched_to);
+      fetch_rows(tile_of(n), fetched_to);
   } else if (SUMS && warp == STORE_WARP) {
     // ---------------------------------------------------------------- stores of sums
     // An SM writes 32 bytes a clock to L2 at most, by whichever unit: the 128 KB of a tile take 4130 clocks, and after a few
@@ -794,7 +855,7 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
     Place t{}, next{};
     if (first_tile < num_tiles && (ok = await_tile(0, ERR_EPILOGUE))) next = place_of(0);
     for (uint32_t n = 0, tile = first_tile; ok && tile < num_tiles; ++n) {
-      tile = snake_tile(n + 1, first_tile, tile_step);
+      tile = tile_of(n + 1);
       t = next;
       took_tile(n);
       next.sum = 0;
@@ -862,6 +923,10 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
       float* dst;                                     // FP32 results: this thread's row
       uint32_t* amax_bits;
       float alpha;                                    // SUMS: lane i has the scale of product i
+      float out_scale;                                // hand-off
+      uint8_t* dst8;                                  // chained problems: this thread's row, its format, the count of its rows
+      int32_t out_fmt;
+      uint32_t* done;
       uint32_t minus_zero;
     };
     auto part_of = [&](const TileInfo& r) {
@@ -880,9 +945,10 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
       if (ONE) {
         uint32_t at_problem = 0;
         TileInfo r;
-        const GemmParams& p = look_up(snake_tile(n, first_tile, tile_step), at_problem, r);
+        const GemmParams& p = look_up(tile_of(n), at_problem, r);
         t = part_of(r);
         t.alpha = __fmul_rn(p.alpha_a[p.slot_a[0]], p.alpha_b[p.slot_b[0]]);
+        if (t.epi == 3) t.out_scale = *p.out_scale;
         return true;
       }
       if (!await(scales_bar(n), info_parity(n), ERR_EPILOGUE)) return false;
@@ -890,6 +956,12 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
       t = part_of(r);
       t.alpha = r.alpha[SUMS ? (uint32_t)lane % kMaxSegments : 0u];
       t.minus_zero = r.minus_zero;
+      if (CHAIN) {
+        t.out_scale = r.alpha[1];
+        t.dst8 = reinterpret_cast<uint8_t*>(r.out) + (size_t)(t.row + lane) * r.ldo + t.col;
+        t.out_fmt = ps.problem(r.problem).out_fmt;
+        t.done = &ps.problem(r.problem).commit.st->rows_done[r.m0 / TILE_M];
+      }
       took_tile(n);
       return true;
     };
@@ -902,7 +974,7 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
     ok = first_tile < num_tiles && take_part(0, now);
     uint32_t n = 0, tile = first_tile;
     for (; ok && tile < num_tiles && !(SUMS && now.minus_zero); ++n) {  // (sums come after all others)
-      tile = snake_tile(n + 1, first_tile, tile_step);
+      tile = tile_of(n + 1);
       const Part t = now;
       const uint32_t nch = t.blocks, blk_row0 = t.row, col0 = t.col;
       const GemmParams& p = ps.problem(t.problem);
@@ -952,14 +1024,17 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
           fence_async_smem();
           __syncwarp();
           if (lane == 0) tma_store_2d(&p.tmD, buf, (int)col, (int)blk_row0);
-        } else if (ONE && t.epi == 3) {  // (chained linears go out one by one)
+        } else if ((ONE || CHAIN) && t.epi == 3) {
           // FP8 hand-off to the consuming linear: round to bf16 (the value that linear would have read), take its
           // magnitude for the amax, multiply by the consumer's scale in FP32 and convert -- the consumer's cast
           // kernel, applied to registers.  32 bytes per row; two 1 KB tiles per warp.
           const uint32_t buf = epi_smem + (n_groups & 1u) * 1024u;
-          if (lane == 0) tma_store_wait_read<1>();
-          __syncwarp();
-          const float qs = *p.out_scale;
+          if (!CHAIN) {
+            if (lane == 0) tma_store_wait_read<1>();
+            __syncwarp();
+          }
+          const float qs = t.out_scale;
+          const int32_t out_fmt = CHAIN ? t.out_fmt : p.out_fmt;
           uint32_t q[8];
 #pragma unroll
           for (int j = 0; j < 8; ++j) {
@@ -971,12 +1046,17 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
             }
             const float2 f01 = make_float2(__fmul_rn(__uint_as_float(w[0] << 16), qs), __fmul_rn(__uint_as_float(w[0] & 0xffff0000u), qs));
             const float2 f23 = make_float2(__fmul_rn(__uint_as_float(w[1] << 16), qs), __fmul_rn(__uint_as_float(w[1] & 0xffff0000u), qs));
-            const uint32_t lo = p.out_fmt == 0 ? __nv_cvt_float2_to_fp8x2(f01, __NV_SATFINITE, __NV_E4M3)
+            const uint32_t lo = out_fmt == 0 ? __nv_cvt_float2_to_fp8x2(f01, __NV_SATFINITE, __NV_E4M3)
                                                : __nv_cvt_float2_to_fp8x2(f01, __NV_SATFINITE, __NV_E5M2);
-            const uint32_t hi = p.out_fmt == 0 ? __nv_cvt_float2_to_fp8x2(f23, __NV_SATFINITE, __NV_E4M3)
+            const uint32_t hi = out_fmt == 0 ? __nv_cvt_float2_to_fp8x2(f23, __NV_SATFINITE, __NV_E4M3)
                                                : __nv_cvt_float2_to_fp8x2(f23, __NV_SATFINITE, __NV_E5M2);
             q[j] = lo | (hi << 16);
           }
+          if (CHAIN) {  // (whole sectors by plain stores: they are there a bulk store's 500 clocks sooner)
+            asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(t.dst8 + ch * 32),
+                         "r"(q[0]), "r"(q[1]), "r"(q[2]), "r"(q[3]), "r"(q[4]), "r"(q[5]), "r"(q[6]), "r"(q[7])
+                         : "memory");
+          } else {
 #pragma unroll
           for (int c = 0; c < 2; ++c) {
             const uint32_t dst = buf + ln * 32u + ((uint32_t)c << 4);
@@ -987,6 +1067,7 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
           fence_async_smem();
           __syncwarp();
           if (lane == 0) tma_store_2d(&p.tmD, buf, (int)col, (int)blk_row0);
+          }
         } else {
           // one tile: waiting for the previous block's store to have read it paces the FP32 traffic, which measured
           // faster than two tiles in flight per warp
@@ -1013,8 +1094,12 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
         if (PAIR) mbar_arrive_cluster(acc ? tempty_leader1 : tempty_leader0);
         else mbar_arrive(acc ? tempty_leader1 : tempty_leader0);
       }
-      uint32_t* const also = ONE ? p.amax_bits2 : nullptr;  // (hand-off)
-      if ((t.epi == 0 || (ONE && t.epi == 3)) && (t.amax_bits || also)) {
+      if (CHAIN && t.epi == 3) {  // the next problem's loads of these rows wait for this
+        __syncwarp();
+        if (lane == 0 && last_of_cta(stored_count, EPI_WARPS)) add_release(t.done, 1u);
+      }
+      uint32_t* const also = ONE || CHAIN ? p.amax_bits2 : nullptr;  // (hand-off)
+      if ((t.epi == 0 || ((ONE || CHAIN) && t.epi == 3)) && (t.amax_bits || also)) {
         // two packed bf16 magnitudes -> FP32 bit pattern of the larger
         const uint32_t w = __reduce_max_sync(0xffffffffu, max(amax_bits & 0xffffu, amax_bits >> 16) << 16);
         if (lane == 0 && w) {
@@ -1084,7 +1169,7 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
             give_buf(ch % BUFS);
           }
           if (!ok) break;
-          tile = snake_tile(n + 1, first_tile, tile_step);
+          tile = tile_of(n + 1);
           if (tile < num_tiles && !(ok = take_part(n + 1, now))) break;
       }
     }
@@ -1100,6 +1185,10 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
         static_assert(kMaxProblems <= EPI_WARPS * 32, "a lane for every problem");
         const uint32_t i = ew + EPI_WARPS * (uint32_t)lane;
         const CommitParams& c = ps.commit(i < ps.count() ? i : 0u);
+        if (CHAIN) {  // all classes of all problems; and nobody waits for rows any more
+          commit_class<true>(c, c.early_mask, true, i < ps.count(), lane);
+          for (uint32_t r = 0; i < ps.count() && r < (ps.problem(i).M + TILE_M - 1) / TILE_M; ++r) c.st->rows_done[r] = 0u;
+        }
         commit_class<true>(c, c.class_mask, false, i < ps.count() && c.st && c.class_mask, lane);
       }
     }
@@ -1150,6 +1239,17 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(SHARED_SM_THREADS, 1
   gemm_body<true>(Problems<NP, false>{g});
 }
 
+// Chained problems: each one's A is the result of the one before, handed on in FP8, in one launch.  Its CTAs wait on one another
+// (a cooperative launch): a tile's loads of A for its rows of the problem before, which are counted as they are stored; those
+// of B do not wait, up to a ring-full, and a tile waits behind earlier ones only.  The scales are committed when all is done.  Of the
+// 7300 clocks from one 512 x 1024 x 1024 to the next (tiles of 64 columns, half of the CTAs) the loads of A take 2400, the MMAs
+// behind them 700, the epilogue 700, and 3500 pass between the last store and the loads that wait for it: the fence, the
+// count, the poll (16 layers: 66 us a launch, 88 as launches of their own).
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(threads_of(false, true), 1)
+    gemm_fp8_pair_chain_kernel(const __grid_constant__ GemmLaunchParams<kMaxChained> g) {
+  gemm_body<true>(Problems<kMaxChained, false, 1, true>{g});
+}
+
 // The same where problems have several products each.
 template <uint32_t EPI_BUFS>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(threads_of(true, true), 1)
@@ -1191,12 +1291,15 @@ uint32_t choose_width(const GemmDesc* d, uint32_t n, uint32_t pairs) {
 // which the loads of a long contraction eat up (1920 x 2176, cast included: 23.7 for 25.3 at 4096, 31.6 for 32.3 at 6528,
 // 39.2 for 38.8 at 8192); at 128 rows the pair's empty half still shares the loads of B (128 x 16384 x 4096, FP32: 17.6
 // for 16.9).  Even row counts have no empty half.
+bool saves_a_wave(const GemmDesc& d, int num_sms) {
+  const uint32_t waves_pairs = ceil_div(tiles_of(d, 256), (uint32_t)num_sms / 2u);
+  const uint32_t waves_ctas = ceil_div((d.M / BM) * ceil_div(d.N, 256), (uint32_t)num_sms);
+  return 6 * waves_ctas < 5 * waves_pairs;
+}
 bool one_cta(const GemmDesc& d, int num_sms) {
   const uint32_t pairs = (uint32_t)num_sms / 2u;
   if (d.M % PAIR_M == 0 || choose_width(&d, 1, pairs) != 0) return false;
-  const uint32_t waves_pairs = ceil_div(tiles_of(d, 256), pairs);
-  const uint32_t waves_ctas = ceil_div((d.M / BM) * ceil_div(d.N, 256), (uint32_t)num_sms);
-  return 6 * waves_ctas < 5 * waves_pairs || (waves_pairs == 1 && d.M > BM && d.Kc <= 6144);
+  return saves_a_wave(d, num_sms) || (tiles_of(d, 256) <= pairs && d.M > BM && d.Kc <= 6144);
 }
 
 // The device's parameter block of one problem at a tile width.
@@ -1217,6 +1320,20 @@ GemmParams problem_of(const GemmDesc& d, uint32_t w, uint32_t tile_m) {
   return p;
 }
 
+// Whether chained problems go out as one launch.  What that saves is a launch's start and end between two of them, about
+// 1.3 us of 5.5 for 512 x 1024 x 1024, and a layer's last wave, which the next one's tiles fill; what it costs is a launch whose
+// blocks all have to be there at once, which starts some us later: us a step of eight microbatches of 512 tokens, one by one / in
+// one launch, two linears of 1024 x 1024 381 / 418, three 485 / 502, sixteen 1713 / 1499; 256 x 256 at 256 tokens, twelve 1252 /
+// 1035; four microbatches of 2048 tokens, eight of 2048 x 2048 1199 / 1072; 4096 tokens, four of 2048 x 2048 912 / 846, 4096 x 4096 1387 /
+// 1349; 256 tokens, six of 4096 x 4096 1254 / 1226.  Half-filled row tiles are not avoided there: where that saved a wave
+// (one_cta) the launches stay (1152 tokens, four of 4096 x 4096 1112 / 1136; 1920 tokens, six of 2304 x 2304, one wave, 1007 / 950).
+bool launch_chained(const GemmDesc* d, uint32_t n, int num_sms) {
+  if (n < kLaunchChained || n > kMaxChained || d->M > PAIR_M * (sizeof(DevState::rows_done) / sizeof(uint32_t))) return false;
+  for (uint32_t i = 0; i < n; ++i)
+    if (d[i].M % PAIR_M && saves_a_wave(d[i], num_sms)) return false;
+  return true;
+}
+
 template <int NP>
 Launch make_launch(const GemmDesc* probs, uint32_t n, int num_sms, const void* func, bool sums, bool alone = false) {
   using P = GemmLaunchParams<NP>;
@@ -1227,11 +1344,12 @@ Launch make_launch(const GemmDesc* probs, uint32_t n, int num_sms, const void* f
   l.params.resize(offsetof(P, prob) + n * sizeof(GemmParams));  // (no unused problems)
   unsigned char* at = l.params.data();
   const uint32_t tile_m = alone ? BM : PAIR_M, ctas = alone ? 1u : 2u, most = (uint32_t)num_sms / ctas;
-  const uint32_t w = choose_width(probs, n, (uint32_t)num_sms / 2u);  // (alone: 0, see one_cta)
+  uint32_t w = probs->chained ? kNumTileWidths - 1 : choose_width(probs, n, (uint32_t)num_sms / 2u);  // (alone: 0, see one_cta)
+  for (uint32_t i = 0; probs->chained && i < n; ++i) w = std::min(w, choose_width(probs + i, 1, (uint32_t)num_sms / 2u));
   uint32_t tiles = 0;
   uint32_t* ticket = nullptr;
   for (uint32_t i = 0; i < n; ++i) {
-    if (!ticket && probs[i].commit.st && probs[i].commit.class_mask) ticket = &probs[i].commit.st->ticket;
+    if (!ticket && probs[i].commit.st && (probs[i].commit.class_mask || probs[i].chained)) ticket = &probs[i].commit.st->ticket;
     tiles += ceil_div(probs[i].M, tile_m) * ceil_div(probs[i].N, kTileWidths[w]);
     std::memcpy(at + offsetof(P, tile_end) + i * sizeof(uint32_t), &tiles, sizeof(tiles));
     const GemmParams p = problem_of(probs[i], w, tile_m);
@@ -1274,7 +1392,7 @@ Launch make_any(const GemmDesc* probs, uint32_t n, int num_sms) {
 bool whole_row_tiles(uint32_t M) { return M % 256 == 0; }
 
 cudaError_t gemm_prepare() {
-  for (const void* f : {(const void*)gemm_fp8_kernel, (const void*)gemm_fp8_pair_kernel, (const void*)gemm_fp8_pair_group_kernel<kFew>,
+  for (const void* f : {(const void*)gemm_fp8_pair_chain_kernel, (const void*)gemm_fp8_kernel, (const void*)gemm_fp8_pair_kernel, (const void*)gemm_fp8_pair_group_kernel<kFew>,
                         (const void*)gemm_fp8_pair_group_kernel<kMaxProblems>, (const void*)gemm_fp8_pair_wide_kernel<1>,
                         (const void*)gemm_fp8_pair_wide_kernel<3>, (const void*)gemm_fp8_pair_wide_kernel<4>}) {
     const cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES);
@@ -1284,6 +1402,12 @@ cudaError_t gemm_prepare() {
 }
 
 bool make_gemm_group(const GemmDesc* probs, uint32_t n, int num_sms, Launch* out) {
+  if (n && probs->chained) {
+    if (!launch_chained(probs, n, num_sms)) return false;
+    *out = make_launch<kMaxChained>(probs, n, num_sms, (const void*)gemm_fp8_pair_chain_kernel, false);
+    out->cooperative = true;
+    return true;
+  }
   if (n < 2 || n > kMaxProblems) return false;
   for (uint32_t i = 0; i < n && n > most_committing(num_sms); ++i)
     if (probs[i].commit.st && probs[i].commit.early_mask) return false;

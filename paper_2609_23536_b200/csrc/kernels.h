@@ -28,7 +28,8 @@ struct DevState {
   uint32_t wmax[4];            // bit pattern of max(history ring) per class, kept by the commit (derived state)
   uint32_t status_all;         // scratch of the multi-layer boundary: OR of several layers' status words
   uint32_t commits;            // whole-step calls whose first layer this is: Announce::word
-  uint32_t pad[37];            // header is 768 bytes; history rings [4][H] follow
+  uint32_t rows_done[32];      // launches of chained GEMMs: parts of 256 rows of this layer's result that are stored; 0 between them
+  uint32_t pad[5];             // header is 768 bytes; history rings [4][H] follow
 };
 static_assert(sizeof(DevState) == 768, "DevState layout");
 
@@ -154,6 +155,7 @@ struct GemmDesc : GemmParams {
   const CUtensorMap* mapA;     // [2]: a_map_of(width); the launch reads those of the width it chooses (gemm_width)
   const CUtensorMap* mapB;     // [kNumTileWidths]
   CommitParams before{};       // of a launch of its own: GemmLaunchParams::before
+  bool chained = false;        // make_gemm_group: each problem's A is the result of the one before (FP8 hand-off)
   GemmDesc() : GemmParams{}, a_fmt(0), b_fmt(0), mapA(nullptr), mapB(nullptr) { nseg = 1; }
   void operands(const CUtensorMap* a, const float* alphas_a, uint32_t slot_of_a, const CUtensorMap* b, const float* alphas_b, uint32_t slot_of_b) {
     mapA = a, mapB = b, alpha_a = alphas_a, alpha_b = alphas_b;
@@ -176,6 +178,7 @@ struct GemmLaunchParams {
   CommitParams before;         // launches of one problem: a class whose amax the launch before completed (before.st != null)
   GemmParams prob[NP];
 };
+constexpr uint32_t kLaunchChained = 4, kMaxChained = 16;  // problems of a launch of chained GEMMs, at least and at most
 constexpr uint32_t kMaxProblems = 56;  // of a launch: what a kernel's parameter space of 32764 bytes holds
 // ... and of one whose problems commit scales at its start, a CTA each: the grid has that many at least
 inline uint32_t most_committing(int num_sms) {
@@ -234,6 +237,7 @@ struct Launch {
   const void* func = nullptr;
   dim3 grid{1, 1, 1}, block{1, 1, 1};
   uint32_t smem = 0;
+  bool cooperative = false;  // its blocks wait on one another
   ParamBytes params;    // the parameter block, without an unused tail ...
   uint32_t nbytes = 0;  // ... of a block of this size
   template <class P>
@@ -260,7 +264,8 @@ Launch make_amax_pass2(const AmaxParams& p);
 Launch make_accumulate(const AccumParams& p);
 Launch make_arena_reduce(const ArenaReduceParams& p);
 Launch make_gemm(const GemmDesc& p, int num_sms);
-// One launch for n = 2..kMaxProblems GEMMs (each may carry its own commit tail); false if there are more.
+// One launch for n = 2..kMaxProblems GEMMs (each may carry its own commit tail); false if there are more, or if they are chained and
+// better launched one by one.
 // (most_committing, where they commit scales at the launch's start)
 bool make_gemm_group(const GemmDesc* probs, uint32_t n, int num_sms, Launch* out);
 uint32_t announce_commits(Launch* gemm, uint32_t* word);  // the launch is to count its problems in *word; how many that are

@@ -158,11 +158,13 @@ cudaError_t launch_pdl(const qe::Launch& l, cudaStream_t stream) {
   cfg.blockDim = l.block;
   cfg.dynamicSmemBytes = l.smem;
   cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeCooperative;
+  attr[1].val.cooperative = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = l.cooperative ? 2 : 1;
   qe::Launch::Block tmp;
   void* args[1] = {l.args_block(&tmp)};
   return cudaLaunchKernelExC(&cfg, l.func, args);

@@ -4,6 +4,27 @@
 
 using namespace qe_impl;
 
+// The GEMMs of a chain in one launch where that is offered, else one by one, each as `alone` has it.
+template <class F>
+static void push_chain(qe_ctx* ctx, std::vector<qe::GemmDesc>& gemms, std::vector<qe::Launch>& ls, F alone) {
+  qe::Launch l;
+  if (gemms.size() > 1 && qe::make_gemm_group(gemms.data(), (uint32_t)gemms.size(), ctx->dev->num_sms, &l)) {
+    ls.push_back(std::move(l));
+    return;
+  }
+  for (uint32_t i = 0; i < gemms.size(); ++i) {
+    gemms[i].chained = false;
+    alone(i, gemms[i]);
+    ls.push_back(qe::make_gemm(gemms[i], ctx->dev->num_sms));
+  }
+}
+
+// Weights cast anew: `together` of them or more in one launch (sixteen of 1024 x 1024 28 us for 82), fewer one by one.
+static void push_refresh(const std::vector<qe::QuantParams>& casts, size_t together, std::vector<qe::Launch>& ls) {
+  if (casts.size() >= together) ls.push_back(qe::make_quantize_multi(casts.data(), (uint32_t)casts.size()));
+  else for (const qe::QuantParams& c : casts) ls.push_back(qe::make_quantize(c));
+}
+
 extern "C" {
 
 int32_t qe_backward_dW_multi(qe_layer* const* layers, const qe_tape* tapes, uint32_t n, float* grad, uint64_t elems,
@@ -103,6 +124,7 @@ int32_t qe_forward_chain(qe_layer* const* layers, uint32_t n, uint32_t mb, uint6
   Handshake handshake(ctx, caller);
   if ((st = handshake.in()) != QE_OK) return st;
   std::vector<qe::Launch> ls;
+  std::vector<qe::QuantParams> casts;  // of weights
   Fnv h;
   h.mix("Fchain", 7);
   for (uint32_t i = 0; i < n; ++i) {
@@ -111,22 +133,25 @@ int32_t qe_forward_chain(qe_layer* const* layers, uint32_t n, uint32_t mb, uint6
       QE_CUDA(cudaStreamWaitEvent(ctx->exec_stream, L->ev_dw[p[i]], 0));
       L->dw_pending[p[i]] = false;
     }
-    if (refresh[i]) add_refresh(L, ls);
+    if (refresh[i]) casts.push_back(refresh_params(L));
     h.mix(&layers[i], sizeof(qe_layer*));
     h.mix(&p[i], sizeof(uint32_t));
     h.mix(&refresh[i], sizeof(int32_t));
   }
+  std::vector<qe::GemmDesc> gemms(n);
+  push_refresh(casts, qe::kLaunchChained, ls);
   for (uint32_t i = 0; i < n; ++i) {
     const bool last = i + 1 == n;
-    qe::GemmDesc g;
-    add_forward(layers[i], p[i], i == 0 ? x : nullptr, last ? y : nullptr, ls, last ? nullptr : layers[i + 1], last ? 0 : p[i + 1], &g);
+    add_forward(layers[i], p[i], i == 0 ? x : nullptr, last ? y : nullptr, ls, last ? nullptr : layers[i + 1], last ? 0 : p[i + 1], &gemms[i]);
+    gemms[i].chained = n > 1;
+  }
+  push_chain(ctx, gemms, ls, [&](uint32_t i, qe::GemmDesc& g) {
     // A layer's Y is committed by the next layer's launch while that computes, the last layer's by its own tail: a tail with a
     // commit lengthens a launch by 2.8 us (ticket, dependent loads), of 8.4 for 512 x 1024 x 1024
     // (sixteen chained 1024 x 1024 linears 2016 -> 1721 us a step, twelve of 256 x 256 1395 -> 1194).
     if (i) g.before = commit_params(layers[i - 1], 1u << QE_CLASS_Y, 0, nullptr);
-    if (!last) g.commit.class_mask = 0;
-    ls.push_back(qe::make_gemm(g, ctx->dev->num_sms));
-  }
+    if (i + 1 < n) g.commit.class_mask = 0;
+  });
   if ((st = run_keyed(ctx, h.key, ls)) != QE_OK) return st;
   if ((st = handshake.out()) != QE_OK) return st;
   for (uint32_t i = 0; i < n; ++i)
@@ -149,13 +174,17 @@ int32_t qe_backward_dI_chain(qe_layer* const* layers, const qe_tape* tapes, uint
   std::vector<qe::Launch> ls;
   Fnv h;
   h.mix("Bchain", 7);
+  std::vector<qe::GemmDesc> gemms(n);
   for (uint32_t k = n; k-- > 0;) {  // last linear first
     const uint32_t pk = tapes[k].ref.slot;
+    qe::GemmDesc& g = gemms[n - 1 - k];
     add_dI(layers[k], pk, k + 1 == n ? dy : nullptr, k == 0 ? dx : nullptr, ls, k ? layers[k - 1] : nullptr,
-           k ? tapes[k - 1].ref.slot : 0);
+           k ? tapes[k - 1].ref.slot : 0, &g);
+    g.chained = n > 1;
     h.mix(&layers[k], sizeof(qe_layer*));
     h.mix(&pk, sizeof(uint32_t));
   }
+  push_chain(ctx, gemms, ls, [](uint32_t, qe::GemmDesc&) {});
   if ((st = run_keyed(ctx, h.key, ls)) != QE_OK) return st;
   if (ctx->dw_stream)
     for (uint32_t i = 0; i < n; ++i) QE_CUDA(cudaEventRecord(layers[i]->ev_di[tapes[i].ref.slot], ctx->exec_stream));

@@ -125,6 +125,30 @@ def test_chain_of_odd_token_counts_equals_layer_by_layer_bitwise(qe, tokens, mon
         assert all(state_equal(x, y) and x["device_token"] == y["device_token"] and x["device_status"] == 0 for x, y in zip(u, v))
 
 
+@pytest.mark.parametrize("mode", [0, 1], ids=["eager", "graph"])
+@pytest.mark.parametrize("tokens,shapes", [(256, [(256, 256)] * 16), (1280, [(512, 1280), (1280, 2048), (2048, 512), (512, 256), (256, 768)]),
+                                           (8192, [(256, 256)] * 4), (8448, [(256, 256)] * 4)])
+def test_chains_in_one_launch_equal_layer_by_layer_bitwise(qe, mode, tokens, shapes, monkeypatch):
+    """Four linears to sixteen in one launch, whose tiles wait for the rows they read: one tile to a linear, several waves of tiles,
+    contractions longer and shorter than the operand ring, the most rows it is offered for and one row tile more."""
+    monkeypatch.setattr(sys.modules[__name__], "T", tokens)
+    monkeypatch.setattr(sys.modules[__name__], "CHAIN", shapes)
+    a = _run(qe, mode, chained=False)
+    b = _run(qe, mode, chained=True)
+    for key in ("Y", "dX", "mg"):
+        for u, v in zip(a[key], b[key]):
+            assert np.array_equal(u.view(np.uint8), v.view(np.uint8)), key
+    for key in ("Xq", "Gq"):
+        for u, v in zip(a[key], b[key]):
+            assert all(np.array_equal(x, y) for x, y in zip(u, v)), key
+    for key in ("state", "state_F", "state_dI"):
+        for u, v in zip(a[key], b[key]):
+            assert all(state_equal(x, y) and x["device_token"] == y["device_token"] and x["device_status"] == 0 for x, y in zip(u, v)), key
+    # per step: the casts between the linears, their GEMMs but one a chain, the weights' casts but one
+    fewer = a["stats"]["kernels_launched"] - b["stats"]["kernels_launched"]
+    assert fewer == 2 * (len(shapes) - 1) * (3 * 2 * (2 if tokens <= 8192 else 1) + 1)
+
+
 def test_chain_against_the_oracle_composition(qe):
     M, steps = 3, 2
     s = sched(M, 2, 1)
