@@ -167,7 +167,8 @@ static int32_t forward_impl(qe_layer* L, uint32_t mb, uint64_t gen, const void* 
   Handshake handshake(ctx, caller);
   const uint32_t T = L->cfg.T, K = L->cfg.K, N = L->cfg.N;
   if ((st = handshake.in()) != QE_OK) return st;
-  if (x_host && (st = host_upload(ctx, const_cast<void*>(x), x_host, 2ull * T * K, caller)) != QE_OK) return st;
+  const uint32_t pieces = x_host ? host_pieces(T, x_host, 2ull * T * K, y_host, 2ull * T * N) : 1;
+  if (x_host && pieces == 1 && (st = host_upload(ctx, const_cast<void*>(x), x_host, 2ull * T * K, caller)) != QE_OK) return st;
   if (L->dw_pending[p]) {  // the slot's buffers are still being read by the dW that released it (other stream)
     QE_CUDA(cudaStreamWaitEvent(ctx->exec_stream, L->ev_dw[p], 0));
     L->dw_pending[p] = false;
@@ -178,9 +179,13 @@ static int32_t forward_impl(qe_layer* L, uint32_t mb, uint64_t gen, const void* 
     if ((st = run_action(ctx, &L->gRefresh, rs)) != QE_OK) return st;
   }
   std::vector<qe::Launch> ls;
-  add_forward(L, p, x, y, ls);
-  if ((st = run_action(ctx, &L->gF[p], ls)) != QE_OK) return st;  // ... run ...
-  if (x_host && (st = host_download(ctx, y_host, y, 2ull * T * N)) != QE_OK) return st;
+  if (pieces > 1) {
+    if ((st = run_host_pieces(L, QE_ACT_F, p, pieces, x_host, y_host, caller)) != QE_OK) return st;
+  } else {
+    add_forward(L, p, x, y, ls);
+    if ((st = run_action(ctx, &L->gF[p], ls)) != QE_OK) return st;  // ... run ...
+  }
+  if (x_host && pieces == 1 && (st = host_download(ctx, y_host, y, 2ull * T * N)) != QE_OK) return st;
   if ((st = handshake.out()) != QE_OK) return st;
   return qe_contract_forward_commit(L->contract, mb, tape_out);  // ... commit
 }
@@ -208,12 +213,17 @@ static int32_t backward_dI_impl(qe_layer* L, const qe_tape* tape, const void* dy
   Handshake handshake(ctx, caller);
   const uint32_t p = tape->ref.slot, T = L->cfg.T, K = L->cfg.K, N = L->cfg.N;
   if ((st = handshake.in()) != QE_OK) return st;
-  if (dy_host && (st = host_upload(ctx, const_cast<void*>(dy), dy_host, 2ull * T * N, caller)) != QE_OK) return st;
+  const uint32_t pieces = dy_host ? host_pieces(T, dy_host, 2ull * T * N, dx_host, 2ull * T * K) : 1;
+  if (dy_host && pieces == 1 && (st = host_upload(ctx, const_cast<void*>(dy), dy_host, 2ull * T * N, caller)) != QE_OK) return st;
   std::vector<qe::Launch> ls;
-  add_dI(L, p, dy, dx, ls);
-  if ((st = run_action(ctx, &L->gDI[p], ls)) != QE_OK) return st;
+  if (pieces > 1) {
+    if ((st = run_host_pieces(L, QE_ACT_DI, p, pieces, dy_host, dx_host, caller)) != QE_OK) return st;
+  } else {
+    add_dI(L, p, dy, dx, ls);
+    if ((st = run_action(ctx, &L->gDI[p], ls)) != QE_OK) return st;
+  }
   if (ctx->dw_stream) QE_CUDA(cudaEventRecord(L->ev_di[p], ctx->exec_stream));
-  if (dy_host && (st = host_download(ctx, dx_host, dx, 2ull * T * K)) != QE_OK) return st;
+  if (dy_host && pieces == 1 && (st = host_download(ctx, dx_host, dx, 2ull * T * K)) != QE_OK) return st;
   if ((st = handshake.out()) != QE_OK) return st;
   return qe_contract_dI_commit(L->contract, tape);
 }

@@ -300,7 +300,8 @@ static int32_t uploads_after_readbacks(qe_ctx* ctx) {
   return QE_OK;
 }
 
-int32_t host_upload(qe_ctx* ctx, void* dst, const void* src_host, size_t bytes, cudaStream_t caller) {
+// Before a call's uploads from [src_host, src_host + bytes).
+static int32_t uploads_begin(qe_ctx* ctx, const void* src_host, size_t bytes, cudaStream_t caller) {
   if (!ctx->h2d_stream) {
     ctx->readbacks.reserve(256);
     cudaError_t e = cudaStreamCreateWithFlags(&ctx->h2d_stream, cudaStreamNonBlocking);
@@ -324,13 +325,21 @@ int32_t host_upload(qe_ctx* ctx, void* dst, const void* src_host, size_t bytes, 
         break;
       }
   }
+  return QE_OK;
+}
+// One upload; the kernels that follow wait for it.
+static int32_t upload(qe_ctx* ctx, void* dst, const void* src_host, size_t bytes) {
   QE_CUDA(cudaMemcpyAsync(dst, src_host, bytes, cudaMemcpyHostToDevice, ctx->h2d_stream));
   QE_CUDA(cudaEventRecord(ctx->ev_h2d, ctx->h2d_stream));
   QE_CUDA(cudaStreamWaitEvent(ctx->exec_stream, ctx->ev_h2d, 0));
   return QE_OK;
 }
-// after the action's kernels: frees the staging input for the next upload and starts the read-back (if any)
-int32_t host_download(qe_ctx* ctx, void* dst_host, const void* src, size_t bytes) {
+int32_t host_upload(qe_ctx* ctx, void* dst, const void* src_host, size_t bytes, cudaStream_t caller) {
+  const int32_t st = uploads_begin(ctx, src_host, bytes, caller);
+  return st != QE_OK ? st : upload(ctx, dst, src_host, bytes);
+}
+// After kernels: frees what they read for the next upload and starts the read-back of what they wrote (if any).
+static int32_t download(qe_ctx* ctx, void* dst_host, const void* src, size_t bytes) {
   QE_CUDA(cudaEventRecord(ctx->ev_kernels, ctx->exec_stream));
   ctx->kernels_recorded = true;
   if (!dst_host) return QE_OK;
@@ -342,8 +351,69 @@ int32_t host_download(qe_ctx* ctx, void* dst_host, const void* src, size_t bytes
   QE_CUDA(cudaStreamWaitEvent(ctx->d2h_stream, ctx->ev_kernels, 0));
   QE_CUDA(cudaMemcpyAsync(dst_host, src, bytes, cudaMemcpyDeviceToHost, ctx->d2h_stream));
   QE_CUDA(cudaEventRecord(ctx->ev_d2h, ctx->d2h_stream));
-  QE_CUDA(cudaStreamWaitEvent(ctx->exec_stream, ctx->ev_d2h, 0));
   return QE_OK;
+}
+// After a call's last read-back: what the execution stream is given next comes after it.
+static int32_t downloads_end(qe_ctx* ctx, const void* dst_host) {
+  if (dst_host) QE_CUDA(cudaStreamWaitEvent(ctx->exec_stream, ctx->ev_d2h, 0));
+  return QE_OK;
+}
+int32_t host_download(qe_ctx* ctx, void* dst_host, const void* src, size_t bytes) {
+  const int32_t st = download(ctx, dst_host, src, bytes);
+  return st != QE_OK ? st : downloads_end(ctx, dst_host);
+}
+
+// Pieces of rows in which a forward or an input gradient with host buffers goes through upload, kernels and read-back: the
+// host link carries both directions at once, but one after the other a call's input, kernels and output used it one at a time.
+// Two pieces, or one for every 512 rows up to four, of whole 256-row tiles, whose larger copy is a megabyte at least (19 us at 53
+// GB/s; a piece costs some 15 us of copy starts, events and kernels that its neighbours' copies have to cover).  us a step in one
+// piece / two / up to four of 256 rows: a block of hidden 1024, 1024 tokens, 6385 / 5716 / 5861; 2048 tokens, 1024 x 3072 and
+// 1024 x 1024, 3252 / 2949 / 2882; 640 tokens, 2048 x 2048 and 2048 x 512, 1377 / 1313 / 1312; up to eight of 128 rows 6428 and 3152.
+// An output that overlaps the input is read back when all of that has been uploaded.
+uint32_t host_pieces(uint32_t rows, const void* in, uint64_t in_bytes, const void* out, uint64_t out_bytes) {
+  if (!out) out_bytes = 0;
+  if ((uintptr_t)in < (uintptr_t)out + out_bytes && (uintptr_t)out < (uintptr_t)in + in_bytes) return 1;
+  const uint64_t most = std::min<uint64_t>(4, std::max<uint64_t>(2, rows / 512u));
+  const uint64_t n = std::min<uint64_t>({most, rows / 256u, std::max(in_bytes, out_bytes) >> 20});
+  return (uint32_t)std::max<uint64_t>(1, n);
+}
+
+// F (kind QE_ACT_F) or dI of slot p with host buffers, in pieces; the scale commits go with the last piece's GEMM, whose launch
+// starts after every piece's cast.
+int32_t run_host_pieces(qe_layer* L, uint32_t kind, uint32_t p, uint32_t pieces, const void* in_host, void* out_host, cudaStream_t caller) {
+  qe_ctx* ctx = L->ctx;
+  const uint32_t T = L->cfg.T, cols_in = kind == QE_ACT_F ? L->cfg.K : L->cfg.N, cols_out = kind == QE_ACT_F ? L->cfg.N : L->cfg.K;
+  uint8_t* const in = kind == QE_ACT_F ? L->x_stage : L->dy_stage;
+  uint8_t* const out = kind == QE_ACT_F ? L->y_stage : L->dx_stage;
+  uint8_t* const q = kind == QE_ACT_F ? L->Xq[p] : L->Gq[p];
+  int32_t st = uploads_begin(ctx, in_host, 2ull * T * cols_in, caller);
+  const uint32_t share = T / pieces / 256u * 256u;
+  for (uint32_t i = 0; i < pieces && st == QE_OK; ++i) {
+    const uint32_t row0 = i * share, rows = i + 1 < pieces ? share : T - row0;
+    const size_t at_in = 2ull * row0 * cols_in, at_out = 2ull * row0 * cols_out;
+    if ((st = upload(ctx, in + at_in, (const uint8_t*)in_host + at_in, 2ull * rows * cols_in)) != QE_OK) break;
+    std::vector<qe::Launch> ls;
+    qe::GemmDesc g;
+    qe::QuantParams cast;
+    if (kind == QE_ACT_F) add_forward(L, p, in + at_in, out + at_out, ls, nullptr, 0, &g, &cast);
+    else add_dI(L, p, in + at_in, out + at_out, ls, nullptr, 0, &g, &cast);
+    cast.q += (size_t)row0 * cols_in;
+    cast.rows = rows;
+    CUtensorMap map[2];  // of this piece's rows
+    if ((st = make_a_maps(ctx->dev, map, Slots{q + (size_t)row0 * cols_in}, rows, cols_in, false)) != QE_OK) break;
+    if ((st = make_out_map(ctx->dev, &g.tmD, g.out, rows, cols_out, cols_out, false)) != QE_OK) break;
+    g.M = rows;
+    g.operands(map, &g.alpha_a[p], 0, g.mapB, g.alpha_b, 0);
+    if (i + 1 < pieces) g.commit = qe::CommitParams{};
+    ls.push_back(qe::make_quantize(cast));
+    ls.push_back(qe::make_gemm(g, ctx->dev->num_sms));
+    for (const qe::Launch& l : ls)  // (no graph: a piece's two launches hide behind the copies, and a new layer has none to make)
+      if ((st = launch_eager(ctx, l, ctx->exec_stream)) != QE_OK) break;
+    if (st != QE_OK) break;
+    st = download(ctx, out_host ? (uint8_t*)out_host + at_out : nullptr, out + at_out, 2ull * rows * cols_out);
+  }
+  const int32_t end = downloads_end(ctx, out_host);  // (also when a piece failed: read-backs may be on their way)
+  return st != QE_OK ? st : end;
 }
 
 int32_t run_action(qe_ctx* ctx, ActionGraph* g, const std::vector<qe::Launch>& ls, cudaStream_t stream) {

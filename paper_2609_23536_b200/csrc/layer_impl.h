@@ -151,6 +151,8 @@ class Handshake {
 };
 int32_t host_upload(qe_ctx* ctx, void* dst, const void* src_host, size_t bytes, cudaStream_t caller);
 int32_t host_download(qe_ctx* ctx, void* dst_host, const void* src, size_t bytes);
+uint32_t host_pieces(uint32_t rows, const void* in, uint64_t in_bytes, const void* out, uint64_t out_bytes);
+int32_t run_host_pieces(qe_layer* L, uint32_t kind, uint32_t p, uint32_t pieces, const void* in_host, void* out_host, cudaStream_t caller);
 int32_t run_action(qe_ctx* ctx, ActionGraph* g, const std::vector<qe::Launch>& ls, cudaStream_t stream = nullptr);
 ActionGraph* keyed_graph(qe_ctx* ctx, uint64_t key, size_t n_launches);
 int32_t run_keyed(qe_ctx* ctx, uint64_t key, const std::vector<qe::Launch>& ls);

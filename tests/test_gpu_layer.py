@@ -795,3 +795,29 @@ def test_odd_row_counts_are_exact_on_integers(qe, T, K, N):
         assert L.state()["classes"]["Y"]["window"][0] == float(y[:T].float().abs().max())
     assert L.state()["device_status"] == 0
     L.optimizer_boundary(2)
+
+
+@pytest.mark.parametrize("mode", [0, 1], ids=["eager", "graph"])
+@pytest.mark.parametrize("T,K,N", [(1152, 512, 1280), (768, 2048, 256), (2176, 256, 512)])
+def test_host_buffers_in_pieces_of_rows_equal_the_device_calls_bitwise(qe, mode, T, K, N):
+    """Copies large enough to be cut into pieces, one of them with an odd number of 128-row tiles; outputs, gradient and state."""
+    M, got = 2, []
+    for host in (False, True):
+        ctx = qe.Context(mode)
+        L = qe.Layer(ctx, T, K, N, 4, 0, M, inputs.weights("HP", 0, 0, N, K).to(DEV), host_io=host)
+        grad = torch.zeros(N * K, device=DEV)
+        place = (lambda t: t.pin_memory()) if host else (lambda t: t.to(DEV))
+        outs = []
+        for step in range(2):
+            for m in range(M):
+                x, dy = place(inputs.activations("HP", 0, step, 0, m, T, K)), place(inputs.upstream_grads("HP", 0, step, 0, m, T, N))
+                y, dx = place(torch.zeros((T, N), dtype=torch.bfloat16)), place(torch.zeros((T, K), dtype=torch.bfloat16))
+                tape = (L.forward_host if host else L.forward)(m, step, x, y)
+                (L.backward_dI_host if host else L.backward_dI)(tape, dy, dx)
+                L.backward_dW(tape, grad, 0)
+                torch.cuda.synchronize()
+                outs += [inputs.bits(y.cpu()), inputs.bits(dx.cpu())]
+            L.optimizer_boundary(M)
+        got.append((outs, grad.cpu().numpy().view(np.uint32), L.state(), ctx.stats()["kernels_launched"]))
+    assert all(np.array_equal(a, b) for a, b in zip(got[0][0], got[1][0])) and np.array_equal(got[0][1], got[1][1])
+    assert state_equal(got[0][2], got[1][2]) and got[1][3] > got[0][3]

@@ -289,6 +289,44 @@ def test_step_casts_overlap_the_gemms_before_them_unless_those_read_the_slot(lib
     s.close()
 
 
+@pytest.mark.parametrize("T,pieces", [(256, 1), (1024, 2), (2048, 4), (640, 2)])
+@pytest.mark.parametrize("own_stream", [True, False], ids=["callers-stream", "execution-stream"])
+def test_host_buffers_go_through_copies_and_kernels_in_pieces_of_rows(lib, T, pieces, own_stream):
+    """Every row once in each direction; a piece's kernels after its upload, its read-back after its kernels, and neither waits for
+    the read-back of the piece before; the caller's stream after all of them, also where a launch in the middle fails."""
+    import ctypes as C
+
+    from paper_2609_23536_b200 import binding as qe
+
+    K, N = 256, 2048
+    s = fake_runtime.Stage(lib, [(K, N)], T=T, host_io=True, slots=3, exec_stream=None if own_stream else fake_runtime.CALLER)
+    x, y, tape = s.buffer(2 * T * K), s.buffer(2 * T * (N + K)), qe.qe_tape()
+    assert lib.qe_forward_host(s.layers[0], 0, 0, x, y, fake_runtime.CALLER, C.byref(tape)) == 0  # (with the weight's cast)
+    lib.fake_reset()
+    assert lib.qe_forward_host(s.layers[0], 1, 0, x, y, fake_runtime.CALLER, C.byref(tape)) == 0
+    order = fake_runtime.Order(lib.fake_log().decode())
+    up, down, run = order.of("h2d"), order.of("d2h"), order.of("launch")
+    assert (len(up), len(down), len(run)) == (pieces, pieces, 2 * pieces)
+    for ops, at, base, row in ((up, 1, x, 2 * K), (down, 0, y, 2 * N)):  # (words of a copy: destination, source, bytes)
+        parts = sorted((int(o[2][at]) - base, int(o[2][2])) for o in ops)
+        assert [a for a, n in parts] == [0] + [a + n for a, n in parts][:-1] and sum(n for a, n in parts) == T * row
+    for i in range(pieces):
+        assert order.before(up[i], run[2 * i]) and order.before(run[2 * i + 1], down[i]) and order.seen_by(fake_runtime.CALLER, down[i])
+        if i:
+            assert not order.before(down[i - 1], run[2 * i]) and not order.before(down[i - 1], up[i])
+    lib.fake_reset()  # an output that overlaps the input: not before all of that is up
+    assert lib.qe_backward_dI_host(s.layers[0], C.byref(tape), y, y + 2 * T * N - 64, fake_runtime.CALLER) == 0
+    order = fake_runtime.Order(lib.fake_log().decode())
+    assert len(order.of("h2d")) == len(order.of("d2h")) == 1
+    assert lib.qe_forward_host(s.layers[0], 2, 0, x, y, fake_runtime.CALLER, C.byref(tape)) == 0
+    lib.fake_reset()
+    lib.fake_fail(b"cudaLaunchKernelExC", 2 * pieces)
+    assert lib.qe_backward_dI_host(s.layers[0], C.byref(tape), y, x, fake_runtime.CALLER) == CUDA
+    order = fake_runtime.Order(lib.fake_log().decode())
+    assert all(order.seen_by(fake_runtime.CALLER, o) for o in order.of("launch") + order.of("d2h"))
+    s.close()
+
+
 @pytest.mark.parametrize("mode", [0, 1], ids=["eager", "graph"])
 def test_casts_that_overlap_go_ahead_on_a_count_of_commits(lib, mode):
     """A cast that does not wait for the GEMM launch before it is told how many problems will have committed by then, and that
