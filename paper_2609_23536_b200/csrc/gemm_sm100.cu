@@ -1380,6 +1380,10 @@ Launch make_any(const GemmDesc* probs, uint32_t n, int num_sms) {
   }
   if (!sums && n <= kFew) return make_launch<kFew>(probs, n, num_sms, (const void*)gemm_fp8_pair_group_kernel<kFew>, false);
   if (!sums) return make_launch<kMaxProblems>(probs, n, num_sms, (const void*)gemm_fp8_pair_group_kernel<kMaxProblems>, false);
+  // Output buffers of a sum's epilogue warps, for each of which there is one operand stage less than six.  Short products are as
+  // good as never short of operands and want to be rid of their results, long ones the other way round: us a step with four / three / one,
+  // 256 tokens 1294 / 1313 / 1446 (4096 / 11008 layer) and 451 / 456 / 498 (2048 / 8192), 512 tokens 4638 / 4597 / 4723 (48 linears of 1024),
+  // 768 748 / 734 / 747 (eight of 2048), 1024 740 / 746 / 722 (six of 2048), 2048 2331 / 2122 / 2120 (block of hidden 2048).
   uint32_t longest = 0;
   for (uint32_t i = 0; i < n; ++i)
     if (probs[i].sum && probs[i].Kc > longest) longest = probs[i].Kc;
