@@ -93,8 +93,20 @@ __device__ __forceinline__ uint32_t ring_max(const uint32_t* ring, uint32_t n, u
 // linear plus the boundary take 55 us when no commit scans; when all three do, 60 us at 4096 entries and the same as without
 // at 1024.  Same values as commit_classes; the token is bumped atomically because two problems of one launch may belong to
 // the same layer (its forward and its input gradient of different microbatches).
+// What a commit of a class reads besides its amax, where that can be read ahead: nothing else commits the class until then.
+struct RingState {
+  uint32_t count = 0, wmax = 0, evicted = 0;
+};
+__device__ __forceinline__ RingState ring_state(const CommitParams& p, int c) {
+  RingState s;
+  s.count = __ldcg(&p.st->count[c]);
+  s.wmax = __ldcg(&p.st->wmax[c]);
+  s.evicted = __ldcg(reinterpret_cast<const uint32_t*>(p.hist + (size_t)c * p.H) + s.count % p.H);
+  return s;
+}
+
 template <bool EACH>
-__device__ __forceinline__ void commit_class(const CommitParams& p, uint32_t class_mask, bool bump, bool active, int lane) {
+__device__ __forceinline__ void commit_class(const CommitParams& p, uint32_t class_mask, bool bump, bool active, int lane, const RingState* ahead = nullptr) {
   DevState* st = p.st;
   const int c = !EACH || active ? __ffs(class_mask) - 1 : 0;
   uint32_t* h = reinterpret_cast<uint32_t*>(p.hist + (size_t)c * p.H);
@@ -102,11 +114,11 @@ __device__ __forceinline__ void commit_class(const CommitParams& p, uint32_t cla
   uint32_t cnt = 0, newest = 0, m = 0, pos = 0;
   bool scan = false;
   if (!EACH || active) {
-    cnt = __ldcg(&st->count[c]);
     newest = p.amax_override ? (__float_as_uint(__ldcg(p.amax_override)) & 0x7fffffffu) : __ldcg(&st->pending_amax[c]);
-    const uint32_t wmax = __ldcg(&st->wmax[c]);
+    const RingState now = ahead ? *ahead : ring_state(p, c);
+    const uint32_t wmax = now.wmax, evicted = now.evicted;
+    cnt = now.count;
     pos = cnt % H;
-    const uint32_t evicted = __ldcg(h + pos);
     m = newest >= wmax ? newest : wmax;
     scan = newest < wmax && evicted >= wmax;  // the maximum leaves: scan what stays
   }

@@ -174,6 +174,14 @@ __device__ __forceinline__ bool last_of_cta(uint32_t* count /* shared */, uint32
   asm volatile("atom.acq_rel.cta.shared::cta.add.u32 %0, [%1], 1;" : "=r"(before) : "r"(smem_u32(count)) : "memory");
   return (before + 1) % warps == 0;
 }
+// Whether a CTA is the last of the grid to say so.  What any of them did before is visible to who learns that it is.
+__device__ __forceinline__ bool last_of_grid(uint32_t* ticket, uint32_t ctas) {
+  uint32_t before;
+  asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(before) : "l"(ticket) : "memory");
+  if (before != ctas - 1) return false;
+  *ticket = 0u;  // ready for the next kernel that uses it
+  return true;
+}
 __device__ __forceinline__ void add_release(uint32_t* p, uint32_t v) {
   asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
@@ -487,7 +495,7 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
   auto info_parity = [](uint32_t n) { return n / INFO_SLOTS & 1u; };
   volatile uint32_t* abort_flag = tmem_slot + 1;
   uint32_t* last_flag = tmem_slot + 2;
-  uint32_t* stored_count = tmem_slot + 3;  // chained problems: epilogue warps that have stored their part of a tile
+  uint32_t* warps_done = tmem_slot + 3;  // epilogue warps that have come to where the CTA is counted
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = PAIR ? cluster_ctarank() : 0u;  // position in the CTA pair; rank 0 issues the MMAs
@@ -575,7 +583,7 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
       mbar_init(taken_bar(i), EPI_WARPS + 1 + (SUMS ? 1u : 0u) + (rank == 0 ? 1u : 0u));  // epilogue, producer, storing warp, MMA issuer
     }
     *abort_flag = 0u;
-    *stored_count = 0u;
+    *warps_done = 0u;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
@@ -970,6 +978,8 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
       for (uint32_t j = 0; j < 4; ++j)
         if (j < t.blocks) asm volatile("prefetch.global.L2 [%0];" ::"l"(t.dst + 32 * j));
     };
+    RingState ring_of_Y;  // (the class that the tail commits)
+    if (ONE && ps.ticket()) ring_of_Y = ring_state(ps.commit(0), __ffs(ps.commit(0).class_mask) - 1);
     Part now;
     ok = first_tile < num_tiles && take_part(0, now);
     uint32_t n = 0, tile = first_tile;
@@ -1096,7 +1106,7 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
       }
       if (CHAIN && t.epi == 3) {  // the next problem's loads of these rows wait for this
         __syncwarp();
-        if (lane == 0 && last_of_cta(stored_count, EPI_WARPS)) add_release(t.done, 1u);
+        if (lane == 0 && last_of_cta(warps_done, EPI_WARPS)) add_release(t.done, 1u);
       }
       uint32_t* const also = ONE || CHAIN ? p.amax_bits2 : nullptr;  // (hand-off)
       if ((t.epi == 0 || ((ONE || CHAIN) && t.epi == 3)) && (t.amax_bits || also)) {
@@ -1176,12 +1186,21 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
     // Every epilogue thread of every CTA gets here (also after a timeout); the last CTA commits the scale state of
     // every problem that asks for it.  The commit needs the amax atomics only, so it runs while this CTA's last
     // bulk stores are still draining.
-    if (ps.ticket() && last_block(ps.ticket(), gridDim.x, etid, last_flag, epi_bar_sync)) {
+    // (Of one problem by a warp: the last of its CTA to get here, of the last CTA.  It has read ahead what it needs beside the amax.
+    // Counted by all threads behind a fence and two barriers, the commit read and made after that, the tail was 0.7 us longer:
+    // a 2048 / 8192 layer of 256 tokens action by action 992 -> 980 us a step, 512 to 2048 at 640 tokens 1190 -> 1164.)
+    if (ONE && ps.ticket()) {
+      __syncwarp();
+      const bool last = lane == 0 && last_of_cta(warps_done, EPI_WARPS) && last_of_grid(ps.ticket(), gridDim.x);
+      if (__shfl_sync(0xffffffffu, last ? 1 : 0, 0)) {
+        __syncwarp();
+        commit_class<false>(ps.commit(0), ps.commit(0).class_mask, false, true, lane, &ring_of_Y);
+      }
+    }
+    if (!ONE && ps.ticket() && last_block(ps.ticket(), gridDim.x, etid, last_flag, epi_bar_sync)) {
       // (the token is counted by the early part)
       const uint32_t ew = (uint32_t)(warp - EPI_WARP0);
-      if (PS::ONE) {
-        if (ew == 0) commit_class<false>(ps.commit(0), ps.commit(0).class_mask, false, true, lane);
-      } else if (ew < ps.count()) {  // a lane per problem, dealt to the epilogue's warps
+      if (ew < ps.count()) {  // a lane per problem, dealt to the epilogue's warps
         static_assert(kMaxProblems <= EPI_WARPS * 32, "a lane for every problem");
         const uint32_t i = ew + EPI_WARPS * (uint32_t)lane;
         const CommitParams& c = ps.commit(i < ps.count() ? i : 0u);
