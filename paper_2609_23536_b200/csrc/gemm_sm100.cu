@@ -48,6 +48,7 @@
 
 #include "commit.cuh"
 #include "kernels.h"
+#include "tile_count.h"
 
 namespace qe {
 namespace {
@@ -167,12 +168,12 @@ __device__ __forceinline__ bool rows_wait(const uint32_t* done, uint32_t count, 
   return __all_sync(0xffffffffu, there);
 }
 
-// ... and how they say it: the last warp of a CTA to get here, for all of them.  (An addition of each warp's own, behind a fence of
+// ... and how they say it: the last warp of a CTA to have stored its part (last_of_tile), for all of them.  (An addition of each warp's own, behind a fence of
 // each lane, took 3500 clocks from a tile's last store until its rows were seen to be there; now 2000.)
-__device__ __forceinline__ bool last_of_cta(uint32_t* count /* shared */, uint32_t warps) {
+__device__ __forceinline__ uint32_t add_acq_rel_cta(uint32_t* count /* shared */) {
   uint32_t before;
   asm volatile("atom.acq_rel.cta.shared::cta.add.u32 %0, [%1], 1;" : "=r"(before) : "r"(smem_u32(count)) : "memory");
-  return (before + 1) % warps == 0;
+  return before;
 }
 // Whether a CTA is the last of the grid to say so.  What any of them did before is visible to who learns that it is.
 __device__ __forceinline__ bool last_of_grid(uint32_t* ticket, uint32_t ctas) {
@@ -473,15 +474,15 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
   const uint32_t smem_base = smem_u32(smem_raw);
   const uint32_t epi_base = smem_base + RING_BYTES;  // 1 KB-aligned
   const uint32_t bar_base = smem_base + RING_AND_BUFS;
-  // barrier block: full[MAX_STAGES], empty[MAX_STAGES], tmem_full[2], tmem_empty[2], tmem address + abort flag + last-CTA flag,
-  // of the tile records full, scales and empty[INFO_SLOTS], of the buffers of sums ready and result[2][BUFS]
+  // barrier block: full[MAX_STAGES], empty[MAX_STAGES], tmem_full[2], tmem_empty[2], tmem address + abort flag + last-CTA flag + counts
+  // of warps, of the tile records full, scales and empty[INFO_SLOTS], of the buffers of sums ready and result[2][BUFS]
   auto full_bar = [&](uint32_t s) { return bar_base + 8u * s; };
   auto empty_bar = [&](uint32_t s) { return bar_base + 8u * (MAX_STAGES + s); };
   auto tfull_bar = [&](int a) { return bar_base + 8u * (2 * MAX_STAGES + a); };
   auto tempty_bar = [&](int a) { return bar_base + 8u * (2 * MAX_STAGES + 2 + a); };
   uint8_t* const gen_base = smem_raw;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(gen_base + RING_AND_BUFS + 8 * (2 * MAX_STAGES + 4));
-  constexpr uint32_t INFO_BARS = 8 * (2 * MAX_STAGES + 4) + 16;
+  constexpr uint32_t INFO_BARS = 8 * (2 * MAX_STAGES + 4) + (4 * (3 + kTileCounters) + 7) / 8 * 8;
   constexpr uint32_t BUF_BARS = INFO_BARS + 8 * 3 * INFO_SLOTS;
   static_assert(BUF_BARS + 8 * 4 * BUFS <= BARS_BYTES, "barrier block too large");
   // sums: buffer b of a half of the tile's columns (128 rows x 32 columns) is the epilogue's again (free, or holding what the
@@ -495,7 +496,7 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
   auto info_parity = [](uint32_t n) { return n / INFO_SLOTS & 1u; };
   volatile uint32_t* abort_flag = tmem_slot + 1;
   uint32_t* last_flag = tmem_slot + 2;
-  uint32_t* warps_done = tmem_slot + 3;  // epilogue warps that have come to where the CTA is counted
+  uint32_t* warps_done = tmem_slot + 3;  // [kTileCounters]: epilogue warps that have come to where a tile, or the CTA, is counted
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = PAIR ? cluster_ctarank() : 0u;  // position in the CTA pair; rank 0 issues the MMAs
@@ -583,7 +584,7 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
       mbar_init(taken_bar(i), EPI_WARPS + 1 + (SUMS ? 1u : 0u) + (rank == 0 ? 1u : 0u));  // epilogue, producer, storing warp, MMA issuer
     }
     *abort_flag = 0u;
-    *warps_done = 0u;
+    for (uint32_t i = 0; i < kTileCounters; ++i) warps_done[i] = 0u;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
@@ -1106,7 +1107,7 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
       }
       if (CHAIN && t.epi == 3) {  // the next problem's loads of these rows wait for this
         __syncwarp();
-        if (lane == 0 && last_of_cta(warps_done, EPI_WARPS)) add_release(t.done, 1u);
+        if (lane == 0 && last_of_tile(n, EPI_WARPS, [&](uint32_t i) { return add_acq_rel_cta(warps_done + i); })) add_release(t.done, 1u);
       }
       uint32_t* const also = ONE || CHAIN ? p.amax_bits2 : nullptr;  // (hand-off)
       if ((t.epi == 0 || ((ONE || CHAIN) && t.epi == 3)) && (t.amax_bits || also)) {
@@ -1191,7 +1192,7 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
     // a 2048 / 8192 layer of 256 tokens action by action 992 -> 980 us a step, 512 to 2048 at 640 tokens 1190 -> 1164.)
     if (ONE && ps.ticket()) {
       __syncwarp();
-      const bool last = lane == 0 && last_of_cta(warps_done, EPI_WARPS) && last_of_grid(ps.ticket(), gridDim.x);
+      const bool last = lane == 0 && add_acq_rel_cta(warps_done) == EPI_WARPS - 1 && last_of_grid(ps.ticket(), gridDim.x);
       if (__shfl_sync(0xffffffffu, last ? 1 : 0, 0)) {
         __syncwarp();
         commit_class<false>(ps.commit(0), ps.commit(0).class_mask, false, true, lane, &ring_of_Y);

@@ -127,10 +127,12 @@ def test_chain_of_odd_token_counts_equals_layer_by_layer_bitwise(qe, tokens, mon
 
 @pytest.mark.parametrize("mode", [0, 1], ids=["eager", "graph"])
 @pytest.mark.parametrize("tokens,shapes", [(256, [(256, 256)] * 16), (1280, [(512, 1280), (1280, 2048), (2048, 512), (512, 256), (256, 768)]),
+                                           (4096, [(256, 4096), (4096, 256)] * 2), (8192, [(512, 2048), (2048, 256), (256, 4096), (4096, 256)]),
                                            (8192, [(256, 256)] * 4), (8448, [(256, 256)] * 4)])
 def test_chains_in_one_launch_equal_layer_by_layer_bitwise(qe, mode, tokens, shapes, monkeypatch):
     """Four linears to sixteen in one launch, whose tiles wait for the rows they read: one tile to a linear, several waves of tiles,
-    contractions longer and shorter than the operand ring, the most rows it is offered for and one row tile more."""
+    contractions longer and shorter than the operand ring, four to seven tiles of one linear for each CTA pair, whose epilogue warps drift
+apart (two K blocks a tile), the most rows it is offered for and one row tile more."""
     monkeypatch.setattr(sys.modules[__name__], "T", tokens)
     monkeypatch.setattr(sys.modules[__name__], "CHAIN", shapes)
     a = _run(qe, mode, chained=False)
