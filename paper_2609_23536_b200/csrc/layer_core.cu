@@ -379,38 +379,48 @@ uint32_t host_pieces(uint32_t rows, const void* in, uint64_t in_bytes, const voi
 }
 
 // F (kind QE_ACT_F) or dI of slot p with host buffers, in pieces; the scale commits go with the last piece's GEMM, whose launch
-// starts after every piece's cast.
+// starts after every piece's cast.  All launches are made before the first kernel and the first read-back go out: what can fail for
+// want of memory fails with nothing but an upload on its way.
 int32_t run_host_pieces(qe_layer* L, uint32_t kind, uint32_t p, uint32_t pieces, const void* in_host, void* out_host, cudaStream_t caller) {
   qe_ctx* ctx = L->ctx;
   const uint32_t T = L->cfg.T, cols_in = kind == QE_ACT_F ? L->cfg.K : L->cfg.N, cols_out = kind == QE_ACT_F ? L->cfg.N : L->cfg.K;
   uint8_t* const in = kind == QE_ACT_F ? L->x_stage : L->dy_stage;
   uint8_t* const out = kind == QE_ACT_F ? L->y_stage : L->dx_stage;
   uint8_t* const q = kind == QE_ACT_F ? L->Xq[p] : L->Gq[p];
-  int32_t st = uploads_begin(ctx, in_host, 2ull * T * cols_in, caller);
   const uint32_t share = T / pieces / 256u * 256u;
-  for (uint32_t i = 0; i < pieces && st == QE_OK; ++i) {
-    const uint32_t row0 = i * share, rows = i + 1 < pieces ? share : T - row0;
-    const size_t at_in = 2ull * row0 * cols_in, at_out = 2ull * row0 * cols_out;
-    if ((st = upload(ctx, in + at_in, (const uint8_t*)in_host + at_in, 2ull * rows * cols_in)) != QE_OK) break;
-    std::vector<qe::Launch> ls;
+  const auto first_row = [&](uint32_t i) { return i < pieces ? i * share : T; };
+  const auto upload_piece = [&](uint32_t i) {
+    const size_t at = 2ull * first_row(i) * cols_in;
+    return upload(ctx, in + at, (const uint8_t*)in_host + at, 2ull * first_row(i + 1) * cols_in - at);
+  };
+  int32_t st = uploads_begin(ctx, in_host, 2ull * T * cols_in, caller);
+  if (st == QE_OK) st = upload_piece(0);
+  if (st != QE_OK) return st;
+  std::vector<qe::Launch> ls;
+  ls.reserve(2 * pieces);
+  for (uint32_t i = 0; i < pieces; ++i) {
+    const uint32_t row0 = first_row(i), rows = first_row(i + 1) - row0;
     qe::GemmDesc g;
     qe::QuantParams cast;
-    if (kind == QE_ACT_F) add_forward(L, p, in + at_in, out + at_out, ls, nullptr, 0, &g, &cast);
-    else add_dI(L, p, in + at_in, out + at_out, ls, nullptr, 0, &g, &cast);
+    if (kind == QE_ACT_F) add_forward(L, p, in + 2ull * row0 * cols_in, out + 2ull * row0 * cols_out, ls, nullptr, 0, &g, &cast);
+    else add_dI(L, p, in + 2ull * row0 * cols_in, out + 2ull * row0 * cols_out, ls, nullptr, 0, &g, &cast);
     cast.q += (size_t)row0 * cols_in;
     cast.rows = rows;
     CUtensorMap map[2];  // of this piece's rows
-    if ((st = make_a_maps(ctx->dev, map, Slots{q + (size_t)row0 * cols_in}, rows, cols_in, false)) != QE_OK) break;
-    if ((st = make_out_map(ctx->dev, &g.tmD, g.out, rows, cols_out, cols_out, false)) != QE_OK) break;
+    if ((st = make_a_maps(ctx->dev, map, Slots{q + (size_t)row0 * cols_in}, rows, cols_in, false)) != QE_OK) return st;
+    if ((st = make_out_map(ctx->dev, &g.tmD, g.out, rows, cols_out, cols_out, false)) != QE_OK) return st;
     g.M = rows;
     g.operands(map, &g.alpha_a[p], 0, g.mapB, g.alpha_b, 0);
     if (i + 1 < pieces) g.commit = qe::CommitParams{};
     ls.push_back(qe::make_quantize(cast));
     ls.push_back(qe::make_gemm(g, ctx->dev->num_sms));
-    for (const qe::Launch& l : ls)  // (no graph: a piece's two launches hide behind the copies, and a new layer has none to make)
-      if ((st = launch_eager(ctx, l, ctx->exec_stream)) != QE_OK) break;
-    if (st != QE_OK) break;
-    st = download(ctx, out_host ? (uint8_t*)out_host + at_out : nullptr, out + at_out, 2ull * rows * cols_out);
+  }
+  for (uint32_t i = 0; i < pieces && st == QE_OK; ++i) {
+    if (i) st = upload_piece(i);
+    for (uint32_t k = 2 * i; k < 2 * i + 2 && st == QE_OK; ++k)  // (no graph: a piece's two launches hide behind the copies, and a
+      st = launch_eager(ctx, ls[k], ctx->exec_stream);           // new layer has none to make)
+    const size_t at = 2ull * first_row(i) * cols_out;
+    if (st == QE_OK) st = download(ctx, out_host ? (uint8_t*)out_host + at : nullptr, out + at, 2ull * first_row(i + 1) * cols_out - at);
   }
   const int32_t end = downloads_end(ctx, out_host);  // (also when a piece failed: read-backs may be on their way)
   return st != QE_OK ? st : end;

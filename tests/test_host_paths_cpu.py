@@ -165,7 +165,7 @@ def out_of_memory(so):
             # (a step that finds no memory for one issue plan may still run by another)
             assert st == BAD_ARG and b"out of host memory" in lib.qe_last_error() or (st == 0 and again), (st, lib.qe_last_error())
             order = fake_runtime.Order(lib.fake_log().decode())
-            assert all(order.seen_by(fake_runtime.CALLER, x) for x in order.of("launch"))
+            assert all(order.seen_by(fake_runtime.CALLER, x) for kind in ("launch", "h2d", "d2h") for x in order.of(kind))
             if again:
                 again()
 
@@ -177,6 +177,12 @@ def out_of_memory(so):
         s = fake_runtime.Stage(lib, [(256, 256)] * 3, T=384, slots=4, mode=mode)
         for name, call in _calls(s, lib):
             assert attempts(call) > 1, name
+        for T, pieces in ((256, 1), (1024, 2), (2048, 4)):  # (nothing is on its way before all that the call needs is there)
+            h = fake_runtime.Stage(lib, [(256, 2048)], T=T, host_io=True, slots=4, mode=mode)
+            x, y, tape = h.buffer(2 * T * 256), h.buffer(2 * T * 2048), qe.qe_tape()
+            assert attempts(lambda: lib.qe_forward_host(h.layers[0], 0, 0, x, y, fake_runtime.CALLER, C.byref(tape))) > 1
+            assert attempts(lambda: lib.qe_backward_dI_host(h.layers[0], C.byref(tape), y, x, fake_runtime.CALLER)) > 1
+            h.close()
         view, window = qe.qe_state_view(), (C.c_float * 16)()
         attempts(lambda: lib.qe_get_state(s.layers[0], C.byref(view), window, None))
         out = (C.c_char * 65536)()
