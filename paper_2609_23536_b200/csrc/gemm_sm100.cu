@@ -1425,6 +1425,25 @@ cudaError_t gemm_prepare() {
   return cudaSuccess;
 }
 
+bool chained_fit(int num_sms, cudaStream_t stream) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((uint32_t)num_sms / 2u * 2u, 1, 1);
+  cfg.blockDim = dim3(threads_of(false, true), 1, 1);
+  cfg.dynamicSmemBytes = SMEM_BYTES;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim = {2, 1, 1};
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  int clusters = 0;
+  if (cudaOccupancyMaxActiveClusters(&clusters, (const void*)gemm_fp8_pair_chain_kernel, &cfg) != cudaSuccess) {
+    cudaGetLastError();  // (the question's, not a call's)
+    return false;
+  }
+  return clusters >= num_sms / 2;
+}
+
 bool make_gemm_group(const GemmDesc* probs, uint32_t n, int num_sms, Launch* out) {
   if (n && probs->chained) {
     if (!launch_chained(probs, n, num_sms)) return false;

@@ -268,6 +268,9 @@ Launch make_gemm(const GemmDesc& p, int num_sms);
 // better launched one by one.
 // (most_committing, where they commit scales at the launch's start)
 bool make_gemm_group(const GemmDesc* probs, uint32_t n, int num_sms, Launch* out);
+// Whether the device, as the stream may use it, holds all blocks of a launch of chained GEMMs at once.  (A device whose units have odd
+// numbers of SMs, or a part of one, may not; launches one by one run on any number.)
+bool chained_fit(int num_sms, cudaStream_t stream);
 uint32_t announce_commits(Launch* gemm, uint32_t* word);  // the launch is to count its problems in *word; how many that are
 void withdraw_commits(Launch* gemm, uint32_t* word);      // the launch is to set *word to zero
 uint32_t gemm_width(const GemmDesc* probs, uint32_t n, int num_sms);  // index of the tile width the launch of these will have

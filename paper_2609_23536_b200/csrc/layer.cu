@@ -38,6 +38,7 @@ int32_t qe_ctx_create(const qe_ctx_config* cfg, qe_ctx** out) {
     if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&c->dw_stream, cudaStreamNonBlocking, least);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->ev_dw_in, cudaEventDisableTiming);
   }
+  c->chained_fit = e == cudaSuccess && qe::chained_fit(d->num_sms, c->exec_stream);
   st = e == cudaSuccess ? qe_registry_create(&c->registry) : fail(QE_ERR_CUDA, "context resources: %s", cudaGetErrorString(e));
   if (st != QE_OK) {  // release whatever was created
     if (c->ev_in) cudaEventDestroy(c->ev_in);

@@ -4,11 +4,11 @@
 
 using namespace qe_impl;
 
-// The GEMMs of a chain in one launch where that is offered, else one by one, each as `alone` has it.
+// The GEMMs of a chain in one launch where that is offered and fits the device, else one by one, each as `alone` has it.
 template <class F>
 static void push_chain(qe_ctx* ctx, std::vector<qe::GemmDesc>& gemms, std::vector<qe::Launch>& ls, F alone) {
   qe::Launch l;
-  if (gemms.size() > 1 && qe::make_gemm_group(gemms.data(), (uint32_t)gemms.size(), ctx->dev->num_sms, &l)) {
+  if (gemms.size() > 1 && ctx->chained_fit && qe::make_gemm_group(gemms.data(), (uint32_t)gemms.size(), ctx->dev->num_sms, &l)) {
     ls.push_back(std::move(l));
     return;
   }

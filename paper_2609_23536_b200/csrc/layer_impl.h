@@ -70,6 +70,7 @@ struct qe_ctx {
   cudaStream_t exec_stream = nullptr;
   bool owns_stream = true;
   bool one_way = false;              // QE_CTX_UNSAFE_ONE_WAY_HANDOFF
+  bool chained_fit = false;          // a launch of chained GEMMs can have all its blocks on the device at once
   bool launch_failed = false;        // a whole-step call's: counts of commits in device memory may not be what they should be
   uint32_t step_window = 4;          // qe_step_run: units looked ahead when planning rounds (1: action by action)
   cudaStream_t dw_stream = nullptr;  // only with QE_CTX_OVERLAP_DW

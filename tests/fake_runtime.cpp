@@ -29,7 +29,7 @@ struct State {
   cudaStream_t capturing = nullptr;
   Graph* graph = nullptr;
   long encodes = 0;
-  int sms = 148;
+  int sms = 148, pairs = 74;
 };
 State* g = nullptr;  // (never freed: the library may be used until the process ends)
 State& s() {
@@ -91,6 +91,7 @@ void fake_fail(const char* fn, long nth) { s().fail_in[fn] = nth; }
 void fake_fail_alloc(long nth) { s().alloc_in = nth; }
 long fake_alloc_left() { return s().alloc_in; }
 void fake_sms(int n) { s().sms = n; }  // before the library has looked at the device
+void fake_pairs(int n) { s().pairs = n; }  // CTA pairs that the device holds at once
 long fake_encodes() { return s().encodes; }
 
 cudaError_t cudaGetDeviceCount(int* n) { *n = 1; return cudaSuccess; }
@@ -214,6 +215,7 @@ Launch named(const char* fmt, ...) {
 }  // namespace
 bool whole_row_tiles(uint32_t M) { return M % 256 == 0; }
 cudaError_t gemm_prepare() { return cudaSuccess; }
+bool chained_fit(int sms, cudaStream_t) { return s().pairs >= sms / 2; }
 uint32_t gemm_width(const GemmDesc*, uint32_t, int) { return 1; }
 Launch make_quantize(const QuantParams&) { return named("cast 1"); }
 Launch make_quantize_multi(const QuantParams*, uint32_t n, const Announce& early) {

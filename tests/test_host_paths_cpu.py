@@ -372,6 +372,26 @@ def test_casts_that_overlap_go_ahead_on_a_count_of_commits(lib, mode):
     s.close()
 
 
+@pytest.mark.parametrize("pairs,launches", [(74, 1), (73, 4), (10, 4), (0, 4)])
+def test_chains_go_out_one_by_one_where_the_device_does_not_hold_all_their_blocks(lib, pairs, launches):
+    import ctypes as C
+
+    from paper_2609_23536_b200 import binding as qe
+
+    lib.fake_pairs(pairs)
+    s = fake_runtime.Stage(lib, [(256, 256)] * 4)
+    lib.fake_pairs(74)
+    x, y, tapes = s.buffer(2 * s.T * 256), s.buffer(2 * s.T * 256), (qe.qe_tape * 4)()
+    hs = (C.c_void_p * 4)(*[h.value for h in s.layers])
+    for call in (lambda: lib.qe_forward_chain(hs, 4, 0, 0, x, y, fake_runtime.CALLER, tapes),
+                 lambda: lib.qe_backward_dI_chain(hs, tapes, 4, y, x, fake_runtime.CALLER)):
+        lib.fake_reset()
+        assert call() == 0
+        words = [w.split() for w in lib.fake_log().decode().splitlines() if " gemm " in w]  # launch STREAM gemm N products P
+        assert [int(w[3]) for w in words] == ([4] if launches == 1 else [1] * launches)
+    s.close()
+
+
 @pytest.mark.parametrize("sms", [20, 57, 148])
 def test_launches_that_commit_scales_hold_a_problem_per_cta_at_most(lib, tmp_path, sms):
     """A problem's early commit is made by the CTA of its number: a device of few SMs gets more launches, not lost commits."""
