@@ -672,6 +672,7 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
   if (warp == 0) {
     // ---------------------------------------------------------------- TMA producer
     const bool elected = elect_one();
+    const bool several_waves = num_tiles > ps.count() * tile_step;  // (of each of the problems, on an average)
     uint32_t s = 0, ph = 0;
     bool ok = true;
     for (uint32_t n = 0, tile = first_tile; ok && tile < num_tiles; ++n, tile = tile_of(n)) {
@@ -705,13 +706,15 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
         const CUtensorMap *tmA = &p.tmA, *tmB = &p.tmB;
         const int sa = SUMS ? (int)uniform((uint32_t)slots_a & 255u) : (int)slots_a, sb = SUMS ? (int)uniform((uint32_t)slots_b & 255u) : (int)slots_b;
         uint32_t kb = 0;
-        const GemmParams& q = ps.problem(CHAIN && t.problem ? t.problem - 1 : 0u);  // whose result A is
-        const uint32_t* const rows = &q.commit.st->rows_done[t.m0 / TILE_M];
-        const uint32_t parts = (q.N + tile_n - 1) / tile_n * CTAS;
-        if (CHAIN && t.problem && !rows_there(rows, parts)) {
+        auto rows_before = [&](auto ask) {  // of the result that A is
+          const GemmParams& q = ps.problem(t.problem - 1);
+          return ask(&q.commit.st->rows_done[t.m0 / TILE_M], (q.N + tile_n - 1) / tile_n * CTAS);
+        };
+        if (CHAIN && t.problem && !(several_waves && rows_before(rows_there))) {
           // A is being made by other CTAs: B first, as far as the ring goes, then A when its rows are there.  (Where they are there
           // already, A and B go together: the first A would wait until the tile before had freed the whole ring.  Linears of several
-          // waves meet few rows that they have to wait for: four of 4096 x 4096 at 8192 tokens 448 -> 408 us, at 4096 213 -> 199.)
+          // waves meet few rows that they have to wait for: four of 4096 x 4096 at 8192 tokens 448 -> 408 us, at 4096 213 -> 199.
+          // Linears of one wave find none there, and to ask holds up B: sixteen of 1024 x 1024 at 512 tokens 1497 -> 1516 a step.)
           const uint32_t s0 = s;
           for (uint32_t j = 0; ok && j < ring.stages && kb < t.num_kb; ++j, kb += ring.blocks) {
             if (!(ok = await(empty_bar(s), ph ^ 1u, ERR_PRODUCER))) break;
@@ -721,7 +724,8 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
             }
             if (++s == ring.stages) { s = 0; ph ^= 1u; }
           }
-          if (!(ok = ok && rows_wait(rows, parts, abort_flag, status))) break;
+          ok = ok && rows_before([&](const uint32_t* done, uint32_t count) { return rows_wait(done, count, abort_flag, status); });
+          if (!ok) break;
           for (uint32_t j = s0, at = 0; at < kb; at += ring.blocks) {
             if (elected) tma_load<PAIR>(smem_base + j * ring.stage_bytes, tmA, PAIR ? map_to_cta(full_bar(j), 0) : full_bar(j), a0, a1, (int)at, sa);
             if (++j == ring.stages) j = 0;
