@@ -42,7 +42,6 @@
 #include <type_traits>
 #include <cuda_fp8.h>
 
-#include <algorithm>
 #include <cstddef>
 #include <cstring>
 
@@ -1356,16 +1355,32 @@ GemmParams problem_of(const GemmDesc& d, uint32_t w, uint32_t tile_m) {
 }
 
 // Whether chained problems go out as one launch.  What that saves is a launch's start and end between two of them, about
-// 1.3 us of 5.5 for 512 x 1024 x 1024, and a layer's last wave, which the next one's tiles fill; what it costs is a launch whose
-// blocks all have to be there at once, which starts some us later: us a step of eight microbatches of 512 tokens, one by one / in
-// one launch, two linears of 1024 x 1024 381 / 418, three 485 / 502, sixteen 1713 / 1499; 256 x 256 at 256 tokens, twelve 1252 /
-// 1035; four microbatches of 2048 tokens, eight of 2048 x 2048 1199 / 1072; 4096 tokens, four of 2048 x 2048 912 / 846, 4096 x 4096 1387 /
-// 1349; 256 tokens, six of 4096 x 4096 1254 / 1226.  Half-filled row tiles are not avoided there: where that saved a wave
-// (one_cta) the launches stay (1152 tokens, four of 4096 x 4096 1112 / 1136; 1920 tokens, six of 2304 x 2304, one wave, 1007 / 950).
+// 1.3 us, and a layer's last wave, which the next one's tiles fill; what it costs is a launch whose blocks all have to be there at
+// once, which starts some us later, one tile width for all, and tiles that go row by row, so that a linear's weights are read again
+// with every wave.  One by one / in one launch, us of a forward chain and of an input-gradient chain:
+//   one width       not where linears want different ones: 512 tokens, 2048 - 8192 - 2048 - 8192 - 2048 67 / 78 and 64 / 75; 256 tokens,
+//                   4096 - 16384 - 4096 - 16384 - 4096 107 / 129 and 104 / 125; 2048 tokens, 512 - 2048 - ... 40.4 / 43.0 and 37.9 / 42.0
+//   few and small   four to seven linears pay for the later start only where each fills three fifths of the pairs: 512 tokens, four of 1024
+//                   28.2 / 29.2 and 26.1 / 27.6, of 4096 56.8 / 53.3 and 55.3 / 51.2; 2048 tokens, four of 256 32.3 / 36.3 and 29.7 / 35.3,
+//                   of 1024 36.4 / 34.3 and 33.8 / 32.8; 384 tokens, four of 2560 (40 tiles) 41.1 / 41.0 and 37.9 / 38.9
+//   eight or more   512 tokens, 1024 46.6 / 44.6 and 44.5 / 44.0; 2048 tokens, 256 41.4 / 39.9 and 37.9 / 37.9, 512 50.3 / 44.6 and 46.1 / 43.0
+//   waves           in part-filled ones the gain is largest (eight linears: 4096 tokens, 4096 (3.5 waves) 501 / 431; 2048 tokens, 6144 (2.6)
+//                   549 / 476; 4096 tokens, 6144 (5.2) 1028 / 940); at seven little is left to fill (8192 tokens, 4096 (6.9) 859 / 867)
+//   weights         of more than the L2 cache keeps: bytes times waves 3072 tokens, four of 8192 (348 MB) 661 / 643, 1024 tokens, four of
+//                   10240 (227 MB) 406 / 347, 512 tokens, four of 16384 (464 MB) 423 / 436, 1024 tokens (929 MB) 862 / 1008; 4096 tokens, four
+//                   of 8192 (464 MB) 738 / 842
+// Half-filled row tiles are not avoided there: where that saved a wave (one_cta) the launches stay (us a step of four
+// microbatches: 1152 tokens, four of 4096 x 4096 1112 / 1136; 1920 tokens, six of 2304 x 2304, one wave, 1007 / 950).
+constexpr uint32_t kManyChained = 8;
 bool launch_chained(const GemmDesc* d, uint32_t n, int num_sms) {
   if (n < kLaunchChained || n > kMaxChained || d->M > PAIR_M * (sizeof(DevState::rows_done) / sizeof(uint32_t))) return false;
-  for (uint32_t i = 0; i < n; ++i)
+  const uint32_t pairs = (uint32_t)num_sms / 2u, w = choose_width(d, 1, pairs);
+  for (uint32_t i = 0; i < n; ++i) {
+    const uint32_t tiles = tiles_of(d[i], kTileWidths[w]);
+    if (choose_width(d + i, 1, pairs) != w || (n < kManyChained && 5 * tiles < 3 * pairs) || 2 * tiles > 13 * pairs) return false;
+    if ((uint64_t)d[i].N * d[i].Kc * tiles > 400000000ull * pairs) return false;
     if (d[i].M % PAIR_M && saves_a_wave(d[i], num_sms)) return false;
+  }
   return true;
 }
 
@@ -1379,8 +1394,7 @@ Launch make_launch(const GemmDesc* probs, uint32_t n, int num_sms, const void* f
   l.params.resize(offsetof(P, prob) + n * sizeof(GemmParams));  // (no unused problems)
   unsigned char* at = l.params.data();
   const uint32_t tile_m = alone ? BM : PAIR_M, ctas = alone ? 1u : 2u, most = (uint32_t)num_sms / ctas;
-  uint32_t w = probs->chained ? kNumTileWidths - 1 : choose_width(probs, n, (uint32_t)num_sms / 2u);  // (alone: 0, see one_cta)
-  for (uint32_t i = 0; probs->chained && i < n; ++i) w = std::min(w, choose_width(probs + i, 1, (uint32_t)num_sms / 2u));
+  const uint32_t w = choose_width(probs, probs->chained ? 1 : n, (uint32_t)num_sms / 2u);  // (alone: 0, see one_cta)
   uint32_t tiles = 0;
   uint32_t* ticket = nullptr;
   for (uint32_t i = 0; i < n; ++i) {

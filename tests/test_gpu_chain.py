@@ -126,13 +126,15 @@ def test_chain_of_odd_token_counts_equals_layer_by_layer_bitwise(qe, tokens, mon
 
 
 @pytest.mark.parametrize("mode", [0, 1], ids=["eager", "graph"])
-@pytest.mark.parametrize("tokens,shapes", [(256, [(256, 256)] * 16), (1280, [(512, 1280), (1280, 2048), (2048, 512), (512, 256), (256, 768)]),
-                                           (4096, [(256, 4096), (4096, 256)] * 2), (8192, [(512, 2048), (2048, 256), (256, 4096), (4096, 256)]),
-                                           (8192, [(256, 256)] * 4), (8448, [(256, 256)] * 4)])
-def test_chains_in_one_launch_equal_layer_by_layer_bitwise(qe, mode, tokens, shapes, monkeypatch):
+@pytest.mark.parametrize("tokens,shapes,one_launch", [
+    (256, [(256, 256)] * 16, 2), (1280, [(1280, 1536), (1536, 1792), (1792, 1280), (1280, 1536)], 2), (8192, [(512, 3584), (3584, 512)] * 2, 2),
+    (4096, [(512, 2560), (2560, 1024), (1024, 5632), (5632, 2560)], 1), (8192, [(256, 256)] * 4, 2), (8192, [(256, 3584), (3584, 512), (512, 3584), (3584, 512)], 1),
+    (8448, [(256, 256)] * 4, 0), (1280, [(512, 1280), (1280, 2048), (2048, 512), (512, 256), (256, 768)], 0), (512, [(256, 256)] * 7, 0), (512, [(256, 256)] * 8, 2),
+    (1024, [(512, 2048), (2048, 512)] * 4, 0)])
+def test_chains_in_one_launch_equal_layer_by_layer_bitwise(qe, mode, tokens, shapes, one_launch, monkeypatch):
     """Four linears to sixteen in one launch, whose tiles wait for the rows they read: one tile to a linear, several waves of tiles,
-    contractions longer and shorter than the operand ring, four to seven tiles of one linear for each CTA pair, whose epilogue warps drift
-apart (two K blocks a tile), the most rows it is offered for and one row tile more."""
+    contractions longer and shorter than the operand ring, up to six tiles of one linear for each CTA pair, whose epilogue warps drift
+    apart, the most rows it is offered for and one row tile more; and what goes out one by one.  one_launch: of the two directions."""
     monkeypatch.setattr(sys.modules[__name__], "T", tokens)
     monkeypatch.setattr(sys.modules[__name__], "CHAIN", shapes)
     a = _run(qe, mode, chained=False)
@@ -148,7 +150,7 @@ apart (two K blocks a tile), the most rows it is offered for and one row tile mo
             assert all(state_equal(x, y) and x["device_token"] == y["device_token"] and x["device_status"] == 0 for x, y in zip(u, v)), key
     # per step: the casts between the linears, their GEMMs but one a chain, the weights' casts but one
     fewer = a["stats"]["kernels_launched"] - b["stats"]["kernels_launched"]
-    assert fewer == 2 * (len(shapes) - 1) * (3 * 2 * (2 if tokens <= 8192 else 1) + 1)
+    assert fewer == 2 * (len(shapes) - 1) * (3 * 2 + 3 * one_launch + 1)
 
 
 def test_chain_against_the_oracle_composition(qe):
