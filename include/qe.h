@@ -218,9 +218,9 @@ int32_t qe_backward_dI(qe_layer*, const qe_tape*, const void* dy_dev, void* dx_d
  * read-back writes what the upload reads, which is then uploaded after it; other work of the caller's on that stream
  * that writes a host input must be complete when the call is made.  With any other caller_stream the upload waits for
  * all that the stream holds, the read-backs of its earlier calls among it.  Pinned host memory makes the copies
- * asynchronous; y_host / dx_host may be NULL to skip the read-back.  Large calls whose input and output do not overlap go
- * through in two to four pieces of rows, so that a call's own copies overlap too (kernels of pieces are launched eagerly in
- * graph mode as well).  Same checks, state transitions and results as qe_forward / qe_backward_dI. */
+ * asynchronous; y_host / dx_host may be NULL to skip the read-back.  Large calls whose input and output are pinned and do
+ * not overlap go through in two to four pieces of rows, so that a call's own copies overlap too (kernels of pieces are launched
+ * eagerly in graph mode as well).  Same checks, state transitions and results as qe_forward / qe_backward_dI. */
 int32_t qe_forward_host(qe_layer*, uint32_t mb, uint64_t gen, const void* x_host, void* y_host, void* caller_stream,
                         qe_tape* tape_out);
 int32_t qe_backward_dI_host(qe_layer*, const qe_tape*, const void* dy_host, void* dx_host, void* caller_stream);

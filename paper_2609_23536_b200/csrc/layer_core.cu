@@ -363,19 +363,30 @@ int32_t host_download(qe_ctx* ctx, void* dst_host, const void* src, size_t bytes
   return st != QE_OK ? st : downloads_end(ctx, dst_host);
 }
 
+// Whether copies from or to host memory run beside the host.
+static bool pinned(const void* p) {
+  cudaPointerAttributes a{};
+  if (cudaPointerGetAttributes(&a, p) == cudaSuccess) return a.type != cudaMemoryTypeUnregistered;
+  cudaGetLastError();  // (the question's, not a call's)
+  return false;
+}
+
 // Pieces of rows in which a forward or an input gradient with host buffers goes through upload, kernels and read-back: the
 // host link carries both directions at once, but one after the other a call's input, kernels and output used it one at a time.
 // Two pieces, or one for every 512 rows up to four, of whole 256-row tiles, whose larger copy is a megabyte at least (19 us at 53
 // GB/s; a piece costs some 15 us of copy starts, events and kernels that its neighbours' copies have to cover).  us a step in one
 // piece / two / up to four of 256 rows: a block of hidden 1024, 1024 tokens, 6385 / 5716 / 5861; 2048 tokens, 1024 x 3072 and
-// 1024 x 1024, 3252 / 2949 / 2882; 640 tokens, 2048 x 2048 and 2048 x 512, 1377 / 1313 / 1312; up to eight of 128 rows 6428 and 3152.
-// An output that overlaps the input is read back when all of that has been uploaded.
+// 1024 x 1024, 3252 / 2949 / 2882; 640 tokens, 2048 x 2048 and 2048 x 512, 1377 / 1313 / 1312; up to eight of 128 rows 6428 and 3152.  In one
+// piece / four: 4096 tokens, 1024 x 3072 and 1024 x 1024, 4018 / 3503, 4096 x 4096 5286 / 3927; 8192, 2048 x 2048 and 2048 x 512, 8375 / 6665.
+// An output that overlaps the input is read back when all of that has been uploaded.  Pageable memory goes through in one piece:
+// each of its copies is over before the call goes on, so that pieces would only add waits (F and dI of 1024 x 3072 at 1024 tokens
+// 1050 us in one, 1220 in two; 2048 x 2048 at 2048 tokens 1900 and 2380, at 4096 3580 and 4270 in four).
 uint32_t host_pieces(uint32_t rows, const void* in, uint64_t in_bytes, const void* out, uint64_t out_bytes) {
   if (!out) out_bytes = 0;
   if ((uintptr_t)in < (uintptr_t)out + out_bytes && (uintptr_t)out < (uintptr_t)in + in_bytes) return 1;
   const uint64_t most = std::min<uint64_t>(4, std::max<uint64_t>(2, rows / 512u));
   const uint64_t n = std::min<uint64_t>({most, rows / 256u, std::max(in_bytes, out_bytes) >> 20});
-  return (uint32_t)std::max<uint64_t>(1, n);
+  return n > 1 && pinned(in) && (!out || pinned(out)) ? (uint32_t)n : 1u;
 }
 
 // F (kind QE_ACT_F) or dI of slot p with host buffers, in pieces; the scale commits go with the last piece's GEMM, whose launch

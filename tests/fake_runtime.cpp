@@ -30,6 +30,7 @@ struct State {
   Graph* graph = nullptr;
   long encodes = 0;
   int sms = 148, pairs = 74;
+  size_t pageable_from = 0, pageable_to = 0;
 };
 State* g = nullptr;  // (never freed: the library may be used until the process ends)
 State& s() {
@@ -86,11 +87,12 @@ void operator delete(void* p, size_t, std::align_val_t) noexcept { std::free(p);
 extern "C" {
 const char* fake_log() { return s().log.c_str(); }
 const char* fake_replayed() { return s().replayed.c_str(); }
-void fake_reset() { s().log.clear(); s().replayed.clear(); s().fail_in.clear(); s().alloc_in = -1; s().encodes = 0; }
+void fake_reset() { s().log.clear(); s().replayed.clear(); s().fail_in.clear(); s().alloc_in = -1; s().encodes = 0; s().pageable_from = s().pageable_to = 0; }
 void fake_fail(const char* fn, long nth) { s().fail_in[fn] = nth; }
 void fake_fail_alloc(long nth) { s().alloc_in = nth; }
 long fake_alloc_left() { return s().alloc_in; }
 void fake_sms(int n) { s().sms = n; }  // before the library has looked at the device
+void fake_pageable(size_t from, size_t to) { s().pageable_from = from, s().pageable_to = to; }  // other host memory is pinned
 void fake_pairs(int n) { s().pairs = n; }  // CTA pairs that the device holds at once
 long fake_encodes() { return s().encodes; }
 
@@ -134,6 +136,12 @@ cudaError_t cudaMemcpyAsync(void* d, const void* src, size_t n, cudaMemcpyKind k
   note("%s %ld %zu %zu %zu", k == cudaMemcpyHostToDevice ? "h2d" : "d2h", sid(st), (size_t)d, (size_t)src, n);
   return cudaSuccess;
 }
+cudaError_t cudaPointerGetAttributes(cudaPointerAttributes* a, const void* p) {
+  FAILS(cudaPointerGetAttributes);
+  a->type = (size_t)p >= s().pageable_from && (size_t)p < s().pageable_to ? cudaMemoryTypeUnregistered : cudaMemoryTypeHost;
+  return cudaSuccess;
+}
+cudaError_t cudaGetLastError() { return cudaSuccess; }
 cudaError_t cudaGetSymbolAddress(void** p, const void* sym) { *p = const_cast<void*>(sym); return cudaSuccess; }
 
 cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void*, void** args) {

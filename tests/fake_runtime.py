@@ -41,6 +41,7 @@ def load(so):
     lib.fake_log.restype = lib.fake_replayed.restype = C.c_char_p
     lib.fake_fail.argtypes = [C.c_char_p, C.c_long]
     lib.fake_fail_alloc.argtypes = [C.c_long]
+    lib.fake_pageable.argtypes = [C.c_size_t, C.c_size_t]
     lib.fake_alloc_left.restype = lib.fake_encodes.restype = C.c_long
     lib.fake_reset()
     return lib

@@ -333,6 +333,33 @@ def test_host_buffers_go_through_copies_and_kernels_in_pieces_of_rows(lib, T, pi
     s.close()
 
 
+@pytest.mark.parametrize("which", ["none", "input", "output", "unknown"])
+def test_host_buffers_that_are_not_pinned_go_through_in_one_piece(lib, which):
+    """A copy from or to pageable memory ends before the call that starts it does: pieces would only add waits."""
+    import ctypes as C
+
+    from paper_2609_23536_b200 import binding as qe
+
+    T, K, N = 2048, 256, 2048
+    s = fake_runtime.Stage(lib, [(K, N)], T=T, host_io=True, slots=2)
+    x, y, tape = s.buffer(2 * T * K), s.buffer(2 * T * N), qe.qe_tape()
+    for forward in (True, False):
+        a, b, bytes_of = (x, y, {x: 2 * T * K, y: 2 * T * N}) if forward else (y, x, {x: 2 * T * K, y: 2 * T * N})
+        lib.fake_reset()
+        if which in ("input", "output"):
+            p = a if which == "input" else b
+            lib.fake_pageable(p, p + bytes_of[p])
+        if which == "unknown":
+            lib.fake_fail(b"cudaPointerGetAttributes", 1)
+        if forward:
+            assert lib.qe_forward_host(s.layers[0], 0, 0, a, b, fake_runtime.CALLER, C.byref(tape)) == 0
+        else:
+            assert lib.qe_backward_dI_host(s.layers[0], C.byref(tape), a, b, fake_runtime.CALLER) == 0
+        order = fake_runtime.Order(lib.fake_log().decode())
+        assert len(order.of("h2d")) == len(order.of("d2h")) == (4 if which == "none" else 1)
+    s.close()
+
+
 @pytest.mark.parametrize("mode", [0, 1], ids=["eager", "graph"])
 def test_casts_that_overlap_go_ahead_on_a_count_of_commits(lib, mode):
     """A cast that does not wait for the GEMM launch before it is told how many problems will have committed by then, and that
