@@ -343,11 +343,16 @@ static int32_t download(qe_ctx* ctx, void* dst_host, const void* src, size_t byt
   QE_CUDA(cudaEventRecord(ctx->ev_kernels, ctx->exec_stream));
   ctx->kernels_recorded = true;
   if (!dst_host) return QE_OK;
-  if (ctx->readbacks.size() == 256) {
-    const int32_t st = uploads_after_readbacks(ctx);
-    if (st != QE_OK) return st;
+  const uintptr_t lo = (uintptr_t)dst_host;
+  if (!ctx->readbacks.empty() && ctx->readbacks.back().hi == lo) {
+    ctx->readbacks.back().hi += bytes;  // a call's next piece
+  } else {
+    if (ctx->readbacks.size() == 256) {
+      const int32_t st = uploads_after_readbacks(ctx);
+      if (st != QE_OK) return st;
+    }
+    ctx->readbacks.push_back({lo, lo + bytes});
   }
-  ctx->readbacks.push_back({(uintptr_t)dst_host, (uintptr_t)dst_host + bytes});
   QE_CUDA(cudaStreamWaitEvent(ctx->d2h_stream, ctx->ev_kernels, 0));
   QE_CUDA(cudaMemcpyAsync(dst_host, src, bytes, cudaMemcpyDeviceToHost, ctx->d2h_stream));
   QE_CUDA(cudaEventRecord(ctx->ev_d2h, ctx->d2h_stream));

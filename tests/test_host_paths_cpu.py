@@ -333,6 +333,25 @@ def test_host_buffers_go_through_copies_and_kernels_in_pieces_of_rows(lib, T, pi
     s.close()
 
 
+def test_no_upload_of_a_call_waits_for_its_own_read_back_however_many_calls_were_before(lib):
+    import ctypes as C
+
+    from paper_2609_23536_b200 import binding as qe
+
+    T, K, N, pieces = 1536, 256, 2048, 3
+    s = fake_runtime.Stage(lib, [(K, N)], T=T, host_io=True, slots=2, exec_stream=fake_runtime.CALLER)
+    x, ys, tape = s.buffer(2 * T * K), s.buffer(4 * T * N), qe.qe_tape()
+    lib.fake_reset()
+    for i in range(300):  # (outputs in turn, so that they do not follow one another)
+        assert lib.qe_forward_host(s.layers[0], 0, 0, x, ys + (i % 2) * 2 * T * N, fake_runtime.CALLER, C.byref(tape)) == 0
+        assert lib.qe_abort_step(s.layers[0]) == 0 and lib.qe_arena_rebuild(s.layers[0]) == 0
+    order = fake_runtime.Order(lib.fake_log().decode())
+    up, down = order.of("h2d"), order.of("d2h")
+    assert len(up) == len(down) == 300 * pieces
+    assert not any(order.before(down[j], up[i]) for i in range(len(up)) for j in range(i - i % pieces, i))
+    s.close()
+
+
 @pytest.mark.parametrize("which", ["none", "input", "output", "unknown"])
 def test_host_buffers_that_are_not_pinned_go_through_in_one_piece(lib, which):
     """A copy from or to pageable memory ends before the call that starts it does: pieces would only add waits."""
