@@ -174,8 +174,8 @@ __device__ __forceinline__ bool rows_wait(const uint32_t* done, uint32_t count, 
   return __all_sync(0xffffffffu, there);
 }
 
-// ... and how they say it: the last warp of a CTA to have stored its part (last_of_tile), for all of them.  (An addition of each warp's own, behind a fence of
-// each lane, took 3500 clocks from a tile's last store until its rows were seen to be there; now 2000.)
+// ... and how they say it: the last warp of a CTA to have stored its part (last_of_tile), for all of them.  (An addition of each
+// warp's own, behind a fence of each lane, took 3500 clocks from a tile's last store until its rows were seen to be there; now 2000.)
 __device__ __forceinline__ uint32_t add_acq_rel_cta(uint32_t* count /* shared */) {
   uint32_t before;
   asm volatile("atom.acq_rel.cta.shared::cta.add.u32 %0, [%1], 1;" : "=r"(before) : "r"(smem_u32(count)) : "memory");
@@ -191,6 +191,13 @@ __device__ __forceinline__ bool last_of_grid(uint32_t* ticket, uint32_t ctas) {
 }
 __device__ __forceinline__ void add_release(uint32_t* p, uint32_t v) {
   asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+
+// Of a role that loads into shared memory, when the launch is being abandoned: gives copies already in flight a bounded chance to
+// land before the CTA's shared memory goes away.
+__device__ __forceinline__ void let_copies_land() {
+  const long long t0 = clock64();
+  while (clock64() - t0 < 2000000ll) { }
 }
 
 // Arrival on a barrier that may live in the peer CTA.  What it announces are tensor-memory reads, ordered by the
@@ -745,11 +752,7 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
         }
       }
     }
-    if (!ok) {
-      // give copies already in flight a bounded chance to land before the CTA's shared memory goes away
-      const long long t0 = clock64();
-      while (clock64() - t0 < 2000000ll) { }
-    }
+    if (!ok) let_copies_land();
   } else if (warp == 1) {
     // ---------------------------------------------------------------- MMA issuer
     if (rank == 0) {
@@ -916,6 +919,7 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
       }
     }
     if (lane == 0) tma_store_wait_read<0>();
+    if (!ok) let_copies_land();
   } else if (!SUMS || warp >= EPI_WARP0) {
     // ---------------------------------------------------------------- epilogue
     if (SUMS) asm volatile("setmaxnreg.inc.sync.aligned.u32 224;");
