@@ -457,9 +457,9 @@ struct Problems {
   __device__ __forceinline__ uint32_t* status_of(uint32_t i) const { return g.prob[i].status; }
 };
 
-// What the roles need to know of a tile (INFO_BYTES of shared memory at most).  `alpha` is filled in later than the rest: scales
+// What the roles need to know of a tile (INFO_BYTES of shared memory at most; written 16 bytes at a time up to amax_bits).  `alpha` is filled in later than the rest: scales
 // come from kernels before this one.
-struct TileInfo {
+struct alignas(16) TileInfo {
   uint32_t problem, m0, n0, num_kb;
   uint32_t nseg, epi, a_mn, b_mn;
   uint32_t idesc, b_desc_hi, b_step, ldo;
@@ -470,7 +470,8 @@ struct TileInfo {
   float alpha[kMaxSegments];
   uint32_t minus_zero;  // see mul2; 0 where the tile is no sum
 };
-static_assert(sizeof(TileInfo) <= INFO_BYTES && offsetof(TileInfo, alpha) % 4 == 0, "");
+static_assert(sizeof(TileInfo) <= INFO_BYTES && INFO_BYTES % alignof(TileInfo) == 0 && BARS_BYTES % alignof(TileInfo) == 0 &&
+              offsetof(TileInfo, amax_bits) % 16 == 0, "");
 // The same value in every lane, and known to be: kept in a uniform register, as the instructions of the issuing roles want it.
 __device__ __forceinline__ uint32_t uniform(uint32_t v) { return __reduce_or_sync(0xffffffffu, v); }
 
