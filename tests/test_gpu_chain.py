@@ -16,6 +16,7 @@ pytestmark = pytest.mark.gpu
 DEV = "cuda:0"
 T = 256
 CHAIN = [(256, 512), (512, 256), (256, 768)]  # (K, N): each layer consumes the one before
+EIGHT = [(256, 512), (512, 256), (256, 768), (768, 256), (256, 512), (512, 512), (512, 256), (256, 768)]  # these go out in one launch
 
 
 @pytest.fixture(scope="module")
@@ -153,6 +154,76 @@ def test_chains_in_one_launch_equal_layer_by_layer_bitwise(qe, mode, tokens, sha
     assert fewer == 2 * (len(shapes) - 1) * (3 * 2 + 3 * one_launch + 1)
 
 
+@pytest.mark.parametrize("mode", [0, 1], ids=["eager", "graph"])
+@pytest.mark.parametrize("tokens,shapes", [(256, EIGHT), (2048, [(1536, 2048), (2048, 1536), (1536, 1536), (1536, 2048)])])
+def test_chains_in_one_launch_beside_weight_gradients_on_the_second_stream_equal_layer_by_layer_bitwise(qe, mode, tokens, shapes, monkeypatch):
+    monkeypatch.setattr(sys.modules[__name__], "T", tokens)
+    monkeypatch.setattr(sys.modules[__name__], "CHAIN", shapes)
+    a = _run(qe, mode, chained=False, steps=3, M=5, overlap=True)
+    b = _run(qe, mode, chained=True, steps=3, M=5, overlap=True)
+    for key in ("Y", "dX", "mg"):
+        for u, v in zip(a[key], b[key]):
+            assert np.array_equal(u.view(np.uint8), v.view(np.uint8)), key
+    for u, v in zip(a["state"], b["state"]):
+        assert all(state_equal(x, y) and x["device_token"] == y["device_token"] and x["device_status"] == 0 for x, y in zip(u, v))
+    assert a["stats"]["kernels_launched"] - b["stats"]["kernels_launched"] == 3 * (len(shapes) - 1) * (5 * 4 + 1)
+
+
+@pytest.mark.parametrize("mode", [0, 1], ids=["eager", "graph"])
+@pytest.mark.parametrize("t,h,n", [(512, 1024, 8), (2048, 2048, 4)], ids=["both-fit", "one-fits"])
+def test_chains_of_two_contexts_at_a_time_equal_those_of_one(qe, mode, t, h, n):
+    """A launch has all its blocks (64; 128 of 148) on the device at once; two streams ask for that at the same time, with weight
+    gradients beside them."""
+    M = 4
+
+    class Stage:
+        def __init__(self, seed):
+            self.ctx = qe.Context(mode, overlap_dw=True)
+            self.layers = [qe.Layer(self.ctx, t, h, h, 4, 0, M, inputs.weights("C2C", seed, j, h, h).to(DEV), unit=j) for j in range(n)]
+            self.x = [inputs.activations("C2C", seed, 0, 0, m, t, h).to(DEV) for m in range(M)]
+            self.dy = [inputs.upstream_grads("C2C", seed, 0, 0, m, t, h).to(DEV) for m in range(M)]
+            self.y, self.dx = [torch.empty_like(v) for v in self.x], [torch.empty_like(v) for v in self.x]
+            self.grad = torch.zeros(n * h * h, device=DEV)
+            self.stream, self.tapes = torch.cuda.Stream(), {}
+
+        def forward(self, step, m):
+            with torch.cuda.stream(self.stream):
+                self.tapes[m] = qe.forward_chain(self.layers, m, step, self.x[m], self.y[m])
+
+        def backward(self, m):
+            with torch.cuda.stream(self.stream):
+                qe.backward_dI_chain(self.layers, self.tapes[m], self.dy[m], self.dx[m])
+                qe.backward_dW_multi(self.layers, self.tapes[m], self.grad, [j * h * h for j in range(n)])
+
+        def result(self):
+            torch.cuda.synchronize()
+            states = [L.state() for L in self.layers]
+            assert all(s["device_status"] == 0 for s in states)
+            return [inputs.bits(v.cpu()) for v in self.y + self.dx] + [self.grad.cpu().numpy().view(np.uint32)], states
+
+    got = []
+    for together in (False, True):
+        stages = [Stage(0), Stage(1)]
+        torch.cuda.synchronize()
+        for step in range(3):
+            for order in ([stages] if together else [[s] for s in stages]):
+                for m in range(M):
+                    for s in order:
+                        s.forward(step, m)
+                for m in range(M):
+                    for s in order:
+                        s.backward(m)
+                if not together:
+                    torch.cuda.synchronize()
+            for s in stages:
+                with torch.cuda.stream(s.stream):
+                    qe.optimizer_boundary_all(s.layers, M)
+        got.append([s.result() for s in stages])
+    for (u, su), (v, sv) in zip(*got):
+        assert all(np.array_equal(x, y) for x, y in zip(u, v))
+        assert all(state_equal(x, y) and x["device_token"] == y["device_token"] for x, y in zip(su, sv))
+
+
 def test_chain_against_the_oracle_composition(qe):
     M, steps = 3, 2
     s = sched(M, 2, 1)
@@ -207,14 +278,15 @@ def test_chain_against_the_oracle_composition(qe):
         assert gs["token"] == os_["token"] and gs["e_W"] == os_["e_W"] and gs["slots"] == os_["slots"]
 
 
-@pytest.mark.parametrize("mode", [0, 1], ids=["eager", "graph"])
-def test_chain_layer_by_layer_against_a_teacher_forced_oracle(qe, mode):
+@pytest.mark.parametrize("mode,shapes", [(0, CHAIN), (1, CHAIN), (1, EIGHT)], ids=["eager", "graph", "one-launch"])
+def test_chain_layer_by_layer_against_a_teacher_forced_oracle(qe, mode, shapes, monkeypatch):
     """Every layer of the chain against the oracle at the single-GEMM tolerance.  The free-running comparison above
     lets a one-ulp difference in an interior bf16 value move an FP8 code downstream, so it cannot be tight.  Here the
     oracle layer j+1 is fed the bf16 tensor the GPU's layer j produced (taken from the layer-by-layer run, which the
     chained run equals bit for bit): what the hand-off deposits in the consumer -- FP8 bytes, amax, inverse-scale
     snapshot, the consumer's X / G scale state -- is then fixed exactly by the delayed-scaling recipe (Sec. 2.1) and
     must match bit for bit, and each GEMM output must lie within 1e-3 (Frobenius) and 4 bf16 ulp of the oracle's."""
+    monkeypatch.setattr(sys.modules[__name__], "CHAIN", shapes)
     M, steps = 3, 2
     s = sched(M, 2, 1)
     P = peak_live(s)
