@@ -84,16 +84,7 @@ __device__ __forceinline__ uint32_t ring_max(const uint32_t* ring, uint32_t n, u
   return __reduce_max_sync(0xffffffffu, top);
 }
 
-// The same commit of ONE class (class_mask has one bit: X or G at a GEMM launch's start, Y in its tail) by one warp; EACH: of a
-// class per lane, for lanes with `active`.  A grouped launch may carry dozens of problems, all committed side by side by lanes
-// of the epilogue's warps: a commit is a chain of dependent global accesses, and one after the other the commits of a launch
-// took as long as its tiles.  The code runs once per launch, from cold instruction memory, so it is short, with one loop for
-// the rare ring scan, which a whole warp makes for one lane after the other (launches of one problem keep the form without
-// lanes: with it twelve chained linears of 256 x 256 took 1402 us a step, without it 1389).  F, dI and dW of a 256 x 256 x 256
-// linear plus the boundary take 55 us when no commit scans; when all three do, 60 us at 4096 entries and the same as without
-// at 1024.  Same values as commit_classes; the token is bumped atomically because two problems of one launch may belong to
-// the same layer (its forward and its input gradient of different microbatches).
-// What a commit of a class reads besides its amax, where that can be read ahead: nothing else commits the class until then.
+// What a commit of a class reads besides its amax.
 struct RingState {
   uint32_t count = 0, wmax = 0, evicted = 0;
 };
@@ -105,6 +96,16 @@ __device__ __forceinline__ RingState ring_state(const CommitParams& p, int c) {
   return s;
 }
 
+// The same commit of ONE class (class_mask has one bit: X or G at a GEMM launch's start, Y in its tail) by one warp; EACH: of a
+// class per lane, for lanes with `active`.  A grouped launch may carry dozens of problems, all committed side by side by lanes
+// of the epilogue's warps: a commit is a chain of dependent global accesses, and one after the other the commits of a launch
+// took as long as its tiles.  The code runs once per launch, from cold instruction memory, so it is short, with one loop for
+// the rare ring scan, which a whole warp makes for one lane after the other (launches of one problem keep the form without
+// lanes: with it twelve chained linears of 256 x 256 took 1402 us a step, without it 1389).  F, dI and dW of a 256 x 256 x 256
+// linear plus the boundary take 55 us when no commit scans; when all three do, 60 us at 4096 entries and the same as without
+// at 1024.  Same values as commit_classes; the token is bumped atomically because two problems of one launch may belong to
+// the same layer (its forward and its input gradient of different microbatches).  `ahead`: the class's state, read after
+// grid_dep_wait() and with no other commit of the class between that and this one.
 template <bool EACH>
 __device__ __forceinline__ void commit_class(const CommitParams& p, uint32_t class_mask, bool bump, bool active, int lane, const RingState* ahead = nullptr) {
   DevState* st = p.st;

@@ -2,7 +2,7 @@
 // stored contraction-major ([rows, Kc]) or MN-major ([Kc, rows]: the transposed view of a row-major tensor, read by the
 // tensor cores directly), FP32 accumulation in tensor memory.
 //
-// Structure: persistent clusters of two CTAs on neighbouring SMs, 320 or 384 threads each, that compute one tile of 256 rows
+// Structure: persistent clusters of two CTAs on neighbouring SMs, 320, 352 or 384 threads each, that compute one tile of 256 rows
 // and 256, 128 or 64 columns together with tcgen05.mma.cta_group::2:
 //   warp 0      TMA producer: cp.async.bulk.tensor boxes into a shared-memory ring (six stages of a 128-byte K block, or four
 //               of two blocks for tiles of 128 or 64 columns); each CTA loads its own 128 rows of A and its own half of the
@@ -174,8 +174,8 @@ __device__ __forceinline__ bool rows_wait(const uint32_t* done, uint32_t count, 
   return __all_sync(0xffffffffu, there);
 }
 
-// ... and how they say it: the last warp of a CTA to have stored its part (last_of_tile), for all of them.  (An addition of each
-// warp's own, behind a fence of each lane, took 3500 clocks from a tile's last store until its rows were seen to be there; now 2000.)
+// ... and how they say it: the last warp of a CTA to have stored its part (last_of_tile), for all of them.  (By an addition of
+// each warp's own, behind a fence of each lane, sixteen linears of 1024 x 1024 at 512 tokens took 1636 us a step; 1500 now.)
 __device__ __forceinline__ uint32_t add_acq_rel_cta(uint32_t* count /* shared */) {
   uint32_t before;
   asm volatile("atom.acq_rel.cta.shared::cta.add.u32 %0, [%1], 1;" : "=r"(before) : "r"(smem_u32(count)) : "memory");
@@ -1281,9 +1281,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(SHARED_SM_THREADS, 1
 // Chained problems: each one's A is the result of the one before, handed on in FP8, in one launch.  Its CTAs wait on one another
 // (a cooperative launch): a tile's loads of A for its rows of the problem before, which are counted as they are stored; those
 // of B do not wait, up to a ring-full, and a tile waits behind earlier ones only.  The scales are committed when all is done.  Of the
-// 7300 clocks from one 512 x 1024 x 1024 to the next (tiles of 64 columns, half of the CTAs) the loads of A take 2400, the MMAs
-// behind them 700, the epilogue 700, and 3500 pass between the last store and the loads that wait for it: the fence, the
-// count, the poll (16 layers: 66 us a launch, 88 as launches of their own).
+// 7800 clocks from one 512 x 1024 x 1024 to the next (tiles of 64 columns, half of the CTAs) the loads of A take 2560, the MMAs
+// behind them 680, the epilogue 670, the count among a CTA's warps 300, and some 3600 pass until the next linear's loads are let
+// go: the release, 1050 of them, and the poll (16 layers: 66 us a launch, 88 as launches of their own).
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(threads_of(false, true), 1)
     gemm_fp8_pair_chain_kernel(const __grid_constant__ GemmLaunchParams<kMaxChained> g) {
   gemm_body<true>(Problems<kMaxChained, false, 1, true>{g});
