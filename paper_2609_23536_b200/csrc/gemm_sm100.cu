@@ -1145,7 +1145,7 @@ __device__ __forceinline__ void gemm_body(const PS& ps) {
       // order, each with its own scale -- the additions that launches of their own would have done in L2, at one read and one
       // write of the destination instead of one per product.  (A loop of its own behind the other tiles': in one loop with them
       // the values did not fit the registers, and the few bytes of them in local memory, for which shared memory leaves no L1,
-      // cost more than all that is saved here.)
+      // cost more than all that is saved here.  12 bytes a thread are still there.)
       f32x2 v[4][16];                    // this thread's row
       const uint32_t all = tile_n / 64u;  // blocks of a tile that is not ragged: what buffers are handed on for
       if (lane == 0) tma_store_wait_read<0>();

@@ -1,6 +1,6 @@
 """Small single-kernel cases for profiling (ncu) and quick timing.
 
-    python profile_case.py gemm_f|gemm_di|gemm_dw|gemm_narrow|gemm_odd|gemm_microbatch|gemm_microbatch_grouped|gemm_step|step_sums|step_many|step_block|quantize|quantize_t|amax|accumulate [--reps N] [--timeline]
+    python profile_case.py gemm_f|gemm_di|gemm_dw|gemm_narrow|gemm_odd|gemm_microbatch|gemm_microbatch_grouped|gemm_step|step_sums|step_many|step_block|chain|quantize|quantize_t|amax|accumulate [--reps N] [--timeline]
 
 Each case holds well under 2 GB on the device, uses operands larger than the 126 MB L2 where DRAM traffic is
 the question, does 2 warm-up launches and then `reps` launches, and prints the CUDA-event time per launch.
@@ -107,6 +107,23 @@ def main():
             qe.optimizer_boundary_all(layers, M)
 
         work = {"flop": 6.0 * t * M * sum(K * N for K, N in shapes), "bytes": sum(4 * t * M * (K + N) + 6 * K * N for K, N in shapes)}
+    elif a.case == "chain":
+        # sixteen linears of 1024 x 1024 that feed one another, 512 tokens: a forward and an input-gradient chain, a launch each
+        # (gemm_fp8_pair_chain_kernel), and the launches around them
+        t, n = 512, 16
+        ctx = qe.Context(qe.EAGER)
+        rnd = lambda *shape: torch.randn(shape, device=dev).to(torch.bfloat16)
+        layers = [qe.Layer(ctx, t, 1024, 1024, 16, 0, 1, rnd(1024, 1024).mul_(0.02), unit=u) for u in range(n)]
+        x, y, dy, dx = (rnd(t, 1024) for _ in range(4))
+        grad, epoch = torch.zeros(n << 20, device=dev), iter(range(1 << 30))
+
+        def fn():
+            tapes = qe.forward_chain(layers, 0, next(epoch), x, y)
+            qe.backward_dI_chain(layers, tapes, dy, dx)
+            qe.backward_dW_multi(layers, tapes, grad, [u << 20 for u in range(n)])
+            qe.optimizer_boundary_all(layers, 1)
+
+        work = {"flop": 6.0 * t * n * 2**20, "bytes": 8 * t * 1024 + 6 * n * 2**20}
     elif a.case.startswith("gemm"):
         # gate/up projection: F: [T,H]x[F,H]^T ; dI: [T,F]x[H,F]^T ; dW: [F,T]x[H,T]^T (FP32 accumulate); a weight
         # gradient small enough for tiles of 64 columns; a forward of nine 128-row tiles, a CTA to a tile
